@@ -214,6 +214,7 @@ class Analyzer:
         if rc != OK:
             raise CcldError(rc, "ccld_create failed")
         self._keep: Dict[int, list] = {}
+        self._bufs: Dict[type, np.ndarray] = {}
 
     # -- helpers
     def _check(self, rc: int):
@@ -292,28 +293,34 @@ class Analyzer:
         self._check(self.lib.ccld_set_speculation(self.h, 1 if on else 0))
 
     @staticmethod
-    def _records(buf, struct, count, cap):
-        dt = np.dtype([(k, _NP_OF[t]) for k, t in struct._fields_])
-        a = np.frombuffer(buf, dtype=dt, count=max(cap, 1))[:count]
-        return {k: a[k].copy() for k in dt.names}
+    def _columns(a, count):
+        """The first `count` entries of a structured array as one array per field."""
+        a = a[:count]
+        return {k: a[k].copy() for k in a.dtype.names}
+
+    def _list_buf(self, struct, cap):
+        """Room for `cap` entries of a C struct. Kept between calls: the library writes only the entries there are, and a fresh
+        buffer of a default capacity (7 MB of rows) would be zeroed and faulted in on every call."""
+        b = self._bufs.get(struct)
+        if b is None or len(b) < cap:
+            b = self._bufs[struct] = np.empty(max(cap, 1), np.dtype([(k, _NP_OF[t]) for k, t in struct._fields_]))
+        return b
 
     def get_verdict(self, window_id: int, comm_rows_cap: int = 1 << 16, alerts_cap: int = MAX_ALERTS_PER_WINDOW,
                     suspects_cap: int = 1 << 16, check: bool = True) -> Dict[str, object]:
-        rows = (CommVerdict * max(comm_rows_cap, 1))()
-        alerts = (HangAlert * max(alerts_cap, 1))()
-        sus = (Suspect * max(suspects_cap, 1))()
+        rows, alerts, sus = self._list_buf(CommVerdict, comm_rows_cap), self._list_buf(HangAlert, alerts_cap), self._list_buf(Suspect, suspects_cap)
         v = Verdict()
-        v.comm_rows = C.cast(rows, C.POINTER(CommVerdict)); v.comm_rows_cap = comm_rows_cap
-        v.alerts = C.cast(alerts, C.POINTER(HangAlert)); v.alerts_cap = alerts_cap
-        v.suspects = C.cast(sus, C.POINTER(Suspect)); v.suspects_cap = suspects_cap
+        v.comm_rows = C.cast(rows.ctypes.data, C.POINTER(CommVerdict)); v.comm_rows_cap = comm_rows_cap
+        v.alerts = C.cast(alerts.ctypes.data, C.POINTER(HangAlert)); v.alerts_cap = alerts_cap
+        v.suspects = C.cast(sus.ctypes.data, C.POINTER(Suspect)); v.suspects_cap = suspects_cap
         rc = self.lib.ccld_get_verdict(self.h, window_id, C.byref(v))
         if check:
             self._check(rc)
         out: Dict[str, object] = {k: int(getattr(v, k)) for k, _ in Verdict._fields_[:15]}
         out["rc"] = rc
-        out["comm_rows"] = self._records(rows, CommVerdict, min(v.n_comm_rows_total, comm_rows_cap), comm_rows_cap)
-        out["alerts"] = self._records(alerts, HangAlert, min(v.n_alerts_total, alerts_cap, MAX_ALERTS_PER_WINDOW), alerts_cap)
-        out["suspects"] = self._records(sus, Suspect, min(v.n_suspects_total, suspects_cap), suspects_cap)
+        out["comm_rows"] = self._columns(rows, min(v.n_comm_rows_total, comm_rows_cap))
+        out["alerts"] = self._columns(alerts, min(v.n_alerts_total, alerts_cap, MAX_ALERTS_PER_WINDOW))
+        out["suspects"] = self._columns(sus, min(v.n_suspects_total, suspects_cap))
         return out
 
     def locate_hang(self, window_id: int, comm: int, seq: int, roots_cap: int = MAX_COMM_SIZE) -> Dict[str, object]:
@@ -380,9 +387,9 @@ class Analyzer:
     def get_ranges(self, window_id: int) -> Dict[str, np.ndarray]:
         n = C.c_uint32(0)
         self._check(self.lib.ccld_get_ranges(self.h, window_id, None, 0, C.byref(n)))
-        rows = (CommRange * max(n.value, 1))()
-        self._check(self.lib.ccld_get_ranges(self.h, window_id, C.cast(rows, C.c_void_p), n.value, C.byref(n)))
-        return self._records(rows, CommRange, n.value, n.value)
+        rows = self._list_buf(CommRange, n.value)
+        self._check(self.lib.ccld_get_ranges(self.h, window_id, rows.ctypes.data, n.value, C.byref(n)))
+        return self._columns(rows, n.value)
 
     def get_optable(self, window_id: int, to_host: bool = True) -> Dict[str, object]:
         """Per-op table of an analysed window; with to_host the columns come back as numpy arrays."""

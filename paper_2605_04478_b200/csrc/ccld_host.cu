@@ -14,6 +14,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "ccld_kernels.cuh"
+#include "ccld_verdict.cuh"
 #include "ccld_rates.cuh"
 #include "ccld_opset.cuh"
 
@@ -97,6 +98,8 @@ struct ccld_ctx {
   std::map<u32, WindowHost> windows;
   Pool pool; std::string err;
   u64* h_pinned = nullptr; size_t h_pinned_bytes = 0;
+  char* h_verdict = nullptr;                             // pinned area of ccld_get_verdict (VerdictArea)
+  u64 batches_redone = 0;                                // batches settle() had to analyse again
   std::vector<PendingBatch> pending; std::vector<std::pair<u64*, size_t>> pinned_free; std::vector<ShapeEntry> shapes;
   u32* d_poison = nullptr; int speculate = 1;
   // optional per-kernel timing: a ring of event pairs, harvested lazily
@@ -157,14 +160,27 @@ struct TimedLaunch {                                     // a named range and, w
 };
 
 // Layout of the scratch block used by get_verdict and locate_hang.
-struct MiscLayout { size_t sus_a, sus_b, alerts, count, entered, done, frame, roots, tot, hang_out, total; };
+struct MiscLayout { size_t sus, keys, counts, alerts, entered, done, frame, roots, tot, hang_out, total; };
 MiscLayout misc_layout(u32 n_ranks, u32 max_n) {
   MiscLayout L; size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + std::max<size_t>(b, 1)); return o; };
-  L.sus_a = take(2ull * n_ranks * sizeof(ccld_suspect)); L.sus_b = take(2ull * n_ranks * sizeof(ccld_suspect));
-  L.alerts = take(CCLD_MAX_ALERTS_PER_WINDOW * sizeof(ccld_hang_alert)); L.count = take(16);
+  const size_t pieces = (n_ranks + VD_THREADS - 1) / VD_THREADS;
+  L.sus = take(2ull * n_ranks * sizeof(ccld_suspect)); L.keys = take(pieces * VD_KEYS * 8); L.counts = take(pieces * 4);
+  L.alerts = take(CCLD_MAX_ALERTS_PER_WINDOW * sizeof(ccld_hang_alert));
   L.entered = take(max_n); L.done = take(max_n); L.frame = take(max_n * 4ull); L.roots = take(max_n * 4ull);
   L.tot = take(max_n * 8ull); L.hang_out = take(sizeof(ccld_hang_verdict));
+  L.total = off;
+  return L;
+}
+
+// Layout of the pinned area the verdict kernels write to.
+struct VerdictArea { size_t rows, alerts, suspects, total; u32 sus_cap; };
+VerdictArea verdict_area(u32 n_comms, u32 n_ranks) {
+  VerdictArea L; size_t off = align_up(sizeof(VerdictHead));
+  auto take = [&](size_t b) { size_t o = off; off = align_up(off + b); return o; };
+  L.sus_cap = std::min<u32>(2 * n_ranks, VD_SUS_HOST);
+  L.rows = take((size_t)n_comms * sizeof(ccld_comm_verdict)); L.alerts = take(CCLD_MAX_ALERTS_PER_WINDOW * sizeof(ccld_hang_alert));
+  L.suspects = take((size_t)L.sus_cap * sizeof(ccld_suspect));
   L.total = off;
   return L;
 }
@@ -328,6 +344,7 @@ int settle(ccld_ctx* ctx) {
       if (it == ctx->windows.end()) { present = false; continue; }
       drop_results(it->second);
     }
+    ++ctx->batches_redone;
     if (!present) continue;                                // released in the meantime: nothing to analyse
     const int r = analyze_batch(ctx, b.first, b.n, b.now, false);
     if (r != CCLD_OK && rc == CCLD_OK) rc = r;
@@ -384,6 +401,7 @@ int ccld_destroy(ccld_ctx* ctx) {
   ctx->pool.put(ctx->reg_blk); ctx->pool.put(ctx->misc_blk);
   ctx->pool.clear();
   if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
+  if (ctx->h_verdict) cudaFreeHost(ctx->h_verdict);
   for (auto& b : ctx->pending) cudaFreeHost(b.h_tot);
   for (auto& f : ctx->pinned_free) cudaFreeHost(f.first);
   for (auto& sl : ctx->ring) for (int i = 0; i < TIMER_PAIRS; ++i) { cudaEventDestroy(sl.a[i]); cudaEventDestroy(sl.b[i]); }
@@ -716,13 +734,40 @@ extern "C" {
 int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
   NvtxRange nvtx_range("ccld_get_verdict");
   if (!ctx || !out) return CCLD_ERR_ARG;
-  WindowHost* w;
-  { int rc = find_analysed(ctx, window_id, &w); if (rc != CCLD_OK) return rc; }
+  WindowHost* w = nullptr;
   CK(cudaSetDevice(ctx->device));
-  cudaStream_t st = ctx->stream;
-  u64 cnt[C_COUNT];
-  CK(cudaMemcpyAsync(cnt, w->d.counters, sizeof cnt, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
+  // The kernels that gather the verdict are enqueued before batches still in doubt are settled: one wait serves both. In
+  // the rare case that a batch has to be analysed again (settle() counts those) what was gathered is gathered once more.
+  const VerdictHead* head = nullptr; VerdictArea area{};
+  u32 n_rows = 0;
+  char* m = (char*)ctx->misc_blk.p;
+  MiscLayout L{};
+  for (int attempt = 0; ; ++attempt) {
+    auto it = ctx->windows.find(window_id);
+    if (it == ctx->windows.end() || !it->second.analysed) { int rc = find_analysed(ctx, window_id, &w); if (rc != CCLD_OK) return rc; }
+    else w = &it->second;
+    area = verdict_area(ctx->reg.n_comms, ctx->n_ranks);
+    L = misc_layout(ctx->n_ranks, ctx->max_n);
+    if (!ctx->h_verdict) CK(cudaMallocHost((void**)&ctx->h_verdict, area.total));
+    head = (const VerdictHead*)ctx->h_verdict;
+    n_rows = std::min<u32>((u32)w->totals[T_ROWS], out->comm_rows ? out->comm_rows_cap : 0);
+    VerdictArgs A;
+    A.counters = w->d.counters; A.rows = w->d.comm_rows; A.n_rows = n_rows; A.alerts = w->d.alerts;
+    A.keys = (u64*)(m + L.keys); A.counts = (u32*)(m + L.counts);
+    A.head = (VerdictHead*)ctx->h_verdict; A.rows_out = (ccld_comm_verdict*)(ctx->h_verdict + area.rows);
+    A.alerts_out = (ccld_hang_alert*)(ctx->h_verdict + area.alerts);
+    A.sus_host = (ccld_suspect*)(ctx->h_verdict + area.suspects); A.sus_host_cap = area.sus_cap; A.sus_dev = (ccld_suspect*)(m + L.sus);
+    const u32 pieces = (ctx->n_ranks + VD_THREADS - 1) / VD_THREADS;
+    k_verdict_collect<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg, ctx->dp);
+    if (pieces > 1) k_verdict_merge<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(ctx->stream));
+    const u64 redone = ctx->batches_redone;
+    { int rc = settle(ctx); if (rc != CCLD_OK) return rc; }
+    if (ctx->batches_redone == redone) break;
+    if (attempt > 2) return fail(ctx, CCLD_ERR_CUDA, "internal: a settled batch changed again");
+  }
+  const u64* cnt = head->counters;
   out->n_records = w->n_rec; out->n_groups = w->totals[T_GROUPS]; out->n_slots = w->totals[T_SLOTS];
   out->n_rejected = w->n_rec - cnt[C_PRESENT]; out->n_complete = cnt[C_COMPLETE]; out->n_incomplete = cnt[C_INCOMPLETE];
   out->n_barrier = cnt[C_BARRIER]; out->n_analysed = cnt[C_ANALYSED]; out->n_flag_skew = cnt[C_FLAG_SKEW]; out->n_flag_dur = cnt[C_FLAG_DUR];
@@ -731,38 +776,19 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
   if (!w->totals[T_FAILED] && w->n_rec - cnt[C_PRESENT] != cnt[C_REJECTED]) err |= CCLD_E_DUPLICATE;   // a slot was written twice
   out->error_bits = err;
   out->n_comm_rows_total = (u32)w->totals[T_ROWS];
-  const u32 n_rows = std::min<u32>(out->n_comm_rows_total, out->comm_rows ? out->comm_rows_cap : 0);
-  if (n_rows) CK(cudaMemcpyAsync(out->comm_rows, w->d.comm_rows, n_rows * sizeof(ccld_comm_verdict), cudaMemcpyDeviceToHost, st));
-  char* m = (char*)ctx->misc_blk.p;
-  const MiscLayout L = misc_layout(ctx->n_ranks, ctx->max_n);
-  ccld_suspect* sus_a = (ccld_suspect*)(m + L.sus_a); ccld_suspect* sus_b = (ccld_suspect*)(m + L.sus_b);
-  ccld_hang_alert* al_b = (ccld_hang_alert*)(m + L.alerts);
-  u32* d_count = (u32*)(m + L.count);
+  if (n_rows) std::memcpy(out->comm_rows, ctx->h_verdict + area.rows, n_rows * sizeof(ccld_comm_verdict));
   // hang alerts, ordered by (communicator, seq)
   out->n_alerts_total = (u32)std::min<u64>(cnt[C_ALERTS], 0xFFFFFFFFull);
-  const u32 n_al_dev = std::min<u32>(out->n_alerts_total, CCLD_MAX_ALERTS_PER_WINDOW);
-  const u32 n_al = std::min<u32>(n_al_dev, out->alerts ? out->alerts_cap : 0);
-  if (n_al) {
-    k_rank_sort_alerts<<<(n_al_dev + 127) / 128, 128, 0, st>>>(w->d.alerts, n_al_dev, al_b, ctx->reg);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(out->alerts, al_b, n_al * sizeof(ccld_hang_alert), cudaMemcpyDeviceToHost, st));
-  }
+  const u32 n_al = std::min<u32>(std::min<u32>(out->n_alerts_total, CCLD_MAX_ALERTS_PER_WINDOW), out->alerts ? out->alerts_cap : 0);
+  if (n_al) std::memcpy(out->alerts, ctx->h_verdict + area.alerts, n_al * sizeof(ccld_hang_alert));
   // cumulative suspects
-  const u32 sus_cap = 2 * ctx->n_ranks;
-  u32 n_sus = 0;
-  CK(cudaMemsetAsync(d_count, 0, 4, st));
-  k_suspects<<<(ctx->n_ranks + 255) / 256, 256, 0, st>>>(ctx->reg, ctx->dp, sus_a, sus_cap, d_count);
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(&n_sus, d_count, 4, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  out->n_suspects_total = n_sus;
-  const u32 n_out = std::min<u32>(n_sus, out->suspects ? out->suspects_cap : 0);
-  if (n_out) {
-    k_rank_sort_suspects<<<(n_sus + 127) / 128, 128, 0, st>>>(sus_a, n_sus, sus_b);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(out->suspects, sus_b, n_out * sizeof(ccld_suspect), cudaMemcpyDeviceToHost, st));
+  out->n_suspects_total = head->n_suspects;
+  const u32 n_out = std::min<u32>(head->n_suspects, out->suspects ? out->suspects_cap : 0);
+  if (n_out && head->n_suspects <= area.sus_cap) std::memcpy(out->suspects, ctx->h_verdict + area.suspects, n_out * sizeof(ccld_suspect));
+  else if (n_out) {
+    CK(cudaMemcpyAsync(out->suspects, m + L.sus, n_out * sizeof(ccld_suspect), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
   }
-  CK(cudaStreamSynchronize(st));
   if (cnt[C_INTERNAL]) return fail(ctx, CCLD_ERR_CUDA, "internal: slot index out of range");
   if (err & CCLD_E_UNKNOWN_COMM) return fail(ctx, CCLD_ERR_UNKNOWN_COMM, "record of an unregistered communicator");
   if (err & CCLD_E_NOT_MEMBER) return fail(ctx, CCLD_ERR_NOT_MEMBER, "record of a rank that is not a member of its communicator");
@@ -830,7 +856,7 @@ int ccld_locate_hangs(ccld_ctx* ctx, uint32_t window_id, ccld_hang_alert* alerts
   char* m = (char*)ctx->misc_blk.p;
   const MiscLayout L = misc_layout(ctx->n_ranks, ctx->max_n);
   ccld_hang_alert* al_b = (ccld_hang_alert*)(m + L.alerts);
-  k_rank_sort_alerts<<<(n_dev + 127) / 128, 128, 0, st>>>(w->d.alerts, n_dev, al_b, ctx->reg);
+  k_order_alerts<<<1, VD_THREADS, 0, st>>>(w->d.counters, w->d.alerts, al_b, ctx->reg);
   CK(cudaGetLastError());
   std::vector<ccld_hang_alert> al(n);
   CK(cudaMemcpyAsync(al.data(), al_b, n * sizeof(ccld_hang_alert), cudaMemcpyDeviceToHost, st));

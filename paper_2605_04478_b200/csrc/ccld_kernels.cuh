@@ -15,7 +15,7 @@
 //   k_window_rounds Eq. 2 per (communicator, window): round counts, selected round, location candidates
 //   k_window_decide Eq. 1, 3, 4 per communicator, windows in order: baseline state, class, slow location
 //   k_hang_locate   hang decision tree over presence / completion / progress counters
-//   k_suspects, k_rank_sort_*  suspect list and ordered output lists
+// The suspect list and the ordered output lists are in ccld_verdict.cuh.
 #pragma once
 #include "ccld_device.cuh"
 
@@ -1318,53 +1318,3 @@ __global__ void __launch_bounds__(1024) k_hang_locate_many(const WinDesc* __rest
 
 }  // namespace ccld
 #include "ccld_tree.cuh"
-namespace ccld {
-
-// ------------------------------------------------------------------------------------------------
-// suspects and ordered lists
-// ------------------------------------------------------------------------------------------------
-__global__ void k_suspects(Registry R, Params P, ccld_suspect* __restrict__ out, u32 cap, u32* __restrict__ count) {
-  const u32 r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R.n_ranks) return;
-  const u32 ops = R.ops[r];
-  if (ops == 0) return;
-  const u32 cnt = R.bw_cnt[r];
-  const double bw = cnt ? R.bw_sum[r] / (double)cnt : 0.0;
-  const u32 v[2] = {R.votes[(u64)r * 4 + 0], R.votes[(u64)r * 4 + 2]};
-  for (u32 kind = 1; kind <= 2; ++kind) {
-    if ((u64)v[kind - 1] * 1000u >= (u64)P.vote_rep_milli * ops) {
-      const u32 k = atomicAdd(count, 1u);
-      if (k < cap) { ccld_suspect s; s.kind = kind; s.rank = r; s.votes = v[kind - 1]; s.ops = ops; s.mean_busbw = bw; out[k] = s; }
-    }
-  }
-}
-
-// Rank-by-counting sort of short lists: element i goes to the number of elements that precede it.
-__global__ void k_rank_sort_suspects(const ccld_suspect* __restrict__ in, u32 n, ccld_suspect* __restrict__ out) {
-  const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const ccld_suspect a = in[i];
-  u32 before = 0;
-  for (u32 j = 0; j < n; ++j) {
-    const ccld_suspect b = in[j];
-    const bool lt = b.kind != a.kind ? b.kind < a.kind : (b.votes != a.votes ? b.votes > a.votes : b.rank < a.rank);
-    before += lt;
-  }
-  out[before] = a;
-}
-
-__global__ void k_rank_sort_alerts(const ccld_hang_alert* __restrict__ in, u32 n, ccld_hang_alert* __restrict__ out, Registry R) {
-  const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const ccld_hang_alert a = in[i];
-  const u32 ca = comm_lookup(R, a.comm);
-  u32 before = 0;
-  for (u32 j = 0; j < n; ++j) {
-    const ccld_hang_alert b = in[j];
-    const u32 cb = comm_lookup(R, b.comm);
-    before += cb != ca ? cb < ca : b.seq < a.seq;
-  }
-  out[before] = a;
-}
-
-}  // namespace ccld

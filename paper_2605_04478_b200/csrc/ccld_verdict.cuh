@@ -1,0 +1,153 @@
+// What ccld_get_verdict hands out, gathered on the device and written straight into pinned host memory (sm_100a).
+//
+//   k_verdict_collect  a CTA per 1,024 ranks: which of its ranks are suspects (vote shares against the threshold), as one
+//                      64-bit key each that orders like the list - kind, votes descending, rank -, sorted in shared
+//                      memory; the CTAs also copy the window's communicator rows and counters, the first one orders the
+//                      hang alerts. A job of up to 1,024 ranks is done after this launch.
+//   k_verdict_merge    more than 1,024 ranks: the sorted pieces become one list. A key's place is its place in its own
+//                      piece plus, for every other piece, the number of keys before it (a binary search).
+//
+// Bound by latency: the inputs are a few hundred KB at most. One launch (two for larger jobs), no copy and one wait of the
+// host per verdict, where a copy of the counters, a launch, a copy of the count, a launch and two more copies with three
+// waits used to be; the rank-by-counting sort of an 8,000-suspect list over global memory took 243 us, the sorted pieces
+// with the merge take under 10 (communicators of four ranks, whose MAD rests on two values, name that many).
+#pragma once
+#include "ccld_kernels.cuh"
+
+namespace ccld {
+
+constexpr int VD_THREADS = 1024;             // ranks per CTA
+constexpr int VD_KEYS = 2 * VD_THREADS;      // a rank is on the list at most twice
+constexpr u32 VD_SUS_HOST = 65536;           // suspects the pinned area holds at most; longer lists stay in device memory
+
+struct VerdictHead { u64 counters[C_COUNT]; u32 n_suspects, pad; };
+struct VerdictArgs {
+  const u64* counters;                       // the window's
+  const ccld_comm_verdict* rows; u32 n_rows; // (null, 0): nothing to copy
+  const ccld_hang_alert* alerts;
+  u64* keys; u32* counts;                    // device scratch: [CTAs][VD_KEYS] sorted keys, [CTAs] how many
+  VerdictHead* head;                         // pinned: counters and number of suspects
+  ccld_comm_verdict* rows_out;               // pinned [n_rows]
+  ccld_hang_alert* alerts_out;               // [CCLD_MAX_ALERTS_PER_WINDOW]
+  ccld_suspect* sus_host; u32 sus_host_cap;  // pinned; lists longer than that go to sus_dev
+  ccld_suspect* sus_dev;
+};
+
+__device__ __forceinline__ u64 suspect_key(u32 kind, u32 votes, u32 rank) { return ((u64)(kind - 1) << 54) | ((u64)(~votes) << 22) | rank; }
+static_assert(CCLD_MAX_RANK_ID <= (1u << 22), "a rank id fits its field of the key");
+__device__ __forceinline__ ccld_suspect suspect_of(const Registry& R, u64 key) {
+  ccld_suspect s;
+  s.kind = (u32)(key >> 54) + 1; s.votes = ~(u32)(key >> 22); s.rank = (u32)key & ((1u << 22) - 1);
+  s.ops = R.ops[s.rank];
+  const u32 cnt = R.bw_cnt[s.rank];
+  s.mean_busbw = cnt ? R.bw_sum[s.rank] / (double)cnt : 0.0;
+  return s;
+}
+
+// The alerts of a window in the order they are listed: registration order of the communicator, then op counter (then the
+// place in the unordered list: an op raises one alert). One CTA; s_key holds CCLD_MAX_ALERTS_PER_WINDOW keys.
+__device__ __forceinline__ void order_alerts(const Registry& R, const ccld_hang_alert* __restrict__ in, u32 n, ccld_hang_alert* __restrict__ out, u64* s_key) {
+  for (u32 i = threadIdx.x; i < n; i += blockDim.x) s_key[i] = ((u64)comm_lookup(R, in[i].comm) << 32) | in[i].seq;
+  __syncthreads();
+  for (u32 i = threadIdx.x; i < n; i += blockDim.x) {
+    const u64 k = s_key[i];
+    u32 before = 0;
+    for (u32 j = 0; j < n; ++j) before += (s_key[j] < k || (s_key[j] == k && j < i)) ? 1u : 0u;
+    out[before] = in[i];
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(VD_THREADS) k_verdict_collect(VerdictArgs A, Registry R, Params P) {
+  __shared__ u64 s_key[VD_KEYS];
+  __shared__ u32 s_n;
+  const u32 lane = threadIdx.x & 31;
+  // communicator rows, all CTAs: whole 8-byte words
+  {
+    const u64 words = (u64)A.n_rows * (sizeof(ccld_comm_verdict) / 8);
+    static_assert(sizeof(ccld_comm_verdict) % 8 == 0, "rows are copied as 8-byte words");
+    const u64* src = (const u64*)A.rows; u64* dst = (u64*)A.rows_out;
+    for (u64 i = (u64)blockIdx.x * VD_THREADS + threadIdx.x; i < words; i += (u64)gridDim.x * VD_THREADS) dst[i] = src[i];
+  }
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < C_COUNT) A.head->counters[threadIdx.x] = A.counters[threadIdx.x];
+    const u64 n_al = A.counters[C_ALERTS];
+    if (n_al) order_alerts(R, A.alerts, n_al < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n_al : CCLD_MAX_ALERTS_PER_WINDOW, A.alerts_out, s_key);
+  }
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
+  const u32 r = blockIdx.x * VD_THREADS + threadIdx.x;
+  u32 ops = 0; uint4 v = make_uint4(0, 0, 0, 0);
+  if (r < R.n_ranks) { ops = R.ops[r]; v = *reinterpret_cast<const uint4*>(R.votes + (u64)r * 4); }
+#pragma unroll
+  for (u32 kind = 1; kind <= 2; ++kind) {
+    const u32 votes = kind == 1 ? v.x : v.z;
+    const bool is = ops != 0 && (u64)votes * 1000u >= (u64)P.vote_rep_milli * ops;
+    const u32 bal = __ballot_sync(0xFFFFFFFFu, is);
+    u32 base = 0;
+    if (lane == 0 && bal) base = atomicAdd(&s_n, (u32)__popc(bal));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    if (is) s_key[base + __popc(bal & ((1u << lane) - 1u))] = suspect_key(kind, votes, r);
+  }
+  __syncthreads();
+  // bitonic sort over the next power of two
+  const u32 n = s_n;
+  u32 n_pad = 1; while (n_pad < n) n_pad <<= 1;
+  for (u32 i = n + threadIdx.x; i < n_pad; i += VD_THREADS) s_key[i] = U64_MAX_;
+  __syncthreads();
+  for (u32 k = 2; k <= n_pad; k <<= 1) {
+    for (u32 j = k >> 1; j > 0; j >>= 1) {
+      const u32 q = threadIdx.x;                                // VD_KEYS / 2 pairs at most: one per thread
+      if (q < n_pad >> 1) {
+        const u32 i = ((q & ~(j - 1)) << 1) | (q & (j - 1)), l = i | j;
+        const u64 a = s_key[i], b = s_key[l];
+        if ((a > b) == ((i & k) == 0)) { s_key[i] = b; s_key[l] = a; }
+      }
+      __syncthreads();
+    }
+  }
+  if (gridDim.x == 1) {
+    ccld_suspect* dst = n <= A.sus_host_cap ? A.sus_host : A.sus_dev;
+    for (u32 i = threadIdx.x; i < n; i += VD_THREADS) dst[i] = suspect_of(R, s_key[i]);
+    if (threadIdx.x == 0) A.head->n_suspects = n;
+  } else {
+    for (u32 i = threadIdx.x; i < n; i += VD_THREADS) A.keys[(u64)blockIdx.x * VD_KEYS + i] = s_key[i];
+    if (threadIdx.x == 0) A.counts[blockIdx.x] = n;
+  }
+}
+
+__global__ void __launch_bounds__(VD_THREADS) k_verdict_merge(VerdictArgs A, Registry R) {
+  __shared__ u32 s_tot;
+  if (threadIdx.x == 0) s_tot = 0;
+  __syncthreads();
+  u32 t = 0;
+  for (u32 o = threadIdx.x; o < gridDim.x; o += VD_THREADS) t += A.counts[o];
+  t = __reduce_add_sync(0xFFFFFFFFu, t);
+  if ((threadIdx.x & 31) == 0 && t) atomicAdd(&s_tot, t);
+  __syncthreads();
+  const u32 total = s_tot, n = A.counts[blockIdx.x];
+  if (blockIdx.x == 0 && threadIdx.x == 0) A.head->n_suspects = total;
+  ccld_suspect* dst = total <= A.sus_host_cap ? A.sus_host : A.sus_dev;
+  const u64* mine = A.keys + (u64)blockIdx.x * VD_KEYS;
+  for (u32 i = threadIdx.x; i < n; i += VD_THREADS) {
+    const u64 key = mine[i];
+    u32 pos = i;
+    for (u32 o = 0; o < gridDim.x; ++o) {
+      if (o == blockIdx.x) continue;
+      const u64* other = A.keys + (u64)o * VD_KEYS;
+      u32 lo = 0, hi = A.counts[o];                             // keys are unique: how many of the other piece are smaller
+      while (lo < hi) { const u32 mid = (lo + hi) >> 1; if (other[mid] < key) lo = mid + 1; else hi = mid; }
+      pos += lo;
+    }
+    dst[pos] = suspect_of(R, key);
+  }
+}
+
+// the ordered alerts alone, for the hang sweep
+__global__ void __launch_bounds__(VD_THREADS) k_order_alerts(const u64* __restrict__ counters, const ccld_hang_alert* __restrict__ in, ccld_hang_alert* __restrict__ out, Registry R) {
+  __shared__ u64 s_key[CCLD_MAX_ALERTS_PER_WINDOW];
+  const u64 n = counters[C_ALERTS];
+  order_alerts(R, in, n < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n : CCLD_MAX_ALERTS_PER_WINDOW, out, s_key);
+}
+
+}  // namespace ccld
