@@ -73,7 +73,7 @@ constexpr u32 RANK_TAB_OVERFLOW = 0xFFFFFFFEu;
 constexpr u32 RANK_TAB_POS_BITS = 13;  // positions < CCLD_MAX_COMM_SIZE = 8192
 
 // Which op counters a communicator covers in a window and where its groups / slots start.
-// tile0 / n_units: where the communicator's TileSum entries start (index into its summary array) and how many it has.
+// tile0 / n_units: where the communicator's TileSum entries start (index into the window's part of its summary array) and how many it has.
 struct RangeRow { u32 seq_lo, n_seq, row_idx, n; u64 group0, slot0; u32 tile0, n_units; };
 
 enum { C_REJECTED = 0, C_COMPLETE, C_INCOMPLETE, C_BARRIER, C_ANALYSED, C_FLAG_SKEW, C_FLAG_DUR, C_MISMATCH,
@@ -106,13 +106,14 @@ struct WinDesc {
   const u32 *send_chg, *recv_chg;   // may be null
   u64 n_rec;
   u64 slot_cap;                      // plan fails the window if it would need more slots
-  u32 cta0, n_cta;                   // this window's CTAs in the record-streaming grids
   u32 *rmin, *rmax;                  // [n_comms] op counter range seen
   RangeRow* ranges;                  // [n_comms]
   uint4* srow;                       // [n_comms] scatter rows: first slot low, high, op counters covered (0 = nothing to place), first op counter
   uint4* rent;                       // [n_ranks][RANK_TAB_K] a rank's inline pairs resolved for this window: (communicator id, op counters
                                      //   covered (0: unused), first op counter, first slot of the member's column); 32-bit slots only
   u64* totals;                       // [T_COUNT]
+  uint2* chunks;                     // [CHUNK_MAX + 1] first CTA (x) and first warp-tile (y) of every chunk, relative to the window
+  u64* totals_host;                  // [T_COUNT] the totals once more, in pinned host memory
   const u64* expect;                 // [T_COUNT] totals the host sized this window's results for without waiting (null: it waited)
   u32* poison;                       // set once a window's layout differs from what the host expected: every window planned later gives up too
   u64* counters;                     // [C_COUNT]
@@ -128,7 +129,7 @@ struct WinDesc {
   ccld_hang_alert* alerts;           // [CCLD_MAX_ALERTS_PER_WINDOW]
   u32 base[B_COUNT];                 // this window's first entry in the batch-wide lists (B_*)
   u32 pad;
-  TileSum* tsum[3];                  // tile summaries of the whole batch: fused classes, class 2, class 3
+  TileSum* tsum[3];                  // this window's tile summaries: fused classes, class 2, class 3
 };
 
 enum { GI_E_MIN = 0, GI_ARRIVAL_SKEW, GI_T_MAX, GI_T_MIN, GI_SPAN, GI_MED_SKEW, GI_MAD_SKEW, GI_MED_DUR, GI_MAD_DUR, GI_COUNT };

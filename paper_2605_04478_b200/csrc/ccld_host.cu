@@ -78,7 +78,8 @@ struct WindowHost {
 
 // A batch that was enqueued on totals the host expected instead of waiting for the plan: its actual totals arrive in
 // pinned memory behind the batch's kernels and are checked at the next call that synchronizes anyway.
-struct PendingBatch { u32 first = 0, n = 0; i64 now = 0; u64* h_tot = nullptr; size_t h_bytes = 0; };
+// A batch that waited is listed only for its pinned block, which its last descriptor copy still reads.
+struct PendingBatch { u32 first = 0, n = 0; i64 now = 0; u64* h_tot = nullptr; size_t h_bytes = 0; bool speculative = false; };
 // Totals of the last batches that were planned with a wait, by shape (record count of every window).
 struct ShapeEntry { std::vector<u64> n_rec; std::vector<u64> totals; };
 constexpr size_t SHAPE_CACHE = 4;
@@ -97,7 +98,6 @@ struct ccld_ctx {
   const TreeRef* d_trees = nullptr; u32 n_trees = 0;     // tree communicators whose layers are known
   std::map<u32, WindowHost> windows;
   Pool pool; std::string err;
-  u64* h_pinned = nullptr; size_t h_pinned_bytes = 0;
   char* h_verdict = nullptr;                             // pinned area of ccld_get_verdict (VerdictArea)
   u64 batches_redone = 0;                                // batches settle() had to analyse again
   std::vector<PendingBatch> pending; std::vector<std::pair<u64*, size_t>> pinned_free; std::vector<ShapeEntry> shapes;
@@ -116,15 +116,6 @@ int fail(ccld_ctx* c, int code, const std::string& msg) { if (c) c->err = msg; r
   do { cudaError_t e_ = (call);                                                                    \
        if (e_ != cudaSuccess) return fail(ctx, e_ == cudaErrorMemoryAllocation ? CCLD_ERR_NOMEM : CCLD_ERR_CUDA, \
                                           std::string(#call) + ": " + cudaGetErrorString(e_)); } while (0)
-
-int ensure_pinned(ccld_ctx* ctx, size_t bytes) {
-  if (ctx->h_pinned_bytes >= bytes) return CCLD_OK;
-  if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
-  ctx->h_pinned = nullptr; ctx->h_pinned_bytes = 0;
-  CK(cudaMallocHost((void**)&ctx->h_pinned, bytes));
-  ctx->h_pinned_bytes = bytes;
-  return CCLD_OK;
-}
 
 // Adds the elapsed times of a slot's finished event pairs to the sums (waits for the last one).
 void timer_harvest(ccld_ctx* ctx, TimerSlot& s) {
@@ -317,7 +308,8 @@ int settle(ccld_ctx* ctx) {
   CK(cudaSetDevice(ctx->device));
   CK(cudaStreamSynchronize(ctx->stream));
   std::vector<PendingBatch> todo;
-  todo.swap(ctx->pending);
+  for (PendingBatch& b : ctx->pending) { if (b.speculative) todo.push_back(b); else ctx->pinned_free.emplace_back(b.h_tot, b.h_bytes); }
+  ctx->pending.clear();
   bool failed = false;
   int rc = CCLD_OK;
   for (PendingBatch& b : todo) {
@@ -400,7 +392,6 @@ int ccld_destroy(ccld_ctx* ctx) {
   ctx->windows.clear();
   ctx->pool.put(ctx->reg_blk); ctx->pool.put(ctx->misc_blk);
   ctx->pool.clear();
-  if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
   if (ctx->h_verdict) cudaFreeHost(ctx->h_verdict);
   for (auto& b : ctx->pending) cudaFreeHost(b.h_tot);
   for (auto& f : ctx->pinned_free) cudaFreeHost(f.first);
@@ -570,24 +561,37 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   // ---- plan block: descriptors, op-counter ranges, layout rows, totals, counters ----
   size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + b); return o; };
-  const size_t o_desc = take(B * sizeof(WinDesc)), o_rmin = take((size_t)B * nc * 4), o_rmax = take((size_t)B * nc * 4),
-               o_rng = take((size_t)B * nc * sizeof(RangeRow)), o_srow = take((size_t)B * nc * sizeof(uint4)), o_rent = take((size_t)B * ctx->n_ranks * RANK_TAB_K * sizeof(uint4)), o_tot = take((size_t)B * T_COUNT * 8), o_cnt = take((size_t)B * C_COUNT * 8),
-               o_zero_end = off, o_exp = take(expect ? (size_t)B * T_COUNT * 8 : 0);
+  const size_t tot_bytes = (size_t)B * T_COUNT * 8;
+  const size_t o_desc = take(B * sizeof(WinDesc)), o_exp = take(expect ? tot_bytes : 0), up_bytes = off,      // what comes from the host
+               o_zero = off, o_rmax = take((size_t)B * nc * 4), o_cnt = take((size_t)B * C_COUNT * 8), o_defn = take(16), o_zero_end = off,
+               o_rmin = take((size_t)B * nc * 4), o_rng = take((size_t)B * nc * sizeof(RangeRow)), o_srow = take((size_t)B * nc * sizeof(uint4)),
+               o_rent = take((size_t)B * ctx->n_ranks * RANK_TAB_K * sizeof(uint4)), o_tot = take(tot_bytes), o_chunk = take((size_t)B * (CHUNK_MAX + 1) * sizeof(uint2));
   cudaError_t e;
   Block pb = ctx->pool.get(off, &e);
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "plan allocation failed");
   auto plan_blk = std::make_shared<Shared>(&ctx->pool, pb);
   char* pbase = (char*)pb.p;
-  std::vector<WinDesc> hd(B);
+  // pinned: the totals the layout finds, then the descriptors and expected totals on their way to the device. It belongs to
+  // the batch until the next call that synchronizes.
+  PendingBatch pbatch; pbatch.first = first_window; pbatch.n = B; pbatch.now = now_ns; pbatch.speculative = expect != nullptr;
+  pbatch.h_tot = pinned_get(ctx, align_up(tot_bytes) + up_bytes, &pbatch.h_bytes);
+  if (!pbatch.h_tot) return fail(ctx, CCLD_ERR_NOMEM, "pinned allocation failed");
+  struct Guard {                                           // whatever way the call ends, the batch's pinned block is accounted for
+    ccld_ctx* ctx; PendingBatch& b; bool queued = false;
+    ~Guard() { if (!queued) { cudaStreamSynchronize(ctx->stream); ctx->pinned_free.emplace_back(b.h_tot, b.h_bytes); } }
+  } guard{ctx, pbatch};
+  char* const h_up = (char*)pbatch.h_tot + align_up(tot_bytes);
+  WinDesc* const hd = (WinDesc*)h_up;
   u64 cta = 0;
   for (u32 k = 0; k < B; ++k) {
     WinDesc d = ws[k]->d;
     d.slot_cap = 2 * d.n_rec + ctx->sum_n;
-    d.n_cta = (u32)((d.n_rec + REC_PER_CTA - 1) / REC_PER_CTA); d.cta0 = 0; cta = std::max<u64>(cta, d.n_cta);
+    cta = std::max<u64>(cta, (d.n_rec + REC_PER_CTA - 1) / REC_PER_CTA);
     d.rmin = (u32*)(pbase + o_rmin) + (size_t)k * nc; d.rmax = (u32*)(pbase + o_rmax) + (size_t)k * nc;
     d.ranges = (RangeRow*)(pbase + o_rng) + (size_t)k * nc; d.srow = (uint4*)(pbase + o_srow) + (size_t)k * nc;
     d.rent = (uint4*)(pbase + o_rent) + (size_t)k * ctx->n_ranks * RANK_TAB_K;
     d.totals = (u64*)(pbase + o_tot) + (size_t)k * T_COUNT; d.counters = (u64*)(pbase + o_cnt) + (size_t)k * C_COUNT;
+    d.chunks = (uint2*)(pbase + o_chunk) + (size_t)k * (CHUNK_MAX + 1); d.totals_host = pbatch.h_tot + (size_t)k * T_COUNT;
     d.expect = expect ? (const u64*)(pbase + o_exp) + (size_t)k * T_COUNT : nullptr; d.poison = ctx->d_poison;
     d.n_groups = d.n_slots = 0; d.perm = nullptr; d.flags = nullptr; d.skey = d.dkey = nullptr; d.gi64 = nullptr; d.gu32 = nullptr; d.gbw = nullptr;
     d.comm_rows = nullptr; d.alerts = nullptr;
@@ -595,15 +599,16 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     d.pad = 0; d.tsum[0] = d.tsum[1] = d.tsum[2] = nullptr;
     hd[k] = d;
   }
+  if (expect) std::memcpy(h_up + o_exp, expect->totals.data(), tot_bytes);
   if (cta > 0x7FFFFFFFull) return fail(ctx, CCLD_ERR_CAPACITY, "batch too large for one launch");
   WinDesc* d_desc = (WinDesc*)(pbase + o_desc);
   TimerSlot* ts = timer_begin(ctx);
-  auto start_plan = [&]() -> cudaError_t {               // clears the plan block, uploads the descriptors, runs the range pass and the layout
-    cudaError_t r = cudaMemsetAsync(pbase, 0, o_zero_end, st);
-    if (r == cudaSuccess) r = cudaMemsetAsync(pbase + o_rmin, 0xFF, (size_t)B * nc * 4, st);
-    if (r == cudaSuccess && expect) r = cudaMemcpyAsync(pbase + o_exp, expect->totals.data(), (size_t)B * T_COUNT * 8, cudaMemcpyHostToDevice, st);
-    if (r == cudaSuccess) r = cudaMemcpyAsync(d_desc, hd.data(), B * sizeof(WinDesc), cudaMemcpyHostToDevice, st);
-    if (r != cudaSuccess) return r;
+  auto start_plan = [&](u32 fill_ctas) -> cudaError_t {    // uploads the descriptors, sets the start values, runs the range pass and the layout
+    BeginArgs ba;
+    ba.desc_host = (const u32*)h_up; ba.desc = (u32*)(pbase + o_desc); ba.desc_words = up_bytes / 4;
+    ba.rmin = (u32*)(pbase + o_rmin); ba.n_rmin = (u64)B * nc; ba.zero = (u32*)(pbase + o_zero); ba.n_zero = (o_zero_end - o_zero) / 4;
+    const u64 most = std::max<u64>(std::max<u64>(ba.desc_words, ba.n_rmin), ba.n_zero);
+    k_begin<<<(u32)std::min<u64>((most + BEGIN_THREADS - 1) / BEGIN_THREADS, 2ull * ctx->n_sms), BEGIN_THREADS, 0, st>>>(ba);
     if (cta > 0) {
       // enough CTAs to fill the device several times over, then as many blocks per CTA as that leaves
       const u64 want = 32ull * ctx->n_sms;
@@ -611,23 +616,24 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
       TimedLaunch tl(ts, 0, st);
       k_seq_range<<<dim3((u32)((cta + per - 1) / per), B), REC_THREADS, range_smem_bytes(nc), st>>>(d_desc, ctx->reg, per);
     }
-    { TimedLaunch tl(ts, 1, st); k_plan<<<B, PLAN_THREADS, 0, st>>>(d_desc, ctx->reg, PlanLists{nullptr, nullptr, nullptr, nullptr}, 0); }
+    { TimedLaunch tl(ts, 1, st); k_layout<<<dim3(1 + fill_ctas, B), LAYOUT_THREADS, 0, st>>>(d_desc, ctx->reg, fill_ctas != 0); }
     return cudaGetLastError();
   };
   const u64* tot = nullptr;                                // [B][T_COUNT] totals the results are sized from
+  std::vector<u64> found;
   if (!expect) {
-    CK(start_plan());
-    { int rc = ensure_pinned(ctx, (size_t)B * T_COUNT * 8); if (rc != CCLD_OK) return rc; }
-    CK(cudaMemcpyAsync(ctx->h_pinned, pbase + o_tot, (size_t)B * T_COUNT * 8, cudaMemcpyDeviceToHost, st));
+    CK(start_plan(0));
     CK(cudaStreamSynchronize(st));
-    tot = ctx->h_pinned;
+    found.assign(pbatch.h_tot, pbatch.h_tot + (size_t)B * T_COUNT);
+    tot = found.data();
   } else tot = expect->totals.data();
 
   // ---- result block: sized from the totals ----
   off = 0;
-  u64 total_slots = 0, n_list[B_COUNT] = {0, 0, 0, 0, 0};       // batch-wide list lengths (B_*)
+  u64 total_slots = 0, max_slots = 0, n_list[B_COUNT] = {0, 0, 0, 0, 0};       // batch-wide list lengths (B_*)
+  u32 chunk_ctas = 1;
   const int t_of[B_COUNT] = {T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3};
-  for (u32 k = 0; k < B; ++k) { const u64* t = tot + (size_t)k * T_COUNT; total_slots += t[T_SLOTS]; }
+  for (u32 k = 0; k < B; ++k) { const u64* t = tot + (size_t)k * T_COUNT; total_slots += t[T_SLOTS]; max_slots = std::max(max_slots, t[T_SLOTS]); chunk_ctas = std::max(chunk_ctas, (u32)t[T_CHUNKS]); }
   const size_t o_perm = take(total_slots * 4 + ALIGN);
   std::vector<size_t> o_flags(B), o_gi(B), o_gu(B), o_gb(B), o_rows(B), o_al(B), perm_off(B);
   { size_t po = 0;
@@ -646,7 +652,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   // groups the fused kernel may set aside for the deferred kernel: at most every group of the batch
   u64 total_groups = 0;
   for (u32 k = 0; k < B; ++k) total_groups += tot[(size_t)k * T_COUNT + T_GROUPS];
-  const size_t o_defn = take(16), o_def = take(n_list[B_FCTA] ? total_groups * 8 : 0),
+  const size_t o_def = take(n_list[B_FCTA] ? total_groups * 8 : 0),
                o_def3 = take(n_list[B_T3] * (size_t)LARGE_SEQS * 8),          // likewise for the kernel of the largest communicators
                o_lgrp = take(n_list[B_T3] * (size_t)LARGE_SEQS * sizeof(LargeGroup)),
                o_skey = take(n_list[B_T3] ? total_slots * 4 : 0), o_dkey = take(n_list[B_T3] ? total_slots * 4 : 0);
@@ -662,31 +668,40 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     if (n_list[B_T3]) { d.skey = (u32*)(rbase + o_skey + perm_off[k]); d.dkey = (u32*)(rbase + o_dkey + perm_off[k]); }
     d.gi64 = (i64*)(rbase + o_gi[k]); d.gu32 = (u32*)(rbase + o_gu[k]); d.gbw = (double*)(rbase + o_gb[k]);
     d.comm_rows = (ccld_comm_verdict*)(rbase + o_rows[k]); d.alerts = (ccld_hang_alert*)(rbase + o_al[k]);
-    d.tsum[0] = (TileSum*)(rbase + o_fsum); d.tsum[1] = (TileSum*)(rbase + o_s2); d.tsum[2] = (TileSum*)(rbase + o_s3);
+    d.tsum[0] = (TileSum*)(rbase + o_fsum) + d.base[B_FSUM]; d.tsum[1] = (TileSum*)(rbase + o_s2) + d.base[B_T2]; d.tsum[2] = (TileSum*)(rbase + o_s3) + d.base[B_T3];
   }
-  if (expect) CK(start_plan());                            // descriptors already complete: nothing was waited for
-  else CK(cudaMemcpyAsync(d_desc, hd.data(), B * sizeof(WinDesc), cudaMemcpyHostToDevice, st));
-  if (total_slots) CK(cudaMemsetAsync(rbase + o_perm, 0xFF, total_slots * 4, st));
+  if (expect) {
+    // Descriptors already complete: nothing was waited for, and the slot table is filled beside the layout's one CTA per
+    // window. Two CTAs per SM share the filling.
+    const u64 want = (max_slots + 16ull * LAYOUT_THREADS - 1) / (16ull * LAYOUT_THREADS);
+    CK(start_plan((u32)std::max<u64>(1, std::min<u64>(want, 2ull * ctx->n_sms / B))));
+  } else {
+    CK(cudaMemcpyAsync(d_desc, hd, B * sizeof(WinDesc), cudaMemcpyHostToDevice, st));
+    if (total_slots) CK(cudaMemsetAsync(rbase + o_perm, 0xFF, total_slots * 4, st));
+  }
   PlanLists pl; pl.fcta = (FusedCta*)(rbase + o_fcta); pl.fwt = (WarpTile*)(rbase + o_fwt); pl.t2 = (Tile*)(rbase + o_t2); pl.t3 = (Tile*)(rbase + o_t3);
-  { TimedLaunch tl(ts, 1, st); k_plan<<<B, PLAN_THREADS, 0, st>>>(d_desc, ctx->reg, pl, 1); }
+  pl.grp_words = (u32*)(rbase + o_lgrp); pl.grp_words_per_tile = LARGE_SEQS * sizeof(LargeGroup) / 4;
+  {
+    const u32 rank_ctas = std::min<u32>((2 * ctx->n_ranks + EMIT_THREADS - 1) / EMIT_THREADS, 2 * ctx->n_sms);
+    TimedLaunch tl(ts, 1, st);
+    k_emit<<<dim3(chunk_ctas + rank_ctas, B), EMIT_THREADS, 0, st>>>(d_desc, ctx->reg, pl, chunk_ctas);
+  }
   if (cta > 0) {
     const u64 blocks = (cta * REC_PER_CTA + SCAT_PER_CTA - 1) / SCAT_PER_CTA;      // of the largest window
     const u32 per = (u32)std::min<u64>(SCAT_BLOCKS_MAX, std::max<u64>(1, blocks * B / (16ull * ctx->n_sms)));
     TimedLaunch tl(ts, 2, st);
     k_slot_scatter<<<dim3((u32)((blocks + per - 1) / per), B), SCAT_THREADS, 0, st>>>(d_desc, ctx->reg, per);
   }
-  CK(cudaMemsetAsync(rbase + o_defn, 0, 16, st));
   if (n_list[B_FCTA]) {
-    const DeferList dl{(u64*)(rbase + o_def), (u32*)(rbase + o_defn)};
+    const DeferList dl{(u64*)(rbase + o_def), (u32*)(pbase + o_defn)};
     TimedLaunch tl(ts, 3, st);
     k_reduce_fused<<<(u32)n_list[B_FCTA], SMALL_SEQS, 0, st>>>(d_desc, pl.fcta, pl.fwt, (TileSum*)(rbase + o_fsum), ctx->reg, ctx->dp, dl);
     k_reduce_deferred<<<DEF_GRID, DEF_WARPS * 32, 0, st>>>(d_desc, dl, ctx->reg, ctx->dp, now_ns);
   }
   if (n_list[B_T2]) { TimedLaunch tl(ts, 4, st); k_reduce_mid<<<(u32)n_list[B_T2], MID_THREADS, mid_smem_bytes(2 * WARP_N), st>>>(d_desc, pl.t2, (TileSum*)(rbase + o_s2), ctx->reg, ctx->dp, now_ns); }
   if (n_list[B_T3]) {
-    const DeferList dl{(u64*)(rbase + o_def3), (u32*)(rbase + o_defn) + 2};
+    const DeferList dl{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
     LargeGroup* lgrp = (LargeGroup*)(rbase + o_lgrp);
-    CK(cudaMemsetAsync(lgrp, 0, n_list[B_T3] * (size_t)LARGE_SEQS * sizeof(LargeGroup), st));
     TimedLaunch tl(ts, 5, st);
     k_large_stage<<<dim3((u32)n_list[B_T3], (ctx->max_large_n + LS_MEMBERS - 1) / LS_MEMBERS), LS_THREADS, 0, st>>>(d_desc, pl.t3, lgrp, ctx->reg);
     const u32 grid = (u32)std::min<u64>(n_list[B_T3], 2ull * ctx->n_sms);      // persistent: two CTAs per SM take the tiles in turn
@@ -705,14 +720,9 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     w.analysed = true; w.plan_blk = plan_blk; w.res_blk = res_blk; w.d_desc = d_desc + k; w.d = hd[k];
     std::memcpy(w.totals, tot + (size_t)k * T_COUNT, sizeof w.totals);
   }
-  if (expect) {
-    // what the plan really found follows the batch into pinned memory; settle() reads it
-    PendingBatch pbatch; pbatch.first = first_window; pbatch.n = B; pbatch.now = now_ns;
-    pbatch.h_tot = pinned_get(ctx, (size_t)B * T_COUNT * 8, &pbatch.h_bytes);
-    if (!pbatch.h_tot) { cudaStreamSynchronize(st); return fail(ctx, CCLD_ERR_NOMEM, "pinned allocation failed"); }
-    CK(cudaMemcpyAsync(pbatch.h_tot, pbase + o_tot, (size_t)B * T_COUNT * 8, cudaMemcpyDeviceToHost, st));
-    ctx->pending.push_back(pbatch);
-  } else {
+  // what the layout really found is in pinned memory once the stream has passed it; settle() reads it
+  ctx->pending.push_back(pbatch); guard.queued = true;
+  if (!expect) {
     // remember the totals of this shape, unless a window was refused
     bool clean = true;
     for (u32 k = 0; k < B && clean; ++k) clean = tot[(size_t)k * T_COUNT + T_FAILED] == 0;

@@ -2,8 +2,8 @@
 // the host side only sizes buffers and launches.
 //
 //   k_seq_range     group-by, part 1: op-counter range per (window, communicator)
-//   k_plan          group-by, part 2: closed-form slot layout (prefix sums over communicators),
-//                   and the work list for the reduction kernels
+//   k_layout, k_emit  group-by, part 2: closed-form slot layout (prefix sums over communicators) and the work lists of the
+//                   reduction kernels (ccld_plan.cuh)
 //   k_slot_scatter  group-by, part 3: perm[slot] = record index
 //   k_reduce_fused  per-op reductions + median/MAD + flags + votes for n <= 128, chunk-major work list:
 //                   n <= 8 one thread per group (warp-tiles), 9 <= n <= 128 n_pad / 8 lanes per group (register /
@@ -18,6 +18,7 @@
 // The suspect list and the ordered output lists are in ccld_verdict.cuh.
 #pragma once
 #include "ccld_device.cuh"
+#include "ccld_plan.cuh"
 
 namespace ccld {
 
@@ -298,314 +299,6 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* __rest
   for (u32 c = threadIdx.x; c < R.n_comms; c += REC_THREADS) {
     const u32 mn = s_mn[c];
     if (mn != NONE) { atomicMin(&D.rmin[c], mn); atomicMax(&D.rmax[c], s_mx[c]); }      // nothing waits for these
-  }
-}
-
-// ------------------------------------------------------------------------------------------------
-// group-by, part 2: closed-form layout and work lists. One CTA per window scans the communicators.
-//   slot(comm, seq, pos) = slot0[comm] + (seq - seq_lo[comm]) * n[comm] + pos
-// ------------------------------------------------------------------------------------------------
-struct PlanAcc { u64 groups, slots; u32 rows, t2, t3, pad; };
-
-__device__ __forceinline__ PlanAcc plan_add(const PlanAcc& a, const PlanAcc& b) {
-  PlanAcc r; r.groups = a.groups + b.groups; r.slots = a.slots + b.slots; r.rows = a.rows + b.rows;
-  r.t2 = a.t2 + b.t2; r.t3 = a.t3 + b.t3; r.pad = 0; return r;
-}
-__device__ __forceinline__ PlanAcc plan_shfl_up(const PlanAcc& a, int d) {
-  PlanAcc r;
-  r.groups = __shfl_up_sync(0xFFFFFFFFu, a.groups, d); r.slots = __shfl_up_sync(0xFFFFFFFFu, a.slots, d);
-  r.rows = __shfl_up_sync(0xFFFFFFFFu, a.rows, d); r.t2 = __shfl_up_sync(0xFFFFFFFFu, a.t2, d);
-  r.t3 = __shfl_up_sync(0xFFFFFFFFu, a.t3, d); r.pad = 0;
-  return r;
-}
-
-// op counters communicator c covers in the window (0 if none; clamped to 2^32 - 1)
-__device__ __forceinline__ u32 plan_nseq(const WinDesc& D, const Registry& R, u32 c) {
-  if (c >= R.n_comms) return 0;
-  const u32 lo = D.rmin[c], hi = D.rmax[c];
-  if (!(lo <= hi && lo != NONE)) return 0;
-  const u64 ns = (u64)hi - lo + 1;
-  return ns > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)ns;
-}
-
-__device__ __forceinline__ PlanAcc plan_item(const WinDesc& D, const Registry& R, u32 c) {
-  PlanAcc a = {0, 0, 0, 0, 0, 0};
-  const u32 ns = plan_nseq(D, R, c);
-  if (ns) {
-    const u32 n = R.comm_n[c], cls = comm_class(n);
-    a.groups = ns; a.slots = (u64)ns * n; a.rows = 1;
-    const u32 t = ceil_div(ns, tile_seqs(n));
-    a.t2 = cls == 2 ? t : 0; a.t3 = cls == 3 ? t : 0;
-  }
-  return a;
-}
-
-// Exclusive prefix of `v` over the CTA's threads plus the CTA total, for PLAN_THREADS = 1024.
-constexpr int PLAN_THREADS = 1024;
-__device__ PlanAcc plan_block_scan(PlanAcc v, PlanAcc* total, PlanAcc* s_warp /*[33]*/) {
-  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  PlanAcc inc = v;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) { PlanAcc o = plan_shfl_up(inc, d); if (lane >= (u32)d) inc = plan_add(inc, o); }
-  if (lane == 31) s_warp[wid] = inc;
-  __syncthreads();
-  if (wid == 0) {
-    PlanAcc x = s_warp[lane], xi = x;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) { PlanAcc o = plan_shfl_up(xi, d); if (lane >= (u32)d) xi = plan_add(xi, o); }
-    PlanAcc ex = plan_shfl_up(xi, 1);
-    if (lane == 0) ex = PlanAcc{0, 0, 0, 0, 0, 0};
-    s_warp[lane] = ex;
-    if (lane == 31) s_warp[32] = xi;
-  }
-  __syncthreads();
-  PlanAcc ex = plan_shfl_up(inc, 1);
-  if (lane == 0) ex = PlanAcc{0, 0, 0, 0, 0, 0};
-  PlanAcc r = plan_add(s_warp[wid], ex);
-  *total = s_warp[32];
-  __syncthreads();
-  return r;
-}
-
-// The same for a pair of 32-bit counters.
-__device__ uint2 plan_scan2(uint2 v, uint2* total, uint2* s_pair /*[33]*/) {
-  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint2 inc = v;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const u32 ox = __shfl_up_sync(0xFFFFFFFFu, inc.x, d), oy = __shfl_up_sync(0xFFFFFFFFu, inc.y, d);
-    if (lane >= (u32)d) { inc.x += ox; inc.y += oy; }
-  }
-  if (lane == 31) s_pair[wid] = inc;
-  __syncthreads();
-  if (wid == 0) {
-    const uint2 x = s_pair[lane]; uint2 xi = x;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const u32 ox = __shfl_up_sync(0xFFFFFFFFu, xi.x, d), oy = __shfl_up_sync(0xFFFFFFFFu, xi.y, d);
-      if (lane >= (u32)d) { xi.x += ox; xi.y += oy; }
-    }
-    s_pair[lane] = make_uint2(xi.x - x.x, xi.y - x.y);
-    if (lane == 31) s_pair[32] = xi;
-  }
-  __syncthreads();
-  const uint2 r = make_uint2(s_pair[wid].x + inc.x - v.x, s_pair[wid].y + inc.y - v.y);
-  *total = s_pair[32];
-  __syncthreads();
-  return r;
-}
-
-// Work units (warp-tiles of class 0, CTA tiles of class 1) of communicator c in chunk tau; 0 for other classes.
-__device__ __forceinline__ u32 chunk_units(u32 ns, u32 n, u32 T, u32 tau) {
-  if (ns == 0 || comm_class(n) > 1) return 0;
-  return ceil_div(chunk_size(ns, T, tau), tile_seqs(n));
-}
-// All units of communicator c in the window (its TileSum entries): full chunks plus the last one.
-__device__ __forceinline__ u32 comm_units(u32 ns, u32 n, u32 T) {
-  if (ns == 0 || comm_class(n) > 1) return 0;
-  const u32 S = chunk_len(ns, T), nch = ceil_div(ns, S), U = tile_seqs(n);
-  return (nch - 1) * ceil_div(S, U) + ceil_div(ns - (nch - 1) * S, U);
-}
-
-struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; };
-
-// A window that is given up leaves no work behind: zero ranges and scatter rows, zero totals.
-__device__ __forceinline__ void plan_clear_rows(WinDesc& D, const Registry& R) {
-  for (u32 c = threadIdx.x; c < R.n_comms; c += PLAN_THREADS) { RangeRow z = {0, 0, 0, R.comm_n[c], 0, 0, 0, 0}; D.ranges[c] = z; D.srow[c] = make_uint4(0, 0, 0, 0); }
-  for (u64 i = threadIdx.x; i < (u64)R.n_ranks * RANK_TAB_K; i += PLAN_THREADS) D.rent[i] = make_uint4(0, 0, 0, 0);
-}
-__device__ __forceinline__ void plan_give_up(WinDesc& D, const Registry& R, u64 why) {
-  plan_clear_rows(D, R);
-  if (threadIdx.x == 0) {
-    for (int q = 0; q < T_COUNT; ++q) D.totals[q] = 0;
-    D.totals[T_FAILED] = why; D.totals[T_CHUNKS] = 1;
-  }
-}
-
-// emit == 0: ranges, scatter rows and totals (the window is refused if it needs more than slot_cap slots).
-// emit == 1: the work lists (base[] filled by the host from the totals).
-// When the host sized the results from totals it expected (D.expect) instead of waiting for these, a window whose totals
-// differ gives up and raises the poison flag; so does every window planned after the flag went up - in the same batch
-// (seen here at emit == 1) or in a later one - so that windows are never analysed out of order. A window that gave up
-// fills its stretch of the work lists with entries that hold no work, because the kernels that follow are launched
-// over the expected lengths.
-__global__ void __launch_bounds__(PLAN_THREADS) k_plan(WinDesc* __restrict__ wd, Registry R, PlanLists L, int emit) {
-  __shared__ PlanAcc s_warp[33];
-  __shared__ uint2 s_pair[33];
-  __shared__ u32 s_red[32];
-  __shared__ int s_failed;
-  WinDesc& D = wd[blockIdx.x];
-  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (emit) {
-    if (D.expect != nullptr) {
-      if (!D.totals[T_FAILED] && *(volatile u32*)D.poison != 0) { __syncthreads(); plan_give_up(D, R, FAILED_EXPECT); __syncthreads(); }
-      if (D.totals[T_FAILED]) {
-        const u64 n_cta = D.expect[T_FCTA], n2 = D.expect[T_TILES2], n3 = D.expect[T_TILES3];
-        for (u64 j = threadIdx.x; j < n_cta; j += PLAN_THREADS) {
-          FusedCta x; x.w = blockIdx.x; x.cls = 0; x.c = 0; x.seq_off = 0; x.count = 0; x.sum_idx = 0; x.wt_first = 0; x.wt_count = 0; x.moff = 0;
-          x.row = RangeRow{0, 0, 0, 0, 0, 0, 0, 0};
-          L.fcta[D.base[B_FCTA] + j] = x;
-        }
-        for (u64 j = threadIdx.x; j < n2; j += PLAN_THREADS) { Tile t; t.w = blockIdx.x; t.c = 0; t.seq_off = 0; t.count = 0; L.t2[D.base[B_T2] + j] = t; }
-        for (u64 j = threadIdx.x; j < n3; j += PLAN_THREADS) { Tile t; t.w = blockIdx.x; t.c = 0; t.seq_off = 0; t.count = 0; L.t3[D.base[B_T3] + j] = t; }
-        return;
-      }
-    } else if (D.totals[T_FAILED]) return;
-  }
-
-  if (!emit) {
-    // 1. layout: groups, slots, rows; tiles of the two big classes; busiest fused-class communicator
-    PlanAcc run = {0, 0, 0, 0, 0, 0};
-    u32 mx = 0;
-    for (u32 c0 = 0; c0 < R.n_comms; c0 += PLAN_THREADS) {
-      const u32 c = c0 + threadIdx.x;
-      PlanAcc it = plan_item(D, R, c), tot;
-      PlanAcc ex = plan_add(run, plan_block_scan(it, &tot, s_warp));
-      if (c < R.n_comms) {
-        RangeRow r;
-        r.seq_lo = it.rows ? D.rmin[c] : 0; r.n_seq = (u32)it.groups; r.row_idx = ex.rows; r.n = R.comm_n[c];
-        r.group0 = ex.groups; r.slot0 = ex.slots; r.tile0 = 0; r.n_units = 0;
-        D.ranges[c] = r;
-        D.srow[c] = make_uint4((u32)r.slot0, (u32)(r.slot0 >> 32), r.n_seq, r.seq_lo);
-        if (it.rows && comm_class(r.n) <= 1) mx = r.n_seq > mx ? r.n_seq : mx;
-      }
-      run = plan_add(run, tot);
-    }
-    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-    if (lane == 0) s_red[wid] = mx;
-    __syncthreads();
-    mx = 0;
-    for (int q = 0; q < PLAN_THREADS / 32; ++q) mx = s_red[q] > mx ? s_red[q] : mx;
-    u32 T = mx ? ceil_div(mx, CHUNK_REF) : 1u;
-    T = T > CHUNK_MAX ? CHUNK_MAX : T;
-    __syncthreads();
-    // 2. summary entries of the fused classes
-    u32 urun = 0;
-    for (u32 c0 = 0; c0 < R.n_comms; c0 += PLAN_THREADS) {
-      const u32 c = c0 + threadIdx.x;
-      const u32 ns = plan_nseq(D, R, c), n = c < R.n_comms ? R.comm_n[c] : 1u;
-      const u32 u = comm_units(ns, n, T);
-      uint2 tot; const uint2 ex = plan_scan2(make_uint2(u, 0), &tot, s_pair);
-      if (c < R.n_comms && u) { D.ranges[c].tile0 = urun + ex.x; D.ranges[c].n_units = u; }
-      urun += tot.x;
-    }
-    // 3. CTAs and warp-tiles of the fused kernel, chunk by chunk
-    u64 n_cta = 0, n_wt = 0;
-    for (u32 tau = 0; tau < T; ++tau) {
-      u32 wt = 0, c1 = 0;
-      for (u32 c = threadIdx.x; c < R.n_comms; c += PLAN_THREADS) {
-        const u32 n = R.comm_n[c], u = chunk_units(plan_nseq(D, R, c), n, T, tau);
-        if (comm_class(n) == 0) wt += u; else c1 += u;
-      }
-      uint2 tot; plan_scan2(make_uint2(wt, c1), &tot, s_pair);
-      n_cta += ceil_div(tot.x, FUSED_WT_PER_CTA) + tot.y; n_wt += tot.x;
-    }
-    if (threadIdx.x == 0) {
-      // op counters further apart than 2^31, or more slots than the cap: refuse the window
-      u64 failed = (run.slots > D.slot_cap || run.groups > 0x7FFFFFFFull || n_cta > 0x7FFFFFFFull || n_wt > 0x7FFFFFFFull) ? FAILED_CAPACITY : 0;
-      if (!failed && D.expect != nullptr) {
-        const u64* e = D.expect;
-        const bool same = e[T_GROUPS] == run.groups && e[T_SLOTS] == run.slots && e[T_FCTA] == n_cta && e[T_FWT] == n_wt && e[T_FSUM] == urun &&
-                          e[T_TILES2] == run.t2 && e[T_TILES3] == run.t3 && e[T_ROWS] == run.rows && e[T_CHUNKS] == T;
-        if (!same || *(volatile u32*)D.poison != 0) { failed = FAILED_EXPECT; atomicExch(D.poison, 1u); }
-      }
-      s_failed = failed != 0;
-      D.totals[T_GROUPS] = failed ? 0 : run.groups; D.totals[T_SLOTS] = failed ? 0 : run.slots;
-      D.totals[T_FCTA] = failed ? 0 : n_cta; D.totals[T_FWT] = failed ? 0 : n_wt; D.totals[T_FSUM] = failed ? 0 : urun;
-      D.totals[T_TILES2] = failed ? 0 : run.t2; D.totals[T_TILES3] = failed ? 0 : run.t3;
-      D.totals[T_ROWS] = failed ? 0 : run.rows; D.totals[T_FAILED] = failed; D.totals[T_CHUNKS] = T;
-      if (failed == FAILED_CAPACITY) atomicOr((unsigned*)&D.counters[C_ERR], (unsigned)CCLD_E_CAPACITY);
-    }
-    __syncthreads();
-    if (s_failed) { plan_clear_rows(D, R); return; }
-    // 4. every rank's inline (communicator, position) pairs resolved against this window's scatter rows, so that the
-    //    scatter pass finds (op counters covered, first op counter, first slot of the member's column) with one load.
-    //    Only where slots fit 32 bits and the member's whole column lies inside the table; other entries stay unused.
-    if (run.slots <= 0xFFFFFFFFull) {
-#pragma unroll 4
-      for (u64 i = threadIdx.x; i < (u64)R.n_ranks * 2; i += PLAN_THREADS) {
-        const uint4 t = R.rank_tab[i];
-        uint4 e[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const u32 id = h ? t.z : t.x, cp = h ? t.w : t.y;
-          if (id != NONE && cp != NONE && cp != RANK_TAB_OVERFLOW) {
-            const uint4 sr = D.srow[cp >> RANK_TAB_POS_BITS];
-            const u64 b = ((u64)sr.x | ((u64)sr.y << 32)) + (u64)(cp & ((1u << RANK_TAB_POS_BITS) - 1)) * sr.z;
-            if (sr.z != 0 && b + sr.z <= run.slots) e[h] = make_uint4(id, sr.z, sr.w, (u32)b);
-          }
-        }
-        D.rent[i * 2] = e[0]; D.rent[i * 2 + 1] = e[1];
-      }
-    }
-    return;
-  }
-
-  // ---- emit ----
-  const u32 T = (u32)D.totals[T_CHUNKS];
-  // tiles of classes 2 and 3, communicator by communicator; summary indices of every communicator become batch-wide
-  {
-    PlanAcc run = {0, 0, 0, 0, 0, 0};
-    for (u32 c0 = 0; c0 < R.n_comms; c0 += PLAN_THREADS) {
-      const u32 c = c0 + threadIdx.x;
-      PlanAcc it = plan_item(D, R, c), tot;
-      PlanAcc ex = plan_add(run, plan_block_scan(it, &tot, s_warp));
-      if (c < R.n_comms && it.rows) {
-        const u32 n = R.comm_n[c], S = tile_seqs(n), cls = comm_class(n);
-        if (cls <= 1) D.ranges[c].tile0 += D.base[B_FSUM];
-        else {
-          const u32 first = cls == 2 ? D.base[B_T2] + ex.t2 : D.base[B_T3] + ex.t3, nt = cls == 2 ? it.t2 : it.t3;
-          Tile* dst = (cls == 2 ? L.t2 : L.t3) + first;
-          D.ranges[c].tile0 = first; D.ranges[c].n_units = nt;
-          for (u32 k = 0; k < nt; ++k) {
-            Tile t; t.w = blockIdx.x; t.c = c; t.seq_off = k * S;
-            const u64 left = it.groups - (u64)k * S; t.count = left < S ? (u32)left : S;
-            dst[k] = t;
-          }
-        }
-      }
-      run = plan_add(run, tot);
-    }
-  }
-  __syncthreads();
-  // fused classes: chunk-major list of CTAs; a class-0 CTA takes eight consecutive warp-tiles
-  u32 cta_base = D.base[B_FCTA], wt_base = D.base[B_FWT];
-  for (u32 tau = 0; tau < T; ++tau) {
-    u32 wt_run = 0, c1_run = 0;
-    // class-1 CTAs come after the chunk's class-0 CTAs, whose number needs the chunk's warp-tile total first
-    u32 wt_total = 0;
-    {
-      u32 wt = 0;
-      for (u32 c = threadIdx.x; c < R.n_comms; c += PLAN_THREADS) { const u32 n = R.comm_n[c]; if (comm_class(n) == 0) wt += chunk_units(plan_nseq(D, R, c), n, T, tau); }
-      uint2 tot; plan_scan2(make_uint2(wt, 0), &tot, s_pair);
-      wt_total = tot.x;
-    }
-    const u32 n0 = ceil_div(wt_total, FUSED_WT_PER_CTA);
-    for (u32 c0 = 0; c0 < R.n_comms; c0 += PLAN_THREADS) {
-      const u32 c = c0 + threadIdx.x;
-      const u32 ns = plan_nseq(D, R, c), n = c < R.n_comms ? R.comm_n[c] : 1u, cls = comm_class(n);
-      const u32 u = chunk_units(ns, n, T, tau);
-      uint2 tot; const uint2 ex = plan_scan2(make_uint2(cls == 0 ? u : 0, cls == 1 ? u : 0), &tot, s_pair);
-      if (u) {
-        const u32 S = chunk_len(ns, T), U = tile_seqs(n), cnt = chunk_size(ns, T, tau);
-        const RangeRow crow = D.ranges[c]; const u64 cmoff = R.comm_moff[c];
-        const u32 sum0 = crow.tile0 + tau * ceil_div(S, U);
-        for (u32 k = 0; k < u; ++k) {
-          const u32 off = tau * S + k * U, len = cnt - k * U < U ? cnt - k * U : U;
-          if (cls == 0) { WarpTile x; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.row = crow; x.moff = cmoff; L.fwt[wt_base + wt_run + ex.x + k] = x; }
-          else { FusedCta x; x.w = blockIdx.x; x.cls = 1; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.wt_first = 0; x.wt_count = 0;
-                 x.row = crow; x.moff = cmoff; L.fcta[cta_base + n0 + c1_run + ex.y + k] = x; }
-        }
-      }
-      wt_run += tot.x; c1_run += tot.y;
-    }
-    for (u32 j = threadIdx.x; j < n0; j += PLAN_THREADS) {
-      FusedCta x; x.w = blockIdx.x; x.cls = 0; x.c = 0; x.seq_off = 0; x.count = 0; x.sum_idx = 0; x.moff = 0;
-      x.row = RangeRow{0, 0, 0, 0, 0, 0, 0, 0};
-      x.wt_first = wt_base + FUSED_WT_PER_CTA * j; x.wt_count = wt_total - FUSED_WT_PER_CTA * j < FUSED_WT_PER_CTA ? wt_total - FUSED_WT_PER_CTA * j : FUSED_WT_PER_CTA;
-      L.fcta[cta_base + j] = x;
-    }
-    cta_base += n0 + c1_run; wt_base += wt_total;
   }
 }
 
@@ -1034,7 +727,7 @@ __global__ void __launch_bounds__(128) k_window_rounds(const WinDesc* __restrict
   const i64* t_max = D.gi64 + (u64)GI_T_MAX * G + row.group0;
   const i64* t_min = D.gi64 + (u64)GI_T_MIN * G + row.group0;
   // round counts and the Eq. 2 candidate come from the tile summaries the reduce kernels left behind
-  const TileSum* ts = D.tsum[cls <= 1 ? 0 : cls - 1] + row.tile0;
+  const TileSum* ts = D.tsum[cls <= 1 ? 0 : cls - 1] + row.tile0;   // both relative to the window
   const u32 nt = row.n_units;
   u32 n_rounds = 0, n_an = 0;
   u64 best_rng = 0; u32 best_k = NONE;

@@ -1,0 +1,347 @@
+// Group-by, part 2: the closed-form layout of every window and the work lists of the reduction kernels (sm_100a).
+//   slot(comm, seq, pos) = slot0[comm] + (seq - seq_lo[comm]) * n[comm] + pos
+//
+//   k_begin   the batch's descriptors move from pinned host memory to the device and its op-counter ranges, counters and list
+//             lengths get their start values
+//   k_layout  one CTA per window: prefix sums over the communicators (groups, slots, rows, work units) and the start of every
+//             chunk of the work lists; the other CTAs of the launch fill the slot table of a batch that does not wait
+//   k_emit    a CTA per (window, chunk) writes that chunk's part of the work lists; further CTAs resolve every rank's inline
+//             pairs against the window's rows
+//
+// All three are bound by latency: little data, a chain of dependent reads and barriers. The layout used to be one CTA per
+// window for everything - one scan over the communicators per chunk, the rank table of the whole job walked by one SM -
+// and took 20 us (one communicator, 1,000 ops) to 155 us (2,185 communicators, 16,384 ranks), twice per batch. What a
+// chunk holds follows from the chunk lengths alone, so the chunks' starts come from a histogram of where the
+// communicators end, and the lists and rank entries are written by as many CTAs as there are chunks and ranks.
+#pragma once
+#include "ccld_device.cuh"
+
+namespace ccld {
+
+constexpr int BEGIN_THREADS = 256;
+constexpr int LAYOUT_THREADS = 1024;
+constexpr int EMIT_THREADS = 256;
+
+struct BeginArgs {
+  const u32* desc_host; u32* desc; u64 desc_words;     // pinned source, device copy: descriptors (and expected totals behind them)
+  u32* rmin; u64 n_rmin;                               // set to NONE
+  u32* zero; u64 n_zero;                               // set to 0: rmax, counters, list lengths
+};
+
+__global__ void __launch_bounds__(BEGIN_THREADS) k_begin(BeginArgs A) {
+  const u64 i0 = (u64)blockIdx.x * BEGIN_THREADS + threadIdx.x, st = (u64)gridDim.x * BEGIN_THREADS;
+  for (u64 i = i0; i < A.desc_words; i += st) A.desc[i] = A.desc_host[i];
+  for (u64 i = i0; i < A.n_rmin; i += st) A.rmin[i] = NONE;
+  for (u64 i = i0; i < A.n_zero; i += st) A.zero[i] = 0;
+}
+
+// op counters communicator c covers in the window (0 if none; clamped to 2^32 - 1)
+__device__ __forceinline__ u32 plan_nseq(const WinDesc& D, u32 c) {
+  const u32 lo = D.rmin[c], hi = D.rmax[c];
+  if (!(lo <= hi && lo != NONE)) return 0;
+  const u64 ns = (u64)hi - lo + 1;
+  return ns > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)ns;
+}
+
+// Work units (warp-tiles of class 0, CTA tiles of class 1) of a communicator in chunk tau; 0 for other classes.
+__device__ __forceinline__ u32 chunk_units(u32 ns, u32 n, u32 T, u32 tau) {
+  if (ns == 0 || comm_class(n) > 1) return 0;
+  return ceil_div(chunk_size(ns, T, tau), tile_seqs(n));
+}
+// Its chunks, its units in every chunk but the last and in the last one.
+struct ChunkShape { u32 n, full, last; };
+__device__ __forceinline__ ChunkShape chunk_shape(u32 ns, u32 n, u32 T) {
+  ChunkShape x = {0, 0, 0};
+  if (ns == 0 || comm_class(n) > 1) return x;
+  const u32 S = chunk_len(ns, T), U = tile_seqs(n);
+  x.n = ceil_div(ns, S); x.full = ceil_div(S, U); x.last = ceil_div(ns - (x.n - 1) * S, U);
+  return x;
+}
+
+struct PlanAcc { u64 groups, slots; u32 rows, units, t2, t3; };
+__device__ __forceinline__ PlanAcc plan_add(const PlanAcc& a, const PlanAcc& b) {
+  PlanAcc r; r.groups = a.groups + b.groups; r.slots = a.slots + b.slots; r.rows = a.rows + b.rows; r.units = a.units + b.units;
+  r.t2 = a.t2 + b.t2; r.t3 = a.t3 + b.t3; return r;
+}
+__device__ __forceinline__ PlanAcc plan_shfl_up(const PlanAcc& a, int d) {
+  PlanAcc r;
+  r.groups = __shfl_up_sync(0xFFFFFFFFu, a.groups, d); r.slots = __shfl_up_sync(0xFFFFFFFFu, a.slots, d);
+  r.rows = __shfl_up_sync(0xFFFFFFFFu, a.rows, d); r.units = __shfl_up_sync(0xFFFFFFFFu, a.units, d);
+  r.t2 = __shfl_up_sync(0xFFFFFFFFu, a.t2, d); r.t3 = __shfl_up_sync(0xFFFFFFFFu, a.t3, d);
+  return r;
+}
+__device__ __forceinline__ PlanAcc plan_item(u32 ns, u32 n, u32 T) {
+  PlanAcc a = {0, 0, 0, 0, 0, 0};
+  if (ns == 0) return a;
+  const u32 cls = comm_class(n);
+  a.groups = ns; a.slots = (u64)ns * n; a.rows = 1;
+  if (cls <= 1) { const ChunkShape x = chunk_shape(ns, n, T); a.units = (x.n - 1) * x.full + x.last; }
+  else { const u32 t = ceil_div(ns, tile_seqs(n)); a.t2 = cls == 2 ? t : 0; a.t3 = cls == 3 ? t : 0; }
+  return a;
+}
+
+// Work lists of the batch; grp: one record per op counter of the class-3 tiles, zeroed with the tile's entry.
+struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; u32* grp_words; u32 grp_words_per_tile; };
+
+// When the host sized the results from totals it expected (D.expect) instead of waiting for these, a window whose totals
+// differ gives up and raises the poison flag; so does every window planned after the flag went up - in the same batch
+// (seen by k_emit) or in a later one - so that windows are never analysed out of order.
+// Grid: (1 + filling CTAs, windows). fill: whether the slot table (sized from the expectation) is to be set to NONE.
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __restrict__ wd, Registry R, int fill) {
+  __shared__ PlanAcc s_warp[33];
+  __shared__ u32 s_red[32];
+  __shared__ u32 s_hist[2][CHUNK_MAX + 2];                     // differences along the chunks: warp-tiles of class 0, tiles of class 1
+  const WinDesc& D = wd[blockIdx.y];
+  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (blockIdx.x > 0) {
+    if (!fill) return;
+    u32* __restrict__ perm = D.perm; const u64 n = D.n_slots;
+    const u64 head = min(n, (u64)((16 - ((uintptr_t)perm & 15)) & 15) / 4), n4 = (n - head) / 4;
+    const u64 i0 = (u64)(blockIdx.x - 1) * LAYOUT_THREADS + threadIdx.x, st = (u64)(gridDim.x - 1) * LAYOUT_THREADS;
+    uint4* p4 = reinterpret_cast<uint4*>(perm + head);
+    for (u64 i = i0; i < n4; i += st) p4[i] = make_uint4(NONE, NONE, NONE, NONE);
+    if (i0 < head) perm[i0] = NONE;
+    if (i0 < n - head - n4 * 4) perm[head + n4 * 4 + i0] = NONE;
+    return;
+  }
+  const u32 per = ceil_div(R.n_comms, LAYOUT_THREADS), c_lo = threadIdx.x * per, c_hi = min(R.n_comms, c_lo + per);   // my communicators
+  // the busiest communicator of the fused classes decides how many chunks there are
+  u32 mx = 0;
+  for (u32 c = c_lo; c < c_hi; ++c) { const u32 ns = plan_nseq(D, c); if (comm_class(R.comm_n[c]) <= 1) mx = max(mx, ns); }
+  mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+  if (lane == 0) s_red[wid] = mx;
+  for (u32 i = threadIdx.x; i < 2 * (CHUNK_MAX + 2); i += LAYOUT_THREADS) (&s_hist[0][0])[i] = 0;
+  __syncthreads();
+  mx = __reduce_max_sync(0xFFFFFFFFu, s_red[lane]);
+  u32 T = mx ? ceil_div(mx, CHUNK_REF) : 1u;
+  T = T > CHUNK_MAX ? CHUNK_MAX : T;
+  // sums over my communicators, and where their units begin and end along the chunks
+  PlanAcc mine = {0, 0, 0, 0, 0, 0};
+  for (u32 k = 0; k < per; ++k) {                              // the same number of steps in every thread
+    const u32 c = c_lo + k;
+    const bool in = c < c_hi;
+    const u32 ns = in ? plan_nseq(D, c) : 0, n = in ? R.comm_n[c] : 1u;
+    mine = plan_add(mine, plan_item(ns, n, T));
+    const ChunkShape x = chunk_shape(ns, n, T);
+    // communicators of one family end in the same chunk: one set of atomics for all lanes that agree
+    const u32 key = x.n ? x.n * 2 + comm_class(n) : 0;
+    u32 pend = __ballot_sync(0xFFFFFFFFu, key != 0);
+    while (pend) {
+      const u32 lead = __shfl_sync(0xFFFFFFFFu, key, (u32)__ffs(pend) - 1u);
+      const bool same = key == lead;
+      const u32 full = __reduce_add_sync(0xFFFFFFFFu, same ? x.full : 0u), last = __reduce_add_sync(0xFFFFFFFFu, same ? x.last : 0u);
+      if (lane == 0) {
+        u32* h = s_hist[lead & 1];
+        const u32 nch = lead >> 1;
+        atomicAdd(&h[0], full); atomicAdd(&h[nch - 1], last - full); atomicAdd(&h[nch], 0u - last);
+      }
+      pend &= ~__ballot_sync(0xFFFFFFFFu, same);
+    }
+  }
+  // exclusive prefix over the threads
+  PlanAcc inc = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) { PlanAcc o = plan_shfl_up(inc, d); if (lane >= (u32)d) inc = plan_add(inc, o); }
+  if (lane == 31) s_warp[wid] = inc;
+  __syncthreads();
+  if (wid == 0) {
+    PlanAcc xi = s_warp[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { PlanAcc o = plan_shfl_up(xi, d); if (lane >= (u32)d) xi = plan_add(xi, o); }
+    PlanAcc ex = plan_shfl_up(xi, 1);
+    if (lane == 0) ex = PlanAcc{0, 0, 0, 0, 0, 0};
+    s_warp[lane] = ex;
+    if (lane == 31) s_warp[32] = xi;
+  }
+  __syncthreads();
+  PlanAcc run = plan_shfl_up(inc, 1);
+  if (lane == 0) run = PlanAcc{0, 0, 0, 0, 0, 0};
+  run = plan_add(s_warp[wid], run);
+  const PlanAcc all = s_warp[32];
+  // first CTA and first warp-tile of every chunk, in warp 0; two chunks per lane
+  if (wid == 0) {
+    u32 wt[2], c1[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) { wt[q] = s_hist[0][2 * lane + q]; c1[q] = s_hist[1][2 * lane + q]; }
+    wt[1] += wt[0]; c1[1] += c1[0];                            // differences -> units, along the chunks
+    u32 sw = wt[1], sc = c1[1];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const u32 ow = __shfl_up_sync(0xFFFFFFFFu, sw, d), oc = __shfl_up_sync(0xFFFFFFFFu, sc, d);
+      if (lane >= (u32)d) { sw += ow; sc += oc; }
+    }
+    const u32 bw = sw - wt[1], bc = sc - c1[1];
+    wt[0] += bw; wt[1] += bw; c1[0] += bc; c1[1] += bc;
+    const u32 a0 = ceil_div(wt[0], FUSED_WT_PER_CTA) + c1[0], a1 = ceil_div(wt[1], FUSED_WT_PER_CTA) + c1[1];
+    u32 pc = a0 + a1, pw = wt[0] + wt[1];                      // CTAs and warp-tiles of my two chunks
+    const u32 oc_ = pc, ow_ = pw;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const u32 oc = __shfl_up_sync(0xFFFFFFFFu, pc, d), ow = __shfl_up_sync(0xFFFFFFFFu, pw, d);
+      if (lane >= (u32)d) { pc += oc; pw += ow; }
+    }
+    D.chunks[2 * lane] = make_uint2(pc - oc_, pw - ow_);
+    D.chunks[2 * lane + 1] = make_uint2(pc - oc_ + a0, pw - ow_ + wt[0]);
+    const u64 n_cta = __shfl_sync(0xFFFFFFFFu, pc, 31), n_wt = __shfl_sync(0xFFFFFFFFu, pw, 31);
+    static_assert(CHUNK_MAX == 64, "two chunks per lane");
+    if (lane == 31) D.chunks[CHUNK_MAX] = make_uint2(pc, pw);
+    if (lane == 0) {
+      // op counters further apart than 2^31, or more slots than the cap: refuse the window
+      u64 failed = (all.slots > D.slot_cap || all.groups > 0x7FFFFFFFull) ? FAILED_CAPACITY : 0;
+      if (!failed && D.expect != nullptr) {
+        const u64* e = D.expect;
+        const bool same = e[T_GROUPS] == all.groups && e[T_SLOTS] == all.slots && e[T_FCTA] == n_cta && e[T_FWT] == n_wt && e[T_FSUM] == all.units &&
+                          e[T_TILES2] == all.t2 && e[T_TILES3] == all.t3 && e[T_ROWS] == all.rows && e[T_CHUNKS] == T;
+        if (!same || *(volatile u32*)D.poison != 0) { failed = FAILED_EXPECT; atomicExch(D.poison, 1u); }
+      }
+      u64 t[T_COUNT];
+      for (int q = 0; q < T_COUNT; ++q) t[q] = 0;
+      if (!failed) {
+        t[T_GROUPS] = all.groups; t[T_SLOTS] = all.slots; t[T_FCTA] = n_cta; t[T_FWT] = n_wt; t[T_FSUM] = all.units;
+        t[T_TILES2] = all.t2; t[T_TILES3] = all.t3; t[T_ROWS] = all.rows;
+      }
+      t[T_FAILED] = failed; t[T_CHUNKS] = failed ? 1 : T;
+      for (int q = 0; q < T_COUNT; ++q) { D.totals[q] = t[q]; D.totals_host[q] = t[q]; }
+      if (failed == FAILED_CAPACITY) atomicOr((unsigned*)&D.counters[C_ERR], (unsigned)CCLD_E_CAPACITY);
+      s_red[0] = failed != 0;
+    }
+  }
+  __syncthreads();
+  const bool failed = s_red[0] != 0;                           // a window that is given up leaves no work behind: empty rows
+  for (u32 c = c_lo; c < c_hi; ++c) {
+    const u32 ns = plan_nseq(D, c), n = R.comm_n[c];
+    const PlanAcc it = plan_item(ns, n, T);
+    RangeRow r = {0, 0, 0, n, 0, 0, 0, 0};
+    if (!failed) {
+      const u32 cls = comm_class(n);
+      r.seq_lo = ns ? D.rmin[c] : 0; r.n_seq = ns; r.row_idx = run.rows; r.group0 = run.groups; r.slot0 = run.slots;
+      r.tile0 = cls <= 1 ? run.units : (cls == 2 ? run.t2 : run.t3); r.n_units = it.units + it.t2 + it.t3;
+    }
+    D.ranges[c] = r;
+    D.srow[c] = make_uint4((u32)r.slot0, (u32)(r.slot0 >> 32), r.n_seq, r.seq_lo);
+    run = plan_add(run, it);
+  }
+}
+
+// Grid: (chunk CTAs + rank CTAs, windows); at least as many chunk CTAs as any window of the batch has chunks. base[] of the
+// descriptors is filled. A window that gave up fills its stretch of the lists with entries that hold no work, because the
+// kernels that follow are launched over the expected lengths.
+__global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict__ wd, Registry R, PlanLists L, u32 chunk_ctas) {
+  __shared__ uint2 s_pair[EMIT_THREADS / 32 + 1];
+  const WinDesc& D = wd[blockIdx.y];
+  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const u64 failed = D.totals[T_FAILED];
+  // the flag can only go up while k_layout runs, so every CTA of this launch sees the same value
+  const bool give_up = failed != 0 || (D.expect != nullptr && *(volatile u32*)D.poison != 0);
+  const u64 n_slots = D.totals[T_SLOTS];
+  if (blockIdx.x >= chunk_ctas) {
+    // every rank's inline (communicator, position) pairs resolved against this window's scatter rows, so that the
+    // scatter pass finds (op counters covered, first op counter, first slot of the member's column) with one load. Only
+    // where slots fit 32 bits and the member's whole column lies inside the table; other entries stay unused.
+    const bool usable = !give_up && n_slots <= 0xFFFFFFFFull;
+    const u64 st = (u64)(gridDim.x - chunk_ctas) * EMIT_THREADS;
+    for (u64 i = (u64)(blockIdx.x - chunk_ctas) * EMIT_THREADS + threadIdx.x; i < (u64)R.n_ranks * 2; i += st) {
+      uint4 e[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+      if (usable) {
+        const uint4 t = R.rank_tab[i];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const u32 id = h ? t.z : t.x, cp = h ? t.w : t.y;
+          if (id != NONE && cp != NONE && cp != RANK_TAB_OVERFLOW) {
+            const uint4 sr = D.srow[cp >> RANK_TAB_POS_BITS];
+            const u64 b = ((u64)sr.x | ((u64)sr.y << 32)) + (u64)(cp & ((1u << RANK_TAB_POS_BITS) - 1)) * sr.z;
+            if (sr.z != 0 && b + sr.z <= n_slots) e[h] = make_uint4(id, sr.z, sr.w, (u32)b);
+          }
+        }
+      }
+      D.rent[i * 2] = e[0]; D.rent[i * 2 + 1] = e[1];
+    }
+    return;
+  }
+  const u32 tau = blockIdx.x;
+  if (give_up) {
+    if (D.expect == nullptr) return;                           // the host knows: it sized nothing for this window
+    const u32 i0 = tau * EMIT_THREADS + threadIdx.x, st = chunk_ctas * EMIT_THREADS;
+    if (!failed) {                                             // another window's layout was the surprise: this one's rows go too
+      for (u32 c = i0; c < R.n_comms; c += st) { D.ranges[c] = RangeRow{0, 0, 0, R.comm_n[c], 0, 0, 0, 0}; D.srow[c] = make_uint4(0, 0, 0, 0); }
+      if (i0 == 0) for (int q = 0; q < T_COUNT; ++q) { const u64 v = q == T_FAILED ? FAILED_EXPECT : 0; D.totals_host[q] = v; }
+    }
+    const u64 n_cta = D.expect[T_FCTA], n2 = D.expect[T_TILES2], n3 = D.expect[T_TILES3];
+    for (u64 j = i0; j < n_cta; j += st) {
+      FusedCta x; x.w = blockIdx.y; x.cls = 0; x.c = 0; x.seq_off = 0; x.count = 0; x.sum_idx = 0; x.wt_first = 0; x.wt_count = 0; x.moff = 0;
+      x.row = RangeRow{0, 0, 0, 0, 0, 0, 0, 0};
+      L.fcta[D.base[B_FCTA] + j] = x;
+    }
+    const Tile none = {blockIdx.y, 0, 0, 0};
+    for (u64 j = i0; j < n2; j += st) L.t2[D.base[B_T2] + j] = none;
+    for (u64 j = i0; j < n3; j += st) L.t3[D.base[B_T3] + j] = none;
+    for (u64 j = i0; j < n3 * L.grp_words_per_tile; j += st) L.grp_words[(u64)D.base[B_T3] * L.grp_words_per_tile + j] = 0;
+    return;
+  }
+  const u32 T = (u32)D.totals[T_CHUNKS];
+  if (tau >= T) return;
+  // tiles of classes 2 and 3: a warp per communicator, lanes along its tiles
+  for (u32 c = tau * (EMIT_THREADS / 32) + wid; c < R.n_comms; c += T * (EMIT_THREADS / 32)) {
+    const u32 n = R.comm_n[c], cls = comm_class(n);
+    if (cls < 2) continue;
+    const RangeRow row = D.ranges[c];
+    const u32 S = tile_seqs(n), first = D.base[cls == 2 ? B_T2 : B_T3] + row.tile0;
+    Tile* dst = cls == 2 ? L.t2 : L.t3;
+    for (u32 k = lane; k < row.n_units; k += 32) {
+      Tile t; t.w = blockIdx.y; t.c = c; t.seq_off = k * S;
+      const u32 left = row.n_seq - k * S; t.count = left < S ? left : S;
+      dst[first + k] = t;
+    }
+    if (cls == 3) {
+      u32* g = L.grp_words + (u64)first * L.grp_words_per_tile;
+      for (u64 k = lane; k < (u64)row.n_units * L.grp_words_per_tile; k += 32) g[k] = 0;
+    }
+  }
+  // fused classes: my consecutive communicators' units of this chunk, then where they go
+  const u32 per = ceil_div(R.n_comms, EMIT_THREADS), c_lo = threadIdx.x * per, c_hi = min(R.n_comms, c_lo + per);
+  u32 wt = 0, c1 = 0;
+  for (u32 c = c_lo; c < c_hi; ++c) {
+    const u32 n = R.comm_n[c];
+    if (comm_class(n) > 1) continue;
+    const u32 u = chunk_units(D.ranges[c].n_seq, n, T, tau);
+    if (comm_class(n) == 0) wt += u; else c1 += u;
+  }
+  u32 iw = wt, ic = c1;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const u32 ow = __shfl_up_sync(0xFFFFFFFFu, iw, d), oc = __shfl_up_sync(0xFFFFFFFFu, ic, d);
+    if (lane >= (u32)d) { iw += ow; ic += oc; }
+  }
+  if (lane == 31) s_pair[wid] = make_uint2(iw, ic);
+  __syncthreads();
+  u32 bw = 0, bc = 0;
+#pragma unroll
+  for (u32 q = 0; q < EMIT_THREADS / 32; ++q) { const uint2 x = s_pair[q]; if (q < wid) { bw += x.x; bc += x.y; } }
+  const uint2 here = D.chunks[tau], next = D.chunks[tau + 1];
+  const u32 wt_base = D.base[B_FWT] + here.y, wt_total = next.y - here.y, cta_base = D.base[B_FCTA] + here.x, n0 = ceil_div(wt_total, FUSED_WT_PER_CTA);
+  u32 at_w = wt_base + bw + iw - wt, at_c = cta_base + n0 + bc + ic - c1;        // class-1 CTAs come after the chunk's class-0 CTAs
+  for (u32 c = c_lo; c < c_hi; ++c) {
+    const u32 n = R.comm_n[c], cls = comm_class(n);
+    if (cls > 1) continue;
+    const RangeRow row = D.ranges[c];
+    const u32 u = chunk_units(row.n_seq, n, T, tau);
+    if (u == 0) continue;
+    const u64 moff = R.comm_moff[c];
+    const u32 S = chunk_len(row.n_seq, T), U = tile_seqs(n), cnt = chunk_size(row.n_seq, T, tau);
+    const u32 sum0 = D.base[B_FSUM] + row.tile0 + tau * ceil_div(S, U);
+    for (u32 k = 0; k < u; ++k) {
+      const u32 off = tau * S + k * U, len = cnt - k * U < U ? cnt - k * U : U;
+      if (cls == 0) { WarpTile x; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.row = row; x.moff = moff; L.fwt[at_w++] = x; }
+      else { FusedCta x; x.w = blockIdx.y; x.cls = 1; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.wt_first = 0; x.wt_count = 0;
+             x.row = row; x.moff = moff; L.fcta[at_c++] = x; }
+    }
+  }
+  for (u32 j = threadIdx.x; j < n0; j += EMIT_THREADS) {
+    FusedCta x; x.w = blockIdx.y; x.cls = 0; x.c = 0; x.seq_off = 0; x.count = 0; x.sum_idx = 0; x.moff = 0;
+    x.row = RangeRow{0, 0, 0, 0, 0, 0, 0, 0};
+    x.wt_first = wt_base + FUSED_WT_PER_CTA * j; x.wt_count = wt_total - FUSED_WT_PER_CTA * j < FUSED_WT_PER_CTA ? wt_total - FUSED_WT_PER_CTA * j : FUSED_WT_PER_CTA;
+    L.fcta[cta_base + j] = x;
+  }
+}
+
+}  // namespace ccld
