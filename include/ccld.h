@@ -438,6 +438,8 @@ int ccld_ring_locate_static(int device, void* cuda_stream, uint32_t n_members, c
 
 /* Utility for inspection tools: synchronous copy of `bytes` bytes from device memory of this context to host memory. */
 int ccld_copy_to_host(ccld_ctx* ctx, void* dst_host, const void* src_device, uint64_t bytes);
+/* The same for n arrays at once (array i: bytes[i] bytes from src_device[i] to dst_host[i]), with one wait for all of them. */
+int ccld_copy_many_to_host(ccld_ctx* ctx, uint32_t n, void* const* dst_host, const void* const* src_device, const uint64_t* bytes);
 
 #ifdef __cplusplus
 }

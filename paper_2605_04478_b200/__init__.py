@@ -26,7 +26,7 @@ EXPORTS = ("ccld_params_default", "ccld_create", "ccld_destroy", "ccld_last_erro
            "ccld_trace_upload", "ccld_window_release", "ccld_analyze_window", "ccld_reset", "ccld_get_verdict",
            "ccld_locate_hang", "ccld_get_optable", "ccld_get_ranges", "ccld_get_rank_stats", "ccld_copy_to_host",
            "ccld_timing_enable", "ccld_get_kernel_times", "ccld_set_speculation", "ccld_ring_locate_static", "ccld_derive_rates", "ccld_locate_hangs", "ccld_state_export", "ccld_state_import", "ccld_trace_attach_opset", "ccld_opset_check",
-           "ccld_comm_set_layers")
+           "ccld_comm_set_layers", "ccld_copy_many_to_host")
 STATIC_MAX_MEMBERS = 8192
 KERNEL_KINDS = ("k_seq_range", "k_plan", "k_slot_scatter", "k_reduce_fused", "k_reduce_mid", "k_reduce_large", "k_window_decide")
 
@@ -134,6 +134,7 @@ def load_library() -> C.CDLL:
         lib.ccld_get_ranges.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_uint32, C.POINTER(C.c_uint32)]
         lib.ccld_get_rank_stats.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_copy_to_host.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_uint64]
+        lib.ccld_copy_many_to_host.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_derive_rates.argtypes = [C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p, C.c_uint32, C.c_uint64] + [C.c_void_p] * 6
         lib.ccld_timing_enable.argtypes = [C.c_void_p, C.c_int]
         lib.ccld_get_kernel_times.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p]
@@ -215,6 +216,7 @@ class Analyzer:
             raise CcldError(rc, "ccld_create failed")
         self._keep: Dict[int, list] = {}
         self._bufs: Dict[type, np.ndarray] = {}
+        self._n_comms = 0
 
     # -- helpers
     def _check(self, rc: int):
@@ -233,16 +235,20 @@ class Analyzer:
         except Exception:
             pass
 
-    def _to_host(self, ptr, count: int, dtype) -> np.ndarray:
-        out = np.empty(count, dtype=dtype)
-        if count:
-            self._check(self.lib.ccld_copy_to_host(self.h, out.ctypes.data, ptr, out.nbytes))
+    def _to_host(self, arrays):
+        """[(device pointer, count, dtype)] -> numpy arrays, with one wait for all of them."""
+        out = [np.empty(n, dtype) for _, n, dtype in arrays]
+        k = len(out)
+        dst = (C.c_void_p * k)(*[a.ctypes.data for a in out]); src = (C.c_void_p * k)(*[p for p, _, _ in arrays])
+        size = (C.c_uint64 * k)(*[a.nbytes for a in out])
+        self._check(self.lib.ccld_copy_many_to_host(self.h, k, dst, src, size))
         return out
 
     # -- the boundary
     def comm_register(self, comm: int, ranks, algo: int = 0, seq0: int = 0) -> None:
         r = np.ascontiguousarray(np.asarray(ranks, dtype=np.uint32))
         self._check(self.lib.ccld_comm_register(self.h, comm, r.ctypes.data, len(r), algo, seq0))
+        self._n_comms += 1
 
     def comm_set_layers(self, comm: int, layers) -> None:
         a = np.ascontiguousarray(np.asarray(layers, dtype=np.uint32))
@@ -251,30 +257,28 @@ class Analyzer:
     def trace_upload(self, window_id: int, cols, frames=None, n_channels: int = 0) -> None:
         """cols: dict of torch tensors or numpy arrays, all on the CPU (copied) or all on this GPU (borrowed)."""
         torch = self.torch
-        t = {}
+        t, ptrs, cuda = {}, [], set()
         for k, dt in _COL_DTYPES.items():
             v = cols.get(k)
             if v is None:
-                t[k] = None
+                t[k] = None; ptrs.append(None)
                 continue
             v = _as_tensor(torch, v, dt)
-            assert str(v.dtype) == "torch." + dt, (k, v.dtype)
-            t[k] = v.contiguous()
-        devs = {v.device.type for v in t.values() if v is not None}
+            assert v.dtype is getattr(torch, dt), (k, v.dtype)
+            t[k] = v = v.contiguous()
+            cuda.add(v.is_cuda)
+            ptrs.append(v.data_ptr() if v.numel() else None)
         fr = {}
         if frames is not None:
             for k in ("f_rank", "f_comm", "f_seq", "progress"):
                 fr[k] = _as_tensor(torch, frames[k], "int32").contiguous()
-                devs.add(fr[k].device.type)
-        assert len(devs) == 1, "all columns must live on the same device"
-        mem_kind = 1 if devs.pop() == "cuda" else 0
+                cuda.add(fr[k].is_cuda)
+        assert len(cuda) == 1, "all columns must live on the same device"
+        mem_kind = 1 if cuda.pop() else 0
         n = int(t["rank"].numel())
         ptr = lambda v: C.c_void_p(v.data_ptr()) if v is not None and v.numel() else C.c_void_p(0)
         nf = int(fr["f_rank"].numel()) if fr else 0
-        rc = self.lib.ccld_trace_upload(self.h, window_id, n, mem_kind, ptr(t["rank"]), ptr(t["comm"]), ptr(t["seq"]), ptr(t["op"]),
-                                        ptr(t["bytes"]), ptr(t["t_enter"]), ptr(t["t_exit"]), ptr(t["send_chg"]), ptr(t["recv_chg"]),
-                                        nf, ptr(fr.get("f_rank")), ptr(fr.get("f_comm")), ptr(fr.get("f_seq")), n_channels,
-                                        ptr(fr.get("progress")))
+        rc = self.lib.ccld_trace_upload(self.h, window_id, n, mem_kind, *ptrs, nf, ptr(fr.get("f_rank")), ptr(fr.get("f_comm")), ptr(fr.get("f_seq")), n_channels, ptr(fr.get("progress")))
         self._check(rc)
         self._keep[window_id] = [t, fr]            # borrowed device memory / pinned host memory stays alive
 
@@ -386,9 +390,8 @@ class Analyzer:
 
     def get_ranges(self, window_id: int) -> Dict[str, np.ndarray]:
         n = C.c_uint32(0)
-        self._check(self.lib.ccld_get_ranges(self.h, window_id, None, 0, C.byref(n)))
-        rows = self._list_buf(CommRange, n.value)
-        self._check(self.lib.ccld_get_ranges(self.h, window_id, rows.ctypes.data, n.value, C.byref(n)))
+        rows = self._list_buf(CommRange, self._n_comms)          # a window has at most one row per communicator
+        self._check(self.lib.ccld_get_ranges(self.h, window_id, rows.ctypes.data, self._n_comms, C.byref(n)))
         return self._columns(rows, n.value)
 
     def get_optable(self, window_id: int, to_host: bool = True) -> Dict[str, object]:
@@ -399,13 +402,9 @@ class Analyzer:
         if not to_host:
             return {k: getattr(t, k) for k, _ in OpTable._fields_}
         out: Dict[str, object] = {"n_groups": G, "n_slots": S}
-        for k in OPTABLE_I64:
-            out[k] = self._to_host(getattr(t, k), G, np.int64)
-        for k in OPTABLE_U32:
-            out[k] = self._to_host(getattr(t, k), G, np.uint32)
-        out["busbw"] = self._to_host(t.busbw, G, np.float64)
-        out["flags"] = self._to_host(t.flags, S, np.uint8)
-        out["perm"] = self._to_host(t.perm, S, np.uint32)
+        cols = [(k, G, np.int64) for k in OPTABLE_I64] + [(k, G, np.uint32) for k in OPTABLE_U32] + [("busbw", G, np.float64), ("flags", S, np.uint8), ("perm", S, np.uint32)]
+        for (k, _, _), a in zip(cols, self._to_host([(getattr(t, k), n, dt) for k, n, dt in cols])):
+            out[k] = a
         # per-group communicator id, op counter and first slot, expanded from the range rows
         r = self.get_ranges(window_id)
         ns = r["n_seq"].astype(np.int64)
@@ -443,7 +442,7 @@ class Analyzer:
         return out_s, out_r
 
     def get_rank_stats(self, n_ranks: int) -> Dict[str, np.ndarray]:
-        votes = np.zeros((n_ranks, 4), np.uint32); ops = np.zeros(n_ranks, np.uint32)
-        cnt = np.zeros(n_ranks, np.uint32); bw = np.zeros(n_ranks, np.float64)
+        votes = np.empty((n_ranks, 4), np.uint32); ops = np.empty(n_ranks, np.uint32)
+        cnt = np.empty(n_ranks, np.uint32); bw = np.empty(n_ranks, np.float64)
         self._check(self.lib.ccld_get_rank_stats(self.h, n_ranks, votes.ctypes.data, ops.ctypes.data, cnt.ctypes.data, bw.ctypes.data))
         return {"votes": votes, "ops": ops, "bw_cnt": cnt, "bw_sum": bw}

@@ -2,12 +2,15 @@
 // read-back. No analysis arithmetic lives here; every step of the hot path is a kernel in
 // ccld_kernels.cuh.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <string>
+#include <thread>
 #include <unordered_map>
 #include <vector>
 
@@ -34,8 +37,44 @@ struct CommHost {
   const u32* d_head = nullptr;      // device copy inside the registry block
 };
 
+// What contexts that are gone leave to those that live: a process-wide store of pinned and device blocks. Allocating is what a
+// context's first pass costs most (measured: cudaMallocHost 1 to 13 ms, cudaMalloc 0.36 ms whatever the size), and programs
+// make a context per job or per device. The store is bounded, every access holds its lock, blocks enter it only once their
+// stream has been waited for, and it is emptied when the last context goes or an allocation fails.
+class BlockStore {
+ public:
+  static BlockStore& get() { static BlockStore* s = new BlockStore; return *s; }      // never destroyed: contexts may outlive static objects
+  void enter() { std::lock_guard<std::mutex> g(m_); ++users_; }
+  void leave() { std::lock_guard<std::mutex> g(m_); if (--users_ == 0) drain(); }
+  bool take(int device, size_t bytes, Block* out) {       // device < 0: pinned
+    std::lock_guard<std::mutex> g(m_);
+    auto& l = lists_[device];
+    int best = -1;
+    for (size_t i = 0; i < l.size(); ++i) if (l[i].bytes >= bytes && l[i].bytes <= 2 * bytes + (1u << 20) && (best < 0 || l[i].bytes < l[best].bytes)) best = (int)i;
+    if (best < 0) return false;
+    *out = l[best]; l.erase(l.begin() + best); held_[device] -= out->bytes;
+    return true;
+  }
+  void put(int device, Block b) {
+    if (!b.p) return;
+    std::lock_guard<std::mutex> g(m_);
+    const size_t most = device < 0 ? PINNED_MOST : DEVICE_MOST;
+    if (held_[device] + b.bytes > most) { free_block(device, b); return; }
+    held_[device] += b.bytes; lists_[device].push_back(b);
+  }
+  void clear() { std::lock_guard<std::mutex> g(m_); drain(); }
+
+ private:
+  static constexpr size_t PINNED_MOST = 64u << 20, DEVICE_MOST = 512u << 20;
+  static void free_block(int device, Block b) { if (device < 0) cudaFreeHost(b.p); else cudaFree(b.p); }   // (cudaFree takes any device's pointer)
+  void drain() { for (auto& kv : lists_) { for (Block& b : kv.second) free_block(kv.first, b); kv.second.clear(); held_[kv.first] = 0; } }
+  std::mutex m_; int users_ = 0;
+  std::map<int, std::vector<Block>> lists_; std::map<int, size_t> held_;
+};
+
 // Device blocks are recycled through a free list so that steady-state analysis allocates nothing.
 struct Pool {
+  int device = 0;
   std::vector<Block> free_list;
   Block get(size_t bytes, cudaError_t* err) {
     bytes = align_up(std::max<size_t>(bytes, ALIGN));
@@ -43,18 +82,22 @@ struct Pool {
     for (size_t i = 0; i < free_list.size(); ++i)
       if (free_list[i].bytes >= bytes && free_list[i].bytes <= 2 * bytes + (1u << 20) && (best < 0 || free_list[i].bytes < free_list[best].bytes)) best = (int)i;
     if (best >= 0) { Block b = free_list[best]; free_list.erase(free_list.begin() + best); *err = cudaSuccess; return b; }
-    Block b; b.bytes = bytes;
+    Block b;
+    if (BlockStore::get().take(device, bytes, &b)) { *err = cudaSuccess; return b; }
+    b.bytes = bytes;
     *err = cudaMalloc(&b.p, bytes);
     if (*err != cudaSuccess) {                 // give cached blocks back to the driver and retry once
+      cudaGetLastError();
       for (auto& f : free_list) cudaFree(f.p);
       free_list.clear();
+      BlockStore::get().clear();
       *err = cudaMalloc(&b.p, bytes);
       if (*err != cudaSuccess) { b.p = nullptr; b.bytes = 0; }
     }
     return b;
   }
   void put(Block b) { if (b.p) free_list.push_back(b); }
-  void clear() { for (auto& f : free_list) cudaFree(f.p); free_list.clear(); }
+  void leave_all() { for (auto& f : free_list) BlockStore::get().put(device, f); free_list.clear(); }      // the stream must be idle
 };
 
 struct Shared {                                 // a pooled block shared by the windows of one batch
@@ -79,10 +122,16 @@ struct WindowHost {
 // A batch that was enqueued on totals the host expected instead of waiting for the plan: its actual totals arrive in
 // pinned memory behind the batch's kernels and are checked at the next call that synchronizes anyway.
 // A batch that waited is listed only for its pinned block, which its last descriptor copy still reads.
-struct PendingBatch { u32 first = 0, n = 0; i64 now = 0; u64* h_tot = nullptr; size_t h_bytes = 0; bool speculative = false; };
+struct PendingBatch { u32 first = 0, n = 0; i64 now = 0; Block pin; bool speculative = false; const u64* h_tot() const { return (const u64*)pin.p; } };
 // Totals of the last batches that were planned with a wait, by shape (record count of every window).
 struct ShapeEntry { std::vector<u64> n_rec; std::vector<u64> totals; };
 constexpr size_t SHAPE_CACHE = 4;
+
+// Pinned pieces that uploads of pageable memory pass through, with an event behind the last copy out of each.
+struct UploadSlot { char* p = nullptr; cudaEvent_t done = nullptr; bool used = false; };
+constexpr size_t UP_PIECE = 1u << 20;                      // a large upload goes piece by piece
+constexpr u32 UP_WORKERS = 6, UP_SLOTS = 2 * UP_WORKERS;   // two pieces per worker: one being filled, one on its way
+constexpr size_t UP_SMALL = 256u << 10;                    // up to this size one piece takes the whole upload, pinned columns too
 
 constexpr u32 TIMER_RING = 32;
 constexpr int TIMER_PAIRS = CCLD_K_KINDS + 1;          // the layout kernel runs twice per call
@@ -98,9 +147,11 @@ struct ccld_ctx {
   const TreeRef* d_trees = nullptr; u32 n_trees = 0;     // tree communicators whose layers are known
   std::map<u32, WindowHost> windows;
   Pool pool; std::string err;
-  char* h_verdict = nullptr;                             // pinned area of ccld_get_verdict (VerdictArea)
+  Block h_verdict;                                       // pinned area of ccld_get_verdict (VerdictArea)
+  Block h_io;                                            // pinned area small results pass through
+  Block h_up; UploadSlot up[UP_SLOTS]; u32 up_next = 0;
   u64 batches_redone = 0;                                // batches settle() had to analyse again
-  std::vector<PendingBatch> pending; std::vector<std::pair<u64*, size_t>> pinned_free; std::vector<ShapeEntry> shapes;
+  std::vector<PendingBatch> pending; std::vector<Block> pinned_free; std::vector<ShapeEntry> shapes;
   u32* d_poison = nullptr; int speculate = 1;
   // optional per-kernel timing: a ring of event pairs, harvested lazily
   bool timing = false; std::vector<TimerSlot> ring; u32 ring_next = 0;
@@ -290,13 +341,122 @@ void drop_results(WindowHost& w) {
 
 int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bool may_speculate);
 
-u64* pinned_get(ccld_ctx* ctx, size_t bytes, size_t* got) {
+Block pinned_get(ccld_ctx* ctx, size_t bytes) {
   for (size_t i = 0; i < ctx->pinned_free.size(); ++i)
-    if (ctx->pinned_free[i].second >= bytes) { auto p = ctx->pinned_free[i]; ctx->pinned_free.erase(ctx->pinned_free.begin() + i); *got = p.second; return p.first; }
-  u64* p = nullptr;
-  if (cudaMallocHost((void**)&p, bytes) != cudaSuccess) return nullptr;
-  *got = bytes;
-  return p;
+    if (ctx->pinned_free[i].bytes >= bytes) { Block b = ctx->pinned_free[i]; ctx->pinned_free.erase(ctx->pinned_free.begin() + i); return b; }
+  Block b;
+  if (BlockStore::get().take(-1, bytes, &b)) return b;
+  b.bytes = (bytes + 65535) / 65536 * 65536;              // whole 64 KB pieces, so that blocks fit other batches too
+  if (cudaMallocHost(&b.p, b.bytes) != cudaSuccess) {
+    cudaGetLastError();
+    BlockStore::get().clear();
+    if (cudaMallocHost(&b.p, b.bytes) != cudaSuccess) { cudaGetLastError(); b.p = nullptr; b.bytes = 0; }
+  }
+  return b;
+}
+// A pinned area of the context of at least `bytes` bytes. Nothing in flight may still use it.
+int pinned_area(ccld_ctx* ctx, Block& area, size_t bytes) {
+  if (area.bytes >= bytes) return CCLD_OK;
+  BlockStore::get().put(-1, area);
+  area = pinned_get(ctx, bytes);
+  return area.p ? CCLD_OK : fail(ctx, CCLD_ERR_NOMEM, "pinned allocation failed");
+}
+
+// Copies device arrays to host memory, all with one wait. Up to FETCH_PINNED bytes in all pass through pinned memory, written
+// there by one kernel: a copy each into pageable memory costs 15 to 20 us apiece, the kernel about 5 us for all. More than
+// that is left to the driver's copies, whose fixed cost no longer counts.
+struct Piece { const void* src; void* dst; size_t n; };
+constexpr size_t FETCH_PINNED = 4u << 20;
+int fetch(ccld_ctx* ctx, const Piece* piece, u32 n_pieces) {
+  size_t total = 0, most = 0;
+  for (u32 i = 0; i < n_pieces; ++i) { total += piece[i].n; most = std::max(most, piece[i].n); }
+  if (total > FETCH_PINNED || n_pieces > GATHER_PIECES) {
+    for (u32 i = 0; i < n_pieces; ++i) if (piece[i].n) CK(cudaMemcpyAsync(piece[i].dst, piece[i].src, piece[i].n, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    return CCLD_OK;
+  }
+  if (total == 0) { CK(cudaStreamSynchronize(ctx->stream)); return CCLD_OK; }
+  { int rc = pinned_area(ctx, ctx->h_io, total + 32ull * n_pieces); if (rc != CCLD_OK) return rc; }
+  GatherArgs A; size_t at[GATHER_PIECES], off = 0; u32 k = 0;
+  unsigned char* base = (unsigned char*)ctx->h_io.p;
+  for (u32 i = 0; i < n_pieces; ++i) {
+    at[i] = (off + 15) / 16 * 16 + ((uintptr_t)piece[i].src & 15);
+    off = at[i] + piece[i].n;
+    if (piece[i].n) { A.piece[k].src = (const unsigned char*)piece[i].src; A.piece[k].dst = base + at[i]; A.piece[k].n = piece[i].n; ++k; }
+  }
+  k_gather<<<dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), k), GATHER_THREADS, 0, ctx->stream>>>(A);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(ctx->stream));
+  for (u32 i = 0; i < n_pieces; ++i) if (piece[i].n) std::memcpy(piece[i].dst, base + at[i], piece[i].n);
+  return CCLD_OK;
+}
+
+// Host columns on their way into one device block.
+struct UpCol { size_t off; const void* src; size_t n; };
+int upload_slots(ccld_ctx* ctx) {
+  if (ctx->h_up.p) return CCLD_OK;
+  for (UploadSlot& u : ctx->up) if (!u.done) CK(cudaEventCreateWithFlags(&u.done, cudaEventDisableTiming));
+  ctx->h_up = pinned_get(ctx, UP_PIECE * UP_SLOTS);
+  if (!ctx->h_up.p) return fail(ctx, CCLD_ERR_NOMEM, "pinned allocation failed");
+  for (u32 i = 0; i < UP_SLOTS; ++i) { ctx->up[i].p = (char*)ctx->h_up.p + i * UP_PIECE; ctx->up[i].used = false; }
+  return CCLD_OK;
+}
+// Copies the columns to `base` (device, `total` bytes with the columns at their offsets). The driver copies pageable memory
+// column by column through its own buffers, one thread, 10 us and more per call. A small upload is put together in one
+// pinned piece instead and crosses in one copy; a large pageable one is cut into pieces that several threads fill while
+// earlier ones cross. Large pinned columns go straight across.
+int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u32 n_cols) {
+  cudaStream_t st = ctx->stream;
+  size_t bytes = 0; const void* first = nullptr;
+  for (u32 i = 0; i < n_cols; ++i) { bytes += col[i].n; if (col[i].n && !first) first = col[i].src; }
+  if (bytes == 0) return CCLD_OK;
+  bool pinned = false;
+  if (total > UP_SMALL) {
+    cudaPointerAttributes at;
+    pinned = cudaPointerGetAttributes(&at, first) == cudaSuccess && at.type != cudaMemoryTypeUnregistered;
+    cudaGetLastError();
+  }
+  if (pinned) {
+    for (u32 i = 0; i < n_cols; ++i) if (col[i].n) CK(cudaMemcpyAsync(base + col[i].off, col[i].src, col[i].n, cudaMemcpyHostToDevice, st));
+    return CCLD_OK;
+  }
+  { int rc = upload_slots(ctx); if (rc != CCLD_OK) return rc; }
+  if (total <= UP_PIECE) {
+    UploadSlot& u = ctx->up[ctx->up_next++ % UP_SLOTS];
+    if (u.used) CK(cudaEventSynchronize(u.done));
+    for (u32 i = 0; i < n_cols; ++i) if (col[i].n) std::memcpy(u.p + col[i].off, col[i].src, col[i].n);
+    CK(cudaMemcpyAsync(base, u.p, total, cudaMemcpyHostToDevice, st));
+    CK(cudaEventRecord(u.done, st));
+    u.used = true;
+    return CCLD_OK;
+  }
+  std::vector<UpCol> piece;
+  for (u32 i = 0; i < n_cols; ++i)
+    for (size_t a = 0; a < col[i].n; a += UP_PIECE) piece.push_back(UpCol{col[i].off + a, (const char*)col[i].src + a, std::min(UP_PIECE, col[i].n - a)});
+  std::atomic<u32> next{0}; std::atomic<int> err{(int)cudaSuccess};
+  const int device = ctx->device;
+  auto work = [&](u32 me) {
+    if (cudaSetDevice(device) != cudaSuccess) { err = (int)cudaErrorInvalidDevice; return; }
+    for (u32 turn = 0; err == (int)cudaSuccess; turn ^= 1) {
+      const u32 k = next.fetch_add(1);
+      if (k >= piece.size()) break;
+      UploadSlot& u = ctx->up[2 * me + turn];
+      cudaError_t e = u.used ? cudaEventSynchronize(u.done) : cudaSuccess;
+      if (e == cudaSuccess) { std::memcpy(u.p, piece[k].src, piece[k].n); e = cudaMemcpyAsync(base + piece[k].off, u.p, piece[k].n, cudaMemcpyHostToDevice, st); }
+      if (e == cudaSuccess) e = cudaEventRecord(u.done, st);
+      u.used = true;
+      if (e != cudaSuccess) err = (int)e;
+    }
+  };
+  const u32 workers = std::max(1u, std::min({UP_WORKERS, (u32)(piece.size() / 4), std::thread::hardware_concurrency() / 2}));
+  std::vector<std::thread> crew;
+  for (u32 i = 1; i < workers; ++i) {
+    try { crew.emplace_back(work, i); } catch (...) { break; }      // no more threads to be had: fewer do the work
+  }
+  work(0);
+  for (auto& t : crew) t.join();
+  CK((cudaError_t)err.load());
+  return CCLD_OK;
 }
 
 // Brings the batches that were enqueued on expected totals to a definite state: waits for the stream, reads the totals
@@ -308,18 +468,18 @@ int settle(ccld_ctx* ctx) {
   CK(cudaSetDevice(ctx->device));
   CK(cudaStreamSynchronize(ctx->stream));
   std::vector<PendingBatch> todo;
-  for (PendingBatch& b : ctx->pending) { if (b.speculative) todo.push_back(b); else ctx->pinned_free.emplace_back(b.h_tot, b.h_bytes); }
+  for (PendingBatch& b : ctx->pending) { if (b.speculative) todo.push_back(b); else ctx->pinned_free.push_back(b.pin); }
   ctx->pending.clear();
   bool failed = false;
   int rc = CCLD_OK;
   for (PendingBatch& b : todo) {
-    for (u32 k = 0; k < b.n && !failed; ++k) if (b.h_tot[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) failed = true;
-    ctx->pinned_free.emplace_back(b.h_tot, b.h_bytes);
+    for (u32 k = 0; k < b.n && !failed; ++k) if (b.h_tot()[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) failed = true;
+    ctx->pinned_free.push_back(b.pin);
     if (!failed) {
       // a window may still have been refused for its size, which the expectation cannot have foreseen: keep what the plan found
       for (u32 k = 0; k < b.n; ++k) {
         auto it = ctx->windows.find(b.first + k);
-        if (it != ctx->windows.end() && it->second.analysed) std::memcpy(it->second.totals, b.h_tot + (size_t)k * T_COUNT, sizeof it->second.totals);
+        if (it != ctx->windows.end() && it->second.analysed) std::memcpy(it->second.totals, b.h_tot() + (size_t)k * T_COUNT, sizeof it->second.totals);
       }
       continue;
     }
@@ -328,7 +488,7 @@ int settle(ccld_ctx* ctx) {
   CK(cudaMemsetAsync(ctx->d_poison, 0, 4, ctx->stream));
   failed = false;
   for (PendingBatch& b : todo) {
-    if (!failed) { for (u32 k = 0; k < b.n && !failed; ++k) if (b.h_tot[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) failed = true; }
+    if (!failed) { for (u32 k = 0; k < b.n && !failed; ++k) if (b.h_tot()[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) failed = true; }
     if (!failed) continue;
     bool present = true;
     for (u32 k = 0; k < b.n; ++k) {
@@ -373,7 +533,8 @@ int ccld_create(ccld_ctx** out, const ccld_params* params, int device, void* cud
   if (cudaSetDevice(device) != cudaSuccess) return CCLD_ERR_CUDA;
   ccld_ctx* ctx = new (std::nothrow) ccld_ctx();
   if (!ctx) return CCLD_ERR_NOMEM;
-  ctx->params = *params; ctx->device = device; ctx->stream = (cudaStream_t)cuda_stream;
+  ctx->params = *params; ctx->device = device; ctx->pool.device = device; ctx->stream = (cudaStream_t)cuda_stream;
+  BlockStore::get().enter();
   { int sms = 0; if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess && sms > 0) ctx->n_sms = (u32)sms; }
   Params& d = ctx->dp;
   d.tbase_init_ns = params->tbase_init_ns; d.m_max_ns = params->m_max_ns; d.hang_ns = params->hang_ns; d.barrier_bytes = params->barrier_bytes;
@@ -388,13 +549,15 @@ int ccld_destroy(ccld_ctx* ctx) {
   if (!ctx) return CCLD_ERR_ARG;
   cudaSetDevice(ctx->device);
   cudaStreamSynchronize(ctx->stream);
-  for (auto& kv : ctx->windows) { drop_results(kv.second); if (kv.second.owns) ctx->pool.put(kv.second.own); }
+  for (auto& kv : ctx->windows) { drop_results(kv.second); if (kv.second.owns) ctx->pool.put(kv.second.own); if (kv.second.owns_opset) ctx->pool.put(kv.second.opset_own); }
   ctx->windows.clear();
   ctx->pool.put(ctx->reg_blk); ctx->pool.put(ctx->misc_blk);
-  ctx->pool.clear();
-  if (ctx->h_verdict) cudaFreeHost(ctx->h_verdict);
-  for (auto& b : ctx->pending) cudaFreeHost(b.h_tot);
-  for (auto& f : ctx->pinned_free) cudaFreeHost(f.first);
+  ctx->pool.leave_all();
+  for (auto& b : ctx->pending) ctx->pinned_free.push_back(b.pin);
+  ctx->pinned_free.push_back(ctx->h_verdict); ctx->pinned_free.push_back(ctx->h_io); ctx->pinned_free.push_back(ctx->h_up);
+  for (UploadSlot& u : ctx->up) if (u.done) cudaEventDestroy(u.done);
+  for (auto& f : ctx->pinned_free) BlockStore::get().put(-1, f);
+  BlockStore::get().leave();
   for (auto& sl : ctx->ring) for (int i = 0; i < TIMER_PAIRS; ++i) { cudaEventDestroy(sl.a[i]); cudaEventDestroy(sl.b[i]); }
   delete ctx;
   return CCLD_OK;
@@ -465,16 +628,12 @@ int ccld_trace_upload(ccld_ctx* ctx, uint32_t window_id, uint64_t n_rec, int mem
     w.own = ctx->pool.get(off, &e);
     if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "window allocation failed");
     w.owns = true;
-    char* b = (char*)w.own.p; cudaStream_t st = ctx->stream;
-    auto up = [&](size_t o, const void* src, size_t nb) { return nb ? cudaMemcpyAsync(b + o, src, nb, cudaMemcpyHostToDevice, st) : cudaSuccess; };
-    cudaError_t ce = cudaSuccess;
-    auto acc = [&](cudaError_t x) { if (ce == cudaSuccess) ce = x; };
-    acc(up(o_rank, rank, n_rec * 4)); acc(up(o_comm, comm, n_rec * 4)); acc(up(o_seq, seq, n_rec * 4)); acc(up(o_op, op, n_rec));
-    acc(up(o_bytes, bytes, n_rec * 8)); acc(up(o_te, t_enter_ns, n_rec * 8)); acc(up(o_tx, t_exit_ns, n_rec * 8));
-    if (send_chg) { acc(up(o_sc, send_chg, n_rec * 4)); acc(up(o_rc, recv_chg, n_rec * 4)); }
-    if (n_frames) { acc(up(o_fr, f_rank, n_frames * 4ull)); acc(up(o_fc, f_comm, n_frames * 4ull)); acc(up(o_fs, f_seq, n_frames * 4ull));
-                    acc(up(o_pr, progress, (size_t)n_frames * n_channels * 8)); }
-    if (ce != cudaSuccess) { ctx->pool.put(w.own); return fail(ctx, CCLD_ERR_CUDA, std::string("upload copy: ") + cudaGetErrorString(ce)); }
+    char* b = (char*)w.own.p;
+    const size_t chg = send_chg ? n_rec * 4 : 0, fr = n_frames * 4ull;
+    const UpCol col[] = {{o_rank, rank, n_rec * 4}, {o_comm, comm, n_rec * 4}, {o_seq, seq, n_rec * 4}, {o_op, op, n_rec}, {o_bytes, bytes, n_rec * 8},
+                         {o_te, t_enter_ns, n_rec * 8}, {o_tx, t_exit_ns, n_rec * 8}, {o_sc, send_chg, chg}, {o_rc, recv_chg, chg},
+                         {o_fr, f_rank, fr}, {o_fc, f_comm, fr}, {o_fs, f_seq, fr}, {o_pr, progress, (size_t)n_frames * n_channels * 8}};
+    { int rc = upload_columns(ctx, b, off, col, sizeof col / sizeof col[0]); if (rc != CCLD_OK) { cudaStreamSynchronize(ctx->stream); ctx->pool.put(w.own); return rc; } }
     d.rank = (const u32*)(b + o_rank); d.comm = (const u32*)(b + o_comm); d.seq = (const u32*)(b + o_seq); d.op = (const u8*)(b + o_op);
     d.bytes = (const u64*)(b + o_bytes); d.t_enter = (const i64*)(b + o_te); d.t_exit = (const i64*)(b + o_tx);
     d.send_chg = send_chg ? (const u32*)(b + o_sc) : nullptr; d.recv_chg = recv_chg ? (const u32*)(b + o_rc) : nullptr;
@@ -503,7 +662,7 @@ int ccld_reset(ccld_ctx* ctx) {
   CK(cudaSetDevice(ctx->device));
   CK(cudaStreamSynchronize(ctx->stream));
   // batches still in doubt need no second analysis: their results are dropped with all the others
-  for (auto& b : ctx->pending) ctx->pinned_free.emplace_back(b.h_tot, b.h_bytes);
+  for (auto& b : ctx->pending) ctx->pinned_free.push_back(b.pin);
   ctx->pending.clear();
   for (auto& kv : ctx->windows) drop_results(kv.second);
   if (ctx->finalized) {
@@ -574,13 +733,13 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   // pinned: the totals the layout finds, then the descriptors and expected totals on their way to the device. It belongs to
   // the batch until the next call that synchronizes.
   PendingBatch pbatch; pbatch.first = first_window; pbatch.n = B; pbatch.now = now_ns; pbatch.speculative = expect != nullptr;
-  pbatch.h_tot = pinned_get(ctx, align_up(tot_bytes) + up_bytes, &pbatch.h_bytes);
-  if (!pbatch.h_tot) return fail(ctx, CCLD_ERR_NOMEM, "pinned allocation failed");
+  pbatch.pin = pinned_get(ctx, align_up(tot_bytes) + up_bytes);
+  if (!pbatch.pin.p) return fail(ctx, CCLD_ERR_NOMEM, "pinned allocation failed");
   struct Guard {                                           // whatever way the call ends, the batch's pinned block is accounted for
     ccld_ctx* ctx; PendingBatch& b; bool queued = false;
-    ~Guard() { if (!queued) { cudaStreamSynchronize(ctx->stream); ctx->pinned_free.emplace_back(b.h_tot, b.h_bytes); } }
+    ~Guard() { if (!queued) { cudaStreamSynchronize(ctx->stream); ctx->pinned_free.push_back(b.pin); } }
   } guard{ctx, pbatch};
-  char* const h_up = (char*)pbatch.h_tot + align_up(tot_bytes);
+  char* const h_up = (char*)pbatch.pin.p + align_up(tot_bytes);
   WinDesc* const hd = (WinDesc*)h_up;
   u64 cta = 0;
   for (u32 k = 0; k < B; ++k) {
@@ -591,7 +750,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     d.ranges = (RangeRow*)(pbase + o_rng) + (size_t)k * nc; d.srow = (uint4*)(pbase + o_srow) + (size_t)k * nc;
     d.rent = (uint4*)(pbase + o_rent) + (size_t)k * ctx->n_ranks * RANK_TAB_K;
     d.totals = (u64*)(pbase + o_tot) + (size_t)k * T_COUNT; d.counters = (u64*)(pbase + o_cnt) + (size_t)k * C_COUNT;
-    d.chunks = (uint2*)(pbase + o_chunk) + (size_t)k * (CHUNK_MAX + 1); d.totals_host = pbatch.h_tot + (size_t)k * T_COUNT;
+    d.chunks = (uint2*)(pbase + o_chunk) + (size_t)k * (CHUNK_MAX + 1); d.totals_host = (u64*)pbatch.pin.p + (size_t)k * T_COUNT;
     d.expect = expect ? (const u64*)(pbase + o_exp) + (size_t)k * T_COUNT : nullptr; d.poison = ctx->d_poison;
     d.n_groups = d.n_slots = 0; d.perm = nullptr; d.flags = nullptr; d.skey = d.dkey = nullptr; d.gi64 = nullptr; d.gu32 = nullptr; d.gbw = nullptr;
     d.comm_rows = nullptr; d.alerts = nullptr;
@@ -624,7 +783,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   if (!expect) {
     CK(start_plan(0));
     CK(cudaStreamSynchronize(st));
-    found.assign(pbatch.h_tot, pbatch.h_tot + (size_t)B * T_COUNT);
+    found.assign(pbatch.h_tot(), pbatch.h_tot() + (size_t)B * T_COUNT);
     tot = found.data();
   } else tot = expect->totals.data();
 
@@ -748,7 +907,7 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
   CK(cudaSetDevice(ctx->device));
   // The kernels that gather the verdict are enqueued before batches still in doubt are settled: one wait serves both. In
   // the rare case that a batch has to be analysed again (settle() counts those) what was gathered is gathered once more.
-  const VerdictHead* head = nullptr; VerdictArea area{};
+  const VerdictHead* head = nullptr; VerdictArea area{}; char* hv = nullptr;
   u32 n_rows = 0;
   char* m = (char*)ctx->misc_blk.p;
   MiscLayout L{};
@@ -758,15 +917,16 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
     else w = &it->second;
     area = verdict_area(ctx->reg.n_comms, ctx->n_ranks);
     L = misc_layout(ctx->n_ranks, ctx->max_n);
-    if (!ctx->h_verdict) CK(cudaMallocHost((void**)&ctx->h_verdict, area.total));
-    head = (const VerdictHead*)ctx->h_verdict;
+    { int rc = pinned_area(ctx, ctx->h_verdict, area.total); if (rc != CCLD_OK) return rc; }
+    hv = (char*)ctx->h_verdict.p;
+    head = (const VerdictHead*)hv;
     n_rows = std::min<u32>((u32)w->totals[T_ROWS], out->comm_rows ? out->comm_rows_cap : 0);
     VerdictArgs A;
     A.counters = w->d.counters; A.rows = w->d.comm_rows; A.n_rows = n_rows; A.alerts = w->d.alerts;
     A.keys = (u64*)(m + L.keys); A.counts = (u32*)(m + L.counts);
-    A.head = (VerdictHead*)ctx->h_verdict; A.rows_out = (ccld_comm_verdict*)(ctx->h_verdict + area.rows);
-    A.alerts_out = (ccld_hang_alert*)(ctx->h_verdict + area.alerts);
-    A.sus_host = (ccld_suspect*)(ctx->h_verdict + area.suspects); A.sus_host_cap = area.sus_cap; A.sus_dev = (ccld_suspect*)(m + L.sus);
+    A.head = (VerdictHead*)hv; A.rows_out = (ccld_comm_verdict*)(hv + area.rows);
+    A.alerts_out = (ccld_hang_alert*)(hv + area.alerts);
+    A.sus_host = (ccld_suspect*)(hv + area.suspects); A.sus_host_cap = area.sus_cap; A.sus_dev = (ccld_suspect*)(m + L.sus);
     const u32 pieces = (ctx->n_ranks + VD_THREADS - 1) / VD_THREADS;
     k_verdict_collect<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg, ctx->dp);
     if (pieces > 1) k_verdict_merge<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg);
@@ -786,15 +946,15 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
   if (!w->totals[T_FAILED] && w->n_rec - cnt[C_PRESENT] != cnt[C_REJECTED]) err |= CCLD_E_DUPLICATE;   // a slot was written twice
   out->error_bits = err;
   out->n_comm_rows_total = (u32)w->totals[T_ROWS];
-  if (n_rows) std::memcpy(out->comm_rows, ctx->h_verdict + area.rows, n_rows * sizeof(ccld_comm_verdict));
+  if (n_rows) std::memcpy(out->comm_rows, hv + area.rows, n_rows * sizeof(ccld_comm_verdict));
   // hang alerts, ordered by (communicator, seq)
   out->n_alerts_total = (u32)std::min<u64>(cnt[C_ALERTS], 0xFFFFFFFFull);
   const u32 n_al = std::min<u32>(std::min<u32>(out->n_alerts_total, CCLD_MAX_ALERTS_PER_WINDOW), out->alerts ? out->alerts_cap : 0);
-  if (n_al) std::memcpy(out->alerts, ctx->h_verdict + area.alerts, n_al * sizeof(ccld_hang_alert));
+  if (n_al) std::memcpy(out->alerts, hv + area.alerts, n_al * sizeof(ccld_hang_alert));
   // cumulative suspects
   out->n_suspects_total = head->n_suspects;
   const u32 n_out = std::min<u32>(head->n_suspects, out->suspects ? out->suspects_cap : 0);
-  if (n_out && head->n_suspects <= area.sus_cap) std::memcpy(out->suspects, ctx->h_verdict + area.suspects, n_out * sizeof(ccld_suspect));
+  if (n_out && head->n_suspects <= area.sus_cap) std::memcpy(out->suspects, hv + area.suspects, n_out * sizeof(ccld_suspect));
   else if (n_out) {
     CK(cudaMemcpyAsync(out->suspects, m + L.sus, n_out * sizeof(ccld_suspect), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
@@ -948,8 +1108,7 @@ int ccld_get_ranges(ccld_ctx* ctx, uint32_t window_id, ccld_comm_range* rows, ui
   CK(cudaSetDevice(ctx->device));
   const u32 nc = ctx->reg.n_comms;
   std::vector<RangeRow> rr(nc);
-  CK(cudaMemcpyAsync(rr.data(), w->d.ranges, nc * sizeof(RangeRow), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  { const Piece pc{w->d.ranges, rr.data(), nc * sizeof(RangeRow)}; int rc = fetch(ctx, &pc, 1); if (rc != CCLD_OK) return rc; }
   u32 k = 0;
   for (u32 c = 0; c < nc; ++c) {
     if (rr[c].n_seq == 0) continue;
@@ -966,16 +1125,10 @@ int ccld_get_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, uint32_t* votes, uint32
   if (!ctx->finalized) return fail(ctx, CCLD_ERR_STATE, "nothing analysed yet");
   { int rc = settle(ctx); if (rc != CCLD_OK) return rc; }
   CK(cudaSetDevice(ctx->device));
-  std::memset(votes, 0, (size_t)n_ranks * 16); std::memset(ops, 0, (size_t)n_ranks * 4);
-  std::memset(bw_cnt, 0, (size_t)n_ranks * 4); std::memset(bw_sum, 0, (size_t)n_ranks * 8);
-  const u32 n = std::min(n_ranks, ctx->reg.n_ranks);
-  cudaStream_t st = ctx->stream;
-  CK(cudaMemcpyAsync(votes, ctx->reg.votes, (size_t)n * 16, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(ops, ctx->reg.ops, (size_t)n * 4, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(bw_cnt, ctx->reg.bw_cnt, (size_t)n * 4, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(bw_sum, ctx->reg.bw_sum, (size_t)n * 8, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  return CCLD_OK;
+  const size_t n = std::min(n_ranks, ctx->reg.n_ranks), rest = n_ranks - n;      // ranks the registry does not know: zeros
+  std::memset(votes + n * 4, 0, rest * 16); std::memset(ops + n, 0, rest * 4); std::memset(bw_cnt + n, 0, rest * 4); std::memset(bw_sum + n, 0, rest * 8);
+  const Piece pc[4] = {{ctx->reg.votes, votes, n * 16}, {ctx->reg.ops, ops, n * 4}, {ctx->reg.bw_cnt, bw_cnt, n * 4}, {ctx->reg.bw_sum, bw_sum, n * 8}};
+  return fetch(ctx, pc, 4);
 }
 
 int ccld_trace_attach_opset(ccld_ctx* ctx, uint32_t window_id, int mem_kind, const uint8_t* algo, const uint8_t* proto) {
@@ -1136,6 +1289,17 @@ int ccld_get_kernel_times(ccld_ctx* ctx, double* ms, uint64_t* launches) {
   for (auto& sl : ctx->ring) timer_harvest(ctx, sl);
   for (int k = 0; k < CCLD_K_KINDS; ++k) { ms[k] = ctx->t_ms[k]; launches[k] = ctx->t_launches[k]; }
   return CCLD_OK;
+}
+
+int ccld_copy_many_to_host(ccld_ctx* ctx, uint32_t n, void* const* dst_host, const void* const* src_device, const uint64_t* bytes) {
+  if (!ctx || (n && (!dst_host || !src_device || !bytes))) return CCLD_ERR_ARG;
+  std::vector<Piece> pc(n);
+  for (u32 i = 0; i < n; ++i) {
+    if (bytes[i] && (!dst_host[i] || !src_device[i])) return fail(ctx, CCLD_ERR_ARG, "null array");
+    pc[i] = Piece{src_device[i], dst_host[i], bytes[i]};
+  }
+  CK(cudaSetDevice(ctx->device));
+  return fetch(ctx, pc.data(), n);
 }
 
 int ccld_copy_to_host(ccld_ctx* ctx, void* dst_host, const void* src_device, uint64_t bytes) {

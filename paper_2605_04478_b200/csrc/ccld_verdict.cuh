@@ -143,6 +143,22 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_merge(VerdictArgs A, Reg
   }
 }
 
+// Several device arrays into one pinned area, one launch: a row of CTAs per piece. Source and destination agree modulo 16, so
+// whole 16-byte words cross PCIe and only a piece's ends go byte by byte.
+constexpr int GATHER_THREADS = 256;
+constexpr u32 GATHER_PIECES = 24;
+struct GatherArgs { struct { const unsigned char* src; unsigned char* dst; u64 n; } piece[GATHER_PIECES]; };
+__global__ void __launch_bounds__(GATHER_THREADS) k_gather(GatherArgs A) {
+  const unsigned char* __restrict__ src = A.piece[blockIdx.y].src; unsigned char* __restrict__ dst = A.piece[blockIdx.y].dst;
+  const u64 n = A.piece[blockIdx.y].n;
+  const u64 head = min(n, (u64)((16 - ((uintptr_t)src & 15)) & 15)), n16 = (n - head) / 16, tail = head + n16 * 16;
+  const u64 i0 = (u64)blockIdx.x * GATHER_THREADS + threadIdx.x, st = (u64)gridDim.x * GATHER_THREADS;
+  const uint4* s16 = reinterpret_cast<const uint4*>(src + head); uint4* d16 = reinterpret_cast<uint4*>(dst + head);
+  for (u64 i = i0; i < n16; i += st) d16[i] = s16[i];
+  if (i0 < head) dst[i0] = src[i0];
+  if (i0 < n - tail) dst[tail + i0] = src[tail + i0];
+}
+
 // the ordered alerts alone, for the hang sweep
 __global__ void __launch_bounds__(VD_THREADS) k_order_alerts(const u64* __restrict__ counters, const ccld_hang_alert* __restrict__ in, ccld_hang_alert* __restrict__ out, Registry R) {
   __shared__ u64 s_key[CCLD_MAX_ALERTS_PER_WINDOW];
