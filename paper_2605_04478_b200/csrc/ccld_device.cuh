@@ -59,12 +59,15 @@ struct Registry {
   const u32* rank_ptr;      // [n_ranks+1] CSR over (communicator index, position) pairs of a rank
   const u32* ent_comm;
   const u32* ent_pos;
+  const u32* const* comm_head;   // [n_comms] trees: [n] lowest position of each member's layer (REG_NO_LAYERS: not known); null for a ring
   CommState* state;         // [n_comms]
   u32* votes;               // [n_ranks][4] skew hi, skew lo, dur hi, dur lo
   u32* ops;                 // [n_ranks]
   u32* bw_cnt;              // [n_ranks]
   double* bw_sum;           // [n_ranks]
 };
+
+#define REG_NO_LAYERS reinterpret_cast<const u32*>(1)    // never dereferenced
 
 // rank_tab: pairs beyond RANK_TAB_K do not fit inline; the last pair then holds (NONE, RANK_TAB_OVERFLOW) and the
 // CSR lists are searched instead. Empty pairs are (NONE, NONE).

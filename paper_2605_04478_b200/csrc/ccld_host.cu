@@ -202,15 +202,13 @@ struct TimedLaunch {                                     // a named range and, w
 };
 
 // Layout of the scratch block used by get_verdict and locate_hang.
-struct MiscLayout { size_t sus, keys, counts, alerts, entered, done, frame, roots, tot, hang_out, total; };
-MiscLayout misc_layout(u32 n_ranks, u32 max_n) {
+struct MiscLayout { size_t sus, keys, counts, alerts, total; };
+MiscLayout misc_layout(u32 n_ranks) {
   MiscLayout L; size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + std::max<size_t>(b, 1)); return o; };
   const size_t pieces = (n_ranks + VD_THREADS - 1) / VD_THREADS;
   L.sus = take(2ull * n_ranks * sizeof(ccld_suspect)); L.keys = take(pieces * VD_KEYS * 8); L.counts = take(pieces * 4);
   L.alerts = take(CCLD_MAX_ALERTS_PER_WINDOW * sizeof(ccld_hang_alert));
-  L.entered = take(max_n); L.done = take(max_n); L.frame = take(max_n * 4ull); L.roots = take(max_n * 4ull);
-  L.tot = take(max_n * 8ull); L.hang_out = take(sizeof(ccld_hang_verdict));
   L.total = off;
   return L;
 }
@@ -278,7 +276,7 @@ int finalize_registry(ccld_ctx* ctx) {
   std::vector<size_t> o_head(nc, 0);
   u32 n_trees = 0;
   for (u32 i = 0; i < nc; ++i) if (!ctx->comms[i].head.empty()) { o_head[i] = take(ctx->comms[i].head.size() * 4); ++n_trees; }
-  const size_t o_trees = take(std::max<u32>(n_trees, 1) * sizeof(TreeRef));
+  const size_t o_trees = take(std::max<u32>(n_trees, 1) * sizeof(TreeRef)), o_chead = take(nc * sizeof(u32*));
   const size_t o_stats = off;
   const size_t o_state = take(nc * sizeof(CommState)), o_votes = take(nr * 16ull), o_ops = take(nr * 4ull), o_cnt = take(nr * 4ull), o_bw = take(nr * 8ull);
   const size_t stats_end = off, o_poison = take(256);
@@ -303,6 +301,9 @@ int finalize_registry(ccld_ctx* ctx) {
     CK(cudaMemcpyAsync(base + o_head[i], c.head.data(), c.head.size() * 4, cudaMemcpyHostToDevice, st));
     c.d_head = (const u32*)(base + o_head[i]);
   }
+  std::vector<const u32*> comm_head(nc, nullptr);
+  for (u32 i = 0; i < nc; ++i) if (ctx->comms[i].algo != 0) comm_head[i] = ctx->comms[i].d_head ? ctx->comms[i].d_head : REG_NO_LAYERS;
+  CK(cudaMemcpyAsync(base + o_chead, comm_head.data(), nc * sizeof(u32*), cudaMemcpyHostToDevice, st));
   std::vector<TreeRef> trees;
   for (u32 i = 0; i < nc; ++i) if (ctx->comms[i].d_head) { TreeRef t; t.c = i; t.pad = 0; t.head = ctx->comms[i].d_head; trees.push_back(t); }
   if (n_trees) CK(cudaMemcpyAsync(base + o_trees, trees.data(), n_trees * sizeof(TreeRef), cudaMemcpyHostToDevice, st));
@@ -314,17 +315,20 @@ int finalize_registry(ccld_ctx* ctx) {
   R.hash = (const uint4*)(base + o_hash); R.rank_tab = (const uint4*)(base + o_rtab); R.comm_id = (const u32*)(base + o_id); R.comm_n = (const u32*)(base + o_n);
   R.comm_seq0 = (const u32*)(base + o_s0); R.comm_moff = (const u64*)(base + o_moff); R.members = (const u32*)(base + o_mem);
   R.rank_ptr = (const u32*)(base + o_ptr); R.ent_comm = (const u32*)(base + o_ec); R.ent_pos = (const u32*)(base + o_ep);
+  R.comm_head = (const u32* const*)(base + o_chead);
   R.state = (CommState*)(base + o_state); R.votes = (u32*)(base + o_votes); R.ops = (u32*)(base + o_ops);
   R.bw_cnt = (u32*)(base + o_cnt); R.bw_sum = (double*)(base + o_bw);
   ctx->stats_off = o_stats; ctx->stats_bytes = stats_end - o_stats; ctx->d_poison = (u32*)(base + o_poison);
   ctx->n_ranks = nr; ctx->max_n = max_n; ctx->max_large_n = max_large; ctx->sum_n = sum_n;
 
   // scratch for suspects, alert ordering and hang location
-  ctx->misc_blk = ctx->pool.get(misc_layout(nr, max_n).total, &e);
+  ctx->misc_blk = ctx->pool.get(misc_layout(nr).total, &e);
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
 
   CK(cudaFuncSetAttribute(k_reduce_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem_bytes(2 * WARP_N)));
   CK(cudaFuncSetAttribute(k_seq_range, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)range_smem_bytes(RANGE_DIRECT)));
+  CK(cudaFuncSetAttribute(k_hang_locate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(HANG_SMEM_N * HANG_MEMBER_BYTES)));
+  CK(cudaFuncSetAttribute(k_opset_check, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(CCLD_MAX_COMM_SIZE * OPSET_MEMBER_BYTES)));
   if (max_large) {
     ctx->large_smem = large_smem(max_large);
     CK(cudaFuncSetAttribute(k_reduce_large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->large_smem));
@@ -869,8 +873,10 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   }
   {
     TimedLaunch tl(ts, 6, st);
-    k_window_rounds<<<dim3((nc + 3) / 4, B), 128, 0, st>>>(d_desc, ctx->reg);
-    k_window_decide<<<(nc + 3) / 4, 128, 0, st>>>(d_desc, B, ctx->reg, ctx->dp);
+    const u32 ctas = (nc + WD_THREADS / 32 - 1) / (WD_THREADS / 32);
+    if (B > 1) k_window_rounds<<<dim3(ctas, B), WD_THREADS, 0, st>>>(d_desc, ctx->reg);
+    if (B > 1) k_window_decide<false><<<ctas, WD_THREADS, 0, st>>>(d_desc, B, ctx->reg, ctx->dp);
+    else k_window_decide<true><<<ctas, WD_THREADS, 0, st>>>(d_desc, B, ctx->reg, ctx->dp);      // one window: both stages in one launch
     if (ctx->n_trees) k_tree_root_comm<<<dim3(ctx->n_trees, B), TREE_THREADS, 0, st>>>(d_desc, ctx->d_trees, ctx->reg);
   }
   CK(cudaGetLastError());
@@ -916,7 +922,7 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
     if (it == ctx->windows.end() || !it->second.analysed) { int rc = find_analysed(ctx, window_id, &w); if (rc != CCLD_OK) return rc; }
     else w = &it->second;
     area = verdict_area(ctx->reg.n_comms, ctx->n_ranks);
-    L = misc_layout(ctx->n_ranks, ctx->max_n);
+    L = misc_layout(ctx->n_ranks);
     { int rc = pinned_area(ctx, ctx->h_verdict, area.total); if (rc != CCLD_OK) return rc; }
     hv = (char*)ctx->h_verdict.p;
     head = (const VerdictHead*)hv;
@@ -968,13 +974,23 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
   return CCLD_OK;
 }
 
-// Tree communicators compare progress counters inside a layer; the kernel needs the layer table for that.
-static int hang_layers(ccld_ctx* ctx, const CommHost& c, HangArgs* A) {
-  A->head = nullptr;
-  if (c.algo == 0) return CCLD_OK;
-  if (!c.d_head) return fail(ctx, CCLD_ERR_STATE, "tree communicator without layers (ccld_comm_set_layers)");
-  A->head = c.d_head;
-  return CCLD_OK;
+// Launches the hang kernel over one op or over the window's alerts (A.alerts set) and waits; results are in pinned memory.
+static int hang_run(ccld_ctx* ctx, const WindowHost* w, HangArgs& A, u32 ctas) {
+  A.n_frames = w->n_frames; A.n_channels = w->n_channels;
+  A.f_rank = w->f_rank; A.f_comm = w->f_comm; A.f_seq = w->f_seq; A.progress = w->progress;
+  A.scratch_stride = (u64)align_up((size_t)ctx->max_n * HANG_MEMBER_BYTES); A.scratch = nullptr;
+  Block blk;
+  if (ctx->max_n > HANG_SMEM_N) {
+    cudaError_t e;
+    blk = ctx->pool.get(A.scratch_stride * ctas, &e);
+    if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
+    A.scratch = (unsigned char*)blk.p;
+  }
+  k_hang_locate<<<ctas, HANG_THREADS, hang_smem(std::min<u32>(ctx->max_n, HANG_SMEM_N)), ctx->stream>>>(w->d_desc, ctx->reg, A);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  ctx->pool.put(blk);
+  return e == cudaSuccess ? CCLD_OK : fail(ctx, CCLD_ERR_CUDA, std::string("hang location: ") + cudaGetErrorString(e));
 }
 
 int ccld_locate_hang(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t seq, ccld_hang_verdict* out) {
@@ -985,103 +1001,62 @@ int ccld_locate_hang(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t 
   auto ci = ctx->comm_idx.find(comm);
   if (ci == ctx->comm_idx.end()) return fail(ctx, CCLD_ERR_UNKNOWN_COMM, "unknown communicator");
   CK(cudaSetDevice(ctx->device));
-  cudaStream_t st = ctx->stream;
   const u32 n = (u32)ctx->comms[ci->second].ranks.size();
-  char* m = (char*)ctx->misc_blk.p;
-  const MiscLayout L = misc_layout(ctx->n_ranks, ctx->max_n);
-  HangArgs A;
-  A.c = ci->second; A.seq = seq; A.n_frames = w->n_frames; A.n_channels = w->n_channels;
-  A.f_rank = w->f_rank; A.f_comm = w->f_comm; A.f_seq = w->f_seq; A.progress = w->progress;
-  A.entered = (u8*)(m + L.entered); A.done = (u8*)(m + L.done); A.frame = (u32*)(m + L.frame); A.roots = (u32*)(m + L.roots);
-  A.tot = (u64*)(m + L.tot); A.out = (ccld_hang_verdict*)(m + L.hang_out);
-  A.roots_cap = n;
-  { int rc = hang_layers(ctx, ctx->comms[ci->second], &A); if (rc != CCLD_OK) return rc; }
-  k_hang_locate<<<1, 1024, 0, st>>>(w->d_desc, ctx->reg, A);
-  CK(cudaGetLastError());
-  ccld_hang_verdict v;
-  CK(cudaMemcpyAsync(&v, A.out, sizeof v, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  u32* roots = out->roots; const u32 cap = roots ? out->roots_cap : 0;
-  *out = v; out->roots = roots; out->roots_cap = cap;
-  const u32 n_copy = std::min<u32>(std::min<u32>(v.n_roots_total, n), cap);
-  if (n_copy) { CK(cudaMemcpyAsync(roots, A.roots, n_copy * 4ull, cudaMemcpyDeviceToHost, st)); CK(cudaStreamSynchronize(st)); }
+  if (ctx->comms[ci->second].algo != 0 && !ctx->comms[ci->second].d_head) return fail(ctx, CCLD_ERR_STATE, "tree communicator without layers (ccld_comm_set_layers)");
+  u32* roots = out->roots; const u32 cap = roots ? out->roots_cap : 0, keep = std::min(cap, n);
+  const size_t o_roots = align_up(sizeof(ccld_hang_verdict));
+  { int rc = pinned_area(ctx, ctx->h_io, o_roots + keep * 4ull); if (rc != CCLD_OK) return rc; }
+  char* h = (char*)ctx->h_io.p;
+  HangArgs A; std::memset(&A, 0, sizeof A);
+  A.c = ci->second; A.seq = seq; A.roots = (u32*)(h + o_roots); A.roots_cap = keep; A.out = (ccld_hang_verdict*)h;
+  { int rc = hang_run(ctx, w, A, 1); if (rc != CCLD_OK) return rc; }
+  std::memcpy(out, h, sizeof *out); out->roots = roots; out->roots_cap = cap;
+  const u32 n_copy = std::min(out->n_roots_total, keep);
+  if (n_copy) std::memcpy(roots, h + o_roots, n_copy * 4ull);
   return CCLD_OK;
 }
 
 int ccld_locate_hangs(ccld_ctx* ctx, uint32_t window_id, ccld_hang_alert* alerts, ccld_hang_verdict* out, uint32_t cap,
                       uint32_t* roots, uint32_t roots_stride, uint32_t* n_total) {
+  NvtxRange nvtx_range("ccld_locate_hangs");
   if (!ctx || !n_total) return CCLD_ERR_ARG;
   if (cap && !out) return fail(ctx, CCLD_ERR_ARG, "out is null");
   WindowHost* w;
   { int rc = find_analysed(ctx, window_id, &w); if (rc != CCLD_OK) return rc; }
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = ctx->stream;
-  u64 n_al64 = 0;
-  CK(cudaMemcpyAsync(&n_al64, w->d.counters + C_ALERTS, 8, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  *n_total = (u32)std::min<u64>(n_al64, 0xFFFFFFFFull);
-  const u32 n_dev = (u32)std::min<u64>(n_al64, CCLD_MAX_ALERTS_PER_WINDOW), n = std::min<u32>(n_dev, cap);
-  if (n == 0) return CCLD_OK;
-  // the alerts in the order ccld_get_verdict lists them
-  char* m = (char*)ctx->misc_blk.p;
-  const MiscLayout L = misc_layout(ctx->n_ranks, ctx->max_n);
-  ccld_hang_alert* al_b = (ccld_hang_alert*)(m + L.alerts);
-  k_order_alerts<<<1, VD_THREADS, 0, st>>>(w->d.counters, w->d.alerts, al_b, ctx->reg);
-  CK(cudaGetLastError());
-  std::vector<ccld_hang_alert> al(n);
-  CK(cudaMemcpyAsync(al.data(), al_b, n * sizeof(ccld_hang_alert), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  // per alert: scratch over the communicator's members, a root list and a verdict
-  std::vector<HangArgs> ha(n);
-  std::vector<size_t> o_roots(n);
-  std::vector<u32> members(n);
+  u32 most = std::min<u32>(cap, CCLD_MAX_ALERTS_PER_WINDOW);
+  const u32 keep = roots ? std::min(roots_stride, ctx->max_n) : 0;                 // roots kept per alert
+  if ((size_t)most * keep * 4 > FETCH_PINNED) {
+    // a pinned area for every alert there could be would be large: ask how many there are
+    u64 n_al64 = 0; const Piece pc{w->d.counters + C_ALERTS, &n_al64, 8};
+    { int rc = fetch(ctx, &pc, 1); if (rc != CCLD_OK) return rc; }
+    most = (u32)std::min<u64>(most, n_al64);
+  }
   size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + b); return o; };
-  const size_t o_args = take(n * sizeof(HangArgs)), o_out = take(n * sizeof(ccld_hang_verdict));
-  std::vector<size_t> o_ent(n), o_done(n), o_frame(n), o_tot(n);
+  const size_t o_n = take(8), o_al = take(most * sizeof(ccld_hang_alert)), o_out = take(most * sizeof(ccld_hang_verdict)), o_roots = take((size_t)most * keep * 4);
+  { int rc = pinned_area(ctx, ctx->h_io, off); if (rc != CCLD_OK) return rc; }
+  char* h = (char*)ctx->h_io.p;
+  ccld_hang_alert* al = (ccld_hang_alert*)((char*)ctx->misc_blk.p + misc_layout(ctx->n_ranks).alerts);
+  k_order_alerts<<<1, VD_THREADS, 0, st>>>(w->d.counters, w->d.alerts, al, ctx->reg);
+  HangArgs A; std::memset(&A, 0, sizeof A);
+  A.alerts = al; A.counters = w->d.counters; A.cap = most; A.roots = (u32*)(h + o_roots); A.roots_cap = keep;
+  A.out = (ccld_hang_verdict*)(h + o_out); A.alerts_out = (ccld_hang_alert*)(h + o_al); A.n_alerts_out = (u64*)(h + o_n);
+  { int rc = hang_run(ctx, w, A, std::max(1u, std::min(most, ctx->n_sms))); if (rc != CCLD_OK) return rc; }
+  const u64 found = *(const u64*)(h + o_n);
+  *n_total = (u32)std::min<u64>(found, 0xFFFFFFFFull);
+  const u32 n = (u32)std::min<u64>(found, most);
+  const ccld_hang_verdict* hv = (const ccld_hang_verdict*)(h + o_out);
+  for (u32 i = 0; i < n; ++i) if (hv[i].cls == HANG_NO_LAYERS) return fail(ctx, CCLD_ERR_STATE, "tree communicator without layers (ccld_comm_set_layers)");
   for (u32 i = 0; i < n; ++i) {
-    auto ci = ctx->comm_idx.find(al[i].comm);
-    if (ci == ctx->comm_idx.end()) return fail(ctx, CCLD_ERR_CUDA, "internal: alert names an unknown communicator");
-    const u32 nm = (u32)ctx->comms[ci->second].ranks.size();
-    members[i] = nm; ha[i].c = ci->second;
-    { int rc = hang_layers(ctx, ctx->comms[ci->second], &ha[i]); if (rc != CCLD_OK) return rc; }
-    o_ent[i] = take(nm); o_done[i] = take(nm); o_frame[i] = take(nm * 4ull); o_tot[i] = take(nm * 8ull); o_roots[i] = take(nm * 4ull);
-  }
-  cudaError_t e;
-  Block blk = ctx->pool.get(off, &e);
-  if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
-  char* b = (char*)blk.p;
-  for (u32 i = 0; i < n; ++i) {
-    HangArgs& A = ha[i];
-    A.seq = al[i].seq; A.n_frames = w->n_frames; A.n_channels = w->n_channels;
-    A.f_rank = w->f_rank; A.f_comm = w->f_comm; A.f_seq = w->f_seq; A.progress = w->progress;
-    A.entered = (u8*)(b + o_ent[i]); A.done = (u8*)(b + o_done[i]); A.frame = (u32*)(b + o_frame[i]); A.tot = (u64*)(b + o_tot[i]);
-    A.roots = (u32*)(b + o_roots[i]); A.roots_cap = members[i];
-    A.out = (ccld_hang_verdict*)(b + o_out) + i;
-  }
-  std::vector<ccld_hang_verdict> hv(n);
-  std::vector<char> host_blk;
-  int rc = CCLD_OK;
-  do {
-    if (cudaMemcpyAsync(b + o_args, ha.data(), n * sizeof(HangArgs), cudaMemcpyHostToDevice, st) != cudaSuccess) { rc = CCLD_ERR_CUDA; break; }
-    k_hang_locate_many<<<n, 1024, 0, st>>>(w->d_desc, ctx->reg, (const HangArgs*)(b + o_args));
-    if (cudaGetLastError() != cudaSuccess) { rc = CCLD_ERR_CUDA; break; }
-    host_blk.resize(off);
-    // verdicts and root lists come back in one copy (they follow each other in the block)
-    if (cudaMemcpyAsync(host_blk.data() + o_out, b + o_out, off - o_out, cudaMemcpyDeviceToHost, st) != cudaSuccess) { rc = CCLD_ERR_CUDA; break; }
-    if (cudaStreamSynchronize(st) != cudaSuccess) { rc = CCLD_ERR_CUDA; break; }
-  } while (0);
-  ctx->pool.put(blk);
-  if (rc != CCLD_OK) return fail(ctx, rc, "hang sweep failed");
-  for (u32 i = 0; i < n; ++i) {
-    ccld_hang_verdict v;
-    std::memcpy(&v, host_blk.data() + o_out + i * sizeof(ccld_hang_verdict), sizeof v);
+    ccld_hang_verdict v = hv[i];
     v.roots = roots ? roots + (size_t)i * roots_stride : nullptr; v.roots_cap = roots ? roots_stride : 0;
-    const u32 n_copy = std::min<u32>(std::min<u32>(v.n_roots_total, members[i]), v.roots_cap);
-    if (n_copy) std::memcpy(v.roots, host_blk.data() + o_roots[i], n_copy * 4ull);
+    const u32 n_copy = std::min(v.n_roots_total, keep);
+    if (n_copy) std::memcpy(v.roots, h + o_roots + (size_t)i * keep * 4, n_copy * 4ull);
     out[i] = v;
-    if (alerts) alerts[i] = al[i];
   }
+  if (alerts && n) std::memcpy(alerts, h + o_al, n * sizeof(ccld_hang_alert));
   return CCLD_OK;
 }
 
@@ -1161,30 +1136,19 @@ int ccld_opset_check(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t 
   auto ci = ctx->comm_idx.find(comm);
   if (ci == ctx->comm_idx.end()) return fail(ctx, CCLD_ERR_UNKNOWN_COMM, "unknown communicator");
   CK(cudaSetDevice(ctx->device));
-  cudaStream_t st = ctx->stream;
   const u32 n = (u32)ctx->comms[ci->second].ranks.size();
-  size_t off = 0;
-  auto take = [&](size_t b) { size_t o = off; off = align_up(off + b); return o; };
-  const size_t o_hi = take(n * 8ull), o_lo = take(n * 4ull), o_rk = take(n * 4ull), o_out = take(sizeof(ccld_opset_verdict));
-  cudaError_t e;
-  Block blk = ctx->pool.get(off, &e);
-  if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
-  char* b = (char*)blk.p;
+  u32* ranks = out->ranks; const u32 cap = ranks ? out->ranks_cap : 0, keep = std::min(cap, n);
+  const size_t o_rk = align_up(sizeof(ccld_opset_verdict));
+  { int rc = pinned_area(ctx, ctx->h_io, o_rk + keep * 4ull); if (rc != CCLD_OK) return rc; }
+  char* h = (char*)ctx->h_io.p;
   OpsetArgs A; A.c = ci->second; A.seq = seq; A.algo = w->algo; A.proto = w->proto;
-  A.key_hi = (u64*)(b + o_hi); A.key_lo = (u32*)(b + o_lo); A.ranks = (u32*)(b + o_rk); A.ranks_cap = n; A.out = (ccld_opset_verdict*)(b + o_out);
-  k_opset_check<<<1, 1024, 0, st>>>(w->d_desc, ctx->reg, A);
-  ccld_opset_verdict v;
-  u32* ranks = out->ranks; const u32 cap = ranks ? out->ranks_cap : 0;
-  int rc = CCLD_OK;
-  if (cudaGetLastError() != cudaSuccess || cudaMemcpyAsync(&v, A.out, sizeof v, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess) rc = CCLD_ERR_CUDA;
-  if (rc == CCLD_OK) {
-    *out = v; out->ranks = ranks; out->ranks_cap = cap;
-    const u32 n_copy = std::min<u32>(std::min<u32>(v.n_deviating_total, n), cap);
-    if (n_copy && (cudaMemcpyAsync(ranks, A.ranks, n_copy * 4ull, cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)) rc = CCLD_ERR_CUDA;
-  }
-  ctx->pool.put(blk);
-  if (rc != CCLD_OK) return fail(ctx, rc, "op-set check failed");
+  A.ranks = (u32*)(h + o_rk); A.ranks_cap = keep; A.out = (ccld_opset_verdict*)h;
+  k_opset_check<<<1, OPSET_THREADS, (size_t)n * OPSET_MEMBER_BYTES, ctx->stream>>>(w->d_desc, ctx->reg, A);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(ctx->stream));
+  std::memcpy(out, h, sizeof *out); out->ranks = ranks; out->ranks_cap = cap;
+  const u32 n_copy = std::min(out->n_deviating_total, keep);
+  if (n_copy) std::memcpy(ranks, h + o_rk, n_copy * 4ull);
   return CCLD_OK;
 }
 

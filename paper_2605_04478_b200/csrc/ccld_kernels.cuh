@@ -14,7 +14,7 @@
 //   k_reduce_large_deferred  the groups k_reduce_large sets aside
 //   k_window_rounds Eq. 2 per (communicator, window): round counts, selected round, location candidates
 //   k_window_decide Eq. 1, 3, 4 per communicator, windows in order: baseline state, class, slow location
-//   k_hang_locate   hang decision tree over presence / completion / progress counters
+//   k_hang_locate   hang decision tree over presence / completion / progress counters (ccld_hang.cuh)
 // The suspect list and the ordered output lists are in ccld_verdict.cuh.
 #pragma once
 #include "ccld_device.cuh"
@@ -709,305 +709,194 @@ inline size_t mid_smem_bytes(u32 n_pad_min) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// window decision per communicator (Sec. 4.2.1 Eq. 1-3, Sec. 4.2.2 Eq. 4): one warp per
-// communicator walks the windows of the batch in order
+// window decision per communicator (Sec. 4.2.1 Eq. 1-3, Sec. 4.2.2 Eq. 4): a warp per communicator.
+// Bound by latency: chains of dependent reads over little data.
 // ------------------------------------------------------------------------------------------------
-// Stage 1, one warp per (communicator, window), all windows at once: everything of the window decision that does not
-// depend on the state carried from window to window - the round and analysed-op counts, the round Eq. 2 selects with its
-// T_max / T_min and the ranks the location step would name - goes into the communicator's verdict row.
-__global__ void __launch_bounds__(128) k_window_rounds(const WinDesc* __restrict__ wd, Registry R) {
-  const u32 c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (c >= R.n_comms) return;
-  const WinDesc& D = wd[blockIdx.y];
-  const RangeRow row = D.ranges[c];
-  if (row.n_seq == 0) return;
-  const u32 n = R.comm_n[c], cls = comm_class(n);
-  const u32* mem = R.members + R.comm_moff[c];
+constexpr int WD_THREADS = 128;
+
+// What of a window's decision does not depend on the state carried from window to window: the round counts, the round Eq. 2
+// selects with its T_max / T_min and the ranks the location step would name.
+struct RoundPart { u32 n_rounds, sel_seq, root_comp, root_comm, rate_source; i64 t_max, t_min; };
+
+__device__ __forceinline__ RoundPart rounds_of(const WinDesc& D, const RangeRow& row, u32 lane, u32* n_analysed) {
+  RoundPart x = {0, NONE, NONE, NONE, 0, 0, 0};
+  *n_analysed = 0;
+  if (row.n_seq == 0) return x;
+  const u32 cls = comm_class(row.n);
   const u64 G = D.n_groups;
   const i64* t_max = D.gi64 + (u64)GI_T_MAX * G + row.group0;
   const i64* t_min = D.gi64 + (u64)GI_T_MIN * G + row.group0;
   // round counts and the Eq. 2 candidate come from the tile summaries the reduce kernels left behind
   const TileSum* ts = D.tsum[cls <= 1 ? 0 : cls - 1] + row.tile0;   // both relative to the window
-  const u32 nt = row.n_units;
   u32 n_rounds = 0, n_an = 0;
   u64 best_rng = 0; u32 best_k = NONE;
   bool redo = false;                                     // a unit left groups to the deferred kernel: its summary is partial
-  for (u32 q = lane; q < nt; q += 32) {
-    const TileSum x = ts[q];
-    n_rounds += x.n_rounds; n_an += x.n_an;
-    best_merge(best_rng, best_k, x.best_rng, x.best_k);
-    redo = redo || x.pad != 0;
+  for (u32 q = lane; q < row.n_units; q += 32) {
+    const TileSum s = ts[q];
+    n_rounds += s.n_rounds; n_an += s.n_an;
+    best_merge(best_rng, best_k, s.best_rng, s.best_k);
+    redo = redo || s.pad != 0;
   }
   if (__any_sync(0xFFFFFFFFu, redo)) {
     // recount the communicator's window from the per-op rows
     const u32* gfl = D.gu32 + (u64)GU_GFLAGS * G + row.group0;
     n_rounds = 0; n_an = 0; best_rng = 0; best_k = NONE;
+#pragma unroll 4
     for (u32 k = lane; k < row.n_seq; k += 32) {
-      const u32 f = gfl[k];
-      if ((f & CCLD_G_COMPLETE) && !(f & CCLD_G_BARRIER)) { ++n_rounds; best_merge(best_rng, best_k, (u64)(t_max[k] - t_min[k]), k); }
+      const u32 f = gfl[k]; const u64 rng = (u64)(t_max[k] - t_min[k]);
+      if ((f & CCLD_G_COMPLETE) && !(f & CCLD_G_BARRIER)) { ++n_rounds; best_merge(best_rng, best_k, rng, k); }
       if (f & CCLD_G_ANALYSED) ++n_an;
     }
   }
-  n_rounds = __reduce_add_sync(0xFFFFFFFFu, n_rounds); n_an = __reduce_add_sync(0xFFFFFFFFu, n_an);
+  x.n_rounds = __reduce_add_sync(0xFFFFFFFFu, n_rounds); *n_analysed = __reduce_add_sync(0xFFFFFFFFu, n_an);
   best_warp_reduce(best_rng, best_k);
-  // analysed ops of this window count towards every member's denominator
-  if (n_an) for (u32 p = lane; p < n; p += 32) atomicAdd(&R.ops[mem[p]], n_an);
-  if (lane == 0) {
-    ccld_comm_verdict v;
-    v.comm = R.comm_id[c]; v.n_rounds = n_rounds; v.sel_seq = NONE; v.cls = 0; v.slow_detected = 0; v.located = 0;
-    v.baseline_static = 0; v.rate_source = 0; v.root_comp = NONE; v.root_comm = NONE;
-    v.t_max = 0; v.t_min = 0; v.R = 0.0; v.P = 0.0; v.t_base = 0; v.rounds_total = 0; v.m = 0; v.slow_count = 0;
-    if (best_k != NONE) {
-      v.sel_seq = row.seq_lo + best_k; v.t_max = t_max[best_k]; v.t_min = t_min[best_k];
-      const u64 gq = row.group0 + best_k;
-      v.root_comp = D.gu32[(u64)GU_RANK_TMIN * G + gq];
-      const u32 mc = D.gu32[(u64)GU_MAX_CHG * G + gq];
-      if (mc > 0) { v.root_comm = D.gu32[(u64)GU_RANK_MAX_CHG * G + gq]; v.rate_source = 0; }
-      else { v.root_comm = D.gu32[(u64)GU_RANK_TMAX * G + gq]; v.rate_source = 1; }
-    }
-    D.comm_rows[row.row_idx] = v;
+  if (best_k != NONE) {
+    const u64 gq = row.group0 + best_k;
+    const u32 mc = D.gu32[(u64)GU_MAX_CHG * G + gq], by_rate = D.gu32[(u64)GU_RANK_MAX_CHG * G + gq], by_time = D.gu32[(u64)GU_RANK_TMAX * G + gq];
+    x.sel_seq = row.seq_lo + best_k; x.t_max = t_max[best_k]; x.t_min = t_min[best_k];
+    x.root_comp = D.gu32[(u64)GU_RANK_TMIN * G + gq];
+    x.root_comm = mc > 0 ? by_rate : by_time; x.rate_source = mc > 0 ? 0u : 1u;
+  }
+  return x;
+}
+
+// Analysed ops of a window count towards every member's denominator: the CTA's communicators one after the other, all
+// threads along the members (a warp alone took 20 us over a communicator of 4,096).
+__device__ __forceinline__ void count_ops(const Registry& R, u32 c0, const u32* __restrict__ s_an) {
+  for (u32 q = 0; q < WD_THREADS / 32; ++q) {
+    const u32 n_an = s_an[q];
+    if (n_an == 0) continue;
+    const u32 n = R.comm_n[c0 + q];
+    const u32* __restrict__ mem = R.members + R.comm_moff[c0 + q];
+#pragma unroll 4
+    for (u32 p = threadIdx.x; p < n; p += WD_THREADS) atomicAdd(&R.ops[mem[p]], n_an);
   }
 }
 
-// Stage 2, one warp per communicator, windows in order: the recurrences - Eq. 1's baseline, which reads the per-op rows
-// until m is fixed, and the repetition counter - and with them Eq. 3, Eq. 4 and the location rule, which complete the
-// row stage 1 wrote. What a window needs is fetched ahead (range rows two windows, the stage-1 row and the result
-// pointers one window), so the walk waits for arithmetic only.
-__global__ void __launch_bounds__(128) k_window_decide(const WinDesc* __restrict__ wd, u32 nw, Registry R, Params P) {
-  const u32 c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (c >= R.n_comms) return;
-  CommState st = R.state[c];
-  struct Res { const RangeRow* ranges; u64 n_groups; const i64* gi64; const u32* gu32; ccld_comm_verdict* comm_rows; };   // pointers of a window
-  struct Part { u32 n_rounds, sel_seq, root_comp, root_comm, rate_source; i64 t_max, t_min; };    // what stage 1 left in the row
-  // three steps, each on values fetched during an earlier window: descriptor -> range row -> stage-1 row
-  auto load_res = [&](u32 w) {
-    Res r = {nullptr, 0, nullptr, nullptr, nullptr};
-    if (w < nw) { r.ranges = wd[w].ranges; r.n_groups = wd[w].n_groups; r.gi64 = wd[w].gi64; r.gu32 = wd[w].gu32; r.comm_rows = wd[w].comm_rows; }
-    return r;
-  };
-  auto load_row = [&](const Res& r) { RangeRow x = {0, 0, 0, 0, 0, 0, 0, 0}; if (r.ranges != nullptr) x = r.ranges[c]; return x; };
-  auto load_part = [&](const Res& r, const RangeRow& row) {
-    Part x = {0, NONE, NONE, NONE, 0, 0, 0};
-    if (r.comm_rows != nullptr && row.n_seq != 0) {
-      const ccld_comm_verdict* v = r.comm_rows + row.row_idx;
-      x.n_rounds = v->n_rounds; x.sel_seq = v->sel_seq; x.root_comp = v->root_comp; x.root_comm = v->root_comm;
-      x.rate_source = v->rate_source; x.t_max = v->t_max; x.t_min = v->t_min;
+// Stage 1 of a batch of several windows, all at once: leaves the part above in the communicator's verdict row.
+__global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* __restrict__ wd, Registry R) {
+  __shared__ u32 s_an[WD_THREADS / 32];
+  const u32 c0 = blockIdx.x * (WD_THREADS / 32), wid = threadIdx.x >> 5, c = c0 + wid, lane = threadIdx.x & 31;
+  const WinDesc& D = wd[blockIdx.y];
+  u32 n_an = 0;
+  if (c < R.n_comms) {
+    const RangeRow row = D.ranges[c];
+    const RoundPart x = rounds_of(D, row, lane, &n_an);
+    if (lane == 0 && row.n_seq) {
+      ccld_comm_verdict* v = D.comm_rows + row.row_idx;
+      v->n_rounds = x.n_rounds; v->sel_seq = x.sel_seq; v->root_comp = x.root_comp; v->root_comm = x.root_comm; v->rate_source = x.rate_source;
+      v->t_max = x.t_max; v->t_min = x.t_min;
     }
-    return x;
-  };
-  Res res_a = load_res(0), res_b = load_res(1), res_c = load_res(2);
-  RangeRow row_a = load_row(res_a), row_b = load_row(res_b);
-  Part part_a = load_part(res_a, row_a);
-  for (u32 w = 0; w < nw; ++w) {
-    const RangeRow row = row_a; const Res D = res_a; const Part pt = part_a;
-    part_a = load_part(res_b, row_b);                    // window w + 1
-    row_a = row_b; row_b = load_row(res_c);              // window w + 2
-    res_a = res_b; res_b = res_c; res_c = load_res(w + 3);
-    if (row.n_seq == 0) continue;
-    const u64 G = D.n_groups;
-    const u32 n_rounds = pt.n_rounds;
-    // Eq. 1: rounds feed the baseline, in op-counter order, until m is fixed
-    u32 walked = 0;
-    if (st.m == 0 && n_rounds > 0) {
-      const u32* gfl = D.gu32 + (u64)GU_GFLAGS * G + row.group0;
-      const i64* e_min = D.gi64 + (u64)GI_E_MIN * G + row.group0;
-      const i64* t_max = D.gi64 + (u64)GI_T_MAX * G + row.group0;
-      for (u32 k0 = 0; k0 < row.n_seq && st.m == 0; k0 += 32) {
-        const u32 k = k0 + lane;
-        const u32 f = k < row.n_seq ? gfl[k] : 0;
-        const bool round = (f & CCLD_G_COMPLETE) && !(f & CCLD_G_BARRIER);
-        u32 rem = __ballot_sync(0xFFFFFFFFu, round);
-        i64 em = 0, tM = 0;
-        if (round) { em = e_min[k]; tM = t_max[k]; }
-        while (rem && st.m == 0) {
-          const int src = __ffs(rem) - 1; rem &= rem - 1;
-          const i64 em_s = __shfl_sync(0xFFFFFFFFu, em, src), tM_s = __shfl_sync(0xFFFFFFFFu, tM, src);
-          if (st.rounds == 0) st.t_first = em_s;
-          if (st.rounds == (u64)P.m_max_rounds || (st.rounds > 0 && em_s - st.t_first >= P.m_max_ns)) st.m = st.rounds;
-          else st.sum_m += tM_s;
-          ++st.rounds; ++walked;
-        }
-      }
-    }
-    st.rounds += n_rounds - walked;
-    if (lane == 0) {
-      ccld_comm_verdict v;
-      v.comm = R.comm_id[c]; v.n_rounds = n_rounds; v.sel_seq = pt.sel_seq; v.cls = 0; v.slow_detected = 0; v.located = 0;
-      v.baseline_static = st.m == 0; v.rate_source = 0; v.root_comp = NONE; v.root_comm = NONE;
-      v.t_max = pt.t_max; v.t_min = pt.t_min; v.R = 0.0; v.P = 0.0;
-      v.t_base = st.m > 0 ? st.sum_m / (i64)st.m : P.tbase_init_ns;
-      v.rounds_total = st.rounds; v.m = st.m;
-      if (pt.sel_seq != NONE) {
-        v.R = (double)(v.t_max - v.t_base) / (double)v.t_base;                                     // Eq. 3
-        const bool slow = v.t_max > v.t_base && mul_gt((u64)(v.t_max - v.t_base), 1000u, (u64)v.t_base, P.theta_slow_milli);
-        v.slow_detected = slow;
-        if (slow) {
-          ++st.slow_count;
-          v.located = st.slow_count > (u64)P.slow_rep_threshold;
-          const u64 num = (u64)(v.t_max - v.t_min), den = (u64)(v.t_max - v.t_base);
-          v.P = (double)num / (double)den;                                                         // Eq. 4
-          v.cls = mul_gt(num, 1000u, den, P.beta_milli) ? 1u : (mul_lt(num, 1000u, den, P.alpha_milli) ? 2u : 3u);
-          v.root_comp = pt.root_comp; v.root_comm = pt.root_comm; v.rate_source = pt.rate_source;
-        }
-      }
-      v.slow_count = st.slow_count;
-      D.comm_rows[row.row_idx] = v;
-    }
-    st.slow_count = __shfl_sync(0xFFFFFFFFu, st.slow_count, 0);
   }
-  if (lane == 0) R.state[c] = st;
+  if (lane == 0) s_an[wid] = n_an;
+  __syncthreads();
+  count_ops(R, c0, s_an);
 }
 
-// ------------------------------------------------------------------------------------------------
-// hang location (Sec. 4.2.2, Fig. 6): one CTA
-// ------------------------------------------------------------------------------------------------
-struct HangArgs {
-  u32 c, seq, n_frames, n_channels;
-  const u32 *f_rank, *f_comm, *f_seq, *progress;
-  u8* entered; u8* done;     // [n] scratch
-  u32* frame;                // [n] scratch
-  u64* tot;                  // [n] scratch
-  u32* roots; u32 roots_cap; // device list
-  ccld_hang_verdict* out;    // device copy of the struct (pointer fields unused)
-  const u32* head;           // [n] tree communicators: lowest position of each member's layer; null for a ring
-};
-
-__device__ __forceinline__ void hang_locate_cta(const WinDesc& D, const Registry& R, const HangArgs& A) {
-  __shared__ u64 s_red64[32];
-  __shared__ u32 s_red32[32];
-  __shared__ u32 s_base;
-  const u32 c = A.c, n = R.comm_n[c], cid = R.comm_id[c];
-  const u32* mem = R.members + R.comm_moff[c];
-  const RangeRow row = D.ranges[c];
-  for (u32 p = threadIdx.x; p < n; p += blockDim.x) { A.entered[p] = 0; A.done[p] = 0; A.frame[p] = NONE; A.tot[p] = 0; }
-  __syncthreads();
-  // a member has entered if it reported this or a later op counter
-  if (row.n_seq > 0 && A.seq <= row.seq_lo + (row.n_seq - 1)) {
-    const u32 s_first = A.seq > row.seq_lo ? A.seq - row.seq_lo : 0;
-    const u64 cnt = (u64)(row.n_seq - s_first) * n;
-    for (u64 e = threadIdx.x; e < cnt; e += blockDim.x) {
-      const u32 so = s_first + (u32)(e / n), p = (u32)(e % n);
-      const u32 idx = D.perm[perm_at(row, so, p)];
-      if (idx != NONE) {
-        A.entered[p] = 1;
-        if (row.seq_lo + so == A.seq && D.t_exit[idx] != -1) A.done[p] = 1;
+// Stage 2, windows in order: the recurrences - Eq. 1's baseline, which reads the per-op rows until m is fixed, and the
+// repetition counter - and with them Eq. 3, Eq. 4 and the location rule, which complete the row. What a window needs is
+// fetched ahead (range rows two windows, the stage-1 row and the result pointers one window), so the walk waits for
+// arithmetic only. SINGLE: a batch of one window, stage 1 is done here too.
+template <bool SINGLE>
+__global__ void __launch_bounds__(WD_THREADS) k_window_decide(const WinDesc* __restrict__ wd, u32 nw, Registry R, Params P) {
+  __shared__ u32 s_an[WD_THREADS / 32];
+  const u32 c0 = blockIdx.x * (WD_THREADS / 32), wid = threadIdx.x >> 5, c = c0 + wid, lane = threadIdx.x & 31;
+  u32 n_an = 0;
+  if (c < R.n_comms) {
+    CommState st = R.state[c];
+    struct Res { const RangeRow* ranges; u64 n_groups; const i64* gi64; const u32* gu32; ccld_comm_verdict* comm_rows; };   // pointers of a window
+    // three steps, each on values fetched during an earlier window: descriptor -> range row -> stage-1 row
+    auto load_res = [&](u32 w) {
+      Res r = {nullptr, 0, nullptr, nullptr, nullptr};
+      if (w < nw) { r.ranges = wd[w].ranges; r.n_groups = wd[w].n_groups; r.gi64 = wd[w].gi64; r.gu32 = wd[w].gu32; r.comm_rows = wd[w].comm_rows; }
+      return r;
+    };
+    auto load_row = [&](const Res& r) { RangeRow x = {0, 0, 0, 0, 0, 0, 0, 0}; if (r.ranges != nullptr) x = r.ranges[c]; return x; };
+    auto load_part = [&](const Res& r, const RangeRow& row) {
+      RoundPart x = {0, NONE, NONE, NONE, 0, 0, 0};
+      if (r.comm_rows != nullptr && row.n_seq != 0) {
+        const ccld_comm_verdict* v = r.comm_rows + row.row_idx;
+        x.n_rounds = v->n_rounds; x.sel_seq = v->sel_seq; x.root_comp = v->root_comp; x.root_comm = v->root_comm;
+        x.rate_source = v->rate_source; x.t_max = v->t_max; x.t_min = v->t_min;
       }
-    }
-  }
-  // progress frames of this op: the first frame uploaded for a member counts
-  for (u32 f = threadIdx.x; f < A.n_frames; f += blockDim.x) {
-    if (A.f_comm[f] != cid || A.f_seq[f] != A.seq) continue;
-    const u32 p = pos_lookup(R, A.f_rank[f], c);
-    if (p != NONE) atomicMin(&A.frame[p], f);
-  }
-  __syncthreads();
-  u32 n_ne = 0, n_ok = 0, n_missing = 0; u64 mn = U64_MAX_;
-  for (u32 p = threadIdx.x; p < n; p += blockDim.x) {
-    n_ne += !A.entered[p]; n_ok += A.done[p];
-    const u32 f = A.frame[p];
-    u64 tot = 0;
-    if (f == NONE) ++n_missing;
-    else for (u32 ch = 0; ch < A.n_channels; ++ch) tot += (u64)A.progress[((u64)f * A.n_channels + ch) * 2] + A.progress[((u64)f * A.n_channels + ch) * 2 + 1];
-    A.tot[p] = tot; mn = tot < mn ? tot : mn;
-  }
-  n_ne = block_reduce(n_ne, OpAddU32(), s_red32);
-  n_ok = block_reduce(n_ok, OpAddU32(), s_red32);
-  n_missing = block_reduce(n_missing, OpAddU32(), s_red32);
-  mn = block_reduce(mn, OpMinU64(), s_red64);
-  __syncthreads();
-  const u32 cls = n_ne > 0 ? 1u : (n_ok > 0 ? 2u : 3u);
-  u32 n_roots = 0, stuck = 0; u64 min_total = 0;
-  if (cls == 3 && A.head != nullptr) {
-    // tree (Sec. 4.2.1): counters are comparable inside a layer only. The lowest position of a layer walks the layer:
-    // its minimum, the first member that holds it, its maximum. The layer whose minimum is furthest behind its maximum
-    // names the root; equal gaps: the lowest position; no gap anywhere: nobody.
-    u64 lag = 0; u32 cand = NONE;
-    for (u32 p = threadIdx.x; p < n; p += blockDim.x) {
-      if (A.head[p] != p) continue;
-      u64 lmn = A.tot[p], lmx = lmn; u32 at = p;
-      for (u32 x = p + 1; x < n; ++x) {
-        if (A.head[x] != p) continue;
-        const u64 t = A.tot[x];
-        if (t < lmn) { lmn = t; at = x; }
-        lmx = t > lmx ? t : lmx;
+      return x;
+    };
+    Res res_a = load_res(0), res_b = load_res(1), res_c = load_res(2);
+    RangeRow row_a = load_row(res_a), row_b = load_row(res_b);
+    RoundPart part_a;
+    if (SINGLE) part_a = rounds_of(wd[0], row_a, lane, &n_an); else part_a = load_part(res_a, row_a);
+    for (u32 w = 0; w < nw; ++w) {
+      const RangeRow row = row_a; const Res D = res_a; const RoundPart pt = part_a;
+      if (!SINGLE) {
+        part_a = load_part(res_b, row_b);                    // window w + 1
+        row_a = row_b; row_b = load_row(res_c);              // window w + 2
+        res_a = res_b; res_b = res_c; res_c = load_res(w + 3);
       }
-      const u64 g = lmx - lmn;
-      if (g > lag || (g == lag && g > 0 && at < cand)) { lag = g; cand = at; }
-    }
-    const u64 best = block_reduce(lag, OpMaxU64(), s_red64);
-    if (lag != best || best == 0) cand = NONE;
-    const u32 root = block_reduce(cand, OpMinU32(), s_red32);
-    if (root != NONE) {
-      n_roots = 1; min_total = A.tot[root];
-      if (threadIdx.x == 0) {
-        if (A.roots_cap > 0) A.roots[0] = mem[root];
-        const u32 f = A.frame[root];
-        if (f != NONE && A.n_channels > 0) {
-          u32 s = NONE;
-          for (u32 ch = 0; ch < A.n_channels; ++ch) { const u32 r = A.progress[((u64)f * A.n_channels + ch) * 2 + 1]; s = r < s ? r : s; }
-          stuck = s;
+      if (row.n_seq == 0) continue;
+      const u64 G = D.n_groups;
+      const u32 n_rounds = pt.n_rounds;
+      // Eq. 1: rounds feed the baseline, in op-counter order, until m is fixed: by the first round that comes after
+      // m_max_rounds others or m_max_ns after the first. 32 ops at a time; a lane knows from the vote how many rounds
+      // precede its own.
+      u32 walked = 0;
+      if (st.m == 0 && n_rounds > 0) {
+        const u32* gfl = D.gu32 + (u64)GU_GFLAGS * G + row.group0;
+        const i64* e_min = D.gi64 + (u64)GI_E_MIN * G + row.group0;
+        const i64* t_max = D.gi64 + (u64)GI_T_MAX * G + row.group0;
+        for (u32 k0 = 0; k0 < row.n_seq && st.m == 0; k0 += 32) {
+          const u32 k = k0 + lane;
+          u32 f = 0; i64 em = 0, tM = 0;
+          if (k < row.n_seq) { f = gfl[k]; em = e_min[k]; tM = t_max[k]; }
+          const bool round = (f & CCLD_G_COMPLETE) && !(f & CCLD_G_BARRIER);
+          const u32 bal = __ballot_sync(0xFFFFFFFFu, round);
+          if (bal == 0) continue;
+          if (st.rounds == 0) st.t_first = __shfl_sync(0xFFFFFFFFu, em, __ffs(bal) - 1);
+          const u64 before = st.rounds + (u32)__popc(bal & ((1u << lane) - 1u));
+          const u32 stop = __ballot_sync(0xFFFFFFFFu, round && (before == (u64)P.m_max_rounds || (before > 0 && em - st.t_first >= P.m_max_ns)));
+          const u32 take = stop ? bal & ((1u << (__ffs(stop) - 1)) - 1u) : bal;      // rounds that still feed the baseline
+          i64 sum = (take >> lane) & 1u ? tM : 0;
+#pragma unroll
+          for (int d = 16; d > 0; d >>= 1) sum += (i64)shfl_xor64((u64)sum, d);
+          st.sum_m += sum;
+          u32 seen = (u32)__popc(take);
+          if (stop) { st.m = st.rounds + seen; ++seen; }
+          st.rounds += seen; walked += seen;
         }
       }
-    }
-  } else if (cls == 3) {
-    // fewest counters; among equals the most upstream of a run (predecessor ahead), then the lowest position
-    u32 up = NONE, any = NONE;
-    for (u32 p = threadIdx.x; p < n; p += blockDim.x) {
-      if (A.tot[p] != mn) continue;
-      any = p < any ? p : any;
-      if (A.tot[(p + n - 1) % n] > mn) up = p < up ? p : up;
-    }
-    up = block_reduce(up, OpMinU32(), s_red32);
-    any = block_reduce(any, OpMinU32(), s_red32);
-    const u32 root = up != NONE ? up : any;
-    n_roots = 1; min_total = mn;
-    if (threadIdx.x == 0) {
-      if (A.roots_cap > 0) A.roots[0] = mem[root];
-      const u32 f = A.frame[root];
-      if (f != NONE && A.n_channels > 0) {
-        u32 s = NONE;
-        for (u32 ch = 0; ch < A.n_channels; ++ch) { const u32 r = A.progress[((u64)f * A.n_channels + ch) * 2 + 1]; s = r < s ? r : s; }
-        stuck = s;
+      st.rounds += n_rounds - walked;
+      if (lane == 0) {
+        ccld_comm_verdict v;
+        v.comm = R.comm_id[c]; v.n_rounds = n_rounds; v.sel_seq = pt.sel_seq; v.cls = 0; v.slow_detected = 0; v.located = 0;
+        v.baseline_static = st.m == 0; v.rate_source = 0; v.root_comp = NONE; v.root_comm = NONE;
+        v.t_max = pt.t_max; v.t_min = pt.t_min; v.R = 0.0; v.P = 0.0;
+        v.t_base = st.m > 0 ? st.sum_m / (i64)st.m : P.tbase_init_ns;
+        v.rounds_total = st.rounds; v.m = st.m;
+        if (pt.sel_seq != NONE) {
+          v.R = (double)(v.t_max - v.t_base) / (double)v.t_base;                                     // Eq. 3
+          const bool slow = v.t_max > v.t_base && mul_gt((u64)(v.t_max - v.t_base), 1000u, (u64)v.t_base, P.theta_slow_milli);
+          v.slow_detected = slow;
+          if (slow) {
+            ++st.slow_count;
+            v.located = st.slow_count > (u64)P.slow_rep_threshold;
+            const u64 num = (u64)(v.t_max - v.t_min), den = (u64)(v.t_max - v.t_base);
+            v.P = (double)num / (double)den;                                                         // Eq. 4
+            v.cls = mul_gt(num, 1000u, den, P.beta_milli) ? 1u : (mul_lt(num, 1000u, den, P.alpha_milli) ? 2u : 3u);
+            v.root_comp = pt.root_comp; v.root_comm = pt.root_comm; v.rate_source = pt.rate_source;
+          }
+        }
+        v.slow_count = st.slow_count;
+        D.comm_rows[row.row_idx] = v;
       }
+      st.slow_count = __shfl_sync(0xFFFFFFFFu, st.slow_count, 0);
     }
-  } else {
-    // ordered compaction of the not-entered (H1) or not-hung (H2) members
-    if (threadIdx.x == 0) s_base = 0;
-    __syncthreads();
-    for (u32 p0 = 0; p0 < n; p0 += blockDim.x) {
-      const u32 p = p0 + threadIdx.x;
-      const bool sel = p < n && (cls == 1 ? !A.entered[p] : A.done[p] != 0);
-      const u32 bal = __ballot_sync(0xFFFFFFFFu, sel);
-      const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-      __syncthreads();
-      if (lane == 0) s_red32[wid] = __popc(bal);
-      __syncthreads();
-      u32 off = s_base;
-      for (u32 q = 0; q < wid; ++q) off += s_red32[q];
-      off += __popc(bal & ((1u << lane) - 1));
-      if (sel && off < A.roots_cap) A.roots[off] = mem[p];
-      __syncthreads();
-      if (threadIdx.x == 0) { u32 tot = 0; for (u32 q = 0; q < blockDim.x / 32; ++q) tot += s_red32[q]; s_base += tot; }
-      __syncthreads();
-    }
-    n_roots = s_base;
+    if (lane == 0) R.state[c] = st;
   }
-  if (threadIdx.x == 0) {
-    ccld_hang_verdict v;
-    v.cls = cls; v.n_roots_total = n_roots; v.n_not_entered = n_ne; v.n_hung = n - n_ok; v.n_not_hung = n_ok;
-    v.n_missing_frames = cls == 3 ? n_missing : 0; v.stuck_step = stuck; v.n_members = n; v.min_total = min_total;
-    v.roots = nullptr; v.roots_cap = 0;
-    *A.out = v;
-  }
-}
-
-__global__ void __launch_bounds__(1024) k_hang_locate(const WinDesc* __restrict__ wd, Registry R, HangArgs A) { hang_locate_cta(wd[0], R, A); }
-
-// every alert of a window in one launch: one CTA per alert, each with its own scratch and output
-__global__ void __launch_bounds__(1024) k_hang_locate_many(const WinDesc* __restrict__ wd, Registry R, const HangArgs* __restrict__ args) {
-  const HangArgs A = args[blockIdx.x];
-  hang_locate_cta(wd[0], R, A);
+  if (!SINGLE) return;
+  if (lane == 0) s_an[wid] = n_an;
+  __syncthreads();
+  count_ops(R, c0, s_an);
 }
 
 }  // namespace ccld
+#include "ccld_hang.cuh"
 #include "ccld_tree.cuh"
