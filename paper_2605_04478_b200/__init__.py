@@ -75,6 +75,8 @@ class HangVerdict(C.Structure):
                [("min_total", C.c_uint64), ("roots", C.POINTER(C.c_uint32)), ("roots_cap", C.c_uint32)]
 
 
+_HANG_KEYS = ("cls", "n_roots_total", "n_not_entered", "n_hung", "n_not_hung", "n_missing_frames", "stuck_step", "n_members", "min_total")
+
 OPTABLE_I64 = ("e_min", "arrival_skew", "t_max", "t_min", "span", "med_skew", "mad_skew", "med_dur", "mad_dur")
 OPTABLE_U32 = ("rank_tmin", "rank_tmax", "max_chg", "rank_max_chg", "n_present", "gflags")
 
@@ -216,6 +218,8 @@ class Analyzer:
             raise CcldError(rc, "ccld_create failed")
         self._keep: Dict[int, list] = {}
         self._bufs: Dict[type, np.ndarray] = {}
+        self._ranks = np.empty(1, np.uint32)
+        self._hang_buf = None
         self._n_comms = 0
 
     # -- helpers
@@ -243,6 +247,12 @@ class Analyzer:
         size = (C.c_uint64 * k)(*[a.nbytes for a in out])
         self._check(self.lib.ccld_copy_many_to_host(self.h, k, dst, src, size))
         return out
+
+    def _rank_buf(self, n):
+        """Room for n rank ids, kept between calls like the lists above."""
+        if len(self._ranks) < n:
+            self._ranks = np.empty(n, np.uint32)
+        return self._ranks
 
     # -- the boundary
     def comm_register(self, comm: int, ranks, algo: int = 0, seq0: int = 0) -> None:
@@ -328,13 +338,12 @@ class Analyzer:
         return out
 
     def locate_hang(self, window_id: int, comm: int, seq: int, roots_cap: int = MAX_COMM_SIZE) -> Dict[str, object]:
-        roots = (C.c_uint32 * max(roots_cap, 1))()
+        roots = self._rank_buf(roots_cap)
         hv = HangVerdict()
-        hv.roots = C.cast(roots, C.POINTER(C.c_uint32)); hv.roots_cap = roots_cap
+        hv.roots = C.cast(roots.ctypes.data, C.POINTER(C.c_uint32)); hv.roots_cap = roots_cap
         self._check(self.lib.ccld_locate_hang(self.h, window_id, comm, seq, C.byref(hv)))
-        out: Dict[str, object] = {k: int(getattr(hv, k)) for k in ("cls", "n_roots_total", "n_not_entered", "n_hung", "n_not_hung",
-                                                                 "n_missing_frames", "stuck_step", "n_members", "min_total")}
-        out["roots"] = np.array(roots[:min(hv.n_roots_total, roots_cap)], dtype=np.uint32)
+        out: Dict[str, object] = {k: int(getattr(hv, k)) for k in _HANG_KEYS}
+        out["roots"] = roots[:min(hv.n_roots_total, roots_cap)].copy()
         return out
 
     def locate_hangs(self, window_id: int, cap: int = 1024, roots_stride: int = 64) -> List[Dict[str, object]]:
@@ -342,17 +351,20 @@ class Analyzer:
         comm, seq and age_ns."""
         n = C.c_uint32(0)
         cap = max(cap, 1)
-        hv = (HangVerdict * cap)(); al = (HangAlert * cap)()
-        roots = (C.c_uint32 * (cap * max(roots_stride, 1)))()
-        self._check(self.lib.ccld_locate_hangs(self.h, window_id, C.cast(al, C.c_void_p), C.cast(hv, C.c_void_p), cap,
-                                               C.cast(roots, C.c_void_p), roots_stride, C.byref(n)))
+        hv = self._hang_buf
+        if hv is None or len(hv) < cap:
+            hv = self._hang_buf = (HangVerdict * cap)()
+        al = self._list_buf(HangAlert, cap)
+        roots = self._rank_buf(cap * max(roots_stride, 1))
+        if cap > MAX_ALERTS_PER_WINDOW:                          # alerts beyond those kept are listed as zeros
+            C.memset(hv, 0, C.sizeof(hv)); al[:] = 0
+        self._check(self.lib.ccld_locate_hangs(self.h, window_id, al.ctypes.data, C.cast(hv, C.c_void_p), cap, roots.ctypes.data, roots_stride, C.byref(n)))
         res = []
         for i in range(min(n.value, cap)):
-            d: Dict[str, object] = {k: int(getattr(hv[i], k)) for k in ("cls", "n_roots_total", "n_not_entered", "n_hung", "n_not_hung",
-                                                                      "n_missing_frames", "stuck_step", "n_members", "min_total")}
-            k = min(hv[i].n_roots_total, roots_stride)
-            d["roots"] = np.array(roots[i * roots_stride:i * roots_stride + k], dtype=np.uint32)
-            d["comm"], d["seq"], d["age_ns"] = int(al[i].comm), int(al[i].seq), int(al[i].age_ns)
+            v = hv[i]
+            d: Dict[str, object] = {k: int(getattr(v, k)) for k in _HANG_KEYS}
+            d["roots"] = roots[i * roots_stride:i * roots_stride + min(v.n_roots_total, roots_stride)].copy()
+            d["comm"], d["seq"], d["age_ns"] = int(al["comm"][i]), int(al["seq"][i]), int(al["age_ns"][i])
             res.append(d)
         return res
 
@@ -367,13 +379,13 @@ class Analyzer:
 
     def opset_check(self, window_id: int, comm: int, seq: int, ranks_cap: int = MAX_COMM_SIZE) -> Dict[str, object]:
         """ccld_opset_check: majority Operation Type Set of op (comm, seq) and the ranks that deviate from it."""
-        ranks = (C.c_uint32 * max(ranks_cap, 1))()
+        ranks = self._rank_buf(ranks_cap)
         v = OpsetVerdict()
-        v.ranks = C.cast(ranks, C.POINTER(C.c_uint32)); v.ranks_cap = ranks_cap
+        v.ranks = C.cast(ranks.ctypes.data, C.POINTER(C.c_uint32)); v.ranks_cap = ranks_cap
         self._check(self.lib.ccld_opset_check(self.h, window_id, comm, seq, C.byref(v)))
         out: Dict[str, object] = {k: int(getattr(v, k)) for k in ("n_members", "n_present", "n_deviating_total", "majority_count",
                                                                 "op", "algo", "proto", "bytes")}
-        out["ranks"] = np.array(ranks[:min(v.n_deviating_total, ranks_cap)], dtype=np.uint32)
+        out["ranks"] = ranks[:min(v.n_deviating_total, ranks_cap)].copy()
         return out
 
     def state_export(self) -> bytes:

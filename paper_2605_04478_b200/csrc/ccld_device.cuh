@@ -27,9 +27,10 @@ constexpr int SMALL_SEQS = 256;        //   threads per CTA: eight warps, each o
 #endif
 constexpr u32 FUSED_WT_PER_CTA = CCLD_FUSED_WT_PER_CTA;   //   warp-tiles a CTA works through (a multiple of its eight warps)
 constexpr int WARP_N = 128;            // up to 128 ranks: one warp per group, bitonic sort in registers
-constexpr int MID_N = 1024;            // up to 1024 ranks: shared-memory bitonic sort, several groups per CTA
+constexpr int MID_ELEMS = 2048;        //   padded records per tile of a communicator of 9 to 128 ranks
+constexpr int MID_N = 1024;            // up to 1024 ranks: a warp per group, keys in its registers
 constexpr int MID_THREADS = 256;
-constexpr int MID_ELEMS = 2048;        //   padded records per tile
+constexpr int MID_SEQS = 8;            //   op counters per tile
 constexpr int LARGE_SEQS = 8;          // above: tiles of up to 8 consecutive op counters (as many as fit shared memory), radix select
 constexpr int LG_THREADS = 512;
 constexpr int LG_WARPS = LG_THREADS / 32;
@@ -152,7 +153,7 @@ __host__ __device__ inline u32 large_g(u32 n) {
 // op counters per work unit: a warp-tile (class 0) or a CTA tile (classes 1 to 3)
 __host__ __device__ inline u32 tile_seqs(u32 n) {
   u32 c = comm_class(n);
-  return c == 0 ? 32u : (c <= 2 ? MID_ELEMS / mid_npad(n) : (u32)LARGE_SEQS);
+  return c == 0 ? 32u : (c == 1 ? MID_ELEMS / mid_npad(n) : (c == 2 ? (u32)MID_SEQS : (u32)LARGE_SEQS));
 }
 __host__ __device__ inline u32 ceil_div(u32 a, u32 b) { return (a + b - 1) / b; }
 // chunking of a fused-class communicator with n_seq op counters in a window of T chunks

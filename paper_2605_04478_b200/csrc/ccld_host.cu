@@ -142,7 +142,8 @@ struct TimerSlot { cudaEvent_t a[TIMER_PAIRS], b[TIMER_PAIRS]; int kind[TIMER_PA
 struct ccld_ctx {
   ccld_params params; Params dp; int device = 0; cudaStream_t stream = nullptr;
   std::vector<CommHost> comms; std::unordered_map<u32, u32> comm_idx;
-  bool finalized = false; u32 n_ranks = 0, max_n = 0, max_large_n = 0; u64 sum_n = 0; size_t large_smem = 0; u32 n_sms = 148;
+  bool finalized = false; u32 n_ranks = 0, max_n = 0, max_large_n = 0, max_mid_n[3] = {0, 0, 0};     // mid: of the communicators padded to 256, 512, 1024 
+  u64 sum_n = 0; size_t large_smem = 0; u32 n_sms = 148;
   Block reg_blk, misc_blk; Registry reg; size_t stats_off = 0, stats_bytes = 0;
   const TreeRef* d_trees = nullptr; u32 n_trees = 0;     // tree communicators whose layers are known
   std::map<u32, WindowHost> windows;
@@ -234,7 +235,9 @@ int finalize_registry(ccld_ctx* ctx) {
   for (auto& c : ctx->comms) {
     for (u32 r : c.ranks) max_rank = std::max(max_rank, r);
     sum_n += c.ranks.size(); max_n = std::max<u32>(max_n, (u32)c.ranks.size());
-    if (c.ranks.size() > MID_N) max_large = std::max<u32>(max_large, (u32)c.ranks.size());
+    const u32 n = (u32)c.ranks.size(), cls = comm_class(n);
+    if (cls == 3) max_large = std::max<u32>(max_large, n);
+    if (cls == 2) { u32& m = ctx->max_mid_n[n <= 256 ? 0 : (n <= 512 ? 1 : 2)]; m = std::max(m, n); }
   }
   const u32 nr = max_rank + 1;
   u32 hsize = 16; while (hsize < 2 * nc) hsize <<= 1;
@@ -325,14 +328,16 @@ int finalize_registry(ccld_ctx* ctx) {
   ctx->misc_blk = ctx->pool.get(misc_layout(nr).total, &e);
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
 
-  CK(cudaFuncSetAttribute(k_reduce_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem_bytes(2 * WARP_N)));
+  CK(cudaFuncSetAttribute(k_reduce_mid<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem_bytes(256)));
+  CK(cudaFuncSetAttribute(k_reduce_mid<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem_bytes(512)));
+  CK(cudaFuncSetAttribute(k_reduce_mid<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem_bytes(MID_N)));
+  CK(cudaFuncSetAttribute(k_reduce_large_deferred, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(16ull * CCLD_MAX_COMM_SIZE)));
   CK(cudaFuncSetAttribute(k_seq_range, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)range_smem_bytes(RANGE_DIRECT)));
   CK(cudaFuncSetAttribute(k_hang_locate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(HANG_SMEM_N * HANG_MEMBER_BYTES)));
   CK(cudaFuncSetAttribute(k_opset_check, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(CCLD_MAX_COMM_SIZE * OPSET_MEMBER_BYTES)));
   if (max_large) {
     ctx->large_smem = large_smem(max_large);
     CK(cudaFuncSetAttribute(k_reduce_large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->large_smem));
-    CK(cudaFuncSetAttribute(k_reduce_large_deferred, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(16ull * max_large)));
   }
   ctx->finalized = true;
   return CCLD_OK;
@@ -816,7 +821,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   u64 total_groups = 0;
   for (u32 k = 0; k < B; ++k) total_groups += tot[(size_t)k * T_COUNT + T_GROUPS];
   const size_t o_def = take(n_list[B_FCTA] ? total_groups * 8 : 0),
-               o_def3 = take(n_list[B_T3] * (size_t)LARGE_SEQS * 8),          // likewise for the kernel of the largest communicators
+               o_def3 = take((n_list[B_T2] + n_list[B_T3]) * (size_t)LARGE_SEQS * 8),          // likewise for the kernels of larger communicators
                o_lgrp = take(n_list[B_T3] * (size_t)LARGE_SEQS * sizeof(LargeGroup)),
                o_skey = take(n_list[B_T3] ? total_slots * 4 : 0), o_dkey = take(n_list[B_T3] ? total_slots * 4 : 0);
   Block rb = ctx->pool.get(off, &e);
@@ -861,15 +866,29 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     k_reduce_fused<<<(u32)n_list[B_FCTA], SMALL_SEQS, 0, st>>>(d_desc, pl.fcta, pl.fwt, (TileSum*)(rbase + o_fsum), ctx->reg, ctx->dp, dl);
     k_reduce_deferred<<<DEF_GRID, DEF_WARPS * 32, 0, st>>>(d_desc, dl, ctx->reg, ctx->dp, now_ns);
   }
-  if (n_list[B_T2]) { TimedLaunch tl(ts, 4, st); k_reduce_mid<<<(u32)n_list[B_T2], MID_THREADS, mid_smem_bytes(2 * WARP_N), st>>>(d_desc, pl.t2, (TileSum*)(rbase + o_s2), ctx->reg, ctx->dp, now_ns); }
+  const DeferList dl_big{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
+  auto deferred_big = [&]() {
+    const u32 n = std::max(std::max(ctx->max_mid_n[0], ctx->max_mid_n[1]), std::max(ctx->max_mid_n[2], ctx->max_large_n));
+    k_reduce_large_deferred<<<LARGE_DEF_GRID, LARGE_DEF_THREADS, 16ull * n, st>>>(d_desc, dl_big, ctx->reg, ctx->dp, now_ns);
+  };
+  static_assert(MID_SEQS == LARGE_SEQS, "one list for the groups of both classes");
+  if (n_list[B_T2]) {
+    TimedLaunch tl(ts, 4, st);
+    const u32 grid = (u32)n_list[B_T2]; TileSum* sums = (TileSum*)(rbase + o_s2);
+    // one launch per padded size the registry has; a tile of another size ends at once
+    const u32* m = ctx->max_mid_n;
+    if (m[0]) k_reduce_mid<8><<<grid, MID_THREADS, mid_smem_bytes(m[0]), st>>>(d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[1]) k_reduce_mid<16><<<grid, MID_THREADS, mid_smem_bytes(m[1]), st>>>(d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[2]) k_reduce_mid<32><<<grid, MID_THREADS, mid_smem_bytes(m[2]), st>>>(d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (!n_list[B_T3]) deferred_big();
+  }
   if (n_list[B_T3]) {
-    const DeferList dl{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
     LargeGroup* lgrp = (LargeGroup*)(rbase + o_lgrp);
     TimedLaunch tl(ts, 5, st);
     k_large_stage<<<dim3((u32)n_list[B_T3], (ctx->max_large_n + LS_MEMBERS - 1) / LS_MEMBERS), LS_THREADS, 0, st>>>(d_desc, pl.t3, lgrp, ctx->reg);
     const u32 grid = (u32)std::min<u64>(n_list[B_T3], 2ull * ctx->n_sms);      // persistent: two CTAs per SM take the tiles in turn
-    k_reduce_large<<<grid, LG_THREADS, ctx->large_smem, st>>>(d_desc, pl.t3, (u32)n_list[B_T3], lgrp, (TileSum*)(rbase + o_s3), ctx->reg, ctx->dp, dl);
-    k_reduce_large_deferred<<<LARGE_DEF_GRID, LARGE_DEF_THREADS, 16ull * ctx->max_large_n, st>>>(d_desc, dl, ctx->reg, ctx->dp, now_ns);
+    k_reduce_large<<<grid, LG_THREADS, ctx->large_smem, st>>>(d_desc, pl.t3, (u32)n_list[B_T3], lgrp, (TileSum*)(rbase + o_s3), ctx->reg, ctx->dp, dl_big);
+    deferred_big();
   }
   {
     TimedLaunch tl(ts, 6, st);

@@ -9,9 +9,9 @@
 //                   n <= 8 one thread per group (warp-tiles), 9 <= n <= 128 n_pad / 8 lanes per group (register /
 //                   shuffle bitonic network); complete groups whose times fit 32-bit offsets
 //   k_reduce_deferred  the groups k_reduce_fused sets aside (incomplete, in flight, 64-bit spreads)
-//   k_reduce_mid    same, 129 <= n <= 1024 (shared-memory bitonic sort, several groups per CTA)
+//   k_reduce_mid    same, 129 <= n <= 1024 (ccld_mid.cuh: tiles of 8 op counters staged in shared memory, a warp per group)
 //   k_reduce_large  same, n > 1024 (ccld_large.cuh: a CTA per tile of 8 op counters, several groups side by side, radix select)
-//   k_reduce_large_deferred  the groups k_reduce_large sets aside
+//   k_reduce_large_deferred  the groups k_reduce_mid and k_reduce_large set aside
 //   k_window_rounds Eq. 2 per (communicator, window): round counts, selected round, location candidates
 //   k_window_decide Eq. 1, 3, 4 per communicator, windows in order: baseline state, class, slow location
 //   k_hang_locate   hang decision tree over presence / completion / progress counters (ccld_hang.cuh)
@@ -443,270 +443,10 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc*
 }  // namespace ccld
 
 #include "ccld_fused.cuh"
+#include "ccld_mid.cuh"
 #include "ccld_large.cuh"
 
 namespace ccld {
-
-// ------------------------------------------------------------------------------------------------
-// per-op reductions, 129 <= n <= 1024: a tile of S groups is staged in shared memory ([group][member],
-// pitch n_pad + 1), reduced by one warp per group, sorted by a bitonic network over all groups at once
-// ------------------------------------------------------------------------------------------------
-struct MidGroup {
-  u64 e_min, gbytes, med_s, mad_s, med_d, mad_d;
-  u32 gfl, gop;
-  u32 complete, analysed;
-};
-
-// Sort phase: full bitonic sort (merge_only = false) or only the final merge of a sequence that
-// falls and then rises (merge_only = true); every group of the tile in parallel.
-__device__ void mid_bitonic(u64* key, u32 S, u32 n_pad, u32 pitch, bool merge_only) {
-  const u32 half = n_pad >> 1, lg_half = 31 - __clz(half);
-  const u32 total = S * half;
-  for (u32 k = merge_only ? n_pad : 2; k <= n_pad; k <<= 1) {
-    for (u32 jj = k >> 1; jj > 0; jj >>= 1) {
-      for (u32 e = threadIdx.x; e < total; e += MID_THREADS) {
-        const u32 grp = e >> lg_half, q = e & (half - 1);
-        const u32 i = ((q & ~(jj - 1)) << 1) | (q & (jj - 1)), l = i | jj;
-        const bool up = (i & k) == 0 || k == n_pad;
-        u64* a = key + grp * pitch + i; u64* b = key + grp * pitch + l;
-        const u64 va = *a, vb = *b;
-        if ((va > vb) == up) { *a = vb; *b = va; }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-__global__ void __launch_bounds__(MID_THREADS) k_reduce_mid(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles,
-                                                            TileSum* __restrict__ sums, Registry R, Params P, i64 now) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const Tile t = tiles[blockIdx.x];
-  const WinDesc& D = wd[t.w];
-  const u32 c = t.c, n = R.comm_n[c];
-  const RangeRow row = D.ranges[c];
-  const u32* mem = R.members + R.comm_moff[c];
-  const u32 n_pad = mid_npad(n), pitch = n_pad + 1, S = t.count, S_max = MID_ELEMS / n_pad;
-  const u32 cap = S_max * pitch;
-  // shared-memory carve-up
-  u64* s_te = (u64*)smem_raw;            // enter time
-  u64* s_du = s_te + cap;                // duration
-  u64* s_key = s_du + cap;               // sort buffer
-  u64* s_by = s_key + cap;               // bytes
-  u32* s_idx = (u32*)(s_by + cap);       // record index
-  u32* s_ch = s_idx + cap;               // max(send_chg, recv_chg)
-  u8* s_op = (u8*)(s_ch + cap);
-  u8* s_st = s_op + cap;                 // 1 present, 2 in flight, 4 bad time
-  MidGroup* s_g = (MidGroup*)(((uintptr_t)(s_st + cap) + 15) & ~(uintptr_t)15);
-  __shared__ u32 s_cnt[8];
-  __shared__ u64 s_brng[MID_THREADS / 32];
-  __shared__ u32 s_bk[MID_THREADS / 32], s_rounds[MID_THREADS / 32];
-  u64 w_brng = 0; u32 w_bk = NONE, w_rounds = 0;          // this warp's Eq. 2 candidate and round count (lane 0)
-
-  const u64 slot_t = row.slot0 + (u64)t.seq_off * n;      // first slot of the tile
-  const u64 g_t = row.group0 + t.seq_off;                  // first group of the tile
-  const u32 n_el = S * n;
-  if (threadIdx.x < 8) s_cnt[threadIdx.x] = 0;
-  // 1. record indices, coalesced along the slot order
-  for (u32 p = threadIdx.x >> 5; p < n; p += MID_THREADS / 32) {
-    const u32* __restrict__ pm = D.perm + perm_at(row, t.seq_off, p);
-    for (u32 jg = threadIdx.x & 31; jg < S; jg += 32) s_idx[jg * pitch + p] = pm[jg];
-  }
-  __syncthreads();
-  // 2. gather: consecutive threads walk consecutive op counters of one member
-  for (u32 e = threadIdx.x; e < n_el; e += MID_THREADS) {
-    const u32 p = e / S, jg = e - p * S, a = jg * pitch + p;
-    const u32 idx = s_idx[a];
-    u64 te = 0, du = 0, by = 0; u32 ch = 0; u8 op = 0, st = 0;
-    if (idx != NONE) {
-      const i64 x = D.t_enter[idx], y = D.t_exit[idx];
-      by = D.bytes[idx]; op = D.op[idx];
-      if (D.send_chg != nullptr) { const u32 sc = D.send_chg[idx], rc = D.recv_chg[idx]; ch = sc > rc ? sc : rc; }
-      st = 1 | (y == -1 ? 2 : ((x < 0 || y < x) ? 4 : 0));
-      te = (u64)x; du = (u64)(y - x);
-    }
-    s_te[a] = te; s_du[a] = du; s_by[a] = by; s_ch[a] = ch; s_op[a] = op; s_st[a] = st;
-  }
-  __syncthreads();
-  // 3. one warp per group: cross-rank reductions
-  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  u32 c_comp = 0, c_inc = 0, c_bar = 0, c_an = 0, c_mis = 0, c_pres = 0;
-  for (u32 jg = wid; jg < S; jg += MID_THREADS / 32) {
-    const u32 b = jg * pitch;
-    u32 npres = 0, first = NONE, stor = 0;
-    for (u32 p = lane; p < n; p += 32) { const u32 st = s_st[b + p]; if (st & 1) { ++npres; first = first == NONE ? p : first; } stor |= st; }
-    npres = __reduce_add_sync(0xFFFFFFFFu, npres); first = __reduce_min_sync(0xFFFFFFFFu, first); stor = __reduce_or_sync(0xFFFFFFFFu, stor);
-    const bool have_first = first != NONE;
-    const u64 gbytes = have_first ? s_by[b + first] : 0; const u32 gop = have_first ? s_op[b + first] : 0;
-    const bool inflight = stor & 2, bad_time = stor & 4, complete = npres == n && !inflight && !bad_time;
-    const bool barrier = have_first && gop == CCLD_OP_ALLREDUCE && gbytes < P.barrier_bytes;
-    u32 mism = 0; i64 age = -1;
-    u64 e_min = U64_MAX_, tmax = 0, tmin = U64_MAX_; i64 x_max = INT64_MIN; u32 pmax = NONE, pmin = NONE; u64 chk = 0;
-    for (u32 p = lane; p < n; p += 32) {
-      const u32 st = s_st[b + p];
-      if (!(st & 1)) continue;
-      if (s_op[b + p] != gop || s_by[b + p] != gbytes) mism = 1;
-      const u64 te = s_te[b + p], du = s_du[b + p];
-      if (st & 2) { const i64 ag = now - (i64)te; age = ag > age ? ag : age; }
-      e_min = te < e_min ? te : e_min;
-      const i64 tx = (i64)(te + du); x_max = tx > x_max ? tx : x_max;
-      if (pmax == NONE || du > tmax) { tmax = du; pmax = p; }
-      if (pmin == NONE || du < tmin) { tmin = du; pmin = p; }
-      const u64 ck = ((u64)s_ch[b + p] << 32) | (u64)(NONE - p);        // most changes, then lowest position
-      chk = ck > chk ? ck : chk;
-    }
-    mism = __reduce_or_sync(0xFFFFFFFFu, mism);
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      const i64 ag = (i64)shfl_xor64((u64)age, d); age = ag > age ? ag : age;
-      const u64 em = shfl_xor64(e_min, d); e_min = em < e_min ? em : e_min;
-      const i64 xm = (i64)shfl_xor64((u64)x_max, d); x_max = xm > x_max ? xm : x_max;
-      const u64 ck = shfl_xor64(chk, d); chk = ck > chk ? ck : chk;
-      const u64 tM = shfl_xor64(tmax, d); const u32 pM = __shfl_xor_sync(0xFFFFFFFFu, pmax, d);
-      if (pM != NONE && (pmax == NONE || tM > tmax || (tM == tmax && pM < pmax))) { tmax = tM; pmax = pM; }
-      const u64 tm = shfl_xor64(tmin, d); const u32 pm = __shfl_xor_sync(0xFFFFFFFFu, pmin, d);
-      if (pm != NONE && (pmin == NONE || tm < tmin || (tm == tmin && pm < pmin))) { tmin = tm; pmin = pm; }
-    }
-    u32 gfl = (mism ? CCLD_G_OPSET_MISMATCH : 0) | (barrier ? CCLD_G_BARRIER : 0) | (inflight ? CCLD_G_INFLIGHT : 0) |
-              (bad_time ? CCLD_G_BAD_TIME : 0) | (complete ? CCLD_G_COMPLETE : CCLD_G_INCOMPLETE);
-    const bool analysed = complete && !barrier && n >= P.min_group;
-    if (analysed) gfl |= CCLD_G_ANALYSED;
-    const bool hang = !complete && inflight && age > P.hang_ns && !barrier;
-    if (hang) gfl |= CCLD_G_HANG_ALERT;
-    if (lane == 0) {
-      const u64 g = g_t + jg, G = D.n_groups;
-      if (hang) raise_alert(D, R.comm_id[c], row.seq_lo + t.seq_off + jg, age);
-      MidGroup mg; mg.e_min = e_min; mg.gbytes = gbytes; mg.gop = gop; mg.gfl = gfl; mg.complete = complete; mg.analysed = analysed;
-      mg.med_s = mg.mad_s = mg.med_d = mg.mad_d = 0;
-      s_g[jg] = mg;
-      i64 span = 0; double gb = 0.0;
-      if (complete) {
-        span = x_max - (i64)e_min;
-        double num, den; bus_factor(gop, n, &num, &den);
-        gb = busbw((double)gbytes * num, den, span);
-      }
-      D.gi64[(u64)GI_E_MIN * G + g] = complete ? (i64)e_min : 0;
-      D.gi64[(u64)GI_T_MAX * G + g] = complete ? (i64)tmax : 0; D.gi64[(u64)GI_T_MIN * G + g] = complete ? (i64)tmin : 0;
-      D.gi64[(u64)GI_SPAN * G + g] = span;
-      D.gu32[(u64)GU_RANK_TMIN * G + g] = complete ? mem[pmin] : 0; D.gu32[(u64)GU_RANK_TMAX * G + g] = complete ? mem[pmax] : 0;
-      D.gu32[(u64)GU_MAX_CHG * G + g] = complete ? (u32)(chk >> 32) : 0;
-      D.gu32[(u64)GU_RANK_MAX_CHG * G + g] = complete ? mem[NONE - (u32)chk] : 0;
-      D.gu32[(u64)GU_N_PRESENT * G + g] = npres; D.gu32[(u64)GU_GFLAGS * G + g] = gfl;
-      D.gbw[g] = gb;
-      c_comp += complete; c_inc += !complete; c_bar += barrier; c_an += analysed; c_mis += mism; c_pres += npres;
-      if (complete && !barrier) { ++w_rounds; best_merge(w_brng, w_bk, tmax - tmin, t.seq_off + jg); }
-    }
-  }
-  if (lane == 0) { s_brng[wid] = w_brng; s_bk[wid] = w_bk; s_rounds[wid] = w_rounds; }
-  __syncthreads();
-  const u32 k_med = (n - 1) >> 1;
-  // 4. arrival skew: sort, median, deviations, merge, MAD
-  for (u32 e = threadIdx.x; e < S * n_pad; e += MID_THREADS) {
-    const u32 jg = e / n_pad, i = e - jg * n_pad;
-    s_key[jg * pitch + i] = (i < n && s_g[jg].analysed) ? s_te[jg * pitch + i] - s_g[jg].e_min : U64_MAX_;
-  }
-  __syncthreads();
-  mid_bitonic(s_key, S, n_pad, pitch, false);
-  for (u32 jg = threadIdx.x; jg < S; jg += MID_THREADS) s_g[jg].med_s = s_key[jg * pitch + k_med];
-  __syncthreads();
-  for (u32 e = threadIdx.x; e < S * n_pad; e += MID_THREADS) {
-    const u32 jg = e / n_pad, i = e - jg * n_pad;
-    if (i < n) s_key[jg * pitch + i] = absdiff(s_key[jg * pitch + i], s_g[jg].med_s);
-  }
-  __syncthreads();
-  mid_bitonic(s_key, S, n_pad, pitch, true);
-  for (u32 jg = threadIdx.x; jg < S; jg += MID_THREADS) {
-    s_g[jg].mad_s = s_key[jg * pitch + k_med];
-    const u64 g = g_t + jg, G = D.n_groups; const bool an = s_g[jg].analysed;
-    D.gi64[(u64)GI_MED_SKEW * G + g] = an ? (i64)s_g[jg].med_s : 0; D.gi64[(u64)GI_MAD_SKEW * G + g] = an ? (i64)s_g[jg].mad_s : 0;
-  }
-  __syncthreads();
-  // 5. duration: the same
-  for (u32 e = threadIdx.x; e < S * n_pad; e += MID_THREADS) {
-    const u32 jg = e / n_pad, i = e - jg * n_pad;
-    s_key[jg * pitch + i] = (i < n && s_g[jg].analysed) ? s_du[jg * pitch + i] : U64_MAX_;
-  }
-  __syncthreads();
-  mid_bitonic(s_key, S, n_pad, pitch, false);
-  for (u32 jg = threadIdx.x; jg < S; jg += MID_THREADS) s_g[jg].med_d = s_key[jg * pitch + k_med];
-  __syncthreads();
-  for (u32 e = threadIdx.x; e < S * n_pad; e += MID_THREADS) {
-    const u32 jg = e / n_pad, i = e - jg * n_pad;
-    if (i < n) s_key[jg * pitch + i] = absdiff(s_key[jg * pitch + i], s_g[jg].med_d);
-  }
-  __syncthreads();
-  mid_bitonic(s_key, S, n_pad, pitch, true);
-  for (u32 jg = threadIdx.x; jg < S; jg += MID_THREADS) {
-    s_g[jg].mad_d = s_key[jg * pitch + k_med];
-    const u64 g = g_t + jg, G = D.n_groups; const bool an = s_g[jg].analysed;
-    D.gi64[(u64)GI_MED_DUR * G + g] = an ? (i64)s_g[jg].med_d : 0; D.gi64[(u64)GI_MAD_DUR * G + g] = an ? (i64)s_g[jg].mad_d : 0;
-  }
-  __syncthreads();
-  // 6. flags and votes, in slot order (coalesced byte stores)
-  u32 n_fs = 0, n_fd = 0;
-  for (u32 e = threadIdx.x; e < n_el; e += MID_THREADS) {
-    const u32 jg = e / n, p = e - jg * n, a = jg * pitch + p;
-    const MidGroup& mg = s_g[jg];
-    u8 f = CCLD_F_NOT_ANALYSED;
-    if (!(s_st[a] & 1)) f |= CCLD_F_MISSING;
-    else if (mg.analysed) {
-      const u64 sk = s_te[a] - mg.e_min, du = s_du[a];
-      const bool so = mul_gt(absdiff(sk, mg.med_s), 1000u, mg.mad_s, P.k_milli), sh = sk > mg.med_s;
-      const bool dq = mul_gt(absdiff(du, mg.med_d), 1000u, mg.mad_d, P.k_milli), dh = du > mg.med_d;
-      f = (so ? CCLD_F_SKEW_OUT : 0) | (dq ? CCLD_F_DUR_OUT : 0) | (sh ? CCLD_F_SKEW_HI : 0) | (dh ? CCLD_F_DUR_HI : 0);
-      if (so) { ++n_fs; atomicAdd(&R.votes[(u64)mem[p] * 4 + (sh ? 0 : 1)], 1u); }
-      if (dq) { ++n_fd; atomicAdd(&R.votes[(u64)mem[p] * 4 + (dh ? 2 : 3)], 1u); }
-    }
-    D.flags[slot_t + e] = f;
-  }
-  // arrival skew = largest enter time minus the smallest, one warp per group
-  for (u32 jg = wid; jg < S; jg += MID_THREADS / 32) {
-    u64 mx = 0;
-    if (s_g[jg].complete) {
-      for (u32 p = lane; p < n; p += 32) { const u64 v = s_te[jg * pitch + p]; mx = v > mx ? v : mx; }
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) { const u64 o = shfl_xor64(mx, d); mx = o > mx ? o : mx; }
-    }
-    if (lane == 0) D.gi64[(u64)GI_ARRIVAL_SKEW * D.n_groups + g_t + jg] = s_g[jg].complete ? (i64)(mx - s_g[jg].e_min) : 0;
-  }
-  // 7. per-rank bus bandwidth: thread p sums member p over the tile's groups
-  u32 n_bwc = 0;
-  for (u32 jg = 0; jg < S; ++jg) n_bwc += (s_g[jg].complete && !(s_g[jg].gfl & CCLD_G_BARRIER)) ? 1u : 0u;
-  if (n_bwc) {
-    for (u32 p = threadIdx.x; p < n; p += MID_THREADS) {
-      double v = 0.0;
-      for (u32 jg = 0; jg < S; ++jg) {
-        const MidGroup& mg = s_g[jg];
-        if (!mg.complete || (mg.gfl & CCLD_G_BARRIER)) continue;
-        double num, den; bus_factor(mg.gop, n, &num, &den);
-        v += busbw((double)mg.gbytes * num, den, (i64)s_du[jg * pitch + p]);
-      }
-      atomicAdd(&R.bw_sum[mem[p]], v);
-      atomicAdd(&R.bw_cnt[mem[p]], n_bwc);
-    }
-  }
-  // 8. counters
-  n_fs = __reduce_add_sync(0xFFFFFFFFu, n_fs); n_fd = __reduce_add_sync(0xFFFFFFFFu, n_fd);
-  if (lane == 0) {
-    atomicAdd(&s_cnt[0], c_comp); atomicAdd(&s_cnt[1], c_inc); atomicAdd(&s_cnt[2], c_bar); atomicAdd(&s_cnt[3], c_an);
-    atomicAdd(&s_cnt[4], c_mis); atomicAdd(&s_cnt[5], c_pres); atomicAdd(&s_cnt[6], n_fs); atomicAdd(&s_cnt[7], n_fd);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    u64 brng = s_brng[0]; u32 bk = s_bk[0], rounds = s_rounds[0];
-    for (int q = 1; q < MID_THREADS / 32; ++q) { best_merge(brng, bk, s_brng[q], s_bk[q]); rounds += s_rounds[q]; }
-    TileSum ts; ts.best_rng = brng; ts.best_k = bk; ts.n_rounds = rounds; ts.n_an = s_cnt[3]; ts.pad = 0;
-    sums[blockIdx.x] = ts;
-    count_add(D.counters, C_COMPLETE, s_cnt[0]); count_add(D.counters, C_INCOMPLETE, s_cnt[1]); count_add(D.counters, C_BARRIER, s_cnt[2]);
-    count_add(D.counters, C_ANALYSED, s_cnt[3]); count_add(D.counters, C_MISMATCH, s_cnt[4]); count_add(D.counters, C_PRESENT, s_cnt[5]);
-    count_add(D.counters, C_FLAG_SKEW, s_cnt[6]); count_add(D.counters, C_FLAG_DUR, s_cnt[7]);
-  }
-}
-
-inline size_t mid_smem_bytes(u32 n_pad_min) {
-  // cap = (MID_ELEMS / n_pad) * (n_pad + 1) is largest for the smallest n_pad
-  size_t cap = (size_t)(MID_ELEMS / n_pad_min) * (n_pad_min + 1);
-  return cap * (4 * 8 + 2 * 4 + 2) + 16 + (MID_ELEMS / n_pad_min) * sizeof(MidGroup);
-}
 
 // ------------------------------------------------------------------------------------------------
 // window decision per communicator (Sec. 4.2.1 Eq. 1-3, Sec. 4.2.2 Eq. 4): a warp per communicator.
