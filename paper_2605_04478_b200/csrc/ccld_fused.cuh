@@ -80,6 +80,12 @@ __device__ __forceinline__ double rcp_newton(double x) {
   e = fma(-x, r, 1.0); r = fma(r, e, r);
   return r;
 }
+// the same from a whole number >= 1, whose single-precision form needs no detour over fp64
+__device__ __forceinline__ double rcp_u32(u32 x) {
+  float s; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__uint2float_rn(x)));
+  const double r = (double)s;
+  return fma(r, fma(-(double)x, r, 1.0), r);
+}
 __device__ __forceinline__ double busbw_fast(double bytes_num, double den, i64 t) {
   return t > 0 ? bytes_num * rcp_newton((double)t * den) : 0.0;
 }
@@ -174,13 +180,14 @@ struct DeferList { u64* entries; u32* count; };    // entry: window index in the
 // Where a window's outputs go; kept in shared memory and read when a group stores, so that the pointers do not occupy
 // registers across the gathers.
 struct OutPtrs { u8* flags; i64* gi64; u32* gu32; double* gbw; u64 G; };
+struct InPtrs { const u32* perm; const i64 *te, *tx; const u64* by; const u8* op; const u32 *sc, *rc; };
 template <class T> __device__ __forceinline__ T ld_volatile(const T& x) { return *(const volatile T*)&x; }
 
 struct FusedShared {
   double bw[SMALL_SEQS / 32][WARP_N];
   u32 comm[SMALL_SEQS / 32], rounds[SMALL_SEQS / 32], n_an[SMALL_SEQS / 32], n_def[SMALL_SEQS / 32], brng[SMALL_SEQS / 32], bk[SMALL_SEQS / 32];
   u32 cnt[SC_COUNT];
-  OutPtrs out;
+  OutPtrs out; InPtrs in;
   // n <= 32: per thread (column) eight enter-time offsets and eight durations. 33 <= n <= 128: the tile's keys as
   // [metric][member][op counter], pitch S + 1 (S = op counters per tile), written by the staging phase of the tile.
   u32 stage[2 * (MID_ELEMS + WARP_N)];
@@ -528,31 +535,282 @@ __device__ __forceinline__ void flush_counters(const WinDesc& D, const FusedShar
   count_add(D.counters, C_FLAG_SKEW, sh.cnt[SC_FS]); count_add(D.counters, C_FLAG_DUR, sh.cnt[SC_FD]);
 }
 
-// Class-0 CTA (n <= 8): up to FUSED_WT_PER_CTA warp-tiles of one window and one time chunk, each up to 32 consecutive op
-// counters of one communicator with its own summary entry. A warp takes every eighth tile and meets the other warps
-// only at the end, so the warps of a CTA drift apart and one warp's gathers overlap another's arithmetic.
+// ------------------------------------------------------------------------------------------------
+// n <= 8: a warp per tile of up to 32 consecutive op counters, one group per lane
+// ------------------------------------------------------------------------------------------------
+// What a warp carries from tile to tile.
+struct SmallAcc { u32 complete = 0, barrier = 0, analysed = 0, mismatch = 0, present = 0, flagged = 0; };   // flagged: this lane's kind of vote (lane % 4)
+
+// A tile's list entry as one word per lane (16 words), so that the next tile's can wait in a single register.
+static_assert(sizeof(WarpTile) == 64, "an entry is sixteen words");
+__device__ __forceinline__ u32 entry_word(u32 e, u32 w) { return __shfl_sync(FULLM, e, w); }
+__device__ __forceinline__ u64 entry_pair(u32 e, u32 w) { return (u64)entry_word(e, w) | ((u64)entry_word(e, w + 1) << 32); }
+
+// The record indices of the tile behind entry e, asked into the warp's slots; lane l reads back what lane l asked for.
+__device__ __forceinline__ void ask_indices(const FusedShared& sh, u32 e, u32 lane, u32* __restrict__ slots /* [8][32] */) {
+  const u32 count = entry_word(e, 2), n_seq = entry_word(e, 5), n = entry_word(e, 7);
+  const u32* pm = ld_volatile(sh.in.perm) + entry_pair(e, 10) + entry_word(e, 1) + (lane < count ? lane : 0u);
+  const u32 dst = (u32)__cvta_generic_to_shared(slots + lane);
+#pragma unroll
+  for (u32 q = 0; q < 8; ++q) {
+    // positions beyond the communicator repeat its first member, which changes no extreme and no comparison
+    const u32* src = pm + (u64)(q < n ? q : 0u) * n_seq;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(dst + q * 128u), "l"(src) : "memory");
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// FULL: eight members. e: the tile's entry, its indices asked for earlier; e_next: the entry of the warp's next tile, if it has
+// one. One exposed round trip to memory per tile: times, sizes and op codes are asked for together as soon as the indices
+// are there, the rate columns while the order statistics are worked out, the next tile's indices before any of it.
+template <bool FULL>
+__device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool has_next, TileSum* __restrict__ sums, const Registry& R, const Params& P,
+                                           const DeferList& DL, FusedShared& sh, u32* __restrict__ slots, u32 lane, SmallAcc& acc) {
+  const u32 n = FULL ? 8u : entry_word(e, 7), count = entry_word(e, 2);
+  const bool active = lane < count;
+  const u32* __restrict__ mem = R.members + entry_pair(e, 14);
+  const u32 mem_l = lane < n ? __ldg(mem + lane) : 0u;        // lane m holds the rank of position m
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  u32 a[8], d[8];                                             // enter time against base, duration
+  u64 base, gby; u32 gop, idx[8], xmax;
+  bool ok, mm;
+  {
+    u32 top = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { idx[q] = slots[q * 32 + lane]; top = max(top, idx[q]); }
+    const bool present = top != NONE;                         // a missing member: the group is deferred
+#pragma unroll
+    for (int q = 0; q < 8; ++q) idx[q] = present ? idx[q] : 0u;
+    if (has_next) ask_indices(sh, e_next, lane, slots);
+    i64 ta[8], tb[8]; u64 by[8]; u32 op[8];
+    const i64* __restrict__ c_te = ld_volatile(sh.in.te); const i64* __restrict__ c_tx = ld_volatile(sh.in.tx);
+    const u64* __restrict__ c_by = ld_volatile(sh.in.by); const u8* __restrict__ c_op = ld_volatile(sh.in.op);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { ta[q] = __ldg(c_te + idx[q]); tb[q] = __ldg(c_tx + idx[q]); }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { by[q] = __ldg(c_by + idx[q]); op[q] = __ldg(c_op + idx[q]); }
+    // The upper words of a group's times are nearly always the same (they change every 4.3 s): the lower words are the keys
+    // then. Otherwise, and for anything irregular, offsets from the first member's enter time - 2^31 decide.
+    const u32 h0 = (u32)((u64)ta[0] >> 32);
+    u32 x = 0; bool back = false;
+    xmax = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      x |= ((u32)((u64)ta[q] >> 32) ^ h0) | ((u32)((u64)tb[q] >> 32) ^ h0);
+      a[q] = (u32)ta[q]; d[q] = (u32)tb[q] - (u32)ta[q];
+      back = back || (u32)tb[q] < (u32)ta[q];
+      xmax = max(xmax, (u32)tb[q]);
+    }
+    base = (u64)h0 << 32;
+    ok = x == 0 && (int)h0 >= 0 && !back;
+    if (!ok) {
+      base = (u64)ta[0] - 0x80000000ull;
+      u32 hx = 0, neg = 0;
+      back = false; xmax = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const u64 ra = (u64)ta[q] - base, rb = (u64)tb[q] - base;
+        a[q] = (u32)ra; d[q] = (u32)rb - (u32)ra; xmax = max(xmax, (u32)rb);
+        hx |= (u32)(ra >> 32) | (u32)(rb >> 32);
+        neg |= (u32)((u64)ta[q] >> 32) | (u32)((u64)tb[q] >> 32);
+        back = back || (u32)rb < (u32)ra;
+      }
+      ok = hx == 0 && (int)neg >= 0 && !back;                 // within 32 bits, not negative, not in flight (t_exit = -1), exit after enter
+    }
+    ok = ok && present;
+    gby = by[0]; gop = op[0];
+    u32 y = 0;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) y |= ((u32)by[q] ^ (u32)gby) | ((u32)(by[q] >> 32) ^ (u32)(gby >> 32)) | (op[q] ^ gop);
+    mm = y != 0;
+  }
+  // the rate columns, read only after the order statistics
+  u32 ch[8];
+  {
+    const u32* __restrict__ c_sc = ld_volatile(sh.in.sc); const u32* __restrict__ c_rc = ld_volatile(sh.in.rc);
+    if (c_sc != nullptr) {
+      u32 rc[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) { ch[q] = __ldg(c_sc + idx[q]); rc[q] = __ldg(c_rc + idx[q]); }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) ch[q] = max(ch[q], rc[q]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) ch[q] = 0;
+    }
+  }
+  const u32 sum_idx = entry_word(e, 3), seq_off = entry_word(e, 1);      // (every lane takes part in these)
+  const u64 group0 = entry_pair(e, 8), slot0 = entry_pair(e, 10);
+  const bool gok = active && ok;
+  if (active && !ok) {
+    const u32 at = atomicAdd(DL.count, 1u);
+    DL.entries[at] = ((u64)w_idx << 32) | (u64)(group0 + seq_off + lane);
+  }
+  const u32 b_ok = __ballot_sync(FULLM, gok);
+  const bool barrier = gop == CCLD_OP_ALLREDUCE && gby < P.barrier_bytes;
+  const bool round = gok && !barrier, analysed = round && n >= P.min_group;
+  const u32 b_an = __ballot_sync(FULLM, analysed), b_round = __ballot_sync(FULLM, round), b_mm = __ballot_sync(FULLM, gok && mm);
+  // ---- extremes and order statistics ----
+  u32 emin, emax, tmx, tmn, ms = 0, ds = 0, md = 0, dm = 0;
+  if (FULL) {
+    // the sorted keys give the extremes and the median (element 3). Below it the deviations L grow downwards, above it R
+    // upwards; the lower-median deviation is the third smallest of the two rows, and that is the least of max(L_i, R_j)
+    // over i + j = 3: no second sort.
+    u32 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = a[q];
+    sort8(v);
+    emin = v[0]; emax = v[7]; ms = v[3] - emin;
+    ds = min(min(v[3] - v[0], v[6] - v[3]), min(max(v[3] - v[2], v[5] - v[3]), max(v[3] - v[1], v[4] - v[3])));
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = d[q];
+    sort8(v);
+    tmn = v[0]; tmx = v[7]; md = v[3] - tmn;
+    dm = min(min(v[3] - v[0], v[6] - v[3]), min(max(v[3] - v[2], v[5] - v[3]), max(v[3] - v[1], v[4] - v[3])));
+  } else {
+    emin = a[0]; emax = a[0]; tmx = d[0]; tmn = d[0];
+#pragma unroll
+    for (int q = 1; q < 8; ++q) { emin = min(emin, a[q]); emax = max(emax, a[q]); tmx = max(tmx, d[q]); tmn = min(tmn, d[q]); }
+    if (b_an != 0) {
+      u32 v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = q < (int)n ? a[q] - emin : 0xFFFFFFFFu;
+      median_mad8<u32>(v, n, &ms, &ds);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = q < (int)n ? d[q] - tmn : 0xFFFFFFFFu;
+      median_mad8<u32>(v, n, &md, &dm);
+    }
+  }
+  if (!analysed) { ms = ds = md = dm = 0; }
+  // ---- flags ----
+  u32 f_lo = 0, f_hi = 0;
+  {
+    // |x - med| * 1000 > k * MAD in whole numbers: |x - med| > T = floor(k * MAD / 1000), which holds outside
+    // [med - T, med + T]; a quotient of 2^32 - 1 or more is never exceeded. One subtraction and one comparison per value.
+    const u64 qs = (u64)ds * P.k_milli / 1000u, qd = (u64)dm * P.k_milli / 1000u;
+    const u32 ts = qs > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qs, td = qd > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qd;
+    const u32 los = ms > ts ? ms - ts : 0u, lod = md > td ? md - td : 0u;
+    const u32 ws = (ms + ts < ms ? 0xFFFFFFFFu : ms + ts) - los, wd = (md + td < md ? 0xFFFFFFFFu : md + td) - lod;
+    const u32 s0 = emin + los, d0 = tmn + lod, sm = emin + ms, dmd = tmn + md;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      u32& f = q < 4 ? f_lo : f_hi;
+      const int at = 8 * (q & 3);
+      if (a[q] - s0 > ws) f |= (u32)CCLD_F_SKEW_OUT << at;
+      if (d[q] - d0 > wd) f |= (u32)CCLD_F_DUR_OUT << at;
+      if (a[q] > sm) f |= (u32)CCLD_F_SKEW_HI << at;
+      if (d[q] > dmd) f |= (u32)CCLD_F_DUR_HI << at;
+    }
+    if (!FULL) {                                              // positions that do not exist
+      f_lo &= n >= 4 ? 0xFFFFFFFFu : (1u << (8 * n)) - 1u;
+      f_hi &= n > 4 ? (n >= 8 ? 0xFFFFFFFFu : (1u << (8 * (n - 4))) - 1u) : 0u;
+    }
+    if (!analysed) { f_lo = 0x80808080u; f_hi = 0x80808080u; }
+  }
+  if (gok) {
+    u8* __restrict__ fp = ld_volatile(sh.out.flags) + slot0 + (u64)(seq_off + lane) * n;
+    if (FULL && (reinterpret_cast<uintptr_t>(fp) & 7) == 0) *reinterpret_cast<uint2*>(fp) = make_uint2(f_lo, f_hi);
+    else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) if (FULL || q < (int)n) fp[q] = (u8)((q < 4 ? f_lo >> (8 * q) : f_hi >> (8 * (q - 4))) & 0xFFu);
+    }
+  }
+  // ---- votes: the four kinds of outlier as one bit per member's byte, summed over the warp four members at a time (a sum
+  // fits its byte); lane 4 m + kind then holds member m's count of its kind and adds it with the warp's one atomic ----
+  static_assert(CCLD_F_SKEW_OUT == 1 && CCLD_F_DUR_OUT == 2 && CCLD_F_SKEW_HI == 4 && CCLD_F_DUR_HI == 8, "flag bit layout");
+  const u32 m = lane >> 2, rank_m = __shfl_sync(FULLM, mem_l, m);
+  {
+    const u32 one = 0x01010101u;
+    u32 mine = 0;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const u32 f = gok ? (half ? f_hi : f_lo) : 0u;
+      const u32 so = f & one, dq = (f >> 1) & one, sh_ = so & (f >> 2), dh = dq & (f >> 3);
+      const u32 v0 = __reduce_add_sync(FULLM, sh_), v1 = __reduce_add_sync(FULLM, so ^ sh_), v2 = __reduce_add_sync(FULLM, dh), v3 = __reduce_add_sync(FULLM, dq ^ dh);
+      const u32 v01 = lane & 1 ? v1 : v0, v23 = lane & 1 ? v3 : v2, v = lane & 2 ? v23 : v01;
+      if ((lane >> 4) == (u32)half) mine = v;
+    }
+    mine = (mine >> (8 * (m & 3))) & 0xFFu;
+    if (mine) atomicAdd(&R.votes[(u64)rank_m * 4 + (lane & 3)], mine);
+    acc.flagged += mine;
+  }
+  // ---- positions of the extremes (lowest among equals), ranks the row names ----
+  u32 cmx = ch[0];
+#pragma unroll
+  for (int q = 1; q < 8; ++q) cmx = max(cmx, ch[q]);
+  u32 pmax = 0, pmin = 0, pchg = 0;
+#pragma unroll
+  for (int q = 7; q >= 0; --q) { pmax = d[q] == tmx ? (u32)q : pmax; pmin = d[q] == tmn ? (u32)q : pmin; pchg = ch[q] == cmx ? (u32)q : pchg; }
+  const u32 r_tmin = __shfl_sync(FULLM, mem_l, pmin), r_tmax = __shfl_sync(FULLM, mem_l, pmax), r_chg = __shfl_sync(FULLM, mem_l, pchg);
+  // bytes * num / den: for eight members the factors 14/8 and 7/8 are exact
+  double fac = 1.0;
+  if (FULL) fac = gop == CCLD_OP_ALLREDUCE ? 1.75 : ((gop == CCLD_OP_ALLGATHER || gop == CCLD_OP_REDUCESCATTER || gop == CCLD_OP_ALLTOALL) ? 0.875 : 1.0);
+  else { double num, den; bus_factor(gop, n, &num, &den); fac = num / den; }
+  const double bn = (double)gby * fac;
+  if (gok) {
+    const u64 g = group0 + seq_off + lane, G = ld_volatile(sh.out.G);
+    i64* __restrict__ gi = ld_volatile(sh.out.gi64) + g; u32* __restrict__ gu = ld_volatile(sh.out.gu32) + g;
+    const u32 span = xmax - emin;
+    gi[(u64)GI_E_MIN * G] = (i64)(base + emin); gi[(u64)GI_ARRIVAL_SKEW * G] = (i64)(u64)(emax - emin);
+    gi[(u64)GI_T_MAX * G] = (i64)(u64)tmx; gi[(u64)GI_T_MIN * G] = (i64)(u64)tmn; gi[(u64)GI_SPAN * G] = (i64)(u64)span;
+    gi[(u64)GI_MED_SKEW * G] = (i64)(u64)ms; gi[(u64)GI_MAD_SKEW * G] = (i64)(u64)ds;
+    gi[(u64)GI_MED_DUR * G] = analysed ? (i64)((u64)tmn + md) : 0; gi[(u64)GI_MAD_DUR * G] = (i64)(u64)dm;
+    gu[(u64)GU_RANK_TMIN * G] = r_tmin; gu[(u64)GU_RANK_TMAX * G] = r_tmax;
+    gu[(u64)GU_MAX_CHG * G] = cmx; gu[(u64)GU_RANK_MAX_CHG * G] = r_chg;
+    gu[(u64)GU_N_PRESENT * G] = n;
+    gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mm ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
+    ld_volatile(sh.out.gbw)[g] = span ? bn * rcp_newton((double)span) : 0.0;
+  }
+  // ---- per-member bandwidth, summed over the warp; the Eq. 2 candidate; counts ----
+  double bw[8];
+  const double bd = round ? bn : 0.0;
+  if (!__any_sync(FULLM, tmn == 0)) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) bw[q] = bd * rcp_u32(d[q]);
+  } else {                                                    // an op of no duration adds nothing
+#pragma unroll
+    for (int q = 0; q < 8; ++q) bw[q] = d[q] != 0 ? bd * rcp_u32(d[q]) : 0.0;
+  }
+  const double tot = warp_sum8(bw, lane);                     // lane l holds member 4 bit4(l) + 2 bit3(l) + bit2(l)
+  const u32 rounds = (u32)__popc(b_round);
+  if ((lane & 3) == 0 && m < n && rounds) { atomicAdd(&R.bw_sum[rank_m], tot); atomicAdd(&R.bw_cnt[rank_m], rounds); }
+  const u32 rng = round ? tmx - tmn : 0u, best = __reduce_max_sync(FULLM, rng);
+  const u32 b_best = __ballot_sync(FULLM, round && rng == best);            // ties: the lowest op counter
+  const u32 n_ok = (u32)__popc(b_ok), n_an = (u32)__popc(b_an);
+  if (lane == 0) {
+    TileSum ts; ts.best_rng = b_best ? best : 0u; ts.best_k = b_best ? seq_off + (u32)__ffs(b_best) - 1u : NONE; ts.n_rounds = rounds; ts.n_an = n_an;
+    ts.pad = count - n_ok;
+    sums[sum_idx] = ts;
+  }
+  acc.complete += n_ok; acc.barrier += n_ok - rounds; acc.analysed += n_an; acc.mismatch += (u32)__popc(b_mm); acc.present += n_ok * n;
+}
+
+// Class-0 CTA: up to FUSED_WT_PER_CTA warp-tiles of one window and one time chunk, each up to 32 consecutive op counters of
+// one communicator with its own summary entry. A warp takes every eighth tile and meets the other warps only at the end, so
+// the warps of a CTA drift apart and one warp's gathers overlap another's arithmetic.
 __device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta& t, const WarpTile* __restrict__ wts, TileSum* __restrict__ sums,
                                                 const Registry& R, const Params& P, const DeferList& DL, FusedShared& sh) {
   const u32 wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();                                          // the CTA's counters are zero
-  for (u32 i = wid; i < t.wt_count; i += SMALL_SEQS / 32) {
-    const WarpTile wt = wts[t.wt_first + i];
-    FastAcc acc; double bw[8];
-    if (wt.row.n == SMALL_N) fast_groups<1, true>(D, t.w, wt.row, R.members + wt.moff, wt.seq_off, wt.count, R, P, DL, sh, acc, bw);
-    else fast_groups<1, false>(D, t.w, wt.row, R.members + wt.moff, wt.seq_off, wt.count, R, P, DL, sh, acc, bw);
-    warp_fold<1>(acc, bw, wt.row.n, sh);
-    __syncwarp();
-    if (lane == 0) {
-      TileSum ts; ts.best_rng = sh.brng[wid]; ts.best_k = sh.bk[wid]; ts.n_rounds = sh.rounds[wid]; ts.n_an = sh.n_an[wid]; ts.pad = sh.n_def[wid];
-      sums[wt.sum_idx] = ts;
-    }
-    // per-rank bandwidth of the tile: lane m < n adds member m's sum
-    const u32 rounds = sh.rounds[wid];
-    if (lane < wt.row.n && rounds) {
-      const u32 rank = R.members[wt.moff + lane];
-      atomicAdd(&R.bw_sum[rank], sh.bw[wid][lane]); atomicAdd(&R.bw_cnt[rank], rounds);
-    }
-    __syncwarp();
+  constexpr u32 NW = SMALL_SEQS / 32;
+  u32* const slots = sh.stage + wid * 256;
+  const u32* __restrict__ list = reinterpret_cast<const u32*>(wts + t.wt_first);
+  const auto entry = [&](u32 i) { return i < t.wt_count ? __ldg(list + (u64)i * 16 + (lane & 15)) : 0u; };
+  u32 e = entry(wid);
+  __syncthreads();                                          // the CTA's counters and pointers are set
+  if (wid < t.wt_count) ask_indices(sh, e, lane, slots);
+  u32 e_next = entry(wid + NW);
+  SmallAcc acc;
+  for (u32 i = wid; i < t.wt_count; i += NW) {
+    const u32 e_after = entry(i + 2 * NW);
+    const bool has_next = i + NW < t.wt_count;
+    if (entry_word(e, 7) == SMALL_N) small_tile<true>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
+    else small_tile<false>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
+    e = e_next; e_next = e_after;
+  }
+  const u32 f_skew = __reduce_add_sync(FULLM, lane & 2 ? 0u : acc.flagged), f_dur = __reduce_add_sync(FULLM, lane & 2 ? acc.flagged : 0u);
+  if (lane == 0) {
+    atomicAdd(&sh.cnt[SC_COMP], acc.complete); atomicAdd(&sh.cnt[SC_BAR], acc.barrier); atomicAdd(&sh.cnt[SC_AN], acc.analysed);
+    atomicAdd(&sh.cnt[SC_MIS], acc.mismatch); atomicAdd(&sh.cnt[SC_PRES], acc.present); atomicAdd(&sh.cnt[SC_FS], f_skew); atomicAdd(&sh.cnt[SC_FD], f_dur);
   }
   __syncthreads();
   if (threadIdx.x == 0) flush_counters(D, sh);
@@ -609,6 +867,7 @@ __global__ void __launch_bounds__(SMALL_SEQS, CCLD_FUSED_MIN_CTAS) k_reduce_fuse
   const WinDesc& D = wd[t.w];
   if (threadIdx.x < SC_COUNT) sh.cnt[threadIdx.x] = 0;
   if (threadIdx.x == 0) { sh.out.flags = D.flags; sh.out.gi64 = D.gi64; sh.out.gu32 = D.gu32; sh.out.gbw = D.gbw; sh.out.G = D.n_groups; }
+  if (threadIdx.x == 32) { sh.in.perm = D.perm; sh.in.te = D.t_enter; sh.in.tx = D.t_exit; sh.in.by = D.bytes; sh.in.op = D.op; sh.in.sc = D.send_chg; sh.in.rc = D.recv_chg; }
   if (t.cls == 0) { fused_small_cta(D, t, wts, sums, R, P, DL, sh); return; }
   __syncthreads();
   const u32 n_pad = mid_npad(t.row.n);
