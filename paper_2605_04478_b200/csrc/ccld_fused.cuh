@@ -147,32 +147,21 @@ __device__ __forceinline__ void sub_merge(K (&v)[8], u32 s) {
   merge8(v);
 }
 
-// Lower median and lower-median absolute deviation of a group's keys (x[q] = maximum key where the position does
-// not exist or the group is not sorted at all). Every lane of the warp must call it.
-template <int L, class K>
-__device__ __forceinline__ void sub_median_mad(const K (&x)[8], u32 n, u32 s, u32 lane, K* med, K* mad) {
-  K v[8];
+// Smallest and largest key, lower median and lower-median absolute deviation of a group's keys (v[q] = largest key where no
+// member exists; any order). Every lane of the warp must call it.
+template <int L, bool FULL>
+__device__ __forceinline__ void sub_stats(u32 (&v)[8], u32 n, u32 s, u32 lane, u32* mn, u32* mx, u32* med, u32* mad) {
+  const u32 first = lane & ~(u32)(L - 1), k = (n - 1) >> 1;
+  sub_sort<L, u32>(v, s);
+  *mn = __shfl_sync(0xFFFFFFFFu, v[0], first);
+  *mx = __shfl_sync(0xFFFFFFFFu, FULL ? v[7] : pick8(v, (n - 1) & 7), first | ((n - 1) >> 3));
+  const u32 m = __shfl_sync(0xFFFFFFFFu, FULL ? v[7] : pick8(v, k & 7), first | (k >> 3));         // full: k = 4 L - 1
 #pragma unroll
-  for (int q = 0; q < 8; ++q) v[q] = x[q];
-  sub_sort<L, K>(v, s);
-  const u32 k = (n - 1) >> 1, src = (lane & ~(u32)(L - 1)) | (k >> 3);
-  const K m = __shfl_sync(0xFFFFFFFFu, pick8(v, k & 7), src);
-#pragma unroll
-  for (int r = 0; r < 8; ++r) v[r] = s * 8 + r < n ? key_absdiff(v[r], m) : KeyMax<K>::v();   // falls to 0 at k, then rises
-  sub_merge<L, K>(v, s);
-  *med = m; *mad = __shfl_sync(0xFFFFFFFFu, pick8(v, k & 7), src);
+  for (int r = 0; r < 8; ++r) v[r] = (FULL || s * 8 + r < n) ? key_absdiff(v[r], m) : 0xFFFFFFFFu;   // falls to 0 at k, then rises
+  sub_merge<L, u32>(v, s);
+  *med = m; *mad = __shfl_sync(0xFFFFFFFFu, FULL ? v[7] : pick8(v, k & 7), first | (k >> 3));
 }
 
-
-// Per-lane running totals of the groups a warp has handled. Group counts live in the first lane of each group, six
-// bits each; flag counts in the lane of the record, sixteen bits each.
-struct FastAcc {
-  u32 groups = 0;          // complete | barrier << 6 | analysed << 12 | mismatch << 18 | round << 24
-  u32 flagged = 0;         // skew flags | duration flags << 16
-  u32 n_def = 0;
-  u32 best_rng = 0, best_k = NONE;
-};
-enum { FA_COMP = 0, FA_BAR = 6, FA_AN = 12, FA_MIS = 18, FA_ROUND = 24 };
 enum { SC_COMP = 0, SC_INC, SC_BAR, SC_AN, SC_MIS, SC_PRES, SC_FS, SC_FD, SC_COUNT };
 
 struct DeferList { u64* entries; u32* count; };    // entry: window index in the batch << 32 | group index in the window
@@ -183,351 +172,21 @@ struct OutPtrs { u8* flags; i64* gi64; u32* gu32; double* gbw; u64 G; };
 struct InPtrs { const u32* perm; const i64 *te, *tx; const u64* by; const u8* op; const u32 *sc, *rc; };
 template <class T> __device__ __forceinline__ T ld_volatile(const T& x) { return *(const volatile T*)&x; }
 
+constexpr u32 TILE_KEYS = 2304;                               // keys of a metric of a staged tile, padding included
+constexpr u32 TILE_OPS = 64;                                  // op counters of a staged tile at most
 struct FusedShared {
-  double bw[SMALL_SEQS / 32][WARP_N];
-  u32 comm[SMALL_SEQS / 32], rounds[SMALL_SEQS / 32], n_an[SMALL_SEQS / 32], n_def[SMALL_SEQS / 32], brng[SMALL_SEQS / 32], bk[SMALL_SEQS / 32];
   u32 cnt[SC_COUNT];
   OutPtrs out; InPtrs in;
-  // n <= 32: per thread (column) eight enter-time offsets and eight durations. 33 <= n <= 128: the tile's keys as
-  // [metric][member][op counter], pitch S + 1 (S = op counters per tile), written by the staging phase of the tile.
-  u32 stage[2 * (MID_ELEMS + WARP_N)];
-  u64 t_base[32], t_gby[32], t_ck[SMALL_SEQS / 32][32];       // staged tiles, per op counter: time base, size of the op, most changes per warp
-  u32 t_gop[32], t_bits[32];                                  //   op code; 1 = some record disqualifies the group, 2 = the op set differs
+  // n <= 8: eight warps' slots for the record indices of a tile. Larger: a tile's keys as [metric][member][op counter].
+  u32 stage[2 * TILE_KEYS];
+  // staged tiles, per op counter: why the group is set aside (1) or its op set differs (2), latest exit, first member's
+  u32 t_bits[TILE_OPS], t_xmax[TILE_OPS], t_gop[TILE_OPS];    //   op code,
+  u64 t_base[TILE_OPS], t_gby[TILE_OPS];                      //   time base and size
+  u64 t_ck[SMALL_SEQS / 32][32];                              //   most changes, per warp
+  double t_bd[TILE_OPS];                                      //   bytes * factor where the group adds bandwidth, else 0
+  u32 mem[WARP_N];                                            // the communicator's ranks
+  u32 brng[SMALL_SEQS / 32], bk[SMALL_SEQS / 32], rounds[SMALL_SEQS / 32], n_an[SMALL_SEQS / 32], n_def[SMALL_SEQS / 32];
 };
-constexpr u32 STAGE_ROWS = SMALL_SEQS;                        // row pitch of the per-thread layout
-
-// Staging phase of a tile of a communicator of 33 to 128 ranks (S = 2048 / n_pad op counters, S <= 32): the CTA's warps
-// share the members, lanes run along the op counter, so the record indices of a warp step are one contiguous piece of
-// the member-major permutation and - in a rank-major upload - the records themselves lie in one short stretch of a
-// rank's stream instead of one sector per lane. Times become 32-bit keys against the group's first member (whose enter
-// time, size and op code every thread loads for its own op counter), the op-set check and the rate column are reduced on
-// the way; the keys land in shared memory as [metric][member][op counter].
-template <int L>
-__device__ __forceinline__ void stage_tile(const WinDesc& D, const RangeRow& row, u32 seq0, u32 count, FusedShared& sh) {
-  constexpr u32 S = 32 / L * (SMALL_SEQS / 32), PITCH = S + 1, NW = SMALL_SEQS / 32;     // S op counters per tile: 32 (n_pad 64), 16 (n_pad 128)
-  constexpr u32 MPS = 32 / S;                                  // members a warp step covers
-  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n = row.n;
-  const u32 sq = lane & (S - 1), ml = lane / S;
-  const bool sv = sq < count;
-  const u32* __restrict__ perm = D.perm + row.slot0 + seq0 + (sv ? sq : 0u);
-  const i64* __restrict__ c_te = D.t_enter; const i64* __restrict__ c_tx = D.t_exit;
-  const u64* __restrict__ c_by = D.bytes; const u8* __restrict__ c_op = D.op;
-  const u32* __restrict__ c_sc = D.send_chg; const u32* __restrict__ c_rc = D.recv_chg;
-  u32 bits = 0; i64 te0 = 0; u64 by0 = 0; u32 op0 = 0;
-  {
-    const u32 i0 = sv ? __ldg(perm) : NONE;
-    if (i0 != NONE) { te0 = c_te[i0]; by0 = c_by[i0]; op0 = c_op[i0]; } else bits = 1;
-  }
-  const u64 base = (u64)te0 - 0x80000000ull;
-  u64 ck = 0;
-  u32* __restrict__ k_a = sh.stage; u32* __restrict__ k_d = sh.stage + (MID_ELEMS + WARP_N);
-  // member of warp step i: wid * MPS + ml + i * NW * MPS
-  for (u32 p0 = wid * MPS + ml; p0 < n; p0 += 4 * NW * MPS) {
-    u32 idx[4]; i64 x[4], y[4]; u64 by[4]; u32 op[4], ch[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) { const u32 p = p0 + q * NW * MPS; idx[q] = (sv && p < n) ? __ldg(perm + (u64)p * row.n_seq) : NONE; }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const u32 ix = idx[q] == NONE ? 0u : idx[q];
-      x[q] = c_te[ix]; y[q] = c_tx[ix]; by[q] = c_by[ix]; op[q] = c_op[ix]; ch[q] = 0;
-      if (c_sc != nullptr) { const u32 sc = c_sc[ix], rc = c_rc[ix]; ch[q] = max(sc, rc); }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const u32 p = p0 + q * NW * MPS;
-      if (p < n) {
-        u32 a_lo = 0, d = 0;
-        if (idx[q] == NONE) { if (sv) bits |= 1; }
-        else {
-          const u64 ra = (u64)x[q] - base, rb = (u64)y[q] - base;
-          a_lo = (u32)ra; const u32 b_lo = (u32)rb; d = b_lo - a_lo;
-          if (((ra | rb) >> 32) != 0 || (x[q] | y[q]) < 0 || b_lo < a_lo) bits |= 1;     // beyond 32 bits, negative or in flight, exit before enter
-          if (op[q] != op0 || by[q] != by0) bits |= 2;
-          const u64 k2 = ((u64)ch[q] << 32) | (u64)(NONE - p); ck = k2 > ck ? k2 : ck;     // most changes, then the lowest position
-        }
-        k_a[p * PITCH + sq] = a_lo; k_d[p * PITCH + sq] = d;
-      }
-    }
-  }
-  if (MPS > 1) {                                              // the lanes that share an op counter
-#pragma unroll
-    for (u32 h = S; h < 32; h <<= 1) { bits |= __shfl_xor_sync(FULLM, bits, h); const u64 o = shfl_xor64(ck, h); ck = o > ck ? o : ck; }
-  }
-  if (lane < S) {
-    sh.t_ck[wid][lane] = ck;
-    if (bits) atomicOr(&sh.t_bits[lane], bits);
-    if (wid == 0) { sh.t_base[lane] = base; sh.t_gby[lane] = by0; sh.t_gop[lane] = op0; }
-  }
-}
-
-// One group per L lanes, eight ring positions per lane (position s * 8 + q in lane s of the group); the warp takes
-// 32 / L consecutive op counters starting at offset seq0 of the communicator's range, `count` of them valid.
-// FULL: the communicator fills every position (n = 8 L). STAGED: the tile's keys and per-op values wait in shared memory
-// (stage_tile); jt0 = the warp's first op counter inside the tile.
-template <int L, bool FULL, bool STAGED = false>
-__device__ __forceinline__ void fast_groups(const WinDesc& D, u32 w_idx, const RangeRow& row, const u32* __restrict__ mem, u32 seq0, u32 count,
-                                            const Registry& R, const Params& P, const DeferList& DL, FusedShared& sh, FastAcc& acc, double (&bw)[8],
-                                            u32 jt0 = 0) {
-  const u32 lane = threadIdx.x & 31, s = lane % L, j = lane / L, base_lane = lane - s, p0 = s * 8;
-  const u32 gmask = L == 32 ? FULLM : (((1u << (L & 31)) - 1u) << base_lane);
-  const u32 n = FULL ? (u32)(L * 8) : row.n;
-  const bool active = j < count, lead = s == 0;
-  constexpr u32 S_T = STAGED ? 32 / L * (SMALL_SEQS / 32) : 1, PITCH = S_T + 1;
-  // where the keys of my eight positions are: a column of the per-thread layout, or rows of the staged tile
-  const u32 jt = STAGED ? (active ? jt0 + j : jt0) : 0u;
-  const u32* __restrict__ ka = STAGED ? sh.stage + p0 * PITCH + jt : &sh.stage[threadIdx.x];
-  const u32* __restrict__ kd = STAGED ? sh.stage + (MID_ELEMS + WARP_N) + p0 * PITCH + jt : &sh.stage[8 * STAGE_ROWS + threadIdx.x];
-  constexpr u32 KSTEP = STAGED ? PITCH : STAGE_ROWS;
-  u32* __restrict__ my = &sh.stage[threadIdx.x];              // my[q * SMALL_SEQS]: offset of position q, my[(8 + q) * SMALL_SEQS]: duration
-
-  bool ok = true;
-  u32 emin = 0xFFFFFFFFu, emax = 0, xmax = 0, tmx = 0, tmn = 0xFFFFFFFFu;
-  u64 base;
-  bool mm = false;
-  u64 gby, ck = 0; u32 gop;
-  // thread per group: lane m fetches the rank of ring position m now, so that the ranks a row names are a shuffle away
-  // when the row is written instead of one more round trip to memory
-  u32 mem_l = 0;
-  if (L == 1) mem_l = lane < n ? __ldg(mem + lane) : 0u;
-  if (STAGED) {
-    base = sh.t_base[jt]; gby = sh.t_gby[jt]; gop = sh.t_gop[jt];
-    const u32 bits = sh.t_bits[jt];
-    ok = !(bits & 1); mm = (bits & 2) != 0;
-#pragma unroll
-    for (int w = 0; w < SMALL_SEQS / 32; ++w) { const u64 o = sh.t_ck[w][jt]; ck = o > ck ? o : ck; }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      if (FULL || p0 + q < n) {
-        const u32 a_lo = ka[q * KSTEP], d = kd[q * KSTEP];
-        emin = min(emin, a_lo); emax = max(emax, a_lo); xmax = max(xmax, a_lo + d);
-        tmx = max(tmx, d); tmn = min(tmn, d);
-      }
-    }
-  } else {
-  // ---- record indices of my eight positions (member-major permutation: stride n_seq) ----
-  u32 idx[8];
-  {
-    const u32* __restrict__ pm = D.perm + row.slot0 + (u64)p0 * row.n_seq + seq0 + (active ? j : 0u);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) idx[q] = (active && (FULL || p0 + q < n)) ? __ldg(pm + (u64)q * row.n_seq) : NONE;
-  }
-#pragma unroll
-  for (int q = 0; q < 8; ++q) if ((FULL || p0 + q < n) && idx[q] == NONE) ok = false;      // a missing member: the group is deferred
-
-  // ---- batch 1: times, turned into 32-bit offsets from (first member's enter time - 2^31 ns) as they arrive ----
-  {
-    const i64* __restrict__ c_te = D.t_enter; const i64* __restrict__ c_tx = D.t_exit;
-    i64 ta[8], tb[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) { const u32 ix = idx[q] == NONE ? 0u : idx[q]; ta[q] = c_te[ix]; tb[q] = c_tx[ix]; }
-    base = (L == 1 ? (u64)ta[0] : __shfl_sync(FULLM, (u64)ta[0], base_lane)) - 0x80000000ull;
-    u32 hx = 0, neg = 0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const u64 ra = (u64)ta[q] - base, rb = (u64)tb[q] - base;
-      const u32 a_lo = (u32)ra, b_lo = (u32)rb, d = b_lo - a_lo;
-      my[q * SMALL_SEQS] = a_lo; my[(8 + q) * SMALL_SEQS] = d;
-      if (FULL || p0 + q < n) {
-        hx |= (u32)(ra >> 32) | (u32)(rb >> 32);
-        neg |= (u32)((u64)ta[q] >> 32) | (u32)((u64)tb[q] >> 32);
-        if (b_lo < a_lo) ok = false;
-        emin = min(emin, a_lo); emax = max(emax, a_lo); xmax = max(xmax, b_lo);
-        tmx = max(tmx, d); tmn = min(tmn, d);
-      }
-    }
-    if (hx != 0 || (int)neg < 0) ok = false;       // beyond 32 bits, negative, or in flight (t_exit = -1)
-  }
-  // ---- batch 2: op set (every member against the group's first) and rate column ----
-  {
-    const u64* __restrict__ c_by = D.bytes; const u8* __restrict__ c_op = D.op;
-    const u32* __restrict__ c_sc = D.send_chg; const u32* __restrict__ c_rc = D.recv_chg;
-    u64 by[8]; u32 op[8], ch[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const u32 ix = idx[q] == NONE ? 0u : idx[q];
-      by[q] = c_by[ix]; op[q] = c_op[ix]; ch[q] = 0;
-      if (c_sc != nullptr) { const u32 sc = c_sc[ix], rc = c_rc[ix]; ch[q] = max(sc, rc); }
-    }
-    gby = L == 1 ? by[0] : __shfl_sync(FULLM, by[0], base_lane);
-    gop = L == 1 ? op[0] : __shfl_sync(FULLM, op[0], base_lane);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      if (FULL || p0 + q < n) {
-        if (op[q] != gop || by[q] != gby) mm = true;
-        const u64 k2 = ((u64)ch[q] << 32) | (u64)(NONE - (p0 + q));          // most changes, then the lowest position
-        ck = k2 > ck ? k2 : ck;
-      }
-    }
-  }
-  }
-  // ---- the lanes of a group meet ----
-  bool gok = active && ok;
-  if (L > 1) { const u32 b_ok = __ballot_sync(FULLM, ok); gok = active && (b_ok & gmask) == gmask; }     // every lane votes
-  if (active && !gok && lead) {
-    const u32 e = atomicAdd(DL.count, 1u);
-    DL.entries[e] = ((u64)w_idx << 32) | (u64)(row.group0 + seq0 + j);
-    ++acc.n_def;
-  }
-#pragma unroll
-  for (int q = 0; q < 8; ++q) bw[q] = 0.0;
-  if (!__any_sync(FULLM, gok)) return;
-  if (L > 1) {
-#pragma unroll
-    for (int h = 1; h < L; h <<= 1) {
-      emin = min(emin, __shfl_xor_sync(FULLM, emin, h)); emax = max(emax, __shfl_xor_sync(FULLM, emax, h));
-      xmax = max(xmax, __shfl_xor_sync(FULLM, xmax, h));
-      tmx = max(tmx, __shfl_xor_sync(FULLM, tmx, h)); tmn = min(tmn, __shfl_xor_sync(FULLM, tmn, h));
-      if (!STAGED) { const u64 o = shfl_xor64(ck, h); ck = o > ck ? o : ck; }
-    }
-  }
-  // lowest position that holds the longest / shortest duration
-  u32 pmax = NONE, pmin = NONE;
-#pragma unroll
-  for (int q = 7; q >= 0; --q) {
-    if (FULL || p0 + q < n) { const u32 d = kd[q * KSTEP]; if (d == tmx) pmax = p0 + q; if (d == tmn) pmin = p0 + q; }
-  }
-  u32 r_tmin = 0, r_tmax = 0, r_chg = 0;                      // ranks the row names
-  if (L == 1) {                                             // all lanes are still here
-    r_tmin = __shfl_sync(FULLM, mem_l, pmin & 31u); r_tmax = __shfl_sync(FULLM, mem_l, pmax & 31u); r_chg = __shfl_sync(FULLM, mem_l, (NONE - (u32)ck) & 31u);
-  }
-  bool mismatch = mm;
-  if (L > 1) {
-#pragma unroll
-    for (int h = 1; h < L; h <<= 1) { pmax = min(pmax, __shfl_xor_sync(FULLM, pmax, h)); pmin = min(pmin, __shfl_xor_sync(FULLM, pmin, h)); }
-    if (!STAGED) mismatch = (__ballot_sync(FULLM, mm) & gmask) != 0;
-  }
-  const bool barrier = gop == CCLD_OP_ALLREDUCE && gby < P.barrier_bytes;
-  const bool analysed = gok && !barrier && n >= P.min_group;
-
-  // ---- order statistics: one metric at a time, keys read back from shared memory ----
-  u32 ms = 0, ds = 0, md = 0, dm = 0;
-  if (__any_sync(FULLM, analysed)) {
-    u32 v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = (FULL || p0 + q < n) ? ka[q * KSTEP] - emin : 0xFFFFFFFFu;
-    if (L == 1) median_mad8<u32>(v, n, &ms, &ds); else sub_median_mad<L, u32>(v, n, s, lane, &ms, &ds);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = (FULL || p0 + q < n) ? kd[q * KSTEP] - tmn : 0xFFFFFFFFu;
-    if (L == 1) median_mad8<u32>(v, n, &md, &dm); else sub_median_mad<L, u32>(v, n, s, lane, &md, &dm);
-    if (!analysed) { ms = ds = md = dm = 0; }
-  }
-  if (!gok) return;
-
-  // ---- flags, votes, per-member bandwidth ----
-  double num, den; bus_factor(gop, n, &num, &den);
-  const double bn = (double)gby * num;
-  u32 f_lo = 0, f_hi = 0;                                   // my eight flag bytes
-  {
-    // |x - med| * 1000 > k * MAD, exact: deviations and MADs are below 2^32, so both sides fit 64 bits, and for whole
-    // numbers a * 1000 > T is a > floor(T / 1000); a quotient of 2^32 - 1 or more can never be exceeded
-    const u64 qs = (u64)ds * P.k_milli / 1000u, qd = (u64)dm * P.k_milli / 1000u;
-    const u32 ts = qs > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qs, td = qd > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qd;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      if (FULL || p0 + q < n) {
-        const u32 d = kd[q * KSTEP];
-        const u32 sk = ka[q * KSTEP] - emin, dd = d - tmn;
-        const u32 f = (__usad(sk, ms, 0u) > ts ? (u32)CCLD_F_SKEW_OUT : 0u) | (__usad(dd, md, 0u) > td ? (u32)CCLD_F_DUR_OUT : 0u) |
-                      (sk > ms ? (u32)CCLD_F_SKEW_HI : 0u) | (dd > md ? (u32)CCLD_F_DUR_HI : 0u);
-        if (q < 4) f_lo |= f << (8 * q); else f_hi |= f << (8 * (q - 4));
-        if (!barrier && d != 0) bw[q] = bn * rcp_newton1((double)d * den);
-      }
-    }
-    if (!analysed) {
-      // every position that exists carries the not-analysed mark
-      const u32 cnt = FULL ? 8u : (n > p0 ? (n - p0 < 8u ? n - p0 : 8u) : 0u);
-      f_lo = 0x80808080u & (cnt >= 4 ? 0xFFFFFFFFu : (1u << (8 * cnt)) - 1u);
-      f_hi = cnt > 4 ? 0x80808080u & (cnt >= 8 ? 0xFFFFFFFFu : (1u << (8 * (cnt - 4))) - 1u) : 0u;
-    }
-    // votes: outliers are rare, so they are taken off the flag bytes afterwards, one set bit at a time
-    static_assert(CCLD_F_SKEW_OUT == 1 && CCLD_F_DUR_OUT == 2 && CCLD_F_SKEW_HI == 4 && CCLD_F_DUR_HI == 8, "flag bit layout");
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const u32 fw = half ? f_hi : f_lo;
-      u32 o = fw & 0x03030303u;
-      while (o) {
-        const u32 b = (u32)__ffs(o) - 1u, q = (b >> 3) + 4u * half, dur = b & 1u;
-        const u32 hi = (fw >> (b + 2u)) & 1u;               // the HI bit of the same metric sits two places up
-        atomicAdd(&R.votes[(u64)mem[p0 + q] * 4 + 2u * dur + (hi ? 0u : 1u)], 1u);
-        o &= o - 1u;
-      }
-    }
-    acc.flagged += (u32)__popc(f_lo & 0x01010101u) + (u32)__popc(f_hi & 0x01010101u) +
-                   (((u32)__popc(f_lo & 0x02020202u) + (u32)__popc(f_hi & 0x02020202u)) << 16);
-  }
-  {
-    u8* __restrict__ fp = ld_volatile(sh.out.flags) + row.slot0 + (u64)(seq0 + j) * n + p0;
-    if ((FULL || p0 + 8 <= n) && (reinterpret_cast<uintptr_t>(fp) & 7) == 0) *reinterpret_cast<uint2*>(fp) = make_uint2(f_lo, f_hi);
-    else {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) if (FULL || p0 + q < n) fp[q] = (u8)((q < 4 ? f_lo >> (8 * q) : f_hi >> (8 * (q - 4))) & 0xFFu);
-    }
-  }
-  if (L > 1) { r_tmin = mem[pmin]; r_tmax = mem[pmax]; r_chg = mem[NONE - (u32)ck]; }
-  if (lead) {
-    const u64 g = row.group0 + seq0 + j, G = ld_volatile(sh.out.G);
-    i64* __restrict__ gi = ld_volatile(sh.out.gi64) + g; u32* __restrict__ gu = ld_volatile(sh.out.gu32) + g;
-    const u32 span = xmax - emin;
-    gi[(u64)GI_E_MIN * G] = (i64)(base + emin); gi[(u64)GI_ARRIVAL_SKEW * G] = (i64)(u64)(emax - emin);
-    gi[(u64)GI_T_MAX * G] = (i64)(u64)tmx; gi[(u64)GI_T_MIN * G] = (i64)(u64)tmn; gi[(u64)GI_SPAN * G] = (i64)(u64)span;
-    gi[(u64)GI_MED_SKEW * G] = (i64)(u64)ms; gi[(u64)GI_MAD_SKEW * G] = (i64)(u64)ds;
-    gi[(u64)GI_MED_DUR * G] = analysed ? (i64)((u64)tmn + md) : 0; gi[(u64)GI_MAD_DUR * G] = (i64)(u64)dm;
-    gu[(u64)GU_RANK_TMIN * G] = r_tmin; gu[(u64)GU_RANK_TMAX * G] = r_tmax;
-    gu[(u64)GU_MAX_CHG * G] = (u32)(ck >> 32); gu[(u64)GU_RANK_MAX_CHG * G] = r_chg;
-    gu[(u64)GU_N_PRESENT * G] = n;
-    gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mismatch ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
-    ld_volatile(sh.out.gbw)[g] = span ? bn * rcp_newton((double)span * den) : 0.0;
-    acc.groups += (1u << FA_COMP) | (barrier ? 1u << FA_BAR : 0u) | (analysed ? 1u << FA_AN : 0u) | (mismatch ? 1u << FA_MIS : 0u) | (barrier ? 0u : 1u << FA_ROUND);
-    if (!barrier) { acc.best_rng = tmx - tmn; acc.best_k = seq0 + j; }
-  }
-}
-
-// Folds a warp's totals: counters into the CTA's shared counters, per-position bandwidth sums and the Eq. 2
-// candidate into the warp's row of `sh`.
-template <int L>
-__device__ __forceinline__ void warp_fold(FastAcc& acc, double (&bw)[8], u32 n, FusedShared& sh) {
-  constexpr int GW = 32 / L;
-  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const u32 n_comp = __reduce_add_sync(FULLM, (acc.groups >> FA_COMP) & 63u), n_bar = __reduce_add_sync(FULLM, (acc.groups >> FA_BAR) & 63u),
-            n_an = __reduce_add_sync(FULLM, (acc.groups >> FA_AN) & 63u), n_mis = __reduce_add_sync(FULLM, (acc.groups >> FA_MIS) & 63u),
-            n_round = __reduce_add_sync(FULLM, acc.groups >> FA_ROUND), n_fs = __reduce_add_sync(FULLM, acc.flagged & 0xFFFFu),
-            n_fd = __reduce_add_sync(FULLM, acc.flagged >> 16), n_def = __reduce_add_sync(FULLM, acc.n_def);
-  u32 rng = acc.best_rng, bk = acc.best_k;
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    const u32 o_rng = __shfl_xor_sync(FULLM, rng, d), o_k = __shfl_xor_sync(FULLM, bk, d);
-    if (o_k != NONE && (bk == NONE || o_rng > rng || (o_rng == rng && o_k < bk))) { rng = o_rng; bk = o_k; }
-  }
-  if (L == 1) {
-    const double tot = warp_sum8(bw, lane);                  // lane l holds member 4 bit4(l) + 2 bit3(l) + bit2(l)
-    if ((lane & 3) == 0) sh.bw[wid][lane >> 2] = tot;
-  } else {
-    // sums over the warp's groups: each round halves the values a lane carries
-    const u32 p0 = (lane % L) * 8;
-    u32 off = 0;
-#pragma unroll
-    for (int bit = 16, w = 4; bit >= L; bit >>= 1, w >>= 1) {
-      const bool hi = (lane & bit) != 0;
-#pragma unroll
-      for (int i = 0; i < w; ++i) {
-        const double send = hi ? bw[i] : bw[i + w], keep = hi ? bw[i + w] : bw[i];
-        bw[i] = keep + __shfl_xor_sync(FULLM, send, bit);
-      }
-      off += hi ? (u32)w : 0u;
-    }
-#pragma unroll
-    for (int i = 0; i < 8 / GW; ++i) sh.bw[wid][p0 + off + i] = bw[i];
-  }
-  if (lane == 0) {
-    sh.rounds[wid] = n_round; sh.n_an[wid] = n_an; sh.n_def[wid] = n_def; sh.brng[wid] = rng; sh.bk[wid] = bk;
-    if (n_comp) { atomicAdd(&sh.cnt[SC_COMP], n_comp); atomicAdd(&sh.cnt[SC_PRES], n_comp * n); }
-    if (n_bar) atomicAdd(&sh.cnt[SC_BAR], n_bar);
-    if (n_an) atomicAdd(&sh.cnt[SC_AN], n_an);
-    if (n_mis) atomicAdd(&sh.cnt[SC_MIS], n_mis);
-    if (n_fs) atomicAdd(&sh.cnt[SC_FS], n_fs);
-    if (n_fd) atomicAdd(&sh.cnt[SC_FD], n_fd);
-  }
-}
 
 __device__ __forceinline__ void flush_counters(const WinDesc& D, const FusedShared& sh) {
   count_add(D.counters, C_COMPLETE, sh.cnt[SC_COMP]); count_add(D.counters, C_BARRIER, sh.cnt[SC_BAR]); count_add(D.counters, C_ANALYSED, sh.cnt[SC_AN]);
@@ -816,44 +475,213 @@ __device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta
   if (threadIdx.x == 0) flush_counters(D, sh);
 }
 
-// Class-1 CTA (9 <= n <= 128): one tile of 2048 / n_pad consecutive op counters of one communicator, 32 / L per warp;
-// one summary entry.
-template <int L>
+// Class-1 CTA (9 <= n <= 128, L = n_pad / 8): one tile of S = 256 / L consecutive op counters of one communicator, eight
+// records per thread. A thread gathers op counter t % S of members t / S, t / S + L, ... - lanes along the op counter, so the
+// record indices of a warp are contiguous and, in a rank-major upload, its records lie in one short stretch of a rank's
+// stream - with one exposed round trip for times, sizes and op codes; the rate columns are on their way while the groups
+// are sorted. Keys meet in shared memory; then L lanes take a group, eight members each (position q L + s in lane s: with
+// the pitch below every access of a column is free of bank conflicts). Last, a thread sums eight op counters of one member's
+// bandwidth.
+template <int L, bool FULL>
 __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& t, TileSum* __restrict__ sums, const Registry& R, const Params& P,
                                               const DeferList& DL, FusedShared& sh) {
-  constexpr u32 GW = 32 / L, NW = SMALL_SEQS / 32;
-  const u32 wid = threadIdx.x >> 5, n = t.row.n;
-  const u32 first = wid * GW;
-  const u32 cnt = first < t.count ? (t.count - first < GW ? t.count - first : GW) : 0u;
-  FastAcc acc; double bw[8];
-  if (L >= 8) {
-    // the tile's records are gathered with lanes along the op counter and wait in shared memory as 32-bit keys
-    if (threadIdx.x < 32) sh.t_bits[threadIdx.x] = 0;
-    __syncthreads();
-    stage_tile<L>(D, t.row, t.seq_off, t.count, sh);
-    __syncthreads();
-    if (n == (u32)(L * 8)) fast_groups<L, true, true>(D, t.w, t.row, R.members + t.moff, t.seq_off + first, cnt, R, P, DL, sh, acc, bw, first);
-    else fast_groups<L, false, true>(D, t.w, t.row, R.members + t.moff, t.seq_off + first, cnt, R, P, DL, sh, acc, bw, first);
-  } else if (n == (u32)(L * 8)) fast_groups<L, true>(D, t.w, t.row, R.members + t.moff, t.seq_off + first, cnt, R, P, DL, sh, acc, bw);
-  else fast_groups<L, false>(D, t.w, t.row, R.members + t.moff, t.seq_off + first, cnt, R, P, DL, sh, acc, bw);
-  warp_fold<L>(acc, bw, n, sh);
+  constexpr u32 S = SMALL_SEQS / L, GW = 32 / L, NW = SMALL_SEQS / 32;
+  constexpr u32 PITCH = L == 4 ? 72 : (L == 8 ? 36 : 18);    // lane (s, j) of an access to a column: bank s PITCH + j, 32 different ones
+  static_assert(8 * L * PITCH <= TILE_KEYS && S <= TILE_OPS, "tile fits");
+  const u32 wid = threadIdx.x >> 5, lane = threadIdx.x & 31, n = FULL ? (u32)(8 * L) : t.row.n, count = t.count;
+  u32* __restrict__ k_a = sh.stage; u32* __restrict__ k_d = sh.stage + TILE_KEYS;
+  if (threadIdx.x < S) { sh.t_bits[threadIdx.x] = 0; sh.t_xmax[threadIdx.x] = 0; }
+  if (threadIdx.x < n) sh.mem[threadIdx.x] = __ldg(R.members + t.moff + threadIdx.x);
+  __syncthreads();                                            // counters and pointers are set, the arrays above clear
+  // ---- gather ----
+  const u32 sq = threadIdx.x % S, mr = threadIdx.x / S;
+  u32 sc[8], rc[8];
+  {
+    const u32* __restrict__ pm = ld_volatile(sh.in.perm) + t.row.slot0 + t.seq_off + (sq < count ? sq : 0u);
+    u32 idx[8], top = 0;
+    const u32 i0 = __ldg(pm);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { const u32 p = mr + (u32)q * L; idx[q] = __ldg(pm + (u64)(FULL || p < n ? p : mr) * t.row.n_seq); top = max(top, idx[q]); }
+    u32 bits = top == NONE || i0 == NONE ? 1u : 0u;           // a missing member: the group is set aside
+#pragma unroll
+    for (int q = 0; q < 8; ++q) idx[q] = idx[q] == NONE ? 0u : idx[q];
+    const i64* __restrict__ c_te = ld_volatile(sh.in.te); const i64* __restrict__ c_tx = ld_volatile(sh.in.tx);
+    const u64* __restrict__ c_by = ld_volatile(sh.in.by); const u8* __restrict__ c_op = ld_volatile(sh.in.op);
+    i64 ta[8], tb[8]; u64 by[8]; u32 op[8];
+    const u32 j0 = i0 == NONE ? 0u : i0;
+    const i64 te0 = __ldg(c_te + j0); const u64 by0 = __ldg(c_by + j0); const u32 op0 = __ldg(c_op + j0);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { ta[q] = __ldg(c_te + idx[q]); tb[q] = __ldg(c_tx + idx[q]); }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { by[q] = __ldg(c_by + idx[q]); op[q] = __ldg(c_op + idx[q]); }
+    const u64 base = (u64)te0 - 0x80000000ull;
+    u32 hx = 0, neg = 0, xmax = 0; bool back = false;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const u32 p = mr + (u32)q * L;
+      const u64 ra = (u64)ta[q] - base, rb = (u64)tb[q] - base;
+      const u32 a = (u32)ra, b = (u32)rb;
+      hx |= (u32)(ra >> 32) | (u32)(rb >> 32);
+      neg |= (u32)((u64)ta[q] >> 32) | (u32)((u64)tb[q] >> 32);
+      back = back || b < a; xmax = max(xmax, b);
+      k_a[p * PITCH + sq] = FULL || p < n ? a : 0xFFFFFFFFu; k_d[p * PITCH + sq] = FULL || p < n ? b - a : 0xFFFFFFFFu;
+    }
+    if (hx != 0 || (int)neg < 0 || back) bits |= 1;           // beyond 32 bits, negative or in flight, exit before enter
+    u32 y = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) y |= ((u32)by[q] ^ (u32)by0) | ((u32)(by[q] >> 32) ^ (u32)(by0 >> 32)) | (op[q] ^ op0);
+    if (y) bits |= 2;
+    if (bits) atomicOr(&sh.t_bits[sq], bits);
+    atomicMax(&sh.t_xmax[sq], xmax);
+    if (mr == 0) { sh.t_base[sq] = base; sh.t_gby[sq] = by0; sh.t_gop[sq] = op0; }
+    const u32* __restrict__ c_sc = ld_volatile(sh.in.sc); const u32* __restrict__ c_rc = ld_volatile(sh.in.rc);
+    if (c_sc != nullptr) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) { sc[q] = __ldg(c_sc + idx[q]); rc[q] = __ldg(c_rc + idx[q]); }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) sc[q] = rc[q] = 0;
+    }
+  }
+  __syncthreads();
+  // ---- a group in L lanes ----
+  {
+    const u32 s = lane % L, jt = wid * GW + lane / L;         // my group's op counter inside the tile
+    const bool lead = s == 0, active = jt < count;
+    const u32 bits = sh.t_bits[jt], gop = sh.t_gop[jt]; const u64 gby = sh.t_gby[jt];
+    const bool gok = active && !(bits & 1), mm = (bits & 2) != 0;
+    const bool barrier = gop == CCLD_OP_ALLREDUCE && gby < P.barrier_bytes;
+    const bool round = gok && !barrier, analysed = round && n >= P.min_group;
+    const u32* __restrict__ ka = k_a + s * PITCH + jt; const u32* __restrict__ kd = k_d + s * PITCH + jt;     // member q L + s: q * L * PITCH further
+    u32 emin, emax, ms, ds, tmn, tmx, md, dm;
+    {
+      u32 v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = ka[q * L * PITCH];
+      sub_stats<L, FULL>(v, n, s, lane, &emin, &emax, &ms, &ds);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = kd[q * L * PITCH];
+      sub_stats<L, FULL>(v, n, s, lane, &tmn, &tmx, &md, &dm);
+    }
+    ms -= emin; md -= tmn;
+    if (!analysed) { ms = ds = md = dm = 0; }
+    // lowest position that holds the longest / shortest duration; flags, votes
+    u32 pmax = NONE, pmin = NONE, n_fs = 0, n_fd = 0;
+    {
+      const u64 qs = (u64)ds * P.k_milli / 1000u, qd = (u64)dm * P.k_milli / 1000u;     // outside [med - T, med + T], T = floor(k * MAD / 1000)
+      const u32 ts = qs > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qs, td = qd > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qd;
+      const u32 los = ms > ts ? ms - ts : 0u, lod = md > td ? md - td : 0u;
+      const u32 ws = (ms + ts < ms ? 0xFFFFFFFFu : ms + ts) - los, wd = (md + td < md ? 0xFFFFFFFFu : md + td) - lod;
+      const u32 s0 = emin + los, d0 = tmn + lod, sm = emin + ms, dmd = tmn + md;
+      u8* __restrict__ fp = ld_volatile(sh.out.flags) + t.row.slot0 + (u64)(t.seq_off + (active ? jt : 0u)) * n + s;
+      u32 out = 0;                                            // outlier bits of my eight members, four apiece
+#pragma unroll
+      for (int q = 7; q >= 0; --q) {
+        if (!FULL && q * L + s >= n) continue;
+        const u32 a = ka[q * L * PITCH], d = kd[q * L * PITCH];
+        u32 f = a - s0 > ws ? (u32)CCLD_F_SKEW_OUT : 0u;
+        if (d - d0 > wd) f |= CCLD_F_DUR_OUT;
+        if (a > sm) f |= CCLD_F_SKEW_HI;
+        if (d > dmd) f |= CCLD_F_DUR_HI;
+        if (d == tmx) pmax = q * L + s;
+        if (d == tmn) pmin = q * L + s;
+        out |= f << (4 * q);
+        if (gok) fp[q * L] = analysed ? (u8)f : (u8)CCLD_F_NOT_ANALYSED;
+      }
+      // votes: outliers are rare, so they are taken off the flag bits one at a time
+      if (analysed) {
+        n_fs = (u32)__popc(out & 0x11111111u); n_fd = (u32)__popc(out & 0x22222222u);
+        for (u32 o = out & 0x33333333u; o; o &= o - 1u) {
+          const u32 b = (u32)__ffs(o) - 1u, dur = b & 1u, hi = (out >> (b + 2u)) & 1u;
+          atomicAdd(&R.votes[(u64)sh.mem[(b >> 2) * L + s] * 4 + 2u * dur + (hi ? 0u : 1u)], 1u);
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 1; h < L; h <<= 1) { pmax = min(pmax, __shfl_xor_sync(FULLM, pmax, h)); pmin = min(pmin, __shfl_xor_sync(FULLM, pmin, h)); }
+    double num, den; bus_factor(gop, n, &num, &den);
+    const double bd = (double)gby * (num / den);
+    if (lead && active) {
+      sh.t_bd[jt] = round ? bd : 0.0;
+      if (gok) {
+        const u64 g = t.row.group0 + t.seq_off + jt, G = ld_volatile(sh.out.G);
+        i64* __restrict__ gi = ld_volatile(sh.out.gi64) + g; u32* __restrict__ gu = ld_volatile(sh.out.gu32) + g;
+        const u32 span = sh.t_xmax[jt] - emin;
+        gi[(u64)GI_E_MIN * G] = (i64)(sh.t_base[jt] + emin); gi[(u64)GI_ARRIVAL_SKEW * G] = (i64)(u64)(emax - emin);
+        gi[(u64)GI_T_MAX * G] = (i64)(u64)tmx; gi[(u64)GI_T_MIN * G] = (i64)(u64)tmn; gi[(u64)GI_SPAN * G] = (i64)(u64)span;
+        gi[(u64)GI_MED_SKEW * G] = (i64)(u64)ms; gi[(u64)GI_MAD_SKEW * G] = (i64)(u64)ds;
+        gi[(u64)GI_MED_DUR * G] = analysed ? (i64)((u64)tmn + md) : 0; gi[(u64)GI_MAD_DUR * G] = (i64)(u64)dm;
+        gu[(u64)GU_RANK_TMIN * G] = sh.mem[pmin]; gu[(u64)GU_RANK_TMAX * G] = sh.mem[pmax];
+        gu[(u64)GU_N_PRESENT * G] = n;
+        gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mm ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
+        ld_volatile(sh.out.gbw)[g] = span ? bd * rcp_newton((double)span) : 0.0;
+      } else {
+        const u32 e = atomicAdd(DL.count, 1u);
+        DL.entries[e] = ((u64)t.w << 32) | (u64)(t.row.group0 + t.seq_off + jt);
+      }
+    }
+    // the warp's counts and Eq. 2 candidate (ties: the lowest op counter)
+    const u32 rng = round ? tmx - tmn : 0u, best = __reduce_max_sync(FULLM, rng);
+    const u32 b_best = __ballot_sync(FULLM, round && rng == best), b_ok = __ballot_sync(FULLM, gok && lead), b_round = __ballot_sync(FULLM, round && lead),
+              b_an = __ballot_sync(FULLM, analysed && lead), b_mm = __ballot_sync(FULLM, gok && mm && lead), b_act = __ballot_sync(FULLM, active && lead);
+    n_fs = __reduce_add_sync(FULLM, n_fs); n_fd = __reduce_add_sync(FULLM, n_fd);
+    if (lane == 0) {
+      const u32 n_ok = (u32)__popc(b_ok), n_round = (u32)__popc(b_round);
+      sh.brng[wid] = best; sh.bk[wid] = b_best ? t.seq_off + wid * GW + ((u32)__ffs(b_best) - 1u) / L : NONE;
+      sh.rounds[wid] = n_round; sh.n_an[wid] = (u32)__popc(b_an); sh.n_def[wid] = (u32)__popc(b_act) - n_ok;
+      if (n_ok) { atomicAdd(&sh.cnt[SC_COMP], n_ok); atomicAdd(&sh.cnt[SC_PRES], n_ok * n); }
+      if (n_ok != n_round) atomicAdd(&sh.cnt[SC_BAR], n_ok - n_round);
+      if (b_an) atomicAdd(&sh.cnt[SC_AN], (u32)__popc(b_an));
+      if (b_mm) atomicAdd(&sh.cnt[SC_MIS], (u32)__popc(b_mm));
+      if (n_fs) atomicAdd(&sh.cnt[SC_FS], n_fs);
+      if (n_fd) atomicAdd(&sh.cnt[SC_FD], n_fd);
+    }
+  }
+  // ---- most changes, then the lowest position: my members, the lanes that share my op counter, later the warps ----
+  {
+    u64 ck = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const u32 p = mr + (u32)q * L;
+      const u64 k = ((u64)max(sc[q], rc[q]) << 32) | (u64)(NONE - p);
+      if (FULL || p < n) ck = k > ck ? k : ck;
+    }
+#pragma unroll
+    for (u32 h = S; h < 32; h <<= 1) { const u64 o = shfl_xor64(ck, h); ck = o > ck ? o : ck; }
+    sh.t_ck[wid][lane] = ck;
+  }
   __syncthreads();
   u32 rounds = 0;
 #pragma unroll
   for (u32 q = 0; q < NW; ++q) rounds += sh.rounds[q];
-  if (rounds) {
-    const u32* mem = R.members + t.moff;
-    for (u32 p = threadIdx.x; p < n; p += SMALL_SEQS) {
-      double v = 0.0;
+  if (threadIdx.x < count && !(sh.t_bits[threadIdx.x] & 1)) {
+    u64 ck = 0;
+    constexpr u32 W0 = S / 32 ? S / 32 : 1;                   // warps that cover all op counters once
 #pragma unroll
-      for (u32 q = 0; q < NW; ++q) v += sh.bw[q][p];
-      atomicAdd(&R.bw_sum[mem[p]], v);
-      atomicAdd(&R.bw_cnt[mem[p]], rounds);
+    for (u32 w = 0; w < NW; w += W0) { const u64 o = sh.t_ck[w + threadIdx.x / 32 % W0][threadIdx.x & 31]; ck = o > ck ? o : ck; }
+    const u64 g = t.row.group0 + t.seq_off + threadIdx.x, G = ld_volatile(sh.out.G);
+    u32* __restrict__ gu = ld_volatile(sh.out.gu32) + g;
+    gu[(u64)GU_MAX_CHG * G] = (u32)(ck >> 32); gu[(u64)GU_RANK_MAX_CHG * G] = sh.mem[NONE - (u32)ck];
+  }
+  if (rounds) {
+    constexpr u32 TPM = GW;                                   // threads per member, eight op counters each
+    const u32 p = threadIdx.x / TPM, part = threadIdx.x % TPM;
+    double v = 0.0;
+    if (FULL || p < n) {
+#pragma unroll
+      for (u32 i = 0; i < 8; ++i) {
+        const u32 o = part + TPM * i, d = k_d[p * PITCH + o];
+        const double bd = o < count ? sh.t_bd[o] : 0.0;
+        if (bd != 0.0 && d != 0) v += bd * rcp_u32(d);
+      }
     }
+#pragma unroll
+    for (u32 h = 1; h < TPM; h <<= 1) v += __shfl_xor_sync(FULLM, v, h);
+    if (part == 0 && (FULL || p < n)) { atomicAdd(&R.bw_sum[sh.mem[p]], v); atomicAdd(&R.bw_cnt[sh.mem[p]], rounds); }
   }
   if (threadIdx.x == 0) {
-    u64 brng = sh.brng[0]; u32 bk = sh.bk[0], n_an = sh.n_an[0], n_def = sh.n_def[0];
-    for (u32 q = 1; q < NW; ++q) { best_merge(brng, bk, sh.brng[q], sh.bk[q]); n_an += sh.n_an[q]; n_def += sh.n_def[q]; }
+    u64 brng = 0; u32 bk = NONE, n_an = 0, n_def = 0;
+    for (u32 q = 0; q < NW; ++q) { best_merge(brng, bk, sh.brng[q], sh.bk[q]); n_an += sh.n_an[q]; n_def += sh.n_def[q]; }
     TileSum ts; ts.best_rng = brng; ts.best_k = bk; ts.n_rounds = rounds; ts.n_an = n_an; ts.pad = n_def;
     sums[t.sum_idx] = ts;
     flush_counters(D, sh);
@@ -869,11 +697,10 @@ __global__ void __launch_bounds__(SMALL_SEQS, CCLD_FUSED_MIN_CTAS) k_reduce_fuse
   if (threadIdx.x == 0) { sh.out.flags = D.flags; sh.out.gi64 = D.gi64; sh.out.gu32 = D.gu32; sh.out.gbw = D.gbw; sh.out.G = D.n_groups; }
   if (threadIdx.x == 32) { sh.in.perm = D.perm; sh.in.te = D.t_enter; sh.in.tx = D.t_exit; sh.in.by = D.bytes; sh.in.op = D.op; sh.in.sc = D.send_chg; sh.in.rc = D.recv_chg; }
   if (t.cls == 0) { fused_small_cta(D, t, wts, sums, R, P, DL, sh); return; }
-  __syncthreads();
-  const u32 n_pad = mid_npad(t.row.n);
-  if (n_pad == 32) fused_sub_cta<4>(D, t, sums, R, P, DL, sh);
-  else if (n_pad == 64) fused_sub_cta<8>(D, t, sums, R, P, DL, sh);
-  else fused_sub_cta<16>(D, t, sums, R, P, DL, sh);
+  const u32 n = t.row.n;
+  if (n <= 32) { if (n == 32) fused_sub_cta<4, true>(D, t, sums, R, P, DL, sh); else fused_sub_cta<4, false>(D, t, sums, R, P, DL, sh); }
+  else if (n <= 64) { if (n == 64) fused_sub_cta<8, true>(D, t, sums, R, P, DL, sh); else fused_sub_cta<8, false>(D, t, sums, R, P, DL, sh); }
+  else { if (n == 128) fused_sub_cta<16, true>(D, t, sums, R, P, DL, sh); else fused_sub_cta<16, false>(D, t, sums, R, P, DL, sh); }
 }
 
 // ------------------------------------------------------------------------------------------------

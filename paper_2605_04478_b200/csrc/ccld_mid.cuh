@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(cons
 #pragma unroll
       for (u32 g = 0; g < MID_SEQS; ++g) {
         const u32 d = k_d[p * MID_PITCH + g];
-        if ((s_state[g] & 1) && d != 0) v += s_bn[g] * rcp_newton1((double)d * s_den[g]);
+        if ((s_state[g] & 1) && d != 0) v += s_bn[g] * rcp_newton((double)d * s_den[g]);
       }
       atomicAdd(&Reg.bw_sum[mem[p]], v); atomicAdd(&Reg.bw_cnt[mem[p]], rounds);
     }
