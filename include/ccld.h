@@ -247,6 +247,21 @@ typedef struct {
 int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out /* host */);
 
 /*
+ * The same verdict with its lists column by column, for callers that keep them that way (array libraries): nothing is copied,
+ * the pointers lead into host memory of the context and are valid until its next call. A list of n entries starts with its
+ * 64-bit fields, then come its 32-bit fields, both in the order of the struct, each column n entries long:
+ *   rows      slow_count, rounds_total, m, t_max, t_min, t_base, R, P, then comm .. root_comm
+ *   alerts    age_ns, then comm, seq (at most CCLD_MAX_ALERTS_PER_WINDOW)
+ *   suspects  mean_busbw, then kind, rank, votes, ops
+ * The pointers and capacities in *out are not used.
+ */
+typedef struct {
+  const void *rows, *alerts, *suspects;
+  uint32_t n_rows, n_alerts, n_suspects, pad;
+} ccld_verdict_columns;
+int ccld_get_verdict_columns(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out /* host */, ccld_verdict_columns* columns /* host */);
+
+/*
  * Hang location (Sec. 4.2.2, Fig. 6) for op (comm, seq) as seen in window `window_id`:
  *   H1 (cls 1): members with no record of an op counter >= seq - they never entered; roots = those.
  *   H2 (cls 2): all entered, some members' record of `seq` is complete - roots = those non-hung ranks.

@@ -26,7 +26,7 @@ EXPORTS = ("ccld_params_default", "ccld_create", "ccld_destroy", "ccld_last_erro
            "ccld_trace_upload", "ccld_window_release", "ccld_analyze_window", "ccld_reset", "ccld_get_verdict",
            "ccld_locate_hang", "ccld_get_optable", "ccld_get_ranges", "ccld_get_rank_stats", "ccld_copy_to_host",
            "ccld_timing_enable", "ccld_get_kernel_times", "ccld_set_speculation", "ccld_ring_locate_static", "ccld_derive_rates", "ccld_locate_hangs", "ccld_state_export", "ccld_state_import", "ccld_trace_attach_opset", "ccld_opset_check",
-           "ccld_comm_set_layers", "ccld_copy_many_to_host")
+           "ccld_comm_set_layers", "ccld_copy_many_to_host", "ccld_get_verdict_columns")
 STATIC_MAX_MEMBERS = 8192
 KERNEL_KINDS = ("k_seq_range", "k_plan", "k_slot_scatter", "k_reduce_fused", "k_reduce_mid", "k_reduce_large", "k_window_decide")
 
@@ -69,6 +69,10 @@ class Verdict(C.Structure):
                 ("suspects", C.POINTER(Suspect)), ("suspects_cap", C.c_uint32)]
 
 
+class VerdictColumns(C.Structure):
+    _fields_ = [(k, C.c_void_p) for k in ("rows", "alerts", "suspects")] + [(k, C.c_uint32) for k in ("n_rows", "n_alerts", "n_suspects", "pad")]
+
+
 class HangVerdict(C.Structure):
     _fields_ = [(k, C.c_uint32) for k in ("cls", "n_roots_total", "n_not_entered", "n_hung", "n_not_hung",
                                            "n_missing_frames", "stuck_step", "n_members")] + \
@@ -98,6 +102,18 @@ class CommRange(C.Structure):
 
 
 _NP_OF = {C.c_uint32: "u4", C.c_uint64: "u8", C.c_int64: "i8", C.c_double: "f8"}
+
+
+def _column_plan(struct):
+    """(name, dtype, bytes of an entry that lie before the column) per field, in field order; 64-bit columns come first."""
+    size = {k: np.dtype(_NP_OF[t]).itemsize for k, t in struct._fields_}
+    order = [k for k, _ in struct._fields_ if size[k] == 8] + [k for k, _ in struct._fields_ if size[k] == 4]
+    at = {k: sum(size[x] for x in order[:i]) for i, k in enumerate(order)}
+    return [(k, np.dtype(_NP_OF[t]), at[k]) for k, t in struct._fields_], sum(size.values())
+
+
+_ROW_PLAN, _ALERT_PLAN, _SUSPECT_PLAN = _column_plan(CommVerdict), _column_plan(HangAlert), _column_plan(Suspect)
+_VERDICT_KEYS = tuple(k for k, _ in Verdict._fields_[:15])
 _lib = None
 
 
@@ -136,6 +152,7 @@ def load_library() -> C.CDLL:
         lib.ccld_get_ranges.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_uint32, C.POINTER(C.c_uint32)]
         lib.ccld_get_rank_stats.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_copy_to_host.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_uint64]
+        lib.ccld_get_verdict_columns.argtypes = [C.c_void_p, C.c_uint32, C.POINTER(Verdict), C.POINTER(VerdictColumns)]
         lib.ccld_copy_many_to_host.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_derive_rates.argtypes = [C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p, C.c_uint32, C.c_uint64] + [C.c_void_p] * 6
         lib.ccld_timing_enable.argtypes = [C.c_void_p, C.c_int]
@@ -312,9 +329,21 @@ class Analyzer:
         a = a[:count]
         return {k: a[k].copy() for k in a.dtype.names}
 
+    @staticmethod
+    def _take(ptr, n, cap, plan):
+        """A list of n entries that the library holds column by column, as one array per field (the first `cap` entries)."""
+        fields, size = plan
+        if n == 0:
+            return {k: np.empty(0, dt) for k, dt, _ in fields}
+        buf = np.empty(n * size, np.uint8)
+        C.memmove(buf.ctypes.data, ptr, n * size)
+        if cap < n:
+            return {k: np.frombuffer(buf, dt, n, at * n)[:cap] for k, dt, at in fields}
+        return {k: np.frombuffer(buf, dt, n, at * n) for k, dt, at in fields}
+
     def _list_buf(self, struct, cap):
         """Room for `cap` entries of a C struct. Kept between calls: the library writes only the entries there are, and a fresh
-        buffer of a default capacity (7 MB of rows) would be zeroed and faulted in on every call."""
+        buffer of a default capacity would be zeroed and faulted in on every call."""
         b = self._bufs.get(struct)
         if b is None or len(b) < cap:
             b = self._bufs[struct] = np.empty(max(cap, 1), np.dtype([(k, _NP_OF[t]) for k, t in struct._fields_]))
@@ -322,19 +351,15 @@ class Analyzer:
 
     def get_verdict(self, window_id: int, comm_rows_cap: int = 1 << 16, alerts_cap: int = MAX_ALERTS_PER_WINDOW,
                     suspects_cap: int = 1 << 16, check: bool = True) -> Dict[str, object]:
-        rows, alerts, sus = self._list_buf(CommVerdict, comm_rows_cap), self._list_buf(HangAlert, alerts_cap), self._list_buf(Suspect, suspects_cap)
-        v = Verdict()
-        v.comm_rows = C.cast(rows.ctypes.data, C.POINTER(CommVerdict)); v.comm_rows_cap = comm_rows_cap
-        v.alerts = C.cast(alerts.ctypes.data, C.POINTER(HangAlert)); v.alerts_cap = alerts_cap
-        v.suspects = C.cast(sus.ctypes.data, C.POINTER(Suspect)); v.suspects_cap = suspects_cap
-        rc = self.lib.ccld_get_verdict(self.h, window_id, C.byref(v))
+        v, c = Verdict(), VerdictColumns()
+        rc = self.lib.ccld_get_verdict_columns(self.h, window_id, C.byref(v), C.byref(c))
         if check:
             self._check(rc)
-        out: Dict[str, object] = {k: int(getattr(v, k)) for k, _ in Verdict._fields_[:15]}
+        out: Dict[str, object] = {k: getattr(v, k) for k in _VERDICT_KEYS}
         out["rc"] = rc
-        out["comm_rows"] = self._columns(rows, min(v.n_comm_rows_total, comm_rows_cap))
-        out["alerts"] = self._columns(alerts, min(v.n_alerts_total, alerts_cap, MAX_ALERTS_PER_WINDOW))
-        out["suspects"] = self._columns(sus, min(v.n_suspects_total, suspects_cap))
+        out["comm_rows"] = self._take(c.rows, c.n_rows, comm_rows_cap, _ROW_PLAN)
+        out["alerts"] = self._take(c.alerts, c.n_alerts, alerts_cap, _ALERT_PLAN)
+        out["suspects"] = self._take(c.suspects, c.n_suspects, suspects_cap, _SUSPECT_PLAN)
         return out
 
     def locate_hang(self, window_id: int, comm: int, seq: int, roots_cap: int = MAX_COMM_SIZE) -> Dict[str, object]:

@@ -150,6 +150,7 @@ struct ccld_ctx {
   Pool pool; std::string err;
   Block h_verdict;                                       // pinned area of ccld_get_verdict (VerdictArea)
   Block h_io;                                            // pinned area small results pass through
+  std::vector<char> long_suspects;                       // columns of a suspect list that outgrew the pinned area
   Block h_up; UploadSlot up[UP_SLOTS]; u32 up_next = 0;
   u64 batches_redone = 0;                                // batches settle() had to analyse again
   std::vector<PendingBatch> pending; std::vector<Block> pinned_free; std::vector<ShapeEntry> shapes;
@@ -850,9 +851,10 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   PlanLists pl; pl.fcta = (FusedCta*)(rbase + o_fcta); pl.fwt = (WarpTile*)(rbase + o_fwt); pl.t2 = (Tile*)(rbase + o_t2); pl.t3 = (Tile*)(rbase + o_t3);
   pl.grp_words = (u32*)(rbase + o_lgrp); pl.grp_words_per_tile = LARGE_SEQS * sizeof(LargeGroup) / 4;
   {
-    const u32 rank_ctas = std::min<u32>((2 * ctx->n_ranks + EMIT_THREADS - 1) / EMIT_THREADS, 2 * ctx->n_sms);
+    const u32 rank_ctas = std::min<u32>((2 * ctx->n_ranks + EMIT_THREADS - 1) / EMIT_THREADS, 2 * ctx->n_sms), comm_blocks = (nc + EMIT_THREADS - 1) / EMIT_THREADS,
+              per_slice = (comm_blocks + EMIT_SLICES - 1) / EMIT_SLICES, slices = (comm_blocks + per_slice - 1) / per_slice;
     TimedLaunch tl(ts, 1, st);
-    k_emit<<<dim3(chunk_ctas + rank_ctas, B), EMIT_THREADS, 0, st>>>(d_desc, ctx->reg, pl, chunk_ctas);
+    k_emit<<<dim3(chunk_ctas * slices + rank_ctas, B), EMIT_THREADS, 0, st>>>(d_desc, ctx->reg, pl, chunk_ctas * slices, slices, per_slice);
   }
   if (cta > 0) {
     const u64 blocks = (cta * REC_PER_CTA + SCAT_PER_CTA - 1) / SCAT_PER_CTA;      // of the largest window
@@ -925,9 +927,8 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
 
 extern "C" {
 
-int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
-  NvtxRange nvtx_range("ccld_get_verdict");
-  if (!ctx || !out) return CCLD_ERR_ARG;
+// Fills out's counts and, unless `columns` is given, its lists; with `columns` the lists stay in pinned memory, column by column.
+static int verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out, ccld_verdict_columns* columns) {
   WindowHost* w = nullptr;
   CK(cudaSetDevice(ctx->device));
   // The kernels that gather the verdict are enqueued before batches still in doubt are settled: one wait serves both. In
@@ -945,9 +946,9 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
     { int rc = pinned_area(ctx, ctx->h_verdict, area.total); if (rc != CCLD_OK) return rc; }
     hv = (char*)ctx->h_verdict.p;
     head = (const VerdictHead*)hv;
-    n_rows = std::min<u32>((u32)w->totals[T_ROWS], out->comm_rows ? out->comm_rows_cap : 0);
+    n_rows = columns ? (u32)w->totals[T_ROWS] : std::min<u32>((u32)w->totals[T_ROWS], out->comm_rows ? out->comm_rows_cap : 0);
     VerdictArgs A;
-    A.counters = w->d.counters; A.rows = w->d.comm_rows; A.n_rows = n_rows; A.alerts = w->d.alerts;
+    A.counters = w->d.counters; A.rows = w->d.comm_rows; A.n_rows = n_rows; A.alerts = w->d.alerts; A.columns = columns != nullptr;
     A.keys = (u64*)(m + L.keys); A.counts = (u32*)(m + L.counts);
     A.head = (VerdictHead*)hv; A.rows_out = (ccld_comm_verdict*)(hv + area.rows);
     A.alerts_out = (ccld_hang_alert*)(hv + area.alerts);
@@ -971,14 +972,27 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
   if (!w->totals[T_FAILED] && w->n_rec - cnt[C_PRESENT] != cnt[C_REJECTED]) err |= CCLD_E_DUPLICATE;   // a slot was written twice
   out->error_bits = err;
   out->n_comm_rows_total = (u32)w->totals[T_ROWS];
-  if (n_rows) std::memcpy(out->comm_rows, hv + area.rows, n_rows * sizeof(ccld_comm_verdict));
+  if (columns) {
+    const u32 n_al = (u32)std::min<u64>(cnt[C_ALERTS], CCLD_MAX_ALERTS_PER_WINDOW), n_sus = head->n_suspects;
+    columns->n_rows = n_rows; columns->n_alerts = n_al; columns->n_suspects = n_sus;
+    columns->rows = hv + area.rows; columns->alerts = hv + area.alerts; columns->suspects = hv + area.suspects;
+    if (n_sus > area.sus_cap) {                                 // a list this long was left in device memory, as structs
+      std::vector<ccld_suspect> list(n_sus);
+      { const Piece pc{m + L.sus, list.data(), n_sus * sizeof(ccld_suspect)}; int rc = fetch(ctx, &pc, 1); if (rc != CCLD_OK) return rc; }
+      ctx->long_suspects.resize((size_t)n_sus * sizeof(ccld_suspect));
+      double* d = (double*)ctx->long_suspects.data(); u32* u = (u32*)(d + n_sus);
+      for (size_t i = 0; i < n_sus; ++i) { d[i] = list[i].mean_busbw; u[i] = list[i].kind; u[n_sus + i] = list[i].rank; u[2ull * n_sus + i] = list[i].votes; u[3ull * n_sus + i] = list[i].ops; }
+      columns->suspects = ctx->long_suspects.data();
+    }
+  }
+  if (!columns && n_rows) std::memcpy(out->comm_rows, hv + area.rows, n_rows * sizeof(ccld_comm_verdict));
   // hang alerts, ordered by (communicator, seq)
   out->n_alerts_total = (u32)std::min<u64>(cnt[C_ALERTS], 0xFFFFFFFFull);
-  const u32 n_al = std::min<u32>(std::min<u32>(out->n_alerts_total, CCLD_MAX_ALERTS_PER_WINDOW), out->alerts ? out->alerts_cap : 0);
+  const u32 n_al = columns ? 0 : std::min<u32>(std::min<u32>(out->n_alerts_total, CCLD_MAX_ALERTS_PER_WINDOW), out->alerts ? out->alerts_cap : 0);
   if (n_al) std::memcpy(out->alerts, hv + area.alerts, n_al * sizeof(ccld_hang_alert));
   // cumulative suspects
   out->n_suspects_total = head->n_suspects;
-  const u32 n_out = std::min<u32>(head->n_suspects, out->suspects ? out->suspects_cap : 0);
+  const u32 n_out = columns ? 0 : std::min<u32>(head->n_suspects, out->suspects ? out->suspects_cap : 0);
   if (n_out && head->n_suspects <= area.sus_cap) std::memcpy(out->suspects, hv + area.suspects, n_out * sizeof(ccld_suspect));
   else if (n_out) {
     CK(cudaMemcpyAsync(out->suspects, m + L.sus, n_out * sizeof(ccld_suspect), cudaMemcpyDeviceToHost, ctx->stream));
@@ -991,6 +1005,18 @@ int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
   if (err & CCLD_E_DUPLICATE) return fail(ctx, CCLD_ERR_DUPLICATE, "duplicate (communicator, op counter, rank) record");
   if (err & CCLD_E_CAPACITY) return fail(ctx, CCLD_ERR_CAPACITY, "op counters of the window span too many slots");
   return CCLD_OK;
+}
+
+int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
+  NvtxRange nvtx_range("ccld_get_verdict");
+  if (!ctx || !out) return CCLD_ERR_ARG;
+  return verdict(ctx, window_id, out, nullptr);
+}
+
+int ccld_get_verdict_columns(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out, ccld_verdict_columns* columns) {
+  NvtxRange nvtx_range("ccld_get_verdict_columns");
+  if (!ctx || !out || !columns) return CCLD_ERR_ARG;
+  return verdict(ctx, window_id, out, columns);
 }
 
 // Launches the hang kernel over one op or over the window's alerts (A.alerts set) and waits; results are in pinned memory.

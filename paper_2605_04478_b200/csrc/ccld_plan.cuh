@@ -5,8 +5,8 @@
 //             lengths get their start values
 //   k_layout  one CTA per window: prefix sums over the communicators (groups, slots, rows, work units) and the start of every
 //             chunk of the work lists; the other CTAs of the launch fill the slot table of a batch that does not wait
-//   k_emit    a CTA per (window, chunk) writes that chunk's part of the work lists; further CTAs resolve every rank's inline
-//             pairs against the window's rows
+//   k_emit    a CTA per (window, chunk, 256 communicators) writes their part of the chunk's work lists; further CTAs resolve
+//             every rank's inline pairs against the window's rows
 //
 // All three are bound by latency: little data, a chain of dependent reads and barriers. The layout used to be one CTA per
 // window for everything - one scan over the communicators per chunk, the rank table of the whole job walked by one SM -
@@ -20,7 +20,9 @@ namespace ccld {
 
 constexpr int BEGIN_THREADS = 256;
 constexpr int LAYOUT_THREADS = 1024;
+constexpr u32 LAYOUT_CACHED = 4;                       // communicators per thread whose ranges wait in registers (4,096 per window)
 constexpr int EMIT_THREADS = 256;
+constexpr u32 EMIT_SLICES = 32;
 
 struct BeginArgs {
   const u32* desc_host; u32* desc; u64 desc_words;     // pinned source, device copy: descriptors (and expected totals behind them)
@@ -35,13 +37,13 @@ __global__ void __launch_bounds__(BEGIN_THREADS) k_begin(BeginArgs A) {
   for (u64 i = i0; i < A.n_zero; i += st) A.zero[i] = 0;
 }
 
-// op counters communicator c covers in the window (0 if none; clamped to 2^32 - 1)
-__device__ __forceinline__ u32 plan_nseq(const WinDesc& D, u32 c) {
-  const u32 lo = D.rmin[c], hi = D.rmax[c];
+// op counters a communicator covers in the window (0 if none; clamped to 2^32 - 1)
+__device__ __forceinline__ u32 range_len(u32 lo, u32 hi) {
   if (!(lo <= hi && lo != NONE)) return 0;
   const u64 ns = (u64)hi - lo + 1;
   return ns > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)ns;
 }
+__device__ __forceinline__ u32 plan_nseq(const WinDesc& D, u32 c) { return range_len(D.rmin[c], D.rmax[c]); }
 
 // Work units (warp-tiles of class 0, CTA tiles of class 1) of a communicator in chunk tau; 0 for other classes.
 __device__ __forceinline__ u32 chunk_units(u32 ns, u32 n, u32 T, u32 tau) {
@@ -105,9 +107,26 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
     return;
   }
   const u32 per = ceil_div(R.n_comms, LAYOUT_THREADS), c_lo = threadIdx.x * per, c_hi = min(R.n_comms, c_lo + per);   // my communicators
+  // counters covered and members of my first few communicators stay in registers, all loads issued at once
+  u32 c_ns[LAYOUT_CACHED], c_n[LAYOUT_CACHED];
+  {
+    u32 lo[LAYOUT_CACHED], hi[LAYOUT_CACHED];
+#pragma unroll
+    for (u32 k = 0; k < LAYOUT_CACHED; ++k) {
+      const bool in = c_lo + k < c_hi;
+      lo[k] = in ? D.rmin[c_lo + k] : NONE; hi[k] = in ? D.rmax[c_lo + k] : 0; c_n[k] = in ? R.comm_n[c_lo + k] : 1u;
+    }
+#pragma unroll
+    for (u32 k = 0; k < LAYOUT_CACHED; ++k) c_ns[k] = range_len(lo[k], hi[k]);
+  }
+  const auto each = [&](auto&& f) {                            // f(k, counters covered, members), the same number of steps in every thread
+#pragma unroll
+    for (u32 k = 0; k < LAYOUT_CACHED; ++k) if (k < per) f(k, c_ns[k], c_n[k]);
+    for (u32 k = LAYOUT_CACHED; k < per; ++k) { const bool in = c_lo + k < c_hi; f(k, in ? plan_nseq(D, c_lo + k) : 0u, in ? R.comm_n[c_lo + k] : 1u); }
+  };
   // the busiest communicator of the fused classes decides how many chunks there are
   u32 mx = 0;
-  for (u32 c = c_lo; c < c_hi; ++c) { const u32 ns = plan_nseq(D, c); if (comm_class(R.comm_n[c]) <= 1) mx = max(mx, ns); }
+  each([&](u32, u32 ns, u32 n) { if (comm_class(n) <= 1) mx = max(mx, ns); });
   mx = __reduce_max_sync(0xFFFFFFFFu, mx);
   if (lane == 0) s_red[wid] = mx;
   for (u32 i = threadIdx.x; i < 2 * (CHUNK_MAX + 2); i += LAYOUT_THREADS) (&s_hist[0][0])[i] = 0;
@@ -117,10 +136,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
   T = T > CHUNK_MAX ? CHUNK_MAX : T;
   // sums over my communicators, and where their units begin and end along the chunks
   PlanAcc mine = {0, 0, 0, 0, 0, 0};
-  for (u32 k = 0; k < per; ++k) {                              // the same number of steps in every thread
-    const u32 c = c_lo + k;
-    const bool in = c < c_hi;
-    const u32 ns = in ? plan_nseq(D, c) : 0, n = in ? R.comm_n[c] : 1u;
+  each([&](u32, u32 ns, u32 n) {
     mine = plan_add(mine, plan_item(ns, n, T));
     const ChunkShape x = chunk_shape(ns, n, T);
     // communicators of one family end in the same chunk: one set of atomics for all lanes that agree
@@ -137,7 +153,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
       }
       pend &= ~__ballot_sync(0xFFFFFFFFu, same);
     }
-  }
+  });
   // exclusive prefix over the threads
   PlanAcc inc = mine;
 #pragma unroll
@@ -208,8 +224,9 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
   }
   __syncthreads();
   const bool failed = s_red[0] != 0;                           // a window that is given up leaves no work behind: empty rows
-  for (u32 c = c_lo; c < c_hi; ++c) {
-    const u32 ns = plan_nseq(D, c), n = R.comm_n[c];
+  each([&](u32 k, u32 ns, u32 n) {
+    const u32 c = c_lo + k;
+    if (c >= c_hi) return;
     const PlanAcc it = plan_item(ns, n, T);
     RangeRow r = {0, 0, 0, n, 0, 0, 0, 0};
     if (!failed) {
@@ -220,14 +237,15 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
     D.ranges[c] = r;
     D.srow[c] = make_uint4((u32)r.slot0, (u32)(r.slot0 >> 32), r.n_seq, r.seq_lo);
     run = plan_add(run, it);
-  }
+  });
 }
 
-// Grid: (chunk CTAs + rank CTAs, windows); at least as many chunk CTAs as any window of the batch has chunks. base[] of the
-// descriptors is filled. A window that gave up fills its stretch of the lists with entries that hold no work, because the
-// kernels that follow are launched over the expected lengths.
-__global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict__ wd, Registry R, PlanLists L, u32 chunk_ctas) {
-  __shared__ uint2 s_pair[EMIT_THREADS / 32 + 1];
+// Grid: (chunk CTAs + rank CTAs, windows); chunk CTA x takes slice x % slices of chunk x / slices: `blocks` times EMIT_THREADS
+// communicators (one time, unless a registry has more than EMIT_SLICES times as many). There are enough of them for every
+// chunk of any window of the batch. base[] of the descriptors is filled. A window that gave up fills its stretch of the
+// lists with entries that hold no work, because the kernels that follow are launched over the expected lengths.
+__global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict__ wd, Registry R, PlanLists L, u32 chunk_ctas, u32 slices, u32 blocks) {
+  __shared__ uint4 s_pair[EMIT_THREADS / 32];
   const WinDesc& D = wd[blockIdx.y];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const u64 failed = D.totals[T_FAILED];
@@ -258,10 +276,9 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict
     }
     return;
   }
-  const u32 tau = blockIdx.x;
   if (give_up) {
     if (D.expect == nullptr) return;                           // the host knows: it sized nothing for this window
-    const u32 i0 = tau * EMIT_THREADS + threadIdx.x, st = chunk_ctas * EMIT_THREADS;
+    const u32 i0 = blockIdx.x * EMIT_THREADS + threadIdx.x, st = chunk_ctas * EMIT_THREADS;
     if (!failed) {                                             // another window's layout was the surprise: this one's rows go too
       for (u32 c = i0; c < R.n_comms; c += st) { D.ranges[c] = RangeRow{0, 0, 0, R.comm_n[c], 0, 0, 0, 0}; D.srow[c] = make_uint4(0, 0, 0, 0); }
       if (i0 == 0) for (int q = 0; q < T_COUNT; ++q) { const u64 v = q == T_FAILED ? FAILED_EXPECT : 0; D.totals_host[q] = v; }
@@ -278,10 +295,10 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict
     for (u64 j = i0; j < n3 * L.grp_words_per_tile; j += st) L.grp_words[(u64)D.base[B_T3] * L.grp_words_per_tile + j] = 0;
     return;
   }
-  const u32 T = (u32)D.totals[T_CHUNKS];
+  const u32 T = (u32)D.totals[T_CHUNKS], tau = blockIdx.x / slices, slice = blockIdx.x % slices;
   if (tau >= T) return;
   // tiles of classes 2 and 3: a warp per communicator, lanes along its tiles
-  for (u32 c = tau * (EMIT_THREADS / 32) + wid; c < R.n_comms; c += T * (EMIT_THREADS / 32)) {
+  for (u32 c = blockIdx.x * (EMIT_THREADS / 32) + wid; c < R.n_comms; c += T * slices * (EMIT_THREADS / 32)) {
     const u32 n = R.comm_n[c], cls = comm_class(n);
     if (cls < 2) continue;
     const RangeRow row = D.ranges[c];
@@ -297,46 +314,50 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict
       for (u64 k = lane; k < (u64)row.n_units * L.grp_words_per_tile; k += 32) g[k] = 0;
     }
   }
-  // fused classes: my consecutive communicators' units of this chunk, then where they go
-  const u32 per = ceil_div(R.n_comms, EMIT_THREADS), c_lo = threadIdx.x * per, c_hi = min(R.n_comms, c_lo + per);
-  u32 wt = 0, c1 = 0;
-  for (u32 c = c_lo; c < c_hi; ++c) {
-    const u32 n = R.comm_n[c];
-    if (comm_class(n) > 1) continue;
-    const u32 u = chunk_units(D.ranges[c].n_seq, n, T, tau);
-    if (comm_class(n) == 0) wt += u; else c1 += u;
-  }
-  u32 iw = wt, ic = c1;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const u32 ow = __shfl_up_sync(0xFFFFFFFFu, iw, d), oc = __shfl_up_sync(0xFFFFFFFFu, ic, d);
-    if (lane >= (u32)d) { iw += ow; ic += oc; }
-  }
-  if (lane == 31) s_pair[wid] = make_uint2(iw, ic);
-  __syncthreads();
-  u32 bw = 0, bc = 0;
-#pragma unroll
-  for (u32 q = 0; q < EMIT_THREADS / 32; ++q) { const uint2 x = s_pair[q]; if (q < wid) { bw += x.x; bc += x.y; } }
+  // fused classes: the units of this chunk that earlier slices hold, those of my communicator, then where they go
+  const auto units_of = [&](u32 c, u32& wt, u32& c1) {
+    const u32 n = R.comm_n[c], cls = comm_class(n), u = cls <= 1 ? chunk_units(D.srow[c].z, n, T, tau) : 0u;
+    if (cls == 0) wt += u; else c1 += u;
+  };
   const uint2 here = D.chunks[tau], next = D.chunks[tau + 1];
   const u32 wt_base = D.base[B_FWT] + here.y, wt_total = next.y - here.y, cta_base = D.base[B_FCTA] + here.x, n0 = ceil_div(wt_total, FUSED_WT_PER_CTA);
-  u32 at_w = wt_base + bw + iw - wt, at_c = cta_base + n0 + bc + ic - c1;        // class-1 CTAs come after the chunk's class-0 CTAs
-  for (u32 c = c_lo; c < c_hi; ++c) {
-    const u32 n = R.comm_n[c], cls = comm_class(n);
-    if (cls > 1) continue;
-    const RangeRow row = D.ranges[c];
-    const u32 u = chunk_units(row.n_seq, n, T, tau);
-    if (u == 0) continue;
-    const u64 moff = R.comm_moff[c];
-    const u32 S = chunk_len(row.n_seq, T), U = tile_seqs(n), cnt = chunk_size(row.n_seq, T, tau);
-    const u32 sum0 = D.base[B_FSUM] + row.tile0 + tau * ceil_div(S, U);
-    for (u32 k = 0; k < u; ++k) {
-      const u32 off = tau * S + k * U, len = cnt - k * U < U ? cnt - k * U : U;
-      if (cls == 0) { WarpTile x; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.row = row; x.moff = moff; L.fwt[at_w++] = x; }
-      else { FusedCta x; x.w = blockIdx.y; x.cls = 1; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.wt_first = 0; x.wt_count = 0;
-             x.row = row; x.moff = moff; L.fcta[at_c++] = x; }
+  u32 ew = 0, ec = 0;                                          // this thread's share of what lies before
+#pragma unroll 4
+  for (u32 k = 0; k < slice * blocks; ++k) units_of(k * EMIT_THREADS + threadIdx.x, ew, ec);
+  for (u32 m = 0; m < blocks; ++m) {
+    const u32 c = (slice * blocks + m) * EMIT_THREADS + threadIdx.x;
+    u32 wt = 0, c1 = 0;
+    if (c < R.n_comms) units_of(c, wt, c1);
+    u32 iw = wt, ic = c1;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const u32 ow = __shfl_up_sync(0xFFFFFFFFu, iw, d), oc = __shfl_up_sync(0xFFFFFFFFu, ic, d);
+      if (lane >= (u32)d) { iw += ow; ic += oc; }
     }
+    const u32 rw = __reduce_add_sync(0xFFFFFFFFu, ew), rc = __reduce_add_sync(0xFFFFFFFFu, ec);
+    if (lane == 31) s_pair[wid] = make_uint4(iw, ic, rw, rc);
+    __syncthreads();
+    u32 bw = 0, bc = 0;                                        // before my warp: all that came earlier, and the warps before mine
+#pragma unroll
+    for (u32 q = 0; q < EMIT_THREADS / 32; ++q) { const uint4 x = s_pair[q]; bw += x.z; bc += x.w; if (q < wid) { bw += x.x; bc += x.y; } }
+    u32 at_w = wt_base + bw + iw - wt, at_c = cta_base + n0 + bc + ic - c1;      // class-1 CTAs come after the chunk's class-0 CTAs
+    if (wt + c1 != 0) {
+      const u32 n = R.comm_n[c], cls = comm_class(n);
+      const RangeRow row = D.ranges[c];
+      const u64 moff = R.comm_moff[c];
+      const u32 S = chunk_len(row.n_seq, T), U = tile_seqs(n), cnt = chunk_size(row.n_seq, T, tau);
+      const u32 sum0 = D.base[B_FSUM] + row.tile0 + tau * ceil_div(S, U);
+      for (u32 k = 0; k < wt + c1; ++k) {
+        const u32 off = tau * S + k * U, len = cnt - k * U < U ? cnt - k * U : U;
+        if (cls == 0) { WarpTile x; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.row = row; x.moff = moff; L.fwt[at_w++] = x; }
+        else { FusedCta x; x.w = blockIdx.y; x.cls = 1; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.wt_first = 0; x.wt_count = 0;
+               x.row = row; x.moff = moff; L.fcta[at_c++] = x; }
+      }
+    }
+    ew += wt; ec += c1;
+    __syncthreads();
   }
-  for (u32 j = threadIdx.x; j < n0; j += EMIT_THREADS) {
+  for (u32 j = slice * EMIT_THREADS + threadIdx.x; j < n0; j += slices * EMIT_THREADS) {
     FusedCta x; x.w = blockIdx.y; x.cls = 0; x.c = 0; x.seq_off = 0; x.count = 0; x.sum_idx = 0; x.moff = 0;
     x.row = RangeRow{0, 0, 0, 0, 0, 0, 0, 0};
     x.wt_first = wt_base + FUSED_WT_PER_CTA * j; x.wt_count = wt_total - FUSED_WT_PER_CTA * j < FUSED_WT_PER_CTA ? wt_total - FUSED_WT_PER_CTA * j : FUSED_WT_PER_CTA;

@@ -12,6 +12,7 @@
 // waits used to be; the rank-by-counting sort of an 8,000-suspect list over global memory took 243 us, the sorted pieces
 // with the merge take under 10 (communicators of four ranks, whose MAD rests on two values, name that many).
 #pragma once
+#include <cstddef>
 #include "ccld_kernels.cuh"
 
 namespace ccld {
@@ -27,9 +28,10 @@ struct VerdictArgs {
   const ccld_hang_alert* alerts;
   u64* keys; u32* counts;                    // device scratch: [CTAs][VD_KEYS] sorted keys, [CTAs] how many
   VerdictHead* head;                         // pinned: counters and number of suspects
+  int columns;                               // 1: the pinned lists column by column, 64-bit fields first, each column as long as the list
   ccld_comm_verdict* rows_out;               // pinned [n_rows]
-  ccld_hang_alert* alerts_out;               // [CCLD_MAX_ALERTS_PER_WINDOW]
-  ccld_suspect* sus_host; u32 sus_host_cap;  // pinned; lists longer than that go to sus_dev
+  ccld_hang_alert* alerts_out;               // pinned [CCLD_MAX_ALERTS_PER_WINDOW]
+  ccld_suspect* sus_host; u32 sus_host_cap;  // pinned; lists longer than that go to sus_dev (as structs)
   ccld_suspect* sus_dev;
 };
 
@@ -44,16 +46,28 @@ __device__ __forceinline__ ccld_suspect suspect_of(const Registry& R, u64 key) {
   return s;
 }
 
+// Entry i of n into a list of structs, or into its columns.
+__device__ __forceinline__ void put_suspect(ccld_suspect* out, u32 i, u32 n, bool columns, const ccld_suspect& s) {
+  if (!columns) { out[i] = s; return; }
+  double* d = (double*)out; u32* u = (u32*)(d + n);
+  d[i] = s.mean_busbw; u[i] = s.kind; u[n + i] = s.rank; u[2 * n + i] = s.votes; u[3 * n + i] = s.ops;
+}
+__device__ __forceinline__ void put_alert(ccld_hang_alert* out, u32 i, u32 n, bool columns, const ccld_hang_alert& a) {
+  if (!columns) { out[i] = a; return; }
+  i64* t = (i64*)out; u32* u = (u32*)(t + n);
+  t[i] = a.age_ns; u[i] = a.comm; u[n + i] = a.seq;
+}
+
 // The alerts of a window in the order they are listed: registration order of the communicator, then op counter (then the
 // place in the unordered list: an op raises one alert). One CTA; s_key holds CCLD_MAX_ALERTS_PER_WINDOW keys.
-__device__ __forceinline__ void order_alerts(const Registry& R, const ccld_hang_alert* __restrict__ in, u32 n, ccld_hang_alert* __restrict__ out, u64* s_key) {
+__device__ __forceinline__ void order_alerts(const Registry& R, const ccld_hang_alert* __restrict__ in, u32 n, ccld_hang_alert* __restrict__ out, bool columns, u64* s_key) {
   for (u32 i = threadIdx.x; i < n; i += blockDim.x) s_key[i] = ((u64)comm_lookup(R, in[i].comm) << 32) | in[i].seq;
   __syncthreads();
   for (u32 i = threadIdx.x; i < n; i += blockDim.x) {
     const u64 k = s_key[i];
     u32 before = 0;
     for (u32 j = 0; j < n; ++j) before += (s_key[j] < k || (s_key[j] == k && j < i)) ? 1u : 0u;
-    out[before] = in[i];
+    put_alert(out, before, n, columns, in[i]);
   }
   __syncthreads();
 }
@@ -62,17 +76,24 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_collect(VerdictArgs A, R
   __shared__ u64 s_key[VD_KEYS];
   __shared__ u32 s_n;
   const u32 lane = threadIdx.x & 31;
-  // communicator rows, all CTAs: whole 8-byte words
+  // communicator rows, all CTAs: whole 8-byte words, or the struct's ten 32-bit and eight 64-bit fields as columns
   {
-    const u64 words = (u64)A.n_rows * (sizeof(ccld_comm_verdict) / 8);
-    static_assert(sizeof(ccld_comm_verdict) % 8 == 0, "rows are copied as 8-byte words");
+    static_assert(sizeof(ccld_comm_verdict) == 13 * 8 && offsetof(ccld_comm_verdict, slow_count) == 40, "ten 32-bit fields, then eight of 64");
+    const u64 t0 = (u64)blockIdx.x * VD_THREADS + threadIdx.x, st = (u64)gridDim.x * VD_THREADS;
     const u64* src = (const u64*)A.rows; u64* dst = (u64*)A.rows_out;
-    for (u64 i = (u64)blockIdx.x * VD_THREADS + threadIdx.x; i < words; i += (u64)gridDim.x * VD_THREADS) dst[i] = src[i];
+    if (!A.columns) for (u64 i = t0; i < (u64)A.n_rows * 13; i += st) dst[i] = src[i];
+    else {
+      u32* dst32 = (u32*)(dst + (u64)A.n_rows * 8);
+      for (u64 i = t0; i < (u64)A.n_rows * 18; i += st) {
+        const u32 f = (u32)(i / A.n_rows), r = (u32)(i % A.n_rows);
+        if (f < 8) dst[i] = src[(u64)r * 13 + 5 + f]; else dst32[(u64)(f - 8) * A.n_rows + r] = ((const u32*)A.rows)[(u64)r * 26 + f - 8];
+      }
+    }
   }
   if (blockIdx.x == 0) {
     if (threadIdx.x < C_COUNT) A.head->counters[threadIdx.x] = A.counters[threadIdx.x];
     const u64 n_al = A.counters[C_ALERTS];
-    if (n_al) order_alerts(R, A.alerts, n_al < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n_al : CCLD_MAX_ALERTS_PER_WINDOW, A.alerts_out, s_key);
+    if (n_al) order_alerts(R, A.alerts, n_al < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n_al : CCLD_MAX_ALERTS_PER_WINDOW, A.alerts_out, A.columns != 0, s_key);
   }
   if (threadIdx.x == 0) s_n = 0;
   __syncthreads();
@@ -107,8 +128,8 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_collect(VerdictArgs A, R
     }
   }
   if (gridDim.x == 1) {
-    ccld_suspect* dst = n <= A.sus_host_cap ? A.sus_host : A.sus_dev;
-    for (u32 i = threadIdx.x; i < n; i += VD_THREADS) dst[i] = suspect_of(R, s_key[i]);
+    const bool host = n <= A.sus_host_cap;
+    for (u32 i = threadIdx.x; i < n; i += VD_THREADS) put_suspect(host ? A.sus_host : A.sus_dev, i, n, host && A.columns, suspect_of(R, s_key[i]));
     if (threadIdx.x == 0) A.head->n_suspects = n;
   } else {
     for (u32 i = threadIdx.x; i < n; i += VD_THREADS) A.keys[(u64)blockIdx.x * VD_KEYS + i] = s_key[i];
@@ -127,7 +148,7 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_merge(VerdictArgs A, Reg
   __syncthreads();
   const u32 total = s_tot, n = A.counts[blockIdx.x];
   if (blockIdx.x == 0 && threadIdx.x == 0) A.head->n_suspects = total;
-  ccld_suspect* dst = total <= A.sus_host_cap ? A.sus_host : A.sus_dev;
+  const bool host = total <= A.sus_host_cap;
   const u64* mine = A.keys + (u64)blockIdx.x * VD_KEYS;
   for (u32 i = threadIdx.x; i < n; i += VD_THREADS) {
     const u64 key = mine[i];
@@ -139,7 +160,7 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_merge(VerdictArgs A, Reg
       while (lo < hi) { const u32 mid = (lo + hi) >> 1; if (other[mid] < key) lo = mid + 1; else hi = mid; }
       pos += lo;
     }
-    dst[pos] = suspect_of(R, key);
+    put_suspect(host ? A.sus_host : A.sus_dev, pos, total, host && A.columns, suspect_of(R, key));
   }
 }
 
@@ -163,7 +184,7 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(GatherArgs A) {
 __global__ void __launch_bounds__(VD_THREADS) k_order_alerts(const u64* __restrict__ counters, const ccld_hang_alert* __restrict__ in, ccld_hang_alert* __restrict__ out, Registry R) {
   __shared__ u64 s_key[CCLD_MAX_ALERTS_PER_WINDOW];
   const u64 n = counters[C_ALERTS];
-  order_alerts(R, in, n < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n : CCLD_MAX_ALERTS_PER_WINDOW, out, s_key);
+  order_alerts(R, in, n < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n : CCLD_MAX_ALERTS_PER_WINDOW, out, false, s_key);
 }
 
 }  // namespace ccld
