@@ -150,6 +150,7 @@ struct ccld_ctx {
   Pool pool; std::string err;
   Block h_verdict;                                       // pinned area of ccld_get_verdict (VerdictArea)
   Block h_io;                                            // pinned area small results pass through
+  bool long_list = false;                                // the last suspect list was longer than VD_MERGE
   std::vector<char> long_suspects;                       // columns of a suspect list that outgrew the pinned area
   Block h_up; UploadSlot up[UP_SLOTS]; u32 up_next = 0;
   u64 batches_redone = 0;                                // batches settle() had to analyse again
@@ -204,12 +205,12 @@ struct TimedLaunch {                                     // a named range and, w
 };
 
 // Layout of the scratch block used by get_verdict and locate_hang.
-struct MiscLayout { size_t sus, keys, counts, alerts, total; };
+struct MiscLayout { size_t sus, keys, counts, done, alerts, total; };
 MiscLayout misc_layout(u32 n_ranks) {
   MiscLayout L; size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + std::max<size_t>(b, 1)); return o; };
   const size_t pieces = (n_ranks + VD_THREADS - 1) / VD_THREADS;
-  L.sus = take(2ull * n_ranks * sizeof(ccld_suspect)); L.keys = take(pieces * VD_KEYS * 8); L.counts = take(pieces * 4);
+  L.sus = take(2ull * n_ranks * sizeof(ccld_suspect)); L.keys = take(pieces * VD_KEYS * 8); L.counts = take(pieces * 4); L.done = take(4);
   L.alerts = take(CCLD_MAX_ALERTS_PER_WINDOW * sizeof(ccld_hang_alert));
   L.total = off;
   return L;
@@ -328,6 +329,7 @@ int finalize_registry(ccld_ctx* ctx) {
   // scratch for suspects, alert ordering and hang location
   ctx->misc_blk = ctx->pool.get(misc_layout(nr).total, &e);
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
+  CK(cudaMemsetAsync((char*)ctx->misc_blk.p + misc_layout(nr).done, 0, 4, st));
 
   CK(cudaFuncSetAttribute(k_reduce_mid<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem_bytes(256)));
   CK(cudaFuncSetAttribute(k_reduce_mid<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem_bytes(512)));
@@ -949,15 +951,22 @@ static int verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out, ccld_ve
     n_rows = columns ? (u32)w->totals[T_ROWS] : std::min<u32>((u32)w->totals[T_ROWS], out->comm_rows ? out->comm_rows_cap : 0);
     VerdictArgs A;
     A.counters = w->d.counters; A.rows = w->d.comm_rows; A.n_rows = n_rows; A.alerts = w->d.alerts; A.columns = columns != nullptr;
-    A.keys = (u64*)(m + L.keys); A.counts = (u32*)(m + L.counts);
+    A.keys = (u64*)(m + L.keys); A.counts = (u32*)(m + L.counts); A.done = (u32*)(m + L.done);
     A.head = (VerdictHead*)hv; A.rows_out = (ccld_comm_verdict*)(hv + area.rows);
     A.alerts_out = (ccld_hang_alert*)(hv + area.alerts);
     A.sus_host = (ccld_suspect*)(hv + area.suspects); A.sus_host_cap = area.sus_cap; A.sus_dev = (ccld_suspect*)(m + L.sus);
     const u32 pieces = (ctx->n_ranks + VD_THREADS - 1) / VD_THREADS;
-    k_verdict_collect<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg, ctx->dp);
-    if (pieces > 1) k_verdict_merge<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg);
+    k_verdict_collect<<<pieces + 1 + n_rows / VD_THREADS, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg, ctx->dp, pieces);
+    // suspect lists keep their length from call to call, roughly: where the last one was long, the merge goes along at once
+    if (pieces > 1 && ctx->long_list) k_verdict_merge<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(ctx->stream));
+    if (!head->listed) {
+      k_verdict_merge<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg);
+      CK(cudaGetLastError());
+      CK(cudaStreamSynchronize(ctx->stream));
+    }
+    ctx->long_list = head->n_suspects > (u32)VD_MERGE;
     const u64 redone = ctx->batches_redone;
     { int rc = settle(ctx); if (rc != CCLD_OK) return rc; }
     if (ctx->batches_redone == redone) break;

@@ -2,12 +2,13 @@
 //
 //   k_verdict_collect  a CTA per 1,024 ranks: which of its ranks are suspects (vote shares against the threshold), as one
 //                      64-bit key each that orders like the list - kind, votes descending, rank -, sorted in shared
-//                      memory; the CTAs also copy the window's communicator rows and counters, the first one orders the
-//                      hang alerts. A job of up to 1,024 ranks is done after this launch.
-//   k_verdict_merge    more than 1,024 ranks: the sorted pieces become one list. A key's place is its place in its own
+//                      memory; the last of them to finish puts the pieces of a list of up to 1,024 together. Further CTAs
+//                      copy the window's communicator rows and counters and order the hang alerts (apart, so that the fence
+//                      before "finished" does not wait for their writes across PCIe).
+//   k_verdict_merge    longer lists: the sorted pieces become one list. A key's place is its place in its own
 //                      piece plus, for every other piece, the number of keys before it (a binary search).
 //
-// Bound by latency: the inputs are a few hundred KB at most. One launch (two for larger jobs), no copy and one wait of the
+// Bound by latency: the inputs are a few hundred KB at most. One launch (two for long lists), no copy and one wait of the
 // host per verdict, where a copy of the counters, a launch, a copy of the count, a launch and two more copies with three
 // waits used to be; the rank-by-counting sort of an 8,000-suspect list over global memory took 243 us, the sorted pieces
 // with the merge take under 10 (communicators of four ranks, whose MAD rests on two values, name that many).
@@ -21,12 +22,15 @@ constexpr int VD_THREADS = 1024;             // ranks per CTA
 constexpr int VD_KEYS = 2 * VD_THREADS;      // a rank is on the list at most twice
 constexpr u32 VD_SUS_HOST = 65536;           // suspects the pinned area holds at most; longer lists stay in device memory
 
-struct VerdictHead { u64 counters[C_COUNT]; u32 n_suspects, pad; };
+constexpr int VD_MERGE = 1024;               // lists up to this long are put together by the last CTA of k_verdict_collect
+
+struct VerdictHead { u64 counters[C_COUNT]; u32 n_suspects, listed; };     // listed: the suspects are in place
 struct VerdictArgs {
   const u64* counters;                       // the window's
   const ccld_comm_verdict* rows; u32 n_rows; // (null, 0): nothing to copy
   const ccld_hang_alert* alerts;
   u64* keys; u32* counts;                    // device scratch: [CTAs][VD_KEYS] sorted keys, [CTAs] how many
+  u32* done;                                 // device: CTAs finished so far (0 between launches)
   VerdictHead* head;                         // pinned: counters and number of suspects
   int columns;                               // 1: the pinned lists column by column, 64-bit fields first, each column as long as the list
   ccld_comm_verdict* rows_out;               // pinned [n_rows]
@@ -72,28 +76,34 @@ __device__ __forceinline__ void order_alerts(const Registry& R, const ccld_hang_
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(VD_THREADS) k_verdict_collect(VerdictArgs A, Registry R, Params P) {
+__global__ void __launch_bounds__(VD_THREADS) k_verdict_collect(VerdictArgs A, Registry R, Params P, u32 pieces) {
   __shared__ u64 s_key[VD_KEYS];
   __shared__ u32 s_n;
   const u32 lane = threadIdx.x & 31;
-  // communicator rows, all CTAs: whole 8-byte words, or the struct's ten 32-bit and eight 64-bit fields as columns
-  {
+  if (blockIdx.x >= pieces) {
+    // communicator rows: whole 8-byte words, or the struct's ten 32-bit and eight 64-bit fields as columns
     static_assert(sizeof(ccld_comm_verdict) == 13 * 8 && offsetof(ccld_comm_verdict, slow_count) == 40, "ten 32-bit fields, then eight of 64");
-    const u64 t0 = (u64)blockIdx.x * VD_THREADS + threadIdx.x, st = (u64)gridDim.x * VD_THREADS;
+    const u64 t0 = (u64)(blockIdx.x - pieces) * VD_THREADS + threadIdx.x, st = (u64)(gridDim.x - pieces) * VD_THREADS;
     const u64* src = (const u64*)A.rows; u64* dst = (u64*)A.rows_out;
     if (!A.columns) for (u64 i = t0; i < (u64)A.n_rows * 13; i += st) dst[i] = src[i];
     else {
       u32* dst32 = (u32*)(dst + (u64)A.n_rows * 8);
-      for (u64 i = t0; i < (u64)A.n_rows * 18; i += st) {
-        const u32 f = (u32)(i / A.n_rows), r = (u32)(i % A.n_rows);
-        if (f < 8) dst[i] = src[(u64)r * 13 + 5 + f]; else dst32[(u64)(f - 8) * A.n_rows + r] = ((const u32*)A.rows)[(u64)r * 26 + f - 8];
+      for (u64 r = t0; r < A.n_rows; r += st) {                // a thread per row: lanes write along the columns
+        u64 x[13];
+#pragma unroll
+        for (int k = 0; k < 13; ++k) x[k] = src[r * 13 + k];
+#pragma unroll
+        for (int f = 0; f < 8; ++f) dst[(u64)f * A.n_rows + r] = x[5 + f];
+#pragma unroll
+        for (int f = 0; f < 5; ++f) { dst32[(u64)(2 * f) * A.n_rows + r] = (u32)x[f]; dst32[(u64)(2 * f + 1) * A.n_rows + r] = (u32)(x[f] >> 32); }
       }
     }
-  }
-  if (blockIdx.x == 0) {
-    if (threadIdx.x < C_COUNT) A.head->counters[threadIdx.x] = A.counters[threadIdx.x];
-    const u64 n_al = A.counters[C_ALERTS];
-    if (n_al) order_alerts(R, A.alerts, n_al < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n_al : CCLD_MAX_ALERTS_PER_WINDOW, A.alerts_out, A.columns != 0, s_key);
+    if (blockIdx.x == pieces) {
+      if (threadIdx.x < C_COUNT) A.head->counters[threadIdx.x] = A.counters[threadIdx.x];
+      const u64 n_al = A.counters[C_ALERTS];
+      if (n_al) order_alerts(R, A.alerts, n_al < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n_al : CCLD_MAX_ALERTS_PER_WINDOW, A.alerts_out, A.columns != 0, s_key);
+    }
+    return;
   }
   if (threadIdx.x == 0) s_n = 0;
   __syncthreads();
@@ -127,13 +137,46 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_collect(VerdictArgs A, R
       __syncthreads();
     }
   }
-  if (gridDim.x == 1) {
+  if (pieces == 1) {
     const bool host = n <= A.sus_host_cap;
     for (u32 i = threadIdx.x; i < n; i += VD_THREADS) put_suspect(host ? A.sus_host : A.sus_dev, i, n, host && A.columns, suspect_of(R, s_key[i]));
-    if (threadIdx.x == 0) A.head->n_suspects = n;
-  } else {
-    for (u32 i = threadIdx.x; i < n; i += VD_THREADS) A.keys[(u64)blockIdx.x * VD_KEYS + i] = s_key[i];
-    if (threadIdx.x == 0) A.counts[blockIdx.x] = n;
+    if (threadIdx.x == 0) { A.head->n_suspects = n; A.head->listed = 1; }
+    return;
+  }
+  for (u32 i = threadIdx.x; i < n; i += VD_THREADS) A.keys[(u64)blockIdx.x * VD_KEYS + i] = s_key[i];
+  if (threadIdx.x == 0) A.counts[blockIdx.x] = n;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_n = atomicAdd(A.done, 1u);
+  __syncthreads();
+  if (s_n != pieces - 1) return;
+  // the last CTA: short lists are put together here, longer ones are left to k_verdict_merge
+  __threadfence();
+  __shared__ u32 s_tot;
+  if (threadIdx.x == 0) { s_tot = 0; *A.done = 0; }
+  __syncthreads();
+  u32 t = 0;
+  for (u32 o = threadIdx.x; o < pieces; o += VD_THREADS) t += __ldcg(&A.counts[o]);
+  t = __reduce_add_sync(0xFFFFFFFFu, t);
+  if (lane == 0 && t) atomicAdd(&s_tot, t);
+  __syncthreads();
+  const u32 total = s_tot;
+  if (threadIdx.x == 0) { A.head->n_suspects = total; A.head->listed = total <= VD_MERGE; s_n = 0; }
+  if (total > VD_MERGE) return;
+  __syncthreads();
+  for (u32 o = threadIdx.x >> 5; o < pieces; o += VD_THREADS / 32) {                // a warp per piece, in any order
+    const u32 k = __ldcg(&A.counts[o]);
+    u32 at = 0;
+    if (lane == 0 && k) at = atomicAdd(&s_n, k);
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    for (u32 i = lane; i < k; i += 32) s_key[at + i] = __ldcg(&A.keys[(u64)o * VD_KEYS + i]);
+  }
+  __syncthreads();
+  if (threadIdx.x < total) {
+    const u64 key = s_key[threadIdx.x];
+    u32 pos = 0;
+    for (u32 i = 0; i < total; ++i) pos += s_key[i] < key ? 1u : 0u;                 // keys are unique
+    put_suspect(A.sus_host, pos, total, A.columns, suspect_of(R, key));
   }
 }
 
@@ -147,7 +190,7 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_merge(VerdictArgs A, Reg
   if ((threadIdx.x & 31) == 0 && t) atomicAdd(&s_tot, t);
   __syncthreads();
   const u32 total = s_tot, n = A.counts[blockIdx.x];
-  if (blockIdx.x == 0 && threadIdx.x == 0) A.head->n_suspects = total;
+  if (blockIdx.x == 0 && threadIdx.x == 0) { A.head->n_suspects = total; A.head->listed = 1; }
   const bool host = total <= A.sus_host_cap;
   const u64* mine = A.keys + (u64)blockIdx.x * VD_KEYS;
   for (u32 i = threadIdx.x; i < n; i += VD_THREADS) {
