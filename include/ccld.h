@@ -387,7 +387,7 @@ int ccld_state_import(ccld_ctx* ctx, const void* buf /* host */, uint64_t n_byte
  *   >= n_ranks, gets 0.
  * Every pointer is device memory of the context's device, owned by the caller and left untouched except for the two
  * outputs (n_rec entries each). The kernels are enqueued on the context's stream and the call returns without
- * synchronizing; scratch (8 bytes per tick) comes from the context's block pool. Counts are 32-bit:
+ * synchronizing; scratch (half a byte per tick and 32 bytes per rank) comes from the context's block pool. Counts are 32-bit:
  * n_ticks >= 2^32 - 1 is refused with CCLD_ERR_CAPACITY. Other errors: CCLD_ERR_ARG (null pointers, n_ranks = 0),
  * CCLD_ERR_NOMEM, CCLD_ERR_CUDA.
  */

@@ -465,16 +465,16 @@ class Analyzer:
         this GPU; returns (send_chg, recv_chg) as int32 tensors on this GPU (bit pattern uint32), written asynchronously on
         the analyzer's stream."""
         torch = self.torch
-        cols = [_as_tensor(torch, rank, "int32"), _as_tensor(torch, t_enter, "int64"), _as_tensor(torch, t_exit, "int64"),
-                _as_tensor(torch, tick_off, "int64"), _as_tensor(torch, tick_ns, "int64"), _as_tensor(torch, send_count, "int32"),
-                _as_tensor(torch, recv_count, "int32")]
-        assert all(c.device.type == "cuda" for c in cols), "ccld_derive_rates takes device memory"
-        cols = [c.contiguous() for c in cols]
-        n = int(cols[0].numel()); n_ranks = int(cols[3].numel()) - 1; n_ticks = int(cols[4].numel())
+        cols = [rank, t_enter, t_exit, tick_off, tick_ns, send_count, recv_count]
+        for i, v in enumerate(cols):
+            if type(v) is not torch.Tensor or not v.is_contiguous():
+                cols[i] = v = _as_tensor(torch, v, "int32" if i in (0, 5, 6) else "int64").contiguous()
+            assert v.is_cuda, "ccld_derive_rates takes device memory"
+        n = cols[0].numel()
         out_s = torch.empty(n, dtype=torch.int32, device=cols[0].device); out_r = torch.empty_like(out_s)
-        ptr = lambda v: C.c_void_p(v.data_ptr()) if v.numel() else C.c_void_p(0)
-        self._check(self.lib.ccld_derive_rates(self.h, n, ptr(cols[0]), ptr(cols[1]), ptr(cols[2]), n_ranks, n_ticks, ptr(cols[3]),
-                                               ptr(cols[4]), ptr(cols[5]), ptr(cols[6]), ptr(out_s), ptr(out_r)))
+        p = [c.data_ptr() for c in cols]                   # (null for an empty tensor)
+        self._check(self.lib.ccld_derive_rates(self.h, n, p[0], p[1], p[2], cols[3].numel() - 1, cols[4].numel(), p[3], p[4], p[5], p[6],
+                                               out_s.data_ptr(), out_r.data_ptr()))
         self._rate_keep = cols                     # inputs stay alive until the next call or a synchronization
         return out_s, out_r
 

@@ -1268,17 +1268,20 @@ int ccld_derive_rates(ccld_ctx* ctx, uint64_t n_rec, const uint32_t* rank, const
   const u64 n_tiles = (n_ticks + RT_TILE - 1) / RT_TILE;
   size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + b); return o; };
-  const size_t o_blk = take(((n_ticks + 31) / 32 + 1) * sizeof(TickBlock)), o_sum = take((n_tiles + 1) * 8);
+  const size_t o_blk = take(n_tiles * (RT_TILE / 32) * sizeof(TickBlock)), o_tile = take(n_tiles * sizeof(uint2)), o_rank = take(n_ranks * sizeof(RankTicks));
   cudaError_t e;
   Block blk = ctx->pool.get(off, &e);
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
-  TickArgs A; A.n_ticks = n_ticks; A.n_ranks = n_ranks; A.tick_off = tick_off; A.tick_ns = tick_ns; A.send = send_count; A.recv = recv_count;
-  A.blk = (TickBlock*)((char*)blk.p + o_blk); A.tile_sum = (u64*)((char*)blk.p + o_sum);
-  if (n_tiles) {
-    k_tick_blocks<<<(u32)n_tiles, RT_THREADS, 0, st>>>(A);
-    k_tile_scan<<<1, TS_THREADS, 0, st>>>(A.tile_sum, n_tiles);
-    k_block_prefix<<<(u32)n_tiles, RB_PER_TILE, 0, st>>>(A);
-  }
+  TickArgs A; A.n_ticks = n_ticks; A.n_ranks = n_ranks; A.n_tiles = (u32)n_tiles;
+  A.tick_off = tick_off; A.tick_ns = tick_ns; A.send = send_count; A.recv = recv_count;
+  A.blk = (TickBlock*)((char*)blk.p + o_blk); A.tile = (uint2*)((char*)blk.p + o_tile); A.ranks = (RankTicks*)((char*)blk.p + o_rank);
+  A.vec = (((uintptr_t)send_count | (uintptr_t)recv_count) & 15) == 0;
+  // A record adds up the tiles its op spans. Ops of one rank hardly overlap, so that is a read or two per record while a
+  // rank's samples cover a few tiles (8 tiles = 16 s at a sample per millisecond); with longer segments an op in flight
+  // since their beginning would add up many, and the scan (5 to 15 us) pays.
+  A.scanned = n_tiles > 256 && n_tiles > 8ull * n_ranks;
+  k_tick_blocks<<<(u32)(n_tiles + ((u64)n_ranks + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, st>>>(A);
+  if (A.scanned) k_tile_scan<<<1, TS_THREADS, 0, st>>>(A.tile, A.n_tiles);
   k_record_rates<<<(u32)((n_rec + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, st>>>(A, n_rec, rank, t_enter_ns, t_exit_ns, send_chg, recv_chg);
   const cudaError_t le = cudaGetLastError();
   ctx->pool.put(blk);           // later work on this stream runs after these kernels: the block can be handed out again
