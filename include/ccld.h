@@ -451,6 +451,22 @@ int ccld_ring_locate_static(int device, void* cuda_stream, uint32_t n_members, c
                             const uint8_t* state /* device */, uint32_t n_channels, const uint32_t* progress /* device */,
                             ccld_hang_verdict* out /* host */, char* err /* host */, uint32_t err_cap);
 
+/*
+ * Results in pinned host memory that the caller keeps, for callers whose arrays can live there: what the accessors above copy
+ * into the caller's buffers arrives in one block, without a second copy on the host. The pointers in the results lead into
+ * `block`, which stays valid - also beyond ccld_destroy - until ccld_host_release (any thread) gives it back. A block holds at
+ * most 16 MiB and all blocks in use at most 64 MiB: beyond that CCLD_ERR_CAPACITY is returned, nothing is taken and the copying
+ * accessors serve. Both calls synchronize the stream.
+ *   ccld_take_optable     the per-op table of a window with, per group, its communicator id, op counter and first slot
+ *   ccld_take_rank_stats  the cumulative statistics of ranks [0, n_ranks), n_ranks not beyond the largest registered rank
+ */
+typedef struct { void* p; uint64_t bytes; } ccld_host_block;
+typedef struct { ccld_optable t; const uint32_t *comm, *seq; const uint64_t* slot0; ccld_host_block block; } ccld_host_optable;
+typedef struct { const uint32_t *votes, *ops, *bw_cnt; const double* bw_sum; ccld_host_block block; } ccld_host_rank_stats;
+int ccld_take_optable(ccld_ctx* ctx, uint32_t window_id, ccld_host_optable* out /* host */);
+int ccld_take_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, ccld_host_rank_stats* out /* host */);
+void ccld_host_release(ccld_host_block* block /* host */);
+
 /* Utility for inspection tools: synchronous copy of `bytes` bytes from device memory of this context to host memory. */
 int ccld_copy_to_host(ccld_ctx* ctx, void* dst_host, const void* src_device, uint64_t bytes);
 /* The same for n arrays at once (array i: bytes[i] bytes from src_device[i] to dst_host[i]), with one wait for all of them. */

@@ -26,7 +26,8 @@ EXPORTS = ("ccld_params_default", "ccld_create", "ccld_destroy", "ccld_last_erro
            "ccld_trace_upload", "ccld_window_release", "ccld_analyze_window", "ccld_reset", "ccld_get_verdict",
            "ccld_locate_hang", "ccld_get_optable", "ccld_get_ranges", "ccld_get_rank_stats", "ccld_copy_to_host",
            "ccld_timing_enable", "ccld_get_kernel_times", "ccld_set_speculation", "ccld_ring_locate_static", "ccld_derive_rates", "ccld_locate_hangs", "ccld_state_export", "ccld_state_import", "ccld_trace_attach_opset", "ccld_opset_check",
-           "ccld_comm_set_layers", "ccld_copy_many_to_host", "ccld_get_verdict_columns")
+           "ccld_comm_set_layers", "ccld_copy_many_to_host", "ccld_get_verdict_columns", "ccld_take_optable", "ccld_take_rank_stats",
+           "ccld_host_release")
 STATIC_MAX_MEMBERS = 8192
 KERNEL_KINDS = ("k_seq_range", "k_plan", "k_slot_scatter", "k_reduce_fused", "k_reduce_mid", "k_reduce_large", "k_window_decide")
 
@@ -96,11 +97,25 @@ class OpTable(C.Structure):
                [(k, C.c_void_p) for k in OPTABLE_U32] + [("busbw", C.c_void_p), ("flags", C.c_void_p), ("perm", C.c_void_p)]
 
 
+class HostBlock(C.Structure):
+    _fields_ = [("p", C.c_void_p), ("bytes", C.c_uint64)]
+
+
+class HostOpTable(C.Structure):
+    _fields_ = [("t", OpTable), ("comm", C.c_void_p), ("seq", C.c_void_p), ("slot0", C.c_void_p), ("block", HostBlock)]
+
+
+class HostRankStats(C.Structure):
+    _fields_ = [(k, C.c_void_p) for k in ("votes", "ops", "bw_cnt", "bw_sum")] + [("block", HostBlock)]
+
+
 class CommRange(C.Structure):
     _fields_ = [("comm", C.c_uint32), ("n", C.c_uint32), ("seq_lo", C.c_uint32), ("n_seq", C.c_uint32),
                 ("group0", C.c_uint64), ("slot0", C.c_uint64)]
 
 
+_TABLE_DTYPES = [(k, np.int64) for k in OPTABLE_I64] + [(k, np.uint32) for k in OPTABLE_U32] + [("busbw", np.float64)]
+_NO_BLOCK = (-2, -8)                  # no pinned block to be had: the copying accessors serve
 _NP_OF = {C.c_uint32: "u4", C.c_uint64: "u8", C.c_int64: "i8", C.c_double: "f8"}
 
 
@@ -153,6 +168,10 @@ def load_library() -> C.CDLL:
         lib.ccld_get_rank_stats.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_copy_to_host.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_uint64]
         lib.ccld_get_verdict_columns.argtypes = [C.c_void_p, C.c_uint32, C.POINTER(Verdict), C.POINTER(VerdictColumns)]
+        lib.ccld_take_optable.argtypes = [C.c_void_p, C.c_uint32, C.POINTER(HostOpTable)]
+        lib.ccld_take_rank_stats.argtypes = [C.c_void_p, C.c_uint32, C.POINTER(HostRankStats)]
+        lib.ccld_host_release.restype = None
+        lib.ccld_host_release.argtypes = [C.POINTER(HostBlock)]
         lib.ccld_copy_many_to_host.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_derive_rates.argtypes = [C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p, C.c_uint32, C.c_uint64] + [C.c_void_p] * 6
         lib.ccld_timing_enable.argtypes = [C.c_void_p, C.c_int]
@@ -181,6 +200,19 @@ def _as_tensor(torch, v, dt):
     if a.dtype != np.dtype(dt):
         a = a.view(dt) if a.dtype.itemsize == np.dtype(dt).itemsize else a.astype(dt)
     return torch.from_numpy(a)
+
+
+class _Pinned:
+    """A pinned block of the library as an array buffer; given back once no array refers to it any more."""
+    __slots__ = ("block", "__array_interface__")
+
+    def __init__(self, block):
+        self.block = HostBlock(block.p, block.bytes)
+        self.__array_interface__ = {"shape": (block.bytes,), "typestr": "|u1", "data": (block.p, False), "version": 3}
+
+    def __del__(self):
+        if _lib is not None:
+            _lib.ccld_host_release(C.byref(self.block))
 
 
 def ring_locate_static(ranks, state, progress=None, device: int = 0, stream=None, roots_cap: int = STATIC_MAX_MEMBERS):
@@ -433,12 +465,29 @@ class Analyzer:
 
     def get_optable(self, window_id: int, to_host: bool = True) -> Dict[str, object]:
         """Per-op table of an analysed window; with to_host the columns come back as numpy arrays."""
+        if to_host:
+            h = HostOpTable()
+            rc = self.lib.ccld_take_optable(self.h, window_id, C.byref(h))
+            if rc == OK:
+                t, first = h.t, h.block.p
+                G, S = t.n_groups, t.n_slots
+                buf = np.asarray(_Pinned(h.block))
+                out: Dict[str, object] = {"n_groups": G, "n_slots": S}
+                for k, dt in _TABLE_DTYPES:
+                    out[k] = np.frombuffer(buf, dt, G, getattr(t, k) - first) if G else np.empty(0, dt)
+                for k, dt in (("flags", np.uint8), ("perm", np.uint32)):
+                    out[k] = np.frombuffer(buf, dt, S, getattr(t, k) - first) if S else np.empty(0, dt)
+                for k, dt in (("comm", np.uint32), ("seq", np.uint32), ("slot0", np.uint64)):
+                    out[k] = np.frombuffer(buf, dt, G, getattr(h, k) - first) if G else np.empty(0, dt)
+                return out
+            if rc not in _NO_BLOCK:
+                self._check(rc)
         t = OpTable()
         self._check(self.lib.ccld_get_optable(self.h, window_id, C.byref(t)))
         G, S = int(t.n_groups), int(t.n_slots)
         if not to_host:
             return {k: getattr(t, k) for k, _ in OpTable._fields_}
-        out: Dict[str, object] = {"n_groups": G, "n_slots": S}
+        out = {"n_groups": G, "n_slots": S}
         cols = [(k, G, np.int64) for k in OPTABLE_I64] + [(k, G, np.uint32) for k in OPTABLE_U32] + [("busbw", G, np.float64), ("flags", S, np.uint8), ("perm", S, np.uint32)]
         for (k, _, _), a in zip(cols, self._to_host([(getattr(t, k), n, dt) for k, n, dt in cols])):
             out[k] = a
@@ -479,6 +528,15 @@ class Analyzer:
         return out_s, out_r
 
     def get_rank_stats(self, n_ranks: int) -> Dict[str, np.ndarray]:
+        h = HostRankStats()
+        rc = self.lib.ccld_take_rank_stats(self.h, n_ranks, C.byref(h))
+        if rc == OK:
+            buf, first = np.asarray(_Pinned(h.block)), h.block.p
+            return {"votes": np.frombuffer(buf, np.uint32, n_ranks * 4, h.votes - first).reshape(n_ranks, 4),
+                    "ops": np.frombuffer(buf, np.uint32, n_ranks, h.ops - first), "bw_cnt": np.frombuffer(buf, np.uint32, n_ranks, h.bw_cnt - first),
+                    "bw_sum": np.frombuffer(buf, np.float64, n_ranks, h.bw_sum - first)}
+        if rc not in _NO_BLOCK:
+            self._check(rc)
         votes = np.empty((n_ranks, 4), np.uint32); ops = np.empty(n_ranks, np.uint32)
         cnt = np.empty(n_ranks, np.uint32); bw = np.empty(n_ranks, np.float64)
         self._check(self.lib.ccld_get_rank_stats(self.h, n_ranks, votes.ctypes.data, ops.ctypes.data, cnt.ctypes.data, bw.ctypes.data))

@@ -63,12 +63,19 @@ class BlockStore {
     held_[device] += b.bytes; lists_[device].push_back(b);
   }
   void clear() { std::lock_guard<std::mutex> g(m_); drain(); }
+  // Pinned blocks that callers keep (ccld_host_block): at most LENT_MOST bytes at a time.
+  bool lend(size_t bytes) { std::lock_guard<std::mutex> g(m_); if (lent_ + bytes > LENT_MOST) return false; lent_ += bytes; return true; }
+  void give_back(Block b, size_t lent) {
+    bool used;
+    { std::lock_guard<std::mutex> g(m_); lent_ -= lent; used = users_ > 0; }
+    if (used) put(-1, b); else if (b.p) free_block(-1, b);
+  }
 
  private:
-  static constexpr size_t PINNED_MOST = 64u << 20, DEVICE_MOST = 512u << 20;
+  static constexpr size_t PINNED_MOST = 64u << 20, DEVICE_MOST = 512u << 20, LENT_MOST = 64u << 20;
   static void free_block(int device, Block b) { if (device < 0) cudaFreeHost(b.p); else cudaFree(b.p); }   // (cudaFree takes any device's pointer)
   void drain() { for (auto& kv : lists_) { for (Block& b : kv.second) free_block(kv.first, b); kv.second.clear(); held_[kv.first] = 0; } }
-  std::mutex m_; int users_ = 0;
+  std::mutex m_; int users_ = 0; size_t lent_ = 0;
   std::map<int, std::vector<Block>> lists_; std::map<int, size_t> held_;
 };
 
@@ -379,27 +386,46 @@ int pinned_area(ccld_ctx* ctx, Block& area, size_t bytes) {
 // that is left to the driver's copies, whose fixed cost no longer counts.
 struct Piece { const void* src; void* dst; size_t n; };
 constexpr size_t FETCH_PINNED = 4u << 20;
+// Lays pieces out behind `off` in the pinned area at `base` (each as far from a 16-byte boundary as its source is) and launches
+// the kernel that copies them there; at[i] receives their offsets.
+cudaError_t gather(ccld_ctx* ctx, const Piece* piece, u32 n_pieces, char* base, size_t off, size_t* at) {
+  GatherArgs A; u32 k = 0; size_t most = 0;
+  for (u32 i = 0; i < n_pieces; ++i) {
+    at[i] = (off + 15) / 16 * 16 + ((uintptr_t)piece[i].src & 15);
+    off = at[i] + piece[i].n; most = std::max(most, piece[i].n);
+    if (piece[i].n) { A.piece[k].src = (const unsigned char*)piece[i].src; A.piece[k].dst = (unsigned char*)base + at[i]; A.piece[k].n = piece[i].n; ++k; }
+  }
+  if (k) k_gather<<<dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), k), GATHER_THREADS, 0, ctx->stream>>>(A);
+  return cudaGetLastError();
+}
+size_t gather_room(const Piece* piece, u32 n_pieces) { size_t t = 0; for (u32 i = 0; i < n_pieces; ++i) t += piece[i].n + 32; return t; }
+
 int fetch(ccld_ctx* ctx, const Piece* piece, u32 n_pieces) {
-  size_t total = 0, most = 0;
-  for (u32 i = 0; i < n_pieces; ++i) { total += piece[i].n; most = std::max(most, piece[i].n); }
+  size_t total = 0;
+  for (u32 i = 0; i < n_pieces; ++i) total += piece[i].n;
   if (total > FETCH_PINNED || n_pieces > GATHER_PIECES) {
     for (u32 i = 0; i < n_pieces; ++i) if (piece[i].n) CK(cudaMemcpyAsync(piece[i].dst, piece[i].src, piece[i].n, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     return CCLD_OK;
   }
-  if (total == 0) { CK(cudaStreamSynchronize(ctx->stream)); return CCLD_OK; }
-  { int rc = pinned_area(ctx, ctx->h_io, total + 32ull * n_pieces); if (rc != CCLD_OK) return rc; }
-  GatherArgs A; size_t at[GATHER_PIECES], off = 0; u32 k = 0;
-  unsigned char* base = (unsigned char*)ctx->h_io.p;
-  for (u32 i = 0; i < n_pieces; ++i) {
-    at[i] = (off + 15) / 16 * 16 + ((uintptr_t)piece[i].src & 15);
-    off = at[i] + piece[i].n;
-    if (piece[i].n) { A.piece[k].src = (const unsigned char*)piece[i].src; A.piece[k].dst = base + at[i]; A.piece[k].n = piece[i].n; ++k; }
-  }
-  k_gather<<<dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), k), GATHER_THREADS, 0, ctx->stream>>>(A);
-  CK(cudaGetLastError());
+  { int rc = pinned_area(ctx, ctx->h_io, gather_room(piece, n_pieces)); if (rc != CCLD_OK) return rc; }
+  size_t at[GATHER_PIECES];
+  char* base = (char*)ctx->h_io.p;
+  CK(gather(ctx, piece, n_pieces, base, 0, at));
   CK(cudaStreamSynchronize(ctx->stream));
   for (u32 i = 0; i < n_pieces; ++i) if (piece[i].n) std::memcpy(piece[i].dst, base + at[i], piece[i].n);
+  return CCLD_OK;
+}
+
+// A pinned block for the caller to keep, if it is not too large and not too much is out already.
+constexpr size_t TAKE_MOST = 16u << 20;
+int take_block(ccld_ctx* ctx, size_t bytes, ccld_host_block* blk) {
+  blk->p = nullptr; blk->bytes = 0;
+  if (bytes > TAKE_MOST) return fail(ctx, CCLD_ERR_CAPACITY, "too large for a pinned block");
+  Block b = pinned_get(ctx, bytes);
+  if (!b.p) return fail(ctx, CCLD_ERR_NOMEM, "pinned allocation failed");
+  if (!BlockStore::get().lend(b.bytes)) { ctx->pinned_free.push_back(b); return fail(ctx, CCLD_ERR_CAPACITY, "too many pinned blocks in use"); }
+  blk->p = b.p; blk->bytes = b.bytes;
   return CCLD_OK;
 }
 
@@ -1146,6 +1172,63 @@ int ccld_get_ranges(ccld_ctx* ctx, uint32_t window_id, ccld_comm_range* rows, ui
     ++k;
   }
   *n_total = k;
+  return CCLD_OK;
+}
+
+void ccld_host_release(ccld_host_block* blk) {
+  if (!blk || !blk->p) return;
+  Block b; b.p = blk->p; b.bytes = blk->bytes;
+  BlockStore::get().give_back(b, b.bytes);
+  blk->p = nullptr; blk->bytes = 0;
+}
+
+int ccld_take_optable(ccld_ctx* ctx, uint32_t window_id, ccld_host_optable* out) {
+  NvtxRange nvtx_range("ccld_take_optable");
+  if (!ctx || !out) return CCLD_ERR_ARG;
+  std::memset(out, 0, sizeof *out);
+  WindowHost* w;
+  { int rc = find_analysed(ctx, window_id, &w); if (rc != CCLD_OK) return rc; }
+  CK(cudaSetDevice(ctx->device));
+  const WinDesc& d = w->d; const u64 G = d.n_groups, S = d.n_slots;
+  // the table's columns follow each other on the device, so five pieces make it up; the key columns are written beside them
+  const Piece pc[5] = {{d.gi64, nullptr, G * 8 * GI_COUNT}, {d.gu32, nullptr, G * 4 * GU_COUNT}, {d.gbw, nullptr, G * 8}, {d.flags, nullptr, S}, {d.perm, nullptr, S * 4}};
+  const size_t keys = G * 16;
+  if (S > TAKE_MOST || G > TAKE_MOST) return fail(ctx, CCLD_ERR_CAPACITY, "too large for a pinned block");
+  { int rc = take_block(ctx, align_up(keys) + gather_room(pc, 5), &out->block); if (rc != CCLD_OK) return rc; }
+  char* base = (char*)out->block.p; size_t at[5];
+  u64* slot0 = (u64*)base; u32* comm = (u32*)(slot0 + G); u32* seq = comm + G;
+  cudaError_t e = cudaSuccess;
+  if (G) { k_op_keys<<<(u32)((G + 255) / 256), 256, 0, ctx->stream>>>(d.ranges, ctx->reg, G, comm, seq, slot0); e = cudaGetLastError(); }
+  if (e == cudaSuccess) e = gather(ctx, pc, 5, base, align_up(keys), at);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  if (e != cudaSuccess) { cudaStreamSynchronize(ctx->stream); ccld_host_release(&out->block); return fail(ctx, CCLD_ERR_CUDA, std::string("table copy: ") + cudaGetErrorString(e)); }
+  ccld_optable& t = out->t;
+  const i64* gi = (const i64*)(base + at[0]); const u32* gu = (const u32*)(base + at[1]);
+  t.n_groups = G; t.n_slots = S;
+  t.e_min = gi + GI_E_MIN * G; t.arrival_skew = gi + GI_ARRIVAL_SKEW * G; t.t_max = gi + GI_T_MAX * G; t.t_min = gi + GI_T_MIN * G; t.span = gi + GI_SPAN * G;
+  t.med_skew = gi + GI_MED_SKEW * G; t.mad_skew = gi + GI_MAD_SKEW * G; t.med_dur = gi + GI_MED_DUR * G; t.mad_dur = gi + GI_MAD_DUR * G;
+  t.rank_tmin = gu + GU_RANK_TMIN * G; t.rank_tmax = gu + GU_RANK_TMAX * G; t.max_chg = gu + GU_MAX_CHG * G;
+  t.rank_max_chg = gu + GU_RANK_MAX_CHG * G; t.n_present = gu + GU_N_PRESENT * G; t.gflags = gu + GU_GFLAGS * G;
+  t.busbw = (const double*)(base + at[2]); t.flags = (const u8*)(base + at[3]); t.perm = (const u32*)(base + at[4]);
+  out->comm = comm; out->seq = seq; out->slot0 = slot0;
+  return CCLD_OK;
+}
+
+int ccld_take_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, ccld_host_rank_stats* out) {
+  if (!ctx || !out) return CCLD_ERR_ARG;
+  std::memset(out, 0, sizeof *out);
+  if (!ctx->finalized) return fail(ctx, CCLD_ERR_STATE, "nothing analysed yet");
+  if (n_ranks > ctx->reg.n_ranks) return fail(ctx, CCLD_ERR_CAPACITY, "more ranks than the registry knows");
+  { int rc = settle(ctx); if (rc != CCLD_OK) return rc; }
+  CK(cudaSetDevice(ctx->device));
+  const size_t n = n_ranks;
+  const Piece pc[4] = {{ctx->reg.votes, nullptr, n * 16}, {ctx->reg.ops, nullptr, n * 4}, {ctx->reg.bw_cnt, nullptr, n * 4}, {ctx->reg.bw_sum, nullptr, n * 8}};
+  { int rc = take_block(ctx, gather_room(pc, 4), &out->block); if (rc != CCLD_OK) return rc; }
+  char* base = (char*)out->block.p; size_t at[4];
+  cudaError_t e = gather(ctx, pc, 4, base, 0, at);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  if (e != cudaSuccess) { cudaStreamSynchronize(ctx->stream); ccld_host_release(&out->block); return fail(ctx, CCLD_ERR_CUDA, std::string("statistics copy: ") + cudaGetErrorString(e)); }
+  out->votes = (const u32*)(base + at[0]); out->ops = (const u32*)(base + at[1]); out->bw_cnt = (const u32*)(base + at[2]); out->bw_sum = (const double*)(base + at[3]);
   return CCLD_OK;
 }
 

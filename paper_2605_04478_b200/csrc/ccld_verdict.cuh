@@ -223,6 +223,17 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(GatherArgs A) {
   if (i0 < n - tail) dst[tail + i0] = src[tail + i0];
 }
 
+// communicator id, op counter and first slot of every group of a window
+__global__ void __launch_bounds__(256) k_op_keys(const RangeRow* __restrict__ ranges, Registry R, u64 n_groups, u32* __restrict__ comm, u32* __restrict__ seq, u64* __restrict__ slot0) {
+  const u64 g = (u64)blockIdx.x * 256 + threadIdx.x;
+  if (g >= n_groups) return;
+  u32 lo = 0, hi = R.n_comms - 1;                              // owner: the last communicator whose first group is <= g
+  while (lo < hi) { const u32 mid = (lo + hi + 1) >> 1; if (ranges[mid].group0 <= g) lo = mid; else hi = mid - 1; }
+  const RangeRow row = ranges[lo];
+  const u32 k = (u32)(g - row.group0);
+  comm[g] = R.comm_id[lo]; seq[g] = row.seq_lo + k; slot0[g] = row.slot0 + (u64)k * row.n;
+}
+
 // the ordered alerts alone, for the hang sweep
 __global__ void __launch_bounds__(VD_THREADS) k_order_alerts(const u64* __restrict__ counters, const ccld_hang_alert* __restrict__ in, ccld_hang_alert* __restrict__ out, Registry R) {
   __shared__ u64 s_key[CCLD_MAX_ALERTS_PER_WINDOW];
