@@ -38,6 +38,13 @@ constexpr int LG_KEYS = 16;            //   (member, group) pairs a thread of th
 constexpr int LS_THREADS = 256;        //   staging kernel: a CTA takes LS_MEMBERS members of a tile
 constexpr int LS_MEMBERS = 512;
 
+// First thing in every kernel: what the kernel before it in the stream wrote is visible from here on, and the next one may be
+// brought to the SMs.
+__device__ __forceinline__ void begin_after() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 struct Params {
   i64 tbase_init_ns, m_max_ns, hang_ns;
   u64 barrier_bytes;

@@ -690,6 +690,7 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
 
 __global__ void __launch_bounds__(SMALL_SEQS, CCLD_FUSED_MIN_CTAS) k_reduce_fused(const WinDesc* __restrict__ wd, const FusedCta* __restrict__ ctas,
     const WarpTile* __restrict__ wts, TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
+  begin_after();
   __shared__ FusedShared sh;
   const FusedCta t = ctas[blockIdx.x];
   const WinDesc& D = wd[t.w];
@@ -742,6 +743,7 @@ __device__ __forceinline__ u64 rank_select(const u64 (&x)[DEF_Q], u32 n, u32 k, 
 }
 
 __global__ void __launch_bounds__(DEF_WARPS * 32) k_reduce_deferred(const WinDesc* __restrict__ wd, DeferList DL, Registry R, Params P, i64 now) {
+  begin_after();
   __shared__ u64 s_key[DEF_WARPS][WARP_N];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   u64* key = s_key[wid];

@@ -175,6 +175,7 @@ __device__ __forceinline__ void hang_locate_cta(const WinDesc& D, const Registry
 }
 
 __global__ void __launch_bounds__(HANG_THREADS) k_hang_locate(const WinDesc* __restrict__ wd, Registry R, HangArgs A) {
+  begin_after();
   const WinDesc& D = wd[0];
   if (A.alerts == nullptr) { hang_locate_cta(D, R, A, A.c, A.seq, 0); return; }
   // every alert of the window

@@ -12,6 +12,7 @@
 #include <string>
 #include <thread>
 #include <unordered_map>
+#include <utility>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -211,6 +212,19 @@ struct TimedLaunch {                                     // a named range and, w
   ~TimedLaunch() { if (i >= 0) cudaEventRecord(s->b[i], st); }
 };
 
+// Every kernel of the library starts with begin_after(): it may be launched while the one before it in the stream still runs,
+// waits there until that one is done, and lets the next one be launched. A launch then costs its latency beside the kernel
+// before it instead of after it.
+template <class... P, class... A>
+void launch(cudaStream_t st, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);      // the caller looks at cudaGetLastError()
+}
+
 // Layout of the scratch block used by get_verdict and locate_hang.
 struct MiscLayout { size_t sus, keys, counts, done, alerts, total; };
 MiscLayout misc_layout(u32 n_ranks) {
@@ -395,7 +409,7 @@ cudaError_t gather(ccld_ctx* ctx, const Piece* piece, u32 n_pieces, char* base, 
     off = at[i] + piece[i].n; most = std::max(most, piece[i].n);
     if (piece[i].n) { A.piece[k].src = (const unsigned char*)piece[i].src; A.piece[k].dst = (unsigned char*)base + at[i]; A.piece[k].n = piece[i].n; ++k; }
   }
-  if (k) k_gather<<<dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), k), GATHER_THREADS, 0, ctx->stream>>>(A);
+  if (k) launch(ctx->stream, k_gather, dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), k), GATHER_THREADS, 0, A);
   return cudaGetLastError();
 }
 size_t gather_room(const Piece* piece, u32 n_pieces) { size_t t = 0; for (u32 i = 0; i < n_pieces; ++i) t += piece[i].n + 32; return t; }
@@ -805,15 +819,15 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     ba.desc_host = (const u32*)h_up; ba.desc = (u32*)(pbase + o_desc); ba.desc_words = up_bytes / 4;
     ba.rmin = (u32*)(pbase + o_rmin); ba.n_rmin = (u64)B * nc; ba.zero = (u32*)(pbase + o_zero); ba.n_zero = (o_zero_end - o_zero) / 4;
     const u64 most = std::max<u64>(std::max<u64>(ba.desc_words, ba.n_rmin), ba.n_zero);
-    k_begin<<<(u32)std::min<u64>((most + BEGIN_THREADS - 1) / BEGIN_THREADS, 2ull * ctx->n_sms), BEGIN_THREADS, 0, st>>>(ba);
+    launch(st, k_begin, (u32)std::min<u64>((most + BEGIN_THREADS - 1) / BEGIN_THREADS, 2ull * ctx->n_sms), BEGIN_THREADS, 0, ba);
     if (cta > 0) {
       // enough CTAs to fill the device several times over, then as many blocks per CTA as that leaves
       const u64 want = 32ull * ctx->n_sms;
       const u32 per = (u32)std::min<u64>(RANGE_BLOCKS_MAX, std::max<u64>(1, cta * B / want));
       TimedLaunch tl(ts, 0, st);
-      k_seq_range<<<dim3((u32)((cta + per - 1) / per), B), REC_THREADS, range_smem_bytes(nc), st>>>(d_desc, ctx->reg, per);
+      launch(st, k_seq_range, dim3((u32)((cta + per - 1) / per), B), REC_THREADS, range_smem_bytes(nc), d_desc, ctx->reg, per);
     }
-    { TimedLaunch tl(ts, 1, st); k_layout<<<dim3(1 + fill_ctas, B), LAYOUT_THREADS, 0, st>>>(d_desc, ctx->reg, fill_ctas != 0); }
+    { TimedLaunch tl(ts, 1, st); launch(st, k_layout, dim3(1 + fill_ctas, B), LAYOUT_THREADS, 0, d_desc, ctx->reg, fill_ctas != 0); }
     return cudaGetLastError();
   };
   const u64* tot = nullptr;                                // [B][T_COUNT] totals the results are sized from
@@ -882,24 +896,24 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     const u32 rank_ctas = std::min<u32>((2 * ctx->n_ranks + EMIT_THREADS - 1) / EMIT_THREADS, 2 * ctx->n_sms), comm_blocks = (nc + EMIT_THREADS - 1) / EMIT_THREADS,
               per_slice = (comm_blocks + EMIT_SLICES - 1) / EMIT_SLICES, slices = (comm_blocks + per_slice - 1) / per_slice;
     TimedLaunch tl(ts, 1, st);
-    k_emit<<<dim3(chunk_ctas * slices + rank_ctas, B), EMIT_THREADS, 0, st>>>(d_desc, ctx->reg, pl, chunk_ctas * slices, slices, per_slice);
+    launch(st, k_emit, dim3(chunk_ctas * slices + rank_ctas, B), EMIT_THREADS, 0, d_desc, ctx->reg, pl, chunk_ctas * slices, slices, per_slice);
   }
   if (cta > 0) {
     const u64 blocks = (cta * REC_PER_CTA + SCAT_PER_CTA - 1) / SCAT_PER_CTA;      // of the largest window
     const u32 per = (u32)std::min<u64>(SCAT_BLOCKS_MAX, std::max<u64>(1, blocks * B / (16ull * ctx->n_sms)));
     TimedLaunch tl(ts, 2, st);
-    k_slot_scatter<<<dim3((u32)((blocks + per - 1) / per), B), SCAT_THREADS, 0, st>>>(d_desc, ctx->reg, per);
+    launch(st, k_slot_scatter, dim3((u32)((blocks + per - 1) / per), B), SCAT_THREADS, 0, d_desc, ctx->reg, per);
   }
   if (n_list[B_FCTA]) {
     const DeferList dl{(u64*)(rbase + o_def), (u32*)(pbase + o_defn)};
     TimedLaunch tl(ts, 3, st);
-    k_reduce_fused<<<(u32)n_list[B_FCTA], SMALL_SEQS, 0, st>>>(d_desc, pl.fcta, pl.fwt, (TileSum*)(rbase + o_fsum), ctx->reg, ctx->dp, dl);
-    k_reduce_deferred<<<DEF_GRID, DEF_WARPS * 32, 0, st>>>(d_desc, dl, ctx->reg, ctx->dp, now_ns);
+    launch(st, k_reduce_fused, (u32)n_list[B_FCTA], SMALL_SEQS, 0, d_desc, pl.fcta, pl.fwt, (TileSum*)(rbase + o_fsum), ctx->reg, ctx->dp, dl);
+    launch(st, k_reduce_deferred, DEF_GRID, DEF_WARPS * 32, 0, d_desc, dl, ctx->reg, ctx->dp, now_ns);
   }
   const DeferList dl_big{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
   auto deferred_big = [&]() {
     const u32 n = std::max(std::max(ctx->max_mid_n[0], ctx->max_mid_n[1]), std::max(ctx->max_mid_n[2], ctx->max_large_n));
-    k_reduce_large_deferred<<<LARGE_DEF_GRID, LARGE_DEF_THREADS, 16ull * n, st>>>(d_desc, dl_big, ctx->reg, ctx->dp, now_ns);
+    launch(st, k_reduce_large_deferred, LARGE_DEF_GRID, LARGE_DEF_THREADS, 16ull * n, d_desc, dl_big, ctx->reg, ctx->dp, now_ns);
   };
   static_assert(MID_SEQS == LARGE_SEQS, "one list for the groups of both classes");
   if (n_list[B_T2]) {
@@ -907,26 +921,26 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     const u32 grid = (u32)n_list[B_T2]; TileSum* sums = (TileSum*)(rbase + o_s2);
     // one launch per padded size the registry has; a tile of another size ends at once
     const u32* m = ctx->max_mid_n;
-    if (m[0]) k_reduce_mid<8><<<grid, MID_THREADS, mid_smem_bytes(m[0]), st>>>(d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
-    if (m[1]) k_reduce_mid<16><<<grid, MID_THREADS, mid_smem_bytes(m[1]), st>>>(d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
-    if (m[2]) k_reduce_mid<32><<<grid, MID_THREADS, mid_smem_bytes(m[2]), st>>>(d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[0]) launch(st, k_reduce_mid<8>, grid, MID_THREADS, mid_smem_bytes(m[0]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[1]) launch(st, k_reduce_mid<16>, grid, MID_THREADS, mid_smem_bytes(m[1]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[2]) launch(st, k_reduce_mid<32>, grid, MID_THREADS, mid_smem_bytes(m[2]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
     if (!n_list[B_T3]) deferred_big();
   }
   if (n_list[B_T3]) {
     LargeGroup* lgrp = (LargeGroup*)(rbase + o_lgrp);
     TimedLaunch tl(ts, 5, st);
-    k_large_stage<<<dim3((u32)n_list[B_T3], (ctx->max_large_n + LS_MEMBERS - 1) / LS_MEMBERS), LS_THREADS, 0, st>>>(d_desc, pl.t3, lgrp, ctx->reg);
+    launch(st, k_large_stage, dim3((u32)n_list[B_T3], (ctx->max_large_n + LS_MEMBERS - 1) / LS_MEMBERS), LS_THREADS, 0, d_desc, pl.t3, lgrp, ctx->reg);
     const u32 grid = (u32)std::min<u64>(n_list[B_T3], 2ull * ctx->n_sms);      // persistent: two CTAs per SM take the tiles in turn
-    k_reduce_large<<<grid, LG_THREADS, ctx->large_smem, st>>>(d_desc, pl.t3, (u32)n_list[B_T3], lgrp, (TileSum*)(rbase + o_s3), ctx->reg, ctx->dp, dl_big);
+    launch(st, k_reduce_large, grid, LG_THREADS, ctx->large_smem, d_desc, pl.t3, (u32)n_list[B_T3], lgrp, (TileSum*)(rbase + o_s3), ctx->reg, ctx->dp, dl_big);
     deferred_big();
   }
   {
     TimedLaunch tl(ts, 6, st);
     const u32 ctas = (nc + WD_THREADS / 32 - 1) / (WD_THREADS / 32);
-    if (B > 1) k_window_rounds<<<dim3(ctas, B), WD_THREADS, 0, st>>>(d_desc, ctx->reg);
-    if (B > 1) k_window_decide<false><<<ctas, WD_THREADS, 0, st>>>(d_desc, B, ctx->reg, ctx->dp);
-    else k_window_decide<true><<<ctas, WD_THREADS, 0, st>>>(d_desc, B, ctx->reg, ctx->dp);      // one window: both stages in one launch
-    if (ctx->n_trees) k_tree_root_comm<<<dim3(ctx->n_trees, B), TREE_THREADS, 0, st>>>(d_desc, ctx->d_trees, ctx->reg);
+    if (B > 1) launch(st, k_window_rounds, dim3(ctas, B), WD_THREADS, 0, d_desc, ctx->reg);
+    if (B > 1) launch(st, k_window_decide<false>, ctas, WD_THREADS, 0, d_desc, B, ctx->reg, ctx->dp);
+    else launch(st, k_window_decide<true>, ctas, WD_THREADS, 0, d_desc, B, ctx->reg, ctx->dp);      // one window: both stages in one launch
+    if (ctx->n_trees) launch(st, k_tree_root_comm, dim3(ctx->n_trees, B), TREE_THREADS, 0, d_desc, ctx->d_trees, ctx->reg);
   }
   CK(cudaGetLastError());
   for (u32 k = 0; k < B; ++k) {
@@ -982,13 +996,13 @@ static int verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out, ccld_ve
     A.alerts_out = (ccld_hang_alert*)(hv + area.alerts);
     A.sus_host = (ccld_suspect*)(hv + area.suspects); A.sus_host_cap = area.sus_cap; A.sus_dev = (ccld_suspect*)(m + L.sus);
     const u32 pieces = (ctx->n_ranks + VD_THREADS - 1) / VD_THREADS;
-    k_verdict_collect<<<pieces + 1 + n_rows / VD_THREADS, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg, ctx->dp, pieces);
+    launch(ctx->stream, k_verdict_collect, pieces + 1 + n_rows / VD_THREADS, VD_THREADS, 0, A, ctx->reg, ctx->dp, pieces);
     // suspect lists keep their length from call to call, roughly: where the last one was long, the merge goes along at once
-    if (pieces > 1 && ctx->long_list) k_verdict_merge<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg);
+    if (pieces > 1 && ctx->long_list) launch(ctx->stream, k_verdict_merge, pieces, VD_THREADS, 0, A, ctx->reg);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(ctx->stream));
     if (!head->listed) {
-      k_verdict_merge<<<pieces, VD_THREADS, 0, ctx->stream>>>(A, ctx->reg);
+      launch(ctx->stream, k_verdict_merge, pieces, VD_THREADS, 0, A, ctx->reg);
       CK(cudaGetLastError());
       CK(cudaStreamSynchronize(ctx->stream));
     }
@@ -1066,7 +1080,7 @@ static int hang_run(ccld_ctx* ctx, const WindowHost* w, HangArgs& A, u32 ctas) {
     if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
     A.scratch = (unsigned char*)blk.p;
   }
-  k_hang_locate<<<ctas, HANG_THREADS, hang_smem(std::min<u32>(ctx->max_n, HANG_SMEM_N)), ctx->stream>>>(w->d_desc, ctx->reg, A);
+  launch(ctx->stream, k_hang_locate, ctas, HANG_THREADS, hang_smem(std::min<u32>(ctx->max_n, HANG_SMEM_N)), w->d_desc, ctx->reg, A);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   ctx->pool.put(blk);
@@ -1119,7 +1133,7 @@ int ccld_locate_hangs(ccld_ctx* ctx, uint32_t window_id, ccld_hang_alert* alerts
   { int rc = pinned_area(ctx, ctx->h_io, off); if (rc != CCLD_OK) return rc; }
   char* h = (char*)ctx->h_io.p;
   ccld_hang_alert* al = (ccld_hang_alert*)((char*)ctx->misc_blk.p + misc_layout(ctx->n_ranks).alerts);
-  k_order_alerts<<<1, VD_THREADS, 0, st>>>(w->d.counters, w->d.alerts, al, ctx->reg);
+  launch(st, k_order_alerts, 1, VD_THREADS, 0, w->d.counters, w->d.alerts, al, ctx->reg);
   HangArgs A; std::memset(&A, 0, sizeof A);
   A.alerts = al; A.counters = w->d.counters; A.cap = most; A.roots = (u32*)(h + o_roots); A.roots_cap = keep;
   A.out = (ccld_hang_verdict*)(h + o_out); A.alerts_out = (ccld_hang_alert*)(h + o_al); A.n_alerts_out = (u64*)(h + o_n);
@@ -1198,7 +1212,7 @@ int ccld_take_optable(ccld_ctx* ctx, uint32_t window_id, ccld_host_optable* out)
   char* base = (char*)out->block.p; size_t at[5];
   u64* slot0 = (u64*)base; u32* comm = (u32*)(slot0 + G); u32* seq = comm + G;
   cudaError_t e = cudaSuccess;
-  if (G) { k_op_keys<<<(u32)((G + 255) / 256), 256, 0, ctx->stream>>>(d.ranges, ctx->reg, G, comm, seq, slot0); e = cudaGetLastError(); }
+  if (G) { launch(ctx->stream, k_op_keys, (u32)((G + 255) / 256), 256, 0, d.ranges, ctx->reg, G, comm, seq, slot0); e = cudaGetLastError(); }
   if (e == cudaSuccess) e = gather(ctx, pc, 5, base, align_up(keys), at);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) { cudaStreamSynchronize(ctx->stream); ccld_host_release(&out->block); return fail(ctx, CCLD_ERR_CUDA, std::string("table copy: ") + cudaGetErrorString(e)); }
@@ -1280,7 +1294,7 @@ int ccld_opset_check(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t 
   char* h = (char*)ctx->h_io.p;
   OpsetArgs A; A.c = ci->second; A.seq = seq; A.algo = w->algo; A.proto = w->proto;
   A.ranks = (u32*)(h + o_rk); A.ranks_cap = keep; A.out = (ccld_opset_verdict*)h;
-  k_opset_check<<<1, OPSET_THREADS, (size_t)n * OPSET_MEMBER_BYTES, ctx->stream>>>(w->d_desc, ctx->reg, A);
+  launch(ctx->stream, k_opset_check, 1, OPSET_THREADS, (size_t)n * OPSET_MEMBER_BYTES, w->d_desc, ctx->reg, A);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(ctx->stream));
   std::memcpy(out, h, sizeof *out); out->ranks = ranks; out->ranks_cap = cap;
@@ -1363,9 +1377,9 @@ int ccld_derive_rates(ccld_ctx* ctx, uint64_t n_rec, const uint32_t* rank, const
   // rank's samples cover a few tiles (8 tiles = 16 s at a sample per millisecond); with longer segments an op in flight
   // since their beginning would add up many, and the scan (5 to 15 us) pays.
   A.scanned = n_tiles > 256 && n_tiles > 8ull * n_ranks;
-  k_tick_blocks<<<(u32)(n_tiles + ((u64)n_ranks + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, st>>>(A);
-  if (A.scanned) k_tile_scan<<<1, TS_THREADS, 0, st>>>(A.tile, A.n_tiles);
-  k_record_rates<<<(u32)((n_rec + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, st>>>(A, n_rec, rank, t_enter_ns, t_exit_ns, send_chg, recv_chg);
+  launch(st, k_tick_blocks, (u32)(n_tiles + ((u64)n_ranks + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, A);
+  if (A.scanned) launch(st, k_tile_scan, 1, TS_THREADS, 0, A.tile, A.n_tiles);
+  launch(st, k_record_rates, (u32)((n_rec + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, A, n_rec, rank, t_enter_ns, t_exit_ns, send_chg, recv_chg);
   const cudaError_t le = cudaGetLastError();
   ctx->pool.put(blk);           // later work on this stream runs after these kernels: the block can be handed out again
   if (le != cudaSuccess) return fail(ctx, CCLD_ERR_CUDA, std::string("rate kernels: ") + cudaGetErrorString(le));

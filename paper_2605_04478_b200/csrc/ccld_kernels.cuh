@@ -167,6 +167,7 @@ __device__ __forceinline__ u32 first_left(const u32 (&cid)[REC_RUN], u32 left) {
 }
 
 __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* __restrict__ wd, Registry R, u32 blocks_per_cta) {
+  begin_after();
   extern __shared__ u32 s_dyn[];
   u32* const s_mn = R.n_comms <= RANGE_DIRECT ? s_dyn : nullptr;
   u32* const s_mx = R.n_comms <= RANGE_DIRECT ? s_dyn + R.n_comms : nullptr;
@@ -344,6 +345,7 @@ constexpr u32 SCAT_LOCAL = 8;     // ranks, counted from the rank of the CTA's f
 // fewer than 2^32 slots, only 32-bit arithmetic. Any other record (another rank, a communicator beyond the inline pairs,
 // a counter outside the range, a rejected record) takes the two dependent table loads and the full checks.
 __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc* __restrict__ wd, Registry R, u32 blocks_per_cta) {
+  begin_after();
   // (communicator id, counters covered, first counter, first slot) per resolved pair; counters covered 0: unused. Every
   // warp keeps its own copy, so no warp waits for another; two copies, because the entries of the next block are written
   // while lanes may still read those of the current one.
@@ -515,6 +517,7 @@ __device__ __forceinline__ void count_ops(const Registry& R, u32 c0, const u32* 
 
 // Stage 1 of a batch of several windows, all at once: leaves the part above in the communicator's verdict row.
 __global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* __restrict__ wd, Registry R) {
+  begin_after();
   __shared__ u32 s_an[WD_THREADS / 32];
   const u32 c0 = blockIdx.x * (WD_THREADS / 32), wid = threadIdx.x >> 5, c = c0 + wid, lane = threadIdx.x & 31;
   const WinDesc& D = wd[blockIdx.y];
@@ -539,6 +542,7 @@ __global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* __r
 // arithmetic only. SINGLE: a batch of one window, stage 1 is done here too.
 template <bool SINGLE>
 __global__ void __launch_bounds__(WD_THREADS) k_window_decide(const WinDesc* __restrict__ wd, u32 nw, Registry R, Params P) {
+  begin_after();
   __shared__ u32 s_an[WD_THREADS / 32];
   const u32 c0 = blockIdx.x * (WD_THREADS / 32), wid = threadIdx.x >> 5, c = c0 + wid, lane = threadIdx.x & 31;
   u32 n_an = 0;

@@ -33,6 +33,7 @@ struct LargeScal { u64 ts, td; double bn, den; u32 emin, tmn, ms, md; u32 state,
 constexpr u32 LS_PITCH = LS_MEMBERS + 4;     // lanes (op counter 0..7, member 0..3) hit 32 distinct banks
 
 __global__ void __launch_bounds__(LS_THREADS, 4) k_large_stage(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles, LargeGroup* __restrict__ grp, Registry R) {
+  begin_after();
   __shared__ u32 s_a[LARGE_SEQS * LS_PITCH], s_d[LARGE_SEQS * LS_PITCH];
   __shared__ LargeGroup s_part[LS_THREADS / 32][LARGE_SEQS];
   const Tile t = tiles[blockIdx.x];
@@ -183,6 +184,7 @@ inline size_t large_smem(u32 max_n) { return (size_t)8 * large_npad(max_n); }
 __global__ void __launch_bounds__(LG_THREADS, 2) k_reduce_large(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles, u32 n_tiles,
                                                                  const LargeGroup* __restrict__ grp, TileSum* __restrict__ sums,
                                                                  Registry R, Params P, DeferList DL) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* s_bw = (double*)smem_raw;
   __shared__ u32 s_hist[LARGE_SEQS * LG_BINS];
@@ -415,6 +417,7 @@ __device__ u64 radix_select(F key, u32 n, u32 k, u64 max_key, u32* hist /*[256]*
 }
 
 __global__ void __launch_bounds__(LARGE_DEF_THREADS) k_reduce_large_deferred(const WinDesc* __restrict__ wd, DeferList DL, Registry R, Params P, i64 now) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ u64 s_red64[32];
   __shared__ u32 s_red32[32];

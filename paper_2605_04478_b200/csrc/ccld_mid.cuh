@@ -111,6 +111,7 @@ __device__ __forceinline__ MidPart mid_shfl_xor(const MidPart& a, int h) {
 template <int R>
 __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles,
     TileSum* __restrict__ sums, Registry R_, Params P, DeferList DL) {
+  begin_after();
   extern __shared__ __align__(16) u32 mid_keys[];
   __shared__ MidPart s_part[MID_WARPS][MID_SEQS];
   __shared__ u64 s_base[MID_SEQS], s_gby[MID_SEQS];

@@ -24,6 +24,7 @@ struct OpsetArgs {
 };
 
 __global__ void __launch_bounds__(OPSET_THREADS) k_opset_check(const WinDesc* __restrict__ wd, Registry R, OpsetArgs A) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char opset_smem[];
   constexpr u32 PRESENT = 0x80000000u, COUNTED = 0x40000000u, TUPLE = 0xFFFFFFu;
   __shared__ u32 s_cnt[3], s_next[3], s_red32[32], s_present;

@@ -31,6 +31,7 @@ struct BeginArgs {
 };
 
 __global__ void __launch_bounds__(BEGIN_THREADS) k_begin(BeginArgs A) {
+  begin_after();
   const u64 i0 = (u64)blockIdx.x * BEGIN_THREADS + threadIdx.x, st = (u64)gridDim.x * BEGIN_THREADS;
   for (u64 i = i0; i < A.desc_words; i += st) A.desc[i] = A.desc_host[i];
   for (u64 i = i0; i < A.n_rmin; i += st) A.rmin[i] = NONE;
@@ -90,6 +91,7 @@ struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; u32* grp_w
 // (seen by k_emit) or in a later one - so that windows are never analysed out of order.
 // Grid: (1 + filling CTAs, windows). fill: whether the slot table (sized from the expectation) is to be set to NONE.
 __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __restrict__ wd, Registry R, int fill) {
+  begin_after();
   __shared__ PlanAcc s_warp[33];
   __shared__ u32 s_red[32];
   __shared__ u32 s_hist[2][CHUNK_MAX + 2];                     // differences along the chunks: warp-tiles of class 0, tiles of class 1
@@ -245,6 +247,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
 // chunk of any window of the batch. base[] of the descriptors is filled. A window that gave up fills its stretch of the
 // lists with entries that hold no work, because the kernels that follow are launched over the expected lengths.
 __global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict__ wd, Registry R, PlanLists L, u32 chunk_ctas, u32 slices, u32 blocks) {
+  begin_after();
   __shared__ uint4 s_pair[EMIT_THREADS / 32];
   const WinDesc& D = wd[blockIdx.y];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;

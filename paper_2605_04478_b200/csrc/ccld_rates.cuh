@@ -58,6 +58,7 @@ __device__ __forceinline__ u32 change_bits(const u32 (&v)[8], u32 before) {
 
 // Grid: n_tiles CTAs for the ticks, then one per RT_THREADS ranks.
 __global__ void __launch_bounds__(RT_THREADS) k_tick_blocks(TickArgs A) {
+  begin_after();
   __shared__ u32 s_cnt[RT_THREADS / 32];
   if (blockIdx.x >= A.n_tiles) {
     const u64 r = (u64)(blockIdx.x - A.n_tiles) * RT_THREADS + threadIdx.x;
@@ -105,6 +106,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_tick_blocks(TickArgs A) {
 constexpr int TS_THREADS = 1024;
 constexpr int TS_PER = 16;
 __global__ void __launch_bounds__(TS_THREADS) k_tile_scan(uint2* __restrict__ tile, u32 n_tiles) {
+  begin_after();
   __shared__ u64 s_warp[TS_THREADS / 32];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const auto pack = [](uint2 x) { return (u64)x.x | ((u64)x.y << 32); };          // fewer than 2^32 ticks: no carry into the upper half
@@ -168,6 +170,7 @@ __device__ __noinline__ u32 search_from(const i64* __restrict__ tn, u32 n, u32 g
 // every step issued for both before the next, took 58.7 us (58 registers), four 72.9.
 __global__ void __launch_bounds__(RT_THREADS) k_record_rates(TickArgs A, u64 n_rec, const u32* __restrict__ rank, const i64* __restrict__ t_enter,
                                                            const i64* __restrict__ t_exit, u32* __restrict__ send_chg, u32* __restrict__ recv_chg) {
+  begin_after();
   const u64 i = (u64)blockIdx.x * RT_THREADS + threadIdx.x;
   if (i >= n_rec) return;
   const u32 rk = __ldg(rank + i);

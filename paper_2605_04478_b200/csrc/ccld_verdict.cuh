@@ -77,6 +77,7 @@ __device__ __forceinline__ void order_alerts(const Registry& R, const ccld_hang_
 }
 
 __global__ void __launch_bounds__(VD_THREADS) k_verdict_collect(VerdictArgs A, Registry R, Params P, u32 pieces) {
+  begin_after();
   __shared__ u64 s_key[VD_KEYS];
   __shared__ u32 s_n;
   const u32 lane = threadIdx.x & 31;
@@ -181,6 +182,7 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_collect(VerdictArgs A, R
 }
 
 __global__ void __launch_bounds__(VD_THREADS) k_verdict_merge(VerdictArgs A, Registry R) {
+  begin_after();
   __shared__ u32 s_tot;
   if (threadIdx.x == 0) s_tot = 0;
   __syncthreads();
@@ -213,6 +215,7 @@ constexpr int GATHER_THREADS = 256;
 constexpr u32 GATHER_PIECES = 24;
 struct GatherArgs { struct { const unsigned char* src; unsigned char* dst; u64 n; } piece[GATHER_PIECES]; };
 __global__ void __launch_bounds__(GATHER_THREADS) k_gather(GatherArgs A) {
+  begin_after();
   const unsigned char* __restrict__ src = A.piece[blockIdx.y].src; unsigned char* __restrict__ dst = A.piece[blockIdx.y].dst;
   const u64 n = A.piece[blockIdx.y].n;
   const u64 head = min(n, (u64)((16 - ((uintptr_t)src & 15)) & 15)), n16 = (n - head) / 16, tail = head + n16 * 16;
@@ -225,6 +228,7 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(GatherArgs A) {
 
 // communicator id, op counter and first slot of every group of a window
 __global__ void __launch_bounds__(256) k_op_keys(const RangeRow* __restrict__ ranges, Registry R, u64 n_groups, u32* __restrict__ comm, u32* __restrict__ seq, u64* __restrict__ slot0) {
+  begin_after();
   const u64 g = (u64)blockIdx.x * 256 + threadIdx.x;
   if (g >= n_groups) return;
   u32 lo = 0, hi = R.n_comms - 1;                              // owner: the last communicator whose first group is <= g
@@ -236,6 +240,7 @@ __global__ void __launch_bounds__(256) k_op_keys(const RangeRow* __restrict__ ra
 
 // the ordered alerts alone, for the hang sweep
 __global__ void __launch_bounds__(VD_THREADS) k_order_alerts(const u64* __restrict__ counters, const ccld_hang_alert* __restrict__ in, ccld_hang_alert* __restrict__ out, Registry R) {
+  begin_after();
   __shared__ u64 s_key[CCLD_MAX_ALERTS_PER_WINDOW];
   const u64 n = counters[C_ALERTS];
   order_alerts(R, in, n < CCLD_MAX_ALERTS_PER_WINDOW ? (u32)n : CCLD_MAX_ALERTS_PER_WINDOW, out, false, s_key);
