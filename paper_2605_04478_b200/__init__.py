@@ -120,11 +120,18 @@ _NP_OF = {C.c_uint32: "u4", C.c_uint64: "u8", C.c_int64: "i8", C.c_double: "f8"}
 
 
 def _column_plan(struct):
-    """(name, dtype, bytes of an entry that lie before the column) per field, in field order; 64-bit columns come first."""
-    size = {k: np.dtype(_NP_OF[t]).itemsize for k, t in struct._fields_}
-    order = [k for k, _ in struct._fields_ if size[k] == 8] + [k for k, _ in struct._fields_ if size[k] == 4]
-    at = {k: sum(size[x] for x in order[:i]) for i, k in enumerate(order)}
-    return [(k, np.dtype(_NP_OF[t]), at[k]) for k, t in struct._fields_], sum(size.values())
+    """Field names in order, runs of equal types among the columns (64-bit ones first) as (names, dtype, bytes of an entry that
+    lie before the run), bytes of an entry, and the fields of an empty list."""
+    dt = {k: np.dtype(_NP_OF[t]) for k, t in struct._fields_}
+    order = [k for k in dt if dt[k].itemsize == 8] + [k for k in dt if dt[k].itemsize == 4]
+    runs, at = [], 0
+    for k in order:
+        if runs and runs[-1][1] == dt[k]:
+            runs[-1][0].append(k)
+        else:
+            runs.append(([k], dt[k], at))
+        at += dt[k].itemsize
+    return tuple(dt), runs, at, dt
 
 
 _ROW_PLAN, _ALERT_PLAN, _SUSPECT_PLAN = _column_plan(CommVerdict), _column_plan(HangAlert), _column_plan(Suspect)
@@ -190,6 +197,17 @@ def default_params() -> Params:
 
 _COL_DTYPES = {"rank": "int32", "comm": "int32", "seq": "int32", "op": "uint8", "bytes": "int64",
                "t_enter": "int64", "t_exit": "int64", "send_chg": "int32", "recv_chg": "int32"}
+
+
+_COLS = tuple((k, dt, np.dtype(dt).itemsize) for k, dt in _COL_DTYPES.items())
+
+
+def _address(a):
+    """Where a numpy array's data starts (ndarray.ctypes takes three times as long; it serves for read-only arrays)."""
+    try:
+        return C.addressof(C.c_char.from_buffer(a))
+    except TypeError:
+        return a.ctypes.data
 
 
 def _as_tensor(torch, v, dt):
@@ -316,30 +334,37 @@ class Analyzer:
     def trace_upload(self, window_id: int, cols, frames=None, n_channels: int = 0) -> None:
         """cols: dict of torch tensors or numpy arrays, all on the CPU (copied) or all on this GPU (borrowed)."""
         torch = self.torch
-        t, ptrs, cuda = {}, [], set()
-        for k, dt in _COL_DTYPES.items():
+        keep, ptrs, cuda, n = [], [], set(), 0
+        for k, dt, size in _COLS:
             v = cols.get(k)
             if v is None:
-                t[k] = None; ptrs.append(None)
+                ptrs.append(None)
                 continue
-            v = _as_tensor(torch, v, dt)
-            assert v.dtype is getattr(torch, dt), (k, v.dtype)
-            t[k] = v = v.contiguous()
-            cuda.add(v.is_cuda)
-            ptrs.append(v.data_ptr() if v.numel() else None)
+            if type(v) is np.ndarray and v.itemsize == size and v.flags.c_contiguous:      # the column's bits as they are
+                cuda.add(False)
+                m = v.size
+                ptrs.append(_address(v) if m else None)
+            else:
+                v = _as_tensor(torch, v, dt).contiguous()
+                assert v.dtype is getattr(torch, dt), (k, v.dtype)
+                cuda.add(v.is_cuda)
+                m = v.numel()
+                ptrs.append(v.data_ptr() if m else None)
+            keep.append(v)
+            if k == "rank":
+                n = m
         fr = {}
         if frames is not None:
             for k in ("f_rank", "f_comm", "f_seq", "progress"):
                 fr[k] = _as_tensor(torch, frames[k], "int32").contiguous()
                 cuda.add(fr[k].is_cuda)
         assert len(cuda) == 1, "all columns must live on the same device"
-        mem_kind = 1 if cuda.pop() else 0
-        n = int(t["rank"].numel())
-        ptr = lambda v: C.c_void_p(v.data_ptr()) if v is not None and v.numel() else C.c_void_p(0)
+        mem_kind = 1 if True in cuda else 0
+        ptr = lambda v: v.data_ptr() if v is not None and v.numel() else None
         nf = int(fr["f_rank"].numel()) if fr else 0
         rc = self.lib.ccld_trace_upload(self.h, window_id, n, mem_kind, *ptrs, nf, ptr(fr.get("f_rank")), ptr(fr.get("f_comm")), ptr(fr.get("f_seq")), n_channels, ptr(fr.get("progress")))
         self._check(rc)
-        self._keep[window_id] = [t, fr]            # borrowed device memory / pinned host memory stays alive
+        self._keep[window_id] = [keep, fr]         # borrowed device memory / pinned host memory stays alive
 
     def window_release(self, window_id: int) -> None:
         self._check(self.lib.ccld_window_release(self.h, window_id))
@@ -364,14 +389,15 @@ class Analyzer:
     @staticmethod
     def _take(ptr, n, cap, plan):
         """A list of n entries that the library holds column by column, as one array per field (the first `cap` entries)."""
-        fields, size = plan
+        names, runs, size, dtypes = plan
         if n == 0:
-            return {k: np.empty(0, dt) for k, dt, _ in fields}
+            return {k: np.empty(0, dt) for k, dt in dtypes.items()}
         buf = np.empty(n * size, np.uint8)
-        C.memmove(buf.ctypes.data, ptr, n * size)
-        if cap < n:
-            return {k: np.frombuffer(buf, dt, n, at * n)[:cap] for k, dt, at in fields}
-        return {k: np.frombuffer(buf, dt, n, at * n) for k, dt, at in fields}
+        C.memmove(_address(buf), ptr, n * size)
+        out = dict.fromkeys(names)
+        for keys, dt, at in runs:
+            out.update(zip(keys, np.frombuffer(buf, dt, len(keys) * n, at * n).reshape(len(keys), n)))
+        return out if cap >= n else {k: a[:cap] for k, a in out.items()}
 
     def _list_buf(self, struct, cap):
         """Room for `cap` entries of a C struct. Kept between calls: the library writes only the entries there are, and a fresh
