@@ -45,9 +45,6 @@ CSRC = os.path.join(ROOT, "paper_2605_04478_b200", "csrc")
 NCU_TRAFFIC = {
     "k_reduce_fused": {"bytes_per_record": (814.439936e6 + 275.335424e6) / 20.48e6, "files": ("ccld_fused.cuh",),
                        "sha16": "6183e6f855d461c0"},
-    # timed together: the staging pass, the select kernel and the (empty) deferred launch; capture on 5 cfg4w windows
-    "k_reduce_large": {"bytes_per_record": (761.179392e6 + 154.088192e6 + 167.293696e6 + 25.206016e6) / 20.48e6, "files": ("ccld_large.cuh",),
-                       "sha16": "caf65e7091f9eb36"},
 }
 
 MIXES = {"all": ((0, 0, 1, 0, 2), 200), "tp_pp": ((0, 0, 1, 0), 250), "dp": ((2,), 200)}   # op pattern (0 TP, 1 PP, 2 DP), repetitions
@@ -117,8 +114,6 @@ def algorithmic_bytes(kernel, recs, groups):
         return 8 * recs, 0                                     # communicator id and op counter
     if kernel == "k_slot_scatter":
         return 12 * recs, 4 * recs                             # three key columns read; the record index written per slot
-    if kernel == "k_reduce_large":                             # with its staging pass: 32-bit keys written once and read again
-        return (VAL_BYTES + FLAG_BYTES) * recs + ROW_BYTES * groups, (INDEX_BYTES + 16) * recs
     if kernel.startswith("k_reduce"):
         return (VAL_BYTES + FLAG_BYTES) * recs + ROW_BYTES * groups, INDEX_BYTES * recs
     return 0, 0
@@ -366,9 +361,8 @@ def measure(spec, order, steps, warmup, local_rank, world, sample_clocks):
                 "kernels_ms_per_step": {k: kt[k]["ms"] / steps for k in kt},
                 "whole_path": {"algorithmic_bytes_per_step": path_bytes, "achieved": path_gbs, "frac": path_gbs / peak}}
     # every launch of the fused reduce kernel is followed by one of k_reduce_deferred (timed inside the same event pair),
-    # k_reduce_large runs between k_large_stage and k_reduce_large_deferred, and every launch of k_window_decide is preceded by
-    # one of k_window_rounds
-    launches = (sum(x["launches"] for x in kt.values()) + kt["k_reduce_fused"]["launches"] + 2 * kt["k_reduce_large"]["launches"]
+    # k_reduce_large by k_reduce_large_deferred, and every launch of k_window_decide is preceded by one of k_window_rounds
+    launches = (sum(x["launches"] for x in kt.values()) + kt["k_reduce_fused"]["launches"] + kt["k_reduce_large"]["launches"]
                 + kt["k_window_decide"]["launches"])
     return {"n_rec": n_rec, "now": now, "ms_total": ms, "ms_per_step": ms / steps, "ms_best": min(per_step), "ms_median": statistics.median(per_step),
             "value": world * n_rec * steps / (ms * 1e-3), "value_best": world * n_rec / (min(per_step) * 1e-3),

@@ -31,12 +31,7 @@ constexpr int MID_ELEMS = 2048;        //   padded records per tile of a communi
 constexpr int MID_N = 1024;            // up to 1024 ranks: a warp per group, keys in its registers
 constexpr int MID_THREADS = 256;
 constexpr int MID_SEQS = 8;            //   op counters per tile
-constexpr int LARGE_SEQS = 8;          // above: tiles of up to 8 consecutive op counters (as many as fit shared memory), radix select
-constexpr int LG_THREADS = 512;
-constexpr int LG_WARPS = LG_THREADS / 32;
-constexpr int LG_KEYS = 16;            //   (member, group) pairs a thread of the kernel holds at most
-constexpr int LS_THREADS = 256;        //   staging kernel: a CTA takes LS_MEMBERS members of a tile
-constexpr int LS_MEMBERS = 512;
+constexpr int LARGE_SEQS = 8;          // above: a cluster of eight CTAs per tile of 8 consecutive op counters
 
 // First thing in every kernel: what the kernel before it in the stream wrote is visible from here on, and the next one may be
 // brought to the SMs.
@@ -99,9 +94,9 @@ enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS,
 constexpr u64 FAILED_CAPACITY = 1, FAILED_EXPECT = 2;      // T_FAILED: the window needs too many slots / its layout is not the expected one
 enum { B_FCTA = 0, B_FWT, B_FSUM, B_T2, B_T3, B_COUNT };
 
-struct Tile { u32 w, c, seq_off, count; };                 // classes 2 and 3: one CTA each; summary index = tile index
-// Work-list entries of the fused kernel carry a copy of the communicator's range row and member-list offset, so that a
+// Work-list entries carry a copy of the communicator's range row and member-list offset, so that a
 // tile needs no further lookups before its first gather.
+struct alignas(16) Tile { u32 w, c, seq_off, count; RangeRow row; u64 moff, pad; };      // classes 2 and 3: one CTA (a cluster) each; summary index = tile index
 struct alignas(16) WarpTile { u32 c, seq_off, count, sum_idx; RangeRow row; u64 moff; };      // class 0: up to 32 consecutive op counters of one communicator
 struct alignas(16) FusedCta { u32 w, cls, c, seq_off, count, sum_idx, wt_first, wt_count; RangeRow row; u64 moff; };   // class 0: wt_*; class 1: c .. sum_idx, row, moff
 
@@ -132,7 +127,6 @@ struct WinDesc {
   u64 n_groups, n_slots;
   u32* perm;                         // [n_slots]
   u8* flags;                         // [n_slots]
-  u32 *skey, *dkey;                  // [n_slots] staged 32-bit keys of the largest communicators (null when the batch has none)
   i64* gi64;                         // [9][n_groups]
   u32* gu32;                         // [6][n_groups]
   double* gbw;                       // [n_groups]
@@ -149,14 +143,6 @@ enum { GU_RANK_TMIN = 0, GU_RANK_TMAX, GU_MAX_CHG, GU_RANK_MAX_CHG, GU_N_PRESENT
 __host__ __device__ inline u32 next_pow2(u32 n) { u32 p = 1; while (p < n) p <<= 1; return p; }
 __host__ __device__ inline u32 comm_class(u32 n) { return n <= SMALL_N ? 0u : (n <= WARP_N ? 1u : (n <= MID_N ? 2u : 3u)); }
 __host__ __device__ inline u32 mid_npad(u32 n) { u32 p = next_pow2(n); return p < 32 ? 32 : p; }
-// Communicators of more than MID_N ranks: a tile is LARGE_SEQS consecutive op counters; the select kernel works on G of
-// them side by side, as many as let a thread keep its share of the keys (at most LG_KEYS) in registers.
-__host__ __device__ inline u32 large_npad(u32 n) { return (n + 31u) & ~31u; }
-__host__ __device__ inline u32 large_g(u32 n) {
-  u32 G = LARGE_SEQS;
-  while (G > 1 && (u64)G * large_npad(n) > (u64)LG_KEYS * LG_THREADS) G >>= 1;
-  return G;
-}
 // op counters per work unit: a warp-tile (class 0) or a CTA tile (classes 1 to 3)
 __host__ __device__ inline u32 tile_seqs(u32 n) {
   u32 c = comm_class(n);

@@ -150,8 +150,8 @@ struct TimerSlot { cudaEvent_t a[TIMER_PAIRS], b[TIMER_PAIRS]; int kind[TIMER_PA
 struct ccld_ctx {
   ccld_params params; Params dp; int device = 0; cudaStream_t stream = nullptr;
   std::vector<CommHost> comms; std::unordered_map<u32, u32> comm_idx;
-  bool finalized = false; u32 n_ranks = 0, max_n = 0, max_large_n = 0, max_mid_n[3] = {0, 0, 0};     // mid: of the communicators padded to 256, 512, 1024 
-  u64 sum_n = 0; size_t large_smem = 0; u32 n_sms = 148;
+  bool finalized = false; u32 n_ranks = 0, max_n = 0, max_large_n[3] = {0, 0, 0}, max_mid_n[3] = {0, 0, 0};     // largest communicators of up to 2048, 4096, 8192 and of up to 256, 512, 1024 ranks 
+  u64 sum_n = 0; u32 n_sms = 148;
   Block reg_blk, misc_blk; Registry reg; size_t stats_off = 0, stats_bytes = 0;
   const TreeRef* d_trees = nullptr; u32 n_trees = 0;     // tree communicators whose layers are known
   std::map<u32, WindowHost> windows;
@@ -216,13 +216,19 @@ struct TimedLaunch {                                     // a named range and, w
 // waits there until that one is done, and lets the next one be launched. A launch then costs its latency beside the kernel
 // before it instead of after it.
 template <class... P, class... A>
-void launch(cudaStream_t st, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+void launch_cluster(cudaStream_t st, void (*kernel)(P...), u32 cluster, dim3 grid, dim3 block, size_t smem, A&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension; at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
   cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);      // the caller looks at cudaGetLastError()
+}
+
+template <class... P, class... A>
+void launch(cudaStream_t st, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+  launch_cluster(st, kernel, 1, grid, block, smem, std::forward<A>(args)...);
 }
 
 // Layout of the scratch block used by get_verdict and locate_hang.
@@ -254,12 +260,12 @@ int finalize_registry(ccld_ctx* ctx) {
   if (ctx->finalized) return CCLD_OK;
   const u32 nc = (u32)ctx->comms.size();
   if (nc == 0) return fail(ctx, CCLD_ERR_STATE, "no communicator registered");
-  u32 max_rank = 0; u64 sum_n = 0; u32 max_n = 0, max_large = 0;
+  u32 max_rank = 0; u64 sum_n = 0; u32 max_n = 0;
   for (auto& c : ctx->comms) {
     for (u32 r : c.ranks) max_rank = std::max(max_rank, r);
     sum_n += c.ranks.size(); max_n = std::max<u32>(max_n, (u32)c.ranks.size());
     const u32 n = (u32)c.ranks.size(), cls = comm_class(n);
-    if (cls == 3) max_large = std::max<u32>(max_large, n);
+    if (cls == 3) { u32& m = ctx->max_large_n[n <= 2048 ? 0 : (n <= 4096 ? 1 : 2)]; m = std::max(m, n); }
     if (cls == 2) { u32& m = ctx->max_mid_n[n <= 256 ? 0 : (n <= 512 ? 1 : 2)]; m = std::max(m, n); }
   }
   const u32 nr = max_rank + 1;
@@ -345,7 +351,7 @@ int finalize_registry(ccld_ctx* ctx) {
   R.state = (CommState*)(base + o_state); R.votes = (u32*)(base + o_votes); R.ops = (u32*)(base + o_ops);
   R.bw_cnt = (u32*)(base + o_cnt); R.bw_sum = (double*)(base + o_bw);
   ctx->stats_off = o_stats; ctx->stats_bytes = stats_end - o_stats; ctx->d_poison = (u32*)(base + o_poison);
-  ctx->n_ranks = nr; ctx->max_n = max_n; ctx->max_large_n = max_large; ctx->sum_n = sum_n;
+  ctx->n_ranks = nr; ctx->max_n = max_n; ctx->sum_n = sum_n;
 
   // scratch for suspects, alert ordering and hang location
   ctx->misc_blk = ctx->pool.get(misc_layout(nr).total, &e);
@@ -359,10 +365,9 @@ int finalize_registry(ccld_ctx* ctx) {
   CK(cudaFuncSetAttribute(k_seq_range, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)range_smem_bytes(RANGE_DIRECT)));
   CK(cudaFuncSetAttribute(k_hang_locate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(HANG_SMEM_N * HANG_MEMBER_BYTES)));
   CK(cudaFuncSetAttribute(k_opset_check, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(CCLD_MAX_COMM_SIZE * OPSET_MEMBER_BYTES)));
-  if (max_large) {
-    ctx->large_smem = large_smem(max_large);
-    CK(cudaFuncSetAttribute(k_reduce_large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->large_smem));
-  }
+  CK(cudaFuncSetAttribute(k_reduce_large<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(4)));
+  CK(cudaFuncSetAttribute(k_reduce_large<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(8)));
+  CK(cudaFuncSetAttribute(k_reduce_large<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(16)));
   ctx->finalized = true;
   return CCLD_OK;
 }
@@ -804,7 +809,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     d.totals = (u64*)(pbase + o_tot) + (size_t)k * T_COUNT; d.counters = (u64*)(pbase + o_cnt) + (size_t)k * C_COUNT;
     d.chunks = (uint2*)(pbase + o_chunk) + (size_t)k * (CHUNK_MAX + 1); d.totals_host = (u64*)pbatch.pin.p + (size_t)k * T_COUNT;
     d.expect = expect ? (const u64*)(pbase + o_exp) + (size_t)k * T_COUNT : nullptr; d.poison = ctx->d_poison;
-    d.n_groups = d.n_slots = 0; d.perm = nullptr; d.flags = nullptr; d.skey = d.dkey = nullptr; d.gi64 = nullptr; d.gu32 = nullptr; d.gbw = nullptr;
+    d.n_groups = d.n_slots = 0; d.perm = nullptr; d.flags = nullptr; d.gi64 = nullptr; d.gu32 = nullptr; d.gbw = nullptr;
     d.comm_rows = nullptr; d.alerts = nullptr;
     for (int q = 0; q < B_COUNT; ++q) d.base[q] = 0;
     d.pad = 0; d.tsum[0] = d.tsum[1] = d.tsum[2] = nullptr;
@@ -864,9 +869,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   u64 total_groups = 0;
   for (u32 k = 0; k < B; ++k) total_groups += tot[(size_t)k * T_COUNT + T_GROUPS];
   const size_t o_def = take(n_list[B_FCTA] ? total_groups * 8 : 0),
-               o_def3 = take((n_list[B_T2] + n_list[B_T3]) * (size_t)LARGE_SEQS * 8),          // likewise for the kernels of larger communicators
-               o_lgrp = take(n_list[B_T3] * (size_t)LARGE_SEQS * sizeof(LargeGroup)),
-               o_skey = take(n_list[B_T3] ? total_slots * 4 : 0), o_dkey = take(n_list[B_T3] ? total_slots * 4 : 0);
+               o_def3 = take((n_list[B_T2] + n_list[B_T3]) * (size_t)LARGE_SEQS * 8);          // likewise for the kernels of larger communicators
   Block rb = ctx->pool.get(off, &e);
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "result allocation failed");
   auto res_blk = std::make_shared<Shared>(&ctx->pool, rb);
@@ -876,7 +879,6 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     WinDesc& d = hd[k];
     d.n_groups = t[T_GROUPS]; d.n_slots = t[T_SLOTS];
     d.perm = (u32*)(rbase + o_perm + perm_off[k]); d.flags = (u8*)(rbase + o_flags[k]);
-    if (n_list[B_T3]) { d.skey = (u32*)(rbase + o_skey + perm_off[k]); d.dkey = (u32*)(rbase + o_dkey + perm_off[k]); }
     d.gi64 = (i64*)(rbase + o_gi[k]); d.gu32 = (u32*)(rbase + o_gu[k]); d.gbw = (double*)(rbase + o_gb[k]);
     d.comm_rows = (ccld_comm_verdict*)(rbase + o_rows[k]); d.alerts = (ccld_hang_alert*)(rbase + o_al[k]);
     d.tsum[0] = (TileSum*)(rbase + o_fsum) + d.base[B_FSUM]; d.tsum[1] = (TileSum*)(rbase + o_s2) + d.base[B_T2]; d.tsum[2] = (TileSum*)(rbase + o_s3) + d.base[B_T3];
@@ -891,7 +893,6 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     if (total_slots) CK(cudaMemsetAsync(rbase + o_perm, 0xFF, total_slots * 4, st));
   }
   PlanLists pl; pl.fcta = (FusedCta*)(rbase + o_fcta); pl.fwt = (WarpTile*)(rbase + o_fwt); pl.t2 = (Tile*)(rbase + o_t2); pl.t3 = (Tile*)(rbase + o_t3);
-  pl.grp_words = (u32*)(rbase + o_lgrp); pl.grp_words_per_tile = LARGE_SEQS * sizeof(LargeGroup) / 4;
   {
     const u32 rank_ctas = std::min<u32>((2 * ctx->n_ranks + EMIT_THREADS - 1) / EMIT_THREADS, 2 * ctx->n_sms), comm_blocks = (nc + EMIT_THREADS - 1) / EMIT_THREADS,
               per_slice = (comm_blocks + EMIT_SLICES - 1) / EMIT_SLICES, slices = (comm_blocks + per_slice - 1) / per_slice;
@@ -912,7 +913,8 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   }
   const DeferList dl_big{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
   auto deferred_big = [&]() {
-    const u32 n = std::max(std::max(ctx->max_mid_n[0], ctx->max_mid_n[1]), std::max(ctx->max_mid_n[2], ctx->max_large_n));
+    u32 n = 0;
+    for (int q = 0; q < 3; ++q) n = std::max(n, std::max(ctx->max_mid_n[q], ctx->max_large_n[q]));
     launch(st, k_reduce_large_deferred, LARGE_DEF_GRID, LARGE_DEF_THREADS, 16ull * n, d_desc, dl_big, ctx->reg, ctx->dp, now_ns);
   };
   static_assert(MID_SEQS == LARGE_SEQS, "one list for the groups of both classes");
@@ -927,11 +929,12 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     if (!n_list[B_T3]) deferred_big();
   }
   if (n_list[B_T3]) {
-    LargeGroup* lgrp = (LargeGroup*)(rbase + o_lgrp);
     TimedLaunch tl(ts, 5, st);
-    launch(st, k_large_stage, dim3((u32)n_list[B_T3], (ctx->max_large_n + LS_MEMBERS - 1) / LS_MEMBERS), LS_THREADS, 0, d_desc, pl.t3, lgrp, ctx->reg);
-    const u32 grid = (u32)std::min<u64>(n_list[B_T3], 2ull * ctx->n_sms);      // persistent: two CTAs per SM take the tiles in turn
-    launch(st, k_reduce_large, grid, LG_THREADS, ctx->large_smem, d_desc, pl.t3, (u32)n_list[B_T3], lgrp, (TileSum*)(rbase + o_s3), ctx->reg, ctx->dp, dl_big);
+    const u32 grid = (u32)(n_list[B_T3] * LARGE_SEQS); TileSum* sums = (TileSum*)(rbase + o_s3);
+    const u32* m = ctx->max_large_n;
+    if (m[0]) launch_cluster(st, k_reduce_large<4>, LARGE_SEQS, grid, LQ_THREADS, large_smem(4), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[1]) launch_cluster(st, k_reduce_large<8>, LARGE_SEQS, grid, LQ_THREADS, large_smem(8), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[2]) launch_cluster(st, k_reduce_large<16>, LARGE_SEQS, grid, LQ_THREADS, large_smem(16), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
     deferred_big();
   }
   {

@@ -10,7 +10,7 @@
 //                   shuffle bitonic network); complete groups whose times fit 32-bit offsets
 //   k_reduce_deferred  the groups k_reduce_fused sets aside (incomplete, in flight, 64-bit spreads)
 //   k_reduce_mid    same, 129 <= n <= 1024 (ccld_mid.cuh: tiles of 8 op counters staged in shared memory, a warp per group)
-//   k_reduce_large  same, n > 1024 (ccld_large.cuh: a CTA per tile of 8 op counters, several groups side by side, radix select)
+//   k_reduce_large  same, n > 1024 (ccld_large.cuh: a cluster of eight CTAs per tile of 8 op counters)
 //   k_reduce_large_deferred  the groups k_reduce_mid and k_reduce_large set aside
 //   k_window_rounds Eq. 2 per (communicator, window): round counts, selected round, location candidates
 //   k_window_decide Eq. 1, 3, 4 per communicator, windows in order: baseline state, class, slow location

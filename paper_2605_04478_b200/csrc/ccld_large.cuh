@@ -1,345 +1,342 @@
-// Per-op reductions, median / MAD, flags and votes for communicators of more than 1,024 ranks (sm_100a).
+// Per-op reductions, median / MAD, flags and votes for communicators of more than 1,024 ranks (sm_100a). Included by
+// ccld_kernels.cuh.
 //
-// A group of thousands of members has its records spread over as many places of the upload, and its order statistics
-// need every key several times. The work is therefore cut in two:
+// A group of thousands of members has its records spread over as many places of the upload, and its order statistics need
+// every key several times. A cluster of eight CTAs takes a tile of LARGE_SEQS = 8 consecutive op counters of one communicator:
 //
-//   k_large_stage            one pass over the records of a tile (LARGE_SEQS consecutive op counters of one communicator,
-//                            LS_MEMBERS members per CTA). Lanes run along the op counter first: the eight record indices
-//                            of a member are one 32-byte sector of the member-major permutation, and in a rank-major
-//                            upload the eight records are neighbours too, so every gather of a warp fetches whole
-//                            sectors. Times become 32-bit keys (enter-time offset from the group's first member, duration)
-//                            and leave, transposed through shared memory, as two contiguous arrays per group; the extrema,
-//                            the op-set check and the rate column are reduced on the way and merged per group with atomics.
-//   k_reduce_large           the order statistics. A CTA works on G groups of a tile side by side (G = 8, 4, 2 or 1: a
-//                            thread keeps its share of a group's keys, at most LG_KEYS, in registers during a select);
-//                            every CTA-wide step runs once for all G groups, so a sub-tile costs the barriers of one
-//                            group. Keys are read from the staged arrays with coalesced loads; flags, votes and the
-//                            per-member bandwidth sums follow, the sums gathered in shared memory over all tiles a CTA
-//                            handles of one communicator and window (the grid is persistent).
-//   k_reduce_large_deferred  the groups that are not complete and 32-bit clean (a missing member, a record in flight,
-//                            invalid times, spreads beyond 32 bits): one CTA per listed group, 64-bit throughout, hang alerts.
+//   gather    CTA c takes an eighth of the members through all eight op counters. Lanes run along the op counter first: the
+//             eight record indices of a member are one 32-byte sector of the member-major permutation, and in a rank-major
+//             upload its eight records are neighbours too, so every gather of a warp fetches whole sectors. Times become 32-bit
+//             keys against the group's first member (enter-time offset, duration) in the CTA's shared memory; extrema, op-set
+//             check and rate column are reduced on the way.
+//   exchange  CTA j takes op counter j: its keys come out of the eight CTAs' shared memory (distributed shared memory, rows of
+//             consecutive members). The bandwidths of the CTA's members over the eight op counters are added up where they
+//             were gathered, so a member costs one atomic per tile; then the op counter's keys take the place of the tile.
+//   select    medians of both metrics side by side: a histogram of 2,048 bins from the largest key's highest bit down names the
+//             bin of the median, the few keys of that bin are put in a list, and a thread per listed key counts those before
+//             it; then the same for the deviations. Five barriers per median of both metrics.
+//
+// Groups that are not complete and 32-bit clean go to k_reduce_large_deferred (one CTA per listed group, 64-bit, hang alerts).
+//
+// Two kernels did this before: one wrote the keys to memory, the other read them twice and selected with 8-bit digits, every
+// key of a thread looked at in every pass (12 warp instructions per record): 2 x 1,000 groups of 4,096 took 90 + 195 us;
+// this kernel takes 241. A CTA lives 37 us, 14 of them in the gather (the CTAs of a wave gather at the same time, at the memory's
+// rate) and the rest in the barriers and round trips of the other steps.
 #pragma once
+#include <cooperative_groups.h>
 #include "ccld_device.cuh"
 
 namespace ccld {
 
-// What k_large_stage leaves per group; every field is a maximum (minima are stored complemented), so zero is the
-// neutral start. bits: 1 = some record disqualifies the group for the 32-bit path, 2 = the op set differs inside it.
-struct LargeGroup { u64 kmax, n_kmin, ck; u32 n_emin, emax, xmax, bits; };
-struct LargeLead { u64 brng; u32 bk, rounds, an, def, pad; };
-// per-group values the flag pass reads back from shared memory
-struct LargeScal { u64 ts, td; double bn, den; u32 emin, tmn, ms, md; u32 state, pad; };       // state: 1 group handled here, 2 analysed, 4 barrier
+constexpr int LQ_THREADS = 512, LQ_WARPS = LQ_THREADS / 32;
+constexpr u32 LQ_BITS = 11, LQ_BINS = 1u << LQ_BITS;       // bins of a histogram level
+constexpr u32 LQ_LIST = 256;                               // keys a bin may hold to be settled by counting
+constexpr u32 LQ_LEVELS = (32 + LQ_BITS - 1) / LQ_BITS;    // after that many levels no bit is undecided
+static_assert(LARGE_SEQS == 8 && LQ_WARPS == 16 && LQ_LIST == LQ_THREADS / 2, "a CTA of the cluster per op counter, eight warps per metric");
+// members of a CTA: at most 64 Q; the padding sets a row's lanes (op counter 0..7, member 0..3) on 32 different banks
+template <int Q> struct LargeTile { static constexpr u32 M = 64 * Q, PITCH = M + 4; };
+inline size_t large_smem(int q) { return (size_t)2 * LARGE_SEQS * (64 * q + 4) * 4; }
 
-constexpr u32 LS_PITCH = LS_MEMBERS + 4;     // lanes (op counter 0..7, member 0..3) hit 32 distinct banks
+struct LargePick { u32 lo, sh, k, cnt; };                  // the k-th of cnt keys in [lo, lo + 2^sh)
+struct LargeShared {
+  u32 hist[2][LQ_BINS];
+  uint4 list[2][LQ_LIST / 4];
+  MidPart part[LQ_WARPS][LARGE_SEQS], mine[LARGE_SEQS], group;
+  LargePick pick[LQ_LEVELS][2];                            // [level][metric]
+  u32 wsum[LQ_WARPS], n_list[2], res[2], n_fs, n_fd, ranks[3];
+  u64 gby[LARGE_SEQS]; i64 te0[LARGE_SEQS]; u32 gop[LARGE_SEQS];
+  u32 state[LARGE_SEQS], rng[LARGE_SEQS];                  // per op counter: 1 clean, 2 a round; range of durations
+  double bd[LARGE_SEQS];                                   // bytes * factor of an op counter that is a round, else 0
+};
 
-__global__ void __launch_bounds__(LS_THREADS, 4) k_large_stage(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles, LargeGroup* __restrict__ grp, Registry R) {
+// The k-th smallest (0-based) of |a[i] - ma| and of |d[i] - md| over the n keys in shared memory. ba, bd: the largest of them.
+// All threads call it; the histograms are zero on entry and on return.
+template <int Q> __device__ __forceinline__ void large_pick(const u32* __restrict__ s_a, const u32* __restrict__ s_d, u32 n, u32 ma, u32 md, u32 k, u32 ba, u32 bd,
+                                                            LargeShared& sh, u32* ra, u32* rd) {
+  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5, x = wid >> 3;             // eight warps scan a metric's bins
+  u32 lo0 = 0, lo1 = 0, w0 = 32 - (u32)__clz(ba | 1u), w1 = 32 - (u32)__clz(bd | 1u);  // undecided bits
+  u32 k0 = k, k1 = k, c0 = NONE, c1 = NONE;
+  for (u32 level = 0; level < LQ_LEVELS; ++level) {
+    const bool first = level == 0;
+    const bool act0 = first || (w0 > 0 && c0 > LQ_LIST), act1 = first || (w1 > 0 && c1 > LQ_LIST);
+    if (!act0 && !act1) break;                             // the same in every thread
+    const u32 n0 = w0 > LQ_BITS ? w0 - LQ_BITS : 0u, n1 = w1 > LQ_BITS ? w1 - LQ_BITS : 0u;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
+      if (i >= n) break;
+      const u32 a = __usad(s_a[i], ma, 0u) - lo0, d = __usad(s_d[i], md, 0u) - lo1;
+      if (act0 && (first || (a >> w0) == 0)) atomicAdd(&sh.hist[0][(a >> n0) & (LQ_BINS - 1)], 1u);      // (w < 32 after the first level)
+      if (act1 && (first || (d >> w1) == 0)) atomicAdd(&sh.hist[1][(d >> n1) & (LQ_BINS - 1)], 1u);
+    }
+    __syncthreads();
+    u32 loc[8], sum = 0;
+    uint4* h = reinterpret_cast<uint4*>(&sh.hist[x][(wid & 7) * 256 + lane * 8]);
+    { const uint4 a = h[0], b = h[1]; loc[0] = a.x; loc[1] = a.y; loc[2] = a.z; loc[3] = a.w; loc[4] = b.x; loc[5] = b.y; loc[6] = b.z; loc[7] = b.w; }
+    h[0] = make_uint4(0, 0, 0, 0); h[1] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sum += loc[q];
+    u32 inc = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { const u32 o = __shfl_up_sync(FULLM, inc, d); if (lane >= (u32)d) inc += o; }
+    // what this level leaves undecided for a metric that takes no part, and a defined value for one that does
+    if ((wid & 7) == 0 && lane == 0) sh.pick[level][x] = x ? LargePick{lo1, act1 ? 0u : w1, k1, c1} : LargePick{lo0, act0 ? 0u : w0, k0, c0};
+    if (lane == 31) sh.wsum[wid] = inc;
+    __syncthreads();
+    const u32 off = __reduce_add_sync(FULLM, lane < (wid & 7) ? sh.wsum[(wid & 8) + lane] : 0u);
+    const u32 kr = x ? k1 : k0, ex = off + inc - sum;
+    if ((x ? act1 : act0) && kr >= ex && kr < ex + sum) {
+      u32 cum = ex;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (kr >= cum && kr < cum + loc[q]) {
+          const u32 bin = (wid & 7) * 256 + lane * 8 + q, ns = x ? n1 : n0;
+          sh.pick[level][x] = LargePick{(x ? lo1 : lo0) + (bin << ns), ns, kr - cum, loc[q]};
+        }
+        cum += loc[q];
+      }
+    }
+    __syncthreads();
+    const LargePick p0 = sh.pick[level][0], p1 = sh.pick[level][1];
+    lo0 = p0.lo; w0 = p0.sh; k0 = p0.k; c0 = p0.cnt; lo1 = p1.lo; w1 = p1.sh; k1 = p1.k; c1 = p1.cnt;
+  }
+  if (w0 | w1) {
+    // the keys of the bins go into lists; a list's places beyond its end hold the largest key
+    u32* const l0 = reinterpret_cast<u32*>(sh.list[0]); u32* const l1 = reinterpret_cast<u32*>(sh.list[1]);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
+      if (i >= n) break;
+      const u32 a = __usad(s_a[i], ma, 0u) - lo0, d = __usad(s_d[i], md, 0u) - lo1;
+      if (w0 && (a >> w0) == 0) { const u32 at = atomicAdd(&sh.n_list[0], 1u); if (at < LQ_LIST) l0[at] = a; }    // c0 <= LQ_LIST of them
+      if (w1 && (d >> w1) == 0) { const u32 at = atomicAdd(&sh.n_list[1], 1u); if (at < LQ_LIST) l1[at] = d; }
+    }
+    __syncthreads();
+    {
+      // a thread per listed key counts those before it (ties by place); the key with k before it is the one
+      const u32 c = x ? c1 : c0, w = x ? w1 : w0, kr = x ? k1 : k0, i = (wid & 7) * 32 + lane, c4 = min((c + 3) / 4, LQ_LIST / 4);
+      if (w == 0) { if (i == 0) sh.res[x] = x ? lo1 : lo0; }
+      else if ((wid & 7) * 32 < c) {
+        const u32* l = x ? l1 : l0;
+        const u32 v = i < c ? l[i] : NONE;
+        u32 before = 0;
+#pragma unroll 4
+        for (u32 g = 0; g < c4; ++g) {
+          const uint4 y = sh.list[x][g];
+          const u32 j = 4 * g;
+          before += (y.x < v || (y.x == v && j < i)) ? 1u : 0u; before += (y.y < v || (y.y == v && j + 1 < i)) ? 1u : 0u;
+          before += (y.z < v || (y.z == v && j + 2 < i)) ? 1u : 0u; before += (y.w < v || (y.w == v && j + 3 < i)) ? 1u : 0u;
+        }
+        if (i < c && before == kr) sh.res[x] = (x ? lo1 : lo0) + v;
+      }
+    }
+    __syncthreads();
+    lo0 = sh.res[0]; lo1 = sh.res[1];
+    // the lists are empty again for the next call (whose lists are written several barriers on)
+    { const u32 i = threadIdx.x & (LQ_LIST - 1); (x ? l1 : l0)[i] = NONE; if (threadIdx.x < 2) sh.n_list[threadIdx.x] = 0; }
+  }
+  *ra = lo0; *rd = lo1;
+}
+
+template <int Q>
+__global__ void __launch_bounds__(LQ_THREADS, Q == 16 ? 2 : 3) k_reduce_large(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles,
+    TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
   begin_after();
-  __shared__ u32 s_a[LARGE_SEQS * LS_PITCH], s_d[LARGE_SEQS * LS_PITCH];
-  __shared__ LargeGroup s_part[LS_THREADS / 32][LARGE_SEQS];
-  const Tile t = tiles[blockIdx.x];
+  extern __shared__ __align__(16) u32 large_keys[];        // [metric][op counter][member of mine], later [metric][member]: my op counter
+  __shared__ __align__(16) LargeShared sh;
+  namespace cg = cooperative_groups;
+  const Tile t = tiles[blockIdx.x / LARGE_SEQS];
+  const u32 n = t.row.n;
+  if (t.count == 0 || (n <= 2048 ? 4 : (n <= 4096 ? 8 : 16)) != Q) return;     // no work, or another instance's: the same in the whole cluster
+  cg::cluster_group cluster = cg::this_cluster();
+  constexpr u32 PITCH = LargeTile<Q>::PITCH;
+  const u32 me = blockIdx.x % LARGE_SEQS;                   // my eighth of the members, and my op counter
   const WinDesc& D = wd[t.w];
-  const u32 n = R.comm_n[t.c], m0 = blockIdx.y * LS_MEMBERS;
-  if (m0 >= n) return;
-  const RangeRow row = D.ranges[t.c];
+  const RangeRow& row = t.row;
+  const u32* __restrict__ mem = R.members + t.moff;
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const u32 j = lane & 7, pq = lane >> 3;                     // op counter of the tile, member of the quad
-  const bool jvalid = j < t.count;
-  const u32 so = t.seq_off + (jvalid ? j : 0u);
-  const u32* __restrict__ perm = D.perm + row.slot0;
-  const i64* __restrict__ c_te = D.t_enter; const i64* __restrict__ c_tx = D.t_exit;
-  const u64* __restrict__ c_by = D.bytes; const u8* __restrict__ c_op = D.op;
-  const u32* __restrict__ c_sc = D.send_chg; const u32* __restrict__ c_rc = D.recv_chg;
-  // the group's first member gives the time base and the op set
-  u32 bits = 0;
-  i64 te0 = 0; u64 by0 = 0; u32 op0 = 0;
+  const u32 M = (n + LARGE_SEQS - 1) / LARGE_SEQS, m0 = me * M, m_cnt = m0 >= n ? 0u : min(M, n - m0);
+  u32* __restrict__ k_a = large_keys; u32* __restrict__ k_d = large_keys + LARGE_SEQS * PITCH;
+  for (u32 i = threadIdx.x; i < 2 * LQ_BINS / 4; i += LQ_THREADS) reinterpret_cast<uint4*>(&sh.hist[0][0])[i] = make_uint4(0, 0, 0, 0);
+  if (threadIdx.x < 2 * LQ_LIST / 4) (&sh.list[0][0])[threadIdx.x] = make_uint4(NONE, NONE, NONE, NONE);
+  if (threadIdx.x < 2) sh.n_list[threadIdx.x] = 0;
+  if (threadIdx.x == 0) { sh.n_fs = 0; sh.n_fd = 0; }
+  // ---- gather ----
   {
-    const u32 i0 = jvalid ? __ldg(perm + so) : NONE;
-    if (i0 != NONE) { te0 = c_te[i0]; by0 = c_by[i0]; op0 = c_op[i0]; } else bits = 1;
-  }
-  const u64 base = (u64)te0 - 0x80000000ull;
-  u32 emin = 0xFFFFFFFFu, emax = 0, xmax = 0; u64 kmax = 0, kmin = U64_MAX_, ck = 0;
-  constexpr u32 PER_WARP = LS_MEMBERS / (LS_THREADS / 32);    // 64 members per warp, four at a time
-  for (u32 it = 0; it < PER_WARP / 4; it += 4) {
-    u32 idx[4]; i64 x[4], y[4]; u64 by[4]; u32 op[4], ch[4];
+    const u32 j = lane & 7, pq = lane >> 3;                 // op counter of the tile, member of the quad
+    const bool jv = j < t.count;
+    const u32* __restrict__ perm = D.perm + row.slot0 + t.seq_off + (jv ? j : 0u);
+    const i64* __restrict__ c_te = D.t_enter; const i64* __restrict__ c_tx = D.t_exit;
+    const u64* __restrict__ c_by = D.bytes; const u8* __restrict__ c_op = D.op;
+    const u32* __restrict__ c_sc = D.send_chg; const u32* __restrict__ c_rc = D.recv_chg;
+    MidPart x; x.kmax = 0; x.n_kmin = 0; x.ck = 0; x.n_emin = 0; x.emax = 0; x.xmax = 0; x.bits = 0;
+    u32 idx[Q];
+    const u32 i0 = jv ? __ldg(perm) : NONE;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) { const u32 p = m0 + wid * PER_WARP + (it + q) * 4 + pq; idx[q] = (jvalid && p < n) ? __ldg(perm + (u64)p * row.n_seq + so) : NONE; }
+    for (int q = 0; q < Q; ++q) { const u32 m = (wid + LQ_WARPS * (u32)q) * 4 + pq; idx[q] = (jv && m < m_cnt) ? __ldg(perm + (u64)(m0 + m) * row.n_seq) : NONE; }
+    i64 te0 = 0; u64 by0 = 0; u32 op0 = 0;
+    if (i0 != NONE) { te0 = __ldg(c_te + i0); by0 = __ldg(c_by + i0); op0 = __ldg(c_op + i0); } else x.bits = 1;
+    const u64 base = (u64)te0 - 0x80000000ull;
+    constexpr int STEP = Q == 16 ? 4 : 2;                   // records in flight per thread, as many as the registers allow
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const u32 ix = idx[q] == NONE ? 0u : idx[q];
-      x[q] = c_te[ix]; y[q] = c_tx[ix]; by[q] = c_by[ix]; op[q] = c_op[ix]; ch[q] = 0;
-      if (c_sc != nullptr) { const u32 sc = c_sc[ix], rc = c_rc[ix]; ch[q] = sc > rc ? sc : rc; }
-    }
+    for (int q0 = 0; q0 < Q; q0 += STEP) {
+      i64 ta[STEP], tb[STEP]; u64 by[STEP]; u32 op[STEP], ch[STEP];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const u32 pm = wid * PER_WARP + (it + q) * 4 + pq, p = m0 + pm;
-      u32 a_lo = 0, d = 0;
-      if (p < n) {
-        if (idx[q] == NONE) { if (jvalid) bits |= 1; }
+      for (int u = 0; u < STEP; ++u) {
+        const u32 ix = idx[q0 + u] == NONE ? 0u : idx[q0 + u];
+        ta[u] = __ldg(c_te + ix); tb[u] = __ldg(c_tx + ix); by[u] = __ldg(c_by + ix); op[u] = __ldg(c_op + ix); ch[u] = 0;
+        if (c_sc != nullptr) { const u32 sc = __ldg(c_sc + ix), rc = __ldg(c_rc + ix); ch[u] = max(sc, rc); }
+      }
+#pragma unroll
+      for (int u = 0; u < STEP; ++u) {
+        const u32 m = (wid + LQ_WARPS * (u32)(q0 + u)) * 4 + pq, p = m0 + m;
+        if (m >= m_cnt) continue;
+        u32 a = 0, d = 0;
+        if (idx[q0 + u] == NONE) { if (jv) x.bits |= 1; }
         else {
-          const u64 ra = (u64)x[q] - base, rb = (u64)y[q] - base;
-          a_lo = (u32)ra; const u32 b_lo = (u32)rb; d = b_lo - a_lo;
-          if (((ra | rb) >> 32) != 0 || (x[q] | y[q]) < 0 || b_lo < a_lo) bits |= 1;     // beyond 32 bits, negative or in flight, exit before enter
-          if (op[q] != op0 || by[q] != by0) bits |= 2;
-          emin = min(emin, a_lo); emax = max(emax, a_lo); xmax = max(xmax, b_lo);
-          const u64 k1 = ((u64)d << 32) | (u64)(NONE - p); kmax = k1 > kmax ? k1 : kmax;   // longest, then the lowest position
-          const u64 k2 = ((u64)d << 32) | (u64)p; kmin = k2 < kmin ? k2 : kmin;            // shortest, then the lowest position
-          const u64 k3 = ((u64)ch[q] << 32) | (u64)(NONE - p); ck = k3 > ck ? k3 : ck;     // most changes, then the lowest position
+          const u64 ra = (u64)ta[u] - base, rb = (u64)tb[u] - base;
+          a = (u32)ra; const u32 b = (u32)rb; d = b - a;
+          if (((ra | rb) >> 32) != 0 || (ta[u] | tb[u]) < 0 || b < a) x.bits |= 1;       // beyond 32 bits, negative or in flight, exit before enter
+          if (op[u] != op0 || by[u] != by0) x.bits |= 2;
+          x.n_emin = max(x.n_emin, ~a); x.emax = max(x.emax, a); x.xmax = max(x.xmax, b);
+          const u64 k1 = ((u64)d << 32) | (u64)(NONE - p); x.kmax = k1 > x.kmax ? k1 : x.kmax;       // longest, then the lowest position
+          const u64 k2 = ~(((u64)d << 32) | (u64)p); x.n_kmin = k2 > x.n_kmin ? k2 : x.n_kmin;       // shortest, then the lowest position
+          const u64 k3 = ((u64)ch[u] << 32) | (u64)(NONE - p); x.ck = k3 > x.ck ? k3 : x.ck;         // most changes, then the lowest position
         }
+        k_a[j * PITCH + m] = a; k_d[j * PITCH + m] = d;
       }
-      s_a[j * LS_PITCH + pm] = a_lo; s_d[j * LS_PITCH + pm] = d;
     }
+    mid_merge(x, mid_shfl_xor(x, 8)); mid_merge(x, mid_shfl_xor(x, 16));
+    if (lane < LARGE_SEQS) sh.part[wid][lane] = x;
+    if (wid == 0 && lane < LARGE_SEQS) { sh.te0[lane] = te0; sh.gby[lane] = by0; sh.gop[lane] = op0; }
   }
-  // the four members of a warp step meet by shuffles, the warps through shared memory; one thread per op counter merges
-  // the CTA's part into the group's record
-#pragma unroll
-  for (int h = 8; h < 32; h <<= 1) {
-    emin = min(emin, __shfl_xor_sync(0xFFFFFFFFu, emin, h)); emax = max(emax, __shfl_xor_sync(0xFFFFFFFFu, emax, h));
-    xmax = max(xmax, __shfl_xor_sync(0xFFFFFFFFu, xmax, h)); bits |= __shfl_xor_sync(0xFFFFFFFFu, bits, h);
-    const u64 a = shfl_xor64(kmax, h); kmax = a > kmax ? a : kmax;
-    const u64 b = shfl_xor64(kmin, h); kmin = b < kmin ? b : kmin;
-    const u64 e = shfl_xor64(ck, h); ck = e > ck ? e : ck;
-  }
-  if (lane < LARGE_SEQS) { LargeGroup x; x.kmax = kmax; x.n_kmin = ~kmin; x.ck = ck; x.n_emin = ~emin; x.emax = emax; x.xmax = xmax; x.bits = bits; s_part[wid][lane] = x; }
   __syncthreads();
-  if (threadIdx.x < t.count) {
-    LargeGroup a = s_part[0][threadIdx.x];
-    for (u32 w = 1; w < LS_THREADS / 32; ++w) {
-      const LargeGroup x = s_part[w][threadIdx.x];
-      a.kmax = x.kmax > a.kmax ? x.kmax : a.kmax; a.n_kmin = x.n_kmin > a.n_kmin ? x.n_kmin : a.n_kmin; a.ck = x.ck > a.ck ? x.ck : a.ck;
-      a.n_emin = max(a.n_emin, x.n_emin); a.emax = max(a.emax, x.emax); a.xmax = max(a.xmax, x.xmax); a.bits |= x.bits;
-    }
-    LargeGroup* o = grp + (u64)blockIdx.x * LARGE_SEQS + threadIdx.x;
-    atomicMax((ull*)&o->kmax, (ull)a.kmax); atomicMax((ull*)&o->n_kmin, (ull)a.n_kmin); atomicMax((ull*)&o->ck, (ull)a.ck);
-    atomicMax(&o->n_emin, a.n_emin); atomicMax(&o->emax, a.emax); atomicMax(&o->xmax, a.xmax);
-    if (a.bits) atomicOr(&o->bits, a.bits);
+  if (wid < LARGE_SEQS) {                                   // warp j: my part of op counter j
+    MidPart x = sh.part[lane & (LQ_WARPS - 1)][wid];
+#pragma unroll
+    for (int h = 1; h < LQ_WARPS; h <<= 1) mid_merge(x, mid_shfl_xor(x, h));
+    if (lane == 0) sh.mine[wid] = x;
   }
-  // keys leave group by group, members contiguous
-  const u32 cnt = n - m0 < LS_MEMBERS ? n - m0 : (u32)LS_MEMBERS;
-  for (u32 q = 0; q < t.count; ++q) {
-    const u64 o = row.slot0 + (u64)(t.seq_off + q) * n + m0;
-    for (u32 pm = threadIdx.x; pm < cnt; pm += LS_THREADS) { D.skey[o + pm] = s_a[q * LS_PITCH + pm]; D.dkey[o + pm] = s_d[q * LS_PITCH + pm]; }
-  }
-}
-
-constexpr u32 LG_DIGIT = 8, LG_BINS = 1u << LG_DIGIT;      // radix digit of the selects; one histogram of LG_BINS bins per group
-
-// The k-th smallest (0-based) of a group's keys, for every group of the sub-tile at once. A thread holds up to LG_KEYS keys
-// of its own group g in registers (bit q of `have` says whether slot q holds one); `act` says whether the group takes
-// part. Digits of LG_DIGIT bits, most significant first; the first digit starts at the highest bit of `bound`, the
-// largest key of any group, so that it splits the keys as finely as 256 bins can, and a key that drops out of the
-// running costs its thread next to nothing in the passes that follow. After a pass warp w scans and clears group w's
-// histogram and names the digit that holds the k-th key. Histograms must be zero on entry and are zero again on return.
-// All threads of the CTA call it.
-__device__ __forceinline__ u32 large_select(const u32 (&v)[LG_KEYS], u32 have, bool act, u32 k, u32 bound, u32 G, u32 g,
-                                            u32* __restrict__ s_hist, u32* __restrict__ s_pick, u32* __restrict__ s_krem) {
-  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (threadIdx.x < G) s_krem[threadIdx.x] = k;
-  u32* __restrict__ hist = s_hist + g * LG_BINS;
-  u32 hi = 32 - (u32)__clz(bound | 1u);                      // bits still undecided: the result lies below 2^hi
-  u32 prefix = 0;                                            // the decided bits, already in place
-  u32 alive = act ? have : 0u;                               // my keys that still agree with the decided bits
-  while (hi > 0) {
-    const u32 sh = hi > LG_DIGIT ? hi - LG_DIGIT : 0u, w = hi - sh;       // this pass decides bits [sh, hi)
-    const u32 dmask = (1u << w) - 1u;
-    if (alive) {
+  cluster.sync();
+  // ---- exchange: my group's keys come in; op counter j's extrema by warp j ----
+  u32 va[Q], vd[Q];
+  const u32 src = wid & 7, mm0 = (wid >> 3) * 32 + lane;    // my keys: members mm0, mm0 + 64, ... of CTA src
+  const u32 s_cnt = src * M >= n ? 0u : min(M, n - src * M);
+  {
+    const u32* r_a = cluster.map_shared_rank(k_a, src) + me * PITCH; const u32* r_d = r_a + LARGE_SEQS * PITCH;
 #pragma unroll
-      for (int q = 0; q < LG_KEYS; ++q) if ((alive >> q) & 1u) atomicAdd(&hist[(v[q] >> sh) & dmask], 1u);
+    for (int q = 0; q < Q; ++q) {
+      const u32 m = mm0 + 64u * (u32)q;
+      const bool in = m < s_cnt;
+      va[q] = in ? r_a[m] : 0u; vd[q] = in ? r_d[m] : 0u;
     }
-    __syncthreads();
-    if (wid < G) {                                                               // warp w scans and clears group w's histogram
-      u32 loc[8], sum = 0;
-      const u32 kr = s_krem[wid];
+  }
+  if (wid < LARGE_SEQS) {
+    const u32 j = wid;
+    MidPart x = *cluster.map_shared_rank(&sh.mine[j], lane & 7);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) { loc[q] = s_hist[wid * LG_BINS + lane * 8 + q]; sum += loc[q]; s_hist[wid * LG_BINS + lane * 8 + q] = 0; }
-      u32 inc = sum;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) { const u32 o = __shfl_up_sync(0xFFFFFFFFu, inc, d); if (lane >= (u32)d) inc += o; }
-      const u32 ex = inc - sum;
-      if (kr >= ex && kr < inc) {
-        u32 cum = ex;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          if (kr >= cum && kr < cum + loc[q]) { s_pick[wid] = lane * 8 + q; s_krem[wid] = kr - cum; }
-          cum += loc[q];
-        }
+    for (int h = 1; h < (int)LARGE_SEQS; h <<= 1) mid_merge(x, mid_shfl_xor(x, h));
+    if (lane == 0) {
+      const u32 gop = sh.gop[j]; const u64 gby = sh.gby[j];
+      const bool clean = j < t.count && !(x.bits & 1), round = clean && !(gop == CCLD_OP_ALLREDUCE && gby < P.barrier_bytes);
+      double num, den; bus_factor(gop, n, &num, &den);
+      sh.state[j] = (clean ? 1u : 0u) | (round ? 2u : 0u); sh.rng[j] = (u32)(x.kmax >> 32) - (u32)(~x.n_kmin >> 32);
+      sh.bd[j] = round ? (double)gby * (num / den) : 0.0;
+      if (j == me) {
+        sh.group = x;
+        if (clean) { sh.ranks[0] = __ldg(mem + (u32)~x.n_kmin); sh.ranks[1] = __ldg(mem + (NONE - (u32)x.kmax)); sh.ranks[2] = __ldg(mem + (NONE - (u32)x.ck)); }
       }
     }
-    __syncthreads();
-    const u32 pick = s_pick[g];
-    prefix |= pick << sh;
-    if (alive) {                                             // few keys survive the first pass: most threads are done here
-      u32 keep = 0;
-#pragma unroll
-      for (int q = 0; q < LG_KEYS; ++q) keep |= (((v[q] >> sh) & dmask) == pick ? 1u : 0u) << q;
-      alive &= keep;
-    }
-    hi = sh;
   }
-  return prefix;
-}
-
-// dynamic shared memory of k_reduce_large: per-member bandwidth sums of the largest communicator
-inline size_t large_smem(u32 max_n) { return (size_t)8 * large_npad(max_n); }
-
-__global__ void __launch_bounds__(LG_THREADS, 2) k_reduce_large(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles, u32 n_tiles,
-                                                                 const LargeGroup* __restrict__ grp, TileSum* __restrict__ sums,
-                                                                 Registry R, Params P, DeferList DL) {
-  begin_after();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* s_bw = (double*)smem_raw;
-  __shared__ u32 s_hist[LARGE_SEQS * LG_BINS];
-  __shared__ LargeScal s_sc[LARGE_SEQS];
-  __shared__ LargeLead s_lead[LARGE_SEQS];
-  __shared__ u32 s_cnt[SC_COUNT];
-  __shared__ u32 s_bound[2][LARGE_SEQS];
-  __shared__ u32 s_pick[LARGE_SEQS], s_krem[LARGE_SEQS];
-  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  u32 cur_w = NONE, cur_c = NONE, cur_rounds = 0;            // whose bandwidth sums shared memory holds
-  const u32* cur_mem = nullptr; u32 cur_n = 0;
-  for (u32 i = threadIdx.x; i < LARGE_SEQS * LG_BINS; i += LG_THREADS) s_hist[i] = 0;
-  for (u32 ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
-    const Tile t = tiles[ti];
-    const WinDesc& D = wd[t.w];
-    const u32 c = t.c, n = R.comm_n[c];
-    const RangeRow row = D.ranges[c];
-    const u32* __restrict__ mem = R.members + R.comm_moff[c];
-    const u32 G = large_g(n), lgG = 31 - __clz(G);
-    const u32 g = wid & (G - 1), pl = (wid >> lgG) * 32 + lane, MP = (LG_WARPS >> lgG) * 32;      // a warp works on one group, lanes on consecutive members
-    const bool lead = pl == 0;
-    const u64 G_all = D.n_groups;
-
-    __syncthreads();                                          // the previous tile is done with shared memory
-    if (t.w != cur_w || c != cur_c) {
-      // another communicator or window: the sums shared memory holds go out
-      if (cur_rounds) for (u32 p = threadIdx.x; p < cur_n; p += LG_THREADS) { atomicAdd(&R.bw_sum[cur_mem[p]], s_bw[p]); atomicAdd(&R.bw_cnt[cur_mem[p]], cur_rounds); }
-      __syncthreads();
-      cur_w = t.w; cur_c = c; cur_rounds = 0; cur_mem = mem; cur_n = n;
-      for (u32 p = threadIdx.x; p < n; p += LG_THREADS) s_bw[p] = 0.0;
-    }
-    if (threadIdx.x < SC_COUNT) s_cnt[threadIdx.x] = 0;
-    if (threadIdx.x < LARGE_SEQS) { LargeLead z = {0, NONE, 0, 0, 0, 0}; s_lead[threadIdx.x] = z; }
-    u32 have = 0;
+  __syncthreads();
+  // ---- bandwidth of my members over the tile's op counters, where they were gathered ----
+  u32 rounds = 0;
 #pragma unroll
-    for (int q = 0; q < LG_KEYS; ++q) have |= (pl + (u32)q * MP < n ? 1u : 0u) << q;
-
-    for (u32 j0 = 0; j0 < t.count; j0 += G) {
-      const bool gvalid = j0 + g < t.count;
-      const u32 so = t.seq_off + j0 + (gvalid ? g : 0u);      // op-counter offset of my group inside the range
-      const u64 slot = row.slot0 + (u64)so * n;               // first slot of my group (keys and flags, group-major)
-      __syncthreads();                                        // the previous sub-tile's shared-memory values are no longer read
-      // ---- what the staging pass left for the group; op and size of its first member ----
-      const LargeGroup x = grp[(u64)ti * LARGE_SEQS + j0 + (gvalid ? g : 0u)];
-      const u32 emin = ~x.n_emin, tmx = (u32)(x.kmax >> 32), tmn = (u32)(~x.n_kmin >> 32);
-      u64 by0 = 0; u32 op0 = 0; i64 te0 = 0;
-      const bool gok = gvalid && !(x.bits & 1);
-      if (gok) { const u32 i0 = __ldg(D.perm + row.slot0 + so); by0 = D.bytes[i0]; op0 = D.op[i0]; te0 = D.t_enter[i0]; }
-      const bool barrier = op0 == CCLD_OP_ALLREDUCE && by0 < P.barrier_bytes;
-      const bool analysed = gok && !barrier && n >= P.min_group;
-      double num, den; bus_factor(op0, n, &num, &den);
-      const double bn = (double)by0 * num;
-      if (lead) {
-        s_bound[0][g] = analysed ? x.emax - emin : 0u; s_bound[1][g] = analysed ? tmx - tmn : 0u;
-        if (gvalid && !gok) {                                 // set aside for the 64-bit kernel
-          const u32 e = atomicAdd(DL.count, 1u);
-          DL.entries[e] = ((u64)t.w << 32) | (u64)(row.group0 + so);
-          s_lead[g].def += 1;
-        }
-        if (gok) {
-          // everything of the per-op row that needs no order statistic
-          const u64 kmin = ~x.n_kmin;
-          const u64 gi_ = row.group0 + so;
-          i64* __restrict__ gi = D.gi64 + gi_; u32* __restrict__ gu = D.gu32 + gi_;
-          const u32 span = x.xmax - emin;
-          gi[(u64)GI_E_MIN * G_all] = (i64)((u64)te0 - 0x80000000ull + emin); gi[(u64)GI_ARRIVAL_SKEW * G_all] = (i64)(u64)(x.emax - emin);
-          gi[(u64)GI_T_MAX * G_all] = (i64)(u64)tmx; gi[(u64)GI_T_MIN * G_all] = (i64)(u64)tmn; gi[(u64)GI_SPAN * G_all] = (i64)(u64)span;
-          gu[(u64)GU_RANK_TMIN * G_all] = mem[(u32)kmin]; gu[(u64)GU_RANK_TMAX * G_all] = mem[NONE - (u32)x.kmax];
-          gu[(u64)GU_MAX_CHG * G_all] = (u32)(x.ck >> 32); gu[(u64)GU_RANK_MAX_CHG * G_all] = mem[NONE - (u32)x.ck];
-          gu[(u64)GU_N_PRESENT * G_all] = n;
-          const bool mismatch = (x.bits & 2) != 0;
-          gu[(u64)GU_GFLAGS * G_all] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mismatch ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
-          D.gbw[gi_] = span ? bn * rcp_newton((double)span * den) : 0.0;
-          atomicAdd(&s_cnt[SC_COMP], 1u); atomicAdd(&s_cnt[SC_PRES], n);
-          if (barrier) atomicAdd(&s_cnt[SC_BAR], 1u);
-          if (analysed) { atomicAdd(&s_cnt[SC_AN], 1u); s_lead[g].an += 1; }
-          if (mismatch) atomicAdd(&s_cnt[SC_MIS], 1u);
-          if (!barrier) { LargeLead m = s_lead[g]; m.rounds += 1; best_merge(m.brng, m.bk, (u64)(tmx - tmn), so); s_lead[g] = m; }
-        }
+  for (u32 j = 0; j < LARGE_SEQS; ++j) rounds += sh.state[j] >> 1;
+  if (rounds) {
+    for (u32 m = threadIdx.x; m < m_cnt; m += LQ_THREADS) {
+      double v = 0.0;
+#pragma unroll
+      for (u32 j = 0; j < LARGE_SEQS; ++j) {
+        const u32 d = k_d[j * PITCH + m];
+        if (d != 0) v += sh.bd[j] * rcp_u32(d);
+      }
+      const u32 rank = __ldg(mem + m0 + m);
+      atomicAdd(&R.bw_sum[rank], v); atomicAdd(&R.bw_cnt[rank], rounds);
+    }
+  }
+  cluster.sync();                                           // everybody has read what it needs from everybody's shared memory
+  // ---- my group ----
+  const u32 emin = ~sh.group.n_emin, emax = sh.group.emax, tmx = (u32)(sh.group.kmax >> 32), tmn = (u32)(~sh.group.n_kmin >> 32);
+  const u32 so = t.seq_off + me;
+  const bool gvalid = me < t.count, gok = sh.state[me] & 1, barrier = gok && !(sh.state[me] & 2), analysed = gok && !barrier && n >= P.min_group;
+  u32 ms = 0, ds = 0, md = 0, dm = 0;
+  if (gok) {                                                // the same in the whole CTA
+    u8* __restrict__ fp = D.flags + row.slot0 + (u64)so * n;
+    if (analysed) {
+      u32* __restrict__ s_a = large_keys; u32* __restrict__ s_d = large_keys + n;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const u32 m = mm0 + 64u * (u32)q;
+        if (m < s_cnt) { s_a[src * M + m] = va[q] - emin; s_d[src * M + m] = vd[q] - tmn; }
       }
       __syncthreads();
-      u32 bs = 0, bd = 0;
-      for (u32 q = 0; q < G; ++q) { bs = max(bs, s_bound[0][q]); bd = max(bd, s_bound[1][q]); }
-
-      // ---- order statistics, all groups of the sub-tile side by side; a thread's keys sit in registers during a select ----
-      u32 ms = 0, ds = 0, md = 0, dm = 0;
-      if (__syncthreads_or(analysed)) {
-        const u32 k = (n - 1) >> 1;
-        u32 v[LG_KEYS];
-        const u32* __restrict__ sk = D.skey + slot + pl; const u32* __restrict__ du = D.dkey + slot + pl;
-#pragma unroll
-        for (int q = 0; q < LG_KEYS; ++q) v[q] = (analysed && ((have >> q) & 1u)) ? sk[(u32)q * MP] - emin : 0u;
-        ms = large_select(v, have, analysed, k, bs, G, g, s_hist, s_pick, s_krem);
-#pragma unroll
-        for (int q = 0; q < LG_KEYS; ++q) v[q] = __usad(v[q], ms, 0u);
-        ds = large_select(v, have, analysed, k, bs, G, g, s_hist, s_pick, s_krem);
-#pragma unroll
-        for (int q = 0; q < LG_KEYS; ++q) v[q] = (analysed && ((have >> q) & 1u)) ? du[(u32)q * MP] - tmn : 0u;
-        md = large_select(v, have, analysed, k, bd, G, g, s_hist, s_pick, s_krem);
-#pragma unroll
-        for (int q = 0; q < LG_KEYS; ++q) v[q] = __usad(v[q], md, 0u);
-        dm = large_select(v, have, analysed, k, bd, G, g, s_hist, s_pick, s_krem);
-        if (!analysed) { ms = ds = md = dm = 0; }
-      }
-      if (lead) {
-        LargeScal z; z.ts = (u64)ds * P.k_milli; z.td = (u64)dm * P.k_milli; z.bn = bn; z.den = den;   // |x - med| * 1000 > k * MAD: both sides below 2^64
-        z.emin = emin; z.tmn = tmn; z.ms = ms; z.md = md; z.state = (gok ? 1u : 0u) | (analysed ? 2u : 0u) | (barrier ? 4u : 0u); z.pad = 0;
-        s_sc[g] = z;
-        if (gok) {
-          i64* __restrict__ gi = D.gi64 + row.group0 + so;
-          gi[(u64)GI_MED_SKEW * G_all] = (i64)(u64)ms; gi[(u64)GI_MAD_SKEW * G_all] = (i64)(u64)ds;
-          gi[(u64)GI_MED_DUR * G_all] = analysed ? (i64)((u64)tmn + md) : 0; gi[(u64)GI_MAD_DUR * G_all] = (i64)(u64)dm;
-        }
-      }
-      __syncthreads();
-
-      // ---- flags, votes, per-member bandwidth: a thread takes a member through the G groups ----
+      const u32 k = (n - 1) >> 1, ba = emax - emin, bd = tmx - tmn;
+      large_pick<Q>(s_a, s_d, n, 0u, 0u, k, ba, bd, sh, &ms, &md);
+      large_pick<Q>(s_a, s_d, n, ms, md, k, max(ms, ba - ms), max(md, bd - md), sh, &ds, &dm);
+      // |x - med| * 1000 > k * MAD in whole numbers: |x - med| > floor(k * MAD / 1000); a quotient of 2^32 - 1 or more is never exceeded
+      const u64 qs = (u64)ds * P.k_milli / 1000u, qd = (u64)dm * P.k_milli / 1000u;
+      const u32 ts = qs > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qs, td = qd > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qd;
       u32 n_fs = 0, n_fd = 0;
-      const u32 gcnt = t.count - j0 < G ? t.count - j0 : G;
-      const u64 slot0 = row.slot0 + (u64)(t.seq_off + j0) * n;
-      for (u32 q = 0; q < gcnt; ++q) {
-        const LargeScal z = s_sc[q];                                           // the group's values stay in registers over my members
-        if (!(z.state & 1)) continue;
-        const u64 o0 = slot0 + (u64)q * n;
-        for (u32 p = threadIdx.x; p < n; p += LG_THREADS) {                  // a member belongs to one thread: no two threads touch s_bw[p]
-          const u32 d = D.dkey[o0 + p];
-          u32 f = CCLD_F_NOT_ANALYSED;
-          if (z.state & 2) {
-            const u32 skw = D.skey[o0 + p] - z.emin, dd = d - z.tmn;
-            const bool so_ = (u64)__usad(skw, z.ms, 0u) * 1000u > z.ts, shi = skw > z.ms;
-            const bool dq = (u64)__usad(dd, z.md, 0u) * 1000u > z.td, dhi = dd > z.md;
-            f = (so_ ? CCLD_F_SKEW_OUT : 0) | (dq ? CCLD_F_DUR_OUT : 0) | (shi ? CCLD_F_SKEW_HI : 0) | (dhi ? CCLD_F_DUR_HI : 0);
-            if (so_) { ++n_fs; atomicAdd(&R.votes[(u64)mem[p] * 4 + (shi ? 0 : 1)], 1u); }
-            if (dq) { ++n_fd; atomicAdd(&R.votes[(u64)mem[p] * 4 + (dhi ? 2 : 3)], 1u); }
-          }
-          D.flags[o0 + p] = (u8)f;
-          if (!(z.state & 4) && d != 0) s_bw[p] += z.bn * rcp_newton1((double)d * z.den);
-        }
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
+        if (i >= n) break;
+        const u32 a = s_a[i], d = s_d[i];
+        const bool os = __usad(a, ms, 0u) > ts, od = __usad(d, md, 0u) > td, hs = a > ms, hd = d > md;
+        fp[i] = (u8)((os ? CCLD_F_SKEW_OUT : 0) | (od ? CCLD_F_DUR_OUT : 0) | (hs ? CCLD_F_SKEW_HI : 0) | (hd ? CCLD_F_DUR_HI : 0));
+        if (os) { ++n_fs; atomicAdd(&R.votes[(u64)mem[i] * 4 + (hs ? 0 : 1)], 1u); }
+        if (od) { ++n_fd; atomicAdd(&R.votes[(u64)mem[i] * 4 + (hd ? 2 : 3)], 1u); }
       }
-      n_fs = __reduce_add_sync(0xFFFFFFFFu, n_fs); n_fd = __reduce_add_sync(0xFFFFFFFFu, n_fd);
-      if (lane == 0) { if (n_fs) atomicAdd(&s_cnt[SC_FS], n_fs); if (n_fd) atomicAdd(&s_cnt[SC_FD], n_fd); }
-    }  // sub-tiles
-    __syncthreads();
-    for (u32 q = 0; q < LARGE_SEQS; ++q) cur_rounds += s_lead[q].rounds;
-    if (threadIdx.x == 0) {
-      TileSum ts; ts.best_rng = 0; ts.best_k = NONE; ts.n_rounds = 0; ts.n_an = 0; ts.pad = 0;
-      for (u32 q = 0; q < LARGE_SEQS; ++q) { best_merge(ts.best_rng, ts.best_k, s_lead[q].brng, s_lead[q].bk); ts.n_rounds += s_lead[q].rounds; ts.n_an += s_lead[q].an; ts.pad += s_lead[q].def; }
-      sums[ti] = ts;
-      count_add(D.counters, C_COMPLETE, s_cnt[SC_COMP]); count_add(D.counters, C_BARRIER, s_cnt[SC_BAR]); count_add(D.counters, C_ANALYSED, s_cnt[SC_AN]);
-      count_add(D.counters, C_MISMATCH, s_cnt[SC_MIS]); count_add(D.counters, C_PRESENT, s_cnt[SC_PRES]);
-      count_add(D.counters, C_FLAG_SKEW, s_cnt[SC_FS]); count_add(D.counters, C_FLAG_DUR, s_cnt[SC_FD]);
+      n_fs = __reduce_add_sync(FULLM, n_fs); n_fd = __reduce_add_sync(FULLM, n_fd);
+      if (lane == 0) { if (n_fs) atomicAdd(&sh.n_fs, n_fs); if (n_fd) atomicAdd(&sh.n_fd, n_fd); }
+      __syncthreads();
+    } else {
+      for (u32 i = threadIdx.x; i < n; i += LQ_THREADS) fp[i] = CCLD_F_NOT_ANALYSED;
     }
-  }  // tiles of this CTA
-  __syncthreads();
-  if (cur_rounds) for (u32 p = threadIdx.x; p < cur_n; p += LG_THREADS) { atomicAdd(&R.bw_sum[cur_mem[p]], s_bw[p]); atomicAdd(&R.bw_cnt[cur_mem[p]], cur_rounds); }
+  }
+  // ---- the row, the counters; the tile's summary by the first CTA ----
+  if (threadIdx.x == 0) {
+    if (gok) {
+      const u64 G = D.n_groups, gr = row.group0 + so;
+      i64* __restrict__ gi = D.gi64 + gr; u32* __restrict__ gu = D.gu32 + gr;
+      const u32 span = sh.group.xmax - emin;
+      const bool mismatch = (sh.group.bits & 2) != 0;
+      double num, den; bus_factor(sh.gop[me], n, &num, &den);
+      gi[(u64)GI_E_MIN * G] = (i64)((u64)sh.te0[me] - 0x80000000ull + emin); gi[(u64)GI_ARRIVAL_SKEW * G] = (i64)(u64)(emax - emin);
+      gi[(u64)GI_T_MAX * G] = (i64)(u64)tmx; gi[(u64)GI_T_MIN * G] = (i64)(u64)tmn; gi[(u64)GI_SPAN * G] = (i64)(u64)span;
+      gi[(u64)GI_MED_SKEW * G] = (i64)(u64)ms; gi[(u64)GI_MAD_SKEW * G] = (i64)(u64)ds;
+      gi[(u64)GI_MED_DUR * G] = analysed ? (i64)((u64)tmn + md) : 0; gi[(u64)GI_MAD_DUR * G] = (i64)(u64)dm;
+      gu[(u64)GU_RANK_TMIN * G] = sh.ranks[0]; gu[(u64)GU_RANK_TMAX * G] = sh.ranks[1];
+      gu[(u64)GU_MAX_CHG * G] = (u32)(sh.group.ck >> 32); gu[(u64)GU_RANK_MAX_CHG * G] = sh.ranks[2];
+      gu[(u64)GU_N_PRESENT * G] = n;
+      gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mismatch ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
+      D.gbw[gr] = span ? (double)sh.gby[me] * num * rcp_newton((double)span * den) : 0.0;
+      count_add(D.counters, C_COMPLETE, 1); count_add(D.counters, C_PRESENT, n); count_add(D.counters, C_BARRIER, barrier); count_add(D.counters, C_ANALYSED, analysed);
+      count_add(D.counters, C_MISMATCH, mismatch); count_add(D.counters, C_FLAG_SKEW, sh.n_fs); count_add(D.counters, C_FLAG_DUR, sh.n_fd);
+    } else if (gvalid) {                                    // set aside for the 64-bit kernel
+      const u32 e = atomicAdd(DL.count, 1u);
+      DL.entries[e] = ((u64)t.w << 32) | (u64)(row.group0 + so);
+    }
+    if (me == 0) {
+      TileSum ts = {0, NONE, rounds, n >= P.min_group ? rounds : 0u, 0};
+      for (u32 j = 0; j < t.count; ++j) {
+        if (sh.state[j] & 2) best_merge(ts.best_rng, ts.best_k, (u64)sh.rng[j], t.seq_off + j);
+        if (!(sh.state[j] & 1)) ++ts.pad;
+      }
+      sums[blockIdx.x / LARGE_SEQS] = ts;
+    }
+  }
 }
 
 // ------------------------------------------------------------------------------------------------

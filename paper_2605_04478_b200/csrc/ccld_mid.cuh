@@ -121,12 +121,12 @@ __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(cons
   __shared__ u32 s_cnt[SC_COUNT];
   const Registry& Reg = R_;
   const Tile t = tiles[blockIdx.x];
-  const u32 n = Reg.comm_n[t.c];
+  const u32 n = t.row.n;
   if (mid_npad(n) != 32u * R || t.count == 0) return;         // another instance's tile, or none (a window that gave up)
   const WinDesc& D = wd[t.w];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const RangeRow row = D.ranges[t.c];
-  const u32* __restrict__ mem = Reg.members + Reg.comm_moff[t.c];
+  const RangeRow& row = t.row;
+  const u32* __restrict__ mem = Reg.members + t.moff;
   u32* __restrict__ k_a = mid_keys; u32* __restrict__ k_d = mid_keys + n * MID_PITCH;
   if (threadIdx.x < SC_COUNT) s_cnt[threadIdx.x] = 0;
 

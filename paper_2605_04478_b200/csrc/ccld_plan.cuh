@@ -83,8 +83,8 @@ __device__ __forceinline__ PlanAcc plan_item(u32 ns, u32 n, u32 T) {
   return a;
 }
 
-// Work lists of the batch; grp: one record per op counter of the class-3 tiles, zeroed with the tile's entry.
-struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; u32* grp_words; u32 grp_words_per_tile; };
+// Work lists of the batch.
+struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; };
 
 // When the host sized the results from totals it expected (D.expect) instead of waiting for these, a window whose totals
 // differ gives up and raises the poison flag; so does every window planned after the flag went up - in the same batch
@@ -292,10 +292,9 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict
       x.row = RangeRow{0, 0, 0, 0, 0, 0, 0, 0};
       L.fcta[D.base[B_FCTA] + j] = x;
     }
-    const Tile none = {blockIdx.y, 0, 0, 0};
+    const Tile none = {blockIdx.y, 0, 0, 0, RangeRow{0, 0, 0, 0, 0, 0, 0, 0}, 0, 0};
     for (u64 j = i0; j < n2; j += st) L.t2[D.base[B_T2] + j] = none;
     for (u64 j = i0; j < n3; j += st) L.t3[D.base[B_T3] + j] = none;
-    for (u64 j = i0; j < n3 * L.grp_words_per_tile; j += st) L.grp_words[(u64)D.base[B_T3] * L.grp_words_per_tile + j] = 0;
     return;
   }
   const u32 T = (u32)D.totals[T_CHUNKS], tau = blockIdx.x / slices, slice = blockIdx.x % slices;
@@ -307,14 +306,11 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict
     const RangeRow row = D.ranges[c];
     const u32 S = tile_seqs(n), first = D.base[cls == 2 ? B_T2 : B_T3] + row.tile0;
     Tile* dst = cls == 2 ? L.t2 : L.t3;
+    const u64 moff = R.comm_moff[c];
     for (u32 k = lane; k < row.n_units; k += 32) {
-      Tile t; t.w = blockIdx.y; t.c = c; t.seq_off = k * S;
+      Tile t; t.w = blockIdx.y; t.c = c; t.seq_off = k * S; t.row = row; t.moff = moff; t.pad = 0;
       const u32 left = row.n_seq - k * S; t.count = left < S ? left : S;
       dst[first + k] = t;
-    }
-    if (cls == 3) {
-      u32* g = L.grp_words + (u64)first * L.grp_words_per_tile;
-      for (u64 k = lane; k < (u64)row.n_units * L.grp_words_per_tile; k += 32) g[k] = 0;
     }
   }
   // fused classes: the units of this chunk that earlier slices hold, those of my communicator, then where they go
