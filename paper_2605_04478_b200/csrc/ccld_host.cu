@@ -156,6 +156,7 @@ struct ccld_ctx {
   const TreeRef* d_trees = nullptr; u32 n_trees = 0;     // tree communicators whose layers are known
   std::map<u32, WindowHost> windows;
   Pool pool; std::string err;
+  cudaStream_t side[2] = {nullptr, nullptr}; cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};     // see Chains
   Block h_verdict;                                       // pinned area of ccld_get_verdict (VerdictArea)
   Block h_io;                                            // pinned area small results pass through
   bool long_list = false;                                // the last suspect list was longer than VD_MERGE
@@ -215,21 +216,66 @@ struct TimedLaunch {                                     // a named range and, w
 // Every kernel of the library starts with begin_after(): it may be launched while the one before it in the stream still runs,
 // waits there until that one is done, and lets the next one be launched. A launch then costs its latency beside the kernel
 // before it instead of after it.
+struct On {                                               // a stream; overlap = false: the launch follows a wait for another stream
+  cudaStream_t stream; bool overlap;
+  On(cudaStream_t s, bool o = true) : stream(s), overlap(o) {}
+};
 template <class... P, class... A>
-void launch_cluster(cudaStream_t st, void (*kernel)(P...), u32 cluster, dim3 grid, dim3 block, size_t smem, A&&... args) {
+void launch_cluster(On on, void (*kernel)(P...), u32 cluster, dim3 grid, dim3 block, size_t smem, A&&... args) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = on.stream;
   cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = on.overlap ? 1 : 0;
   at[1].id = cudaLaunchAttributeClusterDimension; at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
   cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);      // the caller looks at cudaGetLastError()
 }
 
 template <class... P, class... A>
-void launch(cudaStream_t st, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
-  launch_cluster(st, kernel, 1, grid, block, smem, std::forward<A>(args)...);
+void launch(On on, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+  launch_cluster(on, kernel, 1, grid, block, smem, std::forward<A>(args)...);
 }
+
+// The reductions of the three sizes of communicators do not depend on one another. Where a batch has more than one size, they
+// run on streams of their own between the slot scatter and the window decision: the kernel of the largest communicators
+// waits on barriers and round trips most of the time, that of 129 to 1,024 ranks may have no more than a few CTAs (a warp per
+// group), and the kernel of the small ones, which keeps memory busy, fills the SMs beside both. The side streams have
+// priority over the caller's: what has few CTAs, or long ones, gets its place first. With kernel timing on everything stays
+// on the caller's stream, so that a time belongs to one kernel.
+// A pass over a window of 16,384 ranks in groups of 8, 128, 1,024 and 2,048: 995 -> 872 us; over two windows of 4,128 ranks in
+// groups of 4, 6 and 172: 536 -> 527 us.
+struct Chains {
+  ccld_ctx* ctx; int n; bool used[2] = {false, false};
+  Chains(ccld_ctx* c, int sizes, bool timed) : ctx(c), n(timed ? 0 : sizes - 1) {
+    if (n > 0 && !ready()) n = 0;                          // no stream to be had: one after the other
+    if (n > 0) cudaEventRecord(ctx->fork, ctx->stream);
+  }
+  bool ready() {
+    int low = 0, high = 0;
+    if (ctx->join[1]) return true;
+    cudaDeviceGetStreamPriorityRange(&low, &high);
+    bool ok = ctx->fork || cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < 2 && ok; ++i)
+      ok = (ctx->side[i] || cudaStreamCreateWithPriority(&ctx->side[i], cudaStreamNonBlocking, high) == cudaSuccess) &&
+           (ctx->join[i] || cudaEventCreateWithFlags(&ctx->join[i], cudaEventDisableTiming) == cudaSuccess);
+    if (!ok) cudaGetLastError();
+    return ok;
+  }
+  On open(int i) {                                         // where chain i runs
+    if (i >= n) return On(ctx->stream);
+    used[i] = true;
+    cudaStreamWaitEvent(ctx->side[i], ctx->fork, 0);
+    return On(ctx->side[i], false);
+  }
+  On close() {                                             // the caller's stream, after all chains
+    for (int i = 0; i < 2; ++i) if (used[i]) { cudaEventRecord(ctx->join[i], ctx->side[i]); cudaStreamWaitEvent(ctx->stream, ctx->join[i], 0); }
+    return On(ctx->stream, n <= 0);
+  }
+  static void drop(ccld_ctx* c) {
+    for (int i = 0; i < 2; ++i) { if (c->join[i]) cudaEventDestroy(c->join[i]); if (c->side[i]) cudaStreamDestroy(c->side[i]); }
+    if (c->fork) cudaEventDestroy(c->fork);
+  }
+};
 
 // Layout of the scratch block used by get_verdict and locate_hang.
 struct MiscLayout { size_t sus, keys, counts, done, alerts, total; };
@@ -613,6 +659,7 @@ int ccld_destroy(ccld_ctx* ctx) {
   for (auto& b : ctx->pending) ctx->pinned_free.push_back(b.pin);
   ctx->pinned_free.push_back(ctx->h_verdict); ctx->pinned_free.push_back(ctx->h_io); ctx->pinned_free.push_back(ctx->h_up);
   for (UploadSlot& u : ctx->up) if (u.done) cudaEventDestroy(u.done);
+  Chains::drop(ctx);
   for (auto& f : ctx->pinned_free) BlockStore::get().put(-1, f);
   BlockStore::get().leave();
   for (auto& sl : ctx->ring) for (int i = 0; i < TIMER_PAIRS; ++i) { cudaEventDestroy(sl.a[i]); cudaEventDestroy(sl.b[i]); }
@@ -905,38 +952,43 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     TimedLaunch tl(ts, 2, st);
     launch(st, k_slot_scatter, dim3((u32)((blocks + per - 1) / per), B), SCAT_THREADS, 0, d_desc, ctx->reg, per);
   }
+  const DeferList dl_big{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
+  static_assert(MID_SEQS == LARGE_SEQS, "one list for the groups of both classes");
+  Chains chains(ctx, (n_list[B_FCTA] ? 1 : 0) + (n_list[B_T2] ? 1 : 0) + (n_list[B_T3] ? 1 : 0), ts != nullptr);
+  auto deferred_big = [&](On on) {
+    u32 n = 0;
+    for (int q = 0; q < 3; ++q) n = std::max(n, std::max(ctx->max_mid_n[q], ctx->max_large_n[q]));
+    launch(on, k_reduce_large_deferred, LARGE_DEF_GRID, LARGE_DEF_THREADS, 16ull * n, d_desc, dl_big, ctx->reg, ctx->dp, now_ns);
+  };
+  if (n_list[B_T2]) {
+    On on = chains.open(0);
+    TimedLaunch tl(ts, 4, st);
+    const u32 grid = (u32)n_list[B_T2]; TileSum* sums = (TileSum*)(rbase + o_s2);
+    // one launch per padded size the registry has; a tile of another size ends at once
+    const u32* m = ctx->max_mid_n;
+    if (m[0]) launch(on, k_reduce_mid<8>, grid, MID_THREADS, mid_smem_bytes(m[0]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[1]) launch(on, k_reduce_mid<16>, grid, MID_THREADS, mid_smem_bytes(m[1]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[2]) launch(on, k_reduce_mid<32>, grid, MID_THREADS, mid_smem_bytes(m[2]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
+    if (chains.n <= 0 && !n_list[B_T3]) deferred_big(on);
+  }
+  if (n_list[B_T3]) {
+    On on = chains.open(n_list[B_T2] ? 1 : 0);
+    TimedLaunch tl(ts, 5, st);
+    const u32 grid = (u32)(n_list[B_T3] * LARGE_SEQS); TileSum* sums = (TileSum*)(rbase + o_s3);
+    const u32* m = ctx->max_large_n;
+    if (m[0]) launch_cluster(on, k_reduce_large<4>, LARGE_SEQS, grid, LQ_THREADS, large_smem(4), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[1]) launch_cluster(on, k_reduce_large<8>, LARGE_SEQS, grid, LQ_THREADS, large_smem(8), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[2]) launch_cluster(on, k_reduce_large<16>, LARGE_SEQS, grid, LQ_THREADS, large_smem(16), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
+    if (chains.n <= 0) deferred_big(on);
+  }
   if (n_list[B_FCTA]) {
     const DeferList dl{(u64*)(rbase + o_def), (u32*)(pbase + o_defn)};
     TimedLaunch tl(ts, 3, st);
     launch(st, k_reduce_fused, (u32)n_list[B_FCTA], SMALL_SEQS, 0, d_desc, pl.fcta, pl.fwt, (TileSum*)(rbase + o_fsum), ctx->reg, ctx->dp, dl);
     launch(st, k_reduce_deferred, DEF_GRID, DEF_WARPS * 32, 0, d_desc, dl, ctx->reg, ctx->dp, now_ns);
   }
-  const DeferList dl_big{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
-  auto deferred_big = [&]() {
-    u32 n = 0;
-    for (int q = 0; q < 3; ++q) n = std::max(n, std::max(ctx->max_mid_n[q], ctx->max_large_n[q]));
-    launch(st, k_reduce_large_deferred, LARGE_DEF_GRID, LARGE_DEF_THREADS, 16ull * n, d_desc, dl_big, ctx->reg, ctx->dp, now_ns);
-  };
-  static_assert(MID_SEQS == LARGE_SEQS, "one list for the groups of both classes");
-  if (n_list[B_T2]) {
-    TimedLaunch tl(ts, 4, st);
-    const u32 grid = (u32)n_list[B_T2]; TileSum* sums = (TileSum*)(rbase + o_s2);
-    // one launch per padded size the registry has; a tile of another size ends at once
-    const u32* m = ctx->max_mid_n;
-    if (m[0]) launch(st, k_reduce_mid<8>, grid, MID_THREADS, mid_smem_bytes(m[0]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
-    if (m[1]) launch(st, k_reduce_mid<16>, grid, MID_THREADS, mid_smem_bytes(m[1]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
-    if (m[2]) launch(st, k_reduce_mid<32>, grid, MID_THREADS, mid_smem_bytes(m[2]), d_desc, pl.t2, sums, ctx->reg, ctx->dp, dl_big);
-    if (!n_list[B_T3]) deferred_big();
-  }
-  if (n_list[B_T3]) {
-    TimedLaunch tl(ts, 5, st);
-    const u32 grid = (u32)(n_list[B_T3] * LARGE_SEQS); TileSum* sums = (TileSum*)(rbase + o_s3);
-    const u32* m = ctx->max_large_n;
-    if (m[0]) launch_cluster(st, k_reduce_large<4>, LARGE_SEQS, grid, LQ_THREADS, large_smem(4), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
-    if (m[1]) launch_cluster(st, k_reduce_large<8>, LARGE_SEQS, grid, LQ_THREADS, large_smem(8), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
-    if (m[2]) launch_cluster(st, k_reduce_large<16>, LARGE_SEQS, grid, LQ_THREADS, large_smem(16), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
-    deferred_big();
-  }
+  On joined = chains.close();
+  if (chains.n > 0) deferred_big(joined);                  // its list is filled by two chains
   {
     TimedLaunch tl(ts, 6, st);
     const u32 ctas = (nc + WD_THREADS / 32 - 1) / (WD_THREADS / 32);
