@@ -172,7 +172,7 @@ struct OutPtrs { u8* flags; i64* gi64; u32* gu32; double* gbw; u64 G; };
 struct InPtrs { const u32* perm; const i64 *te, *tx; const u64* by; const u8* op; const u32 *sc, *rc; };
 template <class T> __device__ __forceinline__ T ld_volatile(const T& x) { return *(const volatile T*)&x; }
 
-constexpr u32 TILE_KEYS = 2304;                               // keys of a metric of a staged tile, padding included
+constexpr u32 TILE_KEYS = 8 * SMALL_SEQS;                     // keys of a metric of a staged tile
 constexpr u32 TILE_OPS = 64;                                  // op counters of a staged tile at most
 struct FusedShared {
   u32 cnt[SC_COUNT];
@@ -182,11 +182,17 @@ struct FusedShared {
   // staged tiles, per op counter: why the group is set aside (1) or its op set differs (2), latest exit, first member's
   u32 t_bits[TILE_OPS], t_xmax[TILE_OPS], t_gop[TILE_OPS];    //   op code,
   u64 t_base[TILE_OPS], t_gby[TILE_OPS];                      //   time base and size
-  u64 t_ck[SMALL_SEQS / 32][32];                              //   most changes, per warp
+  u64 t_ck[TILE_OPS];                                         //   most changes, then the lowest position
   double t_bd[TILE_OPS];                                      //   bytes * factor where the group adds bandwidth, else 0
   u32 mem[WARP_N];                                            // the communicator's ranks
   u32 brng[SMALL_SEQS / 32], bk[SMALL_SEQS / 32], rounds[SMALL_SEQS / 32], n_an[SMALL_SEQS / 32], n_def[SMALL_SEQS / 32];
 };
+
+// Three CTAs fit 64 KB of shared memory, which leaves 192 KB of an SM to its L1. How many lines L1 holds is how many gathers can
+// be on their way: on twelve windows of 4,096 ranks in groups of 8 and 64 the kernel takes 1,071 us with 28 KB of L1, 598 with
+// 121, 587 with 156 and 577 with 192; on records uploaded in arrival order 694, 275, 261 and 249.
+static_assert(CCLD_FUSED_MIN_CTAS * (sizeof(FusedShared) + 1024) <= 64 * 1024, "fits the 64 KB split (a CTA's first KB is the system's)");
+constexpr int FUSED_CARVEOUT = (int)((100 * CCLD_FUSED_MIN_CTAS * (sizeof(FusedShared) + 1024) + 228 * 1024 - 1) / (228 * 1024));     // percent
 
 __device__ __forceinline__ void flush_counters(const WinDesc& D, const FusedShared& sh) {
   count_add(D.counters, C_COMPLETE, sh.cnt[SC_COMP]); count_add(D.counters, C_BARRIER, sh.cnt[SC_BAR]); count_add(D.counters, C_ANALYSED, sh.cnt[SC_AN]);
@@ -479,18 +485,19 @@ __device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta
 // records per thread. A thread gathers op counter t % S of members t / S, t / S + L, ... - lanes along the op counter, so the
 // record indices of a warp are contiguous and, in a rank-major upload, its records lie in one short stretch of a rank's
 // stream - with one exposed round trip for times, sizes and op codes; the rate columns are on their way while the groups
-// are sorted. Keys meet in shared memory; then L lanes take a group, eight members each (position q L + s in lane s: with
-// the pitch below every access of a column is free of bank conflicts). Last, a thread sums eight op counters of one member's
+// are sorted. Keys meet in shared memory; then L lanes take a group, eight members each (position q L + s in lane s). Last, a thread sums eight op counters of one member's
 // bandwidth.
 template <int L, bool FULL>
 __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& t, TileSum* __restrict__ sums, const Registry& R, const Params& P,
                                               const DeferList& DL, FusedShared& sh) {
   constexpr u32 S = SMALL_SEQS / L, GW = 32 / L, NW = SMALL_SEQS / 32;
-  constexpr u32 PITCH = L == 4 ? 72 : (L == 8 ? 36 : 18);    // lane (s, j) of an access to a column: bank s PITCH + j, 32 different ones
-  static_assert(8 * L * PITCH <= TILE_KEYS && S <= TILE_OPS, "tile fits");
+  // Member p's key of op counter j lies at p S + (j ^ turn(p)): the lanes of an access, GW op counters of L members (or S of
+  // 32 / S), meet 32 different banks.
+  const auto turn = [](u32 p) { return L == 4 ? (p & 3u) << 3 : (L == 8 ? (p & 7u) << 2 : (p >> 1 & 7u) << 1); };
+  static_assert(8 * L * S == TILE_KEYS && S <= TILE_OPS, "tile fits");
   const u32 wid = threadIdx.x >> 5, lane = threadIdx.x & 31, n = FULL ? (u32)(8 * L) : t.row.n, count = t.count;
   u32* __restrict__ k_a = sh.stage; u32* __restrict__ k_d = sh.stage + TILE_KEYS;
-  if (threadIdx.x < S) { sh.t_bits[threadIdx.x] = 0; sh.t_xmax[threadIdx.x] = 0; }
+  if (threadIdx.x < S) { sh.t_bits[threadIdx.x] = 0; sh.t_xmax[threadIdx.x] = 0; sh.t_ck[threadIdx.x] = 0; }
   if (threadIdx.x < n) sh.mem[threadIdx.x] = __ldg(R.members + t.moff + threadIdx.x);
   __syncthreads();                                            // counters and pointers are set, the arrays above clear
   // ---- gather ----
@@ -524,7 +531,8 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
       hx |= (u32)(ra >> 32) | (u32)(rb >> 32);
       neg |= (u32)((u64)ta[q] >> 32) | (u32)((u64)tb[q] >> 32);
       back = back || b < a; xmax = max(xmax, b);
-      k_a[p * PITCH + sq] = FULL || p < n ? a : 0xFFFFFFFFu; k_d[p * PITCH + sq] = FULL || p < n ? b - a : 0xFFFFFFFFu;
+      const u32 k = p * S + (sq ^ turn(p));
+      k_a[k] = FULL || p < n ? a : 0xFFFFFFFFu; k_d[k] = FULL || p < n ? b - a : 0xFFFFFFFFu;
     }
     if (hx != 0 || (int)neg < 0 || back) bits |= 1;           // beyond 32 bits, negative or in flight, exit before enter
     u32 y = 0;
@@ -552,15 +560,16 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
     const bool gok = active && !(bits & 1), mm = (bits & 2) != 0;
     const bool barrier = gop == CCLD_OP_ALLREDUCE && gby < P.barrier_bytes;
     const bool round = gok && !barrier, analysed = round && n >= P.min_group;
-    const u32* __restrict__ ka = k_a + s * PITCH + jt; const u32* __restrict__ kd = k_d + s * PITCH + jt;     // member q L + s: q * L * PITCH further
+    const u32 mine = s * S + (jt ^ turn(s));                  // member q L + s: 256 q further
+    const u32* __restrict__ ka = k_a + mine; const u32* __restrict__ kd = k_d + mine;
     u32 emin, emax, ms, ds, tmn, tmx, md, dm;
     {
       u32 v[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = ka[q * L * PITCH];
+      for (int q = 0; q < 8; ++q) v[q] = ka[q * SMALL_SEQS];
       sub_stats<L, FULL>(v, n, s, lane, &emin, &emax, &ms, &ds);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = kd[q * L * PITCH];
+      for (int q = 0; q < 8; ++q) v[q] = kd[q * SMALL_SEQS];
       sub_stats<L, FULL>(v, n, s, lane, &tmn, &tmx, &md, &dm);
     }
     ms -= emin; md -= tmn;
@@ -578,7 +587,7 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
 #pragma unroll
       for (int q = 7; q >= 0; --q) {
         if (!FULL && q * L + s >= n) continue;
-        const u32 a = ka[q * L * PITCH], d = kd[q * L * PITCH];
+        const u32 a = ka[q * SMALL_SEQS], d = kd[q * SMALL_SEQS];
         u32 f = a - s0 > ws ? (u32)CCLD_F_SKEW_OUT : 0u;
         if (d - d0 > wd) f |= CCLD_F_DUR_OUT;
         if (a > sm) f |= CCLD_F_SKEW_HI;
@@ -648,17 +657,14 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
     }
 #pragma unroll
     for (u32 h = S; h < 32; h <<= 1) { const u64 o = shfl_xor64(ck, h); ck = o > ck ? o : ck; }
-    sh.t_ck[wid][lane] = ck;
+    if (S >= 32 || lane < S) atomicMax((unsigned long long*)&sh.t_ck[sq], (unsigned long long)ck);
   }
   __syncthreads();
   u32 rounds = 0;
 #pragma unroll
   for (u32 q = 0; q < NW; ++q) rounds += sh.rounds[q];
   if (threadIdx.x < count && !(sh.t_bits[threadIdx.x] & 1)) {
-    u64 ck = 0;
-    constexpr u32 W0 = S / 32 ? S / 32 : 1;                   // warps that cover all op counters once
-#pragma unroll
-    for (u32 w = 0; w < NW; w += W0) { const u64 o = sh.t_ck[w + threadIdx.x / 32 % W0][threadIdx.x & 31]; ck = o > ck ? o : ck; }
+    const u64 ck = sh.t_ck[threadIdx.x];
     const u64 g = t.row.group0 + t.seq_off + threadIdx.x, G = ld_volatile(sh.out.G);
     u32* __restrict__ gu = ld_volatile(sh.out.gu32) + g;
     gu[(u64)GU_MAX_CHG * G] = (u32)(ck >> 32); gu[(u64)GU_RANK_MAX_CHG * G] = sh.mem[NONE - (u32)ck];
@@ -670,7 +676,7 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
     if (FULL || p < n) {
 #pragma unroll
       for (u32 i = 0; i < 8; ++i) {
-        const u32 o = part + TPM * i, d = k_d[p * PITCH + o];
+        const u32 o = part + TPM * i, d = k_d[p * S + (o ^ turn(p))];
         const double bd = o < count ? sh.t_bd[o] : 0.0;
         if (bd != 0.0 && d != 0) v += bd * rcp_u32(d);
       }

@@ -411,6 +411,9 @@ int finalize_registry(ccld_ctx* ctx) {
   CK(cudaFuncSetAttribute(k_seq_range, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)range_smem_bytes(RANGE_DIRECT)));
   CK(cudaFuncSetAttribute(k_hang_locate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(HANG_SMEM_N * HANG_MEMBER_BYTES)));
   CK(cudaFuncSetAttribute(k_opset_check, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(CCLD_MAX_COMM_SIZE * OPSET_MEMBER_BYTES)));
+  // The gathers of the small groups are held up by the cache lines an SM can have on their way: no more shared memory than the
+  // CTAs need, the rest of the SM's 256 KB is L1. (The other kernels are best off with the driver's own choice.)
+  CK(cudaFuncSetAttribute(k_reduce_fused, cudaFuncAttributePreferredSharedMemoryCarveout, FUSED_CARVEOUT));
   CK(cudaFuncSetAttribute(k_reduce_large<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(4)));
   CK(cudaFuncSetAttribute(k_reduce_large<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(8)));
   CK(cudaFuncSetAttribute(k_reduce_large<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(16)));
