@@ -502,28 +502,44 @@ __device__ __forceinline__ RoundPart rounds_of(const WinDesc& D, const RangeRow&
   return x;
 }
 
-// Analysed ops of a window count towards every member's denominator: the CTA's communicators one after the other, all
-// threads along the members (a warp alone took 20 us over a communicator of 4,096).
-__device__ __forceinline__ void count_ops(const Registry& R, u32 c0, const u32* __restrict__ s_an) {
-  for (u32 q = 0; q < WD_THREADS / 32; ++q) {
-    const u32 n_an = s_an[q];
-    if (n_an == 0) continue;
-    const u32 n = R.comm_n[c0 + q];
-    const u32* __restrict__ mem = R.members + R.comm_moff[c0 + q];
-#pragma unroll 4
-    for (u32 p = threadIdx.x; p < n; p += WD_THREADS) atomicAdd(&R.ops[mem[p]], n_an);
+// Analysed ops of a window count towards every member's denominator. A warp goes along the members of its communicator; one
+// of more than OPS_WARP is left to all warps of the CTA, when they have met (a warp alone took 20 us over a communicator of
+// 4,096). Bound by latency: sixteen members per thread are looked up at a time, and what the lookups need was left in shared
+// memory (four at a time, behind three more loads: the whole kernel took 45.6 us instead of 21.0 on a window of 16,384 ranks with
+// communicators of up to 2,048, and 23.5 instead of 18.9 on two windows of one communicator of 4,096).
+constexpr u32 OPS_WARP = 512;
+struct OpsShared { u32 n_an[WD_THREADS / 32], n[WD_THREADS / 32]; u64 moff[WD_THREADS / 32]; };
+template <u32 THREADS> __device__ __forceinline__ void add_ops(const Registry& R, u64 moff, u32 n, u32 n_an, u32 first) {
+  constexpr u32 AHEAD = 16;
+  const u32* __restrict__ mem = R.members + moff;
+  for (u32 p0 = first; p0 < n; p0 += THREADS * AHEAD) {
+    u32 r[AHEAD];
+#pragma unroll
+    for (u32 u = 0; u < AHEAD; ++u) r[u] = p0 + u * THREADS < n ? __ldg(mem + p0 + u * THREADS) : NONE;
+#pragma unroll
+    for (u32 u = 0; u < AHEAD; ++u) if (r[u] != NONE) atomicAdd(&R.ops[r[u]], n_an);
   }
+}
+// All threads of the CTA; a warp brings its communicator's analysed ops, members and their place.
+__device__ __forceinline__ void count_ops(const Registry& R, OpsShared& sh, u32 n_an, u32 n, u64 moff) {
+  const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const bool all = n_an != 0 && n > OPS_WARP;
+  if (lane == 0) { sh.n_an[wid] = all ? n_an : 0u; sh.n[wid] = n; sh.moff[wid] = moff; }
+  if (n_an != 0 && !all) add_ops<32>(R, moff, n, n_an, lane);
+  if (!__syncthreads_or(all)) return;
+  for (u32 q = 0; q < WD_THREADS / 32; ++q) if (sh.n_an[q] != 0) add_ops<WD_THREADS>(R, sh.moff[q], sh.n[q], sh.n_an[q], threadIdx.x);
 }
 
 // Stage 1 of a batch of several windows, all at once: leaves the part above in the communicator's verdict row.
 __global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* __restrict__ wd, Registry R) {
   begin_after();
-  __shared__ u32 s_an[WD_THREADS / 32];
-  const u32 c0 = blockIdx.x * (WD_THREADS / 32), wid = threadIdx.x >> 5, c = c0 + wid, lane = threadIdx.x & 31;
+  __shared__ OpsShared s_ops;
+  const u32 c = blockIdx.x * (WD_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const WinDesc& D = wd[blockIdx.y];
-  u32 n_an = 0;
+  u32 n_an = 0, n = 0; u64 moff = 0;
   if (c < R.n_comms) {
     const RangeRow row = D.ranges[c];
+    n = row.n; moff = R.comm_moff[c];
     const RoundPart x = rounds_of(D, row, lane, &n_an);
     if (lane == 0 && row.n_seq) {
       ccld_comm_verdict* v = D.comm_rows + row.row_idx;
@@ -531,9 +547,7 @@ __global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* __r
       v->t_max = x.t_max; v->t_min = x.t_min;
     }
   }
-  if (lane == 0) s_an[wid] = n_an;
-  __syncthreads();
-  count_ops(R, c0, s_an);
+  count_ops(R, s_ops, n_an, n, moff);
 }
 
 // Stage 2, windows in order: the recurrences - Eq. 1's baseline, which reads the per-op rows until m is fixed, and the
@@ -543,11 +557,12 @@ __global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* __r
 template <bool SINGLE>
 __global__ void __launch_bounds__(WD_THREADS) k_window_decide(const WinDesc* __restrict__ wd, u32 nw, Registry R, Params P) {
   begin_after();
-  __shared__ u32 s_an[WD_THREADS / 32];
-  const u32 c0 = blockIdx.x * (WD_THREADS / 32), wid = threadIdx.x >> 5, c = c0 + wid, lane = threadIdx.x & 31;
-  u32 n_an = 0;
+  __shared__ OpsShared s_ops;
+  const u32 c = blockIdx.x * (WD_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  u32 n_an = 0, n = 0; u64 moff = 0;
   if (c < R.n_comms) {
     CommState st = R.state[c];
+    if (SINGLE) moff = R.comm_moff[c];
     struct Res { const RangeRow* ranges; u64 n_groups; const i64* gi64; const u32* gu32; ccld_comm_verdict* comm_rows; };   // pointers of a window
     // three steps, each on values fetched during an earlier window: descriptor -> range row -> stage-1 row
     auto load_res = [&](u32 w) {
@@ -568,7 +583,7 @@ __global__ void __launch_bounds__(WD_THREADS) k_window_decide(const WinDesc* __r
     Res res_a = load_res(0), res_b = load_res(1), res_c = load_res(2);
     RangeRow row_a = load_row(res_a), row_b = load_row(res_b);
     RoundPart part_a;
-    if (SINGLE) part_a = rounds_of(wd[0], row_a, lane, &n_an); else part_a = load_part(res_a, row_a);
+    if (SINGLE) { n = row_a.n; part_a = rounds_of(wd[0], row_a, lane, &n_an); } else part_a = load_part(res_a, row_a);
     for (u32 w = 0; w < nw; ++w) {
       const RangeRow row = row_a; const Res D = res_a; const RoundPart pt = part_a;
       if (!SINGLE) {
@@ -636,9 +651,7 @@ __global__ void __launch_bounds__(WD_THREADS) k_window_decide(const WinDesc* __r
     if (lane == 0) R.state[c] = st;
   }
   if (!SINGLE) return;
-  if (lane == 0) s_an[wid] = n_an;
-  __syncthreads();
-  count_ops(R, c0, s_an);
+  count_ops(R, s_ops, n_an, n, moff);
 }
 
 }  // namespace ccld
