@@ -70,10 +70,6 @@ class Verdict(C.Structure):
                 ("suspects", C.POINTER(Suspect)), ("suspects_cap", C.c_uint32)]
 
 
-class VerdictColumns(C.Structure):
-    _fields_ = [(k, C.c_void_p) for k in ("rows", "alerts", "suspects")] + [(k, C.c_uint32) for k in ("n_rows", "n_alerts", "n_suspects", "pad")]
-
-
 class HangVerdict(C.Structure):
     _fields_ = [(k, C.c_uint32) for k in ("cls", "n_roots_total", "n_not_entered", "n_hung", "n_not_hung",
                                            "n_missing_frames", "stuck_step", "n_members")] + \
@@ -97,51 +93,33 @@ class OpTable(C.Structure):
                [(k, C.c_void_p) for k in OPTABLE_U32] + [("busbw", C.c_void_p), ("flags", C.c_void_p), ("perm", C.c_void_p)]
 
 
-class HostBlock(C.Structure):
-    _fields_ = [("p", C.c_void_p), ("bytes", C.c_uint64)]
-
-
-class HostOpTable(C.Structure):
-    _fields_ = [("t", OpTable), ("comm", C.c_void_p), ("seq", C.c_void_p), ("slot0", C.c_void_p), ("block", HostBlock)]
-
-
-class HostRankStats(C.Structure):
-    _fields_ = [(k, C.c_void_p) for k in ("votes", "ops", "bw_cnt", "bw_sum")] + [("block", HostBlock)]
-
-
 class CommRange(C.Structure):
     _fields_ = [("comm", C.c_uint32), ("n", C.c_uint32), ("seq_lo", C.c_uint32), ("n_seq", C.c_uint32),
                 ("group0", C.c_uint64), ("slot0", C.c_uint64)]
 
 
-_TABLE_DTYPES = [(k, np.int64) for k in OPTABLE_I64] + [(k, np.uint32) for k in OPTABLE_U32] + [("busbw", np.float64)]
 _NO_BLOCK = (-2, -8)                  # no pinned block to be had: the copying accessors serve
 _NP_OF = {C.c_uint32: "u4", C.c_uint64: "u8", C.c_int64: "i8", C.c_double: "f8"}
 
 
 def _column_plan(struct):
-    """Field names in order, runs of equal types among the columns (64-bit ones first) as (names, dtype, bytes of an entry that
-    lie before the run), bytes of an entry, and the fields of an empty list."""
+    """The fields of a list that the library holds column by column (64-bit ones first): name, kind, bytes, and bytes of an entry
+    that lie before the column; in the order of the struct."""
     dt = {k: np.dtype(_NP_OF[t]) for k, t in struct._fields_}
-    order = [k for k in dt if dt[k].itemsize == 8] + [k for k in dt if dt[k].itemsize == 4]
-    runs, at = [], 0
-    for k in order:
-        if runs and runs[-1][1] == dt[k]:
-            runs[-1][0].append(k)
-        else:
-            runs.append(([k], dt[k], at))
-        at += dt[k].itemsize
-    return tuple(dt), runs, at, dt
+    at, pos = {}, 0
+    for k in sorted(dt, key=lambda k: -dt[k].itemsize):
+        at[k] = pos
+        pos += dt[k].itemsize
+    return tuple((k, dt[k].kind, dt[k].itemsize, at[k]) for k in dt)
 
 
-_ROW_PLAN, _ALERT_PLAN, _SUSPECT_PLAN = _column_plan(CommVerdict), _column_plan(HangAlert), _column_plan(Suspect)
 _VERDICT_KEYS = tuple(k for k, _ in Verdict._fields_[:15])
-_lib = None
+_lib = _native = None
 
 
 def load_library() -> C.CDLL:
     """Loads libccld.so; raises if it has not been built (python -m paper_2605_04478_b200.build)."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(f"{LIB_PATH} is missing: build it with `python -m paper_2605_04478_b200.build`; "
@@ -174,18 +152,22 @@ def load_library() -> C.CDLL:
         lib.ccld_get_ranges.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_uint32, C.POINTER(C.c_uint32)]
         lib.ccld_get_rank_stats.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_copy_to_host.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_uint64]
-        lib.ccld_get_verdict_columns.argtypes = [C.c_void_p, C.c_uint32, C.POINTER(Verdict), C.POINTER(VerdictColumns)]
-        lib.ccld_take_optable.argtypes = [C.c_void_p, C.c_uint32, C.POINTER(HostOpTable)]
-        lib.ccld_take_rank_stats.argtypes = [C.c_void_p, C.c_uint32, C.POINTER(HostRankStats)]
-        lib.ccld_host_release.restype = None
-        lib.ccld_host_release.argtypes = [C.POINTER(HostBlock)]
         lib.ccld_copy_many_to_host.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_derive_rates.argtypes = [C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p, C.c_uint32, C.c_uint64] + [C.c_void_p] * 6
         lib.ccld_timing_enable.argtypes = [C.c_void_p, C.c_int]
         lib.ccld_get_kernel_times.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p]
         lib.ccld_ring_locate_static.argtypes = [C.c_int, C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_uint32, C.c_void_p,
                                                 C.POINTER(HangVerdict), C.c_char_p, C.c_uint32]
-        _lib = lib
+        try:
+            from . import _binding
+        except ImportError as e:
+            raise RuntimeError(f"the binding's compiled module cannot be loaded ({e}): build it with "
+                               "`python -m paper_2605_04478_b200.build`") from e
+        address = lambda f: C.cast(f, C.c_void_p).value
+        _binding.setup(tuple(address(getattr(lib, k)) for k in ("ccld_get_verdict_columns", "ccld_trace_upload", "ccld_take_optable",
+                                                                "ccld_take_rank_stats", "ccld_host_release")),
+                       _VERDICT_KEYS, tuple(_COL_DTYPES), _column_plan(CommVerdict), _column_plan(HangAlert), _column_plan(Suspect))
+        _lib, _native = lib, _binding
     return _lib
 
 
@@ -218,19 +200,6 @@ def _as_tensor(torch, v, dt):
     if a.dtype != np.dtype(dt):
         a = a.view(dt) if a.dtype.itemsize == np.dtype(dt).itemsize else a.astype(dt)
     return torch.from_numpy(a)
-
-
-class _Pinned:
-    """A pinned block of the library as an array buffer; given back once no array refers to it any more."""
-    __slots__ = ("block", "__array_interface__")
-
-    def __init__(self, block):
-        self.block = HostBlock(block.p, block.bytes)
-        self.__array_interface__ = {"shape": (block.bytes,), "typestr": "|u1", "data": (block.p, False), "version": 3}
-
-    def __del__(self):
-        if _lib is not None:
-            _lib.ccld_host_release(C.byref(self.block))
 
 
 def ring_locate_static(ranks, state, progress=None, device: int = 0, stream=None, roots_cap: int = STATIC_MAX_MEMBERS):
@@ -333,6 +302,12 @@ class Analyzer:
 
     def trace_upload(self, window_id: int, cols, frames=None, n_channels: int = 0) -> None:
         """cols: dict of torch tensors or numpy arrays, all on the CPU (copied) or all on this GPU (borrowed)."""
+        if frames is None and type(cols) is dict:
+            done = _native.upload(self.h.value or 0, window_id, cols)        # None: not all plain numpy columns
+            if done is not None:
+                self._check(done[0])
+                self._keep[window_id] = done[1]    # pinned host memory stays alive
+                return
         torch = self.torch
         keep, ptrs, cuda, n = [], [], set(), 0
         for k, dt, size in _COLS:
@@ -386,19 +361,6 @@ class Analyzer:
         a = a[:count]
         return {k: a[k].copy() for k in a.dtype.names}
 
-    @staticmethod
-    def _take(ptr, n, cap, plan):
-        """A list of n entries that the library holds column by column, as one array per field (the first `cap` entries)."""
-        names, runs, size, dtypes = plan
-        if n == 0:
-            return {k: np.empty(0, dt) for k, dt in dtypes.items()}
-        buf = np.empty(n * size, np.uint8)
-        C.memmove(_address(buf), ptr, n * size)
-        out = dict.fromkeys(names)
-        for keys, dt, at in runs:
-            out.update(zip(keys, np.frombuffer(buf, dt, len(keys) * n, at * n).reshape(len(keys), n)))
-        return out if cap >= n else {k: a[:cap] for k, a in out.items()}
-
     def _list_buf(self, struct, cap):
         """Room for `cap` entries of a C struct. Kept between calls: the library writes only the entries there are, and a fresh
         buffer of a default capacity would be zeroed and faulted in on every call."""
@@ -409,15 +371,9 @@ class Analyzer:
 
     def get_verdict(self, window_id: int, comm_rows_cap: int = 1 << 16, alerts_cap: int = MAX_ALERTS_PER_WINDOW,
                     suspects_cap: int = 1 << 16, check: bool = True) -> Dict[str, object]:
-        v, c = Verdict(), VerdictColumns()
-        rc = self.lib.ccld_get_verdict_columns(self.h, window_id, C.byref(v), C.byref(c))
+        out = _native.verdict(self.h.value or 0, window_id, comm_rows_cap, alerts_cap, suspects_cap)
         if check:
-            self._check(rc)
-        out: Dict[str, object] = {k: getattr(v, k) for k in _VERDICT_KEYS}
-        out["rc"] = rc
-        out["comm_rows"] = self._take(c.rows, c.n_rows, comm_rows_cap, _ROW_PLAN)
-        out["alerts"] = self._take(c.alerts, c.n_alerts, alerts_cap, _ALERT_PLAN)
-        out["suspects"] = self._take(c.suspects, c.n_suspects, suspects_cap, _SUSPECT_PLAN)
+            self._check(out["rc"])
         return out
 
     def locate_hang(self, window_id: int, comm: int, seq: int, roots_cap: int = MAX_COMM_SIZE) -> Dict[str, object]:
@@ -492,19 +448,8 @@ class Analyzer:
     def get_optable(self, window_id: int, to_host: bool = True) -> Dict[str, object]:
         """Per-op table of an analysed window; with to_host the columns come back as numpy arrays."""
         if to_host:
-            h = HostOpTable()
-            rc = self.lib.ccld_take_optable(self.h, window_id, C.byref(h))
+            rc, out = _native.optable(self.h.value or 0, window_id)
             if rc == OK:
-                t, first = h.t, h.block.p
-                G, S = t.n_groups, t.n_slots
-                buf = np.asarray(_Pinned(h.block))
-                out: Dict[str, object] = {"n_groups": G, "n_slots": S}
-                for k, dt in _TABLE_DTYPES:
-                    out[k] = np.frombuffer(buf, dt, G, getattr(t, k) - first) if G else np.empty(0, dt)
-                for k, dt in (("flags", np.uint8), ("perm", np.uint32)):
-                    out[k] = np.frombuffer(buf, dt, S, getattr(t, k) - first) if S else np.empty(0, dt)
-                for k, dt in (("comm", np.uint32), ("seq", np.uint32), ("slot0", np.uint64)):
-                    out[k] = np.frombuffer(buf, dt, G, getattr(h, k) - first) if G else np.empty(0, dt)
                 return out
             if rc not in _NO_BLOCK:
                 self._check(rc)
@@ -554,13 +499,9 @@ class Analyzer:
         return out_s, out_r
 
     def get_rank_stats(self, n_ranks: int) -> Dict[str, np.ndarray]:
-        h = HostRankStats()
-        rc = self.lib.ccld_take_rank_stats(self.h, n_ranks, C.byref(h))
+        rc, out = _native.rank_stats(self.h.value or 0, n_ranks)
         if rc == OK:
-            buf, first = np.asarray(_Pinned(h.block)), h.block.p
-            return {"votes": np.frombuffer(buf, np.uint32, n_ranks * 4, h.votes - first).reshape(n_ranks, 4),
-                    "ops": np.frombuffer(buf, np.uint32, n_ranks, h.ops - first), "bw_cnt": np.frombuffer(buf, np.uint32, n_ranks, h.bw_cnt - first),
-                    "bw_sum": np.frombuffer(buf, np.float64, n_ranks, h.bw_sum - first)}
+            return out
         if rc not in _NO_BLOCK:
             self._check(rc)
         votes = np.empty((n_ranks, 4), np.uint32); ops = np.empty(n_ranks, np.uint32)
