@@ -76,7 +76,6 @@ class HangVerdict(C.Structure):
                [("min_total", C.c_uint64), ("roots", C.POINTER(C.c_uint32)), ("roots_cap", C.c_uint32)]
 
 
-_HANG_KEYS = ("cls", "n_roots_total", "n_not_entered", "n_hung", "n_not_hung", "n_missing_frames", "stuck_step", "n_members", "min_total")
 
 OPTABLE_I64 = ("e_min", "arrival_skew", "t_max", "t_min", "span", "med_skew", "mad_skew", "med_dur", "mad_dur")
 OPTABLE_U32 = ("rank_tmin", "rank_tmax", "max_chg", "rank_max_chg", "n_present", "gflags")
@@ -165,7 +164,9 @@ def load_library() -> C.CDLL:
                                "`python -m paper_2605_04478_b200.build`") from e
         address = lambda f: C.cast(f, C.c_void_p).value
         _binding.setup(tuple(address(getattr(lib, k)) for k in ("ccld_get_verdict_columns", "ccld_trace_upload", "ccld_take_optable",
-                                                                "ccld_take_rank_stats", "ccld_host_release")),
+                                                                "ccld_take_rank_stats", "ccld_host_release", "ccld_get_optable",
+                                                                "ccld_locate_hang", "ccld_locate_hangs", "ccld_opset_check",
+                                                                "ccld_derive_rates", "ccld_get_ranges")),
                        _VERDICT_KEYS, tuple(_COL_DTYPES), _column_plan(CommVerdict), _column_plan(HangAlert), _column_plan(Suspect))
         _lib, _native = lib, _binding
     return _lib
@@ -253,9 +254,6 @@ class Analyzer:
         if rc != OK:
             raise CcldError(rc, "ccld_create failed")
         self._keep: Dict[int, list] = {}
-        self._bufs: Dict[type, np.ndarray] = {}
-        self._ranks = np.empty(1, np.uint32)
-        self._hang_buf = None
         self._n_comms = 0
 
     # -- helpers
@@ -283,12 +281,6 @@ class Analyzer:
         size = (C.c_uint64 * k)(*[a.nbytes for a in out])
         self._check(self.lib.ccld_copy_many_to_host(self.h, k, dst, src, size))
         return out
-
-    def _rank_buf(self, n):
-        """Room for n rank ids, kept between calls like the lists above."""
-        if len(self._ranks) < n:
-            self._ranks = np.empty(n, np.uint32)
-        return self._ranks
 
     # -- the boundary
     def comm_register(self, comm: int, ranks, algo: int = 0, seq0: int = 0) -> None:
@@ -355,20 +347,6 @@ class Analyzer:
     def set_speculation(self, on: bool) -> None:
         self._check(self.lib.ccld_set_speculation(self.h, 1 if on else 0))
 
-    @staticmethod
-    def _columns(a, count):
-        """The first `count` entries of a structured array as one array per field."""
-        a = a[:count]
-        return {k: a[k].copy() for k in a.dtype.names}
-
-    def _list_buf(self, struct, cap):
-        """Room for `cap` entries of a C struct. Kept between calls: the library writes only the entries there are, and a fresh
-        buffer of a default capacity would be zeroed and faulted in on every call."""
-        b = self._bufs.get(struct)
-        if b is None or len(b) < cap:
-            b = self._bufs[struct] = np.empty(max(cap, 1), np.dtype([(k, _NP_OF[t]) for k, t in struct._fields_]))
-        return b
-
     def get_verdict(self, window_id: int, comm_rows_cap: int = 1 << 16, alerts_cap: int = MAX_ALERTS_PER_WINDOW,
                     suspects_cap: int = 1 << 16, check: bool = True) -> Dict[str, object]:
         out = _native.verdict(self.h.value or 0, window_id, comm_rows_cap, alerts_cap, suspects_cap)
@@ -377,35 +355,16 @@ class Analyzer:
         return out
 
     def locate_hang(self, window_id: int, comm: int, seq: int, roots_cap: int = MAX_COMM_SIZE) -> Dict[str, object]:
-        roots = self._rank_buf(roots_cap)
-        hv = HangVerdict()
-        hv.roots = C.cast(roots.ctypes.data, C.POINTER(C.c_uint32)); hv.roots_cap = roots_cap
-        self._check(self.lib.ccld_locate_hang(self.h, window_id, comm, seq, C.byref(hv)))
-        out: Dict[str, object] = {k: int(getattr(hv, k)) for k in _HANG_KEYS}
-        out["roots"] = roots[:min(hv.n_roots_total, roots_cap)].copy()
+        rc, out = _native.hang(self.h.value or 0, window_id, comm, seq, roots_cap)
+        self._check(rc)
         return out
 
     def locate_hangs(self, window_id: int, cap: int = 1024, roots_stride: int = 64) -> List[Dict[str, object]]:
         """ccld_locate_hangs: the hang verdict of every alert of the window, one launch; each dict also carries the alert's
         comm, seq and age_ns."""
-        n = C.c_uint32(0)
-        cap = max(cap, 1)
-        hv = self._hang_buf
-        if hv is None or len(hv) < cap:
-            hv = self._hang_buf = (HangVerdict * cap)()
-        al = self._list_buf(HangAlert, cap)
-        roots = self._rank_buf(cap * max(roots_stride, 1))
-        if cap > MAX_ALERTS_PER_WINDOW:                          # alerts beyond those kept are listed as zeros
-            C.memset(hv, 0, C.sizeof(hv)); al[:] = 0
-        self._check(self.lib.ccld_locate_hangs(self.h, window_id, al.ctypes.data, C.cast(hv, C.c_void_p), cap, roots.ctypes.data, roots_stride, C.byref(n)))
-        res = []
-        for i in range(min(n.value, cap)):
-            v = hv[i]
-            d: Dict[str, object] = {k: int(getattr(v, k)) for k in _HANG_KEYS}
-            d["roots"] = roots[i * roots_stride:i * roots_stride + min(v.n_roots_total, roots_stride)].copy()
-            d["comm"], d["seq"], d["age_ns"] = int(al["comm"][i]), int(al["seq"][i]), int(al["age_ns"][i])
-            res.append(d)
-        return res
+        rc, out = _native.hangs(self.h.value or 0, window_id, cap, roots_stride)
+        self._check(rc)
+        return out
 
     def trace_attach_opset(self, window_id: int, algo, proto) -> None:
         """ccld_trace_attach_opset: algorithm and protocol codes per record (uint8), host (copied) or this GPU (borrowed)."""
@@ -418,13 +377,8 @@ class Analyzer:
 
     def opset_check(self, window_id: int, comm: int, seq: int, ranks_cap: int = MAX_COMM_SIZE) -> Dict[str, object]:
         """ccld_opset_check: majority Operation Type Set of op (comm, seq) and the ranks that deviate from it."""
-        ranks = self._rank_buf(ranks_cap)
-        v = OpsetVerdict()
-        v.ranks = C.cast(ranks.ctypes.data, C.POINTER(C.c_uint32)); v.ranks_cap = ranks_cap
-        self._check(self.lib.ccld_opset_check(self.h, window_id, comm, seq, C.byref(v)))
-        out: Dict[str, object] = {k: int(getattr(v, k)) for k in ("n_members", "n_present", "n_deviating_total", "majority_count",
-                                                                "op", "algo", "proto", "bytes")}
-        out["ranks"] = ranks[:min(v.n_deviating_total, ranks_cap)].copy()
+        rc, out = _native.opset(self.h.value or 0, window_id, comm, seq, ranks_cap)
+        self._check(rc)
         return out
 
     def state_export(self) -> bytes:
@@ -440,10 +394,9 @@ class Analyzer:
         self._check(self.lib.ccld_state_import(self.h, C.cast(buf, C.c_void_p), len(blob)))
 
     def get_ranges(self, window_id: int) -> Dict[str, np.ndarray]:
-        n = C.c_uint32(0)
-        rows = self._list_buf(CommRange, self._n_comms)          # a window has at most one row per communicator
-        self._check(self.lib.ccld_get_ranges(self.h, window_id, rows.ctypes.data, self._n_comms, C.byref(n)))
-        return self._columns(rows, n.value)
+        rc, out = _native.ranges(self.h.value or 0, window_id, self._n_comms)      # a window has at most one row per communicator
+        self._check(rc)
+        return out
 
     def get_optable(self, window_id: int, to_host: bool = True) -> Dict[str, object]:
         """Per-op table of an analysed window; with to_host the columns come back as numpy arrays."""
@@ -453,14 +406,14 @@ class Analyzer:
                 return out
             if rc not in _NO_BLOCK:
                 self._check(rc)
-        t = OpTable()
-        self._check(self.lib.ccld_get_optable(self.h, window_id, C.byref(t)))
-        G, S = int(t.n_groups), int(t.n_slots)
+        rc, t = _native.table(self.h.value or 0, window_id)
+        self._check(rc)
         if not to_host:
-            return {k: getattr(t, k) for k, _ in OpTable._fields_}
+            return t
+        G, S = t["n_groups"], t["n_slots"]
         out = {"n_groups": G, "n_slots": S}
         cols = [(k, G, np.int64) for k in OPTABLE_I64] + [(k, G, np.uint32) for k in OPTABLE_U32] + [("busbw", G, np.float64), ("flags", S, np.uint8), ("perm", S, np.uint32)]
-        for (k, _, _), a in zip(cols, self._to_host([(getattr(t, k), n, dt) for k, n, dt in cols])):
+        for (k, _, _), a in zip(cols, self._to_host([(t[k], n, dt) for k, n, dt in cols])):
             out[k] = a
         # per-group communicator id, op counter and first slot, expanded from the range rows
         r = self.get_ranges(window_id)
@@ -493,8 +446,8 @@ class Analyzer:
         n = cols[0].numel()
         out_s = torch.empty(n, dtype=torch.int32, device=cols[0].device); out_r = torch.empty_like(out_s)
         p = [c.data_ptr() for c in cols]                   # (null for an empty tensor)
-        self._check(self.lib.ccld_derive_rates(self.h, n, p[0], p[1], p[2], cols[3].numel() - 1, cols[4].numel(), p[3], p[4], p[5], p[6],
-                                               out_s.data_ptr(), out_r.data_ptr()))
+        self._check(_native.rates(self.h.value or 0, n, p[0], p[1], p[2], cols[3].numel() - 1, cols[4].numel(), p[3], p[4], p[5], p[6],
+                                  out_s.data_ptr(), out_r.data_ptr()))
         self._rate_keep = cols                     # inputs stay alive until the next call or a synchronization
         return out_s, out_r
 

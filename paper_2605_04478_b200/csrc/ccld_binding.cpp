@@ -19,6 +19,12 @@ decltype(&ccld_trace_upload) f_upload = nullptr;
 decltype(&ccld_take_optable) f_optable = nullptr;
 decltype(&ccld_take_rank_stats) f_stats = nullptr;
 decltype(&ccld_host_release) f_release = nullptr;
+decltype(&ccld_get_optable) f_table = nullptr;
+decltype(&ccld_locate_hang) f_hang = nullptr;
+decltype(&ccld_locate_hangs) f_hangs = nullptr;
+decltype(&ccld_opset_check) f_opset = nullptr;
+decltype(&ccld_derive_rates) f_rates = nullptr;
+decltype(&ccld_get_ranges) f_ranges = nullptr;
 
 struct Column { PyObject* name; int type; Py_ssize_t at; };            // at: bytes of an entry before the column
 struct Plan { std::vector<Column> cols; Py_ssize_t size = 0; };        // in the order of the dictionary; size: bytes of an entry
@@ -110,13 +116,15 @@ bool read_names(PyObject* seq, PyObject** to, Py_ssize_t n) {
 
 // setup(addresses, verdict names, upload names, rows, alerts, suspects)
 PyObject* setup(PyObject*, PyObject* args) {
-  unsigned long long a[5];
+  unsigned long long a[11];
   PyObject *v, *u, *r, *al, *s;
-  if (!PyArg_ParseTuple(args, "(KKKKK)O!O!O!O!O!", &a[0], &a[1], &a[2], &a[3], &a[4], &PyTuple_Type, &v, &PyTuple_Type, &u,
+  if (!PyArg_ParseTuple(args, "(KKKKKKKKKKK)O!O!O!O!O!", &a[0], &a[1], &a[2], &a[3], &a[4], &a[5], &a[6], &a[7], &a[8], &a[9], &a[10], &PyTuple_Type, &v, &PyTuple_Type, &u,
                         &PyTuple_Type, &r, &PyTuple_Type, &al, &PyTuple_Type, &s)) return nullptr;
   if (!read_names(v, n_verdict, 15) || !read_names(u, n_upload, 9) || !read_plan(r, p_rows) || !read_plan(al, p_alerts) || !read_plan(s, p_suspects)) return nullptr;
   f_verdict = (decltype(f_verdict))a[0]; f_upload = (decltype(f_upload))a[1]; f_optable = (decltype(f_optable))a[2];
   f_stats = (decltype(f_stats))a[3]; f_release = (decltype(f_release))a[4];
+  f_table = (decltype(f_table))a[5]; f_hang = (decltype(f_hang))a[6]; f_hangs = (decltype(f_hangs))a[7]; f_opset = (decltype(f_opset))a[8];
+  f_rates = (decltype(f_rates))a[9]; f_ranges = (decltype(f_ranges))a[10];
   n_rc = PyUnicode_InternFromString("rc"); n_comm_rows = PyUnicode_InternFromString("comm_rows");
   n_alerts = PyUnicode_InternFromString("alerts"); n_suspects = PyUnicode_InternFromString("suspects");
   Py_RETURN_NONE;
@@ -233,11 +241,189 @@ PyObject* optable(PyObject*, PyObject* args) {
   return Py_BuildValue("(iN)", rc, out);
 }
 
+// table(context, window) -> (return code, dictionary of counts and device addresses); a null address is None
+PyObject* table(PyObject*, PyObject* args) {
+  unsigned long long h; unsigned int window;
+  if (!PyArg_ParseTuple(args, "KI", &h, &window)) return nullptr;
+  ccld_optable t;
+  std::memset(&t, 0, sizeof t);
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = f_table((ccld_ctx*)h, window, &t);
+  Py_END_ALLOW_THREADS
+  PyObject* out = PyDict_New();
+  if (!out) return nullptr;
+  const struct { const char* name; const void* p; } cols[] = {
+      {"e_min", t.e_min}, {"arrival_skew", t.arrival_skew}, {"t_max", t.t_max}, {"t_min", t.t_min}, {"span", t.span}, {"med_skew", t.med_skew},
+      {"mad_skew", t.mad_skew}, {"med_dur", t.med_dur}, {"mad_dur", t.mad_dur}, {"rank_tmin", t.rank_tmin}, {"rank_tmax", t.rank_tmax},
+      {"max_chg", t.max_chg}, {"rank_max_chg", t.rank_max_chg}, {"n_present", t.n_present}, {"gflags", t.gflags}, {"busbw", t.busbw},
+      {"flags", t.flags}, {"perm", t.perm}};
+  bool ok = put(out, "n_groups", PyLong_FromUnsignedLongLong(t.n_groups)) && put(out, "n_slots", PyLong_FromUnsignedLongLong(t.n_slots));
+  for (const auto& c : cols) {
+    if (!ok) break;
+    if (!c.p) Py_INCREF(Py_None);
+    ok = put(out, c.name, c.p ? PyLong_FromVoidPtr(const_cast<void*>(c.p)) : Py_None);
+  }
+  if (!ok) { Py_DECREF(out); return nullptr; }
+  return Py_BuildValue("(iN)", rc, out);
+}
+
+PyObject* rank_list(const uint32_t* p, Py_ssize_t n) {                 // a copy
+  npy_intp dim = n;
+  PyObject* a = PyArray_SimpleNew(1, &dim, NPY_UINT32);
+  if (a && n) std::memcpy(PyArray_DATA((PyArrayObject*)a), p, (size_t)n * 4);
+  return a;
+}
+PyObject* hang_dict(const ccld_hang_verdict& v, const uint32_t* roots, Py_ssize_t cap) {
+  PyObject* out = PyDict_New();
+  const bool ok = out && put(out, "cls", PyLong_FromUnsignedLong(v.cls)) && put(out, "n_roots_total", PyLong_FromUnsignedLong(v.n_roots_total)) &&
+                  put(out, "n_not_entered", PyLong_FromUnsignedLong(v.n_not_entered)) && put(out, "n_hung", PyLong_FromUnsignedLong(v.n_hung)) &&
+                  put(out, "n_not_hung", PyLong_FromUnsignedLong(v.n_not_hung)) && put(out, "n_missing_frames", PyLong_FromUnsignedLong(v.n_missing_frames)) &&
+                  put(out, "stuck_step", PyLong_FromUnsignedLong(v.stuck_step)) && put(out, "n_members", PyLong_FromUnsignedLong(v.n_members)) &&
+                  put(out, "min_total", PyLong_FromUnsignedLongLong(v.min_total)) &&
+                  put(out, "roots", rank_list(roots, (Py_ssize_t)v.n_roots_total < cap ? (Py_ssize_t)v.n_roots_total : cap));
+  if (!ok) { Py_XDECREF(out); return nullptr; }
+  return out;
+}
+
+// Room the library writes lists into, per thread and kept between calls: only the entries there are get touched.
+template <class T> T* room(size_t n) {
+  static thread_local std::vector<T> v;
+  if (v.size() < n) v.resize(n);
+  return v.data();
+}
+
+// hang(context, window, communicator, op counter, roots_cap) -> (return code, dictionary)
+PyObject* hang(PyObject*, PyObject* args) {
+  unsigned long long h; unsigned int window, comm, seq; Py_ssize_t cap;
+  if (!PyArg_ParseTuple(args, "KIIIn", &h, &window, &comm, &seq, &cap)) return nullptr;
+  if (cap < 0) cap = 0;
+  uint32_t* roots = room<uint32_t>((size_t)cap + 1);
+  ccld_hang_verdict v;
+  std::memset(&v, 0, sizeof v);
+  v.roots = roots; v.roots_cap = (uint32_t)cap;
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = f_hang((ccld_ctx*)h, window, comm, seq, &v);
+  Py_END_ALLOW_THREADS
+  if (rc != CCLD_OK) return Py_BuildValue("(iO)", rc, Py_None);
+  PyObject* d = hang_dict(v, roots, cap);
+  return d ? Py_BuildValue("(iN)", rc, d) : nullptr;
+}
+
+// hangs(context, window, cap, roots_stride) -> (return code, list of dictionaries)
+PyObject* hangs(PyObject*, PyObject* args) {
+  unsigned long long h; unsigned int window; Py_ssize_t cap, stride;
+  if (!PyArg_ParseTuple(args, "KInn", &h, &window, &cap, &stride)) return nullptr;
+  if (cap < 1) cap = 1;
+  if (stride < 0) stride = 0;
+  ccld_hang_verdict* hv = room<ccld_hang_verdict>((size_t)cap);
+  ccld_hang_alert* al = room<ccld_hang_alert>((size_t)cap);
+  uint32_t* roots = room<uint32_t>((size_t)cap * (size_t)stride + 1);
+  if (cap > (Py_ssize_t)CCLD_MAX_ALERTS_PER_WINDOW) {                  // alerts beyond those kept are listed as zeros
+    std::memset(hv, 0, (size_t)cap * sizeof *hv); std::memset(al, 0, (size_t)cap * sizeof *al);
+  }
+  uint32_t n = 0;
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = f_hangs((ccld_ctx*)h, window, al, hv, (uint32_t)cap, roots, (uint32_t)stride, &n);
+  Py_END_ALLOW_THREADS
+  if (rc != CCLD_OK) return Py_BuildValue("(iO)", rc, Py_None);
+  const Py_ssize_t m = (Py_ssize_t)n < cap ? (Py_ssize_t)n : cap;
+  PyObject* list = PyList_New(m);
+  if (!list) return nullptr;
+  for (Py_ssize_t i = 0; i < m; ++i) {
+    PyObject* d = hang_dict(hv[i], roots + i * stride, stride);
+    if (!d || !put(d, "comm", PyLong_FromUnsignedLong(al[i].comm)) || !put(d, "seq", PyLong_FromUnsignedLong(al[i].seq)) ||
+        !put(d, "age_ns", PyLong_FromLongLong(al[i].age_ns))) { Py_XDECREF(d); Py_DECREF(list); return nullptr; }
+    PyList_SET_ITEM(list, i, d);
+  }
+  return Py_BuildValue("(iN)", rc, list);
+}
+
+// opset(context, window, communicator, op counter, ranks_cap) -> (return code, dictionary)
+PyObject* opset(PyObject*, PyObject* args) {
+  unsigned long long h; unsigned int window, comm, seq; Py_ssize_t cap;
+  if (!PyArg_ParseTuple(args, "KIIIn", &h, &window, &comm, &seq, &cap)) return nullptr;
+  if (cap < 0) cap = 0;
+  uint32_t* ranks = room<uint32_t>((size_t)cap + 1);
+  ccld_opset_verdict v;
+  std::memset(&v, 0, sizeof v);
+  v.ranks = ranks; v.ranks_cap = (uint32_t)cap;
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = f_opset((ccld_ctx*)h, window, comm, seq, &v);
+  Py_END_ALLOW_THREADS
+  if (rc != CCLD_OK) return Py_BuildValue("(iO)", rc, Py_None);
+  PyObject* out = PyDict_New();
+  const bool ok = out && put(out, "n_members", PyLong_FromUnsignedLong(v.n_members)) && put(out, "n_present", PyLong_FromUnsignedLong(v.n_present)) &&
+                  put(out, "n_deviating_total", PyLong_FromUnsignedLong(v.n_deviating_total)) && put(out, "majority_count", PyLong_FromUnsignedLong(v.majority_count)) &&
+                  put(out, "op", PyLong_FromLong(v.op)) && put(out, "algo", PyLong_FromLong(v.algo)) && put(out, "proto", PyLong_FromLong(v.proto)) &&
+                  put(out, "bytes", PyLong_FromUnsignedLongLong(v.bytes)) &&
+                  put(out, "ranks", rank_list(ranks, (Py_ssize_t)v.n_deviating_total < cap ? (Py_ssize_t)v.n_deviating_total : cap));
+  if (!ok) { Py_XDECREF(out); return nullptr; }
+  return Py_BuildValue("(iN)", rc, out);
+}
+
+// ranges(context, window, cap) -> (return code, dictionary of arrays)
+template <class T, class F> PyObject* column_of(const ccld_comm_range* rows, Py_ssize_t n, int type, F&& field) {
+  npy_intp dim = n;
+  PyObject* a = PyArray_SimpleNew(1, &dim, type);
+  if (a) { T* p = (T*)PyArray_DATA((PyArrayObject*)a); for (Py_ssize_t i = 0; i < n; ++i) p[i] = field(rows[i]); }
+  return a;
+}
+PyObject* ranges(PyObject*, PyObject* args) {
+  unsigned long long h; unsigned int window; Py_ssize_t cap;
+  if (!PyArg_ParseTuple(args, "KIn", &h, &window, &cap)) return nullptr;
+  if (cap < 0) cap = 0;
+  ccld_comm_range* rows = room<ccld_comm_range>((size_t)cap + 1);
+  uint32_t total = 0;
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = f_ranges((ccld_ctx*)h, window, rows, (uint32_t)cap, &total);
+  Py_END_ALLOW_THREADS
+  if (rc != CCLD_OK) return Py_BuildValue("(iO)", rc, Py_None);
+  const Py_ssize_t n = (Py_ssize_t)total < cap ? (Py_ssize_t)total : cap;
+  PyObject* out = PyDict_New();
+  typedef const ccld_comm_range& Row;
+  const bool ok = out && put(out, "comm", column_of<uint32_t>(rows, n, NPY_UINT32, [](Row r) { return r.comm; })) &&
+                  put(out, "n", column_of<uint32_t>(rows, n, NPY_UINT32, [](Row r) { return r.n; })) &&
+                  put(out, "seq_lo", column_of<uint32_t>(rows, n, NPY_UINT32, [](Row r) { return r.seq_lo; })) &&
+                  put(out, "n_seq", column_of<uint32_t>(rows, n, NPY_UINT32, [](Row r) { return r.n_seq; })) &&
+                  put(out, "group0", column_of<uint64_t>(rows, n, NPY_UINT64, [](Row r) { return r.group0; })) &&
+                  put(out, "slot0", column_of<uint64_t>(rows, n, NPY_UINT64, [](Row r) { return r.slot0; }));
+  if (!ok) { Py_XDECREF(out); return nullptr; }
+  return Py_BuildValue("(iN)", rc, out);
+}
+
+// rates(context, records, rank, t_enter, t_exit, ranks, ticks, tick_off, tick_ns, send_count, recv_count, send_chg, recv_chg):
+// device addresses -> return code
+PyObject* rates(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  unsigned long long a[13];
+  if (n != 13) { PyErr_SetString(PyExc_TypeError, "rates takes 13 whole numbers"); return nullptr; }
+  for (int i = 0; i < 13; ++i) {
+    a[i] = PyLong_AsUnsignedLongLongMask(args[i]);
+    if (a[i] == (unsigned long long)-1 && PyErr_Occurred()) return nullptr;
+  }
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = f_rates((ccld_ctx*)a[0], a[1], (const uint32_t*)a[2], (const int64_t*)a[3], (const int64_t*)a[4], (uint32_t)a[5], a[6], (const uint64_t*)a[7],
+               (const int64_t*)a[8], (const uint32_t*)a[9], (const uint32_t*)a[10], (uint32_t*)a[11], (uint32_t*)a[12]);
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(rc);
+}
+
 PyMethodDef methods[] = {{"setup", setup, METH_VARARGS, "Addresses of the library's functions, names of fields."},
                          {"verdict", verdict, METH_VARARGS, "ccld_get_verdict_columns as a dictionary of arrays."},
                          {"upload", upload, METH_VARARGS, "ccld_trace_upload of numpy columns."},
                          {"rank_stats", rank_stats, METH_VARARGS, "ccld_take_rank_stats as a dictionary of arrays."},
                          {"optable", optable, METH_VARARGS, "ccld_take_optable as a dictionary of arrays."},
+                         {"table", table, METH_VARARGS, "ccld_get_optable as a dictionary of device addresses."},
+                         {"hang", hang, METH_VARARGS, "ccld_locate_hang as a dictionary."},
+                         {"hangs", hangs, METH_VARARGS, "ccld_locate_hangs as a list of dictionaries."},
+                         {"opset", opset, METH_VARARGS, "ccld_opset_check as a dictionary."},
+                         {"ranges", ranges, METH_VARARGS, "ccld_get_ranges as a dictionary of arrays."},
+                         {"rates", (PyCFunction)(void (*)(void))rates, METH_FASTCALL, "ccld_derive_rates on device addresses."},
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
