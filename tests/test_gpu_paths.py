@@ -1,0 +1,264 @@
+"""The library's size-dependent paths at the sizes where they can go wrong, against the CPU oracle: whole numbers must be
+identical, fp64 quantities within 1e-9 relative (tests/parity.py)."""
+import ctypes as C
+
+import numpy as np
+import pytest
+import torch
+
+import oracle as orc
+import paper_2605_04478_b200 as ccld
+from helpers import MiB, frames_from, make_cols
+from parity import compare_cumulative, compare_hang, compare_window, make_pair, same
+
+pytestmark = pytest.mark.gpu
+
+
+def job(sizes, n_seq, rng, t0=1_000_000_000, spacing=20_000_000, dur=None, ent=None, order="rank"):
+    """A communicator per entry of `sizes` over ranks of its own, n_seq ops each: (registry, columns, ranks)."""
+    reg, parts, r0 = [], [], 0
+    for cid, n in enumerate(sizes):
+        d = rng.integers(1_000_000, 1_200_000, (n_seq, n)) if dur is None else dur(cid, n)
+        e = rng.integers(0, 40_000, (n_seq, n)) if ent is None else ent(cid, n)
+        reg.append((cid, list(range(r0, r0 + n)), 0))
+        s, r = np.meshgrid(np.arange(n_seq), np.arange(n), indexing="ij")
+        te = t0 + s * spacing + e
+        parts.append((r0 + r.T.ravel(), np.full(n * n_seq, cid), s.T.ravel(), te.T.ravel(), (te + d).T.ravel()))
+        r0 += n
+    rank, comm, seq, te, tx = (np.concatenate(x) for x in zip(*parts))
+    i = np.arange(len(rank)) if order == "rank" else rng.permutation(len(rank))
+    cols = dict(rank=rank[i].astype(np.uint32), comm=comm[i].astype(np.uint32), seq=seq[i].astype(np.uint32),
+                op=np.zeros(len(i), np.uint8), bytes=np.full(len(i), 16 * MiB, np.uint64), t_enter=te[i].astype(np.int64),
+                t_exit=tx[i].astype(np.int64), send_chg=rng.integers(0, 9, len(i)).astype(np.uint32),
+                recv_chg=rng.integers(0, 9, len(i)).astype(np.uint32))
+    return reg, cols, r0
+
+
+def run(reg, cols, n_ranks, params=None, now=10**13, an=None):
+    pair = make_pair(reg, params)
+    an, o = (an or pair[0]), pair[1]
+    an.trace_upload(0, cols)
+    assert o.upload(0, cols) == 0
+    an.analyze_window(0, 1, now)
+    assert o.analyze(0, 1, now) == 0
+    compare_window(an, o, 0)
+    compare_cumulative(an, o, n_ranks, 0)
+    return an, o
+
+
+# ---------------------------------------------------------------- reductions
+@pytest.mark.parametrize("n", [1025, 2048, 2049, 4096, 4097, 8192])
+@pytest.mark.parametrize("spread", ["equal", "ties", "wide"])
+def test_large_communicators(n, spread):
+    """The three instances of the cluster kernel at both ends of their ranges (an eighth of 1,025 or 2,049 members leaves
+    CTAs with uneven shares), with all keys equal, more ties than a bin's list holds, and durations over the whole 32 bits (so
+    that the median takes every level of the histogram); nine ops: a full tile and one of a single op."""
+    rng = np.random.default_rng(n)
+    dur = {"equal": lambda c, n: np.full((9, n), 5_000_000), "ties": lambda c, n: 1_000_000 + rng.integers(0, 3, (9, n)),
+           "wide": lambda c, n: rng.integers(1, (1 << 31) - 1, (9, n))}[spread]
+    ent = {"equal": lambda c, n: np.zeros((9, n), int), "ties": lambda c, n: rng.integers(0, 2, (9, n)) * 4096,
+           "wide": lambda c, n: rng.integers(0, 1 << 31, (9, n))}[spread]
+    run(*job([n], 9, rng, dur=dur, ent=ent, spacing=5_000_000_000))
+
+
+def test_three_sizes_side_by_side_on_a_stream():
+    """Small, middle and large communicators in one batch, on a stream of the caller's, analysed again and again: the three
+    reductions run on streams of their own and share the lists of set-aside groups and the cumulative sums."""
+    rng = np.random.default_rng(3)
+    reg, cols, n = job([4, 8, 64, 129, 513, 1024, 1500], 19, rng)
+    late = rng.random(len(cols["rank"])) < 0.0005
+    cols["t_exit"][late] = -1                                   # groups of every size in flight
+    st = torch.cuda.Stream()
+    an = ccld.Analyzer(stream=st)
+    for cid, ranks, seq0 in reg:
+        an.comm_register(cid, ranks, 0, seq0)
+    an, o = run(reg, cols, n, an=an)
+    for _ in range(20):
+        an.reset()
+        an.analyze_window(0, 1, 10**13)
+        compare_cumulative(an, o, n, 0)
+    compare_window(an, o, 0)
+
+
+@pytest.mark.parametrize("sizes", [(1, 3, 7, 8), (9, 32, 33, 64), (65, 127, 128)])
+def test_times_across_a_boundary_of_32_bits(sizes):
+    """Ops whose enter times, or whose enter and exit, lie on different sides of a multiple of 2^32 ns."""
+    rng = np.random.default_rng(sum(sizes))
+    run(*job(sizes, 70, rng, t0=(1 << 32) * 5 - 35 * 1_000_000, spacing=1_000_000))
+
+
+@pytest.mark.parametrize("n", [129, 256, 257, 512, 513, 1024])
+def test_middle_communicators_ragged_tiles(n):
+    rng = np.random.default_rng(n)
+    run(*job([n, n], 13, rng, dur=lambda c, n: 1_000_000 + rng.integers(0, 5 if c else 200_000, (13, n)), order="shuffled"))
+
+
+@pytest.mark.parametrize("n_comms", [4096, 4097, 8193])
+def test_many_communicators(n_comms):
+    """Registries at and beyond what the layout keeps in registers and a slice of the emit pass covers."""
+    rng = np.random.default_rng(n_comms)
+    run(*job([2] * (n_comms - 3) + [40, 200, 8], 3, rng))
+
+
+@pytest.mark.parametrize("n", [512, 513, 4096])
+def test_op_counts_of_wide_communicators(n):
+    """Members of communicators of up to 512 are counted by one warp, of more by four; several of both in a CTA's four."""
+    rng = np.random.default_rng(n)
+    run(*job([n, 5, n, n, 600, 4], 2, rng))
+
+
+# ---------------------------------------------------------------- verdicts
+@pytest.mark.parametrize("n_ranks,outliers", [(900, 1.0), (1024, 0.9), (1100, 0.2), (2100, 1.0), (5000, 0.1), (5000, 0.9)])
+def test_verdict_lists(n_ranks, outliers):
+    """Suspect lists of one and of several pieces, put together by the last CTA (up to 1,024 entries) and by the merge; the
+    columns and the structs of the two entry points say the same, and a capacity cuts the list off."""
+    rng = np.random.default_rng(n_ranks)
+    # in every group of five, members that are always late or always slow; with a vote share of nothing every outlier counts
+    m = n_ranks // 5
+    lag = (rng.random((m, 5)) < 0.25 * outliers) * 3_000_000
+
+    def ent(c, n):
+        return rng.integers(0, 1000, (12, n)) + lag[c]
+
+    def dur(c, n):
+        return 1_000_000 + rng.integers(0, 1000, (12, n)) + np.roll(lag[c], 1)
+    reg, cols, n = job([5] * m, 12, rng, ent=ent, dur=dur)
+    an, o = run(reg, cols, n, params=dict(vote_rep_milli=200))
+    v = an.get_verdict(0)
+    k = v["n_suspects_total"]
+    assert len(v["suspects"]["rank"]) == k and len(v["comm_rows"]["comm"]) == m and len(v["alerts"]["seq"]) == 0
+    s = ccld.Verdict()
+    sus, rows = (ccld.Suspect * max(k, 1))(), (ccld.CommVerdict * m)()
+    s.suspects, s.suspects_cap, s.comm_rows, s.comm_rows_cap = sus, k, rows, m
+    assert an.lib.ccld_get_verdict(an.h, 0, C.byref(s)) == 0 and s.n_suspects_total == k
+    for f, _ in ccld.Suspect._fields_:
+        same(v["suspects"][f], [getattr(x, f) for x in sus[:k]], f)
+    for f, _ in ccld.CommVerdict._fields_:
+        same(v["comm_rows"][f], [getattr(x, f) for x in rows], f)
+    few = an.get_verdict(0, comm_rows_cap=3, suspects_cap=k // 2)
+    assert len(few["comm_rows"]["comm"]) == 3 and few["n_comm_rows_total"] == m and few["n_suspects_total"] == k
+    same(few["suspects"]["rank"], v["suspects"]["rank"][:k // 2], "cut suspects")
+    if (n_ranks, outliers) == (5000, 0.9):
+        assert k > 1024
+
+
+def test_what_the_binding_hands_out_outlives_the_context():
+    """Tables and statistics lie in pinned blocks that go back when the last array is gone, also after the context; a column
+    that is not a plain array takes the general way in; windows that are not there are named in the error."""
+    rng = np.random.default_rng(8)
+    reg, cols, n = job([700, 8, 3], 150, rng)
+    an, o = run(reg, cols, n)
+    want = o.groups(0)["t_max"].copy()
+    kept = [an.get_optable(0) for _ in range(30)] + [an.get_rank_stats(n) for _ in range(30)]
+    with pytest.raises(ccld.CcldError):
+        an.get_verdict(7)
+    assert an.get_verdict(7, check=False)["rc"] != 0
+    an.trace_upload(1, {k: (torch.from_numpy(v) if k == "t_enter" else v[::1]) for k, v in cols.items()})
+    an.trace_upload(2, {k: np.repeat(v, 2)[::2] for k, v in cols.items()})       # not contiguous
+    an.analyze_window(1, 2, 10**13)
+    for w in (1, 2):
+        same(an.get_optable(w)["t_max"], want, "t_max of window %d" % w)
+    an.close()
+    for t in kept[:30]:
+        same(t["t_max"], want, "kept table")
+    assert int(kept[-1]["ops"].sum()) > 0 and kept[-1]["votes"].shape == (n, 4)
+    del t, kept
+
+
+# ---------------------------------------------------------------- uploads
+# bytes of an upload are 45 per record (37 without rates): one piece up to 256 KB, one 1 MB piece, then pieces of 1 MB by workers
+@pytest.mark.parametrize("n_rec", [1, 5825, 5826, 23301, 23302, 300_000])
+@pytest.mark.parametrize("pinned", [False, True])
+def test_uploads(n_rec, pinned):
+    rng = np.random.default_rng(n_rec)
+    n_seq = (n_rec + 7) // 8
+    reg, cols, n = job([8], n_seq, rng, spacing=2_000_000, order="shuffled")
+    cols = {k: v[:n_rec].copy() for k, v in cols.items()}
+    an, o = make_pair(reg)
+    signed = lambda v: v if v.itemsize == 1 else v.view("i%d" % v.itemsize)      # torch columns are signed, bit for bit the same
+    up = {k: torch.from_numpy(signed(v)).pin_memory() for k, v in cols.items()} if pinned else cols
+    for w in range(3):
+        an.trace_upload(w, up)
+        assert o.upload(w, cols) == 0
+    if not pinned:
+        for v in cols.values():
+            v[:] = 0                                            # pageable memory was copied by the time the call returned
+    an.analyze_window(0, 3, 10**13)
+    assert o.analyze(0, 3, 10**13) == 0
+    for w in range(3):
+        compare_window(an, o, w)
+
+
+# ---------------------------------------------------------------- diagnosis
+@pytest.mark.parametrize("n,kinds", [(200, 47), (200, 60), (3000, 200)])
+def test_opset_with_many_tuples(n, kinds):
+    """More different tuples than the pass over majority candidates takes before it counts them another way."""
+    rng = np.random.default_rng(kinds)
+    reg, cols, _ = job([n], 2, rng)
+    cols["bytes"][:] = (1 + rng.integers(0, kinds, len(cols["bytes"]))) * MiB
+    an, o = make_pair(reg)
+    an.trace_upload(0, cols); assert o.upload(0, cols) == 0
+    an.analyze_window(0, 1, 10**13); assert o.analyze(0, 1, 10**13) == 0
+    for s in (0, 1):
+        a, b = an.opset_check(0, 0, s), o.opset_check(0, 0, s)
+        for k in ("n_members", "n_present", "n_deviating_total", "majority_count", "op", "bytes"):
+            assert a[k] == b[k], (s, k, a[k], b[k])
+        same(a["ranks"], b["ranks"], "deviating ranks")
+
+
+@pytest.mark.parametrize("n", [2048, 2049, 5000])
+def test_hang_in_a_large_ring(n):
+    """Rings at and beyond what the decision keeps in shared memory: members that never entered (H1), some that completed
+    (H2), all hung with counters (H3), and ranks that went on to a later op."""
+    rng = np.random.default_rng(n)
+    reg, cols, _ = job([n], 5, rng)
+    seq, rank = cols["seq"].copy(), cols["rank"].copy()
+    keep = ~((seq == 4) & (rank % 7 != 0))                      # only some enter op 4
+    keep &= ~((seq == 3) & (rank == 11))                        # one never reports op 3
+    cols = {k: v[keep] for k, v in cols.items()}
+    seq, rank = cols["seq"], cols["rank"]
+    cols["t_exit"][(seq == 1)] = -1                             # all hung in op 1
+    cols["t_exit"][(seq == 2) & (rank % 3 != 0)] = -1           # some completed op 2
+    ch = 2
+    frames = frames_from([(r, 0, 1, [(40 + (r * 7) % 5, 40 + (r * 3) % 4)] * ch) for r in range(n) if r != 5], ch)
+    an, o = make_pair(reg)
+    an.trace_upload(0, cols, frames, ch); assert o.upload(0, cols, frames, ch) == 0
+    an.analyze_window(0, 1, 10**13); assert o.analyze(0, 1, 10**13) == 0
+    assert {compare_hang(an, o, 0, 0, s)["cls"] for s in range(5)} >= {1, 2}
+    for d in an.locate_hangs(0):
+        b = o.locate_hang(0, d["comm"], d["seq"])
+        assert d["cls"] == b["cls"] and d["n_roots_total"] == b["n_roots"]
+        same(d["roots"], b["roots"][:64], "sweep roots")
+
+
+# ---------------------------------------------------------------- rates
+@pytest.mark.parametrize("n_ranks,ticks,steps", [(1, 2048 * 257, "even"), (3, 200_000, "uneven"), (40, 2047, "even"), (300, 64, "gaps")])
+def test_rates_by_spacing(n_ranks, ticks, steps):
+    """A stream long enough for the scanned prefix (over 256 tiles, more than eight per rank), samples that are not evenly
+    spaced (the guess of a tick's place misses), ops that span many tiles and ops in flight; columns that start off a 16-byte
+    boundary."""
+    rng = np.random.default_rng(ticks)
+    MS = 1_000_000
+    off = np.arange(n_ranks + 1) * ticks
+    one = np.arange(ticks) * MS
+    if steps == "uneven":
+        one = np.cumsum(rng.integers(1, 4 * MS, ticks))
+    elif steps == "gaps":
+        one = one + (np.arange(ticks) > ticks // 2) * 500 * MS
+    tn = np.tile(one, n_ranks)
+    sc, rc = np.cumsum(rng.integers(0, 2, len(tn))), np.cumsum(rng.random(len(tn)) < 0.3)
+    n_rec = 4001
+    rank = np.sort(rng.integers(0, n_ranks, n_rec))
+    te = rng.integers(-5 * MS, int(one[-1]) + 5 * MS, n_rec)
+    tx = te + np.where(rng.random(n_rec) < 0.1, rng.integers(0, int(one[-1]) + 1, n_rec), rng.integers(0, 20 * MS, n_rec))
+    tx[::37] = -1
+    es, er = orc.derive_rates(rank, te, tx, off, tn, sc, rc)
+    for skip in (0, 1):
+        def put(a, dt):
+            t = torch.zeros(len(a) + skip, dtype=torch.from_numpy(np.zeros(0, dt)).dtype, device="cuda")
+            t[skip:] = torch.from_numpy(np.ascontiguousarray(a).astype(dt))
+            return t[skip:]
+        an = ccld.Analyzer()
+        s, r = an.derive_rates(put(rank, np.int32), put(te, np.int64), put(tx, np.int64), put(off, np.int64), put(tn, np.int64), put(sc, np.int32), put(rc, np.int32))
+        torch.cuda.synchronize()
+        same(s.cpu().numpy().view(np.uint32), es, "send"); same(r.cpu().numpy().view(np.uint32), er, "recv")
