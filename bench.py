@@ -43,8 +43,11 @@ CSRC = os.path.join(ROOT, "paper_2605_04478_b200", "csrc")
 # records, so a launch's traffic is this figure times its records. Each entry names the source files of its kernel and
 # their hash at capture time: once a file changes the figure is stale and the bench reports null.
 NCU_TRAFFIC = {
-    "k_reduce_fused": {"bytes_per_record": (814.439936e6 + 275.335424e6) / 20.48e6, "files": ("ccld_fused.cuh",),
-                       "sha16": "6183e6f855d461c0"},
+    "k_reduce_fused": {"bytes_per_record": (798.90e6 + 249.83e6) / 20.48e6, "files": ("ccld_fused.cuh",),
+                       "sha16": "a34c2c53944622eb"},
+    # capture on 5 cfg4w windows
+    "k_reduce_large": {"bytes_per_record": (770.75e6 + 83.83e6) / 20.48e6, "files": ("ccld_large.cuh",),
+                       "sha16": "c1faf52efbaca2f8"},
 }
 
 MIXES = {"all": ((0, 0, 1, 0, 2), 200), "tp_pp": ((0, 0, 1, 0), 250), "dp": ((2,), 200)}   # op pattern (0 TP, 1 PP, 2 DP), repetitions
