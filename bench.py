@@ -46,8 +46,8 @@ NCU_TRAFFIC = {
     "k_reduce_fused": {"bytes_per_record": (798.90e6 + 249.83e6) / 20.48e6, "files": ("ccld_fused.cuh",),
                        "sha16": "a34c2c53944622eb"},
     # capture on 5 cfg4w windows
-    "k_reduce_large": {"bytes_per_record": (770.75e6 + 83.83e6) / 20.48e6, "files": ("ccld_large.cuh",),
-                       "sha16": "c1faf52efbaca2f8"},
+    "k_reduce_large": {"bytes_per_record": (770.54e6 + 81.91e6) / 20.48e6, "files": ("ccld_large.cuh",),
+                       "sha16": "fcb4a1ab46234123"},
 }
 
 MIXES = {"all": ((0, 0, 1, 0, 2), 200), "tp_pp": ((0, 0, 1, 0), 250), "dp": ((2,), 200)}   # op pattern (0 TP, 1 PP, 2 DP), repetitions

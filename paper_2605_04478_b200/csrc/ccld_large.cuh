@@ -19,9 +19,9 @@
 // Groups that are not complete and 32-bit clean go to k_reduce_large_deferred (one CTA per listed group, 64-bit, hang alerts).
 //
 // Two kernels did this before: one wrote the keys to memory, the other read them twice and selected with 8-bit digits, every
-// key of a thread looked at in every pass (12 warp instructions per record): 2 x 1,000 groups of 4,096 took 90 + 195 us;
-// this kernel takes 241. A CTA lives 37 us, 14 of them in the gather (the CTAs of a wave gather at the same time, at the memory's
-// rate) and the rest in the barriers and round trips of the other steps.
+// key of a thread looked at in every pass (12 warp instructions per record): 2 x 1,000 groups of 4,096 took 90 + 195 us; this
+// kernel takes 231 (241 with the extremes kept as 64-bit keys while gathering). A CTA lives 35 us, 14 of them in the gather
+// and the rest in the barriers and round trips of the other steps.
 #pragma once
 #include <cooperative_groups.h>
 #include "ccld_device.cuh"
@@ -61,13 +61,23 @@ template <int Q> __device__ __forceinline__ void large_pick(const u32* __restric
     const bool act0 = first || (w0 > 0 && c0 > LQ_LIST), act1 = first || (w1 > 0 && c1 > LQ_LIST);
     if (!act0 && !act1) break;                             // the same in every thread
     const u32 n0 = w0 > LQ_BITS ? w0 - LQ_BITS : 0u, n1 = w1 > LQ_BITS ? w1 - LQ_BITS : 0u;
+    if (first) {                                           // every key counts, and none is larger than the bound
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
-      if (i >= n) break;
-      const u32 a = __usad(s_a[i], ma, 0u) - lo0, d = __usad(s_d[i], md, 0u) - lo1;
-      if (act0 && (first || (a >> w0) == 0)) atomicAdd(&sh.hist[0][(a >> n0) & (LQ_BINS - 1)], 1u);      // (w < 32 after the first level)
-      if (act1 && (first || (d >> w1) == 0)) atomicAdd(&sh.hist[1][(d >> n1) & (LQ_BINS - 1)], 1u);
+      for (int q = 0; q < Q; ++q) {
+        const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
+        if (i >= n) break;
+        atomicAdd(&sh.hist[0][__usad(s_a[i], ma, 0u) >> n0], 1u);
+        atomicAdd(&sh.hist[1][__usad(s_d[i], md, 0u) >> n1], 1u);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
+        if (i >= n) break;
+        const u32 a = __usad(s_a[i], ma, 0u) - lo0, d = __usad(s_d[i], md, 0u) - lo1;
+        if (act0 && (a >> w0) == 0) atomicAdd(&sh.hist[0][a >> n0], 1u);      // (w < 32 after the first level)
+        if (act1 && (d >> w1) == 0) atomicAdd(&sh.hist[1][d >> n1], 1u);
+      }
     }
     __syncthreads();
     u32 loc[8], sum = 0;
@@ -139,7 +149,7 @@ template <int Q> __device__ __forceinline__ void large_pick(const u32* __restric
 }
 
 template <int Q>
-__global__ void __launch_bounds__(LQ_THREADS, Q == 16 ? 2 : 3) k_reduce_large(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles,
+__global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles,
     TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
   begin_after();
   extern __shared__ __align__(16) u32 large_keys[];        // [metric][op counter][member of mine], later [metric][member]: my op counter
@@ -169,7 +179,7 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 16 ? 2 : 3) k_reduce_large(co
     const i64* __restrict__ c_te = D.t_enter; const i64* __restrict__ c_tx = D.t_exit;
     const u64* __restrict__ c_by = D.bytes; const u8* __restrict__ c_op = D.op;
     const u32* __restrict__ c_sc = D.send_chg; const u32* __restrict__ c_rc = D.recv_chg;
-    MidPart x; x.kmax = 0; x.n_kmin = 0; x.ck = 0; x.n_emin = 0; x.emax = 0; x.xmax = 0; x.bits = 0;
+    MidTrack x;
     u32 idx[Q];
     const u32 i0 = jv ? __ldg(perm) : NONE;
 #pragma unroll
@@ -198,16 +208,14 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 16 ? 2 : 3) k_reduce_large(co
           a = (u32)ra; const u32 b = (u32)rb; d = b - a;
           if (((ra | rb) >> 32) != 0 || (ta[u] | tb[u]) < 0 || b < a) x.bits |= 1;       // beyond 32 bits, negative or in flight, exit before enter
           if (op[u] != op0 || by[u] != by0) x.bits |= 2;
-          x.n_emin = max(x.n_emin, ~a); x.emax = max(x.emax, a); x.xmax = max(x.xmax, b);
-          const u64 k1 = ((u64)d << 32) | (u64)(NONE - p); x.kmax = k1 > x.kmax ? k1 : x.kmax;       // longest, then the lowest position
-          const u64 k2 = ~(((u64)d << 32) | (u64)p); x.n_kmin = k2 > x.n_kmin ? k2 : x.n_kmin;       // shortest, then the lowest position
-          const u64 k3 = ((u64)ch[u] << 32) | (u64)(NONE - p); x.ck = k3 > x.ck ? k3 : x.ck;         // most changes, then the lowest position
+          x.see(p, a, b, d, ch[u]);
         }
         k_a[j * PITCH + m] = a; k_d[j * PITCH + m] = d;
       }
     }
-    mid_merge(x, mid_shfl_xor(x, 8)); mid_merge(x, mid_shfl_xor(x, 16));
-    if (lane < LARGE_SEQS) sh.part[wid][lane] = x;
+    MidPart mine = x.part();
+    mid_merge(mine, mid_shfl_xor(mine, 8)); mid_merge(mine, mid_shfl_xor(mine, 16));
+    if (lane < LARGE_SEQS) sh.part[wid][lane] = mine;
     if (wid == 0 && lane < LARGE_SEQS) { sh.te0[lane] = te0; sh.gby[lane] = by0; sh.gop[lane] = op0; }
   }
   __syncthreads();
