@@ -98,33 +98,9 @@ __device__ __forceinline__ void best_warp_reduce(u64& rng, u32& k) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// record-streaming kernels (group-by parts 1 and 3). A CTA stages the key columns of REC_PER_CTA
-// consecutive records in shared memory with coalesced 128-bit loads; each thread then walks a run of
-// REC_RUN consecutive records. In rank-major or arrival-ordered uploads a run cycles through a handful
-// of (rank, communicator) pairs, which the thread keeps in registers, so the registry is consulted a
-// few times per run instead of once per record. Any order is handled: a full cache is flushed.
+// record-streaming kernels (group-by parts 1 and 3)
 // ------------------------------------------------------------------------------------------------
 constexpr int REC_RUN = REC_PER_CTA / REC_THREADS;       // consecutive records per thread
-constexpr int REC_PITCH = REC_RUN + 1;                   // shared-memory pitch of a run (conflict-free walks)
-constexpr int RC = 4;                                    // cached pairs per thread
-
-// Copies n_valid <= REC_PER_CTA elements of a u32 column, starting at record `first`, into s[(i / RUN) * PITCH + i % RUN].
-__device__ __forceinline__ void stage_column(const u32* __restrict__ col, u64 first, u32 n_valid, u32* s) {
-  if ((((uintptr_t)(col + first)) & 15) == 0) {
-    for (u32 q = threadIdx.x; q < REC_PER_CTA / 4; q += REC_THREADS) {
-      const u32 i = q * 4;
-      if (i + 4 <= n_valid) {
-        const uint4 v = *reinterpret_cast<const uint4*>(col + first + i);
-        u32* d = s + (i / REC_RUN) * REC_PITCH + (i % REC_RUN);      // REC_RUN is a multiple of 4: the four stay in one run
-        d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
-      } else {
-        for (u32 k = i; k < n_valid; ++k) s[(k / REC_RUN) * REC_PITCH + (k % REC_RUN)] = col[first + k];
-      }
-    }
-  } else {
-    for (u32 i = threadIdx.x; i < n_valid; i += REC_THREADS) s[(i / REC_RUN) * REC_PITCH + (i % REC_RUN)] = col[first + i];
-  }
-}
 
 __device__ __forceinline__ void range_widen(const WinDesc& D, u32 c, u32 mn, u32 mx) {
   if (mn < __ldcg(&D.rmin[c])) atomicMin(&D.rmin[c], mn);
