@@ -300,7 +300,7 @@ class Analyzer:
                 self._keep[window_id] = done[1]    # pinned host memory stays alive
                 return
         torch = self.torch
-        keep, ptrs, cuda, n = [], [], set(), 0
+        keep, ptrs, cuda, n = [], [], set(), None
         for k, dt, size in _COLS:
             v = cols.get(k)
             if v is None:
@@ -325,6 +325,8 @@ class Analyzer:
                 fr[k] = _as_tensor(torch, frames[k], "int32").contiguous()
                 cuda.add(fr[k].is_cuda)
         assert len(cuda) == 1, "all columns must live on the same device"
+        if n is None:
+            raise ValueError("a trace needs its rank column: the number of ranks is the number of records")
         mem_kind = 1 if True in cuda else 0
         ptr = lambda v: v.data_ptr() if v is not None and v.numel() else None
         nf = int(fr["f_rank"].numel()) if fr else 0

@@ -154,7 +154,7 @@ PyObject* verdict(PyObject*, PyObject* args) {
 }
 
 // upload(context, window, columns) -> (return code, arrays to keep), or None where a column is not a plain numpy array of the
-// column's size: the general way is Python's then
+// column's size, or the ranks, whose number is the window's, are not there: the general way is Python's then
 PyObject* upload(PyObject*, PyObject* args) {
   unsigned long long h; unsigned int window; PyObject* cols;
   if (!PyArg_ParseTuple(args, "KIO!", &h, &window, &PyDict_Type, &cols)) return nullptr;
@@ -164,14 +164,13 @@ PyObject* upload(PyObject*, PyObject* args) {
     PyObject* a = PyDict_GetItemWithError(cols, n_upload[i]);
     if (!a && PyErr_Occurred()) return nullptr;
     p[i] = nullptr;
-    if (!a || a == Py_None) continue;
+    if (!a || a == Py_None) { if (i == 0) Py_RETURN_NONE; continue; }
     if (!PyArray_CheckExact(a) || PyArray_ITEMSIZE((PyArrayObject*)a) != UPLOAD_SIZE[i] || !PyArray_IS_C_CONTIGUOUS((PyArrayObject*)a)) Py_RETURN_NONE;
     const unsigned long long m = (unsigned long long)PyArray_SIZE((PyArrayObject*)a);
     if (m) p[i] = PyArray_DATA((PyArrayObject*)a);
     if (i == 0) n = m;
     keep[n_keep++] = a;
   }
-  if (!n_keep) Py_RETURN_NONE;
   PyObject* held = PyTuple_New(n_keep);
   if (!held) return nullptr;
   for (Py_ssize_t i = 0; i < n_keep; ++i) { Py_INCREF(keep[i]); PyTuple_SET_ITEM(held, i, keep[i]); }

@@ -1,0 +1,48 @@
+"""What the Python binding accepts, refuses and hands on before a kernel runs (no GPU needed: the calls that go through
+reach the library with a null context, which it refuses as a bad argument)."""
+import ctypes as C
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2605_04478_b200 as ccld
+from helpers import make_cols
+from paper_2605_04478_b200.build import build
+
+
+@pytest.fixture(scope="module")
+def an():
+    """An analyzer without a context."""
+    build()
+    a = ccld.Analyzer.__new__(ccld.Analyzer)
+    a.lib, a.torch, a.h, a._keep, a._n_comms = ccld.load_library(), torch, C.c_void_p(), {}, 0
+    return a
+
+
+def columns(n=4):
+    return make_cols(dict(rank=i, seq=0, t_enter=1000 + i, t_exit=2000 + i) for i in range(n))
+
+
+def refused_by_the_library(call):
+    with pytest.raises(ccld.CcldError) as e:
+        call()
+    assert e.value.code == -1
+
+
+@pytest.mark.parametrize("missing", ["absent", "none", "misspelt"])
+@pytest.mark.parametrize("general", [False, True])
+def test_upload_without_ranks_is_refused(an, missing, general):
+    """Both ways in: plain numpy columns, and the general way (a column that is a tensor)."""
+    cols = columns()
+    if general:
+        cols["t_enter"] = torch.from_numpy(cols["t_enter"])
+    refused_by_the_library(lambda: an.trace_upload(0, cols))
+    rank = cols.pop("rank")
+    if missing == "none":
+        cols["rank"] = None
+    elif missing == "misspelt":
+        cols["ranks"] = rank
+    with pytest.raises(ValueError):
+        an.trace_upload(0, cols)
+    assert not an._keep
