@@ -306,7 +306,7 @@ class Analyzer:
             if v is None:
                 ptrs.append(None)
                 continue
-            if type(v) is np.ndarray and v.itemsize == size and v.flags.c_contiguous:      # the column's bits as they are
+            if type(v) is np.ndarray and v.itemsize == size and v.flags.c_contiguous and not v.dtype.hasobject:      # the column's bits as they are
                 cuda.add(False)
                 m = v.size
                 ptrs.append(_address(v) if m else None)

@@ -165,7 +165,8 @@ PyObject* upload(PyObject*, PyObject* args) {
     if (!a && PyErr_Occurred()) return nullptr;
     p[i] = nullptr;
     if (!a || a == Py_None) { if (i == 0) Py_RETURN_NONE; continue; }
-    if (!PyArray_CheckExact(a) || PyArray_ITEMSIZE((PyArrayObject*)a) != UPLOAD_SIZE[i] || !PyArray_IS_C_CONTIGUOUS((PyArrayObject*)a)) Py_RETURN_NONE;
+    if (!PyArray_CheckExact(a) || PyArray_ITEMSIZE((PyArrayObject*)a) != UPLOAD_SIZE[i] || !PyArray_IS_C_CONTIGUOUS((PyArrayObject*)a) ||
+        PyDataType_REFCHK(PyArray_DESCR((PyArrayObject*)a))) Py_RETURN_NONE;      // (references to objects have eight bytes too)
     const unsigned long long m = (unsigned long long)PyArray_SIZE((PyArrayObject*)a);
     if (m) p[i] = PyArray_DATA((PyArrayObject*)a);
     if (i == 0) n = m;

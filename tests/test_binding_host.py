@@ -46,3 +46,23 @@ def test_upload_without_ranks_is_refused(an, missing, general):
     with pytest.raises(ValueError):
         an.trace_upload(0, cols)
     assert not an._keep
+
+
+@pytest.mark.parametrize("general", [False, True])
+@pytest.mark.parametrize("name", ["bytes", "t_enter", "t_exit"])
+def test_upload_of_object_columns_is_refused(an, name, general):
+    """An array of Python objects has entries of eight bytes too: their addresses are no column."""
+    cols = columns()
+    cols[name] = np.array([int(v) for v in cols[name]], dtype=object)
+    if general:
+        cols["rank"] = torch.from_numpy(cols["rank"].view(np.int32))
+    with pytest.raises(TypeError):
+        an.trace_upload(0, cols)
+
+
+@pytest.mark.parametrize("name,view", [("rank", "i4"), ("comm", "f4"), ("seq", ">u4"), ("bytes", "f8"), ("t_enter", "M8[ns]"), ("t_exit", "u8"), ("op", "?")])
+def test_upload_takes_columns_by_their_bits(an, name, view):
+    """Plain arrays of another type of the column's size go through as they are."""
+    cols = columns()
+    cols[name] = cols[name].view(view)
+    refused_by_the_library(lambda: an.trace_upload(0, cols))
