@@ -8,7 +8,9 @@
 #include <Python.h>
 #define NPY_NO_DEPRECATED_API NPY_1_7_API_VERSION
 #include <numpy/arrayobject.h>
+#include <cstdlib>
 #include <cstring>
+#include <new>
 #include <vector>
 #include "../../include/ccld.h"
 
@@ -82,7 +84,8 @@ void release_block(PyObject* capsule) {
   if (b) { f_release(b); delete b; }
 }
 PyObject* own_block(const ccld_host_block& block) {
-  ccld_host_block* b = new ccld_host_block(block);
+  ccld_host_block* b = new (std::nothrow) ccld_host_block(block);
+  if (!b) { ccld_host_block gone = block; f_release(&gone); return PyErr_NoMemory(); }
   PyObject* c = PyCapsule_New(b, "ccld_host_block", release_block);
   if (!c) { f_release(b); delete b; }
   return c;
@@ -286,28 +289,32 @@ PyObject* hang_dict(const ccld_hang_verdict& v, const uint32_t* roots, Py_ssize_
   return out;
 }
 
-// Room the library writes lists into, per thread and kept between calls: only the entries there are get touched.
-template <class T> T* room(size_t n) {
-  static thread_local std::vector<T> v;
-  if (v.size() < n) v.resize(n);
-  return v.data();
-}
+// Room the library writes a list of up to n entries into, for one call. The lists have a largest length (members of a
+// communicator, alerts of a window), so a caller's capacity beyond that needs no room.
+template <class T> struct Room {
+  T* const p;
+  explicit Room(size_t n) : p((T*)std::malloc(n ? n * sizeof(T) : 1)) {}
+  ~Room() { std::free(p); }
+  Room(const Room&) = delete; Room& operator=(const Room&) = delete;
+};
+Py_ssize_t at_most(Py_ssize_t cap, Py_ssize_t most) { return cap < 0 ? 0 : (cap < most ? cap : most); }
 
 // hang(context, window, communicator, op counter, roots_cap) -> (return code, dictionary)
 PyObject* hang(PyObject*, PyObject* args) {
   unsigned long long h; unsigned int window, comm, seq; Py_ssize_t cap;
   if (!PyArg_ParseTuple(args, "KIIIn", &h, &window, &comm, &seq, &cap)) return nullptr;
-  if (cap < 0) cap = 0;
-  uint32_t* roots = room<uint32_t>((size_t)cap + 1);
+  cap = at_most(cap, CCLD_MAX_COMM_SIZE);
+  const Room<uint32_t> roots((size_t)cap);
+  if (!roots.p) return PyErr_NoMemory();
   ccld_hang_verdict v;
   std::memset(&v, 0, sizeof v);
-  v.roots = roots; v.roots_cap = (uint32_t)cap;
+  v.roots = roots.p; v.roots_cap = (uint32_t)cap;
   int rc;
   Py_BEGIN_ALLOW_THREADS
   rc = f_hang((ccld_ctx*)h, window, comm, seq, &v);
   Py_END_ALLOW_THREADS
   if (rc != CCLD_OK) return Py_BuildValue("(iO)", rc, Py_None);
-  PyObject* d = hang_dict(v, roots, cap);
+  PyObject* d = hang_dict(v, roots.p, cap);
   return d ? Py_BuildValue("(iN)", rc, d) : nullptr;
 }
 
@@ -316,26 +323,28 @@ PyObject* hangs(PyObject*, PyObject* args) {
   unsigned long long h; unsigned int window; Py_ssize_t cap, stride;
   if (!PyArg_ParseTuple(args, "KInn", &h, &window, &cap, &stride)) return nullptr;
   if (cap < 1) cap = 1;
-  if (stride < 0) stride = 0;
-  ccld_hang_verdict* hv = room<ccld_hang_verdict>((size_t)cap);
-  ccld_hang_alert* al = room<ccld_hang_alert>((size_t)cap);
-  uint32_t* roots = room<uint32_t>((size_t)cap * (size_t)stride + 1);
-  if (cap > (Py_ssize_t)CCLD_MAX_ALERTS_PER_WINDOW) {                  // alerts beyond those kept are listed as zeros
-    std::memset(hv, 0, (size_t)cap * sizeof *hv); std::memset(al, 0, (size_t)cap * sizeof *al);
-  }
+  const Py_ssize_t keep = at_most(cap, CCLD_MAX_ALERTS_PER_WINDOW);
+  stride = at_most(stride, CCLD_MAX_COMM_SIZE);
+  const Room<ccld_hang_verdict> hv((size_t)keep);
+  const Room<ccld_hang_alert> al((size_t)keep);
+  const Room<uint32_t> roots((size_t)keep * (size_t)stride);
+  if (!hv.p || !al.p || !roots.p) return PyErr_NoMemory();
   uint32_t n = 0;
   int rc;
   Py_BEGIN_ALLOW_THREADS
-  rc = f_hangs((ccld_ctx*)h, window, al, hv, (uint32_t)cap, roots, (uint32_t)stride, &n);
+  rc = f_hangs((ccld_ctx*)h, window, al.p, hv.p, (uint32_t)keep, roots.p, (uint32_t)stride, &n);
   Py_END_ALLOW_THREADS
   if (rc != CCLD_OK) return Py_BuildValue("(iO)", rc, Py_None);
   const Py_ssize_t m = (Py_ssize_t)n < cap ? (Py_ssize_t)n : cap;
   PyObject* list = PyList_New(m);
   if (!list) return nullptr;
   for (Py_ssize_t i = 0; i < m; ++i) {
-    PyObject* d = hang_dict(hv[i], roots + i * stride, stride);
-    if (!d || !put(d, "comm", PyLong_FromUnsignedLong(al[i].comm)) || !put(d, "seq", PyLong_FromUnsignedLong(al[i].seq)) ||
-        !put(d, "age_ns", PyLong_FromLongLong(al[i].age_ns))) { Py_XDECREF(d); Py_DECREF(list); return nullptr; }
+    ccld_hang_verdict v; ccld_hang_alert a;                            // alerts beyond those kept are listed as zeros
+    std::memset(&v, 0, sizeof v); std::memset(&a, 0, sizeof a);
+    if (i < keep) { v = hv.p[i]; a = al.p[i]; }
+    PyObject* d = hang_dict(v, roots.p + (i < keep ? i * stride : 0), stride);
+    if (!d || !put(d, "comm", PyLong_FromUnsignedLong(a.comm)) || !put(d, "seq", PyLong_FromUnsignedLong(a.seq)) ||
+        !put(d, "age_ns", PyLong_FromLongLong(a.age_ns))) { Py_XDECREF(d); Py_DECREF(list); return nullptr; }
     PyList_SET_ITEM(list, i, d);
   }
   return Py_BuildValue("(iN)", rc, list);
@@ -345,11 +354,12 @@ PyObject* hangs(PyObject*, PyObject* args) {
 PyObject* opset(PyObject*, PyObject* args) {
   unsigned long long h; unsigned int window, comm, seq; Py_ssize_t cap;
   if (!PyArg_ParseTuple(args, "KIIIn", &h, &window, &comm, &seq, &cap)) return nullptr;
-  if (cap < 0) cap = 0;
-  uint32_t* ranks = room<uint32_t>((size_t)cap + 1);
+  cap = at_most(cap, CCLD_MAX_COMM_SIZE);
+  const Room<uint32_t> ranks((size_t)cap);
+  if (!ranks.p) return PyErr_NoMemory();
   ccld_opset_verdict v;
   std::memset(&v, 0, sizeof v);
-  v.ranks = ranks; v.ranks_cap = (uint32_t)cap;
+  v.ranks = ranks.p; v.ranks_cap = (uint32_t)cap;
   int rc;
   Py_BEGIN_ALLOW_THREADS
   rc = f_opset((ccld_ctx*)h, window, comm, seq, &v);
@@ -360,7 +370,7 @@ PyObject* opset(PyObject*, PyObject* args) {
                   put(out, "n_deviating_total", PyLong_FromUnsignedLong(v.n_deviating_total)) && put(out, "majority_count", PyLong_FromUnsignedLong(v.majority_count)) &&
                   put(out, "op", PyLong_FromLong(v.op)) && put(out, "algo", PyLong_FromLong(v.algo)) && put(out, "proto", PyLong_FromLong(v.proto)) &&
                   put(out, "bytes", PyLong_FromUnsignedLongLong(v.bytes)) &&
-                  put(out, "ranks", rank_list(ranks, (Py_ssize_t)v.n_deviating_total < cap ? (Py_ssize_t)v.n_deviating_total : cap));
+                  put(out, "ranks", rank_list(ranks.p, (Py_ssize_t)v.n_deviating_total < cap ? (Py_ssize_t)v.n_deviating_total : cap));
   if (!ok) { Py_XDECREF(out); return nullptr; }
   return Py_BuildValue("(iN)", rc, out);
 }
@@ -375,8 +385,10 @@ template <class T, class F> PyObject* column_of(const ccld_comm_range* rows, Py_
 PyObject* ranges(PyObject*, PyObject* args) {
   unsigned long long h; unsigned int window; Py_ssize_t cap;
   if (!PyArg_ParseTuple(args, "KIn", &h, &window, &cap)) return nullptr;
-  if (cap < 0) cap = 0;
-  ccld_comm_range* rows = room<ccld_comm_range>((size_t)cap + 1);
+  cap = at_most(cap, (Py_ssize_t)0xFFFFFFFFu);
+  const Room<ccld_comm_range> room((size_t)cap);
+  if (!room.p) return PyErr_NoMemory();
+  ccld_comm_range* const rows = room.p;
   uint32_t total = 0;
   int rc;
   Py_BEGIN_ALLOW_THREADS

@@ -66,3 +66,13 @@ def test_upload_takes_columns_by_their_bits(an, name, view):
     cols = columns()
     cols[name] = cols[name].view(view)
     refused_by_the_library(lambda: an.trace_upload(0, cols))
+
+
+def test_capacities_beyond_any_list(an):
+    """Room is taken for what the library can list, not for what the caller could hold: no capacity takes the process down."""
+    for cap in (0, -5, 1 << 33, 1 << 62, (1 << 63) - 1):
+        refused_by_the_library(lambda: an.locate_hang(0, 0, 0, roots_cap=cap))
+        refused_by_the_library(lambda: an.opset_check(0, 0, 0, ranks_cap=cap))
+        refused_by_the_library(lambda: an.locate_hangs(0, cap=cap))
+        refused_by_the_library(lambda: an.locate_hangs(0, roots_stride=cap))
+        refused_by_the_library(lambda: an.locate_hangs(0, cap=cap, roots_stride=cap))
