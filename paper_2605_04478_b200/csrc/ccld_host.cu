@@ -139,7 +139,7 @@ constexpr size_t SHAPE_CACHE = 4;
 struct UploadSlot { char* p = nullptr; cudaEvent_t done = nullptr; bool used = false; };
 constexpr size_t UP_PIECE = 1u << 20;                      // a large upload goes piece by piece
 constexpr u32 UP_WORKERS = 6, UP_SLOTS = 2 * UP_WORKERS;   // two pieces per worker: one being filled, one on its way
-constexpr size_t UP_SMALL = 256u << 10;                    // up to this size one piece takes the whole upload, pinned columns too
+constexpr size_t UP_SMALL = 256u << 10;                    // up to this size one kernel reads the pinned columns, beyond it they are copied one by one
 
 constexpr u32 TIMER_RING = 32;
 constexpr int TIMER_PAIRS = CCLD_K_KINDS + 1;          // the layout kernel runs twice per call
@@ -499,6 +499,8 @@ int take_block(ccld_ctx* ctx, size_t bytes, ccld_host_block* blk) {
 
 // Host columns on their way into one device block.
 struct UpCol { size_t off; const void* src; size_t n; };
+constexpr u32 UP_COLS = 13;                                // columns of a trace and of its frames
+static_assert(UP_COLS <= GATHER_PIECES, "a piece per column");
 int upload_slots(ccld_ctx* ctx) {
   if (ctx->h_up.p) return CCLD_OK;
   for (UploadSlot& u : ctx->up) if (!u.done) CK(cudaEventCreateWithFlags(&u.done, cudaEventDisableTiming));
@@ -507,30 +509,14 @@ int upload_slots(ccld_ctx* ctx) {
   for (u32 i = 0; i < UP_SLOTS; ++i) { ctx->up[i].p = (char*)ctx->h_up.p + i * UP_PIECE; ctx->up[i].used = false; }
   return CCLD_OK;
 }
-// Copies the columns to `base` (device, `total` bytes with the columns at their offsets). The driver copies pageable memory
-// column by column through its own buffers, one thread, 10 us and more per call. A small upload is put together in one
-// pinned piece instead and crosses in one copy; a large pageable one is cut into pieces that several threads fill while
-// earlier ones cross. Large pinned columns go straight across.
-int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u32 n_cols) {
+// The pageable columns of an upload. (Where they share a piece with others, those are copied behind it.)
+int upload_pageable(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u32 n_cols) {
   cudaStream_t st = ctx->stream;
-  size_t bytes = 0; const void* first = nullptr;
-  for (u32 i = 0; i < n_cols; ++i) { bytes += col[i].n; if (col[i].n && !first) first = col[i].src; }
-  if (bytes == 0) return CCLD_OK;
-  bool pinned = false;
-  if (total > UP_SMALL) {
-    cudaPointerAttributes at;
-    pinned = cudaPointerGetAttributes(&at, first) == cudaSuccess && at.type != cudaMemoryTypeUnregistered;
-    cudaGetLastError();
-  }
-  if (pinned) {
-    for (u32 i = 0; i < n_cols; ++i) if (col[i].n) CK(cudaMemcpyAsync(base + col[i].off, col[i].src, col[i].n, cudaMemcpyHostToDevice, st));
-    return CCLD_OK;
-  }
   { int rc = upload_slots(ctx); if (rc != CCLD_OK) return rc; }
   if (total <= UP_PIECE) {
     UploadSlot& u = ctx->up[ctx->up_next++ % UP_SLOTS];
     if (u.used) CK(cudaEventSynchronize(u.done));
-    for (u32 i = 0; i < n_cols; ++i) if (col[i].n) std::memcpy(u.p + col[i].off, col[i].src, col[i].n);
+    for (u32 i = 0; i < n_cols; ++i) std::memcpy(u.p + col[i].off, col[i].src, col[i].n);
     CK(cudaMemcpyAsync(base, u.p, total, cudaMemcpyHostToDevice, st));
     CK(cudaEventRecord(u.done, st));
     u.used = true;
@@ -562,6 +548,36 @@ int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u3
   work(0);
   for (auto& t : crew) t.join();
   CK((cudaError_t)err.load());
+  return CCLD_OK;
+}
+
+// Copies the columns to `base` (device, `total` bytes with the columns at their offsets). The driver copies pageable memory
+// column by column through its own buffers, one thread, 10 us and more per call. A small upload is put together in one
+// pinned piece instead and crosses in one copy; a large one is cut into pieces that several threads fill while earlier ones
+// cross. Pageable columns are read by the time the call returns. Any other column is read when its turn in the stream comes, so
+// that what earlier work of the stream still writes there is what arrives: large ones go straight across, small ones are
+// read by one kernel.
+int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* cols, u32 n_cols) {
+  cudaStream_t st = ctx->stream;
+  UpCol col[UP_COLS]; u32 n_page = 0;                      // the pageable columns
+  UpCol far[UP_COLS]; u32 n_far = 0;                       // those that are copied one by one
+  GatherArgs G; u32 n_near = 0; size_t most = 0;           // those that a kernel reads
+  for (u32 i = 0; i < n_cols; ++i) {
+    if (!cols[i].n) continue;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, cols[i].src) != cudaSuccess) { cudaGetLastError(); at.type = cudaMemoryTypeUnregistered; }
+    if (at.type == cudaMemoryTypeUnregistered) col[n_page++] = cols[i];
+    else if (total <= UP_SMALL && at.type == cudaMemoryTypeHost && at.devicePointer && ((uintptr_t)at.devicePointer & 15) == 0) {
+      auto& g = G.piece[n_near++];
+      g.src = (const unsigned char*)at.devicePointer; g.dst = (unsigned char*)base + cols[i].off; g.n = cols[i].n; most = std::max(most, cols[i].n);
+    } else far[n_far++] = cols[i];
+  }
+  if (n_page) { int rc = upload_pageable(ctx, base, total, col, n_page); if (rc != CCLD_OK) return rc; }
+  for (u32 i = 0; i < n_far; ++i) CK(cudaMemcpyAsync(base + far[i].off, far[i].src, far[i].n, cudaMemcpyHostToDevice, st));
+  if (n_near) {
+    launch(On(st, false), k_gather, dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), n_near), GATHER_THREADS, 0, G);
+    CK(cudaGetLastError());
+  }
   return CCLD_OK;
 }
 
@@ -740,6 +756,7 @@ int ccld_trace_upload(ccld_ctx* ctx, uint32_t window_id, uint64_t n_rec, int mem
     const UpCol col[] = {{o_rank, rank, n_rec * 4}, {o_comm, comm, n_rec * 4}, {o_seq, seq, n_rec * 4}, {o_op, op, n_rec}, {o_bytes, bytes, n_rec * 8},
                          {o_te, t_enter_ns, n_rec * 8}, {o_tx, t_exit_ns, n_rec * 8}, {o_sc, send_chg, chg}, {o_rc, recv_chg, chg},
                          {o_fr, f_rank, fr}, {o_fc, f_comm, fr}, {o_fs, f_seq, fr}, {o_pr, progress, (size_t)n_frames * n_channels * 8}};
+    static_assert(sizeof col / sizeof col[0] == UP_COLS, "all of them");
     { int rc = upload_columns(ctx, b, off, col, sizeof col / sizeof col[0]); if (rc != CCLD_OK) { cudaStreamSynchronize(ctx->stream); ctx->pool.put(w.own); return rc; } }
     d.rank = (const u32*)(b + o_rank); d.comm = (const u32*)(b + o_comm); d.seq = (const u32*)(b + o_seq); d.op = (const u8*)(b + o_op);
     d.bytes = (const u64*)(b + o_bytes); d.t_enter = (const i64*)(b + o_te); d.t_exit = (const i64*)(b + o_tx);

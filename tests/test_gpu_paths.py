@@ -262,3 +262,32 @@ def test_rates_by_spacing(n_ranks, ticks, steps):
         s, r = an.derive_rates(put(rank, np.int32), put(te, np.int64), put(tx, np.int64), put(off, np.int64), put(tn, np.int64), put(sc, np.int32), put(rc, np.int32))
         torch.cuda.synchronize()
         same(s.cpu().numpy().view(np.uint32), es, "send"); same(r.cpu().numpy().view(np.uint32), er, "recv")
+
+
+# bytes of the columns: within what one kernel reads, one piece, several pieces
+@pytest.mark.parametrize("n_rec", [5000, 20_000, 60_000])
+@pytest.mark.parametrize("pageable", [(), ("rank",), ("comm", "seq", "op", "send_chg")])
+def test_upload_of_columns_the_stream_still_writes(n_rec, pageable):
+    """Pinned columns that a copy of the stream fills when the upload is called: their contents are those of their turn in the
+    stream. Some columns may be pageable; those are read by the call itself."""
+    rng = np.random.default_rng(n_rec)
+    reg, cols, _ = job([8], n_rec // 8, rng, spacing=2_000_000, order="shuffled")
+    an, o = make_pair(reg)
+    assert o.upload(0, cols) == 0
+    dev, up = {}, {}
+    for i, (k, v) in enumerate(cols.items()):
+        t = torch.from_numpy(v if v.itemsize == 1 else v.view("i%d" % v.itemsize))
+        dev[k] = t.cuda()
+        # an odd column lies off a 16-byte boundary
+        up[k] = v.copy() if k in pageable else torch.zeros(len(v) + 3, dtype=t.dtype).pin_memory()[3 * (i % 2):][:len(v)]
+    torch.cuda.synchronize()
+    torch.cuda._sleep(20_000_000)                               # some ten milliseconds of the stream
+    for k in up:
+        if k not in pageable:
+            up[k].copy_(dev[k], non_blocking=True)
+    an.trace_upload(0, up)
+    for k in pageable:
+        up[k][:] = 0
+    an.analyze_window(0, 1, 10**13)
+    assert o.analyze(0, 1, 10**13) == 0
+    compare_window(an, o, 0)
