@@ -598,10 +598,14 @@ int settle(ccld_ctx* ctx) {
     for (u32 k = 0; k < b.n && !failed; ++k) if (b.h_tot()[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) failed = true;
     ctx->pinned_free.push_back(b.pin);
     if (!failed) {
-      // a window may still have been refused for its size, which the expectation cannot have foreseen: keep what the plan found
+      // a window may still have been refused for its size, which the expectation cannot have foreseen: keep what the plan found,
+      // which is then no groups and no slots
       for (u32 k = 0; k < b.n; ++k) {
         auto it = ctx->windows.find(b.first + k);
-        if (it != ctx->windows.end() && it->second.analysed) std::memcpy(it->second.totals, b.h_tot() + (size_t)k * T_COUNT, sizeof it->second.totals);
+        if (it == ctx->windows.end() || !it->second.analysed) continue;
+        WindowHost& w = it->second;
+        std::memcpy(w.totals, b.h_tot() + (size_t)k * T_COUNT, sizeof w.totals);
+        w.d.n_groups = w.totals[T_GROUPS]; w.d.n_slots = w.totals[T_SLOTS];
       }
       continue;
     }
@@ -1087,6 +1091,7 @@ static int verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out, ccld_ve
     if (ctx->batches_redone == redone) break;
     if (attempt > 2) return fail(ctx, CCLD_ERR_CUDA, "internal: a settled batch changed again");
   }
+  n_rows = std::min<u32>(n_rows, (u32)w->totals[T_ROWS]);      // (fewer than were gathered only where the window was refused: none)
   const u64* cnt = head->counters;
   out->n_records = w->n_rec; out->n_groups = w->totals[T_GROUPS]; out->n_slots = w->totals[T_SLOTS];
   out->n_rejected = w->n_rec - cnt[C_PRESENT]; out->n_complete = cnt[C_COMPLETE]; out->n_incomplete = cnt[C_INCOMPLETE];

@@ -291,3 +291,28 @@ def test_upload_of_columns_the_stream_still_writes(n_rec, pageable):
     an.analyze_window(0, 1, 10**13)
     assert o.analyze(0, 1, 10**13) == 0
     compare_window(an, o, 0)
+
+
+@pytest.mark.parametrize("to_host", [True, False])
+def test_a_window_refused_for_its_size_after_one_of_its_shape(to_host):
+    """An op counter far beyond the others makes the window need too many slots. Where an earlier window of as many records made
+    the library size the results without waiting, the refused window lists nothing either, and the next one is analysed."""
+    rng = np.random.default_rng(5)
+    reg, cols, _ = job([8, 4], 50, rng)
+    far = {k: v.copy() for k, v in cols.items()}
+    far["seq"][7] = 3_000_000_000
+    got = []
+    for speculate in (True, False):
+        an = make_pair(reg)[0]
+        an.set_speculation(speculate)
+        for w, c in enumerate((cols, far, cols)):
+            an.trace_upload(w, c)
+            an.analyze_window(w, 1, 10**13)
+        t = an.get_optable(1, to_host=to_host)
+        got.append((t["n_groups"], t["n_slots"], an.get_verdict(1, check=False), an.get_verdict(2)))
+    for G, S, v, after in got:
+        assert G == 0 and S == 0 and v["rc"] == -8 and v["n_groups"] == 0 and v["n_comm_rows_total"] == 0
+        assert all(len(x) == 0 for x in v["comm_rows"].values())
+        assert after["n_groups"] == 100 and after["n_complete"] == 100
+    for k in ("slow_count", "rounds_total", "t_max", "n_rounds"):
+        same(got[0][3]["comm_rows"][k], got[1][3]["comm_rows"][k], k)
