@@ -162,6 +162,7 @@ struct ccld_ctx {
   bool long_list = false;                                // the last suspect list was longer than VD_MERGE
   std::vector<char> long_suspects;                       // columns of a suspect list that outgrew the pinned area
   Block h_up; UploadSlot up[UP_SLOTS]; u32 up_next = 0;
+  cudaStream_t up_stream = nullptr; cudaEvent_t up_event = nullptr;     // see UploadStream
   u64 batches_redone = 0;                                // batches settle() had to analyse again
   std::vector<PendingBatch> pending; std::vector<Block> pinned_free; std::vector<ShapeEntry> shapes;
   u32* d_poison = nullptr; int speculate = 1;
@@ -509,6 +510,29 @@ int upload_slots(ccld_ctx* ctx) {
   for (u32 i = 0; i < UP_SLOTS; ++i) { ctx->up[i].p = (char*)ctx->h_up.p + i * UP_PIECE; ctx->up[i].used = false; }
   return CCLD_OK;
 }
+// The stream that the threads of a large upload copy on. A thread resolves the handle cudaStreamPerThread to its own stream, so
+// for a context on that handle it is a stream of the context's: behind what the caller's stream holds when the upload begins,
+// before what it gets once the upload is through.
+struct UploadStream {
+  ccld_ctx* ctx; cudaStream_t stream;
+  explicit UploadStream(ccld_ctx* c) : ctx(c), stream(c->stream) {}
+  cudaError_t open() {
+    if (ctx->stream != cudaStreamPerThread) return cudaSuccess;
+    cudaError_t e = ctx->up_event ? cudaSuccess : cudaEventCreateWithFlags(&ctx->up_event, cudaEventDisableTiming);
+    if (e == cudaSuccess && !ctx->up_stream) e = cudaStreamCreateWithFlags(&ctx->up_stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->up_event, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->up_stream, ctx->up_event, 0);
+    if (e == cudaSuccess) stream = ctx->up_stream;
+    return e;
+  }
+  cudaError_t close() {                                    // whatever became of the copies
+    if (stream == ctx->stream) return cudaSuccess;
+    const cudaError_t e = cudaEventRecord(ctx->up_event, stream);
+    return e == cudaSuccess ? cudaStreamWaitEvent(ctx->stream, ctx->up_event, 0) : e;
+  }
+  static void drop(ccld_ctx* c) { if (c->up_event) cudaEventDestroy(c->up_event); if (c->up_stream) cudaStreamDestroy(c->up_stream); }
+};
+
 // The pageable columns of an upload. (Where they share a piece with others, those are copied behind it.)
 int upload_pageable(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u32 n_cols) {
   cudaStream_t st = ctx->stream;
@@ -527,6 +551,9 @@ int upload_pageable(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u
     for (size_t a = 0; a < col[i].n; a += UP_PIECE) piece.push_back(UpCol{col[i].off + a, (const char*)col[i].src + a, std::min(UP_PIECE, col[i].n - a)});
   std::atomic<u32> next{0}; std::atomic<int> err{(int)cudaSuccess};
   const int device = ctx->device;
+  UploadStream us(ctx);
+  CK(us.open());
+  st = us.stream;
   auto work = [&](u32 me) {
     if (cudaSetDevice(device) != cudaSuccess) { err = (int)cudaErrorInvalidDevice; return; }
     for (u32 turn = 0; err == (int)cudaSuccess; turn ^= 1) {
@@ -547,6 +574,7 @@ int upload_pageable(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u
   }
   work(0);
   for (auto& t : crew) t.join();
+  CK(us.close());
   CK((cudaError_t)err.load());
   return CCLD_OK;
 }
@@ -682,7 +710,7 @@ int ccld_destroy(ccld_ctx* ctx) {
   for (auto& b : ctx->pending) ctx->pinned_free.push_back(b.pin);
   ctx->pinned_free.push_back(ctx->h_verdict); ctx->pinned_free.push_back(ctx->h_io); ctx->pinned_free.push_back(ctx->h_up);
   for (UploadSlot& u : ctx->up) if (u.done) cudaEventDestroy(u.done);
-  Chains::drop(ctx);
+  Chains::drop(ctx); UploadStream::drop(ctx);
   for (auto& f : ctx->pinned_free) BlockStore::get().put(-1, f);
   BlockStore::get().leave();
   for (auto& sl : ctx->ring) for (int i = 0; i < TIMER_PAIRS; ++i) { cudaEventDestroy(sl.a[i]); cudaEventDestroy(sl.b[i]); }

@@ -316,3 +316,26 @@ def test_a_window_refused_for_its_size_after_one_of_its_shape(to_host):
         assert after["n_groups"] == 100 and after["n_complete"] == 100
     for k in ("slow_count", "rounds_total", "t_max", "n_rounds"):
         same(got[0][3]["comm_rows"][k], got[1][3]["comm_rows"][k], k)
+
+
+def test_large_pageable_upload_on_the_per_thread_stream():
+    """The handle cudaStreamPerThread names another stream in every thread: the library's helpers must not copy on theirs."""
+    from types import SimpleNamespace
+    rng = np.random.default_rng(6)
+    reg, cols, n = job([8], 40_000, rng, spacing=2_000_000, order="shuffled")
+    an, o = ccld.Analyzer(stream=SimpleNamespace(cuda_stream=2)), orc.Oracle()
+    for cid, ranks, seq0 in reg:
+        an.comm_register(cid, ranks, 0, seq0)
+        assert o.comm_register(cid, ranks, seq0) == 0
+    for w in range(3):
+        assert o.upload(w, cols) == 0
+        up = {k: v.copy() for k, v in cols.items()}
+        an.trace_upload(w, up)
+        for v in up.values():
+            v[:] = 0
+        an.analyze_window(w, 1, 10**13)
+        assert o.analyze(w, 1, 10**13) == 0
+        compare_window(an, o, w)
+        if w:
+            an.window_release(w)
+    compare_cumulative(an, o, n, 0)
