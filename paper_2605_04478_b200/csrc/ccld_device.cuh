@@ -35,6 +35,11 @@ constexpr int LARGE_SEQS = 8;          // above: a cluster of eight CTAs per til
 
 // First thing in every kernel: what the kernel before it in the stream wrote is visible from here on, and the next one may be
 // brought to the SMs.
+// A kernel therefore begins while the one before it still writes. What that one may have written - descriptors, ranges, work
+// lists, slot tables, result rows, tick blocks; in the first kernel of a call also the caller's columns - is no read-only memory to
+// it: such memory is read by ordinary loads through pointers that are not restrict, never by __ldg. (Two kernels back is far
+// enough: that one had ended when the wait of the one before let the launch go.) __ldg and const restrict are for the
+// registry's tables and, from the second kernel of a call on, for the caller's columns.
 __device__ __forceinline__ void begin_after() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -195,9 +195,10 @@ static_assert(CCLD_FUSED_MIN_CTAS * (sizeof(FusedShared) + 1024) <= 64 * 1024, "
 constexpr int FUSED_CARVEOUT = (int)((100 * CCLD_FUSED_MIN_CTAS * (sizeof(FusedShared) + 1024) + 228 * 1024 - 1) / (228 * 1024));     // percent
 
 __device__ __forceinline__ void flush_counters(const WinDesc& D, const FusedShared& sh) {
-  count_add(D.counters, C_COMPLETE, sh.cnt[SC_COMP]); count_add(D.counters, C_BARRIER, sh.cnt[SC_BAR]); count_add(D.counters, C_ANALYSED, sh.cnt[SC_AN]);
-  count_add(D.counters, C_MISMATCH, sh.cnt[SC_MIS]); count_add(D.counters, C_PRESENT, sh.cnt[SC_PRES]);
-  count_add(D.counters, C_FLAG_SKEW, sh.cnt[SC_FS]); count_add(D.counters, C_FLAG_DUR, sh.cnt[SC_FD]);
+  u64* const counters = D.counters;
+  count_add(counters, C_COMPLETE, sh.cnt[SC_COMP]); count_add(counters, C_BARRIER, sh.cnt[SC_BAR]); count_add(counters, C_ANALYSED, sh.cnt[SC_AN]);
+  count_add(counters, C_MISMATCH, sh.cnt[SC_MIS]); count_add(counters, C_PRESENT, sh.cnt[SC_PRES]);
+  count_add(counters, C_FLAG_SKEW, sh.cnt[SC_FS]); count_add(counters, C_FLAG_DUR, sh.cnt[SC_FD]);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -453,13 +454,13 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
 // Class-0 CTA: up to FUSED_WT_PER_CTA warp-tiles of one window and one time chunk, each up to 32 consecutive op counters of
 // one communicator with its own summary entry. A warp takes every eighth tile and meets the other warps only at the end, so
 // the warps of a CTA drift apart and one warp's gathers overlap another's arithmetic.
-__device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta& t, const WarpTile* __restrict__ wts, TileSum* __restrict__ sums,
+__device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta& t, const WarpTile* wts, TileSum* __restrict__ sums,
                                                 const Registry& R, const Params& P, const DeferList& DL, FusedShared& sh) {
   const u32 wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr u32 NW = SMALL_SEQS / 32;
   u32* const slots = sh.stage + wid * 256;
-  const u32* __restrict__ list = reinterpret_cast<const u32*>(wts + t.wt_first);
-  const auto entry = [&](u32 i) { return i < t.wt_count ? __ldg(list + (u64)i * 16 + (lane & 15)) : 0u; };
+  const u32* list = reinterpret_cast<const u32*>(wts + t.wt_first);
+  const auto entry = [&](u32 i) { return i < t.wt_count ? list[(u64)i * 16 + (lane & 15)] : 0u; };
   u32 e = entry(wid);
   __syncthreads();                                          // the CTA's counters and pointers are set
   if (wid < t.wt_count) ask_indices(sh, e, lane, slots);
@@ -504,11 +505,11 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
   const u32 sq = threadIdx.x % S, mr = threadIdx.x / S;
   u32 sc[8], rc[8];
   {
-    const u32* __restrict__ pm = ld_volatile(sh.in.perm) + t.row.slot0 + t.seq_off + (sq < count ? sq : 0u);
+    const u32* pm = ld_volatile(sh.in.perm) + t.row.slot0 + t.seq_off + (sq < count ? sq : 0u);
     u32 idx[8], top = 0;
-    const u32 i0 = __ldg(pm);
+    const u32 i0 = *pm;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { const u32 p = mr + (u32)q * L; idx[q] = __ldg(pm + (u64)(FULL || p < n ? p : mr) * t.row.n_seq); top = max(top, idx[q]); }
+    for (int q = 0; q < 8; ++q) { const u32 p = mr + (u32)q * L; idx[q] = pm[(u64)(FULL || p < n ? p : mr) * t.row.n_seq]; top = max(top, idx[q]); }
     u32 bits = top == NONE || i0 == NONE ? 1u : 0u;           // a missing member: the group is set aside
 #pragma unroll
     for (int q = 0; q < 8; ++q) idx[q] = idx[q] == NONE ? 0u : idx[q];
@@ -694,8 +695,8 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
   }
 }
 
-__global__ void __launch_bounds__(SMALL_SEQS, CCLD_FUSED_MIN_CTAS) k_reduce_fused(const WinDesc* __restrict__ wd, const FusedCta* __restrict__ ctas,
-    const WarpTile* __restrict__ wts, TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
+__global__ void __launch_bounds__(SMALL_SEQS, CCLD_FUSED_MIN_CTAS) k_reduce_fused(const WinDesc* wd, const FusedCta* ctas,
+    const WarpTile* wts, TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
   begin_after();
   __shared__ FusedShared sh;
   const FusedCta t = ctas[blockIdx.x];
@@ -748,7 +749,7 @@ __device__ __forceinline__ u64 rank_select(const u64 (&x)[DEF_Q], u32 n, u32 k, 
   return __shfl_sync(FULLM, res, src & 31);
 }
 
-__global__ void __launch_bounds__(DEF_WARPS * 32) k_reduce_deferred(const WinDesc* __restrict__ wd, DeferList DL, Registry R, Params P, i64 now) {
+__global__ void __launch_bounds__(DEF_WARPS * 32) k_reduce_deferred(const WinDesc* wd, DeferList DL, Registry R, Params P, i64 now) {
   begin_after();
   __shared__ u64 s_key[DEF_WARPS][WARP_N];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;

@@ -54,11 +54,12 @@ __device__ __forceinline__ void hang_locate_cta(const WinDesc& D, const Registry
   // a member has entered if it reported this or a later op counter
   const bool covered = row.n_seq > 0 && seq <= row.seq_lo + (row.n_seq - 1);
   const u32 s_first = covered && seq > row.seq_lo ? seq - row.seq_lo : 0;
+  const u32* const perm = D.perm; const i64* const t_exit = D.t_exit;
   for (u32 p = threadIdx.x; p < n; p += HANG_THREADS) {
     u32 st = 0;
     if (covered) {
-      const u32 idx = D.perm[perm_at(row, s_first, p)];
-      if (idx != NONE) st = 1u | (row.seq_lo + s_first == seq && D.t_exit[idx] != -1 ? 2u : 0u);
+      const u32 idx = perm[perm_at(row, s_first, p)];
+      if (idx != NONE) st = 1u | (row.seq_lo + s_first == seq && t_exit[idx] != -1 ? 2u : 0u);
       else if (s_first + 1 < row.n_seq) late[atomicAdd(&s_n_late, 1u)] = p;
     }
     state[p] = st; frame[p] = NONE;
@@ -66,7 +67,7 @@ __device__ __forceinline__ void hang_locate_cta(const WinDesc& D, const Registry
   __syncthreads();
   for (u32 q = wid; q < s_n_late; q += HANG_THREADS / 32) {
     const u32 p = late[q];
-    const u32* __restrict__ col = D.perm + perm_at(row, 0, p);
+    const u32* col = perm + perm_at(row, 0, p);
     bool found = false;
     for (u32 k0 = s_first + 1; k0 < row.n_seq && !found; k0 += 32) found = __any_sync(0xFFFFFFFFu, k0 + lane < row.n_seq && col[k0 + lane] != NONE);
     if (found && lane == 0) state[p] = 1;
@@ -86,7 +87,7 @@ __device__ __forceinline__ void hang_locate_cta(const WinDesc& D, const Registry
       u64 t = 0;
       if (f == NONE) ++n_missing;
       else {
-        const u32* __restrict__ pr = A.progress + (u64)f * A.n_channels * 2;
+        const u32* pr = A.progress + (u64)f * A.n_channels * 2;
         if (((uintptr_t)A.progress & 7) == 0) {
 #pragma unroll 4
           for (u32 ch = 0; ch < A.n_channels; ++ch) { const uint2 x = reinterpret_cast<const uint2*>(pr)[ch]; t += (u64)x.x + x.y; }
@@ -174,7 +175,7 @@ __device__ __forceinline__ void hang_locate_cta(const WinDesc& D, const Registry
   }
 }
 
-__global__ void __launch_bounds__(HANG_THREADS) k_hang_locate(const WinDesc* __restrict__ wd, Registry R, HangArgs A) {
+__global__ void __launch_bounds__(HANG_THREADS) k_hang_locate(const WinDesc* wd, Registry R, HangArgs A) {
   begin_after();
   const WinDesc& D = wd[0];
   if (A.alerts == nullptr) { hang_locate_cta(D, R, A, A.c, A.seq, 0); return; }

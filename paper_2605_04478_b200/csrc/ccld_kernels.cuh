@@ -142,13 +142,14 @@ __device__ __forceinline__ u32 first_left(const u32 (&cid)[REC_RUN], u32 left) {
   return (b & 1u) ? y1 : y0;
 }
 
-__global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* __restrict__ wd, Registry R, u32 blocks_per_cta) {
+__global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Registry R, u32 blocks_per_cta) {
   begin_after();
   extern __shared__ u32 s_dyn[];
   u32* const s_mn = R.n_comms <= RANGE_DIRECT ? s_dyn : nullptr;
   u32* const s_mx = R.n_comms <= RANGE_DIRECT ? s_dyn + R.n_comms : nullptr;
   const WinDesc& D = wd[blockIdx.y];                          // grid: (CTAs of the largest window, windows)
-  if ((u64)blockIdx.x * blocks_per_cta * REC_PER_CTA >= D.n_rec) return;
+  const u64 n_rec = D.n_rec; const u32* const c_comm = D.comm; const u32* const c_seq = D.seq;
+  if ((u64)blockIdx.x * blocks_per_cta * REC_PER_CTA >= n_rec) return;
   const u32 lane = threadIdx.x & 31;
   if (s_mn != nullptr) {
     for (u32 c = threadIdx.x; c < R.n_comms; c += REC_THREADS) { s_mn[c] = NONE; s_mx[c] = 0; }
@@ -158,14 +159,14 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* __rest
   // table's set-up, its barriers and its merge into the window's ranges are paid once
   for (u32 blk = 0; blk < blocks_per_cta; ++blk) {
     const u64 first = ((u64)blockIdx.x * blocks_per_cta + blk) * REC_PER_CTA;
-    if (first >= D.n_rec) break;
-    const u32 n_valid = D.n_rec - first < REC_PER_CTA ? (u32)(D.n_rec - first) : (u32)REC_PER_CTA;
+    if (first >= n_rec) break;
+    const u32 n_valid = n_rec - first < REC_PER_CTA ? (u32)(n_rec - first) : (u32)REC_PER_CTA;
     const u32 r0 = threadIdx.x * REC_RUN;
     const u32 len = r0 >= n_valid ? 0u : (n_valid - r0 < REC_RUN ? n_valid - r0 : (u32)REC_RUN);
     // the run goes straight into registers: four 128-bit loads per column where the column allows it
     u32 cid[REC_RUN], sq[REC_RUN];
     {
-      const u32* __restrict__ pc = D.comm + first + r0; const u32* __restrict__ ps = D.seq + first + r0;
+      const u32* __restrict__ pc = c_comm + first + r0; const u32* __restrict__ ps = c_seq + first + r0;
       if (len == REC_RUN && ((reinterpret_cast<uintptr_t>(pc) | reinterpret_cast<uintptr_t>(ps)) & 15) == 0) {
   #pragma unroll
         for (int q = 0; q < REC_RUN / 4; ++q) {
@@ -273,9 +274,10 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* __rest
   }
   if (s_mn == nullptr) return;
   __syncthreads();
+  u32* const rmin = D.rmin; u32* const rmax = D.rmax;
   for (u32 c = threadIdx.x; c < R.n_comms; c += REC_THREADS) {
     const u32 mn = s_mn[c];
-    if (mn != NONE) { atomicMin(&D.rmin[c], mn); atomicMax(&D.rmax[c], s_mx[c]); }      // nothing waits for these
+    if (mn != NONE) { atomicMin(&rmin[c], mn); atomicMax(&rmax[c], s_mx[c]); }      // nothing waits for these
   }
 }
 
@@ -320,7 +322,7 @@ constexpr u32 SCAT_LOCAL = 8;     // ranks, counted from the rank of the CTA's f
 // first counter), which the layout pass wrote for this window - into shared memory; a record of those ranks then needs no global table at all and, in windows of
 // fewer than 2^32 slots, only 32-bit arithmetic. Any other record (another rank, a communicator beyond the inline pairs,
 // a counter outside the range, a rejected record) takes the two dependent table loads and the full checks.
-__global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc* __restrict__ wd, Registry R, u32 blocks_per_cta) {
+__global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc* wd, Registry R, u32 blocks_per_cta) {
   begin_after();
   // (communicator id, counters covered, first counter, first slot) per resolved pair; counters covered 0: unused. Every
   // warp keeps its own copy, so no warp waits for another; two copies, because the entries of the next block are written
@@ -507,7 +509,7 @@ __device__ __forceinline__ void count_ops(const Registry& R, OpsShared& sh, u32 
 }
 
 // Stage 1 of a batch of several windows, all at once: leaves the part above in the communicator's verdict row.
-__global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* __restrict__ wd, Registry R) {
+__global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* wd, Registry R) {
   begin_after();
   __shared__ OpsShared s_ops;
   const u32 c = blockIdx.x * (WD_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -531,7 +533,7 @@ __global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* __r
 // fetched ahead (range rows two windows, the stage-1 row and the result pointers one window), so the walk waits for
 // arithmetic only. SINGLE: a batch of one window, stage 1 is done here too.
 template <bool SINGLE>
-__global__ void __launch_bounds__(WD_THREADS) k_window_decide(const WinDesc* __restrict__ wd, u32 nw, Registry R, Params P) {
+__global__ void __launch_bounds__(WD_THREADS) k_window_decide(const WinDesc* wd, u32 nw, Registry R, Params P) {
   begin_after();
   __shared__ OpsShared s_ops;
   const u32 c = blockIdx.x * (WD_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;

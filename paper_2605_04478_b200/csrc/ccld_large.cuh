@@ -149,7 +149,7 @@ template <int Q> __device__ __forceinline__ void large_pick(const u32* __restric
 }
 
 template <int Q>
-__global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles,
+__global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(const WinDesc* wd, const Tile* tiles,
     TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
   begin_after();
   extern __shared__ __align__(16) u32 large_keys[];        // [metric][op counter][member of mine], later [metric][member]: my op counter
@@ -175,15 +175,15 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
   {
     const u32 j = lane & 7, pq = lane >> 3;                 // op counter of the tile, member of the quad
     const bool jv = j < t.count;
-    const u32* __restrict__ perm = D.perm + row.slot0 + t.seq_off + (jv ? j : 0u);
+    const u32* perm = D.perm + row.slot0 + t.seq_off + (jv ? j : 0u);
     const i64* __restrict__ c_te = D.t_enter; const i64* __restrict__ c_tx = D.t_exit;
     const u64* __restrict__ c_by = D.bytes; const u8* __restrict__ c_op = D.op;
     const u32* __restrict__ c_sc = D.send_chg; const u32* __restrict__ c_rc = D.recv_chg;
     MidTrack x;
     u32 idx[Q];
-    const u32 i0 = jv ? __ldg(perm) : NONE;
+    const u32 i0 = jv ? *perm : NONE;
 #pragma unroll
-    for (int q = 0; q < Q; ++q) { const u32 m = (wid + LQ_WARPS * (u32)q) * 4 + pq; idx[q] = (jv && m < m_cnt) ? __ldg(perm + (u64)(m0 + m) * row.n_seq) : NONE; }
+    for (int q = 0; q < Q; ++q) { const u32 m = (wid + LQ_WARPS * (u32)q) * 4 + pq; idx[q] = (jv && m < m_cnt) ? perm[(u64)(m0 + m) * row.n_seq] : NONE; }
     i64 te0 = 0; u64 by0 = 0; u32 op0 = 0;
     if (i0 != NONE) { te0 = __ldg(c_te + i0); by0 = __ldg(c_by + i0); op0 = __ldg(c_op + i0); } else x.bits = 1;
     const u64 base = (u64)te0 - 0x80000000ull;
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
   if (threadIdx.x == 0) {
     if (gok) {
       const u64 G = D.n_groups, gr = row.group0 + so;
-      i64* __restrict__ gi = D.gi64 + gr; u32* __restrict__ gu = D.gu32 + gr;
+      i64* __restrict__ gi = D.gi64 + gr; u32* __restrict__ gu = D.gu32 + gr; double* __restrict__ gb = D.gbw + gr; u64* const counters = D.counters;
       const u32 span = sh.group.xmax - emin;
       const bool mismatch = (sh.group.bits & 2) != 0;
       double num, den; bus_factor(sh.gop[me], n, &num, &den);
@@ -329,9 +329,9 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
       gu[(u64)GU_MAX_CHG * G] = (u32)(sh.group.ck >> 32); gu[(u64)GU_RANK_MAX_CHG * G] = sh.ranks[2];
       gu[(u64)GU_N_PRESENT * G] = n;
       gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mismatch ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
-      D.gbw[gr] = span ? (double)sh.gby[me] * num * rcp_newton((double)span * den) : 0.0;
-      count_add(D.counters, C_COMPLETE, 1); count_add(D.counters, C_PRESENT, n); count_add(D.counters, C_BARRIER, barrier); count_add(D.counters, C_ANALYSED, analysed);
-      count_add(D.counters, C_MISMATCH, mismatch); count_add(D.counters, C_FLAG_SKEW, sh.n_fs); count_add(D.counters, C_FLAG_DUR, sh.n_fd);
+      *gb = span ? (double)sh.gby[me] * num * rcp_newton((double)span * den) : 0.0;
+      count_add(counters, C_COMPLETE, 1); count_add(counters, C_PRESENT, n); count_add(counters, C_BARRIER, barrier); count_add(counters, C_ANALYSED, analysed);
+      count_add(counters, C_MISMATCH, mismatch); count_add(counters, C_FLAG_SKEW, sh.n_fs); count_add(counters, C_FLAG_DUR, sh.n_fd);
     } else if (gvalid) {                                    // set aside for the 64-bit kernel
       const u32 e = atomicAdd(DL.count, 1u);
       DL.entries[e] = ((u64)t.w << 32) | (u64)(row.group0 + so);
@@ -421,7 +421,7 @@ __device__ u64 radix_select(F key, u32 n, u32 k, u64 max_key, u32* hist /*[256]*
   return prefix;
 }
 
-__global__ void __launch_bounds__(LARGE_DEF_THREADS) k_reduce_large_deferred(const WinDesc* __restrict__ wd, DeferList DL, Registry R, Params P, i64 now) {
+__global__ void __launch_bounds__(LARGE_DEF_THREADS) k_reduce_large_deferred(const WinDesc* wd, DeferList DL, Registry R, Params P, i64 now) {
   begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ u64 s_red64[32];
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(LARGE_DEF_THREADS) k_reduce_large_deferred(con
     __syncthreads();
     const u64 slot = row.slot0 + (u64)so * n;                      // flags, group-major
     const u32 seq = row.seq_lo + so;
-    const u32* __restrict__ pm = D.perm + perm_at(row, so, 0);     // member p at pm[p * n_seq]
+    const u32* pm = D.perm + perm_at(row, so, 0);     // member p at pm[p * n_seq]
     const u64 pst = row.n_seq;
     // pass 1: gather, presence, first present member
     u32 npres = 0, first = NONE, stor = 0;

@@ -132,7 +132,7 @@ struct MidTrack {
 };
 
 template <int R>
-__global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(const WinDesc* __restrict__ wd, const Tile* __restrict__ tiles,
+__global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(const WinDesc* wd, const Tile* tiles,
     TileSum* __restrict__ sums, Registry R_, Params P, DeferList DL) {
   begin_after();
   extern __shared__ __align__(16) u32 mid_keys[];
@@ -157,19 +157,19 @@ __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(cons
   {
     const u32 j = lane & 7, ml = lane >> 3;
     const bool jv = j < t.count;
-    const u32* __restrict__ perm = D.perm + row.slot0 + t.seq_off + (jv ? j : 0u);
+    const u32* perm = D.perm + row.slot0 + t.seq_off + (jv ? j : 0u);
     const i64* __restrict__ c_te = D.t_enter; const i64* __restrict__ c_tx = D.t_exit;
     const u64* __restrict__ c_by = D.bytes; const u8* __restrict__ c_op = D.op;
     const u32* __restrict__ c_sc = D.send_chg; const u32* __restrict__ c_rc = D.recv_chg;
     MidTrack x;
     i64 te0 = 0; u64 by0 = 0; u32 op0 = 0;
-    const u32 i0 = jv ? __ldg(perm) : NONE;
+    const u32 i0 = jv ? *perm : NONE;
     if (i0 != NONE) { te0 = c_te[i0]; by0 = c_by[i0]; op0 = c_op[i0]; } else x.bits = 1;
     const u64 base = (u64)te0 - 0x80000000ull;
     for (u32 p0 = wid * 4 + ml; p0 < n; p0 += 4 * 4 * MID_WARPS) {
       u32 idx[4]; i64 ta[4], tb[4]; u64 by[4]; u32 op[4], ch[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { const u32 p = p0 + q * 4 * MID_WARPS; idx[q] = (jv && p < n) ? __ldg(perm + (u64)p * row.n_seq) : NONE; }
+      for (int q = 0; q < 4; ++q) { const u32 p = p0 + q * 4 * MID_WARPS; idx[q] = (jv && p < n) ? perm[(u64)p * row.n_seq] : NONE; }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const u32 ix = idx[q] == NONE ? 0u : idx[q];
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(cons
         n_fs = __reduce_add_sync(FULLM, n_fs); n_fd = __reduce_add_sync(FULLM, n_fd);
         if (lane == 0) {
           const u64 G = D.n_groups, gr = row.group0 + so;
-          i64* __restrict__ gi = D.gi64 + gr; u32* __restrict__ gu = D.gu32 + gr;
+          i64* __restrict__ gi = D.gi64 + gr; u32* __restrict__ gu = D.gu32 + gr; double* __restrict__ gb = D.gbw + gr;
           const u32 span = x.xmax - emin;
           gi[(u64)GI_E_MIN * G] = (i64)(s_base[g] + emin); gi[(u64)GI_ARRIVAL_SKEW * G] = (i64)(u64)(x.emax - emin);
           gi[(u64)GI_T_MAX * G] = (i64)(u64)tmx; gi[(u64)GI_T_MIN * G] = (i64)(u64)tmn; gi[(u64)GI_SPAN * G] = (i64)(u64)span;
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(cons
           gu[(u64)GU_MAX_CHG * G] = (u32)(x.ck >> 32); gu[(u64)GU_RANK_MAX_CHG * G] = mem[NONE - (u32)x.ck];
           gu[(u64)GU_N_PRESENT * G] = n;
           gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mismatch ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
-          D.gbw[gr] = span ? bnum * rcp_newton((double)span * den) : 0.0;
+          *gb = span ? bnum * rcp_newton((double)span * den) : 0.0;
           atomicAdd(&s_cnt[SC_COMP], 1u);
           if (barrier) atomicAdd(&s_cnt[SC_BAR], 1u);
           if (analysed) atomicAdd(&s_cnt[SC_AN], 1u);
@@ -294,9 +294,10 @@ __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(cons
       ts.n_an += (s_state[g] >> 1) & 1; ts.pad += s_state[g] >> 2;
     }
     sums[blockIdx.x] = ts;
-    count_add(D.counters, C_COMPLETE, s_cnt[SC_COMP]); count_add(D.counters, C_BARRIER, s_cnt[SC_BAR]); count_add(D.counters, C_ANALYSED, s_cnt[SC_AN]);
-    count_add(D.counters, C_MISMATCH, s_cnt[SC_MIS]); count_add(D.counters, C_PRESENT, s_cnt[SC_COMP] * n);
-    count_add(D.counters, C_FLAG_SKEW, s_cnt[SC_FS]); count_add(D.counters, C_FLAG_DUR, s_cnt[SC_FD]);
+    u64* const counters = D.counters;
+    count_add(counters, C_COMPLETE, s_cnt[SC_COMP]); count_add(counters, C_BARRIER, s_cnt[SC_BAR]); count_add(counters, C_ANALYSED, s_cnt[SC_AN]);
+    count_add(counters, C_MISMATCH, s_cnt[SC_MIS]); count_add(counters, C_PRESENT, s_cnt[SC_COMP] * n);
+    count_add(counters, C_FLAG_SKEW, s_cnt[SC_FS]); count_add(counters, C_FLAG_DUR, s_cnt[SC_FD]);
   }
 }
 

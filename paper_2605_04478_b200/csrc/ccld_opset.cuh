@@ -23,7 +23,7 @@ struct OpsetArgs {
   ccld_opset_verdict* out;       // pinned (pointer fields unused)
 };
 
-__global__ void __launch_bounds__(OPSET_THREADS) k_opset_check(const WinDesc* __restrict__ wd, Registry R, OpsetArgs A) {
+__global__ void __launch_bounds__(OPSET_THREADS) k_opset_check(const WinDesc* wd, Registry R, OpsetArgs A) {
   begin_after();
   extern __shared__ __align__(16) unsigned char opset_smem[];
   constexpr u32 PRESENT = 0x80000000u, COUNTED = 0x40000000u, TUPLE = 0xFFFFFFu;
@@ -40,12 +40,13 @@ __global__ void __launch_bounds__(OPSET_THREADS) k_opset_check(const WinDesc* __
   __syncthreads();
   const bool in_range = row.n_seq > 0 && A.seq >= row.seq_lo && A.seq - row.seq_lo < row.n_seq;
   u32 n_present = 0, first = NONE;
+  const u32* const perm = D.perm; const u64* const c_by = D.bytes; const u8* const c_op = D.op;
   for (u32 p = threadIdx.x; p < n; p += OPSET_THREADS) {
-    const u32 idx = in_range ? D.perm[perm_at(row, A.seq - row.seq_lo, p)] : NONE;
+    const u32 idx = in_range ? perm[perm_at(row, A.seq - row.seq_lo, p)] : NONE;
     u64 h = 0; u32 l = 0;
     if (idx != NONE) {
-      h = D.bytes[idx];
-      l = (u32)D.op[idx] | (A.algo ? (u32)A.algo[idx] << 8 : 0u) | (A.proto ? (u32)A.proto[idx] << 16 : 0u) | PRESENT;
+      h = c_by[idx];
+      l = (u32)c_op[idx] | (A.algo ? (u32)A.algo[idx] << 8 : 0u) | (A.proto ? (u32)A.proto[idx] << 16 : 0u) | PRESENT;
       ++n_present; first = min(first, p);
     }
     hi[p] = h; lo[p] = l;

@@ -90,7 +90,7 @@ struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; };
 // differ gives up and raises the poison flag; so does every window planned after the flag went up - in the same batch
 // (seen by k_emit) or in a later one - so that windows are never analysed out of order.
 // Grid: (1 + filling CTAs, windows). fill: whether the slot table (sized from the expectation) is to be set to NONE.
-__global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __restrict__ wd, Registry R, int fill) {
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Registry R, int fill) {
   begin_after();
   __shared__ PlanAcc s_warp[33];
   __shared__ u32 s_red[32];
@@ -219,13 +219,15 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
         t[T_TILES2] = all.t2; t[T_TILES3] = all.t3; t[T_ROWS] = all.rows;
       }
       t[T_FAILED] = failed; t[T_CHUNKS] = failed ? 1 : T;
-      for (int q = 0; q < T_COUNT; ++q) { D.totals[q] = t[q]; D.totals_host[q] = t[q]; }
+      u64* const totals = D.totals; u64* const totals_host = D.totals_host;
+      for (int q = 0; q < T_COUNT; ++q) { totals[q] = t[q]; totals_host[q] = t[q]; }
       if (failed == FAILED_CAPACITY) atomicOr((unsigned*)&D.counters[C_ERR], (unsigned)CCLD_E_CAPACITY);
       s_red[0] = failed != 0;
     }
   }
   __syncthreads();
   const bool failed = s_red[0] != 0;                           // a window that is given up leaves no work behind: empty rows
+  RangeRow* const ranges = D.ranges; uint4* const srow = D.srow; const u32* const rmin = D.rmin;
   each([&](u32 k, u32 ns, u32 n) {
     const u32 c = c_lo + k;
     if (c >= c_hi) return;
@@ -233,11 +235,11 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
     RangeRow r = {0, 0, 0, n, 0, 0, 0, 0};
     if (!failed) {
       const u32 cls = comm_class(n);
-      r.seq_lo = ns ? D.rmin[c] : 0; r.n_seq = ns; r.row_idx = run.rows; r.group0 = run.groups; r.slot0 = run.slots;
+      r.seq_lo = ns ? rmin[c] : 0; r.n_seq = ns; r.row_idx = run.rows; r.group0 = run.groups; r.slot0 = run.slots;
       r.tile0 = cls <= 1 ? run.units : (cls == 2 ? run.t2 : run.t3); r.n_units = it.units + it.t2 + it.t3;
     }
-    D.ranges[c] = r;
-    D.srow[c] = make_uint4((u32)r.slot0, (u32)(r.slot0 >> 32), r.n_seq, r.seq_lo);
+    ranges[c] = r;
+    srow[c] = make_uint4((u32)r.slot0, (u32)(r.slot0 >> 32), r.n_seq, r.seq_lo);
     run = plan_add(run, it);
   });
 }
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* __rest
 // communicators (one time, unless a registry has more than EMIT_SLICES times as many). There are enough of them for every
 // chunk of any window of the batch. base[] of the descriptors is filled. A window that gave up fills its stretch of the
 // lists with entries that hold no work, because the kernels that follow are launched over the expected lengths.
-__global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict__ wd, Registry R, PlanLists L, u32 chunk_ctas, u32 slices, u32 blocks) {
+__global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* wd, Registry R, PlanLists L, u32 chunk_ctas, u32 slices, u32 blocks) {
   begin_after();
   __shared__ uint4 s_pair[EMIT_THREADS / 32];
   const WinDesc& D = wd[blockIdx.y];
@@ -261,6 +263,7 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict
     // where slots fit 32 bits and the member's whole column lies inside the table; other entries stay unused.
     const bool usable = !give_up && n_slots <= 0xFFFFFFFFull;
     const u64 st = (u64)(gridDim.x - chunk_ctas) * EMIT_THREADS;
+    const uint4* const srow = D.srow; uint4* const rent = D.rent;
     for (u64 i = (u64)(blockIdx.x - chunk_ctas) * EMIT_THREADS + threadIdx.x; i < (u64)R.n_ranks * 2; i += st) {
       uint4 e[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
       if (usable) {
@@ -269,13 +272,13 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* __restrict
         for (int h = 0; h < 2; ++h) {
           const u32 id = h ? t.z : t.x, cp = h ? t.w : t.y;
           if (id != NONE && cp != NONE && cp != RANK_TAB_OVERFLOW) {
-            const uint4 sr = D.srow[cp >> RANK_TAB_POS_BITS];
+            const uint4 sr = srow[cp >> RANK_TAB_POS_BITS];
             const u64 b = ((u64)sr.x | ((u64)sr.y << 32)) + (u64)(cp & ((1u << RANK_TAB_POS_BITS) - 1)) * sr.z;
             if (sr.z != 0 && b + sr.z <= n_slots) e[h] = make_uint4(id, sr.z, sr.w, (u32)b);
           }
         }
       }
-      D.rent[i * 2] = e[0]; D.rent[i * 2 + 1] = e[1];
+      rent[i * 2] = e[0]; rent[i * 2 + 1] = e[1];
     }
     return;
   }

@@ -40,13 +40,13 @@ struct TickArgs {
 };
 
 // the eight counters from tick i on (past the end: the last one there is, so that nothing changes)
-__device__ __forceinline__ void eight_ticks(const u32* __restrict__ c, u64 i, u64 n, bool vec, u32 (&v)[8]) {
+__device__ __forceinline__ void eight_ticks(const u32* c, u64 i, u64 n, bool vec, u32 (&v)[8]) {
   if (vec && i + 8 <= n) {
-    const uint4 a = __ldg(reinterpret_cast<const uint4*>(c + i)), b = __ldg(reinterpret_cast<const uint4*>(c + i) + 1);
+    const uint4 a = reinterpret_cast<const uint4*>(c + i)[0], b = reinterpret_cast<const uint4*>(c + i)[1];
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
   } else {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = __ldg(c + (i + k < n ? i + k : n - 1));
+    for (int k = 0; k < 8; ++k) v[k] = c[i + k < n ? i + k : n - 1];
   }
 }
 __device__ __forceinline__ u32 change_bits(const u32 (&v)[8], u32 before) {
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_tick_blocks(TickArgs A) {
   u32 ps = __shfl_up_sync(0xFFFFFFFFu, sv[7], 1), pr = __shfl_up_sync(0xFFFFFFFFu, rv[7], 1);
   if (lane == 0) {
     const u64 b = i ? (i - 1 < A.n_ticks ? i - 1 : A.n_ticks - 1) : 0;
-    ps = __ldg(A.send + b); pr = __ldg(A.recv + b);
+    ps = A.send[b]; pr = A.recv[b];
   }
   u32 ms = change_bits(sv, ps), mr = change_bits(rv, pr);
   const u32 cnt = (u32)__popc(ms) | ((u32)__popc(mr) << 16);          // a tile has 2,048 ticks: sixteen bits are enough
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_tick_blocks(TickArgs A) {
 // to step; the warps' totals are scanned by every warp.
 constexpr int TS_THREADS = 1024;
 constexpr int TS_PER = 16;
-__global__ void __launch_bounds__(TS_THREADS) k_tile_scan(uint2* __restrict__ tile, u32 n_tiles) {
+__global__ void __launch_bounds__(TS_THREADS) k_tile_scan(uint2* tile, u32 n_tiles) {
   begin_after();
   __shared__ u64 s_warp[TS_THREADS / 32];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_record_rates(TickArgs A, u64 n_r
   RankTicks r; r.t0 = r.t1 = 0; r.lo = r.n = 0; r.scale = 0.f;
   if (rk < A.n_ranks) {
     const uint4* e = reinterpret_cast<const uint4*>(A.ranks + rk);
-    const uint4 x = __ldg(e), y = __ldg(e + 1);
+    const uint4 x = e[0], y = e[1];
     r.t0 = (i64)((u64)x.x | ((u64)x.y << 32)); r.t1 = (i64)((u64)x.z | ((u64)x.w << 32));
     r.lo = y.x; r.n = y.y; r.scale = __uint_as_float(y.z);
   }
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_record_rates(TickArgs A, u64 n_r
   const u32 ia = r.lo + (ca ? ca - 1 : 0u), ib = r.lo + (cb ? cb - 1 : 0u);
   if (ib > ia) {
     const uint4* t = reinterpret_cast<const uint4*>(A.blk);
-    const uint4 ea = __ldg(t + (ia >> 5)), eb = __ldg(t + (ib >> 5));
+    const uint4 ea = t[ia >> 5], eb = t[ib >> 5];
     const u32 pa = changes_upto(TickBlock{ea.x, ea.y, ea.z, 0}, ia), pb = changes_upto(TickBlock{eb.x, eb.y, eb.z, 0}, ib);
     s = (pb & 0xFFFFu) - (pa & 0xFFFFu); q = (pb >> 16) - (pa >> 16);
     const u32 ta = ia / RT_TILE, tb = ib / RT_TILE;

@@ -15,7 +15,7 @@ constexpr int TREE_THREADS = 256;
 // rate columns in the selected round; the root is the member with the most changes above its layer's fewest (equal
 // excesses: the lowest position). If no layer disagrees with itself the rates name nobody and the member with the
 // longest duration stands in, as it does for a window without rate columns.
-__global__ void __launch_bounds__(TREE_THREADS) k_tree_root_comm(const WinDesc* __restrict__ wd, const TreeRef* __restrict__ trees, Registry R) {
+__global__ void __launch_bounds__(TREE_THREADS) k_tree_root_comm(const WinDesc* wd, const TreeRef* __restrict__ trees, Registry R) {
   begin_after();
   __shared__ u32 s_ch[CCLD_MAX_COMM_SIZE];
   __shared__ u32 s_red[32];

@@ -64,7 +64,7 @@ __device__ __forceinline__ void put_alert(ccld_hang_alert* out, u32 i, u32 n, bo
 
 // The alerts of a window in the order they are listed: registration order of the communicator, then op counter (then the
 // place in the unordered list: an op raises one alert). One CTA; s_key holds CCLD_MAX_ALERTS_PER_WINDOW keys.
-__device__ __forceinline__ void order_alerts(const Registry& R, const ccld_hang_alert* __restrict__ in, u32 n, ccld_hang_alert* __restrict__ out, bool columns, u64* s_key) {
+__device__ __forceinline__ void order_alerts(const Registry& R, const ccld_hang_alert* in, u32 n, ccld_hang_alert* out, bool columns, u64* s_key) {
   for (u32 i = threadIdx.x; i < n; i += blockDim.x) s_key[i] = ((u64)comm_lookup(R, in[i].comm) << 32) | in[i].seq;
   __syncthreads();
   for (u32 i = threadIdx.x; i < n; i += blockDim.x) {
@@ -216,7 +216,7 @@ constexpr u32 GATHER_PIECES = 24;
 struct GatherArgs { struct { const unsigned char* src; unsigned char* dst; u64 n; } piece[GATHER_PIECES]; };
 __global__ void __launch_bounds__(GATHER_THREADS) k_gather(GatherArgs A) {
   begin_after();
-  const unsigned char* __restrict__ src = A.piece[blockIdx.y].src; unsigned char* __restrict__ dst = A.piece[blockIdx.y].dst;
+  const unsigned char* src = A.piece[blockIdx.y].src; unsigned char* __restrict__ dst = A.piece[blockIdx.y].dst;
   const u64 n = A.piece[blockIdx.y].n;
   const u64 head = min(n, (u64)((16 - ((uintptr_t)src & 15)) & 15)), n16 = (n - head) / 16, tail = head + n16 * 16;
   const u64 i0 = (u64)blockIdx.x * GATHER_THREADS + threadIdx.x, st = (u64)gridDim.x * GATHER_THREADS;
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(GatherArgs A) {
 }
 
 // communicator id, op counter and first slot of every group of a window
-__global__ void __launch_bounds__(256) k_op_keys(const RangeRow* __restrict__ ranges, Registry R, u64 n_groups, u32* __restrict__ comm, u32* __restrict__ seq, u64* __restrict__ slot0) {
+__global__ void __launch_bounds__(256) k_op_keys(const RangeRow* ranges, Registry R, u64 n_groups, u32* __restrict__ comm, u32* __restrict__ seq, u64* __restrict__ slot0) {
   begin_after();
   const u64 g = (u64)blockIdx.x * 256 + threadIdx.x;
   if (g >= n_groups) return;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(256) k_op_keys(const RangeRow* __restrict__ ra
 }
 
 // the ordered alerts alone, for the hang sweep
-__global__ void __launch_bounds__(VD_THREADS) k_order_alerts(const u64* __restrict__ counters, const ccld_hang_alert* __restrict__ in, ccld_hang_alert* __restrict__ out, Registry R) {
+__global__ void __launch_bounds__(VD_THREADS) k_order_alerts(const u64* counters, const ccld_hang_alert* in, ccld_hang_alert* out, Registry R) {
   begin_after();
   __shared__ u64 s_key[CCLD_MAX_ALERTS_PER_WINDOW];
   const u64 n = counters[C_ALERTS];
