@@ -40,8 +40,10 @@ struct CommHost {
 
 // What contexts that are gone leave to those that live: a process-wide store of pinned and device blocks. Allocating is what a
 // context's first pass costs most (measured: cudaMallocHost 1 to 13 ms, cudaMalloc 0.36 ms whatever the size), and programs
-// make a context per job or per device. The store is bounded, every access holds its lock, blocks enter it only once their
-// stream has been waited for, and it is emptied when the last context goes or an allocation fails.
+// make a context per job or per device. A small or ordinary job's first pass needs some tens of MB; larger ones do not notice
+// an allocation, and their memory is wanted elsewhere in the process. So the store holds at most 64 MB of each kind (of each
+// device). Every access holds its lock, blocks enter it only once their stream has been waited for, and it is emptied when the
+// last context goes or an allocation fails.
 class BlockStore {
  public:
   static BlockStore& get() { static BlockStore* s = new BlockStore; return *s; }      // never destroyed: contexts may outlive static objects
@@ -73,7 +75,7 @@ class BlockStore {
   }
 
  private:
-  static constexpr size_t PINNED_MOST = 64u << 20, DEVICE_MOST = 512u << 20, LENT_MOST = 64u << 20;
+  static constexpr size_t PINNED_MOST = 64u << 20, DEVICE_MOST = 64u << 20, LENT_MOST = 64u << 20;
   static void free_block(int device, Block b) { if (device < 0) cudaFreeHost(b.p); else cudaFree(b.p); }   // (cudaFree takes any device's pointer)
   void drain() { for (auto& kv : lists_) { for (Block& b : kv.second) free_block(kv.first, b); kv.second.clear(); held_[kv.first] = 0; } }
   std::mutex m_; int users_ = 0; size_t lent_ = 0;
@@ -702,7 +704,7 @@ int ccld_create(ccld_ctx** out, const ccld_params* params, int device, void* cud
 int ccld_destroy(ccld_ctx* ctx) {
   if (!ctx) return CCLD_ERR_ARG;
   cudaSetDevice(ctx->device);
-  cudaStreamSynchronize(ctx->stream);
+  if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) { cudaGetLastError(); cudaDeviceSynchronize(); }      // (the caller's stream may be gone)
   for (auto& kv : ctx->windows) { drop_results(kv.second); if (kv.second.owns) ctx->pool.put(kv.second.own); if (kv.second.owns_opset) ctx->pool.put(kv.second.opset_own); }
   ctx->windows.clear();
   ctx->pool.put(ctx->reg_blk); ctx->pool.put(ctx->misc_blk);

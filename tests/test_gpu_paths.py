@@ -1,6 +1,7 @@
 """The library's size-dependent paths at the sizes where they can go wrong, against the CPU oracle: whole numbers must be
 identical, fp64 quantities within 1e-9 relative (tests/parity.py)."""
 import ctypes as C
+import gc
 
 import numpy as np
 import pytest
@@ -339,3 +340,32 @@ def test_large_pageable_upload_on_the_per_thread_stream():
         if w:
             an.window_release(w)
     compare_cumulative(an, o, n, 0)
+
+
+def test_device_memory_goes_back_with_its_context():
+    """While another context lives, a context that is closed leaves it blocks of no more than 64 MB in all; the last one to go
+    leaves nothing."""
+    rng = np.random.default_rng(9)
+    reg, cols, _ = job([8], 400_000, rng, spacing=2_000_000)
+
+    def passes():
+        an = make_pair(reg)[0]
+        an.trace_upload(0, cols)
+        an.analyze_window(0, 1, 10**13)
+        assert an.get_verdict(0)["n_complete"] == 400_000
+        return an
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+    gc.collect()                                                # contexts of earlier tests
+    passes().close()                                            # what the process itself keeps is there by now
+    first = free()
+    other = ccld.Analyzer()
+    an = passes()
+    held = first - free()
+    assert held > 150 << 20
+    an.close()
+    assert first - free() <= 66 << 20
+    other.close()
+    assert first - free() <= 2 << 20
