@@ -76,7 +76,14 @@ class BlockStore {
 
  private:
   static constexpr size_t PINNED_MOST = 64u << 20, DEVICE_MOST = 64u << 20, LENT_MOST = 64u << 20;
-  static void free_block(int device, Block b) { if (device < 0) cudaFreeHost(b.p); else cudaFree(b.p); }   // (cudaFree takes any device's pointer)
+  // Blocks are freed whenever the last array on one goes, also while the caller captures a graph: with this thread's own
+  // captures set aside, freeing is no part of them and does not end them. (cudaFree takes any device's pointer.)
+  static void free_block(int device, Block b) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (device < 0) cudaFreeHost(b.p); else cudaFree(b.p);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
   void drain() { for (auto& kv : lists_) { for (Block& b : kv.second) free_block(kv.first, b); kv.second.clear(); held_[kv.first] = 0; } }
   std::mutex m_; int users_ = 0; size_t lent_ = 0;
   std::map<int, std::vector<Block>> lists_; std::map<int, size_t> held_;

@@ -369,3 +369,23 @@ def test_device_memory_goes_back_with_its_context():
     assert first - free() <= 66 << 20
     other.close()
     assert first - free() <= 2 << 20
+
+
+def test_results_may_be_dropped_while_a_graph_is_captured():
+    """The last array on a pinned block gives it back, and with no context left it is freed: not a step of a capture."""
+    gc.collect()                                                # contexts of earlier tests
+    rng = np.random.default_rng(10)
+    reg, cols, n = job([4], 50, rng)
+    an, _ = run(reg, cols, n)
+    kept = [an.get_optable(0), an.get_rank_stats(n)]
+    an.close()
+    x = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        x += 1
+        kept.clear()
+        x += 1
+    g.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [2] * 8
