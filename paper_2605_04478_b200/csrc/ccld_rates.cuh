@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_tick_blocks(TickArgs A) {
   if (blockIdx.x >= A.n_tiles) {
     const u64 r = (u64)(blockIdx.x - A.n_tiles) * RT_THREADS + threadIdx.x;
     if (r >= A.n_ranks) return;
-    const u64 lo = A.tick_off[r], hi = A.tick_off[r + 1];
+    const u64 lo = min(A.tick_off[r], A.n_ticks), hi = min(A.tick_off[r + 1], A.n_ticks);      // (every rank is looked at, also one without records)
     RankTicks x; x.t0 = 0; x.t1 = 0; x.lo = (u32)lo; x.n = hi > lo ? (u32)(hi - lo) : 0u; x.scale = 0.f; x.pad = 0;
     if (x.n) {
       x.t0 = A.tick_ns[lo]; x.t1 = A.tick_ns[hi - 1];

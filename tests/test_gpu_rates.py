@@ -125,3 +125,21 @@ def test_every_op_spans_hundreds_of_ticks():
     tx[rng.random(n) < 0.1] = -1
     es, _ = _check(ccld.Analyzer(), rank, te, tx, off, tn, sc, rc)
     assert np.median(es) > 50
+
+
+def test_offsets_beyond_the_samples():
+    """A table whose last ranks, which have no records, end beyond the samples there are; one that has some ends with them."""
+    rng = np.random.default_rng(12)
+    off, tn, sc, rc = _series(rng, 4, 3000)
+    n_rec = 2000
+    rank = rng.integers(0, 5, n_rec)
+    te = rng.integers(0, 3000, n_rec) * MS; tx = te + rng.integers(0, 300 * MS, n_rec)
+    tx[::50] = -1
+    es, er = orc.derive_rates(rank, te, tx, off, tn, sc, rc)
+    t = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a).astype(dt)).cuda()
+    for more in ([], [off[-1] + 10**9], [off[-1] + 5, 1 << 40, 1 << 62]):
+        o = np.concatenate([off[:-1], [off[-1] if more else off[-1] + 77], more]).astype(np.int64)
+        keep = rank < 4 if more else np.ones(n_rec, bool)
+        s, r = ccld.Analyzer().derive_rates(t(rank[keep], np.int32), t(te[keep], np.int64), t(tx[keep], np.int64), t(o, np.int64), t(tn, np.int64), t(sc, np.int32), t(rc, np.int32))
+        torch.cuda.synchronize()
+        assert np.array_equal(s.cpu().numpy().view(np.uint32), es[keep]) and np.array_equal(r.cpu().numpy().view(np.uint32), er[keep])
