@@ -1482,7 +1482,8 @@ int ccld_derive_rates(ccld_ctx* ctx, uint64_t n_rec, const uint32_t* rank, const
   const u64 n_tiles = (n_ticks + RT_TILE - 1) / RT_TILE;
   size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + b); return o; };
-  const size_t o_blk = take(n_tiles * (RT_TILE / 32) * sizeof(TickBlock)), o_tile = take(n_tiles * sizeof(uint2)), o_rank = take(n_ranks * sizeof(RankTicks));
+  const size_t o_blk = take(n_tiles * (RT_TILE / 32) * sizeof(TickBlock)), o_tile = take(n_tiles * sizeof(uint2)), o_rank = take(n_ranks * sizeof(RankTicks)),
+               o_far = take((((u64)n_ranks + RT_THREADS - 1) / RT_THREADS + 1) * 4);
   cudaError_t e;
   Block blk = ctx->pool.get(off, &e);
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "scratch allocation failed");
@@ -1490,12 +1491,10 @@ int ccld_derive_rates(ccld_ctx* ctx, uint64_t n_rec, const uint32_t* rank, const
   A.tick_off = tick_off; A.tick_ns = tick_ns; A.send = send_count; A.recv = recv_count;
   A.blk = (TickBlock*)((char*)blk.p + o_blk); A.tile = (uint2*)((char*)blk.p + o_tile); A.ranks = (RankTicks*)((char*)blk.p + o_rank);
   A.vec = (((uintptr_t)send_count | (uintptr_t)recv_count) & 15) == 0;
-  // A record adds up the tiles its op spans. Ops of one rank hardly overlap, so that is a read or two per record while a
-  // rank's samples cover a few tiles (8 tiles = 16 s at a sample per millisecond); with longer segments an op in flight
-  // since their beginning would add up many, and the scan (5 to 15 us) pays.
-  A.scanned = n_tiles > 256 && n_tiles > 8ull * n_ranks;
-  launch(st, k_tick_blocks, (u32)(n_tiles + ((u64)n_ranks + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, A);
-  if (A.scanned) launch(st, k_tile_scan, 1, TS_THREADS, 0, A.tile, A.n_tiles);
+  const u32 rank_ctas = (u32)(((u64)n_ranks + RT_THREADS - 1) / RT_THREADS);
+  A.far = (u32*)((char*)blk.p + o_far); A.scanned = n_tiles > RT_SCAN ? A.far + rank_ctas : nullptr;
+  launch(st, k_tick_blocks, (u32)n_tiles + rank_ctas, RT_THREADS, 0, A);
+  if (A.scanned) launch(st, k_tile_scan, 1, TS_THREADS, 0, A.tile, A.n_tiles, n_tiles > (u64)RT_NEAR * n_ranks ? nullptr : A.far, rank_ctas, A.scanned);
   launch(st, k_record_rates, (u32)((n_rec + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, A, n_rec, rank, t_enter_ns, t_exit_ns, send_chg, recv_chg);
   const cudaError_t le = cudaGetLastError();
   ctx->pool.put(blk);           // later work on this stream runs after these kernels: the block can be handed out again

@@ -4,8 +4,10 @@
 //
 //   k_tick_blocks   per block of 32 ticks: which ticks carry another SendCount / RecvCount than the tick before, as two
 //                   32-bit masks with the number of changes before the block inside its tile of 2,048 ticks; per tile the
-//                   number of changes. Further CTAs note per rank where its ticks lie in the table and in time.
-//   k_tile_scan     only for long segments: exclusive prefix over the tiles' numbers (one CTA)
+//                   number of changes. Further CTAs note per rank where its ticks lie in the table and in time, and
+//                   whether a rank's ticks cover more than RT_NEAR tiles.
+//   k_tile_scan     only for long segments: exclusive prefix over the tiles' numbers (one CTA). Where the host cannot tell from
+//                   the average that there are any, the kernel is launched and looks.
 //   k_record_rates  per record: the two ticks around its enter time and the two around its exit time, at the places even
 //                   spacing gives (checked; a search where the samples are not even), then a difference of prefixes
 //
@@ -23,6 +25,12 @@ namespace ccld {
 
 constexpr int RT_THREADS = 256;
 constexpr int RT_TILE = RT_THREADS * 8;            // ticks per CTA of k_tick_blocks, eight consecutive ones per lane
+// A record adds up the tiles its op spans. Ops of one rank hardly overlap, so that is a read or two per record while no rank's
+// samples cover more than this many tiles (8 tiles = 16 s at a sample per millisecond). With longer segments an op in flight
+// since their beginning would add up many, and the scan pays: 20,000 tiles of one rank among 4,096, 50,000 records: 1,067 -> 99 us. (4,096 equal ranks of 5,600 ticks,
+// whose scan is launched to find that out: 80.1 -> 81.5 us.)
+constexpr u32 RT_NEAR = 8;
+constexpr u64 RT_SCAN = 256;                       // up to so many tiles in all a record adds them up whatever the segments are
 
 // before: changes before the block inside the tile (send in the low half, recv in the high half); the ticks' change bits
 struct alignas(16) TickBlock { u32 before, send, recv, pad; };
@@ -36,7 +44,9 @@ struct TickArgs {
   TickBlock* blk;                                  // [n_tiles * RT_TILE / 32]
   uint2* tile;                                     // [n_tiles] changes inside the tile, or before it once scanned
   RankTicks* ranks;                                // [n_ranks]
-  u32 vec, scanned;                                // send and recv may be read 16 bytes at a time; k_tile_scan ran
+  u32* far;                                        // [CTAs of ranks] 1: one of the CTA's ranks covers more than RT_NEAR tiles
+  u32* scanned;                                    // 1: k_tile_scan made prefixes of the tiles' sums; null: it does not run
+  u32 vec;                                         // send and recv may be read 16 bytes at a time
 };
 
 // the eight counters from tick i on (past the end: the last one there is, so that nothing changes)
@@ -62,14 +72,19 @@ __global__ void __launch_bounds__(RT_THREADS) k_tick_blocks(TickArgs A) {
   __shared__ u32 s_cnt[RT_THREADS / 32];
   if (blockIdx.x >= A.n_tiles) {
     const u64 r = (u64)(blockIdx.x - A.n_tiles) * RT_THREADS + threadIdx.x;
-    if (r >= A.n_ranks) return;
-    const u64 lo = min(A.tick_off[r], A.n_ticks), hi = min(A.tick_off[r + 1], A.n_ticks);      // (every rank is looked at, also one without records)
-    RankTicks x; x.t0 = 0; x.t1 = 0; x.lo = (u32)lo; x.n = hi > lo ? (u32)(hi - lo) : 0u; x.scale = 0.f; x.pad = 0;
-    if (x.n) {
-      x.t0 = A.tick_ns[lo]; x.t1 = A.tick_ns[hi - 1];
-      if (x.t1 > x.t0) x.scale = (float)(x.n - 1) / (float)(x.t1 - x.t0);
+    bool far = false;
+    if (r < A.n_ranks) {
+      const u64 lo = min(A.tick_off[r], A.n_ticks), hi = min(A.tick_off[r + 1], A.n_ticks);      // (every rank is looked at, also one without records)
+      RankTicks x; x.t0 = 0; x.t1 = 0; x.lo = (u32)lo; x.n = hi > lo ? (u32)(hi - lo) : 0u; x.scale = 0.f; x.pad = 0;
+      if (x.n) {
+        x.t0 = A.tick_ns[lo]; x.t1 = A.tick_ns[hi - 1];
+        if (x.t1 > x.t0) x.scale = (float)(x.n - 1) / (float)(x.t1 - x.t0);
+        far = (hi - 1) / RT_TILE - lo / RT_TILE > RT_NEAR;
+      }
+      A.ranks[r] = x;
     }
-    A.ranks[r] = x;
+    far = __syncthreads_or(far);
+    if (threadIdx.x == 0) A.far[blockIdx.x - A.n_tiles] = far;
     return;
   }
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -105,9 +120,14 @@ __global__ void __launch_bounds__(RT_THREADS) k_tick_blocks(TickArgs A) {
 // to step; the warps' totals are scanned by every warp.
 constexpr int TS_THREADS = 1024;
 constexpr int TS_PER = 16;
-__global__ void __launch_bounds__(TS_THREADS) k_tile_scan(uint2* tile, u32 n_tiles) {
+__global__ void __launch_bounds__(TS_THREADS) k_tile_scan(uint2* tile, u32 n_tiles, const u32* far, u32 n_far, u32* scanned) {
   begin_after();
   __shared__ u64 s_warp[TS_THREADS / 32];
+  bool any = far == nullptr;                          // null: the host knows that the scan pays
+  for (u32 k = threadIdx.x; k < n_far && !any; k += TS_THREADS) any = far[k] != 0;
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) *scanned = any;
+  if (!any) return;
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const auto pack = [](uint2 x) { return (u64)x.x | ((u64)x.y << 32); };          // fewer than 2^32 ticks: no carry into the upper half
   u64 carry = 0;
@@ -204,7 +224,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_record_rates(TickArgs A, u64 n_r
     s = (pb & 0xFFFFu) - (pa & 0xFFFFu); q = (pb >> 16) - (pa >> 16);
     const u32 ta = ia / RT_TILE, tb = ib / RT_TILE;
     if (ta != tb) {
-      if (A.scanned) { const uint2 x = A.tile[ta], y = A.tile[tb]; s += y.x - x.x; q += y.y - x.y; }
+      if (A.scanned != nullptr && *A.scanned != 0) { const uint2 x = A.tile[ta], y = A.tile[tb]; s += y.x - x.x; q += y.y - x.y; }
       else for (u32 k = ta; k < tb; ++k) { const uint2 x = A.tile[k]; s += x.x; q += x.y; }
     }
   }

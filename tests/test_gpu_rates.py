@@ -143,3 +143,55 @@ def test_offsets_beyond_the_samples():
         s, r = ccld.Analyzer().derive_rates(t(rank[keep], np.int32), t(te[keep], np.int64), t(tx[keep], np.int64), t(o, np.int64), t(tn, np.int64), t(sc, np.int32), t(rc, np.int32))
         torch.cuda.synchronize()
         assert np.array_equal(s.cpu().numpy().view(np.uint32), es[keep]) and np.array_equal(r.cpu().numpy().view(np.uint32), er[keep])
+
+
+def _lopsided(rng, n_ranks, ticks, n_rec):
+    """One rank with `ticks` samples among `n_ranks` with none or a few, ops of every length and in flight, a last warp that is not full."""
+    sizes = rng.integers(0, 4, n_ranks)
+    sizes[7] = ticks
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    tn = np.concatenate([np.arange(k) * MS for k in sizes])
+    rank = np.where(rng.random(n_rec) < 0.9, 7, rng.integers(0, n_ranks, n_rec))
+    te = rng.integers(0, ticks, n_rec) * MS
+    tx = te + (np.exp(rng.uniform(0, np.log(ticks), n_rec)) * MS).astype(np.int64)
+    tx[rng.random(n_rec) < 0.2] = -1
+    return rank, te, tx, off, tn, np.cumsum(rng.integers(0, 2, len(tn))), np.cumsum(rng.random(len(tn)) < 0.3)
+
+
+@pytest.mark.parametrize("tiles", [9, 10, 127, 128, 129, 600])
+def test_one_rank_holds_most_samples(tiles):
+    """Ops that span up to all tiles of a segment although the ranks' average is below one: tile counts around what a thread adds
+    up alone and what a warp reads at a time."""
+    rng = np.random.default_rng(tiles)
+    es, _ = _check(ccld.Analyzer(), *_lopsided(rng, 4096, tiles * 2048 - 5, 1000 + tiles))
+    assert es.max() > tiles * 512
+
+
+def test_one_rank_holds_most_samples_time():
+    """The same samples in a table of one rank and in one of 4,096 of which the others have none: what the ranks' shares are
+    decides how prefixes are made, not what comes out, and not by much how long it takes."""
+    rng = np.random.default_rng(1)
+    ticks, n_rec = 20_000 * 2048, 50_000
+    g = torch.Generator("cuda").manual_seed(1)
+    tn = torch.arange(ticks, device="cuda") * MS
+    sc, rc = (torch.cumsum((torch.rand(ticks, generator=g, device="cuda") < p).int(), 0, dtype=torch.int32) for p in (0.5, 0.3))
+    te = torch.randint(0, ticks, (n_rec,), generator=g, device="cuda") * MS
+    tx = torch.where(torch.rand(n_rec, generator=g, device="cuda") < 0.3, -1, te + 5 * MS)
+    rank = torch.zeros(n_rec, dtype=torch.int32, device="cuda")
+    an, got, best = ccld.Analyzer(), [], []
+    for n_ranks in (1, 4096):
+        off = torch.full((n_ranks + 1,), ticks, device="cuda")
+        off[0] = 0
+        us = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            out = an.derive_rates(rank, te, tx, off, tn, sc, rc)
+            b.record()
+            b.synchronize()
+            us.append(a.elapsed_time(b) * 1e3)
+        got.append(out)
+        best.append(min(us))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    assert best[1] < 2 * best[0], best
+    print("one rank %.0f us, among 4,096 %.0f us" % tuple(best))
