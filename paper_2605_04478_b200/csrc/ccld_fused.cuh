@@ -408,11 +408,11 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
 #pragma unroll
   for (int q = 7; q >= 0; --q) { pmax = d[q] == tmx ? (u32)q : pmax; pmin = d[q] == tmn ? (u32)q : pmin; pchg = ch[q] == cmx ? (u32)q : pchg; }
   const u32 r_tmin = __shfl_sync(FULLM, mem_l, pmin), r_tmax = __shfl_sync(FULLM, mem_l, pmax), r_chg = __shfl_sync(FULLM, mem_l, pchg);
-  // bytes * num / den: for eight members the factors 14/8 and 7/8 are exact
-  double fac = 1.0;
-  if (FULL) fac = gop == CCLD_OP_ALLREDUCE ? 1.75 : ((gop == CCLD_OP_ALLGATHER || gop == CCLD_OP_REDUCESCATTER || gop == CCLD_OP_ALLTOALL) ? 0.875 : 1.0);
-  else { double num, den; bus_factor(gop, n, &num, &den); fac = num / den; }
-  const double bn = (double)gby * fac;
+  // bytes * num / den: for eight members the factors 14/8 and 7/8 are exact; for others one rounding, and the row's value, which
+  // is a single quotient, is taken from the product before it
+  double bn, bnum = 0.0, den = 1.0;
+  if (FULL) bn = (double)gby * (gop == CCLD_OP_ALLREDUCE ? 1.75 : ((gop == CCLD_OP_ALLGATHER || gop == CCLD_OP_REDUCESCATTER || gop == CCLD_OP_ALLTOALL) ? 0.875 : 1.0));
+  else { double num; bus_factor(gop, n, &num, &den); bnum = (double)gby * num; bn = bnum / den; }
   if (gok) {
     const u64 g = group0 + seq_off + lane, G = ld_volatile(sh.out.G);
     i64* __restrict__ gi = ld_volatile(sh.out.gi64) + g; u32* __restrict__ gu = ld_volatile(sh.out.gu32) + g;
@@ -425,7 +425,7 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
     gu[(u64)GU_MAX_CHG * G] = cmx; gu[(u64)GU_RANK_MAX_CHG * G] = r_chg;
     gu[(u64)GU_N_PRESENT * G] = n;
     gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mm ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
-    ld_volatile(sh.out.gbw)[g] = span ? bn * rcp_newton((double)span) : 0.0;
+    ld_volatile(sh.out.gbw)[g] = !span ? 0.0 : (FULL ? bn * rcp_newton((double)span) : bnum * rcp_newton((double)span * den));
   }
   // ---- per-member bandwidth, summed over the warp; the Eq. 2 candidate; counts ----
   double bw[8];
@@ -610,7 +610,7 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
 #pragma unroll
     for (int h = 1; h < L; h <<= 1) { pmax = min(pmax, __shfl_xor_sync(FULLM, pmax, h)); pmin = min(pmin, __shfl_xor_sync(FULLM, pmin, h)); }
     double num, den; bus_factor(gop, n, &num, &den);
-    const double bd = (double)gby * (num / den);
+    const double bnum = (double)gby * num, bd = bnum / den;   // (a full group's den is a power of two: exact)
     if (lead && active) {
       sh.t_bd[jt] = round ? bd : 0.0;
       if (gok) {
@@ -624,7 +624,7 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
         gu[(u64)GU_RANK_TMIN * G] = sh.mem[pmin]; gu[(u64)GU_RANK_TMAX * G] = sh.mem[pmax];
         gu[(u64)GU_N_PRESENT * G] = n;
         gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mm ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
-        ld_volatile(sh.out.gbw)[g] = span ? bd * rcp_newton((double)span) : 0.0;
+        ld_volatile(sh.out.gbw)[g] = !span ? 0.0 : (FULL ? bd * rcp_newton((double)span) : bnum * rcp_newton((double)span * den));
       } else {
         const u32 e = atomicAdd(DL.count, 1u);
         DL.entries[e] = ((u64)t.w << 32) | (u64)(t.row.group0 + t.seq_off + jt);

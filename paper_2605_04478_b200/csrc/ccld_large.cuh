@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
       const bool clean = j < t.count && !(x.bits & 1), round = clean && !(gop == CCLD_OP_ALLREDUCE && gby < P.barrier_bytes);
       double num, den; bus_factor(gop, n, &num, &den);
       sh.state[j] = (clean ? 1u : 0u) | (round ? 2u : 0u); sh.rng[j] = (u32)(x.kmax >> 32) - (u32)(~x.n_kmin >> 32);
-      sh.bd[j] = round ? (double)gby * (num / den) : 0.0;
+      sh.bd[j] = round ? (double)gby * num / den : 0.0;
       if (j == me) {
         sh.group = x;
         if (clean) { sh.ranks[0] = __ldg(mem + (u32)~x.n_kmin); sh.ranks[1] = __ldg(mem + (NONE - (u32)x.kmax)); sh.ranks[2] = __ldg(mem + (NONE - (u32)x.ck)); }

@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(cons
           gu[(u64)GU_MAX_CHG * G] = (u32)(x.ck >> 32); gu[(u64)GU_RANK_MAX_CHG * G] = mem[NONE - (u32)x.ck];
           gu[(u64)GU_N_PRESENT * G] = n;
           gu[(u64)GU_GFLAGS * G] = CCLD_G_COMPLETE | (barrier ? CCLD_G_BARRIER : 0) | (mismatch ? CCLD_G_OPSET_MISMATCH : 0) | (analysed ? CCLD_G_ANALYSED : 0);
-          *gb = span ? bnum * rcp_newton((double)span * den) : 0.0;
+          *gb = busbw(bnum, den, (i64)span);
           atomicAdd(&s_cnt[SC_COMP], 1u);
           if (barrier) atomicAdd(&s_cnt[SC_BAR], 1u);
           if (analysed) atomicAdd(&s_cnt[SC_AN], 1u);

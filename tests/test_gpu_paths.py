@@ -389,3 +389,21 @@ def test_results_may_be_dropped_while_a_graph_is_captured():
     g.replay()
     torch.cuda.synchronize()
     assert x.tolist() == [2] * 8
+
+
+@pytest.mark.parametrize("n", [3, 6, 7, 11, 172, 500, 1024])
+def test_bus_bandwidth_of_an_op_is_rounded_once_or_twice(n):
+    """bytes * num and span * den are whole numbers that fp64 holds: above 128 members their quotient is rounded once (2^-53), up
+    to 128 it is a product with a reciprocal, both rounded (2^-52, and 2^-56 for the reciprocal's last step)."""
+    rng = np.random.default_rng(n)
+    d = np.exp(rng.normal(np.log(2e6), 1.0, (200, n))).astype(np.int64) + 1
+    reg, cols, _ = job([n], 200, rng, dur=lambda c, n: d, spacing=1_000_000_000)
+    by = np.exp(rng.normal(np.log(32 * MiB), 1.0, 200)).astype(np.uint64)
+    cols["bytes"] = by[cols["seq"]]
+    an = make_pair(reg)[0]
+    an.trace_upload(0, cols)
+    an.analyze_window(0, 1, 10**15)
+    t = an.get_optable(0)
+    want = by.astype(np.longdouble) * (2 * (n - 1)) / (t["span"].astype(np.longdouble) * n)
+    off = float(np.abs((t["busbw"].astype(np.longdouble) - want) / want).max())
+    assert off <= (2.0 ** -53 if n > 128 else 2.0 ** -52 + 2.0 ** -56) * (1 + 1e-3), off
