@@ -63,7 +63,7 @@ class BlockStore {
     std::lock_guard<std::mutex> g(m_);
     const size_t most = device < 0 ? PINNED_MOST : DEVICE_MOST;
     if (held_[device] + b.bytes > most) { free_block(device, b); return; }
-    held_[device] += b.bytes; lists_[device].push_back(b);
+    try { lists_[device].push_back(b); held_[device] += b.bytes; } catch (...) { free_block(device, b); }
   }
   void clear() { std::lock_guard<std::mutex> g(m_); drain(); }
   // Pinned blocks that callers keep (ccld_host_block): at most LENT_MOST bytes at a time.
@@ -189,6 +189,12 @@ int fail(ccld_ctx* c, int code, const std::string& msg) { if (c) c->err = msg; r
   do { cudaError_t e_ = (call);                                                                    \
        if (e_ != cudaSuccess) return fail(ctx, e_ == cudaErrorMemoryAllocation ? CCLD_ERR_NOMEM : CCLD_ERR_CUDA, \
                                           std::string(#call) + ": " + cudaGetErrorString(e_)); } while (0)
+
+// Host memory that runs out inside an entry point is a return code: nothing is thrown through the C boundary.
+int caught(ccld_ctx* ctx) {
+  try { return fail(ctx, CCLD_ERR_NOMEM, "out of host memory"); } catch (...) { return CCLD_ERR_NOMEM; }
+}
+#define CAUGHT catch (...) { return caught(ctx); }
 
 // Adds the elapsed times of a slot's finished event pairs to the sums (waits for the last one).
 void timer_harvest(ccld_ctx* ctx, TimerSlot& s) {
@@ -729,7 +735,7 @@ int ccld_destroy(ccld_ctx* ctx) {
 
 const char* ccld_last_error(ccld_ctx* ctx) { return ctx ? ctx->err.c_str() : "null context"; }
 
-int ccld_comm_register(ccld_ctx* ctx, uint32_t comm, const uint32_t* ranks, uint32_t n, uint8_t algo, uint32_t seq0) {
+int ccld_comm_register(ccld_ctx* ctx, uint32_t comm, const uint32_t* ranks, uint32_t n, uint8_t algo, uint32_t seq0) try {
   if (!ctx) return CCLD_ERR_ARG;
   if (ctx->finalized) return fail(ctx, CCLD_ERR_STATE, "communicators must be registered before the first analysis");
   if (!ranks || n == 0) return fail(ctx, CCLD_ERR_ARG, "empty communicator");
@@ -740,12 +746,12 @@ int ccld_comm_register(ccld_ctx* ctx, uint32_t comm, const uint32_t* ranks, uint
   std::vector<u32> sorted(c.ranks); std::sort(sorted.begin(), sorted.end());
   if (std::adjacent_find(sorted.begin(), sorted.end()) != sorted.end()) return fail(ctx, CCLD_ERR_ARG, "rank listed twice in a communicator");
   if (sorted.back() >= CCLD_MAX_RANK_ID) return fail(ctx, CCLD_ERR_CAPACITY, "rank id not below CCLD_MAX_RANK_ID");
-  ctx->comm_idx[comm] = (u32)ctx->comms.size();
-  ctx->comms.push_back(std::move(c));
+  const auto at = ctx->comm_idx.emplace(comm, (u32)ctx->comms.size()).first;
+  try { ctx->comms.push_back(std::move(c)); } catch (...) { ctx->comm_idx.erase(at); throw; }
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_comm_set_layers(ccld_ctx* ctx, uint32_t comm, const uint32_t* layer) {
+int ccld_comm_set_layers(ccld_ctx* ctx, uint32_t comm, const uint32_t* layer) try {
   if (!ctx) return CCLD_ERR_ARG;
   if (ctx->finalized) return fail(ctx, CCLD_ERR_STATE, "layers must be set before the first analysis");
   if (!layer) return fail(ctx, CCLD_ERR_ARG, "layer is null");
@@ -758,14 +764,14 @@ int ccld_comm_set_layers(ccld_ctx* ctx, uint32_t comm, const uint32_t* layer) {
   c.head.resize(n);
   for (u32 p = 0; p < n; ++p) c.head[p] = first.emplace(layer[p], p).first->second;
   return CCLD_OK;
-}
+} CAUGHT
 
 int ccld_trace_upload(ccld_ctx* ctx, uint32_t window_id, uint64_t n_rec, int mem_kind,
                       const uint32_t* rank, const uint32_t* comm, const uint32_t* seq, const uint8_t* op,
                       const uint64_t* bytes, const int64_t* t_enter_ns, const int64_t* t_exit_ns,
                       const uint32_t* send_chg, const uint32_t* recv_chg,
                       uint32_t n_frames, const uint32_t* f_rank, const uint32_t* f_comm, const uint32_t* f_seq,
-                      uint32_t n_channels, const uint32_t* progress) {
+                      uint32_t n_channels, const uint32_t* progress) try {
   NvtxRange nvtx_range("ccld_trace_upload");
   if (!ctx) return CCLD_ERR_ARG;
   if (mem_kind != 0 && mem_kind != 1) return fail(ctx, CCLD_ERR_ARG, "mem_kind must be 0 (host) or 1 (device)");
@@ -798,7 +804,7 @@ int ccld_trace_upload(ccld_ctx* ctx, uint32_t window_id, uint64_t n_rec, int mem
                          {o_te, t_enter_ns, n_rec * 8}, {o_tx, t_exit_ns, n_rec * 8}, {o_sc, send_chg, chg}, {o_rc, recv_chg, chg},
                          {o_fr, f_rank, fr}, {o_fc, f_comm, fr}, {o_fs, f_seq, fr}, {o_pr, progress, (size_t)n_frames * n_channels * 8}};
     static_assert(sizeof col / sizeof col[0] == UP_COLS, "all of them");
-    { int rc = upload_columns(ctx, b, off, col, sizeof col / sizeof col[0]); if (rc != CCLD_OK) { cudaStreamSynchronize(ctx->stream); ctx->pool.put(w.own); return rc; } }
+    { int rc; try { rc = upload_columns(ctx, b, off, col, sizeof col / sizeof col[0]); } catch (...) { rc = caught(ctx); } if (rc != CCLD_OK) { cudaStreamSynchronize(ctx->stream); ctx->pool.put(w.own); return rc; } }
     d.rank = (const u32*)(b + o_rank); d.comm = (const u32*)(b + o_comm); d.seq = (const u32*)(b + o_seq); d.op = (const u8*)(b + o_op);
     d.bytes = (const u64*)(b + o_bytes); d.t_enter = (const i64*)(b + o_te); d.t_exit = (const i64*)(b + o_tx);
     d.send_chg = send_chg ? (const u32*)(b + o_sc) : nullptr; d.recv_chg = recv_chg ? (const u32*)(b + o_rc) : nullptr;
@@ -806,9 +812,9 @@ int ccld_trace_upload(ccld_ctx* ctx, uint32_t window_id, uint64_t n_rec, int mem
   }
   ctx->windows.emplace(window_id, std::move(w));
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_window_release(ccld_ctx* ctx, uint32_t window_id) {
+int ccld_window_release(ccld_ctx* ctx, uint32_t window_id) try {
   if (!ctx) return CCLD_ERR_ARG;
   { int rc = settle(ctx); if (rc != CCLD_OK) return rc; }
   auto it = ctx->windows.find(window_id);
@@ -820,9 +826,9 @@ int ccld_window_release(ccld_ctx* ctx, uint32_t window_id) {
   if (it->second.owns_opset) ctx->pool.put(it->second.opset_own);
   ctx->windows.erase(it);
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_reset(ccld_ctx* ctx) {
+int ccld_reset(ccld_ctx* ctx) try {
   if (!ctx) return CCLD_ERR_ARG;
   CK(cudaSetDevice(ctx->device));
   CK(cudaStreamSynchronize(ctx->stream));
@@ -835,22 +841,22 @@ int ccld_reset(ccld_ctx* ctx) {
     CK(cudaMemsetAsync(ctx->d_poison, 0, 4, ctx->stream));
   }
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_analyze_window(ccld_ctx* ctx, uint32_t first_window, uint32_t n_windows, int64_t now_ns) {
+int ccld_analyze_window(ccld_ctx* ctx, uint32_t first_window, uint32_t n_windows, int64_t now_ns) try {
   NvtxRange nvtx_range("ccld_analyze_window");
   if (!ctx) return CCLD_ERR_ARG;
   if (n_windows == 0) return fail(ctx, CCLD_ERR_ARG, "n_windows is zero");
   if (n_windows > 65535) return fail(ctx, CCLD_ERR_CAPACITY, "more than 65,535 windows in one batch");
   return analyze_batch(ctx, first_window, n_windows, now_ns, ctx->speculate != 0);
-}
+} CAUGHT
 
-int ccld_set_speculation(ccld_ctx* ctx, int on) {
+int ccld_set_speculation(ccld_ctx* ctx, int on) try {
   if (!ctx) return CCLD_ERR_ARG;
   { int rc = settle(ctx); if (rc != CCLD_OK) return rc; }
   ctx->speculate = on != 0;
   return CCLD_OK;
-}
+} CAUGHT
 
 }  // extern "C"
 
@@ -1173,17 +1179,17 @@ static int verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out, ccld_ve
   return CCLD_OK;
 }
 
-int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) {
+int ccld_get_verdict(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out) try {
   NvtxRange nvtx_range("ccld_get_verdict");
   if (!ctx || !out) return CCLD_ERR_ARG;
   return verdict(ctx, window_id, out, nullptr);
-}
+} CAUGHT
 
-int ccld_get_verdict_columns(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out, ccld_verdict_columns* columns) {
+int ccld_get_verdict_columns(ccld_ctx* ctx, uint32_t window_id, ccld_verdict* out, ccld_verdict_columns* columns) try {
   NvtxRange nvtx_range("ccld_get_verdict_columns");
   if (!ctx || !out || !columns) return CCLD_ERR_ARG;
   return verdict(ctx, window_id, out, columns);
-}
+} CAUGHT
 
 // Launches the hang kernel over one op or over the window's alerts (A.alerts set) and waits; results are in pinned memory.
 static int hang_run(ccld_ctx* ctx, const WindowHost* w, HangArgs& A, u32 ctas) {
@@ -1204,7 +1210,7 @@ static int hang_run(ccld_ctx* ctx, const WindowHost* w, HangArgs& A, u32 ctas) {
   return e == cudaSuccess ? CCLD_OK : fail(ctx, CCLD_ERR_CUDA, std::string("hang location: ") + cudaGetErrorString(e));
 }
 
-int ccld_locate_hang(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t seq, ccld_hang_verdict* out) {
+int ccld_locate_hang(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t seq, ccld_hang_verdict* out) try {
   NvtxRange nvtx_range("ccld_locate_hang");
   if (!ctx || !out) return CCLD_ERR_ARG;
   WindowHost* w;
@@ -1225,10 +1231,10 @@ int ccld_locate_hang(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t 
   const u32 n_copy = std::min(out->n_roots_total, keep);
   if (n_copy) std::memcpy(roots, h + o_roots, n_copy * 4ull);
   return CCLD_OK;
-}
+} CAUGHT
 
 int ccld_locate_hangs(ccld_ctx* ctx, uint32_t window_id, ccld_hang_alert* alerts, ccld_hang_verdict* out, uint32_t cap,
-                      uint32_t* roots, uint32_t roots_stride, uint32_t* n_total) {
+                      uint32_t* roots, uint32_t roots_stride, uint32_t* n_total) try {
   NvtxRange nvtx_range("ccld_locate_hangs");
   if (!ctx || !n_total) return CCLD_ERR_ARG;
   if (cap && !out) return fail(ctx, CCLD_ERR_ARG, "out is null");
@@ -1269,9 +1275,9 @@ int ccld_locate_hangs(ccld_ctx* ctx, uint32_t window_id, ccld_hang_alert* alerts
   }
   if (alerts && n) std::memcpy(alerts, h + o_al, n * sizeof(ccld_hang_alert));
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_get_optable(ccld_ctx* ctx, uint32_t window_id, ccld_optable* out) {
+int ccld_get_optable(ccld_ctx* ctx, uint32_t window_id, ccld_optable* out) try {
   if (!ctx || !out) return CCLD_ERR_ARG;
   WindowHost* w;
   { int rc = find_analysed(ctx, window_id, &w); if (rc != CCLD_OK) return rc; }
@@ -1285,9 +1291,9 @@ int ccld_get_optable(ccld_ctx* ctx, uint32_t window_id, ccld_optable* out) {
   out->rank_max_chg = gu + GU_RANK_MAX_CHG * G; out->n_present = gu + GU_N_PRESENT * G; out->gflags = gu + GU_GFLAGS * G;
   out->busbw = d.gbw; out->flags = d.flags; out->perm = d.perm;
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_get_ranges(ccld_ctx* ctx, uint32_t window_id, ccld_comm_range* rows, uint32_t cap, uint32_t* n_total) {
+int ccld_get_ranges(ccld_ctx* ctx, uint32_t window_id, ccld_comm_range* rows, uint32_t cap, uint32_t* n_total) try {
   if (!ctx || !n_total) return CCLD_ERR_ARG;
   WindowHost* w;
   { int rc = find_analysed(ctx, window_id, &w); if (rc != CCLD_OK) return rc; }
@@ -1304,7 +1310,7 @@ int ccld_get_ranges(ccld_ctx* ctx, uint32_t window_id, ccld_comm_range* rows, ui
   }
   *n_total = k;
   return CCLD_OK;
-}
+} CAUGHT
 
 void ccld_host_release(ccld_host_block* blk) {
   if (!blk || !blk->p) return;
@@ -1313,7 +1319,7 @@ void ccld_host_release(ccld_host_block* blk) {
   blk->p = nullptr; blk->bytes = 0;
 }
 
-int ccld_take_optable(ccld_ctx* ctx, uint32_t window_id, ccld_host_optable* out) {
+int ccld_take_optable(ccld_ctx* ctx, uint32_t window_id, ccld_host_optable* out) try {
   NvtxRange nvtx_range("ccld_take_optable");
   if (!ctx || !out) return CCLD_ERR_ARG;
   std::memset(out, 0, sizeof *out);
@@ -1343,9 +1349,9 @@ int ccld_take_optable(ccld_ctx* ctx, uint32_t window_id, ccld_host_optable* out)
   t.busbw = (const double*)(base + at[2]); t.flags = (const u8*)(base + at[3]); t.perm = (const u32*)(base + at[4]);
   out->comm = comm; out->seq = seq; out->slot0 = slot0;
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_take_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, ccld_host_rank_stats* out) {
+int ccld_take_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, ccld_host_rank_stats* out) try {
   if (!ctx || !out) return CCLD_ERR_ARG;
   std::memset(out, 0, sizeof *out);
   if (!ctx->finalized) return fail(ctx, CCLD_ERR_STATE, "nothing analysed yet");
@@ -1361,9 +1367,9 @@ int ccld_take_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, ccld_host_rank_stats* 
   if (e != cudaSuccess) { cudaStreamSynchronize(ctx->stream); ccld_host_release(&out->block); return fail(ctx, CCLD_ERR_CUDA, std::string("statistics copy: ") + cudaGetErrorString(e)); }
   out->votes = (const u32*)(base + at[0]); out->ops = (const u32*)(base + at[1]); out->bw_cnt = (const u32*)(base + at[2]); out->bw_sum = (const double*)(base + at[3]);
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_get_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, uint32_t* votes, uint32_t* ops, uint32_t* bw_cnt, double* bw_sum) {
+int ccld_get_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, uint32_t* votes, uint32_t* ops, uint32_t* bw_cnt, double* bw_sum) try {
   if (!ctx || !votes || !ops || !bw_cnt || !bw_sum) return CCLD_ERR_ARG;
   if (!ctx->finalized) return fail(ctx, CCLD_ERR_STATE, "nothing analysed yet");
   { int rc = settle(ctx); if (rc != CCLD_OK) return rc; }
@@ -1372,9 +1378,9 @@ int ccld_get_rank_stats(ccld_ctx* ctx, uint32_t n_ranks, uint32_t* votes, uint32
   std::memset(votes + n * 4, 0, rest * 16); std::memset(ops + n, 0, rest * 4); std::memset(bw_cnt + n, 0, rest * 4); std::memset(bw_sum + n, 0, rest * 8);
   const Piece pc[4] = {{ctx->reg.votes, votes, n * 16}, {ctx->reg.ops, ops, n * 4}, {ctx->reg.bw_cnt, bw_cnt, n * 4}, {ctx->reg.bw_sum, bw_sum, n * 8}};
   return fetch(ctx, pc, 4);
-}
+} CAUGHT
 
-int ccld_trace_attach_opset(ccld_ctx* ctx, uint32_t window_id, int mem_kind, const uint8_t* algo, const uint8_t* proto) {
+int ccld_trace_attach_opset(ccld_ctx* ctx, uint32_t window_id, int mem_kind, const uint8_t* algo, const uint8_t* proto) try {
   if (!ctx) return CCLD_ERR_ARG;
   if (mem_kind != 0 && mem_kind != 1) return fail(ctx, CCLD_ERR_ARG, "mem_kind must be 0 (host) or 1 (device)");
   auto it = ctx->windows.find(window_id);
@@ -1395,9 +1401,9 @@ int ccld_trace_attach_opset(ccld_ctx* ctx, uint32_t window_id, int mem_kind, con
   CK(cudaStreamSynchronize(ctx->stream));       // the caller's host arrays are free again
   w.algo = (const u8*)b; w.proto = (const u8*)(b + half);
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_opset_check(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t seq, ccld_opset_verdict* out) {
+int ccld_opset_check(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t seq, ccld_opset_verdict* out) try {
   if (!ctx || !out) return CCLD_ERR_ARG;
   WindowHost* w;
   { int rc = find_analysed(ctx, window_id, &w); if (rc != CCLD_OK) return rc; }
@@ -1418,14 +1424,14 @@ int ccld_opset_check(ccld_ctx* ctx, uint32_t window_id, uint32_t comm, uint32_t 
   const u32 n_copy = std::min(out->n_deviating_total, keep);
   if (n_copy) std::memcpy(ranks, h + o_rk, n_copy * 4ull);
   return CCLD_OK;
-}
+} CAUGHT
 
 namespace {
 struct StateHeader { u64 magic; u32 version, n_comms, n_ranks, pad; u64 stats_bytes; };
 constexpr u64 STATE_MAGIC = 0x3130545344434343ull;    // "CCCDST01"
 }  // namespace
 
-int ccld_state_export(ccld_ctx* ctx, void* buf, uint64_t cap, uint64_t* n_bytes) {
+int ccld_state_export(ccld_ctx* ctx, void* buf, uint64_t cap, uint64_t* n_bytes) try {
   if (!ctx || !n_bytes) return CCLD_ERR_ARG;
   CK(cudaSetDevice(ctx->device));
   { int rc = finalize_registry(ctx); if (rc != CCLD_OK) return rc; }
@@ -1441,9 +1447,9 @@ int ccld_state_export(ccld_ctx* ctx, void* buf, uint64_t cap, uint64_t* n_bytes)
   CK(cudaMemcpyAsync(p, (char*)ctx->reg_blk.p + ctx->stats_off, ctx->stats_bytes, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_state_import(ccld_ctx* ctx, const void* buf, uint64_t n_bytes) {
+int ccld_state_import(ccld_ctx* ctx, const void* buf, uint64_t n_bytes) try {
   if (!ctx || !buf) return CCLD_ERR_ARG;
   CK(cudaSetDevice(ctx->device));
   { int rc = finalize_registry(ctx); if (rc != CCLD_OK) return rc; }
@@ -1465,11 +1471,11 @@ int ccld_state_import(ccld_ctx* ctx, const void* buf, uint64_t n_bytes) {
   CK(cudaMemcpyAsync((char*)ctx->reg_blk.p + ctx->stats_off, p, ctx->stats_bytes, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   return CCLD_OK;
-}
+} CAUGHT
 
 int ccld_derive_rates(ccld_ctx* ctx, uint64_t n_rec, const uint32_t* rank, const int64_t* t_enter_ns, const int64_t* t_exit_ns,
                       uint32_t n_ranks, uint64_t n_ticks, const uint64_t* tick_off, const int64_t* tick_ns,
-                      const uint32_t* send_count, const uint32_t* recv_count, uint32_t* send_chg, uint32_t* recv_chg) {
+                      const uint32_t* send_count, const uint32_t* recv_count, uint32_t* send_chg, uint32_t* recv_chg) try {
   if (!ctx) return CCLD_ERR_ARG;
   if (n_rec && (!rank || !t_enter_ns || !t_exit_ns || !send_chg || !recv_chg)) return fail(ctx, CCLD_ERR_ARG, "null record column");
   if (n_ranks == 0 || !tick_off) return fail(ctx, CCLD_ERR_ARG, "tick_off is required (n_ranks + 1 entries)");
@@ -1500,9 +1506,9 @@ int ccld_derive_rates(ccld_ctx* ctx, uint64_t n_rec, const uint32_t* rank, const
   ctx->pool.put(blk);           // later work on this stream runs after these kernels: the block can be handed out again
   if (le != cudaSuccess) return fail(ctx, CCLD_ERR_CUDA, std::string("rate kernels: ") + cudaGetErrorString(le));
   return CCLD_OK;
-}
+} CAUGHT
 
-int ccld_timing_enable(ccld_ctx* ctx, int on) {
+int ccld_timing_enable(ccld_ctx* ctx, int on) try {
   if (!ctx) return CCLD_ERR_ARG;
   CK(cudaSetDevice(ctx->device));
   CK(cudaStreamSynchronize(ctx->stream));
@@ -1514,7 +1520,7 @@ int ccld_timing_enable(ccld_ctx* ctx, int on) {
   std::memset(ctx->t_ms, 0, sizeof ctx->t_ms); std::memset(ctx->t_launches, 0, sizeof ctx->t_launches);
   ctx->timing = on != 0;
   return CCLD_OK;
-}
+} CAUGHT
 
 int ccld_get_kernel_times(ccld_ctx* ctx, double* ms, uint64_t* launches) {
   if (!ctx || !ms || !launches) return CCLD_ERR_ARG;
@@ -1525,23 +1531,26 @@ int ccld_get_kernel_times(ccld_ctx* ctx, double* ms, uint64_t* launches) {
   return CCLD_OK;
 }
 
-int ccld_copy_many_to_host(ccld_ctx* ctx, uint32_t n, void* const* dst_host, const void* const* src_device, const uint64_t* bytes) {
+int ccld_copy_many_to_host(ccld_ctx* ctx, uint32_t n, void* const* dst_host, const void* const* src_device, const uint64_t* bytes) try {
   if (!ctx || (n && (!dst_host || !src_device || !bytes))) return CCLD_ERR_ARG;
-  std::vector<Piece> pc(n);
-  for (u32 i = 0; i < n; ++i) {
-    if (bytes[i] && (!dst_host[i] || !src_device[i])) return fail(ctx, CCLD_ERR_ARG, "null array");
-    pc[i] = Piece{src_device[i], dst_host[i], bytes[i]};
-  }
+  for (u32 i = 0; i < n; ++i) if (bytes[i] && (!dst_host[i] || !src_device[i])) return fail(ctx, CCLD_ERR_ARG, "null array");
   CK(cudaSetDevice(ctx->device));
-  return fetch(ctx, pc.data(), n);
-}
+  if (n <= GATHER_PIECES) {
+    Piece pc[GATHER_PIECES];
+    for (u32 i = 0; i < n; ++i) pc[i] = Piece{src_device[i], dst_host[i], bytes[i]};
+    return fetch(ctx, pc, n);
+  }
+  for (u32 i = 0; i < n; ++i) if (bytes[i]) CK(cudaMemcpyAsync(dst_host[i], src_device[i], bytes[i], cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  return CCLD_OK;
+} CAUGHT
 
-int ccld_copy_to_host(ccld_ctx* ctx, void* dst_host, const void* src_device, uint64_t bytes) {
+int ccld_copy_to_host(ccld_ctx* ctx, void* dst_host, const void* src_device, uint64_t bytes) try {
   if (!ctx || (bytes && (!dst_host || !src_device))) return CCLD_ERR_ARG;
   CK(cudaSetDevice(ctx->device));
   if (bytes) CK(cudaMemcpyAsync(dst_host, src_device, bytes, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   return CCLD_OK;
-}
+} CAUGHT
 
 }  // extern "C"

@@ -2,6 +2,9 @@
 identical, fp64 quantities within 1e-9 relative (tests/parity.py)."""
 import ctypes as C
 import gc
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -407,3 +410,29 @@ def test_bus_bandwidth_of_an_op_is_rounded_once_or_twice(n):
     want = by.astype(np.longdouble) * (2 * (n - 1)) / (t["span"].astype(np.longdouble) * n)
     off = float(np.abs((t["busbw"].astype(np.longdouble) - want) / want).max())
     assert off <= (2.0 ** -53 if n > 128 else 2.0 ** -52 + 2.0 ** -56) * (1 + 1e-3), off
+
+
+_LITTLE_MEMORY = """
+import resource, sys
+import numpy as np
+import paper_2605_04478_b200 as ccld
+an = ccld.Analyzer()
+an.comm_register(0, range(4))
+n = 60_000_000
+none = np.zeros(n, np.uint64)
+pages = int(open("/proc/self/statm").read().split()[0])
+resource.setrlimit(resource.RLIMIT_AS, (pages * 4096 + (256 << 20),) * 2)
+print("rc", an.lib.ccld_copy_many_to_host(an.h, n, none.ctypes.data, none.ctypes.data, none.ctypes.data))
+"""
+
+
+def test_copies_of_many_arrays():
+    """More arrays than one kernel takes; and so many (empty) ones that a list of them would not fit into memory."""
+    an = ccld.Analyzer()
+    for k in (1, 24, 25, 100):
+        src = [torch.randint(0, 255, (7 * i + 1,), dtype=torch.uint8, device="cuda") for i in range(k)]
+        out = an._to_host([(t.data_ptr(), t.numel(), np.uint8) for t in src])
+        for t, a in zip(src, out):
+            same(a, t.cpu().numpy(), "array")
+    r = subprocess.run([sys.executable, "-c", _LITTLE_MEMORY], capture_output=True, text=True, cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0 and r.stdout.strip() == "rc 0", (r.returncode, r.stdout, r.stderr[-500:])
