@@ -26,7 +26,7 @@ constexpr int SMALL_SEQS = 256;        //   threads per CTA: eight warps, each o
 #define CCLD_FUSED_WT_PER_CTA 16
 #endif
 constexpr u32 FUSED_WT_PER_CTA = CCLD_FUSED_WT_PER_CTA;   //   warp-tiles a CTA works through (a multiple of its eight warps)
-constexpr int WARP_N = 128;            // up to 128 ranks: one warp per group, bitonic sort in registers
+constexpr int WARP_N = 128;            // up to 128 ranks: a CTA per tile of op counters, n_pad / 8 lanes per group
 constexpr int MID_ELEMS = 2048;        //   padded records per tile of a communicator of 9 to 128 ranks
 constexpr int MID_N = 1024;            // up to 1024 ranks: a warp per group, keys in its registers
 constexpr int MID_THREADS = 256;
@@ -156,7 +156,6 @@ __host__ __device__ inline u32 tile_seqs(u32 n) {
 __host__ __device__ inline u32 ceil_div(u32 a, u32 b) { return (a + b - 1) / b; }
 // chunking of a fused-class communicator with n_seq op counters in a window of T chunks
 __host__ __device__ inline u32 chunk_len(u32 n_seq, u32 T) { return ceil_div(n_seq, T); }
-__host__ __device__ inline u32 chunk_count(u32 n_seq, u32 T) { return n_seq ? ceil_div(n_seq, chunk_len(n_seq, T)) : 0u; }
 __host__ __device__ inline u32 chunk_size(u32 n_seq, u32 T, u32 tau) {    // op counters in chunk tau (0 beyond the last)
   const u32 S = chunk_len(n_seq, T);
   return (u64)tau * S >= n_seq ? 0u : (n_seq - tau * S < S ? n_seq - tau * S : S);

@@ -1,16 +1,16 @@
 // Per-op reductions, median / MAD, flags and votes for communicators of up to 128 ranks (sm_100a).
 //
 //   k_reduce_fused     the common case: every member reported, nothing in flight, all times of the group within
-//                      2^31 ns of its first member's enter time. A group sits in L = n_pad / 8 lanes of a warp, eight
-//                      ring positions per lane (n <= 8: one thread per group, lanes along consecutive op counters so
-//                      that the gathers of one member coalesce). Times become 32-bit offsets as they arrive and are
-//                      parked in shared memory, so that a thread never holds more than one batch of gathers plus
-//                      one set of eight sort keys in registers: three CTAs of 256 threads fit an SM. Any other
-//                      group is appended to a list.
+//                      2^31 ns of its first member's enter time (or with equal upper words). n <= 8: one thread per group
+//                      with everything in its registers, lanes along consecutive op counters so that the gathers of one
+//                      member coalesce. Larger: a tile of op counters is gathered by the whole CTA, lanes along the op
+//                      counter, and parked in shared memory as 32-bit keys; then a group sits in L = n_pad / 8 lanes of a
+//                      warp, eight ring positions per lane. Three CTAs of 256 threads fit an SM. Any other group is
+//                      appended to a list.
 //   k_reduce_deferred  the listed groups, one warp each, in full 64-bit generality: missing members, records in
 //                      flight (hang alerts), invalid times, spreads beyond 32 bits.
 //
-// The work list of k_reduce_fused is chunk-major (see k_plan), so CTAs that run together gather from the same stretch
+// The work list of k_reduce_fused is chunk-major (see k_emit), so CTAs that run together gather from the same stretch
 // of every rank's records and share the fetched sectors in L2.
 #pragma once
 #include "ccld_device.cuh"
@@ -65,22 +65,18 @@ template <class K> __device__ __forceinline__ void median_mad8(const K (&x)[8], 
   *med = m; *mad = pick4(s, k);
 }
 
-// 1 / x for x >= 1 to within a few ulp: single-precision seed and two Newton steps
-// one Newton step on the single-precision seed: relative error near 2e-14
-__device__ __forceinline__ float rcp_seed(double x) {     // 1 <= x < 2^64: the approximate reciprocal is good to about 2^-22
-  float r; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)x)); return r;
-}
-__device__ __forceinline__ double rcp_newton1(double x) {
-  const double r = (double)rcp_seed(x);
-  return fma(r, fma(-x, r, 1.0), r);
-}
+// 1 / x, 1 <= x < 2^64, rounded: Newton's method on the approximate single-precision reciprocal. That is good to about 2^-22
+// with the rounding of its argument, and a step squares the relative error (always towards smaller values): two steps leave
+// the rounding of the last one.
 __device__ __forceinline__ double rcp_newton(double x) {
-  double r = (double)rcp_seed(x);
+  float s; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"((float)x));
+  double r = (double)s;
   double e = fma(-x, r, 1.0); r = fma(r, e, r);
   e = fma(-x, r, 1.0); r = fma(r, e, r);
   return r;
 }
-// the same from a whole number >= 1, whose single-precision form needs no detour over fp64
+// The same from a whole number >= 1, whose single-precision form needs no detour over fp64, with one step: at most 2^-44 (6e-14)
+// too small; the sums of members' bandwidths it serves are 0.7 to 1.6e-15 (rms) below extended precision's.
 __device__ __forceinline__ double rcp_u32(u32 x) {
   float s; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__uint2float_rn(x)));
   const double r = (double)s;
