@@ -28,7 +28,8 @@ constexpr int SMALL_SEQS = 256;        //   threads per CTA: eight warps, each o
 constexpr u32 FUSED_WT_PER_CTA = CCLD_FUSED_WT_PER_CTA;   //   warp-tiles a CTA works through (a multiple of its eight warps)
 constexpr int WARP_N = 128;            // up to 128 ranks: a CTA per tile of op counters, n_pad / 8 lanes per group
 constexpr int MID_ELEMS = 2048;        //   padded records per tile of a communicator of 9 to 128 ranks
-constexpr int MID_N = 1024;            // up to 1024 ranks: a warp per group, keys in its registers
+constexpr int MID_N = 1024;            // up to 1024 ranks: a warp per group, keys in its registers (as far as 32 per lane go; ns per op
+                                       //   counter against the cluster kernel's: 31 and 57 at 520 ranks, 40 and 62 at 768, 46 and 66 at 1,024)
 constexpr int MID_THREADS = 256;
 constexpr int MID_SEQS = 8;            //   op counters per tile
 constexpr int LARGE_SEQS = 8;          // above: a cluster of eight CTAs per tile of 8 consecutive op counters

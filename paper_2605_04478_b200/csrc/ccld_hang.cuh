@@ -5,7 +5,7 @@
 // number of dependent steps. Per-member state lives in shared memory (global scratch beyond HANG_SMEM_N members); a member
 // is looked up at the op itself first, and only one that did not report it is searched for at later counters, a warp along
 // its contiguous column of the slot table; the layers of a tree get their extremes by atomics on the layer's entry instead
-// of one thread walking the layer; verdicts and roots go straight to pinned memory. One ring of 1,024 (a tree): 52 -> 9 us.
+// of one thread walking the layer; verdicts and roots go straight to pinned memory. A tree of 1,024: 52 -> 12 us.
 #pragma once
 
 namespace ccld {

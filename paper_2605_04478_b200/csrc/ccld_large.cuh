@@ -148,6 +148,9 @@ template <int Q> __device__ __forceinline__ void large_pick(const u32* __restric
   *ra = lo0; *rd = lo1;
 }
 
+// CTAs per SM, in ns per op counter of one window of 4 M records, two against three: 2,049 to 4,096 members 138 against 129 (3,000)
+// and 169 against 166 (4,096), although three leave 40 registers and spill 120 bytes; above 4,096 two are what shared memory holds.
+// Up to 2,048 members it is two, where three would take 67 against 73 (1,100), 74 against 82 (1,500) and 90 against 95 (2,048).
 template <int Q>
 __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(const WinDesc* wd, const Tile* tiles,
     TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
@@ -187,7 +190,10 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
     i64 te0 = 0; u64 by0 = 0; u32 op0 = 0;
     if (i0 != NONE) { te0 = __ldg(c_te + i0); by0 = __ldg(c_by + i0); op0 = __ldg(c_op + i0); } else x.bits = 1;
     const u64 base = (u64)te0 - 0x80000000ull;
-    constexpr int STEP = Q == 16 ? 4 : 2;                   // records in flight per thread, as many as the registers allow
+    // Records in flight per thread. Four spill at 40 registers: 146 and 185 ns per op counter of 3,000 and 4,096 members against 129
+    // and 166. At 64 registers they make no difference above 4,096 (266 and 264 ns at 8,192) and little below 2,049 (70.5 against 73
+    // ns at 1,100, 92.5 against 95 at 2,048), where it is two.
+    constexpr int STEP = Q == 16 ? 4 : 2;
 #pragma unroll
     for (int q0 = 0; q0 < Q; q0 += STEP) {
       i64 ta[STEP], tb[STEP]; u64 by[STEP]; u32 op[STEP], ch[STEP];

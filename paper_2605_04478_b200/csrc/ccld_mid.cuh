@@ -131,6 +131,8 @@ struct MidTrack {
   }
 };
 
+// CTAs per SM, in ns per op counter of one window of 4 M records: up to 256 members two 7.9, three 6.1, four 5.8 (172 members; 9.0, 7.1, 6.9
+// at 256); of 257 to 512 two 18.3, three 15.0 (512); with 32 keys per lane two are what the registers allow. It is three, two, two.
 template <int R>
 __global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(const WinDesc* wd, const Tile* tiles,
     TileSum* __restrict__ sums, Registry R_, Params P, DeferList DL) {

@@ -16,7 +16,7 @@
 //
 // Measured on 4,096 ranks x 5,600 ticks and 4.1 M records (467 MB to move, 71 us at the measured copy rate): the version
 // before searched the rank of every warp's ticks, loaded 4 bytes per lane and ran two more kernels for a global prefix
-// (k_tick_blocks 61 us, prefix 21 us, k_record_rates 74 us with two dependent searches: 160 us); now 33 + 50 us, 85 us for the call.
+// (k_tick_blocks 61 us, prefix 21 us, k_record_rates 74 us with two dependent searches: 160 us); now 33 + 50 us, 82 us for the call.
 // No kernel waits on another CTA.
 #pragma once
 #include "ccld_device.cuh"
@@ -27,8 +27,8 @@ constexpr int RT_THREADS = 256;
 constexpr int RT_TILE = RT_THREADS * 8;            // ticks per CTA of k_tick_blocks, eight consecutive ones per lane
 // A record adds up the tiles its op spans. Ops of one rank hardly overlap, so that is a read or two per record while no rank's
 // samples cover more than this many tiles (8 tiles = 16 s at a sample per millisecond). With longer segments an op in flight
-// since their beginning would add up many, and the scan pays: 20,000 tiles of one rank among 4,096, 50,000 records: 1,067 -> 99 us. (4,096 equal ranks of 5,600 ticks,
-// whose scan is launched to find that out: 80.1 -> 81.5 us.)
+// since their beginning would add up many, and the scan pays: 20,000 tiles of one rank among 4,096, 50,000 records: 1,067 -> 99 us.
+// (4,096 equal ranks of 5,600 ticks, whose scan is launched to find out that there are none: 80.1 -> 81.5 us.)
 constexpr u32 RT_NEAR = 8;
 constexpr u64 RT_SCAN = 256;                       // up to so many tiles in all a record adds them up whatever the segments are
 
