@@ -43,11 +43,11 @@ CSRC = os.path.join(ROOT, "paper_2605_04478_b200", "csrc")
 # records, so a launch's traffic is this figure times its records. Each entry names the source files of its kernel and
 # their hash at capture time: once a file changes the figure is stale and the bench reports null.
 NCU_TRAFFIC = {
-    "k_reduce_fused": {"bytes_per_record": (798.90e6 + 249.83e6) / 20.48e6, "files": ("ccld_fused.cuh",),
-                       "sha16": "a34c2c53944622eb"},
+    "k_reduce_fused": {"bytes_per_record": (799.50e6 + 243.65e6) / 20.48e6, "files": ("ccld_fused.cuh",),
+                       "sha16": "9270572ed17d433e"},
     # capture on 5 cfg4w windows
-    "k_reduce_large": {"bytes_per_record": (770.54e6 + 81.91e6) / 20.48e6, "files": ("ccld_large.cuh",),
-                       "sha16": "fcb4a1ab46234123"},
+    "k_reduce_large": {"bytes_per_record": (770.69e6 + 77.84e6) / 20.48e6, "files": ("ccld_large.cuh",),
+                       "sha16": "e0be24900dc16ab9"},
 }
 
 MIXES = {"all": ((0, 0, 1, 0, 2), 200), "tp_pp": ((0, 0, 1, 0), 250), "dp": ((2,), 200)}   # op pattern (0 TP, 1 PP, 2 DP), repetitions
