@@ -1498,9 +1498,10 @@ int ccld_derive_rates(ccld_ctx* ctx, uint64_t n_rec, const uint32_t* rank, const
   A.blk = (TickBlock*)((char*)blk.p + o_blk); A.tile = (uint2*)((char*)blk.p + o_tile); A.ranks = (RankTicks*)((char*)blk.p + o_rank);
   A.vec = (((uintptr_t)send_count | (uintptr_t)recv_count) & 15) == 0;
   const u32 rank_ctas = (u32)(((u64)n_ranks + RT_THREADS - 1) / RT_THREADS);
-  A.far = (u32*)((char*)blk.p + o_far); A.scanned = n_tiles > RT_SCAN ? A.far + rank_ctas : nullptr;
+  const bool long_ranks = n_tiles > (u64)RT_NEAR * n_ranks;      // on average
+  A.far = (u32*)((char*)blk.p + o_far); A.scanned = n_tiles > (long_ranks ? RT_SCAN : RT_LOOK) ? A.far + rank_ctas : nullptr;
   launch(st, k_tick_blocks, (u32)n_tiles + rank_ctas, RT_THREADS, 0, A);
-  if (A.scanned) launch(st, k_tile_scan, 1, TS_THREADS, 0, A.tile, A.n_tiles, n_tiles > (u64)RT_NEAR * n_ranks ? nullptr : A.far, rank_ctas, A.scanned);
+  if (A.scanned) launch(st, k_tile_scan, 1, TS_THREADS, 0, A.tile, A.n_tiles, long_ranks ? nullptr : A.far, rank_ctas, A.scanned);
   launch(st, k_record_rates, (u32)((n_rec + RT_THREADS - 1) / RT_THREADS), RT_THREADS, 0, A, n_rec, rank, t_enter_ns, t_exit_ns, send_chg, recv_chg);
   const cudaError_t le = cudaGetLastError();
   ctx->pool.put(blk);           // later work on this stream runs after these kernels: the block can be handed out again

@@ -30,7 +30,11 @@ constexpr int RT_TILE = RT_THREADS * 8;            // ticks per CTA of k_tick_bl
 // since their beginning would add up many, and the scan pays: 20,000 tiles of one rank among 4,096, 50,000 records: 1,067 -> 99 us.
 // (4,096 equal ranks of 5,600 ticks, whose scan is launched to find out that there are none: 80.1 -> 81.5 us.)
 constexpr u32 RT_NEAR = 8;
-constexpr u64 RT_SCAN = 256;                       // up to so many tiles in all a record adds them up whatever the segments are
+// Up to RT_SCAN tiles in all a record adds up what it spans whatever the segments are. Up to RT_LOOK the scan is launched only
+// where the ranks' average is beyond RT_NEAR: calls of that size are bound by the host, and a launch in order to look makes them
+// 2 us longer (11.6 us without it at 2,000 tiles of 4,096 equal ranks, 13.8 with it at 2,100). Without it 2,000 tiles of one rank among
+// 4,096 and 20,000 records, a third in flight, take 59 us instead of 20.
+constexpr u64 RT_SCAN = 256, RT_LOOK = 2048;
 
 // before: changes before the block inside the tile (send in the low half, recv in the high half); the ticks' change bits
 struct alignas(16) TickBlock { u32 before, send, recv, pad; };
