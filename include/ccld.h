@@ -95,7 +95,7 @@ void ccld_params_default(ccld_params* p /* host, out */);
  * Lifecycle. `device` is a CUDA ordinal, `cuda_stream` a cudaStream_t (NULL = default stream) on
  * which every copy and kernel of this context is enqueued. The context owns all memory it allocates
  * and gives it up in ccld_destroy: to the driver, except for blocks that contexts of the same process
- * which are still there may use - at most 64 MB per device, and 64 MB of pinned host memory. When
+ * which are still there may use - at most 256 MB per device, and 64 MB of pinned host memory. When
  * the last context goes, those are freed too.
  */
 int ccld_create(ccld_ctx** out, const ccld_params* params /* host */, int device, void* cuda_stream);
