@@ -363,10 +363,10 @@ def measure(spec, order, steps, warmup, local_rank, world, sample_clocks):
                 "achieved_with_regrouping_bytes": (d_alg + d_over) / (d_ms * 1e-3) / 1e9 if d_ms > 0 else 0.0,
                 "kernels_ms_per_step": {k: kt[k]["ms"] / steps for k in kt},
                 "whole_path": {"algorithmic_bytes_per_step": path_bytes, "achieved": path_gbs, "frac": path_gbs / peak}}
-    # beside the timed launches: k_begin, one per step like k_seq_range; k_reduce_deferred after every launch of the fused reduce
+    # beside the timed launches: k_reduce_deferred after every launch of the fused reduce
     # kernel (inside the same event pair), k_reduce_large_deferred after those of the larger communicators, and k_window_rounds
     # before every k_window_decide
-    launches = (sum(x["launches"] for x in kt.values()) + kt["k_seq_range"]["launches"] + kt["k_reduce_fused"]["launches"]
+    launches = (sum(x["launches"] for x in kt.values()) + kt["k_reduce_fused"]["launches"]
                 + max(kt["k_reduce_mid"]["launches"], kt["k_reduce_large"]["launches"]) + kt["k_window_decide"]["launches"])
     return {"n_rec": n_rec, "now": now, "ms_total": ms, "ms_per_step": ms / steps, "ms_best": min(per_step), "ms_median": statistics.median(per_step),
             "value": world * n_rec * steps / (ms * 1e-3), "value_best": world * n_rec / (min(per_step) * 1e-3),

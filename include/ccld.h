@@ -401,8 +401,8 @@ int ccld_derive_rates(ccld_ctx* ctx, uint64_t n_rec, const uint32_t* rank, const
  * Per-kernel device timing for benchmarks. While enabled, ccld_analyze_window brackets each of its
  * kernel launches with CUDA events on the context's stream. ccld_get_kernel_times synchronizes the
  * stream and returns, per kernel kind, the summed device time in milliseconds and the number of
- * launches since timing was last enabled. Kinds: 0 op-counter range, 1 slot layout and work lists
- * (two launches per call), 2 slot scatter, 3 reductions n <= 128 (fused), 4 reductions n <= 1024,
+ * launches since timing was last enabled. Kinds: 0 op-counter range, 1 start values and slot
+ * layout (two launches per call), 2 slot scatter with the work lists, 3 reductions n <= 128 (fused), 4 reductions n <= 1024,
  * 5 reductions n > 1024, 6 window decision. Enabling (on = 1) clears the sums; on = 0 stops timing.
  * Independently of this switch, every entry point and every stage of ccld_analyze_window opens a named NVTX range
  * ("ccld_analyze_window", "ccld: slot scatter", ...) on the calling thread, which costs nothing unless a timeline

@@ -121,8 +121,6 @@ struct WinDesc {
   u32 *rmin, *rmax;                  // [n_comms] op counter range seen
   RangeRow* ranges;                  // [n_comms]
   uint4* srow;                       // [n_comms] scatter rows: first slot low, high, op counters covered (0 = nothing to place), first op counter
-  uint4* rent;                       // [n_ranks][RANK_TAB_K] a rank's inline pairs resolved for this window: (communicator id, op counters
-                                     //   covered (0: unused), first op counter, first slot of the member's column); 32-bit slots only
   u64* totals;                       // [T_COUNT]
   uint2* chunks;                     // [CHUNK_MAX + 1] first CTA (x) and first warp-tile (y) of every chunk, relative to the window
   u64* totals_host;                  // [T_COUNT] the totals once more, in pinned host memory

@@ -10,7 +10,7 @@
 //   k_reduce_deferred  the listed groups, one warp each, in full 64-bit generality: missing members, records in
 //                      flight (hang alerts), invalid times, spreads beyond 32 bits.
 //
-// The work list of k_reduce_fused is chunk-major (see k_emit), so CTAs that run together gather from the same stretch
+// The work list of k_reduce_fused is chunk-major (see emit_lists), so CTAs that run together gather from the same stretch
 // of every rank's records and share the fetched sectors in L2.
 #pragma once
 #include "ccld_device.cuh"

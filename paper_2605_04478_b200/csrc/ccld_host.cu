@@ -151,7 +151,7 @@ constexpr u32 UP_WORKERS = 6, UP_SLOTS = 2 * UP_WORKERS;   // two pieces per wor
 constexpr size_t UP_SMALL = 256u << 10;                    // up to this size one kernel reads the pinned columns, beyond it they are copied one by one
 
 constexpr u32 TIMER_RING = 32;
-constexpr int TIMER_PAIRS = CCLD_K_KINDS + 1;          // the layout kernel runs twice per call
+constexpr int TIMER_PAIRS = CCLD_K_KINDS + 1;          // two launches of the plan per call
 struct TimerSlot { cudaEvent_t a[TIMER_PAIRS], b[TIMER_PAIRS]; int kind[TIMER_PAIRS]; int n = 0; };
 
 }  // namespace
@@ -895,7 +895,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   const size_t o_desc = take(B * sizeof(WinDesc)), o_exp = take(expect ? tot_bytes : 0), up_bytes = off,      // what comes from the host
                o_zero = off, o_rmax = take((size_t)B * nc * 4), o_cnt = take((size_t)B * C_COUNT * 8), o_defn = take(16), o_zero_end = off,
                o_rmin = take((size_t)B * nc * 4), o_rng = take((size_t)B * nc * sizeof(RangeRow)), o_srow = take((size_t)B * nc * sizeof(uint4)),
-               o_rent = take((size_t)B * ctx->n_ranks * RANK_TAB_K * sizeof(uint4)), o_tot = take(tot_bytes), o_chunk = take((size_t)B * (CHUNK_MAX + 1) * sizeof(uint2));
+               o_tot = take(tot_bytes), o_chunk = take((size_t)B * (CHUNK_MAX + 1) * sizeof(uint2));
   cudaError_t e;
   Block pb = ctx->pool.get(off, &e);
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "plan allocation failed");
@@ -919,7 +919,6 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     cta = std::max<u64>(cta, (d.n_rec + REC_PER_CTA - 1) / REC_PER_CTA);
     d.rmin = (u32*)(pbase + o_rmin) + (size_t)k * nc; d.rmax = (u32*)(pbase + o_rmax) + (size_t)k * nc;
     d.ranges = (RangeRow*)(pbase + o_rng) + (size_t)k * nc; d.srow = (uint4*)(pbase + o_srow) + (size_t)k * nc;
-    d.rent = (uint4*)(pbase + o_rent) + (size_t)k * ctx->n_ranks * RANK_TAB_K;
     d.totals = (u64*)(pbase + o_tot) + (size_t)k * T_COUNT; d.counters = (u64*)(pbase + o_cnt) + (size_t)k * C_COUNT;
     d.chunks = (uint2*)(pbase + o_chunk) + (size_t)k * (CHUNK_MAX + 1); d.totals_host = (u64*)pbatch.pin.p + (size_t)k * T_COUNT;
     d.expect = expect ? (const u64*)(pbase + o_exp) + (size_t)k * T_COUNT : nullptr; d.poison = ctx->d_poison;
@@ -933,12 +932,13 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   if (cta > 0x7FFFFFFFull) return fail(ctx, CCLD_ERR_CAPACITY, "batch too large for one launch");
   WinDesc* d_desc = (WinDesc*)(pbase + o_desc);
   TimerSlot* ts = timer_begin(ctx);
+  const u32 layout_threads = nc <= 128 ? 128 : (nc <= 256 ? 256 : (nc <= 512 ? 512 : LAYOUT_THREADS));
   auto start_plan = [&](u32 fill_ctas) -> cudaError_t {    // uploads the descriptors, sets the start values, runs the range pass and the layout
     BeginArgs ba;
     ba.desc_host = (const u32*)h_up; ba.desc = (u32*)(pbase + o_desc); ba.desc_words = up_bytes / 4;
     ba.rmin = (u32*)(pbase + o_rmin); ba.n_rmin = (u64)B * nc; ba.zero = (u32*)(pbase + o_zero); ba.n_zero = (o_zero_end - o_zero) / 4;
     const u64 most = std::max<u64>(std::max<u64>(ba.desc_words, ba.n_rmin), ba.n_zero);
-    launch(st, k_begin, (u32)std::min<u64>((most + BEGIN_THREADS - 1) / BEGIN_THREADS, 2ull * ctx->n_sms), BEGIN_THREADS, 0, ba);
+    { TimedLaunch tl(ts, 1, st); launch(st, k_begin, (u32)std::min<u64>((most + BEGIN_THREADS - 1) / BEGIN_THREADS, 2ull * ctx->n_sms), BEGIN_THREADS, 0, ba); }
     if (cta > 0) {
       // enough CTAs to fill the device several times over, then as many blocks per CTA as that leaves
       const u64 want = 32ull * ctx->n_sms;
@@ -946,7 +946,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
       TimedLaunch tl(ts, 0, st);
       launch(st, k_seq_range, dim3((u32)((cta + per - 1) / per), B), REC_THREADS, range_smem_bytes(nc), d_desc, ctx->reg, per);
     }
-    { TimedLaunch tl(ts, 1, st); launch(st, k_layout, dim3(1 + fill_ctas, B), LAYOUT_THREADS, 0, d_desc, ctx->reg, fill_ctas != 0); }
+    { TimedLaunch tl(ts, 1, st); launch(st, k_layout, dim3(1 + fill_ctas, B), layout_threads, 0, d_desc, ctx->reg, fill_ctas != 0); }
     return cudaGetLastError();
   };
   const u64* tot = nullptr;                                // [B][T_COUNT] totals the results are sized from
@@ -1000,24 +1000,21 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   if (expect) {
     // Descriptors already complete: nothing was waited for, and the slot table is filled beside the layout's one CTA per
     // window. Two CTAs per SM share the filling.
-    const u64 want = (max_slots + 16ull * LAYOUT_THREADS - 1) / (16ull * LAYOUT_THREADS);
-    CK(start_plan((u32)std::max<u64>(1, std::min<u64>(want, 2ull * ctx->n_sms / B))));
+    const u64 want = (max_slots + 16ull * layout_threads - 1) / (16ull * layout_threads);
+    CK(start_plan((u32)std::max<u64>(1, std::min<u64>(want, 2ull * (LAYOUT_THREADS / layout_threads) * ctx->n_sms / B))));
   } else {
     CK(cudaMemcpyAsync(d_desc, hd, B * sizeof(WinDesc), cudaMemcpyHostToDevice, st));
     if (total_slots) CK(cudaMemsetAsync(rbase + o_perm, 0xFF, total_slots * 4, st));
   }
   PlanLists pl; pl.fcta = (FusedCta*)(rbase + o_fcta); pl.fwt = (WarpTile*)(rbase + o_fwt); pl.t2 = (Tile*)(rbase + o_t2); pl.t3 = (Tile*)(rbase + o_t3);
   {
-    const u32 rank_ctas = std::min<u32>((2 * ctx->n_ranks + EMIT_THREADS - 1) / EMIT_THREADS, 2 * ctx->n_sms), comm_blocks = (nc + EMIT_THREADS - 1) / EMIT_THREADS,
-              per_slice = (comm_blocks + EMIT_SLICES - 1) / EMIT_SLICES, slices = (comm_blocks + per_slice - 1) / per_slice;
-    TimedLaunch tl(ts, 1, st);
-    launch(st, k_emit, dim3(chunk_ctas * slices + rank_ctas, B), EMIT_THREADS, 0, d_desc, ctx->reg, pl, chunk_ctas * slices, slices, per_slice);
-  }
-  if (cta > 0) {
+    // the CTAs that write the work lists come first in the scatter's launch
+    const u32 comm_blocks = (nc + EMIT_THREADS - 1) / EMIT_THREADS, per_slice = (comm_blocks + EMIT_SLICES - 1) / EMIT_SLICES,
+              slices = (comm_blocks + per_slice - 1) / per_slice, emit_ctas = chunk_ctas * slices;
     const u64 blocks = (cta * REC_PER_CTA + SCAT_PER_CTA - 1) / SCAT_PER_CTA;      // of the largest window
     const u32 per = (u32)std::min<u64>(SCAT_BLOCKS_MAX, std::max<u64>(1, blocks * B / (16ull * ctx->n_sms)));
     TimedLaunch tl(ts, 2, st);
-    launch(st, k_slot_scatter, dim3((u32)((blocks + per - 1) / per), B), SCAT_THREADS, 0, d_desc, ctx->reg, per);
+    launch(st, k_slot_scatter, dim3(emit_ctas + (u32)((blocks + per - 1) / per), B), SCAT_THREADS, 0, d_desc, ctx->reg, pl, emit_ctas, slices, per_slice, per);
   }
   const DeferList dl_big{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
   static_assert(MID_SEQS == LARGE_SEQS, "one list for the groups of both classes");

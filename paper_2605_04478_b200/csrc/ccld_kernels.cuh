@@ -2,9 +2,8 @@
 // the host side only sizes buffers and launches.
 //
 //   k_seq_range     group-by, part 1: op-counter range per (window, communicator)
-//   k_layout, k_emit  group-by, part 2: closed-form slot layout (prefix sums over communicators) and the work lists of the
-//                   reduction kernels (ccld_plan.cuh)
-//   k_slot_scatter  group-by, part 3: perm[slot] = record index
+//   k_layout        group-by, part 2: closed-form slot layout (prefix sums over communicators; ccld_plan.cuh)
+//   k_slot_scatter  group-by, part 3: perm[slot] = record index; beside it the work lists of the reduction kernels
 //   k_reduce_fused  per-op reductions + median/MAD + flags + votes for n <= 128, chunk-major work list:
 //                   n <= 8 one thread per group (warp-tiles), 9 <= n <= 128 n_pad / 8 lanes per group (register /
 //                   shuffle bitonic network); complete groups whose times fit 32-bit offsets
@@ -282,9 +281,7 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
 }
 
 // ------------------------------------------------------------------------------------------------
-// group-by, part 3: every accepted record drops its index into its slot. Two dependent loads per
-// record in the common case - the rank's inline (communicator, index, position) pairs, then the
-// communicator's scatter row - issued for four records at a time.
+// group-by, part 3: every accepted record drops its index into its slot.
 // ------------------------------------------------------------------------------------------------
 // Registry walk for a record whose (rank, communicator) pair is not inline: returns index << 13 | position in the
 // low word, or NONE there with the rejecting CCLD_E_* bit in the high word.
@@ -316,39 +313,51 @@ __device__ __forceinline__ bool scatter_slot(const Registry& R, u32 c, u32 ns, u
 }
 
 constexpr u32 SCAT_LOCAL = 8;     // ranks, counted from the rank of the CTA's first record, whose table rows a CTA resolves once
+static_assert(SCAT_THREADS == EMIT_THREADS, "CTAs of both kinds in one launch");
 
-// A CTA's records mostly belong to a few neighbouring ranks (a rank-major upload: one or two), so each warp first copies
-// the resolved inline pairs of SCAT_LOCAL ranks - communicator id -> (counters covered, first counter, slot of the member's
-// first counter), which the layout pass wrote for this window - into shared memory; a record of those ranks then needs no global table at all and, in windows of
+// A CTA's records mostly belong to a few neighbouring ranks (a rank-major upload: one or two), so each warp first resolves
+// the inline pairs of SCAT_LOCAL ranks - communicator id -> (counters covered, first counter, slot of the member's
+// first counter) - against the window's scatter rows into shared memory; a record of those ranks then needs no global table at all and, in windows of
 // fewer than 2^32 slots, only 32-bit arithmetic. Any other record (another rank, a communicator beyond the inline pairs,
 // a counter outside the range, a rejected record) takes the two dependent table loads and the full checks.
-__global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc* wd, Registry R, u32 blocks_per_cta) {
+// Grid: (emitting CTAs + CTAs of the largest window, windows).
+__global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc* wd, Registry R, PlanLists L, u32 emit_ctas, u32 slices, u32 slice_blocks, u32 blocks_per_cta) {
   begin_after();
   // (communicator id, counters covered, first counter, first slot) per resolved pair; counters covered 0: unused. Every
   // warp keeps its own copy, so no warp waits for another; two copies, because the entries of the next block are written
   // while lanes may still read those of the current one.
   __shared__ uint4 s_ent_all[2][SCAT_THREADS / 32][SCAT_LOCAL * RANK_TAB_K];
   static_assert(SCAT_LOCAL * RANK_TAB_K == 32, "one resolved pair per lane");
-  const WinDesc& D = wd[blockIdx.y];                          // grid: (CTAs of the largest window, windows)
-  const u64 base0 = (u64)blockIdx.x * blocks_per_cta * SCAT_PER_CTA;
-  if (base0 >= D.n_rec) return;                               // (a window that was given up has empty scatter rows: nothing is stored)
+  const WinDesc& D = wd[blockIdx.y];
+  if (blockIdx.x < emit_ctas) { emit_lists(D, R, L, emit_ctas, slices, slice_blocks, &s_ent_all[0][0][0]); return; }
+  const u64 base0 = (u64)(blockIdx.x - emit_ctas) * blocks_per_cta * SCAT_PER_CTA;
+  if (base0 >= D.n_rec) return;
+  // a window that was refused has empty scatter rows: nothing is stored, and what it rejects is counted. The rows of one that gives up
+  // because of another window are being cleared: it is left alone and will be analysed again. (Read here, looked at when the first
+  // records have arrived.)
+  const u64 failed = D.totals[T_FAILED]; const u32 poisoned = *(volatile u32*)D.poison; const bool expects = D.expect != nullptr;
   u32 err = 0, rej = 0, internal = 0;
   // descriptor fields in registers: the stores below could alias the descriptor as far as the compiler knows
   u32* const perm = D.perm; const u64 n_slots = D.n_slots; const uint4* const srow = D.srow; const u64 n_rec = D.n_rec;
-  const uint4* const rent = D.rent;
   const u32 *c_rank = D.rank, *c_comm = D.comm, *c_seq = D.seq;
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // the resolved pairs of the SCAT_LOCAL ranks that start at rank r_first, one per lane
-  auto pairs_of = [&](u32 r_first) {
-    const u32 r = r_first + lane / RANK_TAB_K;
-    uint4 e = make_uint4(NONE, 0, 0, 0);
-    if (r_first < R.n_ranks && r < R.n_ranks) e = rent[(u64)r * RANK_TAB_K + lane % RANK_TAB_K];
-    return e;
+  // lane's inline pair (communicator id, index and position) of the SCAT_LOCAL ranks that start at rank r0, and the scatter row it names
+  auto pair_of = [&](u32 r0) {
+    const u32 r = r0 + lane / RANK_TAB_K;
+    return r0 < R.n_ranks && r < R.n_ranks ? reinterpret_cast<const uint2*>(R.rank_tab)[(u64)r * RANK_TAB_K + lane % RANK_TAB_K] : make_uint2(NONE, NONE);
   };
-  // A CTA takes blocks_per_cta consecutive blocks. The chain "first record's rank -> that rank's resolved pairs" of a
+  auto row_of = [&](uint2 p) { return p.x != NONE && p.y < RANK_TAB_OVERFLOW ? srow[p.y >> RANK_TAB_POS_BITS] : make_uint4(0, 0, 0, 0); };
+  // The member's column starts at the communicator's first slot + position * counters covered. Only where slots fit 32 bits and the
+  // whole column lies inside the table; other pairs stay unused, and so that they match no record they carry no communicator's id.
+  auto resolve = [&](uint2 p, uint4 sr) {
+    const u64 b = ((u64)sr.x | ((u64)sr.y << 32)) + (u64)(p.y & ((1u << RANK_TAB_POS_BITS) - 1)) * sr.z;
+    return sr.z != 0 && n_slots <= 0xFFFFFFFFull && b + sr.z <= n_slots ? make_uint4(p.x, sr.z, sr.w, (u32)b) : make_uint4(NONE, 0, 0, 0);
+  };
+  // A CTA takes blocks_per_cta consecutive blocks. The chain "first record's rank -> that rank's pairs -> their rows" of a
   // block is started one block ahead, so a block waits for its records only.
   u32 r_first = c_rank[base0];
-  uint4 e_mine = pairs_of(r_first);
+  uint2 p_mine = pair_of(r_first);
+  uint4 row_mine = row_of(p_mine);
   for (u32 blk = 0; blk < blocks_per_cta; ++blk) {
     const u64 base = base0 + (u64)blk * SCAT_PER_CTA;
     if (base >= n_rec) break;
@@ -363,11 +372,12 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc*
     }
     const u64 base_next = base + SCAT_PER_CTA;
     const bool has_next = blk + 1 < blocks_per_cta && base_next < n_rec;
-    const u32 r_next = has_next ? c_rank[base_next] : 0u;     // in flight with the records
+    const u32 r_next = has_next ? c_rank[base_next] : NONE;   // in flight with the records
     uint4* const s_ent = s_ent_all[blk & 1][wid];
-    if (e_mine.y == 0) e_mine.x = NONE;                       // an unused pair must not shadow a record of communicator 0
-    s_ent[lane] = e_mine;
+    s_ent[lane] = resolve(p_mine, row_mine);
     __syncwarp();
+    if (failed == 0 && expects && poisoned) return;           // the same in the whole launch
+    p_mine = pair_of(r_next);                                 // the next block's pairs: its first rank has arrived with this block's records
 #pragma unroll
     for (int k = 0; k < SCAT_PER_THREAD; ++k) {
       const u32 dr = rk[k] - r_first;
@@ -383,8 +393,7 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc*
         }
       }
     }
-    // the next block's pairs: its first rank has arrived with this block's records
-    if (has_next) e_mine = pairs_of(r_next);
+    row_mine = row_of(p_mine);
     if (__any_sync(0xFFFFFFFFu, todo != 0)) {
 #pragma unroll
       for (int k = 0; k < SCAT_PER_THREAD; ++k) {

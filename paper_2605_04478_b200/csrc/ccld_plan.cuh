@@ -5,21 +5,21 @@
 //             lengths get their start values
 //   k_layout  one CTA per window: prefix sums over the communicators (groups, slots, rows, work units) and the start of every
 //             chunk of the work lists; the other CTAs of the launch fill the slot table of a batch that does not wait
-//   k_emit    a CTA per (window, chunk, 256 communicators) writes their part of the chunk's work lists; further CTAs resolve
-//             every rank's inline pairs against the window's rows
+//   emit_lists  a CTA per (window, chunk, 256 communicators) writes their part of the chunk's work lists, beside the scatter
+//             pass and in its launch (ccld_kernels.cuh)
 //
-// All three are bound by latency: little data, a chain of dependent reads and barriers. The layout used to be one CTA per
+// All are bound by latency: little data, a chain of dependent reads and barriers. The layout used to be one CTA per
 // window for everything - one scan over the communicators per chunk, the rank table of the whole job walked by one SM -
 // and took 20 us (one communicator, 1,000 ops) to 155 us (2,185 communicators, 16,384 ranks), twice per batch. What a
 // chunk holds follows from the chunk lengths alone, so the chunks' starts come from a histogram of where the
-// communicators end, and the lists and rank entries are written by as many CTAs as there are chunks and ranks.
+// communicators end, and the lists are written by as many CTAs as there are chunks.
 #pragma once
 #include "ccld_device.cuh"
 
 namespace ccld {
 
 constexpr int BEGIN_THREADS = 256;
-constexpr int LAYOUT_THREADS = 1024;
+constexpr u32 LAYOUT_THREADS = 1024;                   // at most: as many as there are communicators do for a small registry
 constexpr u32 LAYOUT_CACHED = 4;                       // communicators per thread whose ranges wait in registers (4,096 per window)
 constexpr int EMIT_THREADS = 256;
 constexpr u32 EMIT_SLICES = 32;
@@ -88,7 +88,7 @@ struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; };
 
 // When the host sized the results from totals it expected (D.expect) instead of waiting for these, a window whose totals
 // differ gives up and raises the poison flag; so does every window planned after the flag went up - in the same batch
-// (seen by k_emit) or in a later one - so that windows are never analysed out of order.
+// (seen by emit_lists) or in a later one - so that windows are never analysed out of order.
 // Grid: (1 + filling CTAs, windows). fill: whether the slot table (sized from the expectation) is to be set to NONE.
 __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Registry R, int fill) {
   begin_after();
@@ -101,14 +101,18 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
     if (!fill) return;
     u32* __restrict__ perm = D.perm; const u64 n = D.n_slots;
     const u64 head = min(n, (u64)((16 - ((uintptr_t)perm & 15)) & 15) / 4), n4 = (n - head) / 4;
-    const u64 i0 = (u64)(blockIdx.x - 1) * LAYOUT_THREADS + threadIdx.x, st = (u64)(gridDim.x - 1) * LAYOUT_THREADS;
+    const u64 i0 = (u64)(blockIdx.x - 1) * blockDim.x + threadIdx.x, st = (u64)(gridDim.x - 1) * blockDim.x;
     uint4* p4 = reinterpret_cast<uint4*>(perm + head);
     for (u64 i = i0; i < n4; i += st) p4[i] = make_uint4(NONE, NONE, NONE, NONE);
     if (i0 < head) perm[i0] = NONE;
     if (i0 < n - head - n4 * 4) perm[head + n4 * 4 + i0] = NONE;
     return;
   }
-  const u32 per = ceil_div(R.n_comms, LAYOUT_THREADS), c_lo = threadIdx.x * per, c_hi = min(R.n_comms, c_lo + per);   // my communicators
+  // what warp 0 compares its findings with; poisoned: an earlier batch's layout was not the expected one
+  const u64 slot_cap = D.slot_cap; const bool expects = D.expect != nullptr;
+  u64 expected = 0; bool poisoned = false;
+  if (wid == 0 && expects) { expected = lane < T_COUNT ? D.expect[lane] : 0; poisoned = *(volatile u32*)D.poison != 0; }
+  const u32 per = ceil_div(R.n_comms, blockDim.x), c_lo = threadIdx.x * per, c_hi = min(R.n_comms, c_lo + per);   // my communicators
   // counters covered and members of my first few communicators stay in registers, all loads issued at once
   u32 c_ns[LAYOUT_CACHED], c_n[LAYOUT_CACHED];
   {
@@ -130,10 +134,11 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   u32 mx = 0;
   each([&](u32, u32 ns, u32 n) { if (comm_class(n) <= 1) mx = max(mx, ns); });
   mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+  const u32 n_warps = blockDim.x / 32;
   if (lane == 0) s_red[wid] = mx;
-  for (u32 i = threadIdx.x; i < 2 * (CHUNK_MAX + 2); i += LAYOUT_THREADS) (&s_hist[0][0])[i] = 0;
+  for (u32 i = threadIdx.x; i < 2 * (CHUNK_MAX + 2); i += blockDim.x) (&s_hist[0][0])[i] = 0;
   __syncthreads();
-  mx = __reduce_max_sync(0xFFFFFFFFu, s_red[lane]);
+  mx = __reduce_max_sync(0xFFFFFFFFu, lane < n_warps ? s_red[lane] : 0u);
   u32 T = mx ? ceil_div(mx, CHUNK_REF) : 1u;
   T = T > CHUNK_MAX ? CHUNK_MAX : T;
   // sums over my communicators, and where their units begin and end along the chunks
@@ -163,7 +168,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   if (lane == 31) s_warp[wid] = inc;
   __syncthreads();
   if (wid == 0) {
-    PlanAcc xi = s_warp[lane];
+    PlanAcc xi = lane < n_warps ? s_warp[lane] : PlanAcc{0, 0, 0, 0, 0, 0};
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) { PlanAcc o = plan_shfl_up(xi, d); if (lane >= (u32)d) xi = plan_add(xi, o); }
     PlanAcc ex = plan_shfl_up(xi, 1);
@@ -203,24 +208,21 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
     const u64 n_cta = __shfl_sync(0xFFFFFFFFu, pc, 31), n_wt = __shfl_sync(0xFFFFFFFFu, pw, 31);
     static_assert(CHUNK_MAX == 64, "two chunks per lane");
     if (lane == 31) D.chunks[CHUNK_MAX] = make_uint2(pc, pw);
+    // the totals, one per lane
+    u64 t = 0;
+    t = lane == T_GROUPS ? all.groups : t; t = lane == T_SLOTS ? all.slots : t; t = lane == T_FCTA ? n_cta : t; t = lane == T_FWT ? n_wt : t;
+    t = lane == T_FSUM ? all.units : t; t = lane == T_TILES2 ? all.t2 : t; t = lane == T_TILES3 ? all.t3 : t; t = lane == T_ROWS ? all.rows : t;
+    t = lane == T_CHUNKS ? T : t;
+    // op counters further apart than 2^31, or more slots than the cap: refuse the window
+    u64 failed = (all.slots > slot_cap || all.groups > 0x7FFFFFFFull) ? FAILED_CAPACITY : 0;
+    if (!failed && expects) {
+      const bool same = lane == T_FAILED || lane >= T_COUNT || t == expected;
+      if (!__all_sync(0xFFFFFFFFu, same) || poisoned) { failed = FAILED_EXPECT; if (lane == 0) atomicExch(D.poison, 1u); }
+    }
+    if (failed) t = lane == T_CHUNKS ? 1 : 0;
+    if (lane == T_FAILED) t = failed;
+    if (lane < T_COUNT) { D.totals[lane] = t; D.totals_host[lane] = t; }
     if (lane == 0) {
-      // op counters further apart than 2^31, or more slots than the cap: refuse the window
-      u64 failed = (all.slots > D.slot_cap || all.groups > 0x7FFFFFFFull) ? FAILED_CAPACITY : 0;
-      if (!failed && D.expect != nullptr) {
-        const u64* e = D.expect;
-        const bool same = e[T_GROUPS] == all.groups && e[T_SLOTS] == all.slots && e[T_FCTA] == n_cta && e[T_FWT] == n_wt && e[T_FSUM] == all.units &&
-                          e[T_TILES2] == all.t2 && e[T_TILES3] == all.t3 && e[T_ROWS] == all.rows && e[T_CHUNKS] == T;
-        if (!same || *(volatile u32*)D.poison != 0) { failed = FAILED_EXPECT; atomicExch(D.poison, 1u); }
-      }
-      u64 t[T_COUNT];
-      for (int q = 0; q < T_COUNT; ++q) t[q] = 0;
-      if (!failed) {
-        t[T_GROUPS] = all.groups; t[T_SLOTS] = all.slots; t[T_FCTA] = n_cta; t[T_FWT] = n_wt; t[T_FSUM] = all.units;
-        t[T_TILES2] = all.t2; t[T_TILES3] = all.t3; t[T_ROWS] = all.rows;
-      }
-      t[T_FAILED] = failed; t[T_CHUNKS] = failed ? 1 : T;
-      u64* const totals = D.totals; u64* const totals_host = D.totals_host;
-      for (int q = 0; q < T_COUNT; ++q) { totals[q] = t[q]; totals_host[q] = t[q]; }
       if (failed == FAILED_CAPACITY) atomicOr((unsigned*)&D.counters[C_ERR], (unsigned)CCLD_E_CAPACITY);
       s_red[0] = failed != 0;
     }
@@ -244,48 +246,22 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   });
 }
 
-// Grid: (chunk CTAs + rank CTAs, windows); chunk CTA x takes slice x % slices of chunk x / slices: `blocks` times EMIT_THREADS
-// communicators (one time, unless a registry has more than EMIT_SLICES times as many). There are enough of them for every
-// chunk of any window of the batch. base[] of the descriptors is filled. A window that gave up fills its stretch of the
-// lists with entries that hold no work, because the kernels that follow are launched over the expected lengths.
-__global__ void __launch_bounds__(EMIT_THREADS) k_emit(const WinDesc* wd, Registry R, PlanLists L, u32 chunk_ctas, u32 slices, u32 blocks) {
-  begin_after();
-  __shared__ uint4 s_pair[EMIT_THREADS / 32];
-  const WinDesc& D = wd[blockIdx.y];
+// The work lists, written by the first `ctas` CTAs of k_slot_scatter's launch for every window: CTA x takes slice x % slices of
+// chunk x / slices, `blocks` times EMIT_THREADS communicators (one time, unless a registry has more than EMIT_SLICES times as
+// many). There are enough of them for every chunk of any window of the batch. base[] of the descriptors is filled. A window that
+// gave up fills its stretch of the lists with entries that hold no work, because the kernels that follow are launched over the
+// expected lengths. Neither the lists nor the scatter reads what the other writes; a launch of its own in between took 4.5
+// (one communicator) to 17 us (twelve windows of 1,088 communicators) of every pass.
+__device__ __forceinline__ bool gives_up(const WinDesc& D) {
+  // the flag can only go up while k_layout runs, so every CTA of the launch sees the same value
+  return D.totals[T_FAILED] != 0 || (D.expect != nullptr && *(volatile u32*)D.poison != 0);
+}
+__device__ __forceinline__ void emit_lists(const WinDesc& D, const Registry& R, const PlanLists& L, u32 ctas, u32 slices, u32 blocks, uint4* s_pair /* a warp's */) {
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const u64 failed = D.totals[T_FAILED];
-  // the flag can only go up while k_layout runs, so every CTA of this launch sees the same value
-  const bool give_up = failed != 0 || (D.expect != nullptr && *(volatile u32*)D.poison != 0);
-  const u64 n_slots = D.totals[T_SLOTS];
-  if (blockIdx.x >= chunk_ctas) {
-    // every rank's inline (communicator, position) pairs resolved against this window's scatter rows, so that the
-    // scatter pass finds (op counters covered, first op counter, first slot of the member's column) with one load. Only
-    // where slots fit 32 bits and the member's whole column lies inside the table; other entries stay unused.
-    const bool usable = !give_up && n_slots <= 0xFFFFFFFFull;
-    const u64 st = (u64)(gridDim.x - chunk_ctas) * EMIT_THREADS;
-    const uint4* const srow = D.srow; uint4* const rent = D.rent;
-    for (u64 i = (u64)(blockIdx.x - chunk_ctas) * EMIT_THREADS + threadIdx.x; i < (u64)R.n_ranks * 2; i += st) {
-      uint4 e[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-      if (usable) {
-        const uint4 t = R.rank_tab[i];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const u32 id = h ? t.z : t.x, cp = h ? t.w : t.y;
-          if (id != NONE && cp != NONE && cp != RANK_TAB_OVERFLOW) {
-            const uint4 sr = srow[cp >> RANK_TAB_POS_BITS];
-            const u64 b = ((u64)sr.x | ((u64)sr.y << 32)) + (u64)(cp & ((1u << RANK_TAB_POS_BITS) - 1)) * sr.z;
-            if (sr.z != 0 && b + sr.z <= n_slots) e[h] = make_uint4(id, sr.z, sr.w, (u32)b);
-          }
-        }
-      }
-      rent[i * 2] = e[0]; rent[i * 2 + 1] = e[1];
-    }
-    return;
-  }
-  if (give_up) {
+  if (gives_up(D)) {
     if (D.expect == nullptr) return;                           // the host knows: it sized nothing for this window
-    const u32 i0 = blockIdx.x * EMIT_THREADS + threadIdx.x, st = chunk_ctas * EMIT_THREADS;
-    if (!failed) {                                             // another window's layout was the surprise: this one's rows go too
+    const u32 i0 = blockIdx.x * EMIT_THREADS + threadIdx.x, st = ctas * EMIT_THREADS;
+    if (D.totals[T_FAILED] == 0) {                             // another window's layout was the surprise: this one's rows go too
       for (u32 c = i0; c < R.n_comms; c += st) { D.ranges[c] = RangeRow{0, 0, 0, R.comm_n[c], 0, 0, 0, 0}; D.srow[c] = make_uint4(0, 0, 0, 0); }
       if (i0 == 0) for (int q = 0; q < T_COUNT; ++q) { const u64 v = q == T_FAILED ? FAILED_EXPECT : 0; D.totals_host[q] = v; }
     }
