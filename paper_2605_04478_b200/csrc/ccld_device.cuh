@@ -22,10 +22,8 @@ constexpr int REC_PER_THREAD = 16;     //   each walks a run of consecutive reco
 constexpr int REC_PER_CTA = REC_THREADS * REC_PER_THREAD;
 constexpr int SMALL_N = 8;             // communicators of up to 8 ranks: one thread per group
 constexpr int SMALL_SEQS = 256;        //   threads per CTA: eight warps, each on a warp-tile of up to 32 op counters at a time
-#ifndef CCLD_FUSED_WT_PER_CTA
-#define CCLD_FUSED_WT_PER_CTA 16
-#endif
-constexpr u32 FUSED_WT_PER_CTA = CCLD_FUSED_WT_PER_CTA;   //   warp-tiles a CTA works through (a multiple of its eight warps)
+constexpr u32 FUSED_WT_PER_CTA = 16;   //   warp-tiles a CTA works through: two per warp, or one where that gives every tile of the batch a
+constexpr u32 FUSED_WARPS = 148 * 3 * 8;   //   warp of its own (three CTAs of eight warps on each of a B200's SMs)
 constexpr int WARP_N = 128;            // up to 128 ranks: a CTA per tile of op counters, n_pad / 8 lanes per group
 constexpr int MID_ELEMS = 2048;        //   padded records per tile of a communicator of 9 to 128 ranks
 constexpr int MID_N = 1024;            // up to 1024 ranks: a warp per group, keys in its registers (as far as 32 per lane go; ns per op
@@ -93,10 +91,12 @@ enum { C_REJECTED = 0, C_COMPLETE, C_INCOMPLETE, C_BARRIER, C_ANALYSED, C_FLAG_S
 constexpr int N_CLASSES = 4;           // reduction code paths: n <= 8, <= 128, <= 1024, larger
 // Classes 0 and 1 run in one fused kernel whose work list is ordered by (window, time chunk): a window's op
 // counters are cut into T chunks per communicator, so that the tiles of one chunk - which gather from the same
-// stretch of every rank's records - run together and share the fetched sectors in L2.
+// stretch of every rank's records - run together and share the fetched sectors in L2. A communicator's work units are spread evenly
+// over the chunks (units_before), so that chunks are stretches of time for all communicators and yet every unit but a communicator's last one is full:
+// chunks cut at op counters of their own left a warp-tile 22 or 29 of 32 op counters for 200, 600 and 1,000 per window.
 constexpr u32 CHUNK_REF = 96;          // op counters per chunk of the busiest communicator of a window
 constexpr u32 CHUNK_MAX = 64;          // at most this many chunks per window (longer chunks beyond)
-enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS, T_FAILED, T_CHUNKS, T_COUNT = 12 };
+enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS, T_FAILED, T_CHUNKS, T_WT_PER_CTA, T_COUNT = 12 };
 constexpr u64 FAILED_CAPACITY = 1, FAILED_EXPECT = 2;      // T_FAILED: the window needs too many slots / its layout is not the expected one
 enum { B_FCTA = 0, B_FWT, B_FSUM, B_T2, B_T3, B_COUNT };
 
@@ -153,11 +153,7 @@ __host__ __device__ inline u32 tile_seqs(u32 n) {
   return c == 0 ? 32u : (c == 1 ? MID_ELEMS / mid_npad(n) : (c == 2 ? (u32)MID_SEQS : (u32)LARGE_SEQS));
 }
 __host__ __device__ inline u32 ceil_div(u32 a, u32 b) { return (a + b - 1) / b; }
-// chunking of a fused-class communicator with n_seq op counters in a window of T chunks
-__host__ __device__ inline u32 chunk_len(u32 n_seq, u32 T) { return ceil_div(n_seq, T); }
-__host__ __device__ inline u32 chunk_size(u32 n_seq, u32 T, u32 tau) {    // op counters in chunk tau (0 beyond the last)
-  const u32 S = chunk_len(n_seq, T);
-  return (u64)tau * S >= n_seq ? 0u : (n_seq - tau * S < S ? n_seq - tau * S : S);
-}
+// work units of a communicator's n_units that lie before chunk tau of T (tau <= T <= CHUNK_MAX): n_units * tau / T
+__host__ __device__ inline u32 units_before(u32 n_units, u32 T, u32 tau) { return n_units / T * tau + n_units % T * tau / T; }
 
 }  // namespace ccld

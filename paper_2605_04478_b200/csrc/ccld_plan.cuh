@@ -11,8 +11,7 @@
 // All are bound by latency: little data, a chain of dependent reads and barriers. The layout used to be one CTA per
 // window for everything - one scan over the communicators per chunk, the rank table of the whole job walked by one SM -
 // and took 20 us (one communicator, 1,000 ops) to 155 us (2,185 communicators, 16,384 ranks), twice per batch. What a
-// chunk holds follows from the chunk lengths alone, so the chunks' starts come from a histogram of where the
-// communicators end, and the lists are written by as many CTAs as there are chunks.
+// chunk holds follows from the communicators' unit counts alone, so the chunks' starts come from a histogram along the chunks, and the lists are written by as many CTAs as there are chunks.
 #pragma once
 #include "ccld_device.cuh"
 
@@ -46,20 +45,8 @@ __device__ __forceinline__ u32 range_len(u32 lo, u32 hi) {
 }
 __device__ __forceinline__ u32 plan_nseq(const WinDesc& D, u32 c) { return range_len(D.rmin[c], D.rmax[c]); }
 
-// Work units (warp-tiles of class 0, CTA tiles of class 1) of a communicator in chunk tau; 0 for other classes.
-__device__ __forceinline__ u32 chunk_units(u32 ns, u32 n, u32 T, u32 tau) {
-  if (ns == 0 || comm_class(n) > 1) return 0;
-  return ceil_div(chunk_size(ns, T, tau), tile_seqs(n));
-}
-// Its chunks, its units in every chunk but the last and in the last one.
-struct ChunkShape { u32 n, full, last; };
-__device__ __forceinline__ ChunkShape chunk_shape(u32 ns, u32 n, u32 T) {
-  ChunkShape x = {0, 0, 0};
-  if (ns == 0 || comm_class(n) > 1) return x;
-  const u32 S = chunk_len(ns, T), U = tile_seqs(n);
-  x.n = ceil_div(ns, S); x.full = ceil_div(S, U); x.last = ceil_div(ns - (x.n - 1) * S, U);
-  return x;
-}
+// Work units (warp-tiles of class 0, CTA tiles of class 1) of a communicator; 0 for other classes.
+__device__ __forceinline__ u32 fused_units(u32 ns, u32 n) { return comm_class(n) > 1 ? 0u : ceil_div(ns, tile_seqs(n)); }
 
 struct PlanAcc { u64 groups, slots; u32 rows, units, t2, t3; };
 __device__ __forceinline__ PlanAcc plan_add(const PlanAcc& a, const PlanAcc& b) {
@@ -73,12 +60,12 @@ __device__ __forceinline__ PlanAcc plan_shfl_up(const PlanAcc& a, int d) {
   r.t2 = __shfl_up_sync(0xFFFFFFFFu, a.t2, d); r.t3 = __shfl_up_sync(0xFFFFFFFFu, a.t3, d);
   return r;
 }
-__device__ __forceinline__ PlanAcc plan_item(u32 ns, u32 n, u32 T) {
+__device__ __forceinline__ PlanAcc plan_item(u32 ns, u32 n) {
   PlanAcc a = {0, 0, 0, 0, 0, 0};
   if (ns == 0) return a;
   const u32 cls = comm_class(n);
   a.groups = ns; a.slots = (u64)ns * n; a.rows = 1;
-  if (cls <= 1) { const ChunkShape x = chunk_shape(ns, n, T); a.units = (x.n - 1) * x.full + x.last; }
+  if (cls <= 1) a.units = fused_units(ns, n);
   else { const u32 t = ceil_div(ns, tile_seqs(n)); a.t2 = cls == 2 ? t : 0; a.t3 = cls == 3 ? t : 0; }
   return a;
 }
@@ -94,7 +81,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   begin_after();
   __shared__ PlanAcc s_warp[33];
   __shared__ u32 s_red[32];
-  __shared__ u32 s_hist[2][CHUNK_MAX + 2];                     // differences along the chunks: warp-tiles of class 0, tiles of class 1
+  __shared__ u32 s_hist[2][CHUNK_MAX];                         // units per chunk: warp-tiles of class 0, tiles of class 1
   const WinDesc& D = wd[blockIdx.y];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (blockIdx.x > 0) {
@@ -136,29 +123,23 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   mx = __reduce_max_sync(0xFFFFFFFFu, mx);
   const u32 n_warps = blockDim.x / 32;
   if (lane == 0) s_red[wid] = mx;
-  for (u32 i = threadIdx.x; i < 2 * (CHUNK_MAX + 2); i += blockDim.x) (&s_hist[0][0])[i] = 0;
+  for (u32 i = threadIdx.x; i < 2 * CHUNK_MAX; i += blockDim.x) (&s_hist[0][0])[i] = 0;
   __syncthreads();
   mx = __reduce_max_sync(0xFFFFFFFFu, lane < n_warps ? s_red[lane] : 0u);
   u32 T = mx ? ceil_div(mx, CHUNK_REF) : 1u;
   T = T > CHUNK_MAX ? CHUNK_MAX : T;
-  // sums over my communicators, and where their units begin and end along the chunks
+  // sums over my communicators, and their units along the chunks
   PlanAcc mine = {0, 0, 0, 0, 0, 0};
   each([&](u32, u32 ns, u32 n) {
-    mine = plan_add(mine, plan_item(ns, n, T));
-    const ChunkShape x = chunk_shape(ns, n, T);
-    // communicators of one family end in the same chunk: one set of atomics for all lanes that agree
-    const u32 key = x.n ? x.n * 2 + comm_class(n) : 0;
-    u32 pend = __ballot_sync(0xFFFFFFFFu, key != 0);
+    mine = plan_add(mine, plan_item(ns, n));
+    // communicators of one family have as many units: the lanes that agree are counted, then the lanes run along the chunks
+    const u32 units = fused_units(ns, n), key = units * 2 + comm_class(n);
+    u32 pend = __ballot_sync(0xFFFFFFFFu, units != 0);
     while (pend) {
-      const u32 lead = __shfl_sync(0xFFFFFFFFu, key, (u32)__ffs(pend) - 1u);
-      const bool same = key == lead;
-      const u32 full = __reduce_add_sync(0xFFFFFFFFu, same ? x.full : 0u), last = __reduce_add_sync(0xFFFFFFFFu, same ? x.last : 0u);
-      if (lane == 0) {
-        u32* h = s_hist[lead & 1];
-        const u32 nch = lead >> 1;
-        atomicAdd(&h[0], full); atomicAdd(&h[nch - 1], last - full); atomicAdd(&h[nch], 0u - last);
-      }
-      pend &= ~__ballot_sync(0xFFFFFFFFu, same);
+      const u32 lead = __shfl_sync(0xFFFFFFFFu, key, (u32)__ffs(pend) - 1u), same = __ballot_sync(0xFFFFFFFFu, units != 0 && key == lead);
+      const u32 times = (u32)__popc(same), u = lead >> 1;
+      for (u32 tau = lane; tau < T; tau += 32) atomicAdd(&s_hist[lead & 1][tau], times * (units_before(u, T, tau + 1) - units_before(u, T, tau)));
+      pend &= ~same;
     }
   });
   // exclusive prefix over the threads
@@ -183,19 +164,13 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   const PlanAcc all = s_warp[32];
   // first CTA and first warp-tile of every chunk, in warp 0; two chunks per lane
   if (wid == 0) {
-    u32 wt[2], c1[2];
+    u32 wt[2], c1[2], wt_per_cta;
 #pragma unroll
     for (int q = 0; q < 2; ++q) { wt[q] = s_hist[0][2 * lane + q]; c1[q] = s_hist[1][2 * lane + q]; }
-    wt[1] += wt[0]; c1[1] += c1[0];                            // differences -> units, along the chunks
-    u32 sw = wt[1], sc = c1[1];
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const u32 ow = __shfl_up_sync(0xFFFFFFFFu, sw, d), oc = __shfl_up_sync(0xFFFFFFFFu, sc, d);
-      if (lane >= (u32)d) { sw += ow; sc += oc; }
-    }
-    const u32 bw = sw - wt[1], bc = sc - c1[1];
-    wt[0] += bw; wt[1] += bw; c1[0] += bc; c1[1] += bc;
-    const u32 a0 = ceil_div(wt[0], FUSED_WT_PER_CTA) + c1[0], a1 = ceil_div(wt[1], FUSED_WT_PER_CTA) + c1[1];
+    // (gridDim.y: windows of the batch, which are mostly alike)
+    const u32 wt_all = __reduce_add_sync(0xFFFFFFFFu, wt[0] + wt[1]);
+    wt_per_cta = (u64)wt_all * gridDim.y <= FUSED_WARPS ? FUSED_WT_PER_CTA / 2 : FUSED_WT_PER_CTA;
+    const u32 a0 = ceil_div(wt[0], wt_per_cta) + c1[0], a1 = ceil_div(wt[1], wt_per_cta) + c1[1];
     u32 pc = a0 + a1, pw = wt[0] + wt[1];                      // CTAs and warp-tiles of my two chunks
     const u32 oc_ = pc, ow_ = pw;
 #pragma unroll
@@ -212,14 +187,14 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
     u64 t = 0;
     t = lane == T_GROUPS ? all.groups : t; t = lane == T_SLOTS ? all.slots : t; t = lane == T_FCTA ? n_cta : t; t = lane == T_FWT ? n_wt : t;
     t = lane == T_FSUM ? all.units : t; t = lane == T_TILES2 ? all.t2 : t; t = lane == T_TILES3 ? all.t3 : t; t = lane == T_ROWS ? all.rows : t;
-    t = lane == T_CHUNKS ? T : t;
+    t = lane == T_CHUNKS ? T : t; t = lane == T_WT_PER_CTA ? wt_per_cta : t;
     // op counters further apart than 2^31, or more slots than the cap: refuse the window
     u64 failed = (all.slots > slot_cap || all.groups > 0x7FFFFFFFull) ? FAILED_CAPACITY : 0;
     if (!failed && expects) {
       const bool same = lane == T_FAILED || lane >= T_COUNT || t == expected;
       if (!__all_sync(0xFFFFFFFFu, same) || poisoned) { failed = FAILED_EXPECT; if (lane == 0) atomicExch(D.poison, 1u); }
     }
-    if (failed) t = lane == T_CHUNKS ? 1 : 0;
+    if (failed) t = lane == T_CHUNKS || lane == T_WT_PER_CTA ? 1 : 0;
     if (lane == T_FAILED) t = failed;
     if (lane < T_COUNT) { D.totals[lane] = t; D.totals_host[lane] = t; }
     if (lane == 0) {
@@ -233,7 +208,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   each([&](u32 k, u32 ns, u32 n) {
     const u32 c = c_lo + k;
     if (c >= c_hi) return;
-    const PlanAcc it = plan_item(ns, n, T);
+    const PlanAcc it = plan_item(ns, n);
     RangeRow r = {0, 0, 0, n, 0, 0, 0, 0};
     if (!failed) {
       const u32 cls = comm_class(n);
@@ -294,11 +269,12 @@ __device__ __forceinline__ void emit_lists(const WinDesc& D, const Registry& R, 
   }
   // fused classes: the units of this chunk that earlier slices hold, those of my communicator, then where they go
   const auto units_of = [&](u32 c, u32& wt, u32& c1) {
-    const u32 n = R.comm_n[c], cls = comm_class(n), u = cls <= 1 ? chunk_units(D.srow[c].z, n, T, tau) : 0u;
+    const u32 n = R.comm_n[c], cls = comm_class(n), all = cls <= 1 ? fused_units(D.srow[c].z, n) : 0u;
+    const u32 u = units_before(all, T, tau + 1) - units_before(all, T, tau);
     if (cls == 0) wt += u; else c1 += u;
   };
   const uint2 here = D.chunks[tau], next = D.chunks[tau + 1];
-  const u32 wt_base = D.base[B_FWT] + here.y, wt_total = next.y - here.y, cta_base = D.base[B_FCTA] + here.x, n0 = ceil_div(wt_total, FUSED_WT_PER_CTA);
+  const u32 wt_base = D.base[B_FWT] + here.y, wt_total = next.y - here.y, cta_base = D.base[B_FCTA] + here.x, per_cta = (u32)D.totals[T_WT_PER_CTA], n0 = ceil_div(wt_total, per_cta);
   u32 ew = 0, ec = 0;                                          // this thread's share of what lies before
 #pragma unroll 4
   for (u32 k = 0; k < slice * blocks; ++k) units_of(k * EMIT_THREADS + threadIdx.x, ew, ec);
@@ -323,10 +299,10 @@ __device__ __forceinline__ void emit_lists(const WinDesc& D, const Registry& R, 
       const u32 n = R.comm_n[c], cls = comm_class(n);
       const RangeRow row = D.ranges[c];
       const u64 moff = R.comm_moff[c];
-      const u32 S = chunk_len(row.n_seq, T), U = tile_seqs(n), cnt = chunk_size(row.n_seq, T, tau);
-      const u32 sum0 = D.base[B_FSUM] + row.tile0 + tau * ceil_div(S, U);
+      const u32 U = tile_seqs(n), first = units_before(fused_units(row.n_seq, n), T, tau);
+      const u32 sum0 = D.base[B_FSUM] + row.tile0 + first;
       for (u32 k = 0; k < wt + c1; ++k) {
-        const u32 off = tau * S + k * U, len = cnt - k * U < U ? cnt - k * U : U;
+        const u32 off = (first + k) * U, len = min(U, row.n_seq - off);
         if (cls == 0) { WarpTile x; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.row = row; x.moff = moff; L.fwt[at_w++] = x; }
         else { FusedCta x; x.w = blockIdx.y; x.cls = 1; x.c = c; x.seq_off = off; x.count = len; x.sum_idx = sum0 + k; x.wt_first = 0; x.wt_count = 0;
                x.row = row; x.moff = moff; L.fcta[at_c++] = x; }
@@ -338,7 +314,7 @@ __device__ __forceinline__ void emit_lists(const WinDesc& D, const Registry& R, 
   for (u32 j = slice * EMIT_THREADS + threadIdx.x; j < n0; j += slices * EMIT_THREADS) {
     FusedCta x; x.w = blockIdx.y; x.cls = 0; x.c = 0; x.seq_off = 0; x.count = 0; x.sum_idx = 0; x.moff = 0;
     x.row = RangeRow{0, 0, 0, 0, 0, 0, 0, 0};
-    x.wt_first = wt_base + FUSED_WT_PER_CTA * j; x.wt_count = wt_total - FUSED_WT_PER_CTA * j < FUSED_WT_PER_CTA ? wt_total - FUSED_WT_PER_CTA * j : FUSED_WT_PER_CTA;
+    x.wt_first = wt_base + per_cta * j; x.wt_count = min(per_cta, wt_total - per_cta * j);
     L.fcta[cta_base + j] = x;
   }
 }
