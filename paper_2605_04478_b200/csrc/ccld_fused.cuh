@@ -65,6 +65,14 @@ template <class K> __device__ __forceinline__ void median_mad8(const K (&x)[8], 
   *med = m; *mad = pick4(s, k);
 }
 
+// The same for n <= 4. Of three or four members the median is the second smallest, and its neighbour that is nearer is the
+// second smallest deviation after its own; of one or two it is the smallest, whose own deviation is 0.
+__device__ __forceinline__ void median_mad4(const u32 (&x)[4], u32 n, u32* med, u32* mad) {
+  u32 v0 = x[0], v1 = x[1], v2 = x[2], v3 = x[3];
+  cswap(v0, v1); cswap(v2, v3); cswap(v0, v2); cswap(v1, v3); cswap(v1, v2);
+  *med = n > 2 ? v1 : v0; *mad = n > 2 ? min(v1 - v0, v2 - v1) : 0u;
+}
+
 // 1 / x, 1 <= x < 2^64, rounded: Newton's method on the approximate single-precision reciprocal. That is good to about 2^-22
 // with the rounding of its argument, and a step squares the relative error (always towards smaller values): two steps leave
 // the rounding of the last one.
@@ -86,11 +94,10 @@ __device__ __forceinline__ double busbw_fast(double bytes_num, double den, i64 t
   return t > 0 ? bytes_num * rcp_newton((double)t * den) : 0.0;
 }
 
-// Sums v[m] over the warp for m = 0..7 with 9 shuffles; lane l ends up with the total of member
-// m = 4 * bit4(l) + 2 * bit3(l) + bit2(l).
-__device__ __forceinline__ double warp_sum8(double (&v)[8], u32 lane) {
+// Sums v[m] over the warp for m = 0..P-1; lane l ends up with the total of member l / 4 % P. P = 8: 9 shuffles.
+template <int P> __device__ __forceinline__ double warp_sum(double (&v)[P], u32 lane) {
 #pragma unroll
-  for (int w = 4, bit = 16; w >= 1; w >>= 1, bit >>= 1) {
+  for (int w = P / 2, bit = P * 2; w >= 1; w >>= 1, bit >>= 1) {
     const bool hi = (lane & bit) != 0;
 #pragma unroll
     for (int i = 0; i < w; ++i) {
@@ -98,6 +105,7 @@ __device__ __forceinline__ double warp_sum8(double (&v)[8], u32 lane) {
       v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, bit);
     }
   }
+  if (P == 4) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 16);
   v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 2);
   v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 1);
   return v[0];
@@ -203,6 +211,10 @@ __device__ __forceinline__ void flush_counters(const WinDesc& D, const FusedShar
 // What a warp carries from tile to tile.
 struct SmallAcc { u32 complete = 0, barrier = 0, analysed = 0, mismatch = 0, present = 0, flagged = 0; };   // flagged: this lane's kind of vote (lane % 4)
 
+// Up to four ranks a lane holds four positions: with eight, half of them empty, two windows of groups of 4, 4 and 128 took 86 us
+// instead of 75, of 2 and 3 134 instead of 119. (Five to seven of eight are used above.)
+constexpr u32 HALF_N = 4;
+
 // A tile's list entry as one word per lane (16 words), so that the next tile's can wait in a single register.
 static_assert(sizeof(WarpTile) == 64, "an entry is sixteen words");
 __device__ __forceinline__ u32 entry_word(u32 e, u32 w) { return __shfl_sync(FULLM, e, w); }
@@ -215,6 +227,7 @@ __device__ __forceinline__ void ask_indices(const FusedShared& sh, u32 e, u32 la
   const u32 dst = (u32)__cvta_generic_to_shared(slots + lane);
 #pragma unroll
   for (u32 q = 0; q < 8; ++q) {
+    if (q >= HALF_N && n <= HALF_N) break;
     // positions beyond the communicator repeat its first member, which changes no extreme and no comparison
     const u32* src = pm + (u64)(q < n ? q : 0u) * n_seq;
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(dst + q * 128u), "l"(src) : "memory");
@@ -222,42 +235,43 @@ __device__ __forceinline__ void ask_indices(const FusedShared& sh, u32 e, u32 la
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// FULL: eight members. e: the tile's entry, its indices asked for earlier; e_next: the entry of the warp's next tile, if it has
+// P: positions a lane holds, eight or, for communicators of up to four ranks, four. FULL: as many members. e: the tile's entry, its indices asked for earlier; e_next: the entry of the warp's next tile, if it has
 // one. One exposed round trip to memory per tile: times, sizes and op codes are asked for together as soon as the indices
 // are there, the rate columns while the order statistics are worked out, the next tile's indices before any of it.
-template <bool FULL>
-__device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool has_next, TileSum* __restrict__ sums, const Registry& R, const Params& P,
+template <int P, bool FULL>
+__device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool has_next, TileSum* __restrict__ sums, const Registry& R, const Params& Pm,
                                            const DeferList& DL, FusedShared& sh, u32* __restrict__ slots, u32 lane, SmallAcc& acc) {
+  static_assert(P == 8 || (P == 4 && !FULL), "positions");
   const u32 n = FULL ? 8u : entry_word(e, 7), count = entry_word(e, 2);
   const bool active = lane < count;
   const u32* __restrict__ mem = R.members + entry_pair(e, 14);
   const u32 mem_l = lane < n ? __ldg(mem + lane) : 0u;        // lane m holds the rank of position m
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  u32 a[8], d[8];                                             // enter time against base, duration
-  u64 base, gby; u32 gop, idx[8], xmax;
+  u32 a[P], d[P];                                             // enter time against base, duration
+  u64 base, gby; u32 gop, idx[P], xmax;
   bool ok, mm;
   {
     u32 top = 0;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { idx[q] = slots[q * 32 + lane]; top = max(top, idx[q]); }
+    for (int q = 0; q < P; ++q) { idx[q] = slots[q * 32 + lane]; top = max(top, idx[q]); }
     const bool present = top != NONE;                         // a missing member: the group is deferred
 #pragma unroll
-    for (int q = 0; q < 8; ++q) idx[q] = present ? idx[q] : 0u;
+    for (int q = 0; q < P; ++q) idx[q] = present ? idx[q] : 0u;
     if (has_next) ask_indices(sh, e_next, lane, slots);
-    i64 ta[8], tb[8]; u64 by[8]; u32 op[8];
+    i64 ta[P], tb[P]; u64 by[P]; u32 op[P];
     const i64* __restrict__ c_te = ld_volatile(sh.in.te); const i64* __restrict__ c_tx = ld_volatile(sh.in.tx);
     const u64* __restrict__ c_by = ld_volatile(sh.in.by); const u8* __restrict__ c_op = ld_volatile(sh.in.op);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { ta[q] = __ldg(c_te + idx[q]); tb[q] = __ldg(c_tx + idx[q]); }
+    for (int q = 0; q < P; ++q) { ta[q] = __ldg(c_te + idx[q]); tb[q] = __ldg(c_tx + idx[q]); }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { by[q] = __ldg(c_by + idx[q]); op[q] = __ldg(c_op + idx[q]); }
+    for (int q = 0; q < P; ++q) { by[q] = __ldg(c_by + idx[q]); op[q] = __ldg(c_op + idx[q]); }
     // The upper words of a group's times are nearly always the same (they change every 4.3 s): the lower words are the keys
     // then. Otherwise, and for anything irregular, offsets from the first member's enter time - 2^31 decide.
     const u32 h0 = (u32)((u64)ta[0] >> 32);
     u32 x = 0; bool back = false;
     xmax = 0;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < P; ++q) {
       x |= ((u32)((u64)ta[q] >> 32) ^ h0) | ((u32)((u64)tb[q] >> 32) ^ h0);
       a[q] = (u32)ta[q]; d[q] = (u32)tb[q] - (u32)ta[q];
       back = back || (u32)tb[q] < (u32)ta[q];
@@ -270,7 +284,7 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
       u32 hx = 0, neg = 0;
       back = false; xmax = 0;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < P; ++q) {
         const u64 ra = (u64)ta[q] - base, rb = (u64)tb[q] - base;
         a[q] = (u32)ra; d[q] = (u32)rb - (u32)ra; xmax = max(xmax, (u32)rb);
         hx |= (u32)(ra >> 32) | (u32)(rb >> 32);
@@ -283,22 +297,22 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
     gby = by[0]; gop = op[0];
     u32 y = 0;
 #pragma unroll
-    for (int q = 1; q < 8; ++q) y |= ((u32)by[q] ^ (u32)gby) | ((u32)(by[q] >> 32) ^ (u32)(gby >> 32)) | (op[q] ^ gop);
+    for (int q = 1; q < P; ++q) y |= ((u32)by[q] ^ (u32)gby) | ((u32)(by[q] >> 32) ^ (u32)(gby >> 32)) | (op[q] ^ gop);
     mm = y != 0;
   }
   // the rate columns, read only after the order statistics
-  u32 ch[8];
+  u32 ch[P];
   {
     const u32* __restrict__ c_sc = ld_volatile(sh.in.sc); const u32* __restrict__ c_rc = ld_volatile(sh.in.rc);
     if (c_sc != nullptr) {
-      u32 rc[8];
+      u32 rc[P];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) { ch[q] = __ldg(c_sc + idx[q]); rc[q] = __ldg(c_rc + idx[q]); }
+      for (int q = 0; q < P; ++q) { ch[q] = __ldg(c_sc + idx[q]); rc[q] = __ldg(c_rc + idx[q]); }
 #pragma unroll
-      for (int q = 0; q < 8; ++q) ch[q] = max(ch[q], rc[q]);
+      for (int q = 0; q < P; ++q) ch[q] = max(ch[q], rc[q]);
     } else {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) ch[q] = 0;
+      for (int q = 0; q < P; ++q) ch[q] = 0;
     }
   }
   const u32 sum_idx = entry_word(e, 3), seq_off = entry_word(e, 1);      // (every lane takes part in these)
@@ -309,38 +323,38 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
     DL.entries[at] = ((u64)w_idx << 32) | (u64)(group0 + seq_off + lane);
   }
   const u32 b_ok = __ballot_sync(FULLM, gok);
-  const bool barrier = gop == CCLD_OP_ALLREDUCE && gby < P.barrier_bytes;
-  const bool round = gok && !barrier, analysed = round && n >= P.min_group;
+  const bool barrier = gop == CCLD_OP_ALLREDUCE && gby < Pm.barrier_bytes;
+  const bool round = gok && !barrier, analysed = round && n >= Pm.min_group;
   const u32 b_an = __ballot_sync(FULLM, analysed), b_round = __ballot_sync(FULLM, round), b_mm = __ballot_sync(FULLM, gok && mm);
   // ---- extremes and order statistics ----
   u32 emin, emax, tmx, tmn, ms = 0, ds = 0, md = 0, dm = 0;
-  if (FULL) {
+  if constexpr (FULL) {
     // the sorted keys give the extremes and the median (element 3). Below it the deviations L grow downwards, above it R
     // upwards; the lower-median deviation is the third smallest of the two rows, and that is the least of max(L_i, R_j)
     // over i + j = 3: no second sort.
     u32 v[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = a[q];
+    for (int q = 0; q < P; ++q) v[q] = a[q];
     sort8(v);
     emin = v[0]; emax = v[7]; ms = v[3] - emin;
     ds = min(min(v[3] - v[0], v[6] - v[3]), min(max(v[3] - v[2], v[5] - v[3]), max(v[3] - v[1], v[4] - v[3])));
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = d[q];
+    for (int q = 0; q < P; ++q) v[q] = d[q];
     sort8(v);
     tmn = v[0]; tmx = v[7]; md = v[3] - tmn;
     dm = min(min(v[3] - v[0], v[6] - v[3]), min(max(v[3] - v[2], v[5] - v[3]), max(v[3] - v[1], v[4] - v[3])));
   } else {
     emin = a[0]; emax = a[0]; tmx = d[0]; tmn = d[0];
 #pragma unroll
-    for (int q = 1; q < 8; ++q) { emin = min(emin, a[q]); emax = max(emax, a[q]); tmx = max(tmx, d[q]); tmn = min(tmn, d[q]); }
+    for (int q = 1; q < P; ++q) { emin = min(emin, a[q]); emax = max(emax, a[q]); tmx = max(tmx, d[q]); tmn = min(tmn, d[q]); }
     if (b_an != 0) {
-      u32 v[8];
+      u32 v[P];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = q < (int)n ? a[q] - emin : 0xFFFFFFFFu;
-      median_mad8<u32>(v, n, &ms, &ds);
+      for (int q = 0; q < P; ++q) v[q] = q < (int)n ? a[q] - emin : 0xFFFFFFFFu;
+      if constexpr (P == 8) median_mad8<u32>(v, n, &ms, &ds); else median_mad4(v, n, &ms, &ds);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = q < (int)n ? d[q] - tmn : 0xFFFFFFFFu;
-      median_mad8<u32>(v, n, &md, &dm);
+      for (int q = 0; q < P; ++q) v[q] = q < (int)n ? d[q] - tmn : 0xFFFFFFFFu;
+      if constexpr (P == 8) median_mad8<u32>(v, n, &md, &dm); else median_mad4(v, n, &md, &dm);
     }
   }
   if (!analysed) { ms = ds = md = dm = 0; }
@@ -349,13 +363,13 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
   {
     // |x - med| * 1000 > k * MAD in whole numbers: |x - med| > T = floor(k * MAD / 1000), which holds outside
     // [med - T, med + T]; a quotient of 2^32 - 1 or more is never exceeded. One subtraction and one comparison per value.
-    const u64 qs = (u64)ds * P.k_milli / 1000u, qd = (u64)dm * P.k_milli / 1000u;
+    const u64 qs = (u64)ds * Pm.k_milli / 1000u, qd = (u64)dm * Pm.k_milli / 1000u;
     const u32 ts = qs > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qs, td = qd > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qd;
     const u32 los = ms > ts ? ms - ts : 0u, lod = md > td ? md - td : 0u;
     const u32 ws = (ms + ts < ms ? 0xFFFFFFFFu : ms + ts) - los, wd = (md + td < md ? 0xFFFFFFFFu : md + td) - lod;
     const u32 s0 = emin + los, d0 = tmn + lod, sm = emin + ms, dmd = tmn + md;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < P; ++q) {
       u32& f = q < 4 ? f_lo : f_hi;
       const int at = 8 * (q & 3);
       if (a[q] - s0 > ws) f |= (u32)CCLD_F_SKEW_OUT << at;
@@ -365,27 +379,28 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
     }
     if (!FULL) {                                              // positions that do not exist
       f_lo &= n >= 4 ? 0xFFFFFFFFu : (1u << (8 * n)) - 1u;
-      f_hi &= n > 4 ? (n >= 8 ? 0xFFFFFFFFu : (1u << (8 * (n - 4))) - 1u) : 0u;
+      if (P == 8) f_hi &= n > 4 ? (n >= 8 ? 0xFFFFFFFFu : (1u << (8 * (n - 4))) - 1u) : 0u;
     }
     if (!analysed) { f_lo = 0x80808080u; f_hi = 0x80808080u; }
   }
   if (gok) {
     u8* __restrict__ fp = ld_volatile(sh.out.flags) + slot0 + (u64)(seq_off + lane) * n;
     if (FULL && (reinterpret_cast<uintptr_t>(fp) & 7) == 0) *reinterpret_cast<uint2*>(fp) = make_uint2(f_lo, f_hi);
+    else if (P == 4 && n == 4 && (reinterpret_cast<uintptr_t>(fp) & 3) == 0) *reinterpret_cast<u32*>(fp) = f_lo;
     else {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) if (FULL || q < (int)n) fp[q] = (u8)((q < 4 ? f_lo >> (8 * q) : f_hi >> (8 * (q - 4))) & 0xFFu);
+      for (int q = 0; q < P; ++q) if (FULL || q < (int)n) fp[q] = (u8)((q < 4 ? f_lo >> (8 * q) : f_hi >> (8 * (q - 4))) & 0xFFu);
     }
   }
   // ---- votes: the four kinds of outlier as one bit per member's byte, summed over the warp four members at a time (a sum
   // fits its byte); lane 4 m + kind then holds member m's count of its kind and adds it with the warp's one atomic ----
   static_assert(CCLD_F_SKEW_OUT == 1 && CCLD_F_DUR_OUT == 2 && CCLD_F_SKEW_HI == 4 && CCLD_F_DUR_HI == 8, "flag bit layout");
-  const u32 m = lane >> 2, rank_m = __shfl_sync(FULLM, mem_l, m);
+  const u32 m = lane / 4 % P, rank_m = __shfl_sync(FULLM, mem_l, m);
   {
     const u32 one = 0x01010101u;
     u32 mine = 0;
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
+    for (int half = 0; half < P / 4; ++half) {
       const u32 f = gok ? (half ? f_hi : f_lo) : 0u;
       const u32 so = f & one, dq = (f >> 1) & one, sh_ = so & (f >> 2), dh = dq & (f >> 3);
       const u32 v0 = __reduce_add_sync(FULLM, sh_), v1 = __reduce_add_sync(FULLM, so ^ sh_), v2 = __reduce_add_sync(FULLM, dh), v3 = __reduce_add_sync(FULLM, dq ^ dh);
@@ -399,10 +414,10 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
   // ---- positions of the extremes (lowest among equals), ranks the row names ----
   u32 cmx = ch[0];
 #pragma unroll
-  for (int q = 1; q < 8; ++q) cmx = max(cmx, ch[q]);
+  for (int q = 1; q < P; ++q) cmx = max(cmx, ch[q]);
   u32 pmax = 0, pmin = 0, pchg = 0;
 #pragma unroll
-  for (int q = 7; q >= 0; --q) { pmax = d[q] == tmx ? (u32)q : pmax; pmin = d[q] == tmn ? (u32)q : pmin; pchg = ch[q] == cmx ? (u32)q : pchg; }
+  for (int q = P - 1; q >= 0; --q) { pmax = d[q] == tmx ? (u32)q : pmax; pmin = d[q] == tmn ? (u32)q : pmin; pchg = ch[q] == cmx ? (u32)q : pchg; }
   const u32 r_tmin = __shfl_sync(FULLM, mem_l, pmin), r_tmax = __shfl_sync(FULLM, mem_l, pmax), r_chg = __shfl_sync(FULLM, mem_l, pchg);
   // bytes * num / den: for eight members the factors 14/8 and 7/8 are exact; for others one rounding, and the row's value, which
   // is a single quotient, is taken from the product before it
@@ -424,18 +439,18 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
     ld_volatile(sh.out.gbw)[g] = !span ? 0.0 : (FULL ? bn * rcp_newton((double)span) : bnum * rcp_newton((double)span * den));
   }
   // ---- per-member bandwidth, summed over the warp; the Eq. 2 candidate; counts ----
-  double bw[8];
+  double bw[P];
   const double bd = round ? bn : 0.0;
   if (!__any_sync(FULLM, tmn == 0)) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) bw[q] = bd * rcp_u32(d[q]);
+    for (int q = 0; q < P; ++q) bw[q] = bd * rcp_u32(d[q]);
   } else {                                                    // an op of no duration adds nothing
 #pragma unroll
-    for (int q = 0; q < 8; ++q) bw[q] = d[q] != 0 ? bd * rcp_u32(d[q]) : 0.0;
+    for (int q = 0; q < P; ++q) bw[q] = d[q] != 0 ? bd * rcp_u32(d[q]) : 0.0;
   }
-  const double tot = warp_sum8(bw, lane);                     // lane l holds member 4 bit4(l) + 2 bit3(l) + bit2(l)
+  const double tot = warp_sum<P>(bw, lane);                   // lane l holds member m
   const u32 rounds = (u32)__popc(b_round);
-  if ((lane & 3) == 0 && m < n && rounds) { atomicAdd(&R.bw_sum[rank_m], tot); atomicAdd(&R.bw_cnt[rank_m], rounds); }
+  if ((lane & 3) == 0 && lane < 4 * n && rounds) { atomicAdd(&R.bw_sum[rank_m], tot); atomicAdd(&R.bw_cnt[rank_m], rounds); }
   const u32 rng = round ? tmx - tmn : 0u, best = __reduce_max_sync(FULLM, rng);
   const u32 b_best = __ballot_sync(FULLM, round && rng == best);            // ties: the lowest op counter
   const u32 n_ok = (u32)__popc(b_ok), n_an = (u32)__popc(b_an);
@@ -465,8 +480,10 @@ __device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta
   for (u32 i = wid; i < t.wt_count; i += NW) {
     const u32 e_after = entry(i + 2 * NW);
     const bool has_next = i + NW < t.wt_count;
-    if (entry_word(e, 7) == SMALL_N) small_tile<true>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
-    else small_tile<false>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
+    const u32 n = entry_word(e, 7);
+    if (n == SMALL_N) small_tile<8, true>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
+    else if (n > HALF_N) small_tile<8, false>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
+    else small_tile<4, false>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
     e = e_next; e_next = e_after;
   }
   const u32 f_skew = __reduce_add_sync(FULLM, lane & 2 ? 0u : acc.flagged), f_dur = __reduce_add_sync(FULLM, lane & 2 ? acc.flagged : 0u);
