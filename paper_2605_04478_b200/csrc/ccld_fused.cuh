@@ -762,6 +762,19 @@ __device__ __forceinline__ u64 rank_select(const u64 (&x)[DEF_Q], u32 n, u32 k, 
   return __shfl_sync(FULLM, res, src & 31);
 }
 
+// The communicator of group g: the last one whose first group is <= g (communicators without groups share their successor's start).
+// A warp looks at 32 places at a time: three reads one after the other for 2,185 communicators where halving took eleven.
+__device__ __forceinline__ u32 owner_of(const RangeRow* ranges, u32 n_comms, u64 g, u32 lane) {
+  u32 lo = 0, len = n_comms;                                  // it is one of the len communicators from lo on
+  while (len > 1) {
+    const u32 step = (len + 31) / 32, at = lane * step;
+    const u32 b = __ballot_sync(FULLM, at < len && ranges[lo + at].group0 <= g), k = b ? 31u - (u32)__clz(b) : 0u;
+    lo += k * step; len = min(step, len - k * step);
+  }
+  return lo;
+}
+
+// A group set aside is a chain of dependent reads - count, entry, owner, row, record indices, values - on little data.
 __global__ void __launch_bounds__(DEF_WARPS * 32) k_reduce_deferred(const WinDesc* wd, DeferList DL, Registry R, Params P, i64 now) {
   begin_after();
   __shared__ u64 s_key[DEF_WARPS][WARP_N];
@@ -772,12 +785,7 @@ __global__ void __launch_bounds__(DEF_WARPS * 32) k_reduce_deferred(const WinDes
     const u64 ent = DL.entries[e];
     const WinDesc& D = wd[(u32)(ent >> 32)];
     const u64 g = (u32)ent;
-    u32 c;
-    { // owner: the last communicator whose first group is <= g
-      u32 lo = 0, hi = R.n_comms - 1;
-      while (lo < hi) { const u32 mid = (lo + hi + 1) >> 1; if (D.ranges[mid].group0 <= g) lo = mid; else hi = mid - 1; }
-      c = lo;
-    }
+    const u32 c = owner_of(D.ranges, R.n_comms, g, lane);
     const RangeRow row = D.ranges[c];
     const u32 n = row.n, so = (u32)(g - row.group0);
     const u32* mem = R.members + R.comm_moff[c];
