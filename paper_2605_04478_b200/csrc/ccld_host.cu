@@ -430,9 +430,9 @@ int finalize_registry(ccld_ctx* ctx) {
   // The gathers of the small groups are held up by the cache lines an SM can have on their way: no more shared memory than the
   // CTAs need, the rest of the SM's 256 KB is L1. (The other kernels are best off with the driver's own choice.)
   CK(cudaFuncSetAttribute(k_reduce_fused, cudaFuncAttributePreferredSharedMemoryCarveout, FUSED_CARVEOUT));
-  CK(cudaFuncSetAttribute(k_reduce_large<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(4)));
-  CK(cudaFuncSetAttribute(k_reduce_large<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(8)));
-  CK(cudaFuncSetAttribute(k_reduce_large<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)large_smem(16)));
+  CK(cudaFuncSetAttribute(k_reduce_large<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LargeTile<4>::BYTES));
+  CK(cudaFuncSetAttribute(k_reduce_large<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LargeTile<8>::BYTES));
+  CK(cudaFuncSetAttribute(k_reduce_large<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LargeTile<16>::BYTES));
   ctx->finalized = true;
   return CCLD_OK;
 }
@@ -1040,9 +1040,9 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     TimedLaunch tl(ts, 5, st);
     const u32 grid = (u32)(n_list[B_T3] * LARGE_SEQS); TileSum* sums = (TileSum*)(rbase + o_s3);
     const u32* m = ctx->max_large_n;
-    if (m[0]) launch_cluster(on, k_reduce_large<4>, LARGE_SEQS, grid, LQ_THREADS, large_smem(4), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
-    if (m[1]) launch_cluster(on, k_reduce_large<8>, LARGE_SEQS, grid, LQ_THREADS, large_smem(8), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
-    if (m[2]) launch_cluster(on, k_reduce_large<16>, LARGE_SEQS, grid, LQ_THREADS, large_smem(16), d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[0]) launch_cluster(on, k_reduce_large<4>, LARGE_SEQS, grid, LQ_THREADS, LargeTile<4>::BYTES, d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[1]) launch_cluster(on, k_reduce_large<8>, LARGE_SEQS, grid, LQ_THREADS, LargeTile<8>::BYTES, d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
+    if (m[2]) launch_cluster(on, k_reduce_large<16>, LARGE_SEQS, grid, LQ_THREADS, LargeTile<16>::BYTES, d_desc, pl.t3, sums, ctx->reg, ctx->dp, dl_big);
     if (chains.n <= 0) deferred_big(on);
   }
   if (n_list[B_FCTA]) {

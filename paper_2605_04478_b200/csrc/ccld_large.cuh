@@ -7,21 +7,21 @@
 //   gather    CTA c takes an eighth of the members through all eight op counters. Lanes run along the op counter first: the
 //             eight record indices of a member are one 32-byte sector of the member-major permutation, and in a rank-major
 //             upload its eight records are neighbours too, so every gather of a warp fetches whole sectors. Times become 32-bit
-//             keys against the group's first member (enter-time offset, duration) in the CTA's shared memory; extrema, op-set
-//             check and rate column are reduced on the way.
-//   exchange  CTA j takes op counter j: its keys come out of the eight CTAs' shared memory (distributed shared memory, rows of
-//             consecutive members). The bandwidths of the CTA's members over the eight op counters are added up where they
-//             were gathered, so a member costs one atomic per tile; then the op counter's keys take the place of the tile.
+//             keys against the group's first member (enter-time offset, duration), which go straight to the shared memory of CTA j, whose op
+//             counter they belong to; extrema, op-set check and rate column are reduced on the way.
+//   meet      One barrier of the cluster later CTA j has its op counter's keys, and everybody the eight CTAs' extrema. The bandwidths of
+//             a CTA's members over the eight op counters are added up where they were gathered, so a member costs one atomic per tile.
 //   select    medians of both metrics side by side: a histogram of 2,048 bins from the largest key's highest bit down names the
 //             bin of the median, the few keys of that bin are put in a list, and a thread per listed key counts those before
 //             it; then the same for the deviations. Five barriers per median of both metrics.
 //
 // Groups that are not complete and 32-bit clean go to k_reduce_large_deferred (one CTA per listed group, 64-bit, hang alerts).
 //
-// Two kernels did this before: one wrote the keys to memory, the other read them twice and selected with 8-bit digits, every
-// key of a thread looked at in every pass (12 warp instructions per record): 2 x 1,000 groups of 4,096 took 90 + 195 us; this
-// kernel takes 231 (241 with the extremes kept as 64-bit keys while gathering). A CTA lives 35 us, 14 of them in the gather
-// and the rest in the barriers and round trips of the other steps.
+// Two windows of one communicator of 4,096 ranks, 2 x 1,000 groups: 219 us. A CTA lives 35 us: 16 of them in the gather (four round
+// trips to memory, two records per thread each; more do not fit the registers of three CTAs per SM), 10 in the two selections, the rest in
+// barriers, merges and the row. With the keys staged where they were gathered and pulled over by their owners between two
+// barriers, subtracted and stored once more, and lists ordered by two comparisons per pair, it took 229 (2,000 ranks 160 instead of 151, 3,000 199
+// instead of 190); two kernels with the keys in memory between them 285.
 #pragma once
 #include <cooperative_groups.h>
 #include "ccld_device.cuh"
@@ -30,16 +30,22 @@ namespace ccld {
 
 constexpr int LQ_THREADS = 512, LQ_WARPS = LQ_THREADS / 32;
 constexpr u32 LQ_BITS = 11, LQ_BINS = 1u << LQ_BITS;       // bins of a histogram level
-constexpr u32 LQ_LIST = 256;                               // keys a bin may hold to be settled by counting
+constexpr u32 LQ_LIST = 256, LQ_PLACE_BITS = 8;            // keys a bin may hold to be settled by counting; bits of a place in their list
 constexpr u32 LQ_LEVELS = (32 + LQ_BITS - 1) / LQ_BITS;    // after that many levels no bit is undecided
 static_assert(LARGE_SEQS == 8 && LQ_WARPS == 16 && LQ_LIST == LQ_THREADS / 2, "a CTA of the cluster per op counter, eight warps per metric");
-// members of a CTA: at most 64 Q; the padding sets a row's lanes (op counter 0..7, member 0..3) on 32 different banks
-template <int Q> struct LargeTile { static constexpr u32 M = 64 * Q, PITCH = M + 4; };
-inline size_t large_smem(int q) { return (size_t)2 * LARGE_SEQS * (64 * q + 4) * 4; }
+static_assert(LQ_LIST == 1u << LQ_PLACE_BITS && 32 - LQ_BITS + LQ_PLACE_BITS < 32, "what the first level leaves undecided and a place fit a word");
+// A CTA gathers at most M = 64 Q members; the padding sets a row's lanes (op counter 0..7, member 0..3) on 32 different banks. Dynamic
+// shared memory: the keys of my op counter (pairs), the durations of my members, and the histograms, which take the
+// durations' place where that is large enough.
+template <int Q> struct LargeTile {
+  static constexpr bool STAGED = Q < 16;                   // 33 KB more per CTA would leave L1 28 KB: 289 us instead of 232 on 8,000 members
+  static constexpr u32 M = 64 * Q, PITCH = M + 4, KEYS = LARGE_SEQS * M * 8, DURS = STAGED ? LARGE_SEQS * PITCH * 4 : 0, HIST = 2 * LQ_BINS * 4;
+  static constexpr bool OVERLAY = DURS >= HIST;
+  static constexpr u32 BYTES = KEYS + DURS + (OVERLAY ? 0 : HIST);
+};
 
 struct LargePick { u32 lo, sh, k, cnt; };                  // the k-th of cnt keys in [lo, lo + 2^sh)
 struct LargeShared {
-  u32 hist[2][LQ_BINS];
   uint4 list[2][LQ_LIST / 4];
   MidPart part[LQ_WARPS][LARGE_SEQS], mine[LARGE_SEQS], group;
   LargePick pick[LQ_LEVELS][2];                            // [level][metric]
@@ -49,10 +55,10 @@ struct LargeShared {
   double bd[LARGE_SEQS];                                   // bytes * factor of an op counter that is a round, else 0
 };
 
-// The k-th smallest (0-based) of |a[i] - ma| and of |d[i] - md| over the n keys in shared memory. ba, bd: the largest of them.
-// All threads call it; the histograms are zero on entry and on return.
-template <int Q> __device__ __forceinline__ void large_pick(const u32* __restrict__ s_a, const u32* __restrict__ s_d, u32 n, u32 ma, u32 md, u32 k, u32 ba, u32 bd,
-                                                            LargeShared& sh, u32* ra, u32* rd) {
+// The k-th smallest (0-based) of |a - ma| and of |d - md| over the n pairs in shared memory. ba, bd: the largest of them.
+// All threads call it; the histograms ([2][LQ_BINS]) are zero on entry and on return.
+template <int Q> __device__ __forceinline__ void large_pick(const uint2* __restrict__ keys, u32 n, u32 ma, u32 md, u32 k, u32 ba, u32 bd,
+                                                            u32* hist, LargeShared& sh, u32* ra, u32* rd) {
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5, x = wid >> 3;             // eight warps scan a metric's bins
   u32 lo0 = 0, lo1 = 0, w0 = 32 - (u32)__clz(ba | 1u), w1 = 32 - (u32)__clz(bd | 1u);  // undecided bits
   u32 k0 = k, k1 = k, c0 = NONE, c1 = NONE;
@@ -66,22 +72,24 @@ template <int Q> __device__ __forceinline__ void large_pick(const u32* __restric
       for (int q = 0; q < Q; ++q) {
         const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
         if (i >= n) break;
-        atomicAdd(&sh.hist[0][__usad(s_a[i], ma, 0u) >> n0], 1u);
-        atomicAdd(&sh.hist[1][__usad(s_d[i], md, 0u) >> n1], 1u);
+        const uint2 y = keys[i];
+        atomicAdd(&hist[__usad(y.x, ma, 0u) >> n0], 1u);
+        atomicAdd(&hist[LQ_BINS + (__usad(y.y, md, 0u) >> n1)], 1u);
       }
     } else {
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
         if (i >= n) break;
-        const u32 a = __usad(s_a[i], ma, 0u) - lo0, d = __usad(s_d[i], md, 0u) - lo1;
-        if (act0 && (a >> w0) == 0) atomicAdd(&sh.hist[0][a >> n0], 1u);      // (w < 32 after the first level)
-        if (act1 && (d >> w1) == 0) atomicAdd(&sh.hist[1][d >> n1], 1u);
+        const uint2 y = keys[i];
+        const u32 a = __usad(y.x, ma, 0u) - lo0, d = __usad(y.y, md, 0u) - lo1;
+        if (act0 && (a >> w0) == 0) atomicAdd(&hist[a >> n0], 1u);            // (w < 32 after the first level)
+        if (act1 && (d >> w1) == 0) atomicAdd(&hist[LQ_BINS + (d >> n1)], 1u);
       }
     }
     __syncthreads();
     u32 loc[8], sum = 0;
-    uint4* h = reinterpret_cast<uint4*>(&sh.hist[x][(wid & 7) * 256 + lane * 8]);
+    uint4* h = reinterpret_cast<uint4*>(&hist[x * LQ_BINS + (wid & 7) * 256 + lane * 8]);
     { const uint4 a = h[0], b = h[1]; loc[0] = a.x; loc[1] = a.y; loc[2] = a.z; loc[3] = a.w; loc[4] = b.x; loc[5] = b.y; loc[6] = b.z; loc[7] = b.w; }
     h[0] = make_uint4(0, 0, 0, 0); h[1] = make_uint4(0, 0, 0, 0);
 #pragma unroll
@@ -111,33 +119,32 @@ template <int Q> __device__ __forceinline__ void large_pick(const u32* __restric
     lo0 = p0.lo; w0 = p0.sh; k0 = p0.k; c0 = p0.cnt; lo1 = p1.lo; w1 = p1.sh; k1 = p1.k; c1 = p1.cnt;
   }
   if (w0 | w1) {
-    // the keys of the bins go into lists; a list's places beyond its end hold the largest key
+    // the keys of the bins go into lists, each with its place below its undecided bits, so that no two are equal and one comparison
+    // orders them; a list's places beyond its end hold the largest word
     u32* const l0 = reinterpret_cast<u32*>(sh.list[0]); u32* const l1 = reinterpret_cast<u32*>(sh.list[1]);
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
       if (i >= n) break;
-      const u32 a = __usad(s_a[i], ma, 0u) - lo0, d = __usad(s_d[i], md, 0u) - lo1;
-      if (w0 && (a >> w0) == 0) { const u32 at = atomicAdd(&sh.n_list[0], 1u); if (at < LQ_LIST) l0[at] = a; }    // c0 <= LQ_LIST of them
-      if (w1 && (d >> w1) == 0) { const u32 at = atomicAdd(&sh.n_list[1], 1u); if (at < LQ_LIST) l1[at] = d; }
+      const uint2 y = keys[i];
+      const u32 a = __usad(y.x, ma, 0u) - lo0, d = __usad(y.y, md, 0u) - lo1;
+      if (w0 && (a >> w0) == 0) { const u32 at = atomicAdd(&sh.n_list[0], 1u); if (at < LQ_LIST) l0[at] = a << LQ_PLACE_BITS | at; }    // c0 <= LQ_LIST of them
+      if (w1 && (d >> w1) == 0) { const u32 at = atomicAdd(&sh.n_list[1], 1u); if (at < LQ_LIST) l1[at] = d << LQ_PLACE_BITS | at; }
     }
     __syncthreads();
     {
-      // a thread per listed key counts those before it (ties by place); the key with k before it is the one
+      // a thread per listed key counts those before it; the key with k before it is the one
       const u32 c = x ? c1 : c0, w = x ? w1 : w0, kr = x ? k1 : k0, i = (wid & 7) * 32 + lane, c4 = min((c + 3) / 4, LQ_LIST / 4);
       if (w == 0) { if (i == 0) sh.res[x] = x ? lo1 : lo0; }
       else if ((wid & 7) * 32 < c) {
-        const u32* l = x ? l1 : l0;
-        const u32 v = i < c ? l[i] : NONE;
+        const u32 v = (x ? l1 : l0)[i];
         u32 before = 0;
 #pragma unroll 4
         for (u32 g = 0; g < c4; ++g) {
           const uint4 y = sh.list[x][g];
-          const u32 j = 4 * g;
-          before += (y.x < v || (y.x == v && j < i)) ? 1u : 0u; before += (y.y < v || (y.y == v && j + 1 < i)) ? 1u : 0u;
-          before += (y.z < v || (y.z == v && j + 2 < i)) ? 1u : 0u; before += (y.w < v || (y.w == v && j + 3 < i)) ? 1u : 0u;
+          before += y.x < v ? 1u : 0u; before += y.y < v ? 1u : 0u; before += y.z < v ? 1u : 0u; before += y.w < v ? 1u : 0u;
         }
-        if (i < c && before == kr) sh.res[x] = (x ? lo1 : lo0) + v;
+        if (i < c && before == kr) sh.res[x] = (x ? lo1 : lo0) + (v >> LQ_PLACE_BITS);
       }
     }
     __syncthreads();
@@ -148,29 +155,44 @@ template <int Q> __device__ __forceinline__ void large_pick(const u32* __restric
   *ra = lo0; *rd = lo1;
 }
 
-// CTAs per SM, in ns per op counter of one window of 4 M records, two against three: 2,049 to 4,096 members 138 against 129 (3,000)
-// and 169 against 166 (4,096), although three leave 40 registers and spill 120 bytes; above 4,096 two are what shared memory holds.
-// Up to 2,048 members it is two, where three would take 67 against 73 (1,100), 74 against 82 (1,500) and 90 against 95 (2,048).
+// The cluster's barrier in two halves; every thread of every CTA takes part in each.
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// A pair into the shared memory of CTA `cta` of the cluster, at the place that p is in mine.
+__device__ __forceinline__ u32 cluster_address(const void* p, u32 cta) {
+  u32 r; asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((u32)__cvta_generic_to_shared(p)), "r"(cta)); return r;
+}
+__device__ __forceinline__ void cluster_store(u32 address, u32 a, u32 b) { asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" :: "r"(address), "r"(a), "r"(b) : "memory"); }
+
+// The duration of the pair that CTA `cta` keeps at the place of p.
+__device__ __forceinline__ u32 cluster_duration(const uint2* p, u32 cta) {
+  u32 d; asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(d) : "r"(cluster_address(p, cta) + 4) : "memory"); return d;
+}
+
 template <int Q>
 __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(const WinDesc* wd, const Tile* tiles,
     TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
   begin_after();
-  extern __shared__ __align__(16) u32 large_keys[];        // [metric][op counter][member of mine], later [metric][member]: my op counter
+  extern __shared__ __align__(16) unsigned char large_raw[];
   __shared__ __align__(16) LargeShared sh;
   namespace cg = cooperative_groups;
   const Tile t = tiles[blockIdx.x / LARGE_SEQS];
   const u32 n = t.row.n;
   if (t.count == 0 || (n <= 2048 ? 4 : (n <= 4096 ? 8 : 16)) != Q) return;     // no work, or another instance's: the same in the whole cluster
-  cg::cluster_group cluster = cg::this_cluster();
-  constexpr u32 PITCH = LargeTile<Q>::PITCH;
+  cluster_arrive();                                         // waited for before anything is stored elsewhere: the others have begun
+  using L = LargeTile<Q>;
+  constexpr u32 PITCH = L::PITCH;
   const u32 me = blockIdx.x % LARGE_SEQS;                   // my eighth of the members, and my op counter
   const WinDesc& D = wd[t.w];
   const RangeRow& row = t.row;
   const u32* __restrict__ mem = R.members + t.moff;
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const u32 M = (n + LARGE_SEQS - 1) / LARGE_SEQS, m0 = me * M, m_cnt = m0 >= n ? 0u : min(M, n - m0);
-  u32* __restrict__ k_a = large_keys; u32* __restrict__ k_d = large_keys + LARGE_SEQS * PITCH;
-  for (u32 i = threadIdx.x; i < 2 * LQ_BINS / 4; i += LQ_THREADS) reinterpret_cast<uint4*>(&sh.hist[0][0])[i] = make_uint4(0, 0, 0, 0);
+  uint2* const keys = reinterpret_cast<uint2*>(large_raw);                      // [member] enter time against base, duration: my op counter
+  u32* const k_d = reinterpret_cast<u32*>(large_raw + L::KEYS);                 // [op counter][member of mine] durations
+  u32* const hist = L::OVERLAY ? k_d : reinterpret_cast<u32*>(large_raw + L::KEYS + L::DURS);
+  const auto clear_hist = [&] { for (u32 i = threadIdx.x; i < 2 * LQ_BINS / 4; i += LQ_THREADS) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0, 0, 0, 0); };
+  if (!L::OVERLAY) clear_hist();
   if (threadIdx.x < 2 * LQ_LIST / 4) (&sh.list[0][0])[threadIdx.x] = make_uint4(NONE, NONE, NONE, NONE);
   if (threadIdx.x < 2) sh.n_list[threadIdx.x] = 0;
   if (threadIdx.x == 0) { sh.n_fs = 0; sh.n_fd = 0; }
@@ -182,6 +204,7 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
     const i64* __restrict__ c_te = D.t_enter; const i64* __restrict__ c_tx = D.t_exit;
     const u64* __restrict__ c_by = D.bytes; const u8* __restrict__ c_op = D.op;
     const u32* __restrict__ c_sc = D.send_chg; const u32* __restrict__ c_rc = D.recv_chg;
+    const u32 theirs = cluster_address(keys + m0, j);       // where CTA j keeps my members' keys
     MidTrack x;
     u32 idx[Q];
     const u32 i0 = jv ? *perm : NONE;
@@ -190,10 +213,8 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
     i64 te0 = 0; u64 by0 = 0; u32 op0 = 0;
     if (i0 != NONE) { te0 = __ldg(c_te + i0); by0 = __ldg(c_by + i0); op0 = __ldg(c_op + i0); } else x.bits = 1;
     const u64 base = (u64)te0 - 0x80000000ull;
-    // Records in flight per thread. Four spill at 40 registers: 146 and 185 ns per op counter of 3,000 and 4,096 members against 129
-    // and 166. At 64 registers they make no difference above 4,096 (266 and 264 ns at 8,192) and little below 2,049 (70.5 against 73
-    // ns at 1,100, 92.5 against 95 at 2,048), where it is two.
-    constexpr int STEP = Q == 16 ? 4 : 2;
+    cluster_wait();
+    constexpr int STEP = Q == 16 ? 4 : 2;                   // records in flight per thread
 #pragma unroll
     for (int q0 = 0; q0 < Q; q0 += STEP) {
       i64 ta[STEP], tb[STEP]; u64 by[STEP]; u32 op[STEP], ch[STEP];
@@ -215,8 +236,9 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
           if (((ra | rb) >> 32) != 0 || (ta[u] | tb[u]) < 0 || b < a) x.bits |= 1;       // beyond 32 bits, negative or in flight, exit before enter
           if (op[u] != op0 || by[u] != by0) x.bits |= 2;
           x.see(p, a, b, d, ch[u]);
+          cluster_store(theirs + m * 8, a, d);
         }
-        k_a[j * PITCH + m] = a; k_d[j * PITCH + m] = d;
+        if (L::STAGED) k_d[j * PITCH + m] = d;
       }
     }
     MidPart mine = x.part();
@@ -231,23 +253,10 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
     for (int h = 1; h < LQ_WARPS; h <<= 1) mid_merge(x, mid_shfl_xor(x, h));
     if (lane == 0) sh.mine[wid] = x;
   }
-  cluster.sync();
-  // ---- exchange: my group's keys come in; op counter j's extrema by warp j ----
-  u32 va[Q], vd[Q];
-  const u32 src = wid & 7, mm0 = (wid >> 3) * 32 + lane;    // my keys: members mm0, mm0 + 64, ... of CTA src
-  const u32 s_cnt = src * M >= n ? 0u : min(M, n - src * M);
-  {
-    const u32* r_a = cluster.map_shared_rank(k_a, src) + me * PITCH; const u32* r_d = r_a + LARGE_SEQS * PITCH;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const u32 m = mm0 + 64u * (u32)q;
-      const bool in = m < s_cnt;
-      va[q] = in ? r_a[m] : 0u; vd[q] = in ? r_d[m] : 0u;
-    }
-  }
-  if (wid < LARGE_SEQS) {
+  cluster_arrive(); cluster_wait();                         // all keys and parts of the cluster are where they belong
+  if (wid < LARGE_SEQS) {                                   // op counter j's extrema by warp j
     const u32 j = wid;
-    MidPart x = *cluster.map_shared_rank(&sh.mine[j], lane & 7);
+    MidPart x = *cg::this_cluster().map_shared_rank(&sh.mine[j], lane & 7);
 #pragma unroll
     for (int h = 1; h < (int)LARGE_SEQS; h <<= 1) mid_merge(x, mid_shfl_xor(x, h));
     if (lane == 0) {
@@ -263,6 +272,7 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
     }
   }
   __syncthreads();
+  if (L::STAGED) cluster_arrive();                          // I read nobody's shared memory any more; waited for at the end
   // ---- bandwidth of my members over the tile's op counters, where they were gathered ----
   u32 rounds = 0;
 #pragma unroll
@@ -270,16 +280,16 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
   if (rounds) {
     for (u32 m = threadIdx.x; m < m_cnt; m += LQ_THREADS) {
       double v = 0.0;
+      u32 d[LARGE_SEQS];
 #pragma unroll
-      for (u32 j = 0; j < LARGE_SEQS; ++j) {
-        const u32 d = k_d[j * PITCH + m];
-        if (d != 0) v += sh.bd[j] * rcp_u32(d);
-      }
+      for (u32 j = 0; j < LARGE_SEQS; ++j) d[j] = L::STAGED ? k_d[j * PITCH + m] : cluster_duration(keys + m0 + m, j);
+#pragma unroll
+      for (u32 j = 0; j < LARGE_SEQS; ++j) if (d[j] != 0 && sh.bd[j] != 0.0) v += sh.bd[j] * rcp_u32(d[j]);
       const u32 rank = __ldg(mem + m0 + m);
       atomicAdd(&R.bw_sum[rank], v); atomicAdd(&R.bw_cnt[rank], rounds);
     }
   }
-  cluster.sync();                                           // everybody has read what it needs from everybody's shared memory
+  if (!L::STAGED) cluster_arrive();
   // ---- my group ----
   const u32 emin = ~sh.group.n_emin, emax = sh.group.emax, tmx = (u32)(sh.group.kmax >> 32), tmn = (u32)(~sh.group.n_kmin >> 32);
   const u32 so = t.seq_off + me;
@@ -288,26 +298,21 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
   if (gok) {                                                // the same in the whole CTA
     u8* __restrict__ fp = D.flags + row.slot0 + (u64)so * n;
     if (analysed) {
-      u32* __restrict__ s_a = large_keys; u32* __restrict__ s_d = large_keys + n;
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const u32 m = mm0 + 64u * (u32)q;
-        if (m < s_cnt) { s_a[src * M + m] = va[q] - emin; s_d[src * M + m] = vd[q] - tmn; }
-      }
-      __syncthreads();
+      if (L::OVERLAY) { __syncthreads(); clear_hist(); __syncthreads(); }
       const u32 k = (n - 1) >> 1, ba = emax - emin, bd = tmx - tmn;
-      large_pick<Q>(s_a, s_d, n, 0u, 0u, k, ba, bd, sh, &ms, &md);
-      large_pick<Q>(s_a, s_d, n, ms, md, k, max(ms, ba - ms), max(md, bd - md), sh, &ds, &dm);
+      large_pick<Q>(keys, n, emin, tmn, k, ba, bd, hist, sh, &ms, &md);
+      large_pick<Q>(keys, n, emin + ms, tmn + md, k, max(ms, ba - ms), max(md, bd - md), hist, sh, &ds, &dm);
       // |x - med| * 1000 > k * MAD in whole numbers: |x - med| > floor(k * MAD / 1000); a quotient of 2^32 - 1 or more is never exceeded
       const u64 qs = (u64)ds * P.k_milli / 1000u, qd = (u64)dm * P.k_milli / 1000u;
       const u32 ts = qs > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qs, td = qd > 0xFFFFFFFFull ? 0xFFFFFFFFu : (u32)qd;
+      const u32 ca = emin + ms, cd = tmn + md;
       u32 n_fs = 0, n_fd = 0;
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         const u32 i = threadIdx.x + (u32)q * LQ_THREADS;
         if (i >= n) break;
-        const u32 a = s_a[i], d = s_d[i];
-        const bool os = __usad(a, ms, 0u) > ts, od = __usad(d, md, 0u) > td, hs = a > ms, hd = d > md;
+        const uint2 y = keys[i];
+        const bool os = __usad(y.x, ca, 0u) > ts, od = __usad(y.y, cd, 0u) > td, hs = y.x > ca, hd = y.y > cd;
         fp[i] = (u8)((os ? CCLD_F_SKEW_OUT : 0) | (od ? CCLD_F_DUR_OUT : 0) | (hs ? CCLD_F_SKEW_HI : 0) | (hd ? CCLD_F_DUR_HI : 0));
         if (os) { ++n_fs; atomicAdd(&R.votes[(u64)mem[i] * 4 + (hs ? 0 : 1)], 1u); }
         if (od) { ++n_fd; atomicAdd(&R.votes[(u64)mem[i] * 4 + (hd ? 2 : 3)], 1u); }
@@ -351,6 +356,7 @@ __global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(con
       sums[blockIdx.x / LARGE_SEQS] = ts;
     }
   }
+  cluster_wait();                                           // my shared memory stays until nobody reads it any more
 }
 
 // ------------------------------------------------------------------------------------------------
