@@ -160,10 +160,27 @@ __device__ __forceinline__ void sub_stats(u32 (&v)[8], u32 n, u32 s, u32 lane, u
   *mn = __shfl_sync(0xFFFFFFFFu, v[0], first);
   *mx = __shfl_sync(0xFFFFFFFFu, FULL ? v[7] : pick8(v, (n - 1) & 7), first | ((n - 1) >> 3));
   const u32 m = __shfl_sync(0xFFFFFFFFu, FULL ? v[7] : pick8(v, k & 7), first | (k >> 3));         // full: k = 4 L - 1
+  *med = m;
+  if constexpr (FULL) {
+    // Below the median (element k) the deviations grow downwards, above it upwards. The k + 1 smallest are those of some p .. p + k, p <= k, so
+    // the largest of them is the least of max(med - key[p], key[p + k] - med): no second merge. Element p + k = p + 4 L - 1 is one register
+    // down in lane s + L / 2, and the last one of the lane before it for register 0.
+    u32 best = 0xFFFFFFFFu;
 #pragma unroll
-  for (int r = 0; r < 8; ++r) v[r] = (FULL || s * 8 + r < n) ? key_absdiff(v[r], m) : 0xFFFFFFFFu;   // falls to 0 at k, then rises
-  sub_merge<L, u32>(v, s);
-  *med = m; *mad = __shfl_sync(0xFFFFFFFFu, FULL ? v[7] : pick8(v, k & 7), first | (k >> 3));
+    for (int r = 0; r < 8; ++r) {
+      const u32 o = r ? __shfl_xor_sync(0xFFFFFFFFu, v[r ? r - 1 : 0], L / 2) : __shfl_sync(0xFFFFFFFFu, v[7], first + ((s + L / 2 - 1) & (L - 1)));
+      best = min(best, max(m - v[r], o - m));
+    }
+    if (s >= L / 2) best = 0xFFFFFFFFu;
+#pragma unroll
+    for (int h = 1; h < L; h <<= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, h));
+    *mad = best;
+  } else {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = s * 8 + r < n ? key_absdiff(v[r], m) : 0xFFFFFFFFu;   // falls to 0 at k, then rises
+    sub_merge<L, u32>(v, s);
+    *mad = __shfl_sync(0xFFFFFFFFu, pick8(v, k & 7), first | (k >> 3));
+  }
 }
 
 enum { SC_COMP = 0, SC_INC, SC_BAR, SC_AN, SC_MIS, SC_PRES, SC_FS, SC_FD, SC_COUNT };
