@@ -94,7 +94,10 @@ constexpr int N_CLASSES = 4;           // reduction code paths: n <= 8, <= 128, 
 // stretch of every rank's records - run together and share the fetched sectors in L2. A communicator's work units are spread evenly
 // over the chunks (units_before), so that chunks are stretches of time for all communicators and yet every unit but a communicator's last one is full:
 // chunks cut at op counters of their own left a warp-tile 22 or 29 of 32 op counters for 200, 600 and 1,000 per window.
-constexpr u32 CHUNK_REF = 96;          // op counters per chunk of the busiest communicator of a window
+// A chunk of the busiest communicator is one unit long: what the families share then stays in L2 however many ranks there are.
+// k_reduce_fused with 96, 64, 32: twelve windows of 4,096 ranks 556, 549, 540 us; one of 16,384 ranks (the larger communicators beside it)
+// 401, 382, 361; smaller jobs alike. With 16 the lists take 7 us longer to write and nothing is gained.
+constexpr u32 CHUNK_REF = 32;          // op counters per chunk of the busiest communicator of a window
 constexpr u32 CHUNK_MAX = 64;          // at most this many chunks per window (longer chunks beyond)
 enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS, T_FAILED, T_CHUNKS, T_WT_PER_CTA, T_COUNT = 12 };
 constexpr u64 FAILED_CAPACITY = 1, FAILED_EXPECT = 2;      // T_FAILED: the window needs too many slots / its layout is not the expected one
