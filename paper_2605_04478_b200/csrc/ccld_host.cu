@@ -837,8 +837,8 @@ int ccld_reset(ccld_ctx* ctx) try {
   ctx->pending.clear();
   for (auto& kv : ctx->windows) drop_results(kv.second);
   if (ctx->finalized) {
-    CK(cudaMemsetAsync((char*)ctx->reg_blk.p + ctx->stats_off, 0, ctx->stats_bytes, ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_poison, 0, 4, ctx->stream));
+    char* const from = (char*)ctx->reg_blk.p + ctx->stats_off;          // the statistics and, behind them, the flag
+    CK(cudaMemsetAsync(from, 0, (char*)(ctx->d_poison + 1) - from, ctx->stream));
   }
   return CCLD_OK;
 } CAUGHT
