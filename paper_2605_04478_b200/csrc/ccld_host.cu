@@ -933,7 +933,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   WinDesc* d_desc = (WinDesc*)(pbase + o_desc);
   TimerSlot* ts = timer_begin(ctx);
   const u32 layout_threads = nc <= 128 ? 128 : (nc <= 256 ? 256 : (nc <= 512 ? 512 : LAYOUT_THREADS));
-  auto start_plan = [&](u32 fill_ctas) -> cudaError_t {    // uploads the descriptors, sets the start values, runs the range pass and the layout
+  auto start_plan = [&](bool fill, u32 fill_ctas) -> cudaError_t {        // uploads the descriptors, sets the start values, runs the range pass and the layout
     BeginArgs ba;
     ba.desc_host = (const u32*)h_up; ba.desc = (u32*)(pbase + o_desc); ba.desc_words = up_bytes / 4;
     ba.rmin = (u32*)(pbase + o_rmin); ba.n_rmin = (u64)B * nc; ba.zero = (u32*)(pbase + o_zero); ba.n_zero = (o_zero_end - o_zero) / 4;
@@ -944,15 +944,15 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
       const u64 want = 32ull * ctx->n_sms;
       const u32 per = (u32)std::min<u64>(RANGE_BLOCKS_MAX, std::max<u64>(1, cta * B / want));
       TimedLaunch tl(ts, 0, st);
-      launch(st, k_seq_range, dim3((u32)((cta + per - 1) / per), B), REC_THREADS, range_smem_bytes(nc), d_desc, ctx->reg, per);
+      launch(st, k_seq_range, dim3((u32)((cta + per - 1) / per), B), REC_THREADS, range_smem_bytes(nc), d_desc, ctx->reg, per, fill);
     }
-    { TimedLaunch tl(ts, 1, st); launch(st, k_layout, dim3(1 + fill_ctas, B), layout_threads, 0, d_desc, ctx->reg, fill_ctas != 0); }
+    { TimedLaunch tl(ts, 1, st); launch(st, k_layout, dim3(1 + fill_ctas, B), layout_threads, 0, d_desc, ctx->reg); }
     return cudaGetLastError();
   };
   const u64* tot = nullptr;                                // [B][T_COUNT] totals the results are sized from
   std::vector<u64> found;
   if (!expect) {
-    CK(start_plan(0));
+    CK(start_plan(false, 0));
     CK(cudaStreamSynchronize(st));
     found.assign(pbatch.h_tot(), pbatch.h_tot() + (size_t)B * T_COUNT);
     tot = found.data();
@@ -998,10 +998,12 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     d.tsum[0] = (TileSum*)(rbase + o_fsum) + d.base[B_FSUM]; d.tsum[1] = (TileSum*)(rbase + o_s2) + d.base[B_T2]; d.tsum[2] = (TileSum*)(rbase + o_s3) + d.base[B_T3];
   }
   if (expect) {
-    // Descriptors already complete: nothing was waited for, and the slot table is filled beside the layout's one CTA per
-    // window. Two CTAs per SM share the filling.
+    // Descriptors already complete: nothing was waited for. What fills in the time of the layout's one CTA per window is filled
+    // beside it, two CTAs per SM together; a larger table under the range pass, which has issue slots and not memory for
+    // its limit (twelve windows of 4,096 ranks, 49 M slots: 141 us for both kernels instead of 151; one window of 16.4 M: 70 instead of 65).
+    const bool under_range = cta > 0 && total_slots > FILL_BESIDE;
     const u64 want = (max_slots + 16ull * layout_threads - 1) / (16ull * layout_threads);
-    CK(start_plan((u32)std::max<u64>(1, std::min<u64>(want, 2ull * (LAYOUT_THREADS / layout_threads) * ctx->n_sms / B))));
+    CK(start_plan(under_range, under_range ? 0u : (u32)std::max<u64>(1, std::min<u64>(want, 2ull * (LAYOUT_THREADS / layout_threads) * ctx->n_sms / B))));
   } else {
     CK(cudaMemcpyAsync(d_desc, hd, B * sizeof(WinDesc), cudaMemcpyHostToDevice, st));
     if (total_slots) CK(cudaMemsetAsync(rbase + o_perm, 0xFF, total_slots * 4, st));

@@ -141,7 +141,9 @@ __device__ __forceinline__ u32 first_left(const u32 (&cid)[REC_RUN], u32 left) {
   return (b & 1u) ? y1 : y0;
 }
 
-__global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Registry R, u32 blocks_per_cta) {
+// fill: whether the slot table, sized from what the host expects, is to be set to NONE as well. The stores run under the pass,
+// which issues instructions most of the time (FILL_BESIDE).
+__global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Registry R, u32 blocks_per_cta, int fill) {
   begin_after();
   extern __shared__ u32 s_dyn[];
   u32* const s_mn = R.n_comms <= RANGE_DIRECT ? s_dyn : nullptr;
@@ -150,6 +152,7 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
   const u64 n_rec = D.n_rec; const u32* const c_comm = D.comm; const u32* const c_seq = D.seq;
   if ((u64)blockIdx.x * blocks_per_cta * REC_PER_CTA >= n_rec) return;
   const u32 lane = threadIdx.x & 31;
+  if (fill) fill_slots(D.perm, D.n_slots, blockIdx.x, (u32)((n_rec + blocks_per_cta * REC_PER_CTA - 1) / (blocks_per_cta * REC_PER_CTA)));
   if (s_mn != nullptr) {
     for (u32 c = threadIdx.x; c < R.n_comms; c += REC_THREADS) { s_mn[c] = NONE; s_mx[c] = 0; }
     __syncthreads();

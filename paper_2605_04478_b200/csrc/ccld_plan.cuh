@@ -4,7 +4,7 @@
 //   k_begin   the batch's descriptors move from pinned host memory to the device and its op-counter ranges, counters and list
 //             lengths get their start values
 //   k_layout  one CTA per window: prefix sums over the communicators (groups, slots, rows, work units) and the start of every
-//             chunk of the work lists; the other CTAs of the launch fill the slot table of a batch that does not wait
+//             chunk of the work lists; the other CTAs of the launch, if any, fill the slot table of a batch that does not wait
 //   emit_lists  a CTA per (window, chunk, 256 communicators) writes their part of the chunk's work lists, beside the scatter
 //             pass and in its launch (ccld_kernels.cuh)
 //
@@ -48,6 +48,17 @@ __device__ __forceinline__ u32 plan_nseq(const WinDesc& D, u32 c) { return range
 // Work units (warp-tiles of class 0, CTA tiles of class 1) of a communicator; 0 for other classes.
 __device__ __forceinline__ u32 fused_units(u32 ns, u32 n) { return comm_class(n) > 1 ? 0u : ceil_div(ns, tile_seqs(n)); }
 
+// CTA `cta` of `ctas` sets its part of the slot table to NONE.
+constexpr u64 FILL_BESIDE = 24ull << 20;                // slots of a batch that are filled beside the layout, at most
+__device__ __forceinline__ void fill_slots(u32* perm, u64 n, u32 cta, u32 ctas) {
+  const u64 head = min(n, (u64)((16 - ((uintptr_t)perm & 15)) & 15) / 4), n4 = (n - head) / 4, per = (n4 + ctas - 1) / ctas;
+  uint4* p4 = reinterpret_cast<uint4*>(perm + head);
+  for (u64 i = cta * per + threadIdx.x, end = min(n4, (cta + 1) * per); i < end; i += blockDim.x) p4[i] = make_uint4(NONE, NONE, NONE, NONE);
+  if (cta != 0) return;
+  if (threadIdx.x < head) perm[threadIdx.x] = NONE;
+  if (threadIdx.x < n - head - n4 * 4) perm[head + n4 * 4 + threadIdx.x] = NONE;
+}
+
 struct PlanAcc { u64 groups, slots; u32 rows, units, t2, t3; };
 __device__ __forceinline__ PlanAcc plan_add(const PlanAcc& a, const PlanAcc& b) {
   PlanAcc r; r.groups = a.groups + b.groups; r.slots = a.slots + b.slots; r.rows = a.rows + b.rows; r.units = a.units + b.units;
@@ -76,25 +87,15 @@ struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; };
 // When the host sized the results from totals it expected (D.expect) instead of waiting for these, a window whose totals
 // differ gives up and raises the poison flag; so does every window planned after the flag went up - in the same batch
 // (seen by emit_lists) or in a later one - so that windows are never analysed out of order.
-// Grid: (1 + filling CTAs, windows). fill: whether the slot table (sized from the expectation) is to be set to NONE.
-__global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Registry R, int fill) {
+// Grid: (1 + filling CTAs, windows).
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Registry R) {
   begin_after();
   __shared__ PlanAcc s_warp[33];
   __shared__ u32 s_red[32];
   __shared__ u32 s_hist[2][CHUNK_MAX];                         // units per chunk: warp-tiles of class 0, tiles of class 1
   const WinDesc& D = wd[blockIdx.y];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (blockIdx.x > 0) {
-    if (!fill) return;
-    u32* __restrict__ perm = D.perm; const u64 n = D.n_slots;
-    const u64 head = min(n, (u64)((16 - ((uintptr_t)perm & 15)) & 15) / 4), n4 = (n - head) / 4;
-    const u64 i0 = (u64)(blockIdx.x - 1) * blockDim.x + threadIdx.x, st = (u64)(gridDim.x - 1) * blockDim.x;
-    uint4* p4 = reinterpret_cast<uint4*>(perm + head);
-    for (u64 i = i0; i < n4; i += st) p4[i] = make_uint4(NONE, NONE, NONE, NONE);
-    if (i0 < head) perm[i0] = NONE;
-    if (i0 < n - head - n4 * 4) perm[head + n4 * 4 + i0] = NONE;
-    return;
-  }
+  if (blockIdx.x > 0) { fill_slots(D.perm, D.n_slots, blockIdx.x - 1, gridDim.x - 1); return; }
   // what warp 0 compares its findings with; poisoned: an earlier batch's layout was not the expected one
   const u64 slot_cap = D.slot_cap; const bool expects = D.expect != nullptr;
   u64 expected = 0; bool poisoned = false;
