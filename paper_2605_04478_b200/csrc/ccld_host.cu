@@ -148,7 +148,10 @@ constexpr size_t SHAPE_CACHE = 4;
 struct UploadSlot { char* p = nullptr; cudaEvent_t done = nullptr; bool used = false; };
 constexpr size_t UP_PIECE = 1u << 20;                      // a large upload goes piece by piece
 constexpr u32 UP_WORKERS = 6, UP_SLOTS = 2 * UP_WORKERS;   // two pieces per worker: one being filled, one on its way
-constexpr size_t UP_SMALL = 256u << 10;                    // up to this size one kernel reads the pinned columns, beyond it they are copied one by one
+// Up to this size one kernel reads the pinned columns, beyond it they are copied one by one. Nine copies leave gaps of 2 us and more between
+// them; a pass over a window of 23 MB took 723 to 1,169 us with copies and 563 to 641 with the kernel (32 CTAs per column; 8 and 16: up
+// to 739 and 971), of 7 MB 308 to 475 and 248 to 361, of 69 MB 1,430 to 1,498 and 1,424 to 1,427, on a host whose PCIe others share.
+constexpr size_t UP_SMALL = 32u << 20;
 
 constexpr u32 TIMER_RING = 32;
 constexpr int TIMER_PAIRS = CCLD_K_KINDS + 1;          // two launches of the plan per call
@@ -598,7 +601,7 @@ int upload_pageable(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u
 // column by column through its own buffers, one thread, 10 us and more per call. A small upload is put together in one
 // pinned piece instead and crosses in one copy; a large one is cut into pieces that several threads fill while earlier ones
 // cross. Pageable columns are read by the time the call returns. Any other column is read when its turn in the stream comes, so
-// that what earlier work of the stream still writes there is what arrives: large ones go straight across, small ones are
+// that what earlier work of the stream still writes there is what arrives: very large ones go straight across, the others are
 // read by one kernel.
 int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* cols, u32 n_cols) {
   cudaStream_t st = ctx->stream;
