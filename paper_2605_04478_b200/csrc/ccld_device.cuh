@@ -87,7 +87,7 @@ constexpr u32 RANK_TAB_POS_BITS = 13;  // positions < CCLD_MAX_COMM_SIZE = 8192
 struct RangeRow { u32 seq_lo, n_seq, row_idx, n; u64 group0, slot0; u32 tile0, n_units; };
 
 enum { C_REJECTED = 0, C_COMPLETE, C_INCOMPLETE, C_BARRIER, C_ANALYSED, C_FLAG_SKEW, C_FLAG_DUR, C_MISMATCH,
-       C_PRESENT, C_ALERTS, C_ERR, C_INTERNAL, C_COUNT = 16 };
+       C_PRESENT, C_ALERTS, C_ERR, C_INTERNAL, C_MIXED, C_COUNT = 16 };
 constexpr int N_CLASSES = 4;           // reduction code paths: n <= 8, <= 128, <= 1024, larger
 // Classes 0 and 1 run in one fused kernel whose work list is ordered by (window, time chunk): a window's op
 // counters are cut into T chunks per communicator, so that the tiles of one chunk - which gather from the same
@@ -99,7 +99,7 @@ constexpr int N_CLASSES = 4;           // reduction code paths: n <= 8, <= 128, 
 // 401, 382, 361; smaller jobs alike. With 16 the lists take 7 us longer to write and nothing is gained.
 constexpr u32 CHUNK_REF = 32;          // op counters per chunk of the busiest communicator of a window
 constexpr u32 CHUNK_MAX = 64;          // at most this many chunks per window (longer chunks beyond)
-enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS, T_FAILED, T_CHUNKS, T_WT_PER_CTA, T_COUNT = 12 };
+enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS, T_FAILED, T_CHUNKS, T_WT_PER_CTA, T_MIXED, T_COUNT = 12 };
 constexpr u64 FAILED_CAPACITY = 1, FAILED_EXPECT = 2;      // T_FAILED: the window needs too many slots / its layout is not the expected one
 enum { B_FCTA = 0, B_FWT, B_FSUM, B_T2, B_T3, B_COUNT };
 
@@ -111,6 +111,21 @@ struct alignas(16) FusedCta { u32 w, cls, c, seq_off, count, sum_idx, wt_first, 
 
 // What a tile contributes to its communicator's window decision (Eq. 2 and the round counts).
 struct TileSum { u64 best_rng; u32 best_k, n_rounds, n_an, pad; };   // best_k: op-counter offset in the range, NONE if no round
+
+// What the fused kernel needs of a record, as one sector. Where the records of a rank are not neighbours in the upload, a gather of
+// every column fetches a sector per value - 200 bytes per record -, so such windows are scattered record by record.
+struct PackedRecord { u64 te, tx, by; u32 ch, op; };
+static_assert(sizeof(PackedRecord) == 32, "one sector");
+__device__ __forceinline__ void store_packed(uint4* at, const PackedRecord& r) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" :: "l"(at), "r"((u32)r.te), "r"((u32)(r.te >> 32)), "r"((u32)r.tx), "r"((u32)(r.tx >> 32)),
+               "r"((u32)r.by), "r"((u32)(r.by >> 32)), "r"(r.ch), "r"(r.op) : "memory");
+}
+__device__ __forceinline__ PackedRecord load_packed(const uint4* at) {
+  u32 a, b, c, d, e, f; PackedRecord r;
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d), "=r"(e), "=r"(f), "=r"(r.ch), "=r"(r.op) : "l"(at));
+  r.te = (u64)a | (u64)b << 32; r.tx = (u64)c | (u64)d << 32; r.by = (u64)e | (u64)f << 32;
+  return r;
+}
 
 // One window of a batch: input columns, scratch and result pointers (all device memory).
 struct WinDesc {
@@ -133,6 +148,7 @@ struct WinDesc {
   // sized after the plan:
   u64 n_groups, n_slots;
   u32* perm;                         // [n_slots]
+  uint4* packed;                     // [n_slots][2] the slots' records (PackedRecord); null: the fused kernel gathers through perm
   u8* flags;                         // [n_slots]
   i64* gi64;                         // [9][n_groups]
   u32* gu32;                         // [6][n_groups]

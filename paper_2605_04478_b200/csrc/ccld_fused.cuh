@@ -190,7 +190,7 @@ struct DeferList { u64* entries; u32* count; };    // entry: window index in the
 // Where a window's outputs go; kept in shared memory and read when a group stores, so that the pointers do not occupy
 // registers across the gathers.
 struct OutPtrs { u8* flags; i64* gi64; u32* gu32; double* gbw; u64 G; };
-struct InPtrs { const u32* perm; const i64 *te, *tx; const u64* by; const u8* op; const u32 *sc, *rc; };
+struct InPtrs { const uint4* packed; const u32* perm; const i64 *te, *tx; const u64* by; const u8* op; const u32 *sc, *rc; };
 template <class T> __device__ __forceinline__ T ld_volatile(const T& x) { return *(const volatile T*)&x; }
 
 constexpr u32 TILE_KEYS = 8 * SMALL_SEQS;                     // keys of a metric of a staged tile
@@ -252,10 +252,10 @@ __device__ __forceinline__ void ask_indices(const FusedShared& sh, u32 e, u32 la
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// P: positions a lane holds, eight or, for communicators of up to four ranks, four. FULL: as many members. e: the tile's entry, its indices asked for earlier; e_next: the entry of the warp's next tile, if it has
+// P: positions a lane holds, eight or, for communicators of up to four ranks, four. FULL: as many members. PACKED: the records lie in their slots. e: the tile's entry, its indices asked for earlier; e_next: the entry of the warp's next tile, if it has
 // one. One exposed round trip to memory per tile: times, sizes and op codes are asked for together as soon as the indices
 // are there, the rate columns while the order statistics are worked out, the next tile's indices before any of it.
-template <int P, bool FULL>
+template <int P, bool FULL, bool PACKED>
 __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool has_next, TileSum* __restrict__ sums, const Registry& R, const Params& Pm,
                                            const DeferList& DL, FusedShared& sh, u32* __restrict__ slots, u32 lane, SmallAcc& acc) {
   static_assert(P == 8 || (P == 4 && !FULL), "positions");
@@ -263,11 +263,22 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
   const bool active = lane < count;
   const u32* __restrict__ mem = R.members + entry_pair(e, 14);
   const u32 mem_l = lane < n ? __ldg(mem + lane) : 0u;        // lane m holds the rank of position m
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (!PACKED) asm volatile("cp.async.wait_group 0;" ::: "memory");
   u32 a[P], d[P];                                             // enter time against base, duration
-  u64 base, gby; u32 gop, idx[P], xmax;
+  u64 base, gby; u32 gop, idx[P], xmax, ch[P];
   bool ok, mm;
   {
+    i64 ta[P], tb[P]; u64 by[P]; u32 op[P];
+    if (PACKED) {
+      const u32 n_seq = entry_word(e, 5);
+      const uint4* at = ld_volatile(sh.in.packed) + 2 * (entry_pair(e, 10) + entry_word(e, 1) + (active ? lane : 0u));
+#pragma unroll
+      for (int q = 0; q < P; ++q) {
+        const PackedRecord r = load_packed(at + 2 * (u64)((u32)q < n ? q : 0) * n_seq);
+        ta[q] = (i64)r.te; tb[q] = (i64)r.tx; by[q] = r.by; op[q] = r.op; ch[q] = r.ch;
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
     u32 top = 0;
 #pragma unroll
     for (int q = 0; q < P; ++q) { idx[q] = slots[q * 32 + lane]; top = max(top, idx[q]); }
@@ -275,13 +286,14 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
 #pragma unroll
     for (int q = 0; q < P; ++q) idx[q] = present ? idx[q] : 0u;
     if (has_next) ask_indices(sh, e_next, lane, slots);
-    i64 ta[P], tb[P]; u64 by[P]; u32 op[P];
-    const i64* __restrict__ c_te = ld_volatile(sh.in.te); const i64* __restrict__ c_tx = ld_volatile(sh.in.tx);
-    const u64* __restrict__ c_by = ld_volatile(sh.in.by); const u8* __restrict__ c_op = ld_volatile(sh.in.op);
+    if (!PACKED) {
+      const i64* __restrict__ c_te = ld_volatile(sh.in.te); const i64* __restrict__ c_tx = ld_volatile(sh.in.tx);
+      const u64* __restrict__ c_by = ld_volatile(sh.in.by); const u8* __restrict__ c_op = ld_volatile(sh.in.op);
 #pragma unroll
-    for (int q = 0; q < P; ++q) { ta[q] = __ldg(c_te + idx[q]); tb[q] = __ldg(c_tx + idx[q]); }
+      for (int q = 0; q < P; ++q) { ta[q] = __ldg(c_te + idx[q]); tb[q] = __ldg(c_tx + idx[q]); }
 #pragma unroll
-    for (int q = 0; q < P; ++q) { by[q] = __ldg(c_by + idx[q]); op[q] = __ldg(c_op + idx[q]); }
+      for (int q = 0; q < P; ++q) { by[q] = __ldg(c_by + idx[q]); op[q] = __ldg(c_op + idx[q]); }
+    }
     // The upper words of a group's times are nearly always the same (they change every 4.3 s): the lower words are the keys
     // then. Otherwise, and for anything irregular, offsets from the first member's enter time - 2^31 decide.
     const u32 h0 = (u32)((u64)ta[0] >> 32);
@@ -318,8 +330,7 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
     mm = y != 0;
   }
   // the rate columns, read only after the order statistics
-  u32 ch[P];
-  {
+  if (!PACKED) {
     const u32* __restrict__ c_sc = ld_volatile(sh.in.sc); const u32* __restrict__ c_rc = ld_volatile(sh.in.rc);
     if (c_sc != nullptr) {
       u32 rc[P];
@@ -482,7 +493,7 @@ __device__ __forceinline__ void small_tile(u32 w_idx, u32 e, u32 e_next, bool ha
 // Class-0 CTA: up to FUSED_WT_PER_CTA warp-tiles of one window and one time chunk, each up to 32 consecutive op counters of
 // one communicator with its own summary entry. A warp takes every eighth tile and meets the other warps only at the end, so
 // the warps of a CTA drift apart and one warp's gathers overlap another's arithmetic.
-__device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta& t, const WarpTile* wts, TileSum* __restrict__ sums,
+template <bool PACKED> __device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta& t, const WarpTile* wts, TileSum* __restrict__ sums,
                                                 const Registry& R, const Params& P, const DeferList& DL, FusedShared& sh) {
   const u32 wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr u32 NW = SMALL_SEQS / 32;
@@ -498,9 +509,9 @@ __device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta
     const u32 e_after = entry(i + 2 * NW);
     const bool has_next = i + NW < t.wt_count;
     const u32 n = entry_word(e, 7);
-    if (n == SMALL_N) small_tile<8, true>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
-    else if (n > HALF_N) small_tile<8, false>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
-    else small_tile<4, false>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
+    if (n == SMALL_N) small_tile<8, true, PACKED>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
+    else if (n > HALF_N) small_tile<8, false, PACKED>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
+    else small_tile<4, false, PACKED>(t.w, e, e_next, has_next, sums, R, P, DL, sh, slots, lane, acc);
     e = e_next; e_next = e_after;
   }
   const u32 f_skew = __reduce_add_sync(FULLM, lane & 2 ? 0u : acc.flagged), f_dur = __reduce_add_sync(FULLM, lane & 2 ? acc.flagged : 0u);
@@ -518,7 +529,7 @@ __device__ __forceinline__ void fused_small_cta(const WinDesc& D, const FusedCta
 // stream - with one exposed round trip for times, sizes and op codes; the rate columns are on their way while the groups
 // are sorted. Keys meet in shared memory; then L lanes take a group, eight members each (position q L + s in lane s). Last, a thread sums eight op counters of one member's
 // bandwidth.
-template <int L, bool FULL>
+template <int L, bool FULL, bool PACKED>
 __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& t, TileSum* __restrict__ sums, const Registry& R, const Params& P,
                                               const DeferList& DL, FusedShared& sh) {
   constexpr u32 S = SMALL_SEQS / L, GW = 32 / L, NW = SMALL_SEQS / 32;
@@ -543,15 +554,26 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
     u32 bits = top == NONE || i0 == NONE ? 1u : 0u;           // a missing member: the group is set aside
 #pragma unroll
     for (int q = 0; q < 8; ++q) idx[q] = idx[q] == NONE ? 0u : idx[q];
-    const i64* __restrict__ c_te = ld_volatile(sh.in.te); const i64* __restrict__ c_tx = ld_volatile(sh.in.tx);
-    const u64* __restrict__ c_by = ld_volatile(sh.in.by); const u8* __restrict__ c_op = ld_volatile(sh.in.op);
-    i64 ta[8], tb[8]; u64 by[8]; u32 op[8];
-    const u32 j0 = i0 == NONE ? 0u : i0;
-    const i64 te0 = __ldg(c_te + j0); const u64 by0 = __ldg(c_by + j0); const u32 op0 = __ldg(c_op + j0);
+    i64 ta[8], tb[8], te0; u64 by[8], by0; u32 op[8], op0;
+    if (PACKED) {
+      const uint4* at = ld_volatile(sh.in.packed) + 2 * (t.row.slot0 + t.seq_off + (sq < count ? sq : 0u));
+      { const PackedRecord r = load_packed(at); te0 = (i64)r.te; by0 = r.by; op0 = r.op; }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { ta[q] = __ldg(c_te + idx[q]); tb[q] = __ldg(c_tx + idx[q]); }
+      for (int q = 0; q < 8; ++q) {
+        const u32 p = mr + (u32)q * L;
+        const PackedRecord r = load_packed(at + 2 * (u64)(FULL || p < n ? p : mr) * t.row.n_seq);
+        ta[q] = (i64)r.te; tb[q] = (i64)r.tx; by[q] = r.by; op[q] = r.op; sc[q] = r.ch; rc[q] = 0;
+      }
+    } else {
+      const i64* __restrict__ c_te = ld_volatile(sh.in.te); const i64* __restrict__ c_tx = ld_volatile(sh.in.tx);
+      const u64* __restrict__ c_by = ld_volatile(sh.in.by); const u8* __restrict__ c_op = ld_volatile(sh.in.op);
+      const u32 j0 = i0 == NONE ? 0u : i0;
+      te0 = __ldg(c_te + j0); by0 = __ldg(c_by + j0); op0 = __ldg(c_op + j0);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { by[q] = __ldg(c_by + idx[q]); op[q] = __ldg(c_op + idx[q]); }
+      for (int q = 0; q < 8; ++q) { ta[q] = __ldg(c_te + idx[q]); tb[q] = __ldg(c_tx + idx[q]); }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) { by[q] = __ldg(c_by + idx[q]); op[q] = __ldg(c_op + idx[q]); }
+    }
     const u64 base = (u64)te0 - 0x80000000ull;
     u32 hx = 0, neg = 0, xmax = 0; bool back = false;
 #pragma unroll
@@ -573,13 +595,15 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
     if (bits) atomicOr(&sh.t_bits[sq], bits);
     atomicMax(&sh.t_xmax[sq], xmax);
     if (mr == 0) { sh.t_base[sq] = base; sh.t_gby[sq] = by0; sh.t_gop[sq] = op0; }
-    const u32* __restrict__ c_sc = ld_volatile(sh.in.sc); const u32* __restrict__ c_rc = ld_volatile(sh.in.rc);
-    if (c_sc != nullptr) {
+    if (!PACKED) {
+      const u32* __restrict__ c_sc = ld_volatile(sh.in.sc); const u32* __restrict__ c_rc = ld_volatile(sh.in.rc);
+      if (c_sc != nullptr) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) { sc[q] = __ldg(c_sc + idx[q]); rc[q] = __ldg(c_rc + idx[q]); }
-    } else {
+        for (int q = 0; q < 8; ++q) { sc[q] = __ldg(c_sc + idx[q]); rc[q] = __ldg(c_rc + idx[q]); }
+      } else {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) sc[q] = rc[q] = 0;
+        for (int q = 0; q < 8; ++q) sc[q] = rc[q] = 0;
+      }
     }
   }
   __syncthreads();
@@ -725,6 +749,7 @@ __device__ __forceinline__ void fused_sub_cta(const WinDesc& D, const FusedCta& 
   }
 }
 
+template <bool PACKED>
 __global__ void __launch_bounds__(SMALL_SEQS, CCLD_FUSED_MIN_CTAS) k_reduce_fused(const WinDesc* wd, const FusedCta* ctas,
     const WarpTile* wts, TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
   begin_after();
@@ -733,12 +758,12 @@ __global__ void __launch_bounds__(SMALL_SEQS, CCLD_FUSED_MIN_CTAS) k_reduce_fuse
   const WinDesc& D = wd[t.w];
   if (threadIdx.x < SC_COUNT) sh.cnt[threadIdx.x] = 0;
   if (threadIdx.x == 0) { sh.out.flags = D.flags; sh.out.gi64 = D.gi64; sh.out.gu32 = D.gu32; sh.out.gbw = D.gbw; sh.out.G = D.n_groups; }
-  if (threadIdx.x == 32) { sh.in.perm = D.perm; sh.in.te = D.t_enter; sh.in.tx = D.t_exit; sh.in.by = D.bytes; sh.in.op = D.op; sh.in.sc = D.send_chg; sh.in.rc = D.recv_chg; }
-  if (t.cls == 0) { fused_small_cta(D, t, wts, sums, R, P, DL, sh); return; }
+  if (threadIdx.x == 32) { sh.in.packed = D.packed; sh.in.perm = D.perm; sh.in.te = D.t_enter; sh.in.tx = D.t_exit; sh.in.by = D.bytes; sh.in.op = D.op; sh.in.sc = D.send_chg; sh.in.rc = D.recv_chg; }
+  if (t.cls == 0) { fused_small_cta<PACKED>(D, t, wts, sums, R, P, DL, sh); return; }
   const u32 n = t.row.n;
-  if (n <= 32) { if (n == 32) fused_sub_cta<4, true>(D, t, sums, R, P, DL, sh); else fused_sub_cta<4, false>(D, t, sums, R, P, DL, sh); }
-  else if (n <= 64) { if (n == 64) fused_sub_cta<8, true>(D, t, sums, R, P, DL, sh); else fused_sub_cta<8, false>(D, t, sums, R, P, DL, sh); }
-  else { if (n == 128) fused_sub_cta<16, true>(D, t, sums, R, P, DL, sh); else fused_sub_cta<16, false>(D, t, sums, R, P, DL, sh); }
+  if (n <= 32) { if (n == 32) fused_sub_cta<4, true, PACKED>(D, t, sums, R, P, DL, sh); else fused_sub_cta<4, false, PACKED>(D, t, sums, R, P, DL, sh); }
+  else if (n <= 64) { if (n == 64) fused_sub_cta<8, true, PACKED>(D, t, sums, R, P, DL, sh); else fused_sub_cta<8, false, PACKED>(D, t, sums, R, P, DL, sh); }
+  else { if (n == 128) fused_sub_cta<16, true, PACKED>(D, t, sums, R, P, DL, sh); else fused_sub_cta<16, false, PACKED>(D, t, sums, R, P, DL, sh); }
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -139,7 +139,7 @@ struct WindowHost {
 // A batch that was enqueued on totals the host expected instead of waiting for the plan: its actual totals arrive in
 // pinned memory behind the batch's kernels and are checked at the next call that synchronizes anyway.
 // A batch that waited is listed only for its pinned block, which its last descriptor copy still reads.
-struct PendingBatch { u32 first = 0, n = 0; i64 now = 0; Block pin; bool speculative = false; const u64* h_tot() const { return (const u64*)pin.p; } };
+struct PendingBatch { u32 first = 0, n = 0; i64 now = 0; Block pin; bool speculative = false, mixed = false; const u64* h_tot() const { return (const u64*)pin.p; } };
 // Totals of the last batches that were planned with a wait, by shape (record count of every window).
 struct ShapeEntry { std::vector<u64> n_rec; std::vector<u64> totals; };
 constexpr size_t SHAPE_CACHE = 4;
@@ -152,6 +152,8 @@ constexpr u32 UP_WORKERS = 6, UP_SLOTS = 2 * UP_WORKERS;   // two pieces per wor
 // them; a pass over a window of 23 MB took 723 to 1,169 us with copies and 563 to 641 with the kernel (32 CTAs per column; 8 and 16: up
 // to 739 and 971), of 7 MB 308 to 475 and 248 to 361, of 69 MB 1,430 to 1,498 and 1,424 to 1,427, on a host whose PCIe others share.
 constexpr size_t UP_SMALL = 32u << 20;
+
+constexpr u64 PACK_MOST = 8ull << 30;                      // space for records in their slots, at most
 
 constexpr u32 TIMER_RING = 32;
 constexpr int TIMER_PAIRS = CCLD_K_KINDS + 1;          // two launches of the plan per call
@@ -432,7 +434,8 @@ int finalize_registry(ccld_ctx* ctx) {
   CK(cudaFuncSetAttribute(k_opset_check, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(CCLD_MAX_COMM_SIZE * OPSET_MEMBER_BYTES)));
   // The gathers of the small groups are held up by the cache lines an SM can have on their way: no more shared memory than the
   // CTAs need, the rest of the SM's 256 KB is L1. (The other kernels are best off with the driver's own choice.)
-  CK(cudaFuncSetAttribute(k_reduce_fused, cudaFuncAttributePreferredSharedMemoryCarveout, FUSED_CARVEOUT));
+  CK(cudaFuncSetAttribute(k_reduce_fused<false>, cudaFuncAttributePreferredSharedMemoryCarveout, FUSED_CARVEOUT));
+  CK(cudaFuncSetAttribute(k_reduce_fused<true>, cudaFuncAttributePreferredSharedMemoryCarveout, FUSED_CARVEOUT));
   CK(cudaFuncSetAttribute(k_reduce_large<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LargeTile<4>::BYTES));
   CK(cudaFuncSetAttribute(k_reduce_large<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LargeTile<8>::BYTES));
   CK(cudaFuncSetAttribute(k_reduce_large<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LargeTile<16>::BYTES));
@@ -627,6 +630,9 @@ int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* cols, u
   return CCLD_OK;
 }
 
+// Whether records stand in another order than their ranks': the range pass could not fold most of the warps' stretches.
+bool in_other_order(u64 mixed, u64 n_rec) { return mixed * 2 * 32 * REC_RUN > n_rec; }
+
 // Brings the batches that were enqueued on expected totals to a definite state: waits for the stream, reads the totals
 // their plans really found, and analyses again - this time waiting for the plan - every batch from the first one whose
 // expectation failed (that batch and all later ones gave up on the device without touching any state, so the order of
@@ -644,6 +650,15 @@ int settle(ccld_ctx* ctx) {
     for (u32 k = 0; k < b.n && !failed; ++k) if (b.h_tot()[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) failed = true;
     ctx->pinned_free.push_back(b.pin);
     if (!failed) {
+      u64 mixed = 0, all = 0;
+      for (u32 k = 0; k < b.n; ++k) { auto it = ctx->windows.find(b.first + k); if (it != ctx->windows.end()) { mixed += b.h_tot()[(size_t)k * T_COUNT + T_MIXED]; all += it->second.n_rec; } }
+      if (in_other_order(mixed, all) != b.mixed) {           // the shape's records have come in another order this time
+        for (ShapeEntry& s : ctx->shapes) {
+          bool same = s.n_rec.size() == b.n;
+          for (u32 k = 0; k < b.n && same; ++k) { auto it = ctx->windows.find(b.first + k); same = it != ctx->windows.end() && it->second.n_rec == s.n_rec[k]; }
+          for (u32 k = 0; k < b.n && same; ++k) s.totals[(size_t)k * T_COUNT + T_MIXED] = b.h_tot()[(size_t)k * T_COUNT + T_MIXED];
+        }
+      }
       // a window may still have been refused for its size, which the expectation cannot have foreseen: keep what the plan found,
       // which is then no groups and no slots
       for (u32 k = 0; k < b.n; ++k) {
@@ -865,6 +880,12 @@ int ccld_set_speculation(ccld_ctx* ctx, int on) try {
 
 namespace {
 
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) { cudaGetLastError(); return true; }
+  return s != cudaStreamCaptureStatusNone;
+}
+
 int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bool may_speculate) {
   CK(cudaSetDevice(ctx->device));
   std::vector<WindowHost*> ws(n_windows);
@@ -926,7 +947,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     d.chunks = (uint2*)(pbase + o_chunk) + (size_t)k * (CHUNK_MAX + 1); d.totals_host = (u64*)pbatch.pin.p + (size_t)k * T_COUNT;
     d.expect = expect ? (const u64*)(pbase + o_exp) + (size_t)k * T_COUNT : nullptr; d.poison = ctx->d_poison;
     d.n_groups = d.n_slots = 0; d.perm = nullptr; d.flags = nullptr; d.gi64 = nullptr; d.gu32 = nullptr; d.gbw = nullptr;
-    d.comm_rows = nullptr; d.alerts = nullptr;
+    d.comm_rows = nullptr; d.alerts = nullptr; d.packed = nullptr;
     for (int q = 0; q < B_COUNT; ++q) d.base[q] = 0;
     d.pad = 0; d.tsum[0] = d.tsum[1] = d.tsum[2] = nullptr;
     hd[k] = d;
@@ -991,10 +1012,25 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   if (e != cudaSuccess) return fail(ctx, CCLD_ERR_NOMEM, "result allocation failed");
   auto res_blk = std::make_shared<Shared>(&ctx->pool, rb);
   char* rbase = (char*)rb.p;
+  // Records in another order than their ranks' (as this shape had them last; both ways are right whatever the order): the fused
+  // kernel's records go to their slots. The space is needed until the reductions are through, so whatever the stream does
+  // next may have it; where it is not to be had, and in a graph, whose launches would share it, the kernel gathers.
+  struct PackSpace { ccld_ctx* ctx; Block b; ~PackSpace() { ctx->pool.put(b); } } pack_space{ctx, {}};
+  if (expect) {
+    u64 mixed = 0, all = 0;
+    for (u32 k = 0; k < B; ++k) { mixed += tot[(size_t)k * T_COUNT + T_MIXED]; all += ws[k]->n_rec; }
+    pbatch.mixed = in_other_order(mixed, all);
+    if (pbatch.mixed && n_list[B_FCTA] && total_slots * sizeof(PackedRecord) <= PACK_MOST && !capturing(st)) {
+      pack_space.b = ctx->pool.get(total_slots * sizeof(PackedRecord), &e);
+      if (e != cudaSuccess) { cudaGetLastError(); pack_space.b = Block{}; }
+    }
+  }
+  const bool pack = pack_space.b.p != nullptr;
   for (u32 k = 0; k < B; ++k) {
     const u64* t = tot + (size_t)k * T_COUNT;
     WinDesc& d = hd[k];
     d.n_groups = t[T_GROUPS]; d.n_slots = t[T_SLOTS];
+    if (pack) d.packed = (uint4*)pack_space.b.p + perm_off[k] / 2;         // 32 bytes where perm has 4
     d.perm = (u32*)(rbase + o_perm + perm_off[k]); d.flags = (u8*)(rbase + o_flags[k]);
     d.gi64 = (i64*)(rbase + o_gi[k]); d.gu32 = (u32*)(rbase + o_gu[k]); d.gbw = (double*)(rbase + o_gb[k]);
     d.comm_rows = (ccld_comm_verdict*)(rbase + o_rows[k]); d.alerts = (ccld_hang_alert*)(rbase + o_al[k]);
@@ -1019,7 +1055,8 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     const u64 blocks = (cta * REC_PER_CTA + SCAT_PER_CTA - 1) / SCAT_PER_CTA;      // of the largest window
     const u32 per = (u32)std::min<u64>(SCAT_BLOCKS_MAX, std::max<u64>(1, blocks * B / (16ull * ctx->n_sms)));
     TimedLaunch tl(ts, 2, st);
-    launch(st, k_slot_scatter, dim3(emit_ctas + (u32)((blocks + per - 1) / per), B), SCAT_THREADS, 0, d_desc, ctx->reg, pl, emit_ctas, slices, per_slice, per);
+    if (pack) launch(st, k_slot_pack, dim3(emit_ctas + (u32)((cta * REC_PER_CTA + PACK_PER_CTA - 1) / PACK_PER_CTA), B), SCAT_THREADS, 0, d_desc, ctx->reg, pl, emit_ctas, slices, per_slice);
+    else launch(st, k_slot_scatter, dim3(emit_ctas + (u32)((blocks + per - 1) / per), B), SCAT_THREADS, 0, d_desc, ctx->reg, pl, emit_ctas, slices, per_slice, per);
   }
   const DeferList dl_big{(u64*)(rbase + o_def3), (u32*)(pbase + o_defn) + 2};
   static_assert(MID_SEQS == LARGE_SEQS, "one list for the groups of both classes");
@@ -1053,7 +1090,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   if (n_list[B_FCTA]) {
     const DeferList dl{(u64*)(rbase + o_def), (u32*)(pbase + o_defn)};
     TimedLaunch tl(ts, 3, st);
-    launch(st, k_reduce_fused, (u32)n_list[B_FCTA], SMALL_SEQS, 0, d_desc, pl.fcta, pl.fwt, (TileSum*)(rbase + o_fsum), ctx->reg, ctx->dp, dl);
+    launch(st, pack ? k_reduce_fused<true> : k_reduce_fused<false>, (u32)n_list[B_FCTA], SMALL_SEQS, 0, d_desc, pl.fcta, pl.fwt, (TileSum*)(rbase + o_fsum), ctx->reg, ctx->dp, dl);
     launch(st, k_reduce_deferred, DEF_GRID, DEF_WARPS * 32, 0, d_desc, dl, ctx->reg, ctx->dp, now_ns);
   }
   On joined = chains.close();

@@ -4,6 +4,7 @@
 //   k_seq_range     group-by, part 1: op-counter range per (window, communicator)
 //   k_layout        group-by, part 2: closed-form slot layout (prefix sums over communicators; ccld_plan.cuh)
 //   k_slot_scatter  group-by, part 3: perm[slot] = record index; beside it the work lists of the reduction kernels
+//   k_slot_pack     the same for uploads whose records are not in their ranks' order: the record itself goes along
 //   k_reduce_fused  per-op reductions + median/MAD + flags + votes for n <= 128, chunk-major work list:
 //                   n <= 8 one thread per group (warp-tiles), 9 <= n <= 128 n_pad / 8 lanes per group (register /
 //                   shuffle bitonic network); complete groups whose times fit 32-bit offsets
@@ -157,6 +158,7 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
     for (u32 c = threadIdx.x; c < R.n_comms; c += REC_THREADS) { s_mn[c] = NONE; s_mx[c] = 0; }
     __syncthreads();
   }
+  u32 mixed = 0;                                             // stretches of 32 runs that the warp could not fold
   // a CTA takes blocks_per_cta consecutive blocks of the window, one after the other, and keeps one table for them: the
   // table's set-up, its barriers and its merge into the window's ranges are paid once
   for (u32 blk = 0; blk < blocks_per_cta; ++blk) {
@@ -216,6 +218,7 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
         remaining -= cleared;
         if (!worth) break;
       }
+      mixed += remaining > 32 * REC_RUN / 2 ? 1u : 0u;
     }
     // folds: the communicator of the first record still left takes every record of the run that names it
     for (int f = 0; f < RANGE_FOLDS && __any_sync(0xFFFFFFFFu, left != 0); ++f) {
@@ -274,6 +277,7 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
       }
     }
   }
+  if (lane == 0) count_add(D.counters, C_MIXED, mixed);
   if (s_mn == nullptr) return;
   __syncthreads();
   u32* const rmin = D.rmin; u32* const rmax = D.rmax;
@@ -313,6 +317,18 @@ __device__ __forceinline__ bool scatter_slot(const Registry& R, u32 c, u32 ns, u
   *slot = base_pos + (sq - lo);
   if (sq - lo >= ns || *slot >= n_slots) { *internal = 1; return false; }
   return true;
+}
+
+// What the lanes of a warp found wrong with their records.
+__device__ __forceinline__ void count_rejects(const WinDesc& D, u32 err, u32 rej, u32 internal) {
+  err = __reduce_or_sync(0xFFFFFFFFu, err);
+  rej = __reduce_add_sync(0xFFFFFFFFu, rej);
+  internal = __reduce_or_sync(0xFFFFFFFFu, internal);
+  if ((threadIdx.x & 31) == 0) {
+    if (err) atomicOr((unsigned*)&D.counters[C_ERR], err);
+    count_add(D.counters, C_REJECTED, rej);
+    if (internal) atomicOr((unsigned*)&D.counters[C_INTERNAL], 1u);
+  }
 }
 
 constexpr u32 SCAT_LOCAL = 8;     // ranks, counted from the rank of the CTA's first record, whose table rows a CTA resolves once
@@ -422,14 +438,81 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc*
     }
     r_first = r_next;
   }
-  err = __reduce_or_sync(0xFFFFFFFFu, err);
-  rej = __reduce_add_sync(0xFFFFFFFFu, rej);
-  internal = __reduce_or_sync(0xFFFFFFFFu, internal);
-  if ((threadIdx.x & 31) == 0) {
-    if (err) atomicOr((unsigned*)&D.counters[C_ERR], err);
-    count_add(D.counters, C_REJECTED, rej);
-    if (internal) atomicOr((unsigned*)&D.counters[C_INTERNAL], 1u);
+  count_rejects(D, err, rej, internal);
+}
+
+
+// The same where the upload has its records in another order (see PackedRecord): few of them belong to the ranks a CTA would resolve,
+// so every record takes the two table loads, and its values, which the reading of the columns brings along whole, go to the slot
+// with its index. Two windows of 4,096 ranks in arrival order, 8.2 M records: 208 us, and the fused kernel 93 (16 bytes of tables per record from
+// L1 or L2, 36 bytes to random sectors), where indices alone took 118 and the gathers 252; 0.5 M records each of 512 ranks 26 and 16, 17.5 and
+// 42. In rank-major order it is the other way round (a record read and written twice, 109 instead of 79 bytes).
+// Two records per thread with their values asked for together with the keys; four with the values asked for last took 219, one 283.
+constexpr int PACK_PER_THREAD = 2;
+constexpr int PACK_PER_CTA = SCAT_THREADS * PACK_PER_THREAD;
+// Read once: these leave L1 to the tables.
+__device__ __forceinline__ u32 load_once(const u32* p) { u32 v; asm volatile("ld.global.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
+__device__ __forceinline__ u64 load_once(const u64* p) { u64 v; asm volatile("ld.global.L1::no_allocate.u64 %0, [%1];" : "=l"(v) : "l"(p)); return v; }
+__device__ __forceinline__ u32 load_once(const u8* p) { u32 v; asm volatile("ld.global.L1::no_allocate.u8 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
+__global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_pack(const WinDesc* wd, Registry R, PlanLists L, u32 emit_ctas, u32 slices, u32 slice_blocks) {
+  begin_after();
+  __shared__ uint4 s_pair[EMIT_THREADS / 32];
+  const WinDesc& D = wd[blockIdx.y];
+  if (blockIdx.x < emit_ctas) { emit_lists(D, R, L, emit_ctas, slices, slice_blocks, s_pair); return; }
+  const u64 base = (u64)(blockIdx.x - emit_ctas) * PACK_PER_CTA + threadIdx.x, n_rec = D.n_rec, n_slots = D.n_slots;
+  if (base - threadIdx.x >= n_rec) return;
+  const u64 failed = D.totals[T_FAILED]; const u32 poisoned = *(volatile u32*)D.poison; const bool expects = D.expect != nullptr;
+  u32* const perm = D.perm; uint4* const packed = D.packed; const uint4* const srow = D.srow;
+  u32 err = 0, rej = 0, internal = 0, rk[PACK_PER_THREAD], cid[PACK_PER_THREAD], sq[PACK_PER_THREAD], v[PACK_PER_THREAD];
+  PackedRecord r[PACK_PER_THREAD];
+  {
+    const u32 *c_rank = D.rank, *c_comm = D.comm, *c_seq = D.seq, *c_sc = D.send_chg, *c_rc = D.recv_chg;
+    const u64 *c_te = (const u64*)D.t_enter, *c_tx = (const u64*)D.t_exit, *c_by = D.bytes; const u8* c_op = D.op;
+#pragma unroll
+    for (int k = 0; k < PACK_PER_THREAD; ++k) {
+      const u64 i = min(base + (u64)k * SCAT_THREADS, n_rec - 1);          // beyond the end: not looked at
+      rk[k] = load_once(c_rank + i); cid[k] = load_once(c_comm + i); sq[k] = load_once(c_seq + i);
+    }
+#pragma unroll
+    for (int k = 0; k < PACK_PER_THREAD; ++k) {
+      const u64 i = min(base + (u64)k * SCAT_THREADS, n_rec - 1);
+      r[k].te = load_once(c_te + i); r[k].tx = load_once(c_tx + i); r[k].by = load_once(c_by + i); r[k].op = load_once(c_op + i); r[k].ch = 0;
+      if (c_sc != nullptr) { const u32 sc = load_once(c_sc + i), rc = load_once(c_rc + i); r[k].ch = max(sc, rc); }
+    }
   }
+#pragma unroll
+  for (int k = 0; k < PACK_PER_THREAD; ++k) {
+    v[k] = NONE;
+    if (rk[k] < R.n_ranks) {
+      u32 t[8];
+      asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                   : "=r"(t[0]), "=r"(t[1]), "=r"(t[2]), "=r"(t[3]), "=r"(t[4]), "=r"(t[5]), "=r"(t[6]), "=r"(t[7]) : "l"(R.rank_tab + (u64)rk[k] * 2));
+#pragma unroll
+      for (int q = 0; q < RANK_TAB_K; ++q) v[k] = t[2 * q] == cid[k] ? t[2 * q + 1] : v[k];
+    }
+  }
+  if (failed == 0 && expects && poisoned) return;             // as in k_slot_scatter
+  uint4 sr[PACK_PER_THREAD];
+#pragma unroll
+  for (int k = 0; k < PACK_PER_THREAD; ++k) {
+    if (base + (u64)k * SCAT_THREADS >= n_rec) v[k] = NONE;
+    else if (v[k] == NONE || v[k] == RANK_TAB_OVERFLOW || cid[k] == NONE) {
+      const u64 rs = resolve_slow(R, rk[k], cid[k]);
+      v[k] = (u32)rs;
+      if (rs >> 32) { err |= (u32)(rs >> 32); ++rej; }
+    }
+    sr[k] = v[k] != NONE ? srow[v[k] >> RANK_TAB_POS_BITS] : make_uint4(0, 0, 0, 0);
+  }
+#pragma unroll
+  for (int k = 0; k < PACK_PER_THREAD; ++k) {
+    if (v[k] == NONE) continue;
+    u64 slot;
+    if (!scatter_slot(R, v[k] >> RANK_TAB_POS_BITS, sr[k].z, sr[k].w, ((u64)sr[k].x | ((u64)sr[k].y << 32)) + (u64)(v[k] & ((1u << RANK_TAB_POS_BITS) - 1)) * sr[k].z, sq[k],
+                      n_slots, &slot, &err, &rej, &internal)) continue;
+    perm[slot] = (u32)(base + (u64)k * SCAT_THREADS);
+    store_packed(packed + slot * 2, r[k]);
+  }
+  count_rejects(D, err, rej, internal);
 }
 
 }  // namespace ccld

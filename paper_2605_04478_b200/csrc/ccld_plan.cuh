@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   // what warp 0 compares its findings with; poisoned: an earlier batch's layout was not the expected one
   const u64 slot_cap = D.slot_cap; const bool expects = D.expect != nullptr;
   u64 expected = 0; bool poisoned = false;
+  const u64 mixed = D.counters[C_MIXED];
   if (wid == 0 && expects) { expected = lane < T_COUNT ? D.expect[lane] : 0; poisoned = *(volatile u32*)D.poison != 0; }
   const u32 per = ceil_div(R.n_comms, blockDim.x), c_lo = threadIdx.x * per, c_hi = min(R.n_comms, c_lo + per);   // my communicators
   // counters covered and members of my first few communicators stay in registers, all loads issued at once
@@ -189,10 +190,11 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
     t = lane == T_GROUPS ? all.groups : t; t = lane == T_SLOTS ? all.slots : t; t = lane == T_FCTA ? n_cta : t; t = lane == T_FWT ? n_wt : t;
     t = lane == T_FSUM ? all.units : t; t = lane == T_TILES2 ? all.t2 : t; t = lane == T_TILES3 ? all.t3 : t; t = lane == T_ROWS ? all.rows : t;
     t = lane == T_CHUNKS ? T : t; t = lane == T_WT_PER_CTA ? wt_per_cta : t;
+    t = lane == T_MIXED ? mixed : t;
     // op counters further apart than 2^31, or more slots than the cap: refuse the window
     u64 failed = (all.slots > slot_cap || all.groups > 0x7FFFFFFFull) ? FAILED_CAPACITY : 0;
     if (!failed && expects) {
-      const bool same = lane == T_FAILED || lane >= T_COUNT || t == expected;
+      const bool same = lane == T_FAILED || lane == T_MIXED || lane >= T_COUNT || t == expected;      // (any order of the records is as good)
       if (!__all_sync(0xFFFFFFFFu, same) || poisoned) { failed = FAILED_EXPECT; if (lane == 0) atomicExch(D.poison, 1u); }
     }
     if (failed) t = lane == T_CHUNKS || lane == T_WT_PER_CTA ? 1 : 0;

@@ -437,3 +437,123 @@ def test_copies_of_many_arrays():
             same(a, t.cpu().numpy(), "array")
     r = subprocess.run([sys.executable, "-c", _LITTLE_MEMORY], capture_output=True, text=True, cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert r.returncode == 0 and r.stdout.strip() == "rc 0", (r.returncode, r.stdout, r.stderr[-500:])
+
+
+# ---------------------------------------------------------------- units, positions, records in their slots
+def cut(cols, keep):
+    return {k: v[keep].copy() for k, v in cols.items()}
+
+
+def again(an, o, n_ranks, times=2):
+    """The same window analysed again: sized from what the pass before found."""
+    for _ in range(times):
+        an.reset()
+        an.analyze_window(0, 1, 10**13)
+        compare_window(an, o, 0)
+        compare_cumulative(an, o, n_ranks, 0)
+
+
+@pytest.mark.parametrize("most", [1, 31, 33, 96, 700, 2500])
+def test_units_over_the_chunks(most):
+    """Communicators with fewer, as many and more op counters than a unit and than a chunk, up to more units than there are chunks."""
+    rng = np.random.default_rng(most)
+    sizes = [2, 4, 5, 8, 9, 32, 33, 65, 128]
+    reg, cols, n = job(sizes, most, rng)
+    limit = np.array([max(1, most // (1 + c % 4) - c % 3) for c in range(len(sizes))])
+    cols = cut(cols, cols["seq"] < limit[cols["comm"]])
+    an, o = run(reg, cols, n)
+    again(an, o, n, 1)
+
+
+@pytest.mark.parametrize("n_seq", [1, 32, 45])
+@pytest.mark.parametrize("min_group", [1, 4])
+def test_four_positions(n_seq, min_group):
+    """Groups of one to five, complete and not, all of them tested or only those of four and more; ties."""
+    rng = np.random.default_rng(10 * n_seq + min_group)
+    reg, cols, n = job([1, 2, 3, 4, 5] * 3, n_seq, rng, dur=lambda c, n: 1_000_000 + rng.integers(0, 4, (n_seq, n)), ent=lambda c, n: rng.integers(0, 3, (n_seq, n)))
+    cols["op"] = (cols["seq"] % 3).astype(np.uint8)
+    cols["bytes"][cols["seq"] % 5 == 1] = 2                     # barriers
+    cols["t_exit"][rng.random(len(cols["seq"])) < 0.02] = -1
+    cols = cut(cols, rng.random(len(cols["seq"])) >= 0.02)
+    an, o = run(reg, cols, n, dict(min_group=min_group))
+    again(an, o, n, 1)
+
+
+@pytest.mark.parametrize("sizes", [[1] * 40, [3] * 1100, [2] * 33 + [130] * 3 + [1100]])
+def test_owner_of_a_group_set_aside(sizes):
+    """Every op of a few communicators lacks a member: among fewer than 32 x 32 communicators and more, at both ends."""
+    rng = np.random.default_rng(len(sizes))
+    reg, cols, n = job(sizes, 3, rng)
+    lame = np.isin(cols["comm"], [0, 1, 31, 32, 33, len(sizes) // 2, len(sizes) - 1])
+    cols["t_exit"][lame & (rng.random(len(lame)) < 0.4)] = -1
+    cols["t_exit"][lame & (rng.random(len(lame)) < 0.2)] = 5    # exit before enter
+    cols = cut(cols, ~(lame & (rng.random(len(lame)) < 0.2)))
+    an, o = run(reg, cols, n)
+    again(an, o, n, 1)
+
+
+MANY = list(range(1, 9)) * 12 + [9, 33, 64, 128]
+
+
+@pytest.mark.parametrize("rates", [True, False])
+@pytest.mark.parametrize("n_seq", [3, 37, 64])
+def test_records_in_no_order(n_seq, rates):
+    """From the second pass on such a window's records lie in their slots: complete groups, missing members, ops in flight, sizes that
+    differ, records of strangers, then as many records in their ranks' order, and mixed again."""
+    rng = np.random.default_rng(n_seq)
+    reg, cols, n = job(MANY, n_seq, rng, order="shuffled")
+    cols["bytes"][rng.random(len(cols["seq"])) < 0.003] += 4
+    cols["op"][rng.random(len(cols["seq"])) < 0.003] = 3
+    cols["t_exit"][rng.random(len(cols["seq"])) < 0.003] = -1
+    cols = cut(cols, rng.random(len(cols["seq"])) >= 0.003)
+    if not rates:
+        del cols["send_chg"], cols["recv_chg"]
+    an, o = run(reg, cols, n)
+    again(an, o, n)
+    order = np.lexsort((cols["seq"], cols["comm"], cols["rank"]))
+    sorted_ = {k: v[order] for k, v in cols.items()}
+    for c in (sorted_, sorted_, cols, cols):
+        an.window_release(0)
+        an.reset()
+        an.trace_upload(0, c)
+        an.analyze_window(0, 1, 10**13)
+        p = make_pair(reg)[1]
+        assert p.upload(0, c) == 0 and p.analyze(0, 1, 10**13) == 0
+        compare_window(an, p, 0)
+        compare_cumulative(an, p, n, 0)
+        an.get_verdict(0)
+
+
+def test_records_in_no_order_with_strangers():
+    """Unknown communicators, ranks that are no members or out of range: rejected and counted as where indices alone are placed."""
+    rng = np.random.default_rng(4)
+    reg, cols, n = job(MANY, 20, rng, order="shuffled")
+    i = rng.choice(len(cols["seq"]), 60, replace=False)
+    cols["comm"][i[:20]] = 5000
+    cols["comm"][i[20:40]] = 0xFFFFFFFF
+    cols["rank"][i[40:50]] = n + 7
+    cols["rank"][i[50:]] = 0
+    an, o = make_pair(reg)
+    an.trace_upload(0, cols)
+    o.upload(0, cols)
+    an.analyze_window(0, 1, 10**13)
+    o.analyze(0, 1, 10**13)
+    first = an.get_verdict(0, check=False)
+    assert first["n_rejected"] >= 50 and first["n_rejected"] == o.sizes(0)["n_rejected"]
+    for _ in range(2):
+        an.reset()
+        an.analyze_window(0, 1, 10**13)
+        compare_window(an, o, 0, expect_rc=first["rc"])
+
+
+def test_pinned_upload_beyond_what_a_kernel_reads():
+    """More than 32 MB of pinned columns are copied column by column."""
+    rng = np.random.default_rng(8)
+    n_seq = 100_000
+    reg, cols, n = job([8], n_seq, rng, spacing=2_000_000)
+    an, o = make_pair(reg)
+    assert o.upload(0, cols) == 0 and sum(v.nbytes for v in cols.values()) > 32 << 20
+    an.trace_upload(0, {k: torch.from_numpy(v if v.itemsize == 1 else v.view("i%d" % v.itemsize)).pin_memory() for k, v in cols.items()})
+    an.analyze_window(0, 1, 10**15)
+    assert o.analyze(0, 1, 10**15) == 0
+    compare_window(an, o, 0)
