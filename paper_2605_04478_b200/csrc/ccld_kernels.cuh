@@ -556,11 +556,21 @@ __device__ __forceinline__ RoundPart rounds_of(const WinDesc& D, const RangeRow&
     // recount the communicator's window from the per-op rows
     const u32* gfl = D.gu32 + (u64)GU_GFLAGS * G + row.group0;
     n_rounds = 0; n_an = 0; best_rng = 0; best_k = NONE;
-#pragma unroll 4
-    for (u32 k = lane; k < row.n_seq; k += 32) {
-      const u32 f = gfl[k]; const u64 rng = (u64)(t_max[k] - t_min[k]);
-      if ((f & CCLD_G_COMPLETE) && !(f & CCLD_G_BARRIER)) { ++n_rounds; best_merge(best_rng, best_k, rng, k); }
-      if (f & CCLD_G_ANALYSED) ++n_an;
+    constexpr u32 AHEAD = 8;                             // ops per lane whose rows are asked for at once
+    for (u32 k0 = lane; k0 < row.n_seq; k0 += 32 * AHEAD) {
+      u32 f[AHEAD]; u64 rng[AHEAD];
+#pragma unroll
+      for (u32 u = 0; u < AHEAD; ++u) {
+        const u32 k = min(k0 + 32 * u, row.n_seq - 1);
+        f[u] = gfl[k]; rng[u] = (u64)(t_max[k] - t_min[k]);
+      }
+#pragma unroll
+      for (u32 u = 0; u < AHEAD; ++u) {
+        const u32 k = k0 + 32 * u;
+        if (k >= row.n_seq) break;
+        if ((f[u] & CCLD_G_COMPLETE) && !(f[u] & CCLD_G_BARRIER)) { ++n_rounds; best_merge(best_rng, best_k, rng[u], k); }
+        if (f[u] & CCLD_G_ANALYSED) ++n_an;
+      }
     }
   }
   x.n_rounds = __reduce_add_sync(0xFFFFFFFFu, n_rounds); *n_analysed = __reduce_add_sync(0xFFFFFFFFu, n_an);
@@ -604,7 +614,9 @@ __device__ __forceinline__ void count_ops(const Registry& R, OpsShared& sh, u32 
 }
 
 // Stage 1 of a batch of several windows, all at once: leaves the part above in the communicator's verdict row.
-__global__ void __launch_bounds__(WD_THREADS) k_window_rounds(const WinDesc* wd, Registry R) {
+// (Twelve CTAs per SM: with the registers that eight ops per lane in the recount would like it took 14.8 instead of 11.9 us on twelve windows
+// of 1,088 communicators; recounting 1,000 op counters takes 9.4 us with eight, 12.1 with four at a time.)
+__global__ void __launch_bounds__(WD_THREADS, 12) k_window_rounds(const WinDesc* wd, Registry R) {
   begin_after();
   __shared__ OpsShared s_ops;
   const u32 c = blockIdx.x * (WD_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -675,10 +687,20 @@ __global__ void __launch_bounds__(WD_THREADS) k_window_decide(const WinDesc* wd,
         const u32* gfl = D.gu32 + (u64)GU_GFLAGS * G + row.group0;
         const i64* e_min = D.gi64 + (u64)GI_E_MIN * G + row.group0;
         const i64* t_max = D.gi64 + (u64)GI_T_MAX * G + row.group0;
-        for (u32 k0 = 0; k0 < row.n_seq && st.m == 0; k0 += 32) {
-          const u32 k = k0 + lane;
-          u32 f = 0; i64 em = 0, tM = 0;
-          if (k < row.n_seq) { f = gfl[k]; em = e_min[k]; tM = t_max[k]; }
+        constexpr u32 AHEAD = 4;                             // steps of 32 ops whose rows are asked for at once
+        u32 f_[AHEAD]; i64 em_[AHEAD], tM_[AHEAD];
+        for (u32 k0 = 0, u = 0; k0 < row.n_seq && st.m == 0; k0 += 32, u = (u + 1) % AHEAD) {
+          if (u == 0) {
+#pragma unroll
+            for (u32 q = 0; q < AHEAD; ++q) {
+              const u32 k = k0 + 32 * q + lane;
+              f_[q] = 0; em_[q] = tM_[q] = 0;
+              if (k < row.n_seq) { f_[q] = gfl[k]; em_[q] = e_min[k]; tM_[q] = t_max[k]; }
+            }
+          }
+          u32 f = f_[0]; i64 em = em_[0], tM = tM_[0];
+#pragma unroll
+          for (u32 q = 0; q + 1 < AHEAD; ++q) { f_[q] = f_[q + 1]; em_[q] = em_[q + 1]; tM_[q] = tM_[q + 1]; }
           const bool round = (f & CCLD_G_COMPLETE) && !(f & CCLD_G_BARRIER);
           const u32 bal = __ballot_sync(0xFFFFFFFFu, round);
           if (bal == 0) continue;
