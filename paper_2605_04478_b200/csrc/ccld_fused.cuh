@@ -835,17 +835,28 @@ __global__ void __launch_bounds__(DEF_WARPS * 32) k_reduce_deferred(const WinDes
     bool pres[DEF_Q]; i64 ta[DEF_Q], tb[DEF_Q]; u64 by[DEF_Q]; u32 op[DEF_Q], ch[DEF_Q];
     u32 npres = 0, first_p = NONE; bool miss = false, inflight = false, bad = false;
     i64 age = -1, x_max = INT64_MIN; u64 ck = 0;
+    // all indices, then all values: two round trips, not two per 32 members
+    u32 idx[DEF_Q];
+    {
+      const u32* perm = D.perm; const i64 *c_te = D.t_enter, *c_tx = D.t_exit; const u64* c_by = D.bytes; const u8* c_op = D.op; const u32 *c_sc = D.send_chg, *c_rc = D.recv_chg;
+#pragma unroll
+      for (int i = 0; i < DEF_Q; ++i) { const u32 p = lane + 32u * i; idx[i] = p < n ? perm[perm_at(row, so, p)] : NONE; }
+#pragma unroll
+      for (int i = 0; i < DEF_Q; ++i) {
+        pres[i] = idx[i] != NONE;
+        const u32 ix = pres[i] ? idx[i] : 0u;                // (a window with a group has a record)
+        ta[i] = c_te[ix]; tb[i] = c_tx[ix]; by[i] = c_by[ix]; op[i] = c_op[ix]; ch[i] = 0;
+        if (c_sc != nullptr) { const u32 sc = c_sc[ix], rc = c_rc[ix]; ch[i] = sc > rc ? sc : rc; }
+      }
+    }
 #pragma unroll
     for (int i = 0; i < DEF_Q; ++i) {
       const u32 p = lane + 32u * i;
-      pres[i] = false; ta[i] = 0; tb[i] = 0; by[i] = 0; op[i] = 0; ch[i] = 0;
+      if (!pres[i]) { ta[i] = 0; tb[i] = 0; by[i] = 0; op[i] = 0; ch[i] = 0; }
       if (p < n) {
-        const u32 idx = D.perm[perm_at(row, so, p)];
-        if (idx == NONE) miss = true;
+        if (!pres[i]) miss = true;
         else {
-          pres[i] = true; ++npres; if (first_p == NONE) first_p = p;
-          ta[i] = D.t_enter[idx]; tb[i] = D.t_exit[idx]; by[i] = D.bytes[idx]; op[i] = D.op[idx];
-          if (D.send_chg != nullptr) { const u32 sc = D.send_chg[idx], rc = D.recv_chg[idx]; ch[i] = sc > rc ? sc : rc; }
+          ++npres; if (first_p == NONE) first_p = p;
           if (tb[i] == -1) { inflight = true; const i64 ag = now - ta[i]; age = ag > age ? ag : age; }
           else if (ta[i] < 0 || tb[i] < ta[i]) bad = true;
           x_max = tb[i] > x_max ? tb[i] : x_max;
