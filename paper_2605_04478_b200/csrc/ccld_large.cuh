@@ -169,8 +169,11 @@ __device__ __forceinline__ u32 cluster_duration(const uint2* p, u32 cta) {
   u32 d; asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(d) : "r"(cluster_address(p, cta) + 4) : "memory"); return d;
 }
 
+// CTAs per SM: three up to 4,096 members, although that leaves 40 registers and spills some 80 bytes (two instead: 254 and not 228 us on two windows
+// of 1,100 members, 149 and not 144 of 2,000, 138 and not 129 ns per op counter of 3,000 before keys went to their owners at once);
+// above, two are what shared memory holds. Two records in flight per thread; four spill more, above 4,096 there is room for them.
 template <int Q>
-__global__ void __launch_bounds__(LQ_THREADS, Q == 8 ? 3 : 2) k_reduce_large(const WinDesc* wd, const Tile* tiles,
+__global__ void __launch_bounds__(LQ_THREADS, Q == 16 ? 2 : 3) k_reduce_large(const WinDesc* wd, const Tile* tiles,
     TileSum* __restrict__ sums, Registry R, Params P, DeferList DL) {
   begin_after();
   extern __shared__ __align__(16) unsigned char large_raw[];

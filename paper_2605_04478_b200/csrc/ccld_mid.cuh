@@ -131,10 +131,11 @@ struct MidTrack {
   }
 };
 
-// CTAs per SM, in ns per op counter of one window of 4 M records: up to 256 members two 7.9, three 6.1, four 5.8 (172 members; 9.0, 7.1, 6.9
-// at 256); of 257 to 512 two 18.3, three 15.0 (512); with 32 keys per lane two are what the registers allow. It is three, two, two.
+// CTAs per SM: up to 256 members three (four leave 64 registers and spill: 57.0 instead of 58.8 us on twenty rings of 172, but 20.9 instead of
+// 18.9 on sixteen of 256 and 103 instead of 98 beside groups of 4 and 6), of 257 to 512 three (76.4 instead of 94.2 us with two on ten rings of 400,
+// 82 instead of 100 on one of 500); with 32 keys per lane two are what the registers allow.
 template <int R>
-__global__ void __launch_bounds__(MID_THREADS, R == 8 ? 3 : 2) k_reduce_mid(const WinDesc* wd, const Tile* tiles,
+__global__ void __launch_bounds__(MID_THREADS, R == 32 ? 2 : 3) k_reduce_mid(const WinDesc* wd, const Tile* tiles,
     TileSum* __restrict__ sums, Registry R_, Params P, DeferList DL) {
   begin_after();
   extern __shared__ __align__(16) u32 mid_keys[];
