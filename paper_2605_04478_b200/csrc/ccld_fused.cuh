@@ -10,6 +10,9 @@
 //   k_reduce_deferred  the listed groups, one warp each, in full 64-bit generality: missing members, records in
 //                      flight (hang alerts), invalid times, spreads beyond 32 bits.
 //
+// Windows whose records do not lie in their ranks' order have them in the slots (PackedRecord); the second instance of the kernel
+// reads them there, coalesced, with the presence of a member still taken from its index.
+//
 // The work list of k_reduce_fused is chunk-major (see emit_lists), so CTAs that run together gather from the same stretch
 // of every rank's records and share the fetched sectors in L2.
 #pragma once
@@ -210,8 +213,8 @@ struct FusedShared {
 };
 
 // Three CTAs fit 64 KB of shared memory, which leaves 192 KB of an SM to its L1. How many lines L1 holds is how many gathers can
-// be on their way: on twelve windows of 4,096 ranks in groups of 8 and 64 the kernel takes 1,071 us with 28 KB of L1, 598 with
-// 121, 587 with 156 and 577 with 192; on records uploaded in arrival order 694, 275, 261 and 249.
+// be on their way: on twelve windows of 4,096 ranks in groups of 8 and 64 the kernel took 1,071 us with 28 KB of L1, 598 with
+// 121, 587 with 156 and 577 with 192 (541 now, with full units in short chunks).
 static_assert(CCLD_FUSED_MIN_CTAS * (sizeof(FusedShared) + 1024) <= 64 * 1024, "fits the 64 KB split (a CTA's first KB is the system's)");
 constexpr int FUSED_CARVEOUT = (int)((100 * CCLD_FUSED_MIN_CTAS * (sizeof(FusedShared) + 1024) + 228 * 1024 - 1) / (228 * 1024));     // percent
 
