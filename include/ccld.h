@@ -151,7 +151,8 @@ int ccld_comm_set_layers(ccld_ctx* ctx, uint32_t comm, const uint32_t* layer);
  * this library, e.g. ccld_get_verdict, guarantees that).
  * mem_kind 1: every pointer is device memory on the context's device, borrowed until
  * ccld_window_release or ccld_destroy; the caller keeps it alive and unchanged.
- * At most one (comm, seq, rank) record per window (else CCLD_E_DUPLICATE at the verdict).
+ * At most one (comm, seq, rank) record per window (else CCLD_E_DUPLICATE at the verdict; which copy an op is worked out from is not
+ * specified, but its row, flags and record indices go by the same one).
  * n_rec < 2^32 - 1. A window id may be uploaded once until released.
  */
 int ccld_trace_upload(ccld_ctx* ctx, uint32_t window_id, uint64_t n_rec, int mem_kind,

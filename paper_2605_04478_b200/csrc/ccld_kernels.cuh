@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc*
 
 // The same where the upload has its records in another order (see PackedRecord): few of them belong to the ranks a CTA would resolve,
 // so every record takes the two table loads, and its values, which the reading of the columns brings along whole, go to the slot
-// with its index. Two windows of 4,096 ranks in arrival order, 8.2 M records: 208 us, and the fused kernel 93 (16 bytes of tables per record from
+// with its index. Two windows of 4,096 ranks in arrival order, 8.2 M records: 232 us, and the fused kernel 93 (16 bytes of tables per record from
 // L1 or L2, 36 bytes to random sectors), where indices alone took 118 and the gathers 252; 0.5 M records each of 512 ranks 26 and 16, 17.5 and
 // 42. In rank-major order it is the other way round (a record read and written twice, 109 instead of 79 bytes).
 // Two records per thread with their values asked for together with the keys; four with the values asked for last took 219, one 283.
@@ -504,14 +504,20 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_pack(const WinDesc* wd
     sr[k] = v[k] != NONE ? srow[v[k] >> RANK_TAB_POS_BITS] : make_uint4(0, 0, 0, 0);
   }
 #pragma unroll
+  // Of two copies of a record the first one here has the slot to itself: index and sector are separate stores, and a sector that two wrote was
+  // seen half and half. The answer that is waited for costs a tenth (232 us, 211 with plain stores; an index in each half, to be compared with
+  // the table's, needs two stores instead of one: 268).
+  u64 slot[PACK_PER_THREAD]; u32 before[PACK_PER_THREAD];
+#pragma unroll
   for (int k = 0; k < PACK_PER_THREAD; ++k) {
+    before[k] = 0;
     if (v[k] == NONE) continue;
-    u64 slot;
     if (!scatter_slot(R, v[k] >> RANK_TAB_POS_BITS, sr[k].z, sr[k].w, ((u64)sr[k].x | ((u64)sr[k].y << 32)) + (u64)(v[k] & ((1u << RANK_TAB_POS_BITS) - 1)) * sr[k].z, sq[k],
-                      n_slots, &slot, &err, &rej, &internal)) continue;
-    perm[slot] = (u32)(base + (u64)k * SCAT_THREADS);
-    store_packed(packed + slot * 2, r[k]);
+                      n_slots, &slot[k], &err, &rej, &internal)) continue;
+    before[k] = atomicCAS(perm + slot[k], NONE, (u32)(base + (u64)k * SCAT_THREADS));
   }
+#pragma unroll
+  for (int k = 0; k < PACK_PER_THREAD; ++k) if (before[k] == NONE) store_packed(packed + slot[k] * 2, r[k]);
   count_rejects(D, err, rej, internal);
 }
 

@@ -546,6 +546,39 @@ def test_records_in_no_order_with_strangers():
         compare_window(an, o, 0, expect_rc=first["rc"])
 
 
+@pytest.mark.parametrize("order", ["rank", "shuffled"])
+def test_rows_and_indices_name_the_same_copy_of_a_record(order):
+    """Every record twice, the copies differing: whichever wins its slot, the op's row, its flags and the slot's index belong to it."""
+    rng = np.random.default_rng(len(order))
+    reg, cols, n = job([3, 8, 8, 8, 40] * 60, 100, rng)
+    twice = {k: np.concatenate([v, v]) for k, v in cols.items()}
+    half = len(cols["seq"])
+    twice["t_enter"][half:] += 7_000_000
+    twice["t_exit"][half:] += 7_000_000 + rng.integers(1, 9, half) * 1000
+    twice["bytes"][half:] += 4
+    twice["send_chg"][half:] += 100
+    i = rng.permutation(2 * half) if order == "shuffled" else np.lexsort((twice["t_enter"], twice["seq"], twice["comm"], twice["rank"]))
+    cols = {k: v[i] for k, v in twice.items()}
+    an = make_pair(reg)[0]
+    an.trace_upload(0, cols)
+    for _ in range(12):
+        an.reset()
+        an.analyze_window(0, 1, 10**13)
+        v = an.get_verdict(0, check=False)
+        assert v["rc"] == -10 and v["n_rejected"] == half and v["n_complete"] == v["n_groups"]
+        t, r = an.get_optable(0), an.get_ranges(0)
+        n_seq = r["n_seq"].astype(np.int64)
+        for g0, s0, k, ns in zip(np.cumsum(n_seq) - n_seq, r["slot0"].astype(np.int64), r["n"].astype(np.int64), n_seq):
+            at = t["perm"][s0:s0 + k * ns].reshape(k, ns)
+            te, du = cols["t_enter"][at], cols["t_exit"][at] - cols["t_enter"][at]
+            same(t["e_min"][g0:g0 + ns], te.min(0), "e_min")
+            same(t["t_max"][g0:g0 + ns], du.max(0), "t_max")
+            same(t["t_min"][g0:g0 + ns], du.min(0), "t_min")
+            same(t["max_chg"][g0:g0 + ns], np.maximum(cols["send_chg"][at], cols["recv_chg"][at]).max(0), "max_chg")
+            by = cols["bytes"][at]
+            same(t["gflags"][g0:g0 + ns] & 8 != 0, (by != by[0]).any(0), "sizes differ")
+
+
 def test_pinned_upload_beyond_what_a_kernel_reads():
     """More than 32 MB of pinned columns are copied column by column."""
     rng = np.random.default_rng(8)
