@@ -503,7 +503,6 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_pack(const WinDesc* wd
     }
     sr[k] = v[k] != NONE ? srow[v[k] >> RANK_TAB_POS_BITS] : make_uint4(0, 0, 0, 0);
   }
-#pragma unroll
   // Of two copies of a record the first one here has the slot to itself: index and sector are separate stores, and a sector that two wrote was
   // seen half and half. The answer that is waited for costs a tenth (232 us, 211 with plain stores; an index in each half, to be compared with
   // the table's, needs two stores instead of one: 268).
