@@ -414,6 +414,14 @@ int ccld_timing_enable(ccld_ctx* ctx, int on);
 int ccld_get_kernel_times(ccld_ctx* ctx, double* ms /* host [CCLD_K_KINDS] */, uint64_t* launches /* host [CCLD_K_KINDS] */);
 
 /*
+ * How this context's batches were analysed since it was created, for tests and inspection tools: [0] enqueued without waiting
+ * for their layout, [1] analysed a second time because it was not the expected one, [2] with their records copied to their slots
+ * (records in another order than their ranks'), [3] with the slot table filled during the op-counter pass (large tables).
+ */
+#define CCLD_ROUTES 4
+int ccld_get_route_counts(ccld_ctx* ctx, uint64_t* counts /* host [CCLD_ROUTES] */);
+
+/*
  * Hang location for one ring without any allocation. The paper has no counterpart to this entry
  * point; it exists for callers that cannot allocate device memory when they need a diagnosis: a
  * watchdog thread looking at a job whose memory is exhausted or whose allocator sits behind the

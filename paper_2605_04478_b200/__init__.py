@@ -25,10 +25,11 @@ MAX_ALERTS_PER_WINDOW = 1024
 EXPORTS = ("ccld_params_default", "ccld_create", "ccld_destroy", "ccld_last_error", "ccld_comm_register",
            "ccld_trace_upload", "ccld_window_release", "ccld_analyze_window", "ccld_reset", "ccld_get_verdict",
            "ccld_locate_hang", "ccld_get_optable", "ccld_get_ranges", "ccld_get_rank_stats", "ccld_copy_to_host",
-           "ccld_timing_enable", "ccld_get_kernel_times", "ccld_set_speculation", "ccld_ring_locate_static", "ccld_derive_rates", "ccld_locate_hangs", "ccld_state_export", "ccld_state_import", "ccld_trace_attach_opset", "ccld_opset_check",
+           "ccld_timing_enable", "ccld_get_kernel_times", "ccld_set_speculation", "ccld_get_route_counts", "ccld_ring_locate_static", "ccld_derive_rates", "ccld_locate_hangs", "ccld_state_export", "ccld_state_import", "ccld_trace_attach_opset", "ccld_opset_check",
            "ccld_comm_set_layers", "ccld_copy_many_to_host", "ccld_get_verdict_columns", "ccld_take_optable", "ccld_take_rank_stats",
            "ccld_host_release")
 STATIC_MAX_MEMBERS = 8192
+ROUTES = ("unwaited", "redone", "packed", "filled_under_range")
 KERNEL_KINDS = ("k_seq_range", "k_plan", "k_slot_scatter", "k_reduce_fused", "k_reduce_mid", "k_reduce_large", "k_window_decide")
 
 
@@ -139,6 +140,7 @@ def load_library() -> C.CDLL:
         lib.ccld_analyze_window.argtypes = [C.c_void_p, C.c_uint32, C.c_uint32, C.c_int64]
         lib.ccld_reset.argtypes = [C.c_void_p]
         lib.ccld_set_speculation.argtypes = [C.c_void_p, C.c_int]
+        lib.ccld_get_route_counts.argtypes = [C.c_void_p, C.c_void_p]
         lib.ccld_get_verdict.argtypes = [C.c_void_p, C.c_uint32, C.POINTER(Verdict)]
         lib.ccld_locate_hang.argtypes = [C.c_void_p, C.c_uint32, C.c_uint32, C.c_uint32, C.POINTER(HangVerdict)]
         lib.ccld_trace_attach_opset.argtypes = [C.c_void_p, C.c_uint32, C.c_int, C.c_void_p, C.c_void_p]
@@ -433,6 +435,12 @@ class Analyzer:
         ms = np.zeros(len(KERNEL_KINDS), np.float64); n = np.zeros(len(KERNEL_KINDS), np.uint64)
         self._check(self.lib.ccld_get_kernel_times(self.h, ms.ctypes.data, n.ctypes.data))
         return {k: {"ms": float(ms[i]), "launches": int(n[i])} for i, k in enumerate(KERNEL_KINDS)}
+
+    def get_route_counts(self) -> Dict[str, int]:
+        """Batches of this context by the way they were analysed (ccld_get_route_counts)."""
+        n = np.zeros(len(ROUTES), np.uint64)
+        self._check(self.lib.ccld_get_route_counts(self.h, n.ctypes.data))
+        return {k: int(x) for k, x in zip(ROUTES, n)}
 
     def derive_rates(self, rank, t_enter, t_exit, tick_off, tick_ns, send_count, recv_count):
         """ccld_derive_rates: counter changes per record from raw probe samples (Sec. 4.1.2). All inputs are tensors on

@@ -99,7 +99,8 @@ constexpr int N_CLASSES = 4;           // reduction code paths: n <= 8, <= 128, 
 // 401, 382, 361; smaller jobs alike. With 16 the lists take 7 us longer to write and nothing is gained.
 constexpr u32 CHUNK_REF = 32;          // op counters per chunk of the busiest communicator of a window
 constexpr u32 CHUNK_MAX = 64;          // at most this many chunks per window (longer chunks beyond)
-enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS, T_FAILED, T_CHUNKS, T_WT_PER_CTA, T_MIXED, T_COUNT = 12 };
+enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS, T_FAILED, T_CHUNKS, T_WT_PER_CTA, T_MIXED,
+       T_FUSED, T_COUNT = 13 };        // T_FUSED: slots of classes 0 and 1, in units of 32, each communicator's rounded up
 constexpr u64 FAILED_CAPACITY = 1, FAILED_EXPECT = 2;      // T_FAILED: the window needs too many slots / its layout is not the expected one
 enum { B_FCTA = 0, B_FWT, B_FSUM, B_T2, B_T3, B_COUNT };
 

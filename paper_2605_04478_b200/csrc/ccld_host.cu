@@ -178,6 +178,7 @@ struct ccld_ctx {
   Block h_up; UploadSlot up[UP_SLOTS]; u32 up_next = 0;
   cudaStream_t up_stream = nullptr; cudaEvent_t up_event = nullptr;     // see UploadStream
   u64 batches_redone = 0;                                // batches settle() had to analyse again
+  u64 unwaited = 0, packed = 0, filled_under_range = 0;  // batches that took these ways (ccld_get_route_counts)
   std::vector<PendingBatch> pending; std::vector<Block> pinned_free; std::vector<ShapeEntry> shapes;
   u32* d_poison = nullptr; int speculate = 1;
   // optional per-kernel timing: a ring of event pairs, harvested lazily
@@ -630,7 +631,7 @@ int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* cols, u
   return CCLD_OK;
 }
 
-// Whether records stand in another order than their ranks': the range pass could not fold most of the warps' stretches.
+// Whether records stand in another order than their ranks': most of the warps' stretches in the range pass do.
 bool in_other_order(u64 mixed, u64 n_rec) { return mixed * 2 * 32 * REC_RUN > n_rec; }
 
 // Brings the batches that were enqueued on expected totals to a definite state: waits for the stream, reads the totals
@@ -1015,17 +1016,21 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   // Records in another order than their ranks' (as this shape had them last; both ways are right whatever the order): the fused
   // kernel's records go to their slots. The space is needed until the reductions are through, so whatever the stream does
   // next may have it; where it is not to be had, and in a graph, whose launches would share it, the kernel gathers.
+  // From half of the slots on, because the larger communicators' kernels read through the table anyway (4.1 M records, groups of 8 with a tenth of the
+  // slots beside rings of 256: 399 us for the batch with and 350 without; half 344 and 372, three quarters 289 and 299; groups of 4 with a quarter beside
+  // rings of 172 364 and 338, half 353 and 334), and not for records in their ranks' order (nine communicators in turn per rank: 297 and 271).
   struct PackSpace { ccld_ctx* ctx; Block b; ~PackSpace() { ctx->pool.put(b); } } pack_space{ctx, {}};
   if (expect) {
-    u64 mixed = 0, all = 0;
-    for (u32 k = 0; k < B; ++k) { mixed += tot[(size_t)k * T_COUNT + T_MIXED]; all += ws[k]->n_rec; }
+    u64 mixed = 0, all = 0, fused = 0;
+    for (u32 k = 0; k < B; ++k) { const u64* t = tot + (size_t)k * T_COUNT; mixed += t[T_MIXED]; fused += t[T_FUSED]; all += ws[k]->n_rec; }
     pbatch.mixed = in_other_order(mixed, all);
-    if (pbatch.mixed && n_list[B_FCTA] && total_slots * sizeof(PackedRecord) <= PACK_MOST && !capturing(st)) {
+    if (pbatch.mixed && n_list[B_FCTA] && fused * 32 * 2 >= total_slots && total_slots * sizeof(PackedRecord) <= PACK_MOST && !capturing(st)) {
       pack_space.b = ctx->pool.get(total_slots * sizeof(PackedRecord), &e);
       if (e != cudaSuccess) { cudaGetLastError(); pack_space.b = Block{}; }
     }
   }
   const bool pack = pack_space.b.p != nullptr;
+  if (pack) ++ctx->packed;
   for (u32 k = 0; k < B; ++k) {
     const u64* t = tot + (size_t)k * T_COUNT;
     WinDesc& d = hd[k];
@@ -1041,6 +1046,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     // beside it, two CTAs per SM together; a larger table under the range pass, which has issue slots and not memory for
     // its limit (twelve windows of 4,096 ranks, 49 M slots: 141 us for both kernels instead of 151; one window of 16.4 M: 70 instead of 65).
     const bool under_range = cta > 0 && total_slots > FILL_BESIDE;
+    ++ctx->unwaited; if (under_range) ++ctx->filled_under_range;
     const u64 want = (max_slots + 16ull * layout_threads - 1) / (16ull * layout_threads);
     CK(start_plan(under_range, under_range ? 0u : (u32)std::max<u64>(1, std::min<u64>(want, 2ull * (LAYOUT_THREADS / layout_threads) * ctx->n_sms / B))));
   } else {
@@ -1571,6 +1577,12 @@ int ccld_get_kernel_times(ccld_ctx* ctx, double* ms, uint64_t* launches) {
   CK(cudaStreamSynchronize(ctx->stream));
   for (auto& sl : ctx->ring) timer_harvest(ctx, sl);
   for (int k = 0; k < CCLD_K_KINDS; ++k) { ms[k] = ctx->t_ms[k]; launches[k] = ctx->t_launches[k]; }
+  return CCLD_OK;
+}
+
+int ccld_get_route_counts(ccld_ctx* ctx, uint64_t* counts) {
+  if (!ctx || !counts) return CCLD_ERR_ARG;
+  counts[0] = ctx->unwaited; counts[1] = ctx->batches_redone; counts[2] = ctx->packed; counts[3] = ctx->filled_under_range;
   return CCLD_OK;
 }
 

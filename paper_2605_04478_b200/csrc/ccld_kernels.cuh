@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
     for (u32 c = threadIdx.x; c < R.n_comms; c += REC_THREADS) { s_mn[c] = NONE; s_mx[c] = 0; }
     __syncthreads();
   }
-  u32 mixed = 0;                                             // stretches of 32 runs that the warp could not fold
+  u32 mixed = 0;                                             // stretches of 32 runs in another order than their ranks'
   // a CTA takes blocks_per_cta consecutive blocks of the window, one after the other, and keeps one table for them: the
   // table's set-up, its barriers and its merge into the window's ranges are paid once
   for (u32 blk = 0; blk < blocks_per_cta; ++blk) {
@@ -218,7 +218,11 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
         remaining -= cleared;
         if (!worth) break;
       }
-      mixed += remaining > 32 * REC_RUN / 2 ? 1u : 0u;
+      if (remaining > 32 * REC_RUN / 2) {
+        // Not folded: many communicators take turns. In the order of their ranks all the same if neighbouring runs mostly begin with the same rank.
+        const u32 rk = len ? D.rank[first + r0] : NONE, before = __shfl_up_sync(0xFFFFFFFFu, rk, 1);
+        mixed += __popc(__ballot_sync(0xFFFFFFFFu, lane != 0 && len != 0 && rk != before)) >= 16 ? 1u : 0u;
+      }
     }
     // folds: the communicator of the first record still left takes every record of the run that names it
     for (int f = 0; f < RANGE_FOLDS && __any_sync(0xFFFFFFFFu, left != 0); ++f) {

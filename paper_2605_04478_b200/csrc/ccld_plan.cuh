@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   begin_after();
   __shared__ PlanAcc s_warp[33];
   __shared__ u32 s_red[32];
-  __shared__ u32 s_hist[2][CHUNK_MAX];                         // units per chunk: warp-tiles of class 0, tiles of class 1
+  __shared__ u32 s_hist[2][CHUNK_MAX], s_fused;                // units per chunk: warp-tiles of class 0, tiles of class 1; slots / 32 of both
   const WinDesc& D = wd[blockIdx.y];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (blockIdx.x > 0) { fill_slots(D.perm, D.n_slots, blockIdx.x - 1, gridDim.x - 1); return; }
@@ -126,14 +126,16 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   const u32 n_warps = blockDim.x / 32;
   if (lane == 0) s_red[wid] = mx;
   for (u32 i = threadIdx.x; i < 2 * CHUNK_MAX; i += blockDim.x) (&s_hist[0][0])[i] = 0;
+  if (threadIdx.x == 0) s_fused = 0;
   __syncthreads();
   mx = __reduce_max_sync(0xFFFFFFFFu, lane < n_warps ? s_red[lane] : 0u);
   u32 T = mx ? ceil_div(mx, CHUNK_REF) : 1u;
   T = T > CHUNK_MAX ? CHUNK_MAX : T;
   // sums over my communicators, and their units along the chunks
-  PlanAcc mine = {0, 0, 0, 0, 0, 0};
+  PlanAcc mine = {0, 0, 0, 0, 0, 0}; u32 fused = 0;
   each([&](u32, u32 ns, u32 n) {
     mine = plan_add(mine, plan_item(ns, n));
+    fused += comm_class(n) <= 1 ? (u32)(((u64)ns * n + 31) / 32) : 0u;
     // communicators of one family have as many units: the lanes that agree are counted, then the lanes run along the chunks
     const u32 units = fused_units(ns, n), key = units * 2 + comm_class(n);
     u32 pend = __ballot_sync(0xFFFFFFFFu, units != 0);
@@ -144,6 +146,8 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
       pend &= ~same;
     }
   });
+  fused = __reduce_add_sync(0xFFFFFFFFu, fused);
+  if (lane == 0 && fused) atomicAdd(&s_fused, fused);
   // exclusive prefix over the threads
   PlanAcc inc = mine;
 #pragma unroll
@@ -190,7 +194,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
     t = lane == T_GROUPS ? all.groups : t; t = lane == T_SLOTS ? all.slots : t; t = lane == T_FCTA ? n_cta : t; t = lane == T_FWT ? n_wt : t;
     t = lane == T_FSUM ? all.units : t; t = lane == T_TILES2 ? all.t2 : t; t = lane == T_TILES3 ? all.t3 : t; t = lane == T_ROWS ? all.rows : t;
     t = lane == T_CHUNKS ? T : t; t = lane == T_WT_PER_CTA ? wt_per_cta : t;
-    t = lane == T_MIXED ? mixed : t;
+    t = lane == T_MIXED ? mixed : t; t = lane == T_FUSED ? s_fused : t;
     // op counters further apart than 2^31, or more slots than the cap: refuse the window
     u64 failed = (all.slots > slot_cap || all.groups > 0x7FFFFFFFull) ? FAILED_CAPACITY : 0;
     if (!failed && expects) {

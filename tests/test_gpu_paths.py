@@ -579,6 +579,44 @@ def test_rows_and_indices_name_the_same_copy_of_a_record(order):
             same(t["gflags"][g0:g0 + ns] & 8 != 0, (by != by[0]).any(0), "sizes differ")
 
 
+def in_turn(n_ranks, fams, n_seq, rng, order):
+    """Ranks that are in several communicators (groups of `fams[i]` neighbours each) and take turns over them."""
+    reg, parts = [], []
+    for n in fams:
+        for r0 in range(0, n_ranks, n):
+            reg.append((len(reg), list(range(r0, r0 + n)), 0))
+            r, s = np.meshgrid(np.arange(r0, r0 + n), np.arange(n_seq), indexing="ij")
+            parts.append((r.ravel(), np.full(r.size, reg[-1][0]), s.ravel()))
+    rank, comm, seq = (np.concatenate(x) for x in zip(*parts))
+    i = np.lexsort((comm, seq, rank)) if order == "rank" else rng.permutation(len(rank))
+    rank, comm, seq = rank[i], comm[i], seq[i]
+    te = 1_000_000_000 + seq * 20_000_000 + rng.integers(0, 40_000, len(i))
+    return reg, dict(rank=rank.astype(np.uint32), comm=comm.astype(np.uint32), seq=seq.astype(np.uint32), op=np.zeros(len(i), np.uint8),
+                     bytes=np.full(len(i), 16 * MiB, np.uint64), t_enter=te, t_exit=te + rng.integers(1_000_000, 1_200_000, len(i)),
+                     send_chg=rng.integers(0, 9, len(i)).astype(np.uint32), recv_chg=rng.integers(0, 9, len(i)).astype(np.uint32)), n_ranks
+
+
+ORDERS = {  # what, whether its records go to their slots
+    "small groups in arrival order": (lambda rng: job([8] * 60, 40, rng, order="shuffled"), True),
+    "small groups, rank by rank": (lambda rng: job([8] * 60, 40, rng), False),
+    "larger rings, three in ten records of small groups": (lambda rng: job([256] * 16 + [8] * 220, 30, rng, order="shuffled"), False),
+    "larger rings, six in ten records of small groups": (lambda rng: job([256] * 16 + [8] * 800, 30, rng, order="shuffled"), True),
+    "twelve communicators in turn, rank by rank": (lambda rng: in_turn(64, [8] * 12, 40, rng, "rank"), False),
+    "twelve communicators in turn, in arrival order": (lambda rng: in_turn(64, [8] * 12, 40, rng, "shuffled"), True),
+    "few ops of many ranks, rank by rank": (lambda rng: in_turn(512, [8, 16, 32, 64] * 3, 5, rng, "rank"), False),
+}
+
+
+@pytest.mark.parametrize("what", list(ORDERS))
+def test_which_records_go_to_their_slots(what):
+    """Only those in another order than their ranks', and only where the kernel that reads them there has half of the slots and more."""
+    make, packed = ORDERS[what]
+    reg, cols, n = make(np.random.default_rng(len(what)))
+    an, o = run(reg, cols, n)
+    again(an, o, n)
+    assert an.get_route_counts() == {"unwaited": 2, "redone": 0, "packed": 2 if packed else 0, "filled_under_range": 0}
+
+
 def test_pinned_upload_beyond_what_a_kernel_reads():
     """More than 32 MB of pinned columns are copied column by column."""
     rng = np.random.default_rng(8)
