@@ -170,6 +170,7 @@ struct ccld_ctx {
   const TreeRef* d_trees = nullptr; u32 n_trees = 0;     // tree communicators whose layers are known
   std::map<u32, WindowHost> windows;
   Pool pool; std::string err;
+  Block records;                                         // space for a batch's records in their slots (see record_space)
   cudaStream_t side[2] = {nullptr, nullptr}; cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};     // see Chains
   Block h_verdict;                                       // pinned area of ccld_get_verdict (VerdictArea)
   Block h_io;                                            // pinned area small results pass through
@@ -634,6 +635,18 @@ int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* cols, u
 // Whether records stand in another order than their ranks': most of the warps' stretches in the range pass do.
 bool in_other_order(u64 mixed, u64 n_rec) { return mixed * 2 * 32 * REC_RUN > n_rec; }
 
+// Space for `bytes` bytes of records in their slots, or null. A batch's kernels may still use it when the call that enqueued them has
+// returned, and the next batch's come after them in the stream: so it is one block that only batches use and that is not handed to
+// anything else of the context (an upload on another thread's cudaStreamPerThread is not behind those kernels).
+void* record_space(ccld_ctx* ctx, size_t bytes) {
+  if (ctx->records.bytes >= bytes) return ctx->records.p;
+  if (ctx->records.p) cudaFree(ctx->records.p);            // waits for the device
+  cudaError_t e;
+  ctx->records = ctx->pool.get(bytes, &e);
+  if (e != cudaSuccess) { cudaGetLastError(); ctx->records = Block{}; }
+  return ctx->records.p;
+}
+
 // Brings the batches that were enqueued on expected totals to a definite state: waits for the stream, reads the totals
 // their plans really found, and analyses again - this time waiting for the plan - every batch from the first one whose
 // expectation failed (that batch and all later ones gave up on the device without touching any state, so the order of
@@ -739,7 +752,7 @@ int ccld_destroy(ccld_ctx* ctx) {
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) { cudaGetLastError(); cudaDeviceSynchronize(); }      // (the caller's stream may be gone)
   for (auto& kv : ctx->windows) { drop_results(kv.second); if (kv.second.owns) ctx->pool.put(kv.second.own); if (kv.second.owns_opset) ctx->pool.put(kv.second.opset_own); }
   ctx->windows.clear();
-  ctx->pool.put(ctx->reg_blk); ctx->pool.put(ctx->misc_blk);
+  ctx->pool.put(ctx->reg_blk); ctx->pool.put(ctx->misc_blk); ctx->pool.put(ctx->records);
   ctx->pool.leave_all();
   for (auto& b : ctx->pending) ctx->pinned_free.push_back(b.pin);
   ctx->pinned_free.push_back(ctx->h_verdict); ctx->pinned_free.push_back(ctx->h_io); ctx->pinned_free.push_back(ctx->h_up);
@@ -1014,28 +1027,25 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   auto res_blk = std::make_shared<Shared>(&ctx->pool, rb);
   char* rbase = (char*)rb.p;
   // Records in another order than their ranks' (as this shape had them last; both ways are right whatever the order): the fused
-  // kernel's records go to their slots. The space is needed until the reductions are through, so whatever the stream does
-  // next may have it; where it is not to be had, and in a graph, whose launches would share it, the kernel gathers.
+  // kernel's records go to their slots. Where the space is not to be had, and in a graph, whose launches would share it, the kernel gathers.
   // From half of the slots on, because the larger communicators' kernels read through the table anyway (4.1 M records, groups of 8 with a tenth of the
   // slots beside rings of 256: 399 us for the batch with and 350 without; half 344 and 372, three quarters 289 and 299; groups of 4 with a quarter beside
   // rings of 172 364 and 338, half 353 and 334), and not for records in their ranks' order (nine communicators in turn per rank: 297 and 271).
-  struct PackSpace { ccld_ctx* ctx; Block b; ~PackSpace() { ctx->pool.put(b); } } pack_space{ctx, {}};
+  void* records = nullptr;
   if (expect) {
     u64 mixed = 0, all = 0, fused = 0;
     for (u32 k = 0; k < B; ++k) { const u64* t = tot + (size_t)k * T_COUNT; mixed += t[T_MIXED]; fused += t[T_FUSED]; all += ws[k]->n_rec; }
     pbatch.mixed = in_other_order(mixed, all);
-    if (pbatch.mixed && n_list[B_FCTA] && fused * 32 * 2 >= total_slots && total_slots * sizeof(PackedRecord) <= PACK_MOST && !capturing(st)) {
-      pack_space.b = ctx->pool.get(total_slots * sizeof(PackedRecord), &e);
-      if (e != cudaSuccess) { cudaGetLastError(); pack_space.b = Block{}; }
-    }
+    if (pbatch.mixed && n_list[B_FCTA] && fused * 32 * 2 >= total_slots && total_slots * sizeof(PackedRecord) <= PACK_MOST && !capturing(st))
+      records = record_space(ctx, total_slots * sizeof(PackedRecord));
   }
-  const bool pack = pack_space.b.p != nullptr;
+  const bool pack = records != nullptr;
   if (pack) ++ctx->packed;
   for (u32 k = 0; k < B; ++k) {
     const u64* t = tot + (size_t)k * T_COUNT;
     WinDesc& d = hd[k];
     d.n_groups = t[T_GROUPS]; d.n_slots = t[T_SLOTS];
-    if (pack) d.packed = (uint4*)pack_space.b.p + perm_off[k] / 2;         // 32 bytes where perm has 4
+    if (pack) d.packed = (uint4*)records + perm_off[k] / 2;                // 32 bytes where perm has 4
     d.perm = (u32*)(rbase + o_perm + perm_off[k]); d.flags = (u8*)(rbase + o_flags[k]);
     d.gi64 = (i64*)(rbase + o_gi[k]); d.gu32 = (u32*)(rbase + o_gu[k]); d.gbw = (double*)(rbase + o_gb[k]);
     d.comm_rows = (ccld_comm_verdict*)(rbase + o_rows[k]); d.alerts = (ccld_hang_alert*)(rbase + o_al[k]);

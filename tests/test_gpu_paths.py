@@ -5,6 +5,7 @@ import gc
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -615,6 +616,47 @@ def test_which_records_go_to_their_slots(what):
     an, o = run(reg, cols, n)
     again(an, o, n)
     assert an.get_route_counts() == {"unwaited": 2, "redone": 0, "packed": 2 if packed else 0, "filled_under_range": 0}
+
+
+def test_records_in_their_slots_keep_their_space_until_the_kernels_are_through():
+    """One thread's batch waits on its cudaStreamPerThread while another thread, whose stream is not behind it, uploads windows of about
+    the size of that space: the batch's records and the uploads do not meet."""
+    from types import SimpleNamespace
+    rng = np.random.default_rng(14)
+    reg, cols, n = job([8] * 60, 500, rng, order="shuffled")    # 240,000 records: 7.7 MB in their slots
+    some = cut(cols, np.sort(rng.permutation(len(cols["seq"]))[:160_000])) # 7.2 MB of columns
+    an, o = ccld.Analyzer(stream=SimpleNamespace(cuda_stream=2)), orc.Oracle()
+    for cid, ranks, seq0 in reg:
+        an.comm_register(cid, ranks, 0, seq0)
+        assert o.comm_register(cid, ranks, seq0) == 0
+    for w, c in enumerate((cols, some, some, some)):
+        assert o.upload(w, c) == 0
+    an.trace_upload(0, cols)
+    for _ in range(2):
+        an.reset()
+        an.analyze_window(0, 1, 10**13)
+        an.get_verdict(0)
+    own = torch.cuda.ExternalStream(2)
+    an.reset()
+    with torch.cuda.stream(own):
+        torch.cuda._sleep(20_000_000)                           # some 10 ms
+    an.analyze_window(0, 1, 10**13)
+
+    def upload():
+        for w in (1, 2, 3):
+            an.trace_upload(w, some)
+        torch.cuda.ExternalStream(2).synchronize()
+    t = threading.Thread(target=upload)
+    t.start()
+    t.join()
+    assert an.get_route_counts()["packed"] == 2
+    assert o.analyze(0, 1, 10**13) == 0
+    compare_window(an, o, 0)
+    an.analyze_window(1, 3, 10**13)
+    assert o.analyze(1, 3, 10**13) == 0
+    for w in (1, 2, 3):
+        compare_window(an, o, w)
+    compare_cumulative(an, o, n, 3)
 
 
 def test_pinned_upload_beyond_what_a_kernel_reads():
