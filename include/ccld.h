@@ -96,7 +96,10 @@ void ccld_params_default(ccld_params* p /* host, out */);
  * which every copy and kernel of this context is enqueued. The context owns all memory it allocates
  * and gives it up in ccld_destroy: to the driver, except for blocks that contexts of the same process
  * which are still there may use - at most 256 MB per device, and 64 MB of pinned host memory. When
- * the last context goes, those are freed too.
+ * the last context goes, those are freed too. A context that is given batches of the same shape with their records in another
+ * order than their ranks' keeps 32 bytes per record for them (per slot of the largest such batch) until it is destroyed or an
+ * allocation fails: at most 8 GB and at most half of the device memory that was free when it first took them. Where they
+ * are not to be had the analysis does without, slower.
  */
 int ccld_create(ccld_ctx** out, const ccld_params* params /* host */, int device, void* cuda_stream);
 int ccld_destroy(ccld_ctx* ctx);

@@ -93,6 +93,7 @@ class BlockStore {
 struct Pool {
   int device = 0;
   std::vector<Block> free_list;
+  Block records;                                // space for a batch's records in their slots: see record_space
   Block get(size_t bytes, cudaError_t* err) {
     bytes = align_up(std::max<size_t>(bytes, ALIGN));
     int best = -1;
@@ -107,6 +108,8 @@ struct Pool {
       cudaGetLastError();
       for (auto& f : free_list) cudaFree(f.p);
       free_list.clear();
+      if (records.p) cudaFree(records.p);      // (waits for the kernels that use it; a batch asks for it last)
+      records = Block{};
       BlockStore::get().clear();
       *err = cudaMalloc(&b.p, bytes);
       if (*err != cudaSuccess) { b.p = nullptr; b.bytes = 0; }
@@ -114,7 +117,7 @@ struct Pool {
     return b;
   }
   void put(Block b) { if (b.p) free_list.push_back(b); }
-  void leave_all() { for (auto& f : free_list) BlockStore::get().put(device, f); free_list.clear(); }      // the stream must be idle
+  void leave_all() { put(records); records = Block{}; for (auto& f : free_list) BlockStore::get().put(device, f); free_list.clear(); }      // the stream must be idle
 };
 
 struct Shared {                                 // a pooled block shared by the windows of one batch
@@ -141,7 +144,7 @@ struct WindowHost {
 // A batch that waited is listed only for its pinned block, which its last descriptor copy still reads.
 struct PendingBatch { u32 first = 0, n = 0; i64 now = 0; Block pin; bool speculative = false, mixed = false; const u64* h_tot() const { return (const u64*)pin.p; } };
 // Totals of the last batches that were planned with a wait, by shape (record count of every window).
-struct ShapeEntry { std::vector<u64> n_rec; std::vector<u64> totals; };
+struct ShapeEntry { std::vector<u64> n_rec; std::vector<u64> totals; bool no_record_space = false; };
 constexpr size_t SHAPE_CACHE = 4;
 
 // Pinned pieces that uploads of pageable memory pass through, with an event behind the last copy out of each.
@@ -153,7 +156,7 @@ constexpr u32 UP_WORKERS = 6, UP_SLOTS = 2 * UP_WORKERS;   // two pieces per wor
 // to 739 and 971), of 7 MB 308 to 475 and 248 to 361, of 69 MB 1,430 to 1,498 and 1,424 to 1,427, on a host whose PCIe others share.
 constexpr size_t UP_SMALL = 32u << 20;
 
-constexpr u64 PACK_MOST = 8ull << 30;                      // space for records in their slots, at most
+constexpr u64 PACK_MOST = 8ull << 30;                      // space for records in their slots, at most (and at most half of what is free)
 
 constexpr u32 TIMER_RING = 32;
 constexpr int TIMER_PAIRS = CCLD_K_KINDS + 1;          // two launches of the plan per call
@@ -170,7 +173,6 @@ struct ccld_ctx {
   const TreeRef* d_trees = nullptr; u32 n_trees = 0;     // tree communicators whose layers are known
   std::map<u32, WindowHost> windows;
   Pool pool; std::string err;
-  Block records;                                         // space for a batch's records in their slots (see record_space)
   cudaStream_t side[2] = {nullptr, nullptr}; cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};     // see Chains
   Block h_verdict;                                       // pinned area of ccld_get_verdict (VerdictArea)
   Block h_io;                                            // pinned area small results pass through
@@ -637,14 +639,25 @@ bool in_other_order(u64 mixed, u64 n_rec) { return mixed * 2 * 32 * REC_RUN > n_
 
 // Space for `bytes` bytes of records in their slots, or null. A batch's kernels may still use it when the call that enqueued them has
 // returned, and the next batch's come after them in the stream: so it is one block that only batches use and that is not handed to
-// anything else of the context (an upload on another thread's cudaStreamPerThread is not behind those kernels).
-void* record_space(ccld_ctx* ctx, size_t bytes) {
-  if (ctx->records.bytes >= bytes) return ctx->records.p;
-  if (ctx->records.p) cudaFree(ctx->records.p);            // waits for the device
-  cudaError_t e;
-  ctx->records = ctx->pool.get(bytes, &e);
-  if (e != cudaSuccess) { cudaGetLastError(); ctx->records = Block{}; }
-  return ctx->records.p;
+// anything else of the context (an upload on another thread's cudaStreamPerThread is not behind those kernels). Batches do without
+// it as well: it takes no more than half of the memory that is free, nothing cached is given up for it, and a shape that was
+// refused does not ask again.
+void* record_space(ccld_ctx* ctx, size_t bytes, ShapeEntry& shape) {
+  Block& have = ctx->pool.records;
+  if (have.bytes >= bytes) return have.p;
+  if (shape.no_record_space) return nullptr;
+  size_t free_bytes = 0, total = 0;
+  bool ok = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && bytes <= (free_bytes + have.bytes) / 2;
+  if (ok) {
+    if (have.p) cudaFree(have.p);                          // waits for the device
+    have = Block{};
+    if (!BlockStore::get().take(ctx->device, bytes, &have)) {
+      ok = cudaMalloc(&have.p, align_up(bytes)) == cudaSuccess;
+      if (ok) have.bytes = align_up(bytes); else have.p = nullptr;
+    }
+  }
+  if (!ok) { cudaGetLastError(); shape.no_record_space = true; }
+  return have.bytes >= bytes ? have.p : nullptr;
 }
 
 // Brings the batches that were enqueued on expected totals to a definite state: waits for the stream, reads the totals
@@ -752,7 +765,7 @@ int ccld_destroy(ccld_ctx* ctx) {
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) { cudaGetLastError(); cudaDeviceSynchronize(); }      // (the caller's stream may be gone)
   for (auto& kv : ctx->windows) { drop_results(kv.second); if (kv.second.owns) ctx->pool.put(kv.second.own); if (kv.second.owns_opset) ctx->pool.put(kv.second.opset_own); }
   ctx->windows.clear();
-  ctx->pool.put(ctx->reg_blk); ctx->pool.put(ctx->misc_blk); ctx->pool.put(ctx->records);
+  ctx->pool.put(ctx->reg_blk); ctx->pool.put(ctx->misc_blk);
   ctx->pool.leave_all();
   for (auto& b : ctx->pending) ctx->pinned_free.push_back(b.pin);
   ctx->pinned_free.push_back(ctx->h_verdict); ctx->pinned_free.push_back(ctx->h_io); ctx->pinned_free.push_back(ctx->h_up);
@@ -915,9 +928,9 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
 
   // A batch of a shape seen before (the same record count in every window) is enqueued without waiting for its plan:
   // the results are sized from the totals that shape had last time, and the plan checks them on the device.
-  const ShapeEntry* expect = nullptr;
+  ShapeEntry* expect = nullptr;
   if (may_speculate) {
-    for (const ShapeEntry& e : ctx->shapes) {
+    for (ShapeEntry& e : ctx->shapes) {
       if (e.n_rec.size() != B) continue;
       bool same = true;
       for (u32 k = 0; k < B && same; ++k) same = e.n_rec[k] == ws[k]->n_rec;
@@ -1037,7 +1050,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
     for (u32 k = 0; k < B; ++k) { const u64* t = tot + (size_t)k * T_COUNT; mixed += t[T_MIXED]; fused += t[T_FUSED]; all += ws[k]->n_rec; }
     pbatch.mixed = in_other_order(mixed, all);
     if (pbatch.mixed && n_list[B_FCTA] && fused * 32 * 2 >= total_slots && total_slots * sizeof(PackedRecord) <= PACK_MOST && !capturing(st))
-      records = record_space(ctx, total_slots * sizeof(PackedRecord));
+      records = record_space(ctx, total_slots * sizeof(PackedRecord), *expect);
   }
   const bool pack = records != nullptr;
   if (pack) ++ctx->packed;

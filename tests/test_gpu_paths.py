@@ -659,6 +659,46 @@ def test_records_in_their_slots_keep_their_space_until_the_kernels_are_through()
     compare_cumulative(an, o, n, 3)
 
 
+def test_records_in_their_slots_take_no_more_than_half_of_the_free_memory():
+    """A shape whose records do not get their space is gathered, then and later; another shape, with memory there, is not."""
+    gen = torch.Generator("cuda").manual_seed(15)
+    n_comms, n_seq = 1600, 800                                  # groups of 8: 10.2 M records, 328 MB in their slots
+    i = torch.randperm(8 * n_comms * n_seq, generator=gen, device="cuda")
+    rank, seq = i // n_seq, i % n_seq
+    te = 1_000_000_000 + seq * 5_000_000 + torch.randint(40_000, i.shape, generator=gen, device="cuda")
+    cols = dict(rank=rank.int(), comm=(rank // 8).int(), seq=seq.int(), op=torch.zeros_like(i, dtype=torch.uint8), bytes=torch.full_like(i, 16 * MiB),
+                t_enter=te, t_exit=te + torch.randint(1_000_000, 1_200_000, i.shape, generator=gen, device="cuda"))
+    an = ccld.Analyzer()
+    for c in range(n_comms):
+        an.comm_register(c, list(range(8 * c, 8 * c + 8)), 0, 0)
+    an.trace_upload(0, cols)
+    an.analyze_window(0, 1, 10**13)
+    want = an.get_optable(0)
+
+    def passes(times):
+        for _ in range(times):
+            an.reset()
+            an.analyze_window(0, 1, 10**13)
+            got = an.get_optable(0)
+            for k in want:
+                same(got[k], want[k], k)
+        return an.get_route_counts()["packed"]
+    gc.collect()
+    torch.cuda.empty_cache()
+    room = torch.empty(torch.cuda.mem_get_info()[0] - (600 << 20), dtype=torch.uint8, device="cuda")
+    assert passes(2) == 0
+    del room
+    torch.cuda.empty_cache()
+    assert passes(2) == 0
+    an.window_release(0)
+    an.trace_upload(1, {k: v[:-1] for k, v in cols.items()})
+    for _ in range(3):
+        an.reset()
+        an.analyze_window(1, 1, 10**13)
+        assert an.get_verdict(1)["n_incomplete"] == 1
+    assert an.get_route_counts()["packed"] == 2
+
+
 def test_pinned_upload_beyond_what_a_kernel_reads():
     """More than 32 MB of pinned columns are copied column by column."""
     rng = np.random.default_rng(8)
