@@ -660,6 +660,24 @@ void* record_space(ccld_ctx* ctx, size_t bytes, ShapeEntry& shape) {
   return have.bytes >= bytes ? have.p : nullptr;
 }
 
+// Whether a batch that is through found another layout than it was sized for.
+bool surprised(const PendingBatch& b) {
+  for (u32 k = 0; k < b.n; ++k) if (b.h_tot()[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) return true;
+  return false;
+}
+
+// Takes over the order that a batch's records were in, for the next one of its shape.
+void learn_order(ccld_ctx* ctx, const PendingBatch& b) {
+  u64 mixed = 0, all = 0;
+  for (u32 k = 0; k < b.n; ++k) { auto it = ctx->windows.find(b.first + k); if (it != ctx->windows.end()) { mixed += b.h_tot()[(size_t)k * T_COUNT + T_MIXED]; all += it->second.n_rec; } }
+  if (in_other_order(mixed, all) == b.mixed) return;
+  for (ShapeEntry& s : ctx->shapes) {
+    bool same = s.n_rec.size() == b.n;
+    for (u32 k = 0; k < b.n && same; ++k) { auto it = ctx->windows.find(b.first + k); same = it != ctx->windows.end() && it->second.n_rec == s.n_rec[k]; }
+    for (u32 k = 0; k < b.n && same; ++k) s.totals[(size_t)k * T_COUNT + T_MIXED] = b.h_tot()[(size_t)k * T_COUNT + T_MIXED];
+  }
+}
+
 // Brings the batches that were enqueued on expected totals to a definite state: waits for the stream, reads the totals
 // their plans really found, and analyses again - this time waiting for the plan - every batch from the first one whose
 // expectation failed (that batch and all later ones gave up on the device without touching any state, so the order of
@@ -674,18 +692,10 @@ int settle(ccld_ctx* ctx) {
   bool failed = false;
   int rc = CCLD_OK;
   for (PendingBatch& b : todo) {
-    for (u32 k = 0; k < b.n && !failed; ++k) if (b.h_tot()[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) failed = true;
+    failed = failed || surprised(b);
     ctx->pinned_free.push_back(b.pin);
     if (!failed) {
-      u64 mixed = 0, all = 0;
-      for (u32 k = 0; k < b.n; ++k) { auto it = ctx->windows.find(b.first + k); if (it != ctx->windows.end()) { mixed += b.h_tot()[(size_t)k * T_COUNT + T_MIXED]; all += it->second.n_rec; } }
-      if (in_other_order(mixed, all) != b.mixed) {           // the shape's records have come in another order this time
-        for (ShapeEntry& s : ctx->shapes) {
-          bool same = s.n_rec.size() == b.n;
-          for (u32 k = 0; k < b.n && same; ++k) { auto it = ctx->windows.find(b.first + k); same = it != ctx->windows.end() && it->second.n_rec == s.n_rec[k]; }
-          for (u32 k = 0; k < b.n && same; ++k) s.totals[(size_t)k * T_COUNT + T_MIXED] = b.h_tot()[(size_t)k * T_COUNT + T_MIXED];
-        }
-      }
+      learn_order(ctx, b);
       // a window may still have been refused for its size, which the expectation cannot have foreseen: keep what the plan found,
       // which is then no groups and no slots
       for (u32 k = 0; k < b.n; ++k) {
@@ -702,7 +712,7 @@ int settle(ccld_ctx* ctx) {
   CK(cudaMemsetAsync(ctx->d_poison, 0, 4, ctx->stream));
   failed = false;
   for (PendingBatch& b : todo) {
-    if (!failed) { for (u32 k = 0; k < b.n && !failed; ++k) if (b.h_tot()[(size_t)k * T_COUNT + T_FAILED] == FAILED_EXPECT) failed = true; }
+    failed = failed || surprised(b);
     if (!failed) continue;
     bool present = true;
     for (u32 k = 0; k < b.n; ++k) {
@@ -878,7 +888,12 @@ int ccld_reset(ccld_ctx* ctx) try {
   CK(cudaSetDevice(ctx->device));
   CK(cudaStreamSynchronize(ctx->stream));
   // batches still in doubt need no second analysis: their results are dropped with all the others
-  for (auto& b : ctx->pending) ctx->pinned_free.push_back(b.pin);
+  bool failed = false;
+  for (auto& b : ctx->pending) {
+    failed = failed || (b.speculative && surprised(b));
+    if (b.speculative && !failed) learn_order(ctx, b);
+    ctx->pinned_free.push_back(b.pin);
+  }
   ctx->pending.clear();
   for (auto& kv : ctx->windows) drop_results(kv.second);
   if (ctx->finalized) {

@@ -618,6 +618,21 @@ def test_which_records_go_to_their_slots(what):
     assert an.get_route_counts() == {"unwaited": 2, "redone": 0, "packed": 2 if packed else 0, "filled_under_range": 0}
 
 
+def test_the_order_of_the_records_is_learned_from_batches_nobody_asks_about():
+    """Analysed and reset, again and again, with a window of the shape in another order uploaded in between: the batch after the first
+    in the new order goes the other way."""
+    rng = np.random.default_rng(16)
+    reg, cols, n = job([8] * 60, 40, rng)
+    i = rng.permutation(len(cols["seq"]))
+    an, o = run(reg, cols, n)
+    an.trace_upload(1, {k: v[i] for k, v in cols.items()})
+    for w, packed in ((0, 0), (1, 0), (1, 1), (1, 2), (0, 3), (0, 3)):
+        an.reset()
+        an.analyze_window(w, 1, 10**13)
+        assert an.get_route_counts()["packed"] == packed
+    again(an, o, n, 1)
+
+
 def test_records_in_their_slots_keep_their_space_until_the_kernels_are_through():
     """One thread's batch waits on its cudaStreamPerThread while another thread, whose stream is not behind it, uploads windows of about
     the size of that space: the batch's records and the uploads do not meet."""
