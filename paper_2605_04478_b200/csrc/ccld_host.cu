@@ -152,9 +152,13 @@ struct UploadSlot { char* p = nullptr; cudaEvent_t done = nullptr; bool used = f
 constexpr size_t UP_PIECE = 1u << 20;                      // a large upload goes piece by piece
 constexpr u32 UP_WORKERS = 6, UP_SLOTS = 2 * UP_WORKERS;   // two pieces per worker: one being filled, one on its way
 // Up to this size one kernel reads the pinned columns, beyond it they are copied one by one. Nine copies leave gaps of 2 us and more between
-// them; a pass over a window of 23 MB took 723 to 1,169 us with copies and 563 to 641 with the kernel (32 CTAs per column; 8 and 16: up
-// to 739 and 971), of 7 MB 308 to 475 and 248 to 361, of 69 MB 1,430 to 1,498 and 1,424 to 1,427, on a host whose PCIe others share.
+// them: 0.6 MB take 63 us with copies and 36 with the kernel, 2.3 MB 94 and 69, 6.9 MB 180 and 160, 23 MB 473 and 474, 32 MB 639 and 654; where
+// others share the host's PCIe a pass over 23 MB took 723 to 1,169 us with copies, 563 to 641 with the kernel.
+// One CTA per column with four words per thread on their way, because reads that wait for PCIe hold up what else runs on the GPU: a matrix
+// product beside uploads takes 19 to 28 % longer, a copy of device memory 35 to 40 (beside copies 2 and 2). Twice the words: 30 and 55 % (no faster);
+// half of them 16 and 34, a quarter 5 and 11 (23 MB 477 and 482 us); 32 CTAs of 256 threads and a word each per column: 68 and 60 %.
 constexpr size_t UP_SMALL = 32u << 20;
+constexpr int UP_AHEAD = 4, UP_THREADS = 1024;
 
 constexpr u64 PACK_MOST = 8ull << 30;                      // space for records in their slots, at most (and at most half of what is free)
 
@@ -489,7 +493,7 @@ cudaError_t gather(ccld_ctx* ctx, const Piece* piece, u32 n_pieces, char* base, 
     off = at[i] + piece[i].n; most = std::max(most, piece[i].n);
     if (piece[i].n) { A.piece[k].src = (const unsigned char*)piece[i].src; A.piece[k].dst = (unsigned char*)base + at[i]; A.piece[k].n = piece[i].n; ++k; }
   }
-  if (k) launch(ctx->stream, k_gather, dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), k), GATHER_THREADS, 0, A);
+  if (k) launch(ctx->stream, k_gather<1, GATHER_THREADS>, dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), k), GATHER_THREADS, 0, A);
   return cudaGetLastError();
 }
 size_t gather_room(const Piece* piece, u32 n_pieces) { size_t t = 0; for (u32 i = 0; i < n_pieces; ++i) t += piece[i].n + 32; return t; }
@@ -608,13 +612,13 @@ int upload_pageable(ccld_ctx* ctx, char* base, size_t total, const UpCol* col, u
 // column by column through its own buffers, one thread, 10 us and more per call. A small upload is put together in one
 // pinned piece instead and crosses in one copy; a large one is cut into pieces that several threads fill while earlier ones
 // cross. Pageable columns are read by the time the call returns. Any other column is read when its turn in the stream comes, so
-// that what earlier work of the stream still writes there is what arrives: very large ones go straight across, the others are
+// that what earlier work of the stream still writes there is what arrives: large ones go straight across, the others are
 // read by one kernel.
 int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* cols, u32 n_cols) {
   cudaStream_t st = ctx->stream;
   UpCol col[UP_COLS]; u32 n_page = 0;                      // the pageable columns
   UpCol far[UP_COLS]; u32 n_far = 0;                       // those that are copied one by one
-  GatherArgs G; u32 n_near = 0; size_t most = 0;           // those that a kernel reads
+  GatherArgs G; u32 n_near = 0;                            // those that a kernel reads
   for (u32 i = 0; i < n_cols; ++i) {
     if (!cols[i].n) continue;
     cudaPointerAttributes at;
@@ -622,13 +626,13 @@ int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* cols, u
     if (at.type == cudaMemoryTypeUnregistered) col[n_page++] = cols[i];
     else if (total <= UP_SMALL && at.type == cudaMemoryTypeHost && at.devicePointer && ((uintptr_t)at.devicePointer & 15) == 0) {
       auto& g = G.piece[n_near++];
-      g.src = (const unsigned char*)at.devicePointer; g.dst = (unsigned char*)base + cols[i].off; g.n = cols[i].n; most = std::max(most, cols[i].n);
+      g.src = (const unsigned char*)at.devicePointer; g.dst = (unsigned char*)base + cols[i].off; g.n = cols[i].n;
     } else far[n_far++] = cols[i];
   }
   if (n_page) { int rc = upload_pageable(ctx, base, total, col, n_page); if (rc != CCLD_OK) return rc; }
   for (u32 i = 0; i < n_far; ++i) CK(cudaMemcpyAsync(base + far[i].off, far[i].src, far[i].n, cudaMemcpyHostToDevice, st));
   if (n_near) {
-    launch(On(st, false), k_gather, dim3((u32)std::min<size_t>((most + 16 * GATHER_THREADS - 1) / (16 * GATHER_THREADS), 32), n_near), GATHER_THREADS, 0, G);
+    launch(On(st, false), k_gather<UP_AHEAD, UP_THREADS>, dim3(1, n_near), UP_THREADS, 0, G);
     CK(cudaGetLastError());
   }
   return CCLD_OK;

@@ -210,18 +210,28 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_merge(VerdictArgs A, Reg
 }
 
 // Several device arrays into one pinned area, one launch: a row of CTAs per piece. Source and destination agree modulo 16, so
-// whole 16-byte words cross PCIe and only a piece's ends go byte by byte.
+// whole 16-byte words cross PCIe and only a piece's ends go byte by byte. AHEAD: words a thread asks for at once.
 constexpr int GATHER_THREADS = 256;
 constexpr u32 GATHER_PIECES = 24;
 struct GatherArgs { struct { const unsigned char* src; unsigned char* dst; u64 n; } piece[GATHER_PIECES]; };
-__global__ void __launch_bounds__(GATHER_THREADS) k_gather(GatherArgs A) {
+template <int AHEAD, int THREADS> __global__ void __launch_bounds__(THREADS) k_gather(GatherArgs A) {
   begin_after();
   const unsigned char* src = A.piece[blockIdx.y].src; unsigned char* __restrict__ dst = A.piece[blockIdx.y].dst;
   const u64 n = A.piece[blockIdx.y].n;
   const u64 head = min(n, (u64)((16 - ((uintptr_t)src & 15)) & 15)), n16 = (n - head) / 16, tail = head + n16 * 16;
-  const u64 i0 = (u64)blockIdx.x * GATHER_THREADS + threadIdx.x, st = (u64)gridDim.x * GATHER_THREADS;
+  const u64 i0 = (u64)blockIdx.x * THREADS + threadIdx.x, st = (u64)gridDim.x * THREADS;
   const uint4* s16 = reinterpret_cast<const uint4*>(src + head); uint4* d16 = reinterpret_cast<uint4*>(dst + head);
-  for (u64 i = i0; i < n16; i += st) d16[i] = s16[i];
+  u64 i = i0;
+  if constexpr (AHEAD > 1) {
+    for (; i + (AHEAD - 1) * st < n16; i += AHEAD * st) {
+      uint4 v[AHEAD];
+#pragma unroll
+      for (int k = 0; k < AHEAD; ++k) v[k] = s16[i + k * st];
+#pragma unroll
+      for (int k = 0; k < AHEAD; ++k) d16[i + k * st] = v[k];
+    }
+  }
+  for (; i < n16; i += st) d16[i] = s16[i];
   if (i0 < head) dst[i0] = src[i0];
   if (i0 < n - tail) dst[tail + i0] = src[tail + i0];
 }

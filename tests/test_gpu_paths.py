@@ -714,6 +714,12 @@ def test_records_in_their_slots_take_no_more_than_half_of_the_free_memory():
     assert an.get_route_counts()["packed"] == 2
 
 
+# a thread of the uploading kernel has four words of 16 bytes on their way: columns of 4 and 8 bytes around multiples of 1,024 x 4 words
+@pytest.mark.parametrize("n_rec", [4095, 4097, 8191, 8192, 8193, 12_289, 16_383, 16_384, 16_387])
+def test_pinned_columns_around_the_words_a_kernel_has_in_flight(n_rec):
+    test_uploads(n_rec, True)
+
+
 def test_pinned_upload_beyond_what_a_kernel_reads():
     """More than 32 MB of pinned columns are copied column by column."""
     rng = np.random.default_rng(8)
