@@ -676,16 +676,9 @@ def test_records_in_their_slots_keep_their_space_until_the_kernels_are_through()
 
 def test_records_in_their_slots_take_no_more_than_half_of_the_free_memory():
     """A shape whose records do not get their space is gathered, then and later; another shape, with memory there, is not."""
-    gen = torch.Generator("cuda").manual_seed(15)
-    n_comms, n_seq = 1600, 800                                  # groups of 8: 10.2 M records, 328 MB in their slots
-    i = torch.randperm(8 * n_comms * n_seq, generator=gen, device="cuda")
-    rank, seq = i // n_seq, i % n_seq
-    te = 1_000_000_000 + seq * 5_000_000 + torch.randint(40_000, i.shape, generator=gen, device="cuda")
-    cols = dict(rank=rank.int(), comm=(rank // 8).int(), seq=seq.int(), op=torch.zeros_like(i, dtype=torch.uint8), bytes=torch.full_like(i, 16 * MiB),
-                t_enter=te, t_exit=te + torch.randint(1_000_000, 1_200_000, i.shape, generator=gen, device="cuda"))
-    an = ccld.Analyzer()
-    for c in range(n_comms):
-        an.comm_register(c, list(range(8 * c, 8 * c + 8)), 0, 0)
+    sizes = [8] * 1600
+    cols = device_job(sizes, 800, 15, order="shuffled")         # 10.2 M records, 328 MB in their slots
+    an = device_analyzer(sizes)
     an.trace_upload(0, cols)
     an.analyze_window(0, 1, 10**13)
     want = an.get_optable(0)
@@ -718,6 +711,110 @@ def test_records_in_their_slots_take_no_more_than_half_of_the_free_memory():
 @pytest.mark.parametrize("n_rec", [4095, 4097, 8191, 8192, 8193, 12_289, 16_383, 16_384, 16_387])
 def test_pinned_columns_around_the_words_a_kernel_has_in_flight(n_rec):
     test_uploads(n_rec, True)
+
+
+def test_several_windows_with_records_in_their_slots():
+    """A batch of three windows of different record counts, members missing and in flight, with communicators beside them that read
+    through the table."""
+    rng = np.random.default_rng(17)
+    sizes = [3] * 40 + [8] * 100 + [64] * 10 + [200, 1100]      # 1,560 of 2,860 slots per op counter are read where the records lie
+    o, wins = None, []
+    for w in range(3):
+        reg, cols, n = job(sizes, 20 + 13 * w, rng, order="shuffled")
+        cols["t_exit"][rng.random(len(cols["seq"])) < 0.002] = -1
+        wins.append(cut(cols, rng.random(len(cols["seq"])) >= 0.002))
+    an, o = make_pair(reg)
+    for w, c in enumerate(wins):
+        an.trace_upload(w, c)
+        assert o.upload(w, c) == 0
+    assert o.analyze(0, 3, 10**13) == 0
+    for _ in range(3):
+        an.reset()
+        an.analyze_window(0, 3, 10**13)
+        for w in range(3):
+            compare_window(an, o, w)
+        compare_cumulative(an, o, n, 2)
+    assert an.get_route_counts() == {"unwaited": 2, "redone": 0, "packed": 2, "filled_under_range": 0}
+
+
+def test_a_captured_batch_gathers():
+    """In a graph the space of records in their slots would be shared by whatever is launched beside it: a captured call does without."""
+    rng = np.random.default_rng(18)
+    reg, cols, n = job([8] * 60, 40, rng, order="shuffled")
+    st = torch.cuda.Stream()
+    an = ccld.Analyzer(stream=st)
+    for cid, ranks, seq0 in reg:
+        an.comm_register(cid, ranks, 0, seq0)
+    an, o = run(reg, cols, n, an=an)
+    again(an, o, n, 1)
+    assert an.get_route_counts()["packed"] == 1
+    an.reset()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        an.analyze_window(0, 1, 10**13)
+    with torch.cuda.stream(st):
+        g.replay()
+    torch.cuda.synchronize()
+    assert an.get_route_counts()["packed"] == 1
+    compare_window(an, o, 0)
+    compare_cumulative(an, o, n, 0)
+    again(an, o, n, 1)
+    assert an.get_route_counts()["packed"] == 2
+
+
+def device_job(sizes, n_seq, seed, order="rank", lost=0):
+    """Columns on the GPU: a communicator per entry of `sizes` over ranks of its own, n_seq ops each, `lost` records missing."""
+    gen = torch.Generator("cuda").manual_seed(seed)
+    rnd = lambda lo, hi, n: torch.randint(lo, hi, (n,), generator=gen, device="cuda")
+    n_rec = sum(sizes) * n_seq
+    i = torch.randperm(n_rec, generator=gen, device="cuda")[lost:]
+    if order == "rank":
+        i = torch.sort(i).values
+    rank, seq, n = i // n_seq, i % n_seq, len(i)
+    comm = torch.repeat_interleave(torch.arange(len(sizes), device="cuda"), torch.tensor(sizes, device="cuda"))[rank]
+    te = 1_000_000_000 + seq * 5_000_000 + rnd(0, 40_000, n)
+    return dict(rank=rank.int(), comm=comm.int(), seq=seq.int(), op=torch.zeros(n, dtype=torch.uint8, device="cuda"),
+                bytes=torch.full((n,), 16 * MiB, device="cuda"), t_enter=te, t_exit=te + rnd(1_000_000, 1_200_000, n))
+
+
+def device_analyzer(sizes):
+    an, r0 = ccld.Analyzer(), 0
+    for c, n in enumerate(sizes):
+        an.comm_register(c, list(range(r0, r0 + n)), 0, 0)
+        r0 += n
+    return an
+
+
+def test_a_large_slot_table_filled_during_the_range_pass():
+    """27 M slots in two windows, the second one's table at no 16-byte boundary, on memory that holds the indices of windows that lost
+    other records: what the waiting pass, which fills its table with a copy of its own, finds."""
+    sizes = [8] * 1500 + [5] * 301
+    first = [device_job(sizes, 1001, s, lost=4000) for s in (1, 2)]
+    then = [device_job(sizes, 1001, s, lost=4000) for s in (3, 4)]
+    an = device_analyzer(sizes)
+    for wins in (first, then):
+        for w, c in enumerate(wins):
+            an.trace_upload(w, c)
+        for _ in range(2):
+            an.reset()
+            an.analyze_window(0, 2, 10**13)
+            got = [an.get_optable(w) for w in (0, 1)]
+        if wins is first:
+            del got
+            for w in (0, 1):
+                an.window_release(w)
+    assert an.get_route_counts() == {"unwaited": 3, "redone": 0, "packed": 0, "filled_under_range": 3}
+    waiting = device_analyzer(sizes)
+    waiting.set_speculation(False)
+    for w, c in enumerate(then):
+        waiting.trace_upload(w, c)
+    waiting.analyze_window(0, 2, 10**13)
+    for w in (0, 1):
+        want = waiting.get_optable(w)
+        for k in want:
+            same(got[w][k], want[k], k)
+    assert waiting.get_route_counts()["unwaited"] == 0
 
 
 def test_pinned_upload_beyond_what_a_kernel_reads():
