@@ -23,7 +23,7 @@ constexpr int REC_PER_CTA = REC_THREADS * REC_PER_THREAD;
 constexpr int SMALL_N = 8;             // communicators of up to 8 ranks: one thread per group
 constexpr int SMALL_SEQS = 256;        //   threads per CTA: eight warps, each on a warp-tile of up to 32 op counters at a time
 constexpr u32 FUSED_WT_PER_CTA = 16;   //   warp-tiles a CTA works through: two per warp, or one where that gives every tile of the batch a
-constexpr u32 FUSED_WARPS = 148 * 3 * 8;   //   warp of its own (three CTAs of eight warps on each of a B200's SMs)
+                                       //   warp of its own at once
 constexpr int WARP_N = 128;            // up to 128 ranks: a CTA per tile of op counters, n_pad / 8 lanes per group
 constexpr int MID_ELEMS = 2048;        //   padded records per tile of a communicator of 9 to 128 ranks
 constexpr int MID_N = 1024;            // up to 1024 ranks: a warp per group, keys in its registers (as far as 32 per lane go; ns per op

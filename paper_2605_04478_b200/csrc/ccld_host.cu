@@ -1016,7 +1016,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
       TimedLaunch tl(ts, 0, st);
       launch(st, k_seq_range, dim3((u32)((cta + per - 1) / per), B), REC_THREADS, range_smem_bytes(nc), d_desc, ctx->reg, per, fill);
     }
-    { TimedLaunch tl(ts, 1, st); launch(st, k_layout, dim3(1 + fill_ctas, B), layout_threads, 0, d_desc, ctx->reg); }
+    { TimedLaunch tl(ts, 1, st); launch(st, k_layout, dim3(1 + fill_ctas, B), layout_threads, 0, d_desc, ctx->reg, ctx->n_sms * CCLD_FUSED_MIN_CTAS * (SMALL_SEQS / 32)); }
     return cudaGetLastError();
   };
   const u64* tot = nullptr;                                // [B][T_COUNT] totals the results are sized from

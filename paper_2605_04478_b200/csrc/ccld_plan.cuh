@@ -87,8 +87,8 @@ struct PlanLists { FusedCta* fcta; WarpTile* fwt; Tile* t2; Tile* t3; };
 // When the host sized the results from totals it expected (D.expect) instead of waiting for these, a window whose totals
 // differ gives up and raises the poison flag; so does every window planned after the flag went up - in the same batch
 // (seen by emit_lists) or in a later one - so that windows are never analysed out of order.
-// Grid: (1 + filling CTAs, windows).
-__global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Registry R) {
+// Grid: (1 + filling CTAs, windows). fused_warps: warps of k_reduce_fused that run at a time.
+__global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Registry R, u32 fused_warps) {
   begin_after();
   __shared__ PlanAcc s_warp[33];
   __shared__ u32 s_red[32];
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
     for (int q = 0; q < 2; ++q) { wt[q] = s_hist[0][2 * lane + q]; c1[q] = s_hist[1][2 * lane + q]; }
     // (gridDim.y: windows of the batch, which are mostly alike)
     const u32 wt_all = __reduce_add_sync(0xFFFFFFFFu, wt[0] + wt[1]);
-    wt_per_cta = (u64)wt_all * gridDim.y <= FUSED_WARPS ? FUSED_WT_PER_CTA / 2 : FUSED_WT_PER_CTA;
+    wt_per_cta = (u64)wt_all * gridDim.y <= fused_warps ? FUSED_WT_PER_CTA / 2 : FUSED_WT_PER_CTA;
     const u32 a0 = ceil_div(wt[0], wt_per_cta) + c1[0], a1 = ceil_div(wt[1], wt_per_cta) + c1[1];
     u32 pc = a0 + a1, pw = wt[0] + wt[1];                      // CTAs and warp-tiles of my two chunks
     const u32 oc_ = pc, ow_ = pw;

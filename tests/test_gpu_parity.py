@@ -684,7 +684,7 @@ def test_a_batch_that_does_not_match_its_expected_layout_is_analysed_again_in_or
         an.analyze_window(w, 1, now)
     assert o.analyze(0, spec.n_windows, now) == 0
     v2 = an.get_verdict(2, check=False)
-    # the layout kernel runs twice per analysed batch: five calls, and - when calls do not wait - windows 2, 3 and 4 once more
+    # k_begin and k_layout count as one kind, two launches per analysed batch: five calls, and - when calls do not wait - windows 2, 3 and 4 once more
     assert an.get_kernel_times()["k_plan"]["launches"] == (16 if speculate else 10)
     an.timing_enable(False)
     assert v2["n_incomplete"] == o.sizes(2)["n_incomplete"] > 400 and v2["n_groups"] == o.sizes(2)["n_groups"] > o.sizes(1)["n_groups"] + 400
