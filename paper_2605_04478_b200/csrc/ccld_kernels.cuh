@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
     for (u32 c = threadIdx.x; c < R.n_comms; c += REC_THREADS) { s_mn[c] = NONE; s_mx[c] = 0; }
     __syncthreads();
   }
-  u32 mixed = 0;                                             // stretches of 32 runs in another order than their ranks'
+  u32 mixed = 0;                                             // stretches of 32 runs that the warp could not fold
   // a CTA takes blocks_per_cta consecutive blocks of the window, one after the other, and keeps one table for them: the
   // table's set-up, its barriers and its merge into the window's ranges are paid once
   for (u32 blk = 0; blk < blocks_per_cta; ++blk) {
@@ -218,11 +218,7 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
         remaining -= cleared;
         if (!worth) break;
       }
-      if (remaining > 32 * REC_RUN / 2) {
-        // Not folded: many communicators take turns. In the order of their ranks all the same if neighbouring runs mostly begin with the same rank.
-        const u32 rk = len ? D.rank[first + r0] : NONE, before = __shfl_up_sync(0xFFFFFFFFu, rk, 1);
-        mixed += __popc(__ballot_sync(0xFFFFFFFFu, lane != 0 && len != 0 && rk != before)) >= 16 ? 1u : 0u;
-      }
+      mixed += remaining > 32 * REC_RUN / 2 ? 1u : 0u;
     }
     // folds: the communicator of the first record still left takes every record of the run that names it
     for (int f = 0; f < RANGE_FOLDS && __any_sync(0xFFFFFFFFu, left != 0); ++f) {
@@ -280,6 +276,13 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
         }
       }
     }
+  }
+  if (mixed != 0) {
+    // Many communicators take turns. In the order of their ranks all the same if the runs of the warp's first stretch mostly begin with the
+    // rank of the run before. (Looked at once and not in the loop, where it costs every upload 4 % of the pass.)
+    const u64 at = (u64)blockIdx.x * blocks_per_cta * REC_PER_CTA + threadIdx.x * REC_RUN;
+    const u32 rk = at < n_rec ? D.rank[at] : NONE, before = __shfl_up_sync(0xFFFFFFFFu, rk, 1);
+    if (__popc(__ballot_sync(0xFFFFFFFFu, lane != 0 && at < n_rec && rk != before)) < 16) mixed = 0;
   }
   if (lane == 0) count_add(D.counters, C_MIXED, mixed);
   if (s_mn == nullptr) return;
@@ -448,9 +451,8 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc*
 
 // The same where the upload has its records in another order (see PackedRecord): few of them belong to the ranks a CTA would resolve,
 // so every record takes the two table loads, and its values, which the reading of the columns brings along whole, go to the slot
-// with its index. Two windows of 4,096 ranks in arrival order, 8.2 M records: 232 us, and the fused kernel 93 (16 bytes of tables per record from
-// L1 or L2, 36 bytes to random sectors), where indices alone took 118 and the gathers 252; 0.5 M records each of 512 ranks 26 and 16, 17.5 and
-// 42. In rank-major order it is the other way round (a record read and written twice, 109 instead of 79 bytes).
+// with its index. Two windows of 4,096 ranks in arrival order, 8.2 M records: 232 us, and the fused kernel 98 (48 bytes of tables per record from
+// L1 or L2, 36 bytes to random sectors), where indices alone take 129 and the gathers 252; 0.5 M records each of 512 ranks 35 and 19, 24 and 36. In rank-major order it is the other way round (a record read and written twice, 109 instead of 79 bytes).
 // Two records per thread with their values asked for together with the keys; four with the values asked for last took 219, one 283.
 constexpr int PACK_PER_THREAD = 2;
 constexpr int PACK_PER_CTA = SCAT_THREADS * PACK_PER_THREAD;
