@@ -101,6 +101,8 @@ constexpr u32 CHUNK_REF = 32;          // op counters per chunk of the busiest c
 constexpr u32 CHUNK_MAX = 64;          // at most this many chunks per window (longer chunks beyond)
 enum { T_GROUPS = 0, T_SLOTS, T_FCTA, T_FWT, T_FSUM, T_TILES2, T_TILES3, T_ROWS, T_FAILED, T_CHUNKS, T_WT_PER_CTA, T_MIXED,
        T_FUSED, T_COUNT = 13 };        // T_FUSED: slots of classes 0 and 1, in units of 32, each communicator's rounded up
+// Whether most stretches (of 32 threads' records in the range pass) are among the `mixed` ones.
+__host__ __device__ inline bool mostly_mixed(u64 mixed, u64 n_rec) { return mixed * 2 * 32 * REC_PER_THREAD > n_rec; }
 constexpr u64 FAILED_CAPACITY = 1, FAILED_EXPECT = 2;      // T_FAILED: the window needs too many slots / its layout is not the expected one
 enum { B_FCTA = 0, B_FWT, B_FSUM, B_T2, B_T3, B_COUNT };
 

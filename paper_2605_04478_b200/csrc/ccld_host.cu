@@ -638,9 +638,6 @@ int upload_columns(ccld_ctx* ctx, char* base, size_t total, const UpCol* cols, u
   return CCLD_OK;
 }
 
-// Whether records stand in another order than their ranks': most of the warps' stretches in the range pass do.
-bool in_other_order(u64 mixed, u64 n_rec) { return mixed * 2 * 32 * REC_RUN > n_rec; }
-
 // Space for `bytes` bytes of records in their slots, or null. A batch's kernels may still use it when the call that enqueued them has
 // returned, and the next batch's come after them in the stream: so it is one block that only batches use and that is not handed to
 // anything else of the context (an upload on another thread's cudaStreamPerThread is not behind those kernels). Batches do without
@@ -674,7 +671,7 @@ bool surprised(const PendingBatch& b) {
 void learn_order(ccld_ctx* ctx, const PendingBatch& b) {
   u64 mixed = 0, all = 0;
   for (u32 k = 0; k < b.n; ++k) { auto it = ctx->windows.find(b.first + k); if (it != ctx->windows.end()) { mixed += b.h_tot()[(size_t)k * T_COUNT + T_MIXED]; all += it->second.n_rec; } }
-  if (in_other_order(mixed, all) == b.mixed) return;
+  if (mostly_mixed(mixed, all) == b.mixed) return;
   for (ShapeEntry& s : ctx->shapes) {
     bool same = s.n_rec.size() == b.n;
     for (u32 k = 0; k < b.n && same; ++k) { auto it = ctx->windows.find(b.first + k); same = it != ctx->windows.end() && it->second.n_rec == s.n_rec[k]; }
@@ -1067,7 +1064,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   if (expect) {
     u64 mixed = 0, all = 0, fused = 0;
     for (u32 k = 0; k < B; ++k) { const u64* t = tot + (size_t)k * T_COUNT; mixed += t[T_MIXED]; fused += t[T_FUSED]; all += ws[k]->n_rec; }
-    pbatch.mixed = in_other_order(mixed, all);
+    pbatch.mixed = mostly_mixed(mixed, all);
     if (pbatch.mixed && n_list[B_FCTA] && fused * 32 * 2 >= total_slots && total_slots * sizeof(PackedRecord) <= PACK_MOST && !capturing(st))
       records = record_space(ctx, total_slots * sizeof(PackedRecord), *expect);
   }

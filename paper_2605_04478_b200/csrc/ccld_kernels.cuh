@@ -277,13 +277,6 @@ __global__ void __launch_bounds__(REC_THREADS) k_seq_range(const WinDesc* wd, Re
       }
     }
   }
-  if (mixed != 0) {
-    // Many communicators take turns. In the order of their ranks all the same if the runs of the warp's first stretch mostly begin with the
-    // rank of the run before. (Looked at once and not in the loop, where it costs every upload 4 % of the pass.)
-    const u64 at = (u64)blockIdx.x * blocks_per_cta * REC_PER_CTA + threadIdx.x * REC_RUN;
-    const u32 rk = at < n_rec ? D.rank[at] : NONE, before = __shfl_up_sync(0xFFFFFFFFu, rk, 1);
-    if (__popc(__ballot_sync(0xFFFFFFFFu, lane != 0 && at < n_rec && rk != before)) < 16) mixed = 0;
-  }
   if (lane == 0) count_add(D.counters, C_MIXED, mixed);
   if (s_mn == nullptr) return;
   __syncthreads();

@@ -8,10 +8,9 @@
 //   emit_lists  a CTA per (window, chunk, 256 communicators) writes their part of the chunk's work lists, beside the scatter
 //             pass and in its launch (ccld_kernels.cuh)
 //
-// All are bound by latency: little data, a chain of dependent reads and barriers. The layout used to be one CTA per
-// window for everything - one scan over the communicators per chunk, the rank table of the whole job walked by one SM -
-// and took 20 us (one communicator, 1,000 ops) to 155 us (2,185 communicators, 16,384 ranks), twice per batch. What a
-// chunk holds follows from the communicators' unit counts alone, so the chunks' starts come from a histogram along the chunks, and the lists are written by as many CTAs as there are chunks.
+// All are bound by latency: little data, a chain of dependent reads and barriers. What a chunk holds follows from the communicators' unit
+// counts alone, so the chunks' starts come from a histogram along the chunks, and the lists are written by as many CTAs as there
+// are chunks. (One CTA per window for all of it took 155 us for the 2,185 communicators of 16,384 ranks, k_layout takes 18.)
 #pragma once
 #include "ccld_device.cuh"
 
@@ -93,6 +92,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   __shared__ PlanAcc s_warp[33];
   __shared__ u32 s_red[32];
   __shared__ u32 s_hist[2][CHUNK_MAX], s_fused;                // units per chunk: warp-tiles of class 0, tiles of class 1; slots / 32 of both
+  __shared__ bool s_turns;                                     // records in their ranks' order, only that ranks take turns over many communicators
   const WinDesc& D = wd[blockIdx.y];
   const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (blockIdx.x > 0) { fill_slots(D.perm, D.n_slots, blockIdx.x - 1, gridDim.x - 1); return; }
@@ -101,6 +101,24 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
   u64 expected = 0; bool poisoned = false;
   const u64 mixed = D.counters[C_MIXED];
   if (wid == 0 && expects) { expected = lane < T_COUNT ? D.expect[lane] : 0; poisoned = *(volatile u32*)D.poison != 0; }
+  if (wid == 1) {
+    // Stretches that did not fold: another order than the ranks', unless sixteen records on the rank is mostly the same. Looked at in eight
+    // places of such a window, and not by k_seq_range: there it cost every upload 1 us, in the loop 4 % of the pass.
+    u32 pairs = 0, changes = 0;
+    const u64 n_rec = D.n_rec;
+    if (mostly_mixed(mixed, n_rec)) {
+      u32 rk[8]; bool in[8];
+#pragma unroll
+      for (u32 q = 0; q < 8; ++q) { const u64 at = n_rec / 8 * q + lane * REC_PER_THREAD; in[q] = at < n_rec; rk[q] = in[q] ? D.rank[at] : NONE; }
+#pragma unroll
+      for (u32 q = 0; q < 8; ++q) {
+        const u32 before = __shfl_up_sync(0xFFFFFFFFu, rk[q], 1);
+        in[q] = in[q] && lane != 0;
+        pairs += __popc(__ballot_sync(0xFFFFFFFFu, in[q])); changes += __popc(__ballot_sync(0xFFFFFFFFu, in[q] && rk[q] != before));
+      }
+    }
+    if (lane == 0) s_turns = changes * 2 < pairs;
+  }
   const u32 per = ceil_div(R.n_comms, blockDim.x), c_lo = threadIdx.x * per, c_hi = min(R.n_comms, c_lo + per);   // my communicators
   // counters covered and members of my first few communicators stay in registers, all loads issued at once
   u32 c_ns[LAYOUT_CACHED], c_n[LAYOUT_CACHED];
@@ -194,7 +212,7 @@ __global__ void __launch_bounds__(LAYOUT_THREADS) k_layout(const WinDesc* wd, Re
     t = lane == T_GROUPS ? all.groups : t; t = lane == T_SLOTS ? all.slots : t; t = lane == T_FCTA ? n_cta : t; t = lane == T_FWT ? n_wt : t;
     t = lane == T_FSUM ? all.units : t; t = lane == T_TILES2 ? all.t2 : t; t = lane == T_TILES3 ? all.t3 : t; t = lane == T_ROWS ? all.rows : t;
     t = lane == T_CHUNKS ? T : t; t = lane == T_WT_PER_CTA ? wt_per_cta : t;
-    t = lane == T_MIXED ? mixed : t; t = lane == T_FUSED ? s_fused : t;
+    t = lane == T_MIXED ? (s_turns ? 0 : mixed) : t; t = lane == T_FUSED ? s_fused : t;
     // op counters further apart than 2^31, or more slots than the cap: refuse the window
     u64 failed = (all.slots > slot_cap || all.groups > 0x7FFFFFFFull) ? FAILED_CAPACITY : 0;
     if (!failed && expects) {
