@@ -47,7 +47,7 @@ NCU_TRAFFIC = {
                        "sha16": "f364d4d60597ddbe"},
     # capture on 5 cfg4w windows
     "k_reduce_large": {"bytes_per_record": (770.79e6 + 52.73e6) / 20.48e6, "files": ("ccld_large.cuh",),
-                       "sha16": "01c740b3b9c12b8c"},
+                       "sha16": "731fe1db96b68837"},
 }
 
 MIXES = {"all": ((0, 0, 1, 0, 2), 200), "tp_pp": ((0, 0, 1, 0), 250), "dp": ((2,), 200)}   # op pattern (0 TP, 1 PP, 2 DP), repetitions

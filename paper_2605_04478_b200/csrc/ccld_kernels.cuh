@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(SCAT_THREADS, 4) k_slot_scatter(const WinDesc*
 // The same where the upload has its records in another order (see PackedRecord): few of them belong to the ranks a CTA would resolve,
 // so every record takes the two table loads, and its values, which the reading of the columns brings along whole, go to the slot
 // with its index. Two windows of 4,096 ranks in arrival order, 8.2 M records: 232 us, and the fused kernel 98 (48 bytes of tables per record from
-// L1 or L2, 36 bytes to random sectors), where indices alone take 129 and the gathers 252; 0.5 M records each of 512 ranks 35 and 19, 24 and 36. In rank-major order it is the other way round (a record read and written twice, 109 instead of 79 bytes).
+// L1 or L2, 36 bytes to random sectors), where indices alone take 129 and the gathers 252; 0.5 M records each of 512 ranks 35 and 19, 24 and 36. In
+// rank-major order it is the other way round (a record read and written twice, 109 instead of 79 bytes).
 // Two records per thread with their values asked for together with the keys; four with the values asked for last took 219, one 283.
 constexpr int PACK_PER_THREAD = 2;
 constexpr int PACK_PER_CTA = SCAT_THREADS * PACK_PER_THREAD;

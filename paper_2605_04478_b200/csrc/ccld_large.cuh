@@ -169,8 +169,8 @@ __device__ __forceinline__ u32 cluster_duration(const uint2* p, u32 cta) {
   u32 d; asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(d) : "r"(cluster_address(p, cta) + 4) : "memory"); return d;
 }
 
-// CTAs per SM: three up to 4,096 members, although that leaves 40 registers and spills some 80 bytes (two instead: 254 and not 228 us on two windows
-// of 1,100 members, 149 and not 144 of 2,000, 138 and not 129 ns per op counter of 3,000 before keys went to their owners at once);
+// CTAs per SM: three up to 4,096 members, although that leaves 40 registers and spills some 80 bytes (two instead, with two windows each:
+// 261 and not 232 us for 2 x 2,000 groups of 1,100 members, for 2 x 1,000 of 2,000 155 and 147, of 2,049 173 and 161, of 3,000 199 and 190, of 4,096 224 and 222);
 // above, two are what shared memory holds. Two records in flight per thread; four spill more, above 4,096 there is room for them.
 template <int Q>
 __global__ void __launch_bounds__(LQ_THREADS, Q == 16 ? 2 : 3) k_reduce_large(const WinDesc* wd, const Tile* tiles,
