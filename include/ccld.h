@@ -152,7 +152,7 @@ int ccld_comm_set_layers(ccld_ctx* ctx, uint32_t comm, const uint32_t* layer);
  * copies on the context's stream. Pageable buffers may be reused when the call returns; pinned
  * buffers must stay unchanged until the stream has passed the copies (any synchronizing call of
  * this library, e.g. ccld_get_verdict, guarantees that). Up to 32 MB of pinned columns cross by a kernel of one CTA per
- * column instead of copies, which slows what else runs on the GPU for as long as PCIe takes (a matrix product by up to 28 %).
+ * column instead of copies, which slows what else runs on the GPU for as long as PCIe takes (a matrix product by about a fifth).
  * mem_kind 1: every pointer is device memory on the context's device, borrowed until
  * ccld_window_release or ccld_destroy; the caller keeps it alive and unchanged.
  * At most one (comm, seq, rank) record per window (else CCLD_E_DUPLICATE at the verdict; which copy an op is worked out from is not

@@ -155,7 +155,8 @@ constexpr u32 UP_WORKERS = 6, UP_SLOTS = 2 * UP_WORKERS;   // two pieces per wor
 // them: 0.6 MB take 63 us with copies and 36 with the kernel, 2.3 MB 94 and 69, 6.9 MB 180 and 160, 23 MB 473 and 474, 32 MB 639 and 654; where
 // others share the host's PCIe a pass over 23 MB took 723 to 1,169 us with copies, 563 to 641 with the kernel.
 // One CTA per column with four words per thread on their way, because reads that wait for PCIe hold up what else runs on the GPU: a matrix
-// product beside uploads takes 19 to 28 % longer, a copy of device memory 35 to 40 (beside copies 2 and 2). Twice the words: 30 and 55 % (no faster);
+// product beside uploads takes 18 % longer, a copy of device memory 35 (beside copies 2 and 2; with 64 registers per thread instead of 32, which
+// lets no other CTA onto the SM, 19 to 28 and 35 to 40). Twice the words: 30 and 55 % (no faster);
 // half of them 16 and 34, a quarter 5 and 11 (23 MB 477 and 482 us); 32 CTAs of 256 threads and a word each per column: 68 and 60 %.
 constexpr size_t UP_SMALL = 32u << 20;
 constexpr int UP_AHEAD = 4, UP_THREADS = 1024;
@@ -1154,7 +1155,7 @@ int analyze_batch(ccld_ctx* ctx, u32 first_window, u32 n_windows, i64 now_ns, bo
   CK(cudaGetLastError());
   for (u32 k = 0; k < B; ++k) {
     WindowHost& w = *ws[k];
-    w.analysed = true; w.plan_blk = plan_blk; w.res_blk = res_blk; w.d_desc = d_desc + k; w.d = hd[k];
+    w.analysed = true; w.plan_blk = plan_blk; w.res_blk = res_blk; w.d_desc = d_desc + k; w.d = hd[k]; w.d.packed = nullptr;      // (the batch's, not the window's)
     std::memcpy(w.totals, tot + (size_t)k * T_COUNT, sizeof w.totals);
   }
   // what the layout really found is in pinned memory once the stream has passed it; settle() reads it

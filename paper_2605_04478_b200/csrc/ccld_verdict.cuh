@@ -210,11 +210,12 @@ __global__ void __launch_bounds__(VD_THREADS) k_verdict_merge(VerdictArgs A, Reg
 }
 
 // Several device arrays into one pinned area, one launch: a row of CTAs per piece. Source and destination agree modulo 16, so
-// whole 16-byte words cross PCIe and only a piece's ends go byte by byte. AHEAD: words a thread asks for at once.
+// whole 16-byte words cross PCIe and only a piece's ends go byte by byte. AHEAD: words a thread asks for at once. (32 registers
+// for large CTAs, so that one leaves room for others on its SM.)
 constexpr int GATHER_THREADS = 256;
 constexpr u32 GATHER_PIECES = 24;
 struct GatherArgs { struct { const unsigned char* src; unsigned char* dst; u64 n; } piece[GATHER_PIECES]; };
-template <int AHEAD, int THREADS> __global__ void __launch_bounds__(THREADS) k_gather(GatherArgs A) {
+template <int AHEAD, int THREADS> __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 2 : 1) k_gather(GatherArgs A) {
   begin_after();
   const unsigned char* src = A.piece[blockIdx.y].src; unsigned char* __restrict__ dst = A.piece[blockIdx.y].dst;
   const u64 n = A.piece[blockIdx.y].n;
